@@ -1569,10 +1569,10 @@ static int update_impl(eoq_handle_t handle, int num, int8_t *const *w, const int
         t[i].master = nullptr;
     }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    count_launches(h, 2 * ((num + 63) / 64) + (step_dev ? 1 : 0));
+    count_launches(h, update_launches(t, num, false));
     ProfScope prof(h, EOQ_PROF_UPDATE, s);
     return record(h, launch_update(t, num, lr_mant, lr_exp, round_mode == EOQ_ROUND_STOCHASTIC, seed, step,
-                                   reinterpret_cast<unsigned long long *>(step_dev), h->dev, h->sm_count, s));
+                                   reinterpret_cast<unsigned long long *>(step_dev), h->dev, s));
 }
 
 extern "C" int eoq_update(eoq_handle_t handle, int num, int8_t *const *w, const int8_t *const *g,
@@ -1611,7 +1611,7 @@ extern "C" int eoq_update_wide(eoq_handle_t handle, int num, int32_t *const *mas
         t[i].master = master[i];
     }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    count_launches(h, 2 * ((num + 63) / 64) + (step_dev ? 1 : 0));
+    count_launches(h, update_launches(t, num, true));
     ProfScope prof(h, EOQ_PROF_UPDATE, s);
     return record(h, launch_update_wide(t, num, lr_mant, lr_exp, k_u, k_m, round_mode == EOQ_ROUND_STOCHASTIC, seed, step,
                                         reinterpret_cast<unsigned long long *>(step_dev), h->dev, s));

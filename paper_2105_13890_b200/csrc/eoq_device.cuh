@@ -29,6 +29,15 @@ __device__ __forceinline__ long long rne_shr64(long long a, int s)
 
 __device__ __forceinline__ int32_t clampi(int32_t v, int32_t lo, int32_t hi) { return min(max(v, lo), hi); }
 
+// Four int32 values saturated to int8 and packed into one word, c0 in the lowest byte: two instructions.
+__device__ __forceinline__ uint32_t pack4_sat(int c0, int c1, int c2, int c3)
+{
+    uint32_t hi, r;
+    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(hi) : "r"(c3), "r"(c2), "r"(0));
+    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(c1), "r"(c0), "r"(hi));
+    return r;
+}
+
 // R(log2 M) for M >= 1: floor(log2 M) plus one when M^2 >= 2^(2f+1).
 __device__ __forceinline__ int round_log2_u32(uint32_t M)
 {
@@ -136,6 +145,18 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v
     }
     __syncthreads();
     return v;
+}
+
+// The 32-bit forms use the warp-wide reduction instructions (one instead of five shuffle steps).
+__device__ __forceinline__ uint32_t block_max_u32(uint32_t v)
+{
+    __shared__ uint32_t red_max32[32];
+    v = __reduce_max_sync(0xffffffffu, v);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+    if (lane == 0) red_max32[warp] = v;
+    __syncthreads();
+    if (warp == 0) v = __reduce_max_sync(0xffffffffu, lane < nw ? red_max32[lane] : 0u);
+    return v;  // (a second call in the same kernel must be separated from this one by a barrier)
 }
 
 __device__ __forceinline__ long long block_sum_i64(long long v)

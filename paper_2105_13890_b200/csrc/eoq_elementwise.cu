@@ -1,6 +1,6 @@
 // Bandwidth-bound kernels of the EOQ layer (arXiv 2105.13890): the standalone quantizers Q / CQ / SQ
 // (Sec. 3.2.2), the second phase of the scale quantizer after a convolution, the head of the error
-// chain (Sec. 3.2.1), the 8-bit update (Sec. 3.2.3) and small layout helpers.
+// chain (Sec. 3.2.1) and small layout helpers.
 // Reductions run warp-shuffle -> one atomic per warp; 16 elements per thread with 128-bit accesses.
 #include "eoq_device.cuh"
 #include "eoq_internal.h"
@@ -554,13 +554,6 @@ __global__ void sq_i64_kernel(const long long *__restrict__ src, const int32_t *
 
 // ------------------------------------------------------------------ head of the error chain
 
-__device__ __forceinline__ void unpack16(const int4 &v, int (&o)[16])
-{
-    const int8_t *b = reinterpret_cast<const int8_t *>(&v);
-#pragma unroll
-    for (int k = 0; k < 16; ++k) o[k] = b[k];
-}
-
 // Pass 1: max |e1| and the sums behind g_b2 and g_gamma, with e1 = e0 * [x4 > 0].
 // Expands 4 mask bits into 4 byte masks (0x00 / 0xff).
 __device__ __forceinline__ uint32_t bits_to_bytes(uint32_t nibble)
@@ -814,177 +807,6 @@ prescale_fused_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, cons
         dev->arrivals = 0;
     }
 }
-
-// ------------------------------------------------------------------ 8-bit update
-
-constexpr int kUpdChunk = 64;           // tensors per launch
-constexpr int kUpdElemsPerBlock = 8192;  // elements one block covers
-
-struct UpdateBatch {
-    UpdateTensor t[kUpdChunk];
-    int first_block[kUpdChunk + 1];
-    int num;
-    int tensor_base;  // index of t[0] in the whole call (cell of its maximum, counter of the hash)
-};
-
-__device__ __forceinline__ int find_tensor(const UpdateBatch &b, int block)
-{
-    int k = 0;
-    while (k + 1 < b.num && block >= b.first_block[k + 1]) ++k;
-    return k;
-}
-
-__global__ void update_absmax_kernel(const __grid_constant__ UpdateBatch b, DeviceState *dev)
-{
-    const int k = find_tensor(b, blockIdx.x);
-    const UpdateTensor &T = b.t[k];
-    const size_t begin = (size_t)(blockIdx.x - b.first_block[k]) * kUpdElemsPerBlock;
-    const size_t end = min((size_t)T.n, begin + kUpdElemsPerBlock);
-    uint32_t mx = 0;
-    if (begin < end) {
-        // 16-byte path when the tensor base allows it (it always does for 16-byte aligned tensors)
-        const bool vec = (reinterpret_cast<uintptr_t>(T.g) & 15) == 0;
-        size_t i = begin + (size_t)threadIdx.x * 16;
-        if (vec) {
-            for (; i + 16 <= end; i += (size_t)blockDim.x * 16) {
-                int e[16];
-                unpack16(__ldg(reinterpret_cast<const int4 *>(T.g + i)), e);
-#pragma unroll
-                for (int q = 0; q < 16; ++q) mx = max(mx, (uint32_t)abs(e[q]));
-            }
-        }
-        // remaining elements of this block's range
-        const size_t tail = vec ? begin + ((end - begin) / 16) * 16 : begin;
-        for (size_t j = tail + threadIdx.x; j < end; j += blockDim.x) mx = max(mx, (uint32_t)abs((int)T.g[j]));
-    }
-    mx = (uint32_t)block_max_u64(mx);
-    if (threadIdx.x == 0 && mx) atomicMax(&dev->tensor_absmax[b.tensor_base + k], mx);
-}
-
-// SplitMix64 output function (Steele, Lea, Flood 2014) as a counter hash.
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z)
-{
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
-// w <- Q_w(w - Q_u(lr * g)) on int8 codes (Sec. 3.2.3).
-__device__ __forceinline__ int update_one(int w, int g, int lr_mant, int t, int d, int stochastic,
-                                          unsigned long long key, unsigned long long idx)
-{
-    const int u = sq_code32(lr_mant * g, t);
-    long long next;
-    if (d >= 0) {
-        next = (long long)w - (long long)u * (1ll << min(d, 40));
-    } else if (-d > 40) {
-        next = w;
-    } else {
-        const int s = -d;
-        const long long v = (long long)w * (1ll << s) - u;
-        if (!stochastic) {
-            next = rne_shr64(v, s);
-        } else {
-            const unsigned long long r = mix64(key + 0x9E3779B97F4A7C15ull * (idx + 1)) & ((1ull << s) - 1ull);
-            next = (v + (long long)r) >> s;
-        }
-    }
-    return (int)(next < -127 ? -127 : (next > 127 ? 127 : next));
-}
-
-__global__ void update_apply_kernel(const __grid_constant__ UpdateBatch b, int32_t lr_mant, int32_t lr_exp,
-                                    int stochastic, unsigned long long seed, unsigned long long step,
-                                    const unsigned long long *step_dev, DeviceState *dev)
-{
-    if (step_dev) step = *step_dev;  // device-resident step counter (bumped by step_bump_kernel behind the call)
-    const int k = find_tensor(b, blockIdx.x);
-    const UpdateTensor &T = b.t[k];
-    const uint32_t M = dev->tensor_absmax[b.tensor_base + k] * (uint32_t)lr_mant;  // max |lr_mant * g| < 2^15
-    if (M == 0) {
-        if (threadIdx.x == 0 && blockIdx.x == b.first_block[k]) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-        return;  // u = 0: the weights keep their codes
-    }
-    const int t = round_log2_u32(M);
-    const int d = (__ldg(T.g_exp) + lr_exp + t - 7) + 7;  // exponent of u, relative to the weight grid 2^-7
-    unsigned long long key = 0;
-    if (stochastic) {
-        key = mix64(seed + 0x9E3779B97F4A7C15ull * (step + 1));
-        key = mix64(key + 0x9E3779B97F4A7C15ull * ((unsigned long long)(b.tensor_base + k) + 1));
-    }
-    const size_t begin = (size_t)(blockIdx.x - b.first_block[k]) * kUpdElemsPerBlock;
-    const size_t end = min((size_t)T.n, begin + kUpdElemsPerBlock);
-    if (begin >= end) return;
-    const bool vec = ((reinterpret_cast<uintptr_t>(T.g) | reinterpret_cast<uintptr_t>(T.w)) & 15) == 0;
-    if (vec) {
-        for (size_t i = begin + (size_t)threadIdx.x * 16; i + 16 <= end; i += (size_t)blockDim.x * 16) {
-            int gv[16], wv[16], c[16];
-            unpack16(__ldg(reinterpret_cast<const int4 *>(T.g + i)), gv);
-            unpack16(*reinterpret_cast<const int4 *>(T.w + i), wv);
-#pragma unroll
-            for (int q = 0; q < 16; ++q) c[q] = update_one(wv[q], gv[q], lr_mant, t, d, stochastic, key, i + q);
-            *reinterpret_cast<int4 *>(T.w + i) =
-                make_int4((int)pack4(c[0], c[1], c[2], c[3]), (int)pack4(c[4], c[5], c[6], c[7]),
-                          (int)pack4(c[8], c[9], c[10], c[11]), (int)pack4(c[12], c[13], c[14], c[15]));
-        }
-    }
-    const size_t tail = vec ? begin + ((end - begin) / 16) * 16 : begin;
-    for (size_t j = tail + threadIdx.x; j < end; j += blockDim.x)
-        T.w[j] = (int8_t)update_one(T.w[j], T.g[j], lr_mant, t, d, stochastic, key, j);
-}
-
-// The update with a k_u-bit update quantizer and k_m-bit master codes (Sec. 3.2.3 compares the 8-bit update with a
-// 24-bit one): u = SQ(lr g, k_u), master <- CQ(master - u, k_m) on the grid 2^-(k_m - 1), w = Q_w(master).
-__global__ void update_wide_apply_kernel(const __grid_constant__ UpdateBatch b, int32_t lr_mant, int32_t lr_exp, int k_u, int k_m,
-                                         int stochastic, unsigned long long seed, unsigned long long step,
-                                         const unsigned long long *step_dev, DeviceState *dev)
-{
-    if (step_dev) step = *step_dev;
-    const int k = find_tensor(b, blockIdx.x);
-    const UpdateTensor &T = b.t[k];
-    const uint32_t M = dev->tensor_absmax[b.tensor_base + k] * (uint32_t)lr_mant;
-    if (M == 0) {
-        if (threadIdx.x == 0 && blockIdx.x == b.first_block[k]) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-        return;
-    }
-    const int t = round_log2_u32(M);
-    const int su = t - (k_u - 1);                                  // u code = R(lr_mant g / 2^su)
-    const int d = (__ldg(T.g_exp) + lr_exp + su) + (k_m - 1);      // exponent of u relative to the master grid
-    const long long lim_u = (1ll << (k_u - 1)) - 1, lim_m = (1ll << (k_m - 1)) - 1;
-    unsigned long long key = 0;
-    if (stochastic) {
-        key = mix64(seed + 0x9E3779B97F4A7C15ull * (step + 1));
-        key = mix64(key + 0x9E3779B97F4A7C15ull * ((unsigned long long)(b.tensor_base + k) + 1));
-    }
-    const size_t begin = (size_t)(blockIdx.x - b.first_block[k]) * kUpdElemsPerBlock;
-    const size_t end = min((size_t)T.n, begin + kUpdElemsPerBlock);
-    for (size_t j = begin + threadIdx.x; j < end; j += blockDim.x) {
-        const long long a = (long long)lr_mant * T.g[j];
-        long long u = su >= 0 ? rne_shr64(a, su) : a * (1ll << (-su));
-        u = u < -lim_u ? -lim_u : (u > lim_u ? lim_u : u);
-        const long long th = T.master[j];
-        long long next;
-        if (d >= 0) {
-            next = th - u * (1ll << min(d, 38));
-        } else if (-d > 38) {
-            next = th;
-        } else {
-            const int s = -d;
-            const long long v = th * (1ll << s) - u;
-            if (!stochastic) {
-                next = rne_shr64(v, s);
-            } else {
-                const unsigned long long r = mix64(key + 0x9E3779B97F4A7C15ull * (j + 1)) & ((1ull << s) - 1ull);
-                next = (v + (long long)r) >> s;
-            }
-        }
-        next = next < -lim_m ? -lim_m : (next > lim_m ? lim_m : next);
-        T.master[j] = (int32_t)next;
-        const long long w8 = rne_shr64(next, k_m - 8);
-        T.w[j] = (int8_t)(w8 < -127 ? -127 : (w8 > 127 ? 127 : w8));
-    }
-}
-
-__global__ void step_bump_kernel(unsigned long long *step_dev) { *step_dev += 1ull; }
 
 // ------------------------------------------------------------------ layout helpers
 
@@ -1430,70 +1252,6 @@ cudaError_t launch_err_prescale(const int8_t *e0, const int32_t *e0_exp, const u
     hook(&dev->sum0, 2, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);  // sum0 and sum1 are adjacent
     prescale_apply_kernel<<<grid_for(n16, sm_count), kThreads, 0, s>>>(e0, e0_exp, mask, n16, gamma_c, gamma_dev, e3,
                                                                        e3_exp, sum_e1, sum_e1x2, dev);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32_t lr_exp, int stochastic,
-                          uint64_t seed, uint64_t step, unsigned long long *step_dev, DeviceState *dev, int sm_count,
-                          cudaStream_t s)
-{
-    (void)sm_count;
-    cudaError_t e = cudaMemsetAsync(dev->tensor_absmax, 0, sizeof(unsigned) * 256, s);
-    if (e != cudaSuccess) return e;
-    for (int base = 0; base < num; base += kUpdChunk) {
-        UpdateBatch b;
-        b.num = num - base < kUpdChunk ? num - base : kUpdChunk;
-        b.tensor_base = base;
-        int blocks = 0;
-        for (int k = 0; k < b.num; ++k) {
-            b.t[k] = t[base + k];
-            b.first_block[k] = blocks;
-            blocks += (int)((t[base + k].n + kUpdElemsPerBlock - 1) / kUpdElemsPerBlock);
-        }
-        b.first_block[b.num] = blocks;
-        if (blocks == 0) continue;
-        update_absmax_kernel<<<blocks, kThreads, 0, s>>>(b, dev);
-    }
-    for (int base = 0; base < num; base += kUpdChunk) {
-        UpdateBatch b;
-        b.num = num - base < kUpdChunk ? num - base : kUpdChunk;
-        b.tensor_base = base;
-        int blocks = 0;
-        for (int k = 0; k < b.num; ++k) {
-            b.t[k] = t[base + k];
-            b.first_block[k] = blocks;
-            blocks += (int)((t[base + k].n + kUpdElemsPerBlock - 1) / kUpdElemsPerBlock);
-        }
-        b.first_block[b.num] = blocks;
-        if (blocks == 0) continue;
-        update_apply_kernel<<<blocks, kThreads, 0, s>>>(b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
-    }
-    if (step_dev) step_bump_kernel<<<1, 1, 0, s>>>(step_dev);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_update_wide(const UpdateTensor *t, int num, int32_t lr_mant, int32_t lr_exp, int k_u, int k_m, int stochastic,
-                               uint64_t seed, uint64_t step, unsigned long long *step_dev, DeviceState *dev, cudaStream_t s)
-{
-    cudaError_t e = cudaMemsetAsync(dev->tensor_absmax, 0, sizeof(unsigned) * 256, s);
-    if (e != cudaSuccess) return e;
-    for (int pass = 0; pass < 2; ++pass)
-        for (int base = 0; base < num; base += kUpdChunk) {
-            UpdateBatch b;
-            b.num = num - base < kUpdChunk ? num - base : kUpdChunk;
-            b.tensor_base = base;
-            int blocks = 0;
-            for (int k = 0; k < b.num; ++k) {
-                b.t[k] = t[base + k];
-                b.first_block[k] = blocks;
-                blocks += (int)((t[base + k].n + kUpdElemsPerBlock - 1) / kUpdElemsPerBlock);
-            }
-            b.first_block[b.num] = blocks;
-            if (blocks == 0) continue;
-            if (pass == 0) update_absmax_kernel<<<blocks, kThreads, 0, s>>>(b, dev);
-            else update_wide_apply_kernel<<<blocks, kThreads, 0, s>>>(b, lr_mant, lr_exp, k_u, k_m, stochastic, seed, step, step_dev, dev);
-        }
-    if (step_dev) step_bump_kernel<<<1, 1, 0, s>>>(step_dev);
     return cudaGetLastError();
 }
 

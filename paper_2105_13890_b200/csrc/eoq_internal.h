@@ -23,7 +23,7 @@ struct DeviceState {
     long long sum0, sum1;  // reduction cells for integer sums
     unsigned long long absmax2_u64;  // second maximum of a call that also serves its consumer's error head (masked |.|)
     long long sum2;                  // third sum of such a call
-    unsigned tensor_absmax[256];  // per-tensor maxima of the multi-tensor update
+    unsigned tensor_absmax[256];  // per-tensor maxima of the multi-tensor update (zero between calls)
     unsigned ticket;       // blocks of the kernel that consumes the cells last count themselves here (see last_block_done)
     unsigned arrivals;     // grid-wide barrier of the one-kernel error head (cooperative launch)
     unsigned long long probe_cycles;  // eoq_probe_mma_i8: longest issue loop of the last launch, in SM clock cycles
@@ -284,9 +284,9 @@ struct UpdateTensor {
     int32_t *master;  // wide update only: the k_m-bit master codes (w then receives Q_w of them)
 };
 // step_dev (device, optional): the step counter is read from it and it is incremented behind the update.
-cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32_t lr_exp, int stochastic,
-                          uint64_t seed, uint64_t step, unsigned long long *step_dev, DeviceState *dev, int sm_count,
-                          cudaStream_t s);
+cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32_t lr_exp, int stochastic, uint64_t seed,
+                          uint64_t step, unsigned long long *step_dev, DeviceState *dev, cudaStream_t s);
+int update_launches(const UpdateTensor *t, int num, bool wide);  // kernels the call above (wide: the one below) launches
 // The same update with a k_u-bit update quantizer on k_m-bit master codes (t[i].master); t[i].w receives Q_w(master).
 cudaError_t launch_update_wide(const UpdateTensor *t, int num, int32_t lr_mant, int32_t lr_exp, int k_u, int k_m, int stochastic,
                                uint64_t seed, uint64_t step, unsigned long long *step_dev, DeviceState *dev, cudaStream_t s);
