@@ -4,6 +4,7 @@
 // (Sec. 5.1 leaves it unquantized) written operation by operation so that it is reproducible bit for bit, the
 // quantized error it hands back, and the update of the scalar parameters (Sec. 3.2.3) on their 16-bit range.
 // All of it is bandwidth- or latency-bound support work; none of it touches the tensor cores.
+#include "eoq_cells.cuh"
 #include "eoq_device.cuh"
 #include "eoq_internal.h"
 #include "eoq_next_head.cuh"
@@ -24,24 +25,6 @@ inline int blocks_for(size_t items, int sm_count, int per_sm = 8)
     size_t b = (items + kThreads - 1) / kThreads, cap = (size_t)sm_count * per_sm;
     if (b > cap) b = cap;
     return b < 1 ? 1 : (int)b;
-}
-
-// same protocol as in the elementwise kernels: true in thread 0 of the block that arrives last
-__device__ __forceinline__ bool last_block_done(DeviceState *dev)
-{
-    __shared__ unsigned last_s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned t = atomicAdd(&dev->ticket, 1u);
-        last_s = (t == gridDim.x - 1) ? 1u : 0u;
-        if (last_s) {
-            __threadfence();
-            dev->ticket = 0;
-        }
-    }
-    __syncthreads();
-    return last_s != 0 && threadIdx.x == 0;
 }
 
 // ------------------------------------------------------------------ pooling

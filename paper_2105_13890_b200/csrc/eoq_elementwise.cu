@@ -2,6 +2,9 @@
 // (Sec. 3.2.2), the second phase of the scale quantizer after a convolution, the head of the error
 // chain (Sec. 3.2.1) and small layout helpers.
 // Reductions run warp-shuffle -> one atomic per warp; 16 elements per thread with 128-bit accesses.
+#include <cooperative_groups.h>
+
+#include "eoq_cells.cuh"
 #include "eoq_device.cuh"
 #include "eoq_internal.h"
 #include "eoq_next_head.cuh"
@@ -24,26 +27,6 @@ inline int grid_for(size_t work_items, int sm_count, int per_sm = 8)
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     return (int)blocks;
-}
-
-// Every thread of every block calls this after the block's last use of the handle's reduction cells (no early
-// returns before it).  True in thread 0 of the block that arrives last: by then every block has read what it
-// needed and added what it had to add, so that thread may publish the sums and must put the cells back to zero.
-__device__ __forceinline__ bool last_block_done(DeviceState *dev)
-{
-    __shared__ unsigned last_s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned t = atomicAdd(&dev->ticket, 1u);
-        last_s = (t == gridDim.x - 1) ? 1u : 0u;
-        if (last_s) {
-            __threadfence();
-            dev->ticket = 0;
-        }
-    }
-    __syncthreads();
-    return last_s != 0 && threadIdx.x == 0;
 }
 
 // ------------------------------------------------------------------ fp32 -> Q / CQ / SQ
@@ -87,116 +70,196 @@ __global__ void absmax_f32_kernel(const float *__restrict__ src, size_t n, Devic
     }
 }
 
-// mode 0: Q -> int16, mode 1: CQ -> int8, mode 2: SQ -> int8 under the already reduced maximum.
-__global__ void quantize_f32_kernel(int mode, const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp,
-                                    DeviceState *dev)
+// x * 2^up, exact wherever the code depends on it (a result too small for a normal number codes to 0 either way).
+// 2^up itself may exceed the float range for a tensor of subnormal size, hence two factors.
+struct Pow2Scale {
+    float f1, f2;
+    // nearest, ties to even; NaN gives 0 and an infinity the largest or smallest int, as the conversion defines
+    __device__ __forceinline__ int code(float x) const { return __float2int_rn(__fmul_rn(__fmul_rn(x, f1), f2)); }
+};
+__device__ __forceinline__ Pow2Scale pow2_scale(int up)
 {
-    int up = 7;  // codes = R(x * 2^up)
-    if (mode == 2) {
-        const uint32_t mbits = dev->absmax_u32;
-        if (mbits == 0 || mbits >= 0x7f800000u) {
-            up = 7;
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                if (mbits == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-                *dst_exp = -7;
-            }
-        } else {
-            const int t = round_log2_f32bits(mbits);
-            up = 7 - t;
-            if (blockIdx.x == 0 && threadIdx.x == 0) *dst_exp = t - 7;
-        }
-    } else if (dst_exp && blockIdx.x == 0 && threadIdx.x == 0) {
-        *dst_exp = -7;
-    }
-    const int lim = (mode == 0) ? 32767 : 127;
-    const int lo = (mode == 0) ? -32768 : -127;
-    auto code = [&](float x) -> int {
-        float y = scalbnf(x, up);  // exact: a power-of-two scaling of a value that stays far from overflow
-        if (!(fabsf(y) < 1.0e9f)) return (y > 0.f) ? lim : ((y < 0.f) ? lo : 0);
-        return clampi(__float2int_rn(y), lo, lim);
-    };
-    const size_t n16 = n / 16;
-    const float4 *s4 = reinterpret_cast<const float4 *>(src);
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
-        int c[16];
+    return Pow2Scale{__int_as_float((clampi(up, -126, 127) + 127) << 23), up > 127 ? __int_as_float(up << 23) : 1.0f};
+}
+
+// Shift of SQ under the maximum `mbits` (bit pattern of max |x|): codes = R(x * 2^up), exponent -up.
+__device__ __forceinline__ int sq_up(uint32_t mbits) { return (mbits != 0 && mbits < 0x7f800000u) ? 7 - round_log2_f32bits(mbits) : 7; }
+
+template <int kMode>
+__device__ __forceinline__ int quantize_code(const Pow2Scale &sc, float x)
+{
+    return clampi(sc.code(x), kMode == 0 ? -32768 : -127, kMode == 0 ? 32767 : 127);
+}
+
+// four codes at element index 4 i
+template <int kMode>
+__device__ __forceinline__ void quantize_store4(void *dst, size_t i, const Pow2Scale &sc, const float4 &v)
+{
+    const int a = quantize_code<kMode>(sc, v.x), b = quantize_code<kMode>(sc, v.y), c = quantize_code<kMode>(sc, v.z),
+              d = quantize_code<kMode>(sc, v.w);
+    if (kMode == 0) reinterpret_cast<uint2 *>(dst)[i] = make_uint2((a & 0xffff) | (b << 16), (c & 0xffff) | (d << 16));
+    else reinterpret_cast<uint32_t *>(dst)[i] = pack4_sat(a, b, c, d);
+}
+
+// kMode 0: Q -> int16, 1: CQ -> int8, 2: SQ -> int8 under the already reduced maximum.
+// Bound by memory: 4 B in (from L2 where the maximum's pass left it: the tiles are walked backwards), 1 or 2 B out.  A
+// block takes one tile of kQuantTile float4; eight independent, coalesced loads per thread are in flight before the
+// maximum is needed.  12.8 M floats: 18.1 us with 64 strided bytes per thread and a general power-of-two function per
+// element, 7.7 us so.
+constexpr int kQuantLoads = 8, kQuantTile = kThreads * kQuantLoads;
+template <int kMode>
+__global__ void __launch_bounds__(kThreads)
+quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev)
+{
+    __shared__ uint32_t max_s;
+    const size_t n4 = n / 4, base = (size_t)(gridDim.x - 1 - blockIdx.x) * kQuantTile + threadIdx.x;
+    float4 v[kQuantLoads];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            float4 v = __ldg(s4 + i * 4 + k);
-            c[4 * k + 0] = code(v.x);
-            c[4 * k + 1] = code(v.y);
-            c[4 * k + 2] = code(v.z);
-            c[4 * k + 3] = code(v.w);
-        }
-        if (mode == 0) {
-            int4 *d = reinterpret_cast<int4 *>(dst) + i * 2;
-            d[0] = make_int4((c[0] & 0xffff) | (c[1] << 16), (c[2] & 0xffff) | (c[3] << 16),
-                             (c[4] & 0xffff) | (c[5] << 16), (c[6] & 0xffff) | (c[7] << 16));
-            d[1] = make_int4((c[8] & 0xffff) | (c[9] << 16), (c[10] & 0xffff) | (c[11] << 16),
-                             (c[12] & 0xffff) | (c[13] << 16), (c[14] & 0xffff) | (c[15] << 16));
-        } else {
-            reinterpret_cast<int4 *>(dst)[i] =
-                make_int4((int)pack4(c[0], c[1], c[2], c[3]), (int)pack4(c[4], c[5], c[6], c[7]),
-                          (int)pack4(c[8], c[9], c[10], c[11]), (int)pack4(c[12], c[13], c[14], c[15]));
-        }
+    for (int u = 0; u < kQuantLoads; ++u) {
+        const size_t i = base + (size_t)u * kThreads;
+        if (i < n4) v[u] = __ldg(reinterpret_cast<const float4 *>(src) + i);
     }
-    for (size_t i = n16 * 16 + (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int c = code(src[i]);
-        if (mode == 0) reinterpret_cast<int16_t *>(dst)[i] = (int16_t)c;
+    int up = 7;
+    bool last = false;
+    if (kMode == 2) {
+        if (threadIdx.x == 0) max_s = *reinterpret_cast<volatile uint32_t *>(&dev->absmax_u32);
+        __syncthreads();
+        up = sq_up(max_s);
+        if (threadIdx.x == 0) last = last_reader(dev);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0 && dst_exp) {
+        *dst_exp = -up;
+        if (kMode == 2 && max_s == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
+    }
+    const Pow2Scale sc = pow2_scale(up);
+#pragma unroll
+    for (int u = 0; u < kQuantLoads; ++u) {
+        const size_t i = base + (size_t)u * kThreads;
+        if (i < n4) quantize_store4<kMode>(dst, i, sc, v[u]);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < (n & 3)) {
+        const size_t i = n4 * 4 + threadIdx.x;
+        const int c = quantize_code<kMode>(sc, src[i]);
+        if (kMode == 0) reinterpret_cast<int16_t *>(dst)[i] = (int16_t)c;
         else reinterpret_cast<int8_t *>(dst)[i] = (int8_t)c;
     }
-    if (mode == 2 && last_block_done(dev)) dev->absmax_u32 = 0;
+    if (last) dev->absmax_u32 = 0;
+}
+
+// SQ in one launch for tensors that one cluster can hold in registers (kSmallElems codes per block, up to
+// kSmallCluster blocks): every block reduces its part, the maxima meet in distributed shared memory, no cell and no
+// second read is needed.  Bound by latency.
+constexpr int kSmallThreads = 1024, kSmallLoads = 8, kSmallCluster = 8;
+constexpr size_t kSmallElems = (size_t)kSmallThreads * kSmallLoads * 4;
+__global__ void __launch_bounds__(kSmallThreads)
+quantize_sq_small_kernel(const float *__restrict__ src, size_t n, int8_t *dst, int32_t *dst_exp, DeviceState *dev)
+{
+    namespace cg = cooperative_groups;
+    __shared__ uint32_t max_s;
+    cg::cluster_group cluster = cg::this_cluster();
+    const size_t n4 = n / 4, base = (size_t)blockIdx.x * kSmallThreads + threadIdx.x, step = (size_t)gridDim.x * kSmallThreads;
+    float4 v[kSmallLoads];
+    uint32_t mx = 0;
+#pragma unroll
+    for (int u = 0; u < kSmallLoads; ++u) {
+        const size_t i = base + u * step;
+        v[u] = i < n4 ? __ldg(reinterpret_cast<const float4 *>(src) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float tail = 0.0f;
+    const size_t ti = n4 * 4 + threadIdx.x;
+    if (blockIdx.x == 0 && ti < n) tail = src[ti];
+#pragma unroll
+    for (int u = 0; u < kSmallLoads; ++u)
+        mx = max(max(mx, max(__float_as_uint(v[u].x) & 0x7fffffffu, __float_as_uint(v[u].y) & 0x7fffffffu)),
+                 max(__float_as_uint(v[u].z) & 0x7fffffffu, __float_as_uint(v[u].w) & 0x7fffffffu));
+    mx = max(mx, __float_as_uint(tail) & 0x7fffffffu);
+    mx = block_max_u32(mx);
+    if (threadIdx.x == 0) max_s = mx;
+    cluster.sync();
+    mx = 0;
+    for (unsigned r = 0; r < gridDim.x; ++r) mx = max(mx, *cluster.map_shared_rank(&max_s, r));
+    const int up = sq_up(mx);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *dst_exp = -up;
+        if (mx == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
+        if (mx >= 0x7f800000u) atomicOr(&dev->status, EOQ_DEV_NONFINITE);
+    }
+    const Pow2Scale sc = pow2_scale(up);
+#pragma unroll
+    for (int u = 0; u < kSmallLoads; ++u) {
+        const size_t i = base + u * step;
+        if (i < n4) quantize_store4<2>(dst, i, sc, v[u]);
+    }
+    if (blockIdx.x == 0 && ti < n) dst[ti] = (int8_t)quantize_code<2>(sc, tail);
+    cluster.sync();  // no block leaves while another may still read its maximum
 }
 
 // SQ of an fp32 image under the already reduced maximum: c_src channels in, c_dst (zero-padded) channels out,
 // rows widened by `wmargin` zero pixels at both ends.  A thread writes kG = 16 or 8 channels of a pixel.
+// Bound by memory (12 B in, 8 or 16 B out per RGB pixel).  A block is tx pixels x ty rows and a thread takes its pixel in
+// kImageRows rows, all loads issued before the maximum is needed, no divisions: 3.2 M pixels took 30.4 us with one
+// pixel at a time behind three of them.
+constexpr int kImageRows = 4;
 template <int kG>
-__global__ void quantize_image_kernel(const float *__restrict__ src, int rows, int w, int c_src, int c_dst, int wmargin,
-                                      int8_t *dst, int32_t *dst_exp, DeviceState *dev)
+__global__ void __launch_bounds__(kThreads)
+quantize_image_kernel(const float *__restrict__ src, int rows, int w, int c_src, int c_dst, int wmargin, int8_t *dst, int32_t *dst_exp,
+                      DeviceState *dev)
 {
-    const uint32_t mbits = dev->absmax_u32;
+    __shared__ uint32_t max_s;
+    const int groups = c_dst / kG, w_mem = w + 2 * wmargin, items = w_mem * groups;
+    const int row0 = blockIdx.x * (kImageRows * blockDim.y) + threadIdx.y;
+    const bool t0 = threadIdx.x == 0 && threadIdx.y == 0;
     int up = 7;
-    const bool usable = mbits != 0 && mbits < 0x7f800000u;
-    if (usable) up = 7 - round_log2_f32bits(mbits);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *dst_exp = usable ? -up : -7;
-        if (mbits == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-    }
-    const int groups = c_dst / kG;
-    const int w_mem = w + 2 * wmargin;
-    const size_t items = (size_t)rows * w_mem * groups;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (size_t)gridDim.x * blockDim.x) {
-        int g, xm;
-        size_t row;
-        if (items <= 0xffffffffull) {  // 32-bit index arithmetic: three 64-bit divisions would dominate the item's work
-            const uint32_t mp = (uint32_t)i / (uint32_t)groups, r = mp / (uint32_t)w_mem;
-            g = (int)((uint32_t)i - mp * (uint32_t)groups);
-            xm = (int)(mp - r * (uint32_t)w_mem) - wmargin;
-            row = r;
-        } else {
-            g = (int)(i % groups);
-            const size_t mp = i / groups;            // pixel index in the widened layout
-            xm = (int)(mp % w_mem) - wmargin;
-            row = mp / w_mem;
-        }
-        int c[kG];
+    bool last = false;
+    for (int x0 = 0; x0 < items; x0 += blockDim.x) {   // one round unless a row is wider than the block
+        const int it = x0 + threadIdx.x;
+        const int xp = groups == 1 ? it : it / groups, g = groups == 1 ? 0 : it - xp * groups, xm = xp - wmargin;
+        const int nch = min(kG, c_src - g * kG);       // real channels of this group (none or fewer beyond c_src)
+        const bool in = it < items && xm >= 0 && xm < w;
+        float v[kImageRows][4];                        // the first four channels; more are read when they are coded
 #pragma unroll
-        for (int k = 0; k < kG; ++k) {
-            const int ch = g * kG + k;
-            int v = 0;
-            if (ch < c_src && xm >= 0 && xm < w) {
-                const float y = scalbnf(__ldg(src + (row * w + xm) * c_src + ch), up);
-                v = (fabsf(y) < 1.0e9f) ? clampi(__float2int_rn(y), -127, 127) : (y > 0.f ? 127 : (y < 0.f ? -127 : 0));
-            }
-            c[k] = v;
+        for (int u = 0; u < kImageRows; ++u) {
+            const int row = row0 + u * blockDim.y;
+            const float *p = src + ((size_t)row * w + xm) * c_src + g * kG;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[u][k] = (in && row < rows && k < nch) ? __ldg(p + k) : 0.0f;
         }
-        if (kG == 16)
-            reinterpret_cast<int4 *>(dst)[i] =
-                make_int4((int)pack4(c[0], c[1], c[2], c[3]), (int)pack4(c[4], c[5], c[6], c[7]),
-                          (int)pack4(c[8 % kG], c[9 % kG], c[10 % kG], c[11 % kG]), (int)pack4(c[12 % kG], c[13 % kG], c[14 % kG], c[15 % kG]));
-        else
-            reinterpret_cast<int2 *>(dst)[i] = make_int2((int)pack4(c[0], c[1], c[2], c[3]), (int)pack4(c[4], c[5], c[6], c[7]));
+        if (x0 == 0) {
+            if (t0) max_s = *reinterpret_cast<volatile uint32_t *>(&dev->absmax_u32);
+            __syncthreads();
+            up = sq_up(max_s);
+            if (t0) {
+                last = last_reader(dev);
+                if (blockIdx.x == 0) {
+                    *dst_exp = -up;
+                    if (max_s == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
+                }
+            }
+        }
+        const Pow2Scale sc = pow2_scale(up);
+#pragma unroll
+        for (int u = 0; u < kImageRows; ++u) {
+            const int row = row0 + u * blockDim.y;
+            if (it >= items || row >= rows) continue;
+            int c[kG];
+#pragma unroll
+            for (int k = 0; k < kG; ++k) c[k] = k < 4 ? quantize_code<2>(sc, v[u][k & 3]) : 0;
+            if (in && nch > 4) {
+                const float *p = src + ((size_t)row * w + xm) * c_src + g * kG;
+#pragma unroll
+                for (int k = 4; k < kG; ++k)
+                    if (k < nch) c[k] = quantize_code<2>(sc, __ldg(p + k));
+            }
+            const size_t o = (size_t)row * items + it;
+            if (kG == 16)
+                reinterpret_cast<uint4 *>(dst)[o] = make_uint4(pack4_sat(c[0], c[1], c[2], c[3]), pack4_sat(c[4], c[5], c[6], c[7]),
+                                                               pack4_sat(c[8 % kG], c[9 % kG], c[10 % kG], c[11 % kG]),
+                                                               pack4_sat(c[12 % kG], c[13 % kG], c[14 % kG], c[15 % kG]));
+            else
+                reinterpret_cast<uint2 *>(dst)[o] = make_uint2(pack4_sat(c[0], c[1], c[2], c[3]), pack4_sat(c[4], c[5], c[6], c[7]));
+        }
     }
-    if (last_block_done(dev)) dev->absmax_u32 = 0;
+    if (last) dev->absmax_u32 = 0;
 }
 
 // w[oc][kh][kw][c] -> wp[oc][kh][8][c] with zeros in the unused taps; c = 16 (Pixel = int4) or 8 (int2)
@@ -1113,14 +1176,33 @@ cudaError_t launch_reset_cells(DeviceState *dev, cudaStream_t s)
                            offsetof(DeviceState, tensor_absmax) - offsetof(DeviceState, absmax_u32), s);
 }
 
+bool quantize_is_small(int mode, size_t n, const ReduceHook &hook) { return mode == 2 && !hook.fn && n <= kSmallElems * kSmallCluster; }
+
 cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev,
                                 int sm_count, cudaStream_t s, const ReduceHook &hook)
 {
+    if (quantize_is_small(mode, n, hook)) {
+        int blocks = 1;
+        while ((size_t)blocks * kSmallElems < n) blocks *= 2;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim = {(unsigned)blocks, 1, 1};
+        cfg.gridDim = dim3(blocks);
+        cfg.blockDim = dim3(kSmallThreads);
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, quantize_sq_small_kernel, src, n, static_cast<int8_t *>(dst), dst_exp, dev);
+    }
     if (mode == 2) {
         absmax_f32_kernel<<<grid_for(n / 4 + 1, sm_count), kThreads, 0, s>>>(src, n, dev);
         hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);  // float bit patterns of |x| order like integers
     }
-    quantize_f32_kernel<<<grid_for(n / 16 + 1, sm_count), kThreads, 0, s>>>(mode, src, n, dst, dst_exp, dev);
+    const unsigned blocks = (unsigned)((n / 4 + kQuantTile - 1) / kQuantTile > 0 ? (n / 4 + kQuantTile - 1) / kQuantTile : 1);
+    if (mode == 0) quantize_f32_kernel<0><<<blocks, kThreads, 0, s>>>(src, n, dst, dst_exp, dev);
+    else if (mode == 1) quantize_f32_kernel<1><<<blocks, kThreads, 0, s>>>(src, n, dst, dst_exp, dev);
+    else quantize_f32_kernel<2><<<blocks, kThreads, 0, s>>>(src, n, dst, dst_exp, dev);
     return cudaGetLastError();
 }
 
@@ -1130,13 +1212,13 @@ cudaError_t launch_quantize_image(const float *src, int n, int h, int w, int c_s
     const size_t count = (size_t)n * h * w * c_src;
     absmax_f32_kernel<<<grid_for(count / 4 + 1, sm_count), kThreads, 0, s>>>(src, count, dev);
     hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
-    if (c_dst % 16 == 0) {
-        const size_t items = (size_t)n * h * (w + 2 * wmargin) * (c_dst / 16);
-        quantize_image_kernel<16><<<grid_for(items, sm_count), kThreads, 0, s>>>(src, n * h, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
-    } else {
-        const size_t items = (size_t)n * h * (w + 2 * wmargin) * (c_dst / 8);
-        quantize_image_kernel<8><<<grid_for(items, sm_count), kThreads, 0, s>>>(src, n * h, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
-    }
+    const int g = c_dst % 16 == 0 ? 16 : 8, items = (w + 2 * wmargin) * (c_dst / g), rows = n * h;
+    int tx = 32;
+    while (tx < items && tx < kThreads) tx *= 2;
+    const dim3 block(tx, kThreads / tx);
+    const unsigned grid = (unsigned)((rows + kImageRows * (int)block.y - 1) / (kImageRows * (int)block.y));
+    if (g == 16) quantize_image_kernel<16><<<grid, block, 0, s>>>(src, rows, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
+    else quantize_image_kernel<8><<<grid, block, 0, s>>>(src, rows, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
     return cudaGetLastError();
 }
 

@@ -1,6 +1,7 @@
 // The 8-bit update (arXiv 2105.13890, Sec. 3.2.3): u = Q_u(lr g) = SQ(lr g, 8), w <- Q_w(w - u) on the int8 codes, and
 // its generic-width form on master codes.  All tensors of a call go through one launch pair: a maximum per tensor, then
 // the update under it; when every tensor is small, one block takes a tensor through both passes and one launch does it.
+#include "eoq_cells.cuh"
 #include "eoq_device.cuh"
 #include "eoq_internal.h"
 
@@ -206,10 +207,6 @@ __device__ __forceinline__ void update_range(UpdateMode mode, const UpdateTensor
         default: update_range<kStochasticWide>(T, begin, end, r); break;
     }
 }
-
-// One thread of every block calls this once it has read what the launch shares (step counter, maxima): true for the
-// block that comes last, whose thread may then move the counter on and clear the cells.  The counter wraps to zero.
-__device__ __forceinline__ bool last_reader(DeviceState *dev) { return atomicInc(&dev->ticket, gridDim.x - 1) == gridDim.x - 1; }
 
 // w <- Q_w(w - Q_u(lr * g)).  Bound by instruction issue under stochastic rounding (the 64-bit hash is about 20 of the 30
 // instructions of an element), else by memory (3 B per weight).  Every rounding mode is a loop of its own on 32-bit
