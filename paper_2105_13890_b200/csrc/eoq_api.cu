@@ -1798,7 +1798,7 @@ extern "C" int eoq_aux_head(eoq_handle_t handle, const int32_t *sums, int n, int
     Handle *h = reinterpret_cast<Handle *>(handle);
     if (!h || !sums || !W || !bias || !labels || !dpooled || !logits || n <= 0 || c <= 0 || hw <= 0 || classes <= 0)
         return EOQ_ERR_BAD_ARG;
-    if (c > 1536) return EOQ_ERR_UNSUPPORTED;  // the pooled activations of 32 samples are kept in shared memory
+    if (c > 1536) return EOQ_ERR_UNSUPPORTED;
     size_t need = 0;
     eoq_aux_head_workspace_size(n, c, classes, &need);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < need) return EOQ_ERR_WORKSPACE;
@@ -1807,7 +1807,7 @@ extern "C" int eoq_aux_head(eoq_handle_t handle, const int32_t *sums, int n, int
     float *dl = reinterpret_cast<float *>(ws + 2 * round256((size_t)n * c * sizeof(float)));
     double *loss_n = reinterpret_cast<double *>(ws + 2 * round256((size_t)n * c * sizeof(float)) + round256((size_t)n * classes * sizeof(float)));
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    count_launches(h, lr != 0.0f ? 5 : 4);
+    count_launches(h, (head_folds_pooling(n) ? 3 : 4) + (lr != 0.0f ? 1 : 0));
     ProfScope prof(h, EOQ_PROF_GLUE, s);
     return record(h, launch_head(sums, n, c, hw, classes, W, bias, labels, lr, loss, dpooled, logits, pooled, dl, loss_n, s));
 }
@@ -1837,9 +1837,9 @@ extern "C" int eoq_aux_head_error(eoq_handle_t handle, const float *dpooled, int
     if (c % 16 || !aligned16(e)) return EOQ_ERR_ALIGNMENT;
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < (size_t)n * c * sizeof(float)) return EOQ_ERR_WORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    count_launches(h, 2);
+    count_launches(h, head_error_is_single(n, c, h->hook) ? 1 : 2);
     ProfScope prof(h, EOQ_PROF_GLUE, s);
-    return record(h, launch_head_error(dpooled, n, c, hw, static_cast<float *>(workspace), e, e_exp, h->dev, h->sm_count, s, h->hook));
+    return record(h, launch_head_error(dpooled, n, c, hw, e, e_exp, h->dev, h->sm_count, s, h->hook));
 }
 
 extern "C" int eoq_aux_scalar_update(eoq_handle_t handle, int num, int32_t *const *theta, int32_t *const *mirror,

@@ -1,9 +1,7 @@
 // Glue between the quantized convolution units of a Fixup residual network (arXiv 2105.13890, Sec. 3.2.1 chains the
-// units: x0 of a layer is x5 of the one before, e0 is the error handed back by its successor): max and average
-// pooling on int8 codes, the exact join of two error streams followed by Q_e, the floating-point last layer
-// (Sec. 5.1 leaves it unquantized) written operation by operation so that it is reproducible bit for bit, the
-// quantized error it hands back, and the update of the scalar parameters (Sec. 3.2.3) on their 16-bit range.
-// All of it is bandwidth- or latency-bound support work; none of it touches the tensor cores.
+// units: x0 of a layer is x5 of the one before, e0 the error its successor hands back): max-pooling on int8 codes, the
+// exact join of two error streams followed by Q_e, and the update of the scalar parameters (Sec. 3.2.3) on their 16-bit
+// range.  All of it is bandwidth- or latency-bound support work; none of it touches the tensor cores.
 #include "eoq_cells.cuh"
 #include "eoq_device.cuh"
 #include "eoq_internal.h"
@@ -213,30 +211,6 @@ maxpool_bwd_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, const uin
     }
 }
 
-// sums[b][ch] = sum over the hw positions of x[b][.][ch]; one block per (sample, 16-channel group)
-__global__ void avgpool_sum_kernel(const int8_t *__restrict__ x, int hw, int c, int32_t *__restrict__ sums)
-{
-    __shared__ int part[kThreads][17];
-    const int groups = c / 16, b = blockIdx.x / groups, g = blockIdx.x % groups;
-    int acc[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) acc[q] = 0;
-    for (int i = threadIdx.x; i < hw; i += blockDim.x) {
-        const int4 v = __ldg(reinterpret_cast<const int4 *>(x + ((size_t)b * hw + i) * c + g * 16));
-        const int8_t *e = reinterpret_cast<const int8_t *>(&v);
-#pragma unroll
-        for (int q = 0; q < 16; ++q) acc[q] += e[q];
-    }
-#pragma unroll
-    for (int q = 0; q < 16; ++q) part[threadIdx.x][q] = acc[q];
-    __syncthreads();
-    if (threadIdx.x < 16) {
-        int t = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) t += part[i][threadIdx.x];
-        sums[(size_t)b * c + g * 16 + threadIdx.x] = t;
-    }
-}
-
 // ------------------------------------------------------------------ join of two error streams + Q_e
 
 __device__ __forceinline__ void unpack16(const int4 &v, int (&o)[16])
@@ -375,259 +349,6 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
     }
 }
 
-// ------------------------------------------------------------------ the floating-point last layer
-
-// exp(x) from fused multiply-adds and a power-of-two scaling only (x <= 88): x = k ln2 + r, degree-7 polynomial
-__device__ __forceinline__ float exp_fma(float x)
-{
-    if (x < -87.0f) return 0.0f;
-    if (x > 88.0f) x = 88.0f;
-    const float kf = rintf(__fmul_rn(x, 1.44269504088896341f));
-    float r = __fmaf_rn(-kf, 0.693145751953125f, x);
-    r = __fmaf_rn(-kf, 1.42860682030941723212e-6f, r);
-    float p = 1.0f / 5040.0f;
-    p = __fmaf_rn(p, r, 1.0f / 720.0f);
-    p = __fmaf_rn(p, r, 1.0f / 120.0f);
-    p = __fmaf_rn(p, r, 1.0f / 24.0f);
-    p = __fmaf_rn(p, r, 1.0f / 6.0f);
-    p = __fmaf_rn(p, r, 0.5f);
-    p = __fmaf_rn(p, r, 1.0f);
-    p = __fmaf_rn(p, r, 1.0f);
-    // 2^k with k in [-126, 127] is a normal number and the product is exact short of underflow, which x >= -87 excludes;
-    // p < 2 and k = 127 only for x close to 88, where p * 2^127 stays finite
-    return __fmul_rn(p, __int_as_float(((int)kf + 127) << 23));
-}
-
-// pooled[b][k] = (float)sum * 2^-7 / hw
-__global__ void head_pooled_kernel(const int32_t *__restrict__ sums, int count, int hw, float *pooled)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) pooled[i] = __fdiv_rn(__fmul_rn(__int2float_rn(sums[i]), 0.0078125f), (float)hw);
-}
-
-// logits[b][j] = bias[j] + sum_k fma(W[j][k], pooled[b][k], .), k ascending into one accumulator per (b, j).
-// A warp owns one class j and 32 samples (one per lane), so all lanes walk k together: 32 consecutive weights are
-// loaded by the warp at once and handed round by shuffle, the pooled activations of the 32 samples sit in shared
-// memory as [k][sample].  Every (b, j) still sees its own strictly sequential chain of fused multiply-adds.
-constexpr int kHeadWarps = 8;
-__global__ void head_logits_kernel(const float *__restrict__ pooled, int n, int c, int classes, const float *__restrict__ W,
-                                   const float *__restrict__ bias, float *logits)
-{
-    extern __shared__ float ps[];  // [c][33]: row k holds the 32 samples' activations (padded: the fill walks k, the chains walk samples)
-    const int b0 = blockIdx.y * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < c * 32; i += blockDim.x) {
-        const int sb = i / c, k = i - sb * c;   // consecutive threads read consecutive k of one sample
-        ps[k * 33 + sb] = (b0 + sb < n) ? pooled[(size_t)(b0 + sb) * c + k] : 0.0f;
-    }
-    __syncthreads();
-    const int j = blockIdx.x * kHeadWarps + warp;
-    if (j >= classes) return;
-    float acc = bias[j];
-    const float *wj = W + (size_t)j * c;
-    float wnext = lane < c ? __ldg(wj + lane) : 0.0f;
-    for (int k0 = 0; k0 < c; k0 += 32) {
-        const float wreg = wnext;
-        if (k0 + 32 < c) wnext = (k0 + 32 + lane < c) ? __ldg(wj + k0 + 32 + lane) : 0.0f;   // the next 32 weights travel meanwhile
-        const int kn = min(32, c - k0);
-        if (kn == 32) {
-#pragma unroll
-            for (int kk = 0; kk < 32; ++kk) acc = __fmaf_rn(__shfl_sync(0xffffffffu, wreg, kk), ps[(k0 + kk) * 33 + lane], acc);
-        } else {
-            for (int kk = 0; kk < kn; ++kk) acc = __fmaf_rn(__shfl_sync(0xffffffffu, wreg, kk), ps[(k0 + kk) * 33 + lane], acc);
-        }
-    }
-    if (b0 + lane < n) logits[(size_t)(b0 + lane) * classes + j] = acc;
-}
-
-// One block per sample: softmax with the maximum subtracted, the gradient of the mean cross-entropy with respect to
-// the logits, the sample's loss.  The exponentials are formed in parallel; the denominator is then summed by one
-// thread over j ascending into one accumulator, which is the order that makes the result reproducible.
-__global__ void head_softmax_kernel(const float *__restrict__ logits, int n, int classes, const int32_t *__restrict__ labels, float *dl,
-                                    double *loss_n)
-{
-    __shared__ float red[32];
-    __shared__ float m_s, den_s;
-    const int b = blockIdx.x;
-    const float *l = logits + (size_t)b * classes;
-    float *d = dl + (size_t)b * classes;
-    float m = -3.4e38f;
-    for (int j = threadIdx.x; j < classes; j += blockDim.x) m = l[j] > m ? l[j] : m;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float other = __shfl_xor_sync(0xffffffffu, m, o);
-        m = other > m ? other : m;
-    }
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float mm = red[0];
-        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) mm = red[i] > mm ? red[i] : mm;
-        m_s = mm;
-    }
-    __syncthreads();
-    m = m_s;
-    for (int j = threadIdx.x; j < classes; j += blockDim.x) d[j] = exp_fma(__fsub_rn(l[j], m));
-    __syncthreads();
-    const int y = labels[b];
-    if (threadIdx.x == 0) {
-        float den = 0.0f;
-        for (int j = 0; j < classes; ++j) den = __fadd_rn(den, d[j]);
-        den_s = den;
-        loss_n[b] = (double)logf(den) - (double)__fsub_rn(l[y], m);
-    }
-    __syncthreads();
-    const float den = den_s, inv_n = __fdiv_rn(1.0f, (float)n);
-    for (int j = threadIdx.x; j < classes; j += blockDim.x) {
-        const float pr = __fdiv_rn(d[j], den);
-        d[j] = __fmul_rn(__fsub_rn(pr, j == y ? 1.0f : 0.0f), inv_n);
-    }
-}
-
-// dpooled[b][k] = sum_j fma(dl[b][j], W[j][k], .), j ascending (W before its update); one thread also forms the mean loss.
-// Every output is one chain of `classes` dependent multiply-adds, so the only parallelism is across outputs (n * c of
-// them) and the only thing to hide is the memory traffic: a block owns kDpCh channels x kDpN samples, all its threads
-// fetch the next kDpK rows of W (and of dl) together into registers while the chains run on the current rows in
-// shared memory.
-constexpr int kDpCh = 64, kDpN = 4, kDpK = 32;
-__global__ void __launch_bounds__(kDpCh *kDpN)
-head_dpooled_kernel(const float *__restrict__ dl, const float *__restrict__ W, int n, int c, int classes, float *dpooled,
-                    const double *loss_n, float *loss_out)
-{
-    __shared__ float w_s[2][kDpK][kDpCh];
-    __shared__ float d_s[2][kDpN][kDpK];
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && loss_out) {
-        double s = 0.0;
-        for (int b = 0; b < n; ++b) s += loss_n[b];
-        *loss_out = (float)(s / n);
-    }
-    const int cl = threadIdx.x % kDpCh, nl = threadIdx.x / kDpCh;
-    const int k = blockIdx.x * kDpCh + cl, b = blockIdx.y * kDpN + nl;
-    const bool kin = k < c;
-    constexpr int kRowsPerThread = kDpK / kDpN;   // rows of the W tile one thread fetches
-    float wr[kRowsPerThread], dr = 0.0f;
-    auto fetch = [&](int j0) {
-#pragma unroll
-        for (int r = 0; r < kRowsPerThread; ++r) {
-            const int j = j0 + nl + r * kDpN;
-            wr[r] = (kin && j < classes) ? __ldg(W + (size_t)j * c + k) : 0.0f;
-        }
-        if (threadIdx.x < kDpN * kDpK) {
-            const int bb = blockIdx.y * kDpN + threadIdx.x / kDpK, j = j0 + threadIdx.x % kDpK;
-            dr = (bb < n && j < classes) ? __ldg(dl + (size_t)bb * classes + j) : 0.0f;
-        }
-    };
-    auto stash = [&](int buf) {
-#pragma unroll
-        for (int r = 0; r < kRowsPerThread; ++r) w_s[buf][nl + r * kDpN][cl] = wr[r];
-        if (threadIdx.x < kDpN * kDpK) d_s[buf][threadIdx.x / kDpK][threadIdx.x % kDpK] = dr;
-    };
-    fetch(0);
-    stash(0);
-    __syncthreads();
-    float acc = 0.0f;
-    int buf = 0;
-    for (int j0 = 0; j0 < classes; j0 += kDpK, buf ^= 1) {
-        const bool more = j0 + kDpK < classes;
-        if (more) fetch(j0 + kDpK);
-        const int len = min(kDpK, classes - j0);
-        if (len == kDpK) {
-#pragma unroll
-            for (int jj = 0; jj < kDpK; ++jj) acc = __fmaf_rn(d_s[buf][nl][jj], w_s[buf][jj][cl], acc);
-        } else {
-            for (int jj = 0; jj < len; ++jj) acc = __fmaf_rn(d_s[buf][nl][jj], w_s[buf][jj][cl], acc);
-        }
-        if (more) stash(buf ^ 1);
-        __syncthreads();
-    }
-    if (kin && b < n) dpooled[(size_t)b * c + k] = acc;
-}
-
-// W[j][k] <- fma(-lr, sum_b fma(dl[b][j], pooled[b][k], .), W[j][k]), b ascending; bias[j] alike (thread k == 0)
-__global__ void head_update_kernel(const float *__restrict__ dl, const float *__restrict__ pooled, int n, int c, int classes, float lr,
-                                   float *W, float *bias)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= classes * c) return;
-    const int j = i / c, k = i % c;
-    float acc = 0.0f;
-    int b = 0;
-    for (; b + 8 <= n; b += 8) {
-        float d8[8], p8[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            d8[u] = __ldg(dl + (size_t)(b + u) * classes + j);
-            p8[u] = __ldg(pooled + (size_t)(b + u) * c + k);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc = __fmaf_rn(d8[u], p8[u], acc);
-    }
-    for (; b < n; ++b) acc = __fmaf_rn(__ldg(dl + (size_t)b * classes + j), __ldg(pooled + (size_t)b * c + k), acc);
-    W[i] = __fmaf_rn(-lr, acc, W[i]);
-    if (k == 0) {
-        float db = 0.0f;
-        for (int b = 0; b < n; ++b) db = __fadd_rn(db, dl[(size_t)b * classes + j]);
-        bias[j] = __fmaf_rn(-lr, db, bias[j]);
-    }
-}
-
-// ------------------------------------------------------------------ error handed back by the head
-
-// ef[i] = dpooled[i] / hw and max |ef| (as float bit patterns) into the handle's cell
-__global__ void head_error_scale_kernel(const float *__restrict__ dpooled, int count, int hw, float *ef, DeviceState *dev)
-{
-    uint32_t mx = 0;
-    bool bad = false;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-        const float v = __fdiv_rn(dpooled[i], (float)hw);
-        ef[i] = v;
-        const uint32_t a = __float_as_uint(v) & 0x7fffffffu;
-        bad |= a >= 0x7f800000u;
-        mx = max(mx, a);
-    }
-    mx = (uint32_t)block_max_u64(mx);
-    bad = __syncthreads_or(bad);
-    if (threadIdx.x == 0) {
-        if (mx) atomicMax(&dev->absmax_u32, mx);
-        if (bad) atomicOr(&dev->status, EOQ_DEV_NONFINITE);
-    }
-}
-
-__device__ __forceinline__ int round_log2_f32bits_aux(uint32_t bits)
-{
-    const int eb = (int)((bits >> 23) & 0xffu);
-    const uint32_t frac = bits & 0x7fffffu;
-    if (eb == 0) return round_log2_u32(frac) - 149;
-    const unsigned long long m = (1ull << 23) | frac;
-    return (eb - 127) + ((m * m >= (1ull << 47)) ? 1 : 0);
-}
-
-// e[b][pos][ch] = SQ code of ef[b][ch] for every position; one thread per 16 channels of a pixel
-__global__ void head_error_spread_kernel(const float *__restrict__ ef, int n, int hw, int c, int8_t *e, int32_t *e_exp, DeviceState *dev)
-{
-    const uint32_t mbits = dev->absmax_u32;
-    const bool usable = mbits != 0 && mbits < 0x7f800000u;
-    const int up = usable ? 7 - round_log2_f32bits_aux(mbits) : 7;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *e_exp = usable ? -up : -7;
-        if (mbits == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-    }
-    const int groups = c / 16;
-    const size_t items = (size_t)n * hw * groups;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (size_t)gridDim.x * blockDim.x) {
-        const int g = (int)(i % groups), b = (int)(i / ((size_t)groups * hw));
-        const float *src = ef + (size_t)b * c + g * 16;
-        int q[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const float y = scalbnf(__ldg(src + k), up);
-            q[k] = (fabsf(y) < 1.0e9f) ? clampi(__float2int_rn(y), -127, 127) : (y > 0.f ? 127 : (y < 0.f ? -127 : 0));
-        }
-        reinterpret_cast<int4 *>(e)[i] = make_int4((int)pack4(q[0], q[1], q[2], q[3]), (int)pack4(q[4], q[5], q[6], q[7]),
-                                                    (int)pack4(q[8], q[9], q[10], q[11]), (int)pack4(q[12], q[13], q[14], q[15]));
-    }
-    if (last_block_done(dev)) dev->absmax_u32 = 0;
-}
-
 // ------------------------------------------------------------------ scalar parameters (Sec. 3.2.3 on a single value)
 
 __device__ __forceinline__ unsigned long long mix64_aux(unsigned long long z)
@@ -721,12 +442,6 @@ cudaError_t launch_maxpool_bwd(const int8_t *e, const int32_t *e_exp, const uint
     return cudaGetLastError();
 }
 
-cudaError_t launch_avgpool_sum(const int8_t *x, int n, int hw, int c, int32_t *sums, cudaStream_t st)
-{
-    avgpool_sum_kernel<<<n * (c / 16), kThreads, 0, st>>>(x, hw, c, sums);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_join(const int8_t *a, const int32_t *a_exp, const int8_t *b, const int32_t *b_exp, const uint8_t *mask_b,
                         size_t n_el, int8_t *out, int32_t *out_exp, long long *sum_out, const uint8_t *next_mask,
                         const int16_t *next_x2, const int32_t *next_gamma, int8_t *e3, int32_t *e3_exp, long long *sum_e1,
@@ -767,41 +482,6 @@ cudaError_t launch_join_second(const int8_t *a, const int32_t *a_exp, const int8
     else
         join_kernel<1, false><<<blocks, kThreads, 0, st>>>(a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, nullptr, nullptr,
                                                            nullptr, nullptr, nullptr, nullptr, nullptr, dev);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_head(const int32_t *sums, int n, int c, int hw, int classes, float *W, float *bias, const int32_t *labels,
-                        float lr, float *loss_out, float *dpooled, float *logits, float *pooled, float *dl, double *loss_n,
-                        cudaStream_t st)
-{
-    head_pooled_kernel<<<(n * c + 255) / 256, 256, 0, st>>>(sums, n * c, hw, pooled);
-    {
-        const size_t smem = (size_t)c * 33 * sizeof(float);
-        cudaError_t e = cudaFuncSetAttribute(head_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        dim3 grid((classes + kHeadWarps - 1) / kHeadWarps, (n + 31) / 32);
-        head_logits_kernel<<<grid, 32 * kHeadWarps, smem, st>>>(pooled, n, c, classes, W, bias, logits);
-    }
-    head_softmax_kernel<<<n, 256, 0, st>>>(logits, n, classes, labels, dl, loss_n);
-    head_dpooled_kernel<<<dim3((c + kDpCh - 1) / kDpCh, (n + kDpN - 1) / kDpN), kDpCh * kDpN, 0, st>>>(dl, W, n, c, classes, dpooled,
-                                                                                                   loss_n, loss_out);
-    if (lr != 0.0f) head_update_kernel<<<(classes * c + 127) / 128, 128, 0, st>>>(dl, pooled, n, c, classes, lr, W, bias);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_head_update(const float *dl, const float *pooled, int n, int c, int classes, float lr, float *W, float *bias,
-                               cudaStream_t st)
-{
-    head_update_kernel<<<(classes * c + 127) / 128, 128, 0, st>>>(dl, pooled, n, c, classes, lr, W, bias);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_head_error(const float *dpooled, int n, int c, int hw, float *ef, int8_t *e, int32_t *e_exp, DeviceState *dev,
-                              int sm_count, cudaStream_t st, const ReduceHook &hook)
-{
-    head_error_scale_kernel<<<blocks_for((size_t)n * c, sm_count, 1), kThreads, 0, st>>>(dpooled, n * c, hw, ef, dev);
-    hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, st);
-    head_error_spread_kernel<<<blocks_for((size_t)n * hw * (c / 16), sm_count), kThreads, 0, st>>>(ef, n, hw, c, e, e_exp, dev);
     return cudaGetLastError();
 }
 

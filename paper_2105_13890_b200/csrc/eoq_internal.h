@@ -344,10 +344,12 @@ cudaError_t launch_join_second(const int8_t *a, const int32_t *a_exp, const int8
 cudaError_t launch_head(const int32_t *sums, int n, int c, int hw, int classes, float *W, float *bias, const int32_t *labels,
                         float lr, float *loss_out, float *dpooled, float *logits, float *pooled, float *dl, double *loss_n,
                         cudaStream_t st);
+bool head_folds_pooling(int n);  // launch_head: three kernels (and one for the update) instead of four
 cudaError_t launch_head_update(const float *dl, const float *pooled, int n, int c, int classes, float lr, float *W, float *bias,
                                cudaStream_t st);
-cudaError_t launch_head_error(const float *dpooled, int n, int c, int hw, float *ef, int8_t *e, int32_t *e_exp, DeviceState *dev,
-                              int sm_count, cudaStream_t st, const ReduceHook &hook);
+cudaError_t launch_head_error(const float *dpooled, int n, int c, int hw, int8_t *e, int32_t *e_exp, DeviceState *dev, int sm_count,
+                              cudaStream_t st, const ReduceHook &hook);
+bool head_error_is_single(int n, int c, const ReduceHook &hook);  // one launch instead of two
 struct ScalarItem {
     int32_t *theta;          // the code to update (device)
     int32_t *mirror;         // a second place that receives the new code, or null

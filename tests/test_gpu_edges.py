@@ -53,3 +53,34 @@ def test_update_one_block_per_tensor(lr, stochastic):
         for i in range(len(sizes)):
             ws[i], _, _ = oracle.update(ws[i], gs[i], pgs[i], lr[0], lr[1], stochastic=stochastic, seed=11, step=5 + k, tensor_id=i)
             assert np.array_equal(G.host(w_d[i]).astype(np.int32), ws[i]), (k, i)
+
+
+@pytest.mark.parametrize("n,c,hw,classes", [(1, 16, 1, 1), (8, 36, 4, 63), (9, 528, 9, 65), (3, 1536, 4, 130)])
+def test_float_head_remainders(n, c, hw, classes):
+    """Folded and separate pooling (8 samples), channel counts beyond one 512-channel part, classes around a tile of 64."""
+    hd = G.handle()
+    sums = (synth.relu_codes((n, c), 1530 + n, 0).astype(np.int64) * hw) // 3
+    W = (synth.normal_f32((classes, c), 1530 + n, 1) / np.float32(np.sqrt(c))).astype(np.float32)
+    bias = (synth.normal_f32((classes,), 1530 + n, 2) * np.float32(0.01)).astype(np.float32)
+    labels = synth.labels(n, classes, 1530 + n, 3).astype(np.int32)
+    W_o, bias_o = W.copy(), bias.copy()
+    _, dpooled_o, logits_o = oracle.head(sums, hw, W_o, bias_o, labels, 2.0 ** -6)
+    W_d, bias_d = G.dev(W), G.dev(bias)
+    loss, dpooled, logits = G.zeros(1, torch.float32), G.zeros((n, c), torch.float32), G.zeros((n, classes), torch.float32)
+    ws = G.zeros(eoq.eoq_aux_head_workspace_size(n, c, classes), torch.uint8)
+    eoq.eoq_aux_head(hd, G.dev(sums.astype(np.int32)), n, c, hw, classes, W_d, bias_d, G.dev(labels), 2.0 ** -6, loss, dpooled, logits, ws)
+    torch.cuda.synchronize()
+    assert np.array_equal(G.host(logits), logits_o) and np.array_equal(G.host(dpooled), dpooled_o)
+    assert np.array_equal(G.host(W_d), W_o) and np.array_equal(G.host(bias_d), bias_o)
+
+
+@pytest.mark.parametrize("n,c,hw", [(1, 16, 3), (5, 48, 50), (2, 8208, 2), (200, 512, 2)])
+def test_head_error_sizes(n, c, hw):
+    """Channel groups that do not divide a block, more groups than threads, and more values than one block scans."""
+    d = (synth.normal_f32((n, c), 1540 + n, 0) * np.float32(1e-3)).astype(np.float32)
+    codes, p, _ = oracle.quantize_f32(oracle.MODE_SQ, (d / np.float32(hw)).astype(np.float32))
+    e, pe = G.zeros((n, hw, c), torch.int8), G.zeros(1, torch.int32)
+    for _ in range(2):
+        eoq.eoq_aux_head_error(G.handle(), G.dev(d), n, c, hw, e, pe, G.zeros(n * c * 4, torch.uint8))
+        assert G.status_clear() == 0 and pe.item() == p
+        assert all(np.array_equal(G.host(e)[:, i, :], codes.reshape(n, c)) for i in range(hw))
