@@ -1653,7 +1653,7 @@ extern "C" int eoq_aux_maxpool_fwd(eoq_handle_t handle, const int8_t *x, int n, 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     count_launches(h, 1);
     ProfScope prof(h, EOQ_PROF_GLUE, s);
-    return record(h, launch_maxpool_fwd(x, n, hh, ww, c, k, stride, pad, y, arg, h->sm_count, s));
+    return record(h, launch_maxpool_fwd(x, n, hh, ww, c, k, stride, pad, y, arg, s));
 }
 
 extern "C" int eoq_aux_maxpool_bwd(eoq_handle_t handle, const int8_t *e, const int32_t *e_exp, const uint8_t *arg, int n, int hh,

@@ -1,6 +1,6 @@
 // Glue between the quantized convolution units of a Fixup residual network (arXiv 2105.13890, Sec. 3.2.1 chains the
-// units: x0 of a layer is x5 of the one before, e0 the error its successor hands back): max-pooling on int8 codes, the
-// exact join of two error streams followed by Q_e, and the update of the scalar parameters (Sec. 3.2.3) on their 16-bit
+// units: x0 of a layer is x5 of the one before, e0 the error its successor hands back): the exact join of two error streams
+// followed by Q_e, and the update of the scalar parameters (Sec. 3.2.3) on their 16-bit
 // range.  All of it is bandwidth- or latency-bound support work; none of it touches the tensor cores.
 #include "eoq_cells.cuh"
 #include "eoq_device.cuh"
@@ -23,192 +23,6 @@ inline int blocks_for(size_t items, int sm_count, int per_sm = 8)
     size_t b = (items + kThreads - 1) / kThreads, cap = (size_t)sm_count * per_sm;
     if (b > cap) b = cap;
     return b < 1 ? 1 : (int)b;
-}
-
-// ------------------------------------------------------------------ pooling
-
-// One thread per 16 channels of an output pixel.  arg = kh * k + kw of the first maximum in scan order.
-__global__ void maxpool_fwd_kernel(const int8_t *__restrict__ x, int n, int h, int w, int c, int k, int s, int p, int ho, int wo,
-                                   int8_t *__restrict__ y, uint8_t *__restrict__ arg)
-{
-    const int groups = c / 16;
-    const size_t items = (size_t)n * ho * wo * groups;
-    // (the launcher keeps the item count below 2^32: 64-bit divisions would dominate the work of an item)
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (size_t)gridDim.x * blockDim.x) {
-        const uint32_t i32 = (uint32_t)i, pix = i32 / (uint32_t)groups, row = pix / (uint32_t)wo;
-        const int g = (int)(i32 - pix * (uint32_t)groups), ox = (int)(pix - row * (uint32_t)wo);
-        const int b = (int)(row / (uint32_t)ho), oy = (int)(row - (uint32_t)b * (uint32_t)ho);
-        int best[16], at[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) { best[q] = -1000; at[q] = 0; }
-        for (int kh = 0; kh < k; ++kh) {
-            const int iy = oy * s + kh - p;
-            if (iy < 0 || iy >= h) continue;
-            for (int kw = 0; kw < k; ++kw) {
-                const int ix = ox * s + kw - p;
-                if (ix < 0 || ix >= w) continue;
-                const int4 v = __ldg(reinterpret_cast<const int4 *>(x + (((size_t)b * h + iy) * w + ix) * c + g * 16));
-                const int8_t *e = reinterpret_cast<const int8_t *>(&v);
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    if ((int)e[q] > best[q]) { best[q] = e[q]; at[q] = kh * k + kw; }
-            }
-        }
-        reinterpret_cast<int4 *>(y)[i] = make_int4((int)pack4(best[0], best[1], best[2], best[3]), (int)pack4(best[4], best[5], best[6], best[7]),
-                                                    (int)pack4(best[8], best[9], best[10], best[11]), (int)pack4(best[12], best[13], best[14], best[15]));
-        reinterpret_cast<int4 *>(arg)[i] = make_int4((int)pack4(at[0], at[1], at[2], at[3]), (int)pack4(at[4], at[5], at[6], at[7]),
-                                                      (int)pack4(at[8], at[9], at[10], at[11]), (int)pack4(at[12], at[13], at[14], at[15]));
-    }
-}
-
-// Backward: every output error code is added at the input position its window elected; the exact sums are then
-// coded with Q_e, which needs their maximum over the whole tensor first.  So the kernel runs twice: pass 0 reduces
-// max |sum| into the handle's cell, pass 1 forms the sums again and codes them (no intermediate tensor is written).
-// One thread per 16 channels of an input position gathers from the windows that cover it (at most
-// ceil(k / stride)^2): a window's 16 codes count where its recorded position equals this one.  Four codes are
-// handled per 32-bit word: bytes are compared at once, the chosen codes are kept with an offset of 128 (others as
-// 128 itself) so that they add as unsigned halves of two words without carries between them.
-//
-// kNext: the consumer's error head rides along (the layer in front of the pool: e1 = e_in * [x4 > 0],
-// e3 = Q_e(gamma * e1), sum of e1).  Coding is monotonic in |sum|, so max |e1| is the code of the largest masked
-// |sum|: pass 0 reduces that second maximum as well (into the 64-bit cell), and pass 1 knows both scales, writes
-// e_in (optional) and e3 and adds up e1 - the two kernels of a separate error head and their pass over e_in are gone.
-template <int kPass, bool kNext>
-__global__ void __launch_bounds__(kThreads)
-maxpool_bwd_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, const uint8_t *__restrict__ arg, int n, int h, int w, int c,
-                   int k, int s, int p, int ho, int wo, int8_t *__restrict__ e_in, int32_t *e_in_exp,
-                   const uint8_t *__restrict__ next_mask, const int32_t *next_gamma, int8_t *__restrict__ e3, int32_t *e3_exp,
-                   long long *sum_e1, DeviceState *dev)
-{
-    const int groups = c / 16;
-    const uint32_t items = (uint32_t)n * h * w * groups;   // below 2^31 (checked by the caller), so i + stride cannot wrap
-    int t = 7;
-    NextHead nh = {};
-    if (kPass == 1) {
-        const uint32_t M = dev->absmax_u32;
-        t = M ? round_log2_u32(M) : 7;
-        const int p_in = *e_exp;
-        const int p0 = M ? p_in + t - 7 : p_in;
-        if (kNext) nh = next_head_setup(next_gamma, (uint32_t)abs(sq_code32((int32_t)dev->absmax_u64, t)), dev);
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            if (e_in_exp) *e_in_exp = p0;
-            if (!M) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-            if (kNext) next_head_exponent(nh, p0, e3_exp, dev);
-        }
-    }
-    uint32_t mx = 0, mx_masked = 0;
-    int s1 = 0;
-    long long s1_total = 0;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < items; i += gridDim.x * blockDim.x) {
-        const uint32_t pix = i / (uint32_t)groups, row = pix / (uint32_t)w;
-        const int gi = (int)(i - pix * (uint32_t)groups), ix = (int)(pix - row * (uint32_t)w);
-        const int b = (int)(row / (uint32_t)h), iy = (int)(row - (uint32_t)b * (uint32_t)h);
-        // windows o with o * s - p <= i <= o * s - p + k - 1
-        const int oy_lo = max(0, (iy + p - k + s) / s), oy_hi = min(ho - 1, (iy + p) / s);
-        const int ox_lo = max(0, (ix + p - k + s) / s), ox_hi = min(wo - 1, (ix + p) / s);
-        uint32_t even[4] = {0, 0, 0, 0}, odd[4] = {0, 0, 0, 0};
-        int nwin = 0;
-        auto take = [&](const int4 &ev, const int4 &av, int oy, int ox) {
-            const uint32_t me = (uint32_t)((iy - (oy * s - p)) * k + (ix - (ox * s - p))) * 0x01010101u;
-            const uint32_t ew[4] = {(uint32_t)ev.x, (uint32_t)ev.y, (uint32_t)ev.z, (uint32_t)ev.w};
-            const uint32_t aw[4] = {(uint32_t)av.x, (uint32_t)av.y, (uint32_t)av.z, (uint32_t)av.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t hit = __vcmpeq4(aw[q], me);           // 0xff in the bytes this position won
-                const uint32_t v = (ew[q] & hit) ^ 0x80808080u;      // code + 128 there, 128 elsewhere
-                even[q] += v & 0x00ff00ffu;
-                odd[q] += (v >> 8) & 0x00ff00ffu;
-            }
-            ++nwin;
-        };
-        if (oy_hi - oy_lo <= 1 && ox_hi - ox_lo <= 1) {
-            // the usual case (window at most twice the stride): at most 2 x 2 windows, all eight loads issued together
-            int4 ev[4], av[4];
-            bool in[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int oy = oy_lo + (u >> 1), ox = ox_lo + (u & 1);
-                in[u] = oy <= oy_hi && ox <= ox_hi;
-                const size_t o = (((size_t)b * ho + oy) * wo + ox) * c + gi * 16;
-                ev[u] = in[u] ? __ldg(reinterpret_cast<const int4 *>(e + o)) : make_int4(0, 0, 0, 0);
-                av[u] = in[u] ? __ldg(reinterpret_cast<const int4 *>(arg + o)) : make_int4(0, 0, 0, 0);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (in[u]) take(ev[u], av[u], oy_lo + (u >> 1), ox_lo + (u & 1));
-        } else {
-            for (int oy = oy_lo; oy <= oy_hi; ++oy)
-                for (int ox = ox_lo; ox <= ox_hi; ++ox) {
-                    const size_t o = (((size_t)b * ho + oy) * wo + ox) * c + gi * 16;
-                    take(__ldg(reinterpret_cast<const int4 *>(e + o)), __ldg(reinterpret_cast<const int4 *>(arg + o)), oy, ox);
-                }
-        }
-        int sum[16];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            sum[4 * q + 0] = (int)(even[q] & 0xffffu) - 128 * nwin;
-            sum[4 * q + 1] = (int)(odd[q] & 0xffffu) - 128 * nwin;
-            sum[4 * q + 2] = (int)(even[q] >> 16) - 128 * nwin;
-            sum[4 * q + 3] = (int)(odd[q] >> 16) - 128 * nwin;
-        }
-        const uint32_t mbits = kNext ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(next_mask) + i) : 0u;
-        if (kPass == 0) {
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const uint32_t v = (uint32_t)abs(sum[q]);
-                mx = max(mx, v);
-                if (kNext && ((mbits >> q) & 1u)) mx_masked = max(mx_masked, v);
-            }
-        } else {
-            int cd[16];
-            if (t >= 8) {   // a right shift by t - 7 >= 1 (sums are below 2^15, nothing can wrap)
-                const int sh = t - 7, half_m1 = (1 << (sh - 1)) - 1;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) cd[q] = sq_code32_shr(sum[q], sh, half_m1);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 16; ++q) cd[q] = sq_code32(sum[q], t);
-            }
-            if (e_in)
-                reinterpret_cast<int4 *>(e_in)[i] =
-                    make_int4((int)pack4(cd[0], cd[1], cd[2], cd[3]), (int)pack4(cd[4], cd[5], cd[6], cd[7]),
-                              (int)pack4(cd[8], cd[9], cd[10], cd[11]), (int)pack4(cd[12], cd[13], cd[14], cd[15]));
-            if (kNext) {
-                int c3[16];
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const int e1 = ((mbits >> q) & 1u) ? cd[q] : 0;
-                    s1 += e1;
-                    c3[q] = next_head_code(nh, e1);
-                }
-                reinterpret_cast<int4 *>(e3)[i] =
-                    make_int4((int)pack4(c3[0], c3[1], c3[2], c3[3]), (int)pack4(c3[4], c3[5], c3[6], c3[7]),
-                              (int)pack4(c3[8], c3[9], c3[10], c3[11]), (int)pack4(c3[12], c3[13], c3[14], c3[15]));
-                s1_total += s1;
-                s1 = 0;
-            }
-        }
-    }
-    if (kPass == 0) {
-        mx = (uint32_t)block_max_u64(mx);
-        if (kNext) mx_masked = (uint32_t)block_max_u64(mx_masked);
-        if (threadIdx.x == 0) {
-            if (mx) atomicMax(&dev->absmax_u32, mx);
-            if (kNext && mx_masked) atomicMax(&dev->absmax_u64, (unsigned long long)mx_masked);
-        }
-    } else {
-        if (kNext && sum_e1) {
-            s1_total = block_sum_i64(s1_total);
-            if (threadIdx.x == 0 && s1_total) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)s1_total);
-        }
-        if (last_block_done(dev)) {
-            dev->absmax_u32 = 0;
-            if (kNext) {
-                dev->absmax_u64 = 0;
-                if (sum_e1) *sum_e1 = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum0), 0ull);
-            }
-        }
-    }
 }
 
 // ------------------------------------------------------------------ join of two error streams + Q_e
@@ -408,39 +222,6 @@ __global__ void scalar_update_kernel(const __grid_constant__ ScalarBatch b, int3
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
-
-cudaError_t launch_maxpool_fwd(const int8_t *x, int n, int h, int w, int c, int k, int s, int p, int8_t *y, uint8_t *arg,
-                               int sm_count, cudaStream_t st)
-{
-    const int ho = (h + 2 * p - k) / s + 1, wo = (w + 2 * p - k) / s + 1;
-    maxpool_fwd_kernel<<<blocks_for((size_t)n * ho * wo * (c / 16), sm_count), kThreads, 0, st>>>(x, n, h, w, c, k, s, p, ho, wo, y, arg);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_maxpool_bwd(const int8_t *e, const int32_t *e_exp, const uint8_t *arg, int n, int h, int w, int c, int k, int s,
-                               int p, int8_t *e_in, int32_t *e_in_exp, const uint8_t *next_mask, const int32_t *next_gamma, int8_t *e3,
-                               int32_t *e3_exp, long long *sum_e1, DeviceState *dev, int sm_count, cudaStream_t st,
-                               const ReduceHook &hook)
-{
-    const int ho = (h + 2 * p - k) / s + 1, wo = (w + 2 * p - k) / s + 1;
-    const int blocks = blocks_for((size_t)n * h * w * (c / 16), sm_count, 32);
-    if (e3) {
-        maxpool_bwd_kernel<0, true><<<blocks, kThreads, 0, st>>>(e, e_exp, arg, n, h, w, c, k, s, p, ho, wo, e_in, e_in_exp, next_mask,
-                                                                 next_gamma, e3, e3_exp, sum_e1, dev);
-        hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, st);
-        hook(&dev->absmax_u64, 1, EOQ_REDUCE_I64, EOQ_REDUCE_MAX, st);
-        maxpool_bwd_kernel<1, true><<<blocks, kThreads, 0, st>>>(e, e_exp, arg, n, h, w, c, k, s, p, ho, wo, e_in, e_in_exp, next_mask,
-                                                                 next_gamma, e3, e3_exp, sum_e1, dev);
-        if (sum_e1) hook(sum_e1, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, st);
-    } else {
-        maxpool_bwd_kernel<0, false><<<blocks, kThreads, 0, st>>>(e, e_exp, arg, n, h, w, c, k, s, p, ho, wo, e_in, e_in_exp, nullptr,
-                                                                  nullptr, nullptr, nullptr, nullptr, dev);
-        hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, st);
-        maxpool_bwd_kernel<1, false><<<blocks, kThreads, 0, st>>>(e, e_exp, arg, n, h, w, c, k, s, p, ho, wo, e_in, e_in_exp, nullptr,
-                                                                  nullptr, nullptr, nullptr, nullptr, dev);
-    }
-    return cudaGetLastError();
-}
 
 cudaError_t launch_join(const int8_t *a, const int32_t *a_exp, const int8_t *b, const int32_t *b_exp, const uint8_t *mask_b,
                         size_t n_el, int8_t *out, int32_t *out_exp, long long *sum_out, const uint8_t *next_mask,

@@ -327,7 +327,7 @@ cudaError_t launch_weight_prep(const PrepBatch &b, cudaStream_t s);
 // Network glue (eoq_aux.cu)
 // ---------------------------------------------------------------------------------------------
 cudaError_t launch_maxpool_fwd(const int8_t *x, int n, int h, int w, int c, int k, int s, int p, int8_t *y, uint8_t *arg,
-                               int sm_count, cudaStream_t st);
+                               cudaStream_t st);
 cudaError_t launch_maxpool_bwd(const int8_t *e, const int32_t *e_exp, const uint8_t *arg, int n, int h, int w, int c, int k, int s,
                                int p, int8_t *e_in, int32_t *e_in_exp, const uint8_t *next_mask, const int32_t *next_gamma, int8_t *e3,
                                int32_t *e3_exp, long long *sum_e1, DeviceState *dev, int sm_count, cudaStream_t st,
