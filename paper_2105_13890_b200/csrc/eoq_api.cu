@@ -1127,17 +1127,56 @@ extern "C" int eoq_conv_dgrad_head(eoq_handle_t handle, const eoq_conv_desc_t *d
 
 // ================================================================================= weight gradient
 
-// The b1 tap sums (one pass over e3), in front of the weight-gradient GEMM on the same stream.  (Issued on a second
-// stream "beside" the GEMM they gain nothing: a GEMM CTA fills its SM, so the blocks of this kernel only start as
-// the GEMM's CTAs leave, and the call pays for a fork and a join on top.)
-static cudaError_t launch_tap_sums(Handle *h, const int8_t *e3, long long *tap_sums, size_t tap_bytes,
-                                   const eoq_conv_desc_t &d, int ho, int wo, const BorderClasses &bc, cudaStream_t s)
+// The weight-gradient workspace: [tap sums][256 bytes with the maximum cell][int64 sums][split-K slices].
+struct WgradSpace {
+    long long *tap_sums;
+    size_t tap_stride;            // one copy of the tap sums, in elements
+    unsigned long long *max_cell;
+    size_t zero_bytes;            // tap sums and maximum cell: cleared by the GEMM kernel
+    long long *acc;
+    size_t acc_bytes;
+    int32_t *parts;
+};
+static WgradSpace wgrad_space(const eoq_conv_desc_t &d, const Geometry &g, void *workspace)
 {
-    const size_t tap_stride = tap_bytes / kTapReplicas / sizeof(long long);
-    count_launches(h, 1);
-    ProfScope prof(h, EOQ_PROF_WGRAD_TAPS, s);
-    cudaError_t e = cudaMemsetAsync(tap_sums, 0, tap_bytes, s);  // the kernel adds into them
-    return e != cudaSuccess ? e : launch_b1_error_sums(e3, tap_sums, tap_stride, d, ho, wo, bc, h->sm_count, s);
+    WgradSpace w;
+    char *ws = static_cast<char *>(workspace);
+    w.tap_stride = round256((size_t)d.c_out * g.taps * sizeof(long long)) / sizeof(long long);
+    const size_t tap_bytes = kTapReplicas * w.tap_stride * sizeof(long long);
+    w.tap_sums = reinterpret_cast<long long *>(ws);
+    w.max_cell = reinterpret_cast<unsigned long long *>(ws + tap_bytes);
+    w.zero_bytes = tap_bytes + 256;
+    w.acc = reinterpret_cast<long long *>(ws + w.zero_bytes);
+    w.acc_bytes = round256(g.w_elems * sizeof(long long));
+    w.parts = reinterpret_cast<int32_t *>(ws + w.zero_bytes + w.acc_bytes);
+    return w;
+}
+
+static FinishItem finish_item(const eoq_conv_desc_t &d, const Geometry &g, const WgradSpace &w, const int8_t *e3, const int32_t *e3_exp,
+                              int32_t b1_c, const int32_t *b1_dev, int8_t *gq, int32_t *g_exp, int num_parts)
+{
+    FinishItem it;
+    memset(&it, 0, sizeof(it));
+    it.e3 = e3;
+    it.e3_exp = e3_exp;
+    it.b1_dev = b1_dev;
+    it.b1_c = b1_c;
+    it.use_b1 = b1_dev != nullptr || b1_c != 0;   // a device-resident b1 may be anything: its term is always formed
+    it.tap_sums = w.tap_sums;
+    it.tap_stride = w.tap_stride;
+    it.max_cell = w.max_cell;
+    it.acc = w.acc;
+    it.num_parts = num_parts;
+    it.parts = num_parts > 0 ? w.parts : nullptr;
+    it.g = gq;
+    it.g_exp = g_exp;
+    it.n = g.w_elems;
+    it.pixels = (unsigned long long)d.n * g.ho * g.wo;
+    it.d = d;
+    it.bc = border_classes(d, g);
+    it.ho = g.ho;
+    it.wo = g.wo;
+    return it;
 }
 
 // Weight gradient behind eoq_conv_wgrad and eoq_conv_wgrad_dev: b1 is the host code b1_c, or the code at b1_dev.
@@ -1159,49 +1198,38 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     const eoq_conv_desc_t &d = *desc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
-    // workspace: [tap sums][256 spare bytes][int64 sums][split-K slices]
     const BorderClasses bc = border_classes(d, g);
-    const bool use_b1 = b1_dev != nullptr || b1_c != 0;  // a device-resident b1 may be anything: its term is always formed
+    const bool use_b1 = b1_dev != nullptr || b1_c != 0;
     if (use_b1 && bc.nrc * bc.ncc > kMaxBorderClasses) return EOQ_ERR_UNSUPPORTED;
-    char *ws = reinterpret_cast<char *>(workspace);
-    long long *tap_sums = reinterpret_cast<long long *>(ws);
-    const size_t tap_stride = round256((size_t)d.c_out * g.taps * sizeof(long long)) / sizeof(long long);  // one copy, in elements
-    const size_t tap_bytes = kTapReplicas * tap_stride * sizeof(long long);
-    long long *acc = reinterpret_cast<long long *>(ws + tap_bytes + 256);
-    const size_t acc_bytes = round256(g.w_elems * sizeof(long long));
+    const WgradSpace w = wgrad_space(d, g, workspace);
+    // behind the GEMM (whose kernel leaves sums as [oc][tap][ic], the layout of g)
+    auto finish = [&](int num_parts) -> int {
+        FinishItem it = finish_item(d, g, w, e3, e3_exp, b1_c, b1_dev, gq, g_exp, num_parts);
+        it.copy_out = reinterpret_cast<long long *>(acc_dump);
+        ProfScope prof_q(h, EOQ_PROF_WGRAD_AUX, s);
+        count_launches(h, finish_launches(&it, 1, h->hook));
+        return record(h, launch_wgrad_finish(&it, 1, &h->dev->status, h->sm_count, s, h->hook));
+    };
 
     WgradPatchPlan wp;
     if (plan_wgrad_patch(wp, d, g.ho, g.wo, h->gemm_ctas < kWgradTargetCtas ? h->gemm_ctas : kWgradTargetCtas)) {
-        wp.partials = reinterpret_cast<int32_t *>(ws + tap_bytes + 256 + acc_bytes);
+        wp.partials = w.parts;
+        wp.zero = reinterpret_cast<int4 *>(w.tap_sums);
+        wp.zero_n16 = (unsigned)(w.zero_bytes / 16);
         wp.dev = h->dev;
-        cudaError_t e;
-        if (gemm_only) {
-            CUtensorMap mx, me;
-            if (!make_patch_map(&mx, x, d.n, d.h, d.w, d.c_in, wp.kc, wp.pw, wp.r_rows + d.kh - 1) ||
-                !make_patch_map(&me, e3, d.n, g.ho, g.wo, d.c_out, wp.tile_n, wp.pw, wp.r_rows))
-                return EOQ_ERR_UNSUPPORTED;
-            count_launches(h, 1);
-            if (num_parts_out) *num_parts_out = wp.num_splits;
-            ProfScope prof(h, EOQ_PROF_WGRAD, s);
-            return record(h, launch_wgrad_patch(wp, mx, me, s));
-        }
-        e = use_b1 ? launch_tap_sums(h, e3, tap_sums, tap_bytes, d, g.ho, g.wo, bc, s) : cudaSuccess;
-        if (e != cudaSuccess) return record(h, e);
         CUtensorMap map_x, map_e;
         if (!make_patch_map(&map_x, x, d.n, d.h, d.w, d.c_in, wp.kc, wp.pw, wp.r_rows + d.kh - 1) ||
             !make_patch_map(&map_e, e3, d.n, g.ho, g.wo, d.c_out, wp.tile_n, wp.pw, wp.r_rows))
             return EOQ_ERR_UNSUPPORTED;
         count_launches(h, 1);
+        if (num_parts_out) *num_parts_out = wp.num_splits;
+        cudaError_t e;
         {
             ProfScope prof(h, EOQ_PROF_WGRAD, s);
             e = launch_wgrad_patch(wp, map_x, map_e, s);
         }
-        if (e != cudaSuccess) return record(h, e);
-        ProfScope prof_q(h, EOQ_PROF_WGRAD_AUX, s);
-        e = launch_sq_i64(acc, e3_exp, -7, g.w_elems, gq, g_exp, reinterpret_cast<long long *>(acc_dump),
-                          use_b1 ? tap_sums : nullptr, tap_stride, b1_c, b1_dev, d.c_in, wp.partials, wp.num_splits, h->dev, h->sm_count, s, h->hook);
-        count_launches(h, 2);
-        return record(h, e);
+        if (e != cudaSuccess || gemm_only) return record(h, e);
+        return finish(wp.num_splits);
     }
 
     WgradParams p;
@@ -1274,15 +1302,16 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.tap_dw[t] = (unsigned char)(t % d.kw);
         }
     }
-    p.acc = acc;
+    p.acc = w.acc;
+    p.zero = reinterpret_cast<int4 *>(w.tap_sums);
+    p.zero_n16 = (unsigned)(w.zero_bytes / 16);
     p.dev = h->dev;
 
     cudaError_t e = cudaSuccess;
     if (!h->gemm_only) {
         ProfScope aux(h, EOQ_PROF_WGRAD_AUX, s);
-        e = cudaMemsetAsync(acc, 0, acc_bytes, s);  // the GEMM adds into the int64 sums with atomics
+        e = cudaMemsetAsync(w.acc, 0, w.acc_bytes, s);  // the GEMM adds into the int64 sums with atomics
     }
-    if (e == cudaSuccess && use_b1 && !gemm_only) e = launch_tap_sums(h, e3, tap_sums, tap_bytes, d, g.ho, g.wo, bc, s);
     if (e != cudaSuccess) return record(h, e);
     CUtensorMap map_x, map_e;
     if (!make_matrix_map(&map_e, e3, (size_t)p.P, d.c_out, p.nc, p.pixels_per_stage)) return EOQ_ERR_UNSUPPORTED;
@@ -1298,12 +1327,7 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     }
     if (num_parts_out) *num_parts_out = 0;
     if (e != cudaSuccess || gemm_only) return record(h, e);
-    // the kernel leaves sums as [oc][tap][ic], which is the layout of g
-    ProfScope prof_q(h, EOQ_PROF_WGRAD_AUX, s);
-    e = launch_sq_i64(acc, e3_exp, -7, g.w_elems, gq, g_exp, reinterpret_cast<long long *>(acc_dump),
-                      use_b1 ? tap_sums : nullptr, tap_stride, b1_c, b1_dev, d.c_in, nullptr, 0, h->dev, h->sm_count, s, h->hook);
-    count_launches(h, 2);
-    return record(h, e);
+    return finish(0);
 }
 
 extern "C" int eoq_conv_wgrad(eoq_handle_t handle, const eoq_conv_desc_t *desc, const int8_t *e3,
@@ -1349,45 +1373,18 @@ extern "C" int eoq_wgrad_finish(eoq_handle_t handle, int num, const eoq_conv_des
         if (b1_c[i] && bc.nrc * bc.ncc > kMaxBorderClasses) return EOQ_ERR_UNSUPPORTED;
     }
     for (int base = 0; base < num; base += kFinishChunk) {
-        FinishBatch b;
-        memset(&b, 0, sizeof(b));
-        b.num = num - base < kFinishChunk ? num - base : kFinishChunk;
-        for (int k = 0; k < b.num; ++k) {
+        FinishItem items[kFinishChunk];
+        const int count = num - base < kFinishChunk ? num - base : kFinishChunk;
+        for (int k = 0; k < count; ++k) {
             const eoq_conv_desc_t &d = descs[base + k];
             Geometry g;
             check_desc(&d, &g);
-            FinishItem &it = b.item[k];
-            // the workspace as eoq_conv_wgrad_gemm laid it out: [tap sums][256 spare bytes][int64 sums][split-K slices]
-            char *ws = reinterpret_cast<char *>(workspace[base + k]);
-            const size_t tap_stride = round256((size_t)d.c_out * g.taps * sizeof(long long)) / sizeof(long long);
-            const size_t tap_bytes = kTapReplicas * tap_stride * sizeof(long long);
-            const size_t acc_bytes = round256(g.w_elems * sizeof(long long));
-            it.e3 = e3[base + k];
-            it.e3_exp = e3_exp[base + k];
-            it.b1_dev = b1_c[base + k];
-            it.tap_sums = reinterpret_cast<long long *>(ws);
-            it.tap_stride = tap_stride;
-            it.zero_bytes = tap_bytes + 256;
-            it.max_cell = reinterpret_cast<unsigned long long *>(ws + tap_bytes);
-            it.acc = reinterpret_cast<long long *>(ws + tap_bytes + 256);
-            it.num_parts = num_parts[base + k];
-            it.parts = it.num_parts > 0 ? reinterpret_cast<const int32_t *>(ws + tap_bytes + 256 + acc_bytes) : nullptr;
-            it.g = gq[base + k];
-            it.g_exp = g_exp[base + k];
-            it.n = g.w_elems;
-            it.pixels = (unsigned long long)d.n * g.ho * g.wo;
-            it.d = d;
-            it.bc = border_classes(d, g);
-            it.ho = g.ho;
-            it.wo = g.wo;
-            plan_finish_item(it, h->sm_count);
-            b.tap_first[k + 1] = b.tap_first[k] + it.tap_grid_x * it.tap_grid_y;
-            b.fin_first[k + 1] = b.fin_first[k] + it.fin_blocks;
-            b.sq_first[k + 1] = b.sq_first[k] + it.sq_blocks;
+            items[k] = finish_item(d, g, wgrad_space(d, g, workspace[base + k]), e3[base + k], e3_exp[base + k], 0, b1_c[base + k],
+                                   gq[base + k], g_exp[base + k], num_parts[base + k]);
         }
         ProfScope prof(h, EOQ_PROF_WGRAD_AUX, s);
-        const cudaError_t e = launch_wgrad_finish(b, &h->dev->status, s);
-        count_launches(h, 4);
+        count_launches(h, finish_launches(items, count, h->hook));
+        const cudaError_t e = launch_wgrad_finish(items, count, &h->dev->status, h->sm_count, s, h->hook);
         if (e != cudaSuccess) return record(h, e);
     }
     return EOQ_OK;

@@ -504,117 +504,6 @@ __global__ void sq_i32_scatter_kernel(const int32_t *__restrict__ src, const int
     }
 }
 
-// ------------------------------------------------------------------ int64 -> SQ (Q_g after the weight gradient)
-
-// Last step before Q_g: sums the int32 split-K slices of the patch kernel into int64 (exact whatever the reduction
-// length), or takes the int64 sums the other kernel left in `acc`; adds the b1 term of x1 = x0 + b1 (b1 times the
-// sum of the error over the pixels whose tap falls inside the image); optionally copies the exact sums out; and
-// reduces max |.|.  A block of 256 threads is (256 / groups) elements x `groups` slice groups: every thread adds
-// its share of the slices with independent, coalesced loads and the groups meet in shared memory.
-// (bx of nblocks): the block's place among the blocks of its tensor; max_cell: where max |.| is reduced (null: not at all)
-__device__ __forceinline__ void wgrad_finalize_body(const int32_t *__restrict__ parts, int num_parts, int groups, size_t n, long long *acc,
-                                                    const long long *__restrict__ tap_sums, size_t replica_stride, int32_t b1_c,
-                                                    const int32_t *b1_dev, int c_in, long long *copy_out,
-                                                    unsigned long long *max_cell, int bx, int nblocks)
-{
-    __shared__ long long part[256];
-    if (b1_dev) b1_c = clampi(__ldg(b1_dev), -32768, 32767);
-    const int bw = 256 / groups, tx = threadIdx.x % bw, ty = threadIdx.x / bw;
-    unsigned long long mx = 0;
-    for (size_t base = (size_t)bx * bw; base < n; base += (size_t)nblocks * bw) {
-        const size_t i = base + tx;
-        long long v = 0;
-        if (parts) {
-            if (i < n) {
-                // four slices per round: their loads are independent and in flight together
-                int s = ty;
-                for (; s + 3 * groups < num_parts; s += 4 * groups) {
-                    const int32_t a0 = __ldg(parts + (size_t)s * n + i), a1 = __ldg(parts + (size_t)(s + groups) * n + i);
-                    const int32_t a2 = __ldg(parts + (size_t)(s + 2 * groups) * n + i), a3 = __ldg(parts + (size_t)(s + 3 * groups) * n + i);
-                    v += ((long long)a0 + a1) + ((long long)a2 + a3);
-                }
-                for (; s < num_parts; s += groups) v += (long long)__ldg(parts + (size_t)s * n + i);
-            }
-            if (groups > 1) {
-                part[threadIdx.x] = v;
-                __syncthreads();
-                if (ty == 0) {
-                    v = 0;
-                    for (int k = 0; k < groups; ++k) v += part[k * bw + tx];
-                }
-                __syncthreads();
-            }
-        } else if (i < n) {
-            v = acc[i];
-        }
-        if (ty == 0 && i < n) {
-            if (tap_sums) {  // index of (oc, tap); a 32-bit division whenever the tensor allows it
-                const long long *t = tap_sums + (n <= 0xffffffffull ? (size_t)((uint32_t)i / (uint32_t)c_in) : i / (size_t)c_in);
-                long long ts = 0;
-#pragma unroll
-                for (int r = 0; r < kTapReplicas; ++r) ts += __ldg(t + (size_t)r * replica_stride);
-                v += (long long)b1_c * ts;
-            }
-            if (parts || tap_sums) acc[i] = v;
-            if (copy_out) copy_out[i] = v;
-            const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
-            mx = a > mx ? a : mx;
-        }
-    }
-    mx = block_max_u64(mx);
-    if (threadIdx.x == 0 && mx && max_cell) atomicMax(max_cell, mx);
-}
-
-__global__ void wgrad_finalize_kernel(const int32_t *__restrict__ parts, int num_parts, int groups, size_t n, long long *acc,
-                                      const long long *__restrict__ tap_sums, size_t replica_stride, int32_t b1_c,
-                                      const int32_t *b1_dev, int c_in, long long *copy_out, DeviceState *dev, int sums_only)
-{
-    // sums_only: the sums are completed elsewhere (an all-reduce over replicas) before their maximum is taken
-    wgrad_finalize_body(parts, num_parts, groups, n, acc, tap_sums, replica_stride, b1_c, b1_dev, c_in, copy_out,
-                        sums_only ? nullptr : &dev->absmax_u64, (int)blockIdx.x, (int)gridDim.x);
-}
-
-// max |.| of int64 sums into the handle's 64-bit cell (used when the sums were completed by an all-reduce)
-__global__ void absmax_i64_kernel(const long long *__restrict__ src, size_t n, DeviceState *dev)
-{
-    unsigned long long mx = 0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const long long v = src[i];
-        const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
-        mx = a > mx ? a : mx;
-    }
-    mx = block_max_u64(mx);
-    if (threadIdx.x == 0 && mx) atomicMax(&dev->absmax_u64, mx);
-}
-
-// (bx of nblocks) as above; M: the tensor's max |.|; status: where a zero tensor is flagged
-__device__ __forceinline__ void sq_i64_body(const long long *__restrict__ src, const int32_t *src_exp, int exp_bias, size_t n, int8_t *dst,
-                                            int32_t *dst_exp, unsigned long long M, unsigned *status, int bx, int nblocks)
-{
-    const int t = M ? round_log2_u64(M) : 7;
-    if (bx == 0 && threadIdx.x == 0) {
-        const int p_in = (src_exp ? *src_exp : 0) + exp_bias;
-        *dst_exp = M ? p_in + t - 7 : p_in;
-        if (!M) atomicOr(status, EOQ_DEV_SQ_ZERO);
-    }
-    // four codes per thread and round (one 32-bit store); n is a multiple of 4 for every weight tensor with padded channels
-    const size_t n4 = n / 4;
-    for (size_t i = (size_t)bx * blockDim.x + threadIdx.x; i < n4; i += (size_t)nblocks * blockDim.x) {
-        const longlong2 a = __ldg(reinterpret_cast<const longlong2 *>(src) + 2 * i);
-        const longlong2 b = __ldg(reinterpret_cast<const longlong2 *>(src) + 2 * i + 1);
-        reinterpret_cast<uint32_t *>(dst)[i] = pack4(sq_code64(a.x, t), sq_code64(a.y, t), sq_code64(b.x, t), sq_code64(b.y, t));
-    }
-    for (size_t i = n4 * 4 + (size_t)bx * blockDim.x + threadIdx.x; i < n; i += (size_t)nblocks * blockDim.x)
-        dst[i] = (int8_t)sq_code64(src[i], t);
-}
-
-__global__ void sq_i64_kernel(const long long *__restrict__ src, const int32_t *src_exp, int exp_bias, size_t n,
-                              int8_t *dst, int32_t *dst_exp, DeviceState *dev)
-{
-    sq_i64_body(src, src_exp, exp_bias, n, dst, dst_exp, dev->absmax_u64, &dev->status, (int)blockIdx.x, (int)gridDim.x);
-    if (last_block_done(dev)) dev->absmax_u64 = 0;
-}
-
 // ------------------------------------------------------------------ head of the error chain
 
 // Pass 1: max |e1| and the sums behind g_b2 and g_gamma, with e1 = e0 * [x4 > 0].
@@ -1003,168 +892,6 @@ __global__ void weight_prep_kernel(const __grid_constant__ PrepBatch b)
     }
 }
 
-// tap_sums[oc][tap] += sum of e3[n,y,x,oc] over the pixels for which the tap falls inside the image (the weight
-// gradient adds b1 times this to every input channel).  Pixels are summed per border class first (the taps inside
-// the image are the same for all pixels of a class).  A block owns a range of
-// pixels and a slab of channels; a lane keeps 16 channels (one 128-bit load per pixel), so a warp covers
-// 32 / (slab / 16) pixels per step.  Interior pixels (one class, almost all of a large image) accumulate in
-// registers, border pixels in shared memory.
-constexpr int kClassSlab = 128;
-constexpr int kTapUnroll = 8;
-// (bx, by): the block's place in the grid of its layer (pixel range, channel slab)
-__device__ __forceinline__ void b1_tap_sums_body(const int8_t *__restrict__ e3, long long *tap_sums, size_t replica_stride, int c_out,
-                                                 int ho, int wo, size_t pixels, int pixels_per_block, const BorderClasses &bc,
-                                                 const eoq_conv_desc_t &d, int bx, int by)
-{
-    // the blocks spread their atomics over kTapReplicas copies of the sums (the consumer adds the copies): all
-    // cells of one copy sit in a few kilobytes, i.e. behind one or two L2 slices, whose atomic rate bounds this kernel
-    tap_sums += (size_t)(bx % kTapReplicas) * replica_stride;
-    extern __shared__ int32_t cls_acc[];  // [classes][kClassSlab]
-    const int classes = bc.nrc * bc.ncc;
-    for (int i = threadIdx.x; i < classes * kClassSlab; i += blockDim.x) cls_acc[i] = 0;
-    __syncthreads();
-    const int slab_ch = min(kClassSlab, c_out - by * kClassSlab);  // channels of this slab (multiple of 16)
-    const int lanes_per_pix = slab_ch / 16;
-    const int pix_per_step = blockDim.x / lanes_per_pix;
-    const int sub = threadIdx.x % lanes_per_pix, slot = threadIdx.x / lanes_per_pix;
-    const int ch = by * kClassSlab + sub * 16;
-    const int interior = (bc.nrc != ho && bc.ncc != wo) ? bc.nlo_h * bc.ncc + bc.nlo_w : -1;
-    int acc[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) acc[k] = 0;
-    const size_t begin = (size_t)bx * pixels_per_block;
-    const size_t end = min(pixels, begin + (size_t)pixels_per_block);
-    const bool small = pixels <= 0xffffffffull;
-    if (slot < pix_per_step) {
-        // kTapUnroll pixels per round: their loads are issued together and are in flight side by side
-        for (size_t p0 = begin + slot; p0 < end; p0 += kTapUnroll * (size_t)pix_per_step) {
-            int4 v[kTapUnroll];
-            int cls[kTapUnroll];
-#pragma unroll
-            for (int u = 0; u < kTapUnroll; ++u) {
-                const size_t p = p0 + (size_t)u * pix_per_step;
-                cls[u] = -2;  // beyond the block's range
-                v[u] = make_int4(0, 0, 0, 0);
-                if (p < end) {
-                    int x, y;
-                    if (small) {  // 32-bit index arithmetic (a 64-bit division costs more than the rest of the pixel's work)
-                        const uint32_t q = (uint32_t)p / (uint32_t)wo;
-                        x = (int)((uint32_t)p - q * (uint32_t)wo);
-                        y = (int)(q % (uint32_t)ho);
-                    } else {
-                        x = (int)(p % wo);
-                        y = (int)((p / wo) % ho);
-                    }
-                    cls[u] = border_class(y, ho, bc.nlo_h, bc.nhi_h, bc.nrc) * bc.ncc + border_class(x, wo, bc.nlo_w, bc.nhi_w, bc.ncc);
-                    v[u] = __ldg(reinterpret_cast<const int4 *>(e3 + p * c_out + ch));
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kTapUnroll; ++u) {
-                if (cls[u] == -2) continue;
-                const int8_t *b = reinterpret_cast<const int8_t *>(&v[u]);
-                if (cls[u] == interior) {
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) acc[k] += b[k];
-                } else {
-                    int32_t *dst = cls_acc + cls[u] * kClassSlab + sub * 16;
-#pragma unroll
-                    for (int k = 0; k < 16; ++k)
-                        if (b[k]) atomicAdd(dst + k, (int)b[k]);
-                }
-            }
-        }
-        if (interior >= 0) {
-            int32_t *dst = cls_acc + interior * kClassSlab + sub * 16;
-#pragma unroll
-            for (int k = 0; k < 16; ++k)
-                if (acc[k]) atomicAdd(dst + k, acc[k]);
-        }
-    }
-    __syncthreads();
-    // a tap's sum is the sum over the classes for which the tap falls inside the image: formed here from the
-    // block's class sums, one 64-bit atomic per (channel, tap) and block
-    const int taps = d.kh * d.kw;
-    __shared__ unsigned long long rows_in[32], cols_in[32];  // per filter row / column: the classes it is inside for
-    if (threadIdx.x < d.kh) {
-        unsigned long long m = 0;
-        for (int rc = 0; rc < bc.nrc; ++rc)
-            if (tap_valid(rc, threadIdx.x, ho, d.h, bc.nlo_h, bc.nhi_h, bc.nrc, d.stride, d.pad)) m |= 1ull << rc;
-        rows_in[threadIdx.x] = m;
-    } else if (threadIdx.x >= 32 && threadIdx.x < 32 + d.kw) {
-        unsigned long long m = 0;
-        for (int cc = 0; cc < bc.ncc; ++cc)
-            if (tap_valid(cc, threadIdx.x - 32, wo, d.w, bc.nlo_w, bc.nhi_w, bc.ncc, d.stride, d.pad)) m |= 1ull << cc;
-        cols_in[threadIdx.x - 32] = m;
-    }
-    __syncthreads();
-    // consecutive threads take consecutive taps of a channel: neighbouring cells of tap_sums[oc][tap]
-    for (int i = threadIdx.x; i < taps * slab_ch; i += blockDim.x) {
-        const int c = i / taps, tap = i % taps;
-        const unsigned long long cols = cols_in[tap % d.kw];
-        long long sum = 0;
-        for (unsigned long long rm = rows_in[tap / d.kw]; rm; rm &= rm - 1) {
-            const int32_t *row = cls_acc + (__ffsll((long long)rm) - 1) * bc.ncc * kClassSlab + c;
-            for (unsigned long long cm = cols; cm; cm &= cm - 1) sum += row[(__ffsll((long long)cm) - 1) * kClassSlab];
-        }
-        if (sum)
-            atomicAdd(reinterpret_cast<unsigned long long *>(tap_sums + (size_t)(by * kClassSlab + c) * taps + tap),
-                      (unsigned long long)sum);
-    }
-}
-
-
-__global__ void b1_tap_sums_kernel(const int8_t *__restrict__ e3, long long *tap_sums, size_t replica_stride, int c_out, int ho,
-                                   int wo, size_t pixels, int pixels_per_block, BorderClasses bc, eoq_conv_desc_t d)
-{
-    b1_tap_sums_body(e3, tap_sums, replica_stride, c_out, ho, wo, pixels, pixels_per_block, bc, d, (int)blockIdx.x, (int)blockIdx.y);
-}
-
-// ------------------------------------------------------------------ weight-gradient finish of many layers at once
-// A block finds the layer it works for by its index (first[] holds the first block of every item).
-__device__ __forceinline__ int finish_item_of(const int *first, int num, int block)
-{
-    int k = 0;
-    while (k + 1 < num && block >= first[k + 1]) ++k;
-    return k;
-}
-
-// zeroes what the finish accumulates into: the tap sums of every layer and its maximum cell (one block per layer)
-__global__ void finish_zero_kernel(FinishBatch b)
-{
-    const FinishItem &it = b.item[blockIdx.x];
-    int4 *dst = reinterpret_cast<int4 *>(it.tap_sums);
-    const size_t n16 = it.zero_bytes / 16;
-    for (size_t i = threadIdx.x; i < n16; i += blockDim.x) dst[i] = make_int4(0, 0, 0, 0);
-}
-
-__global__ void finish_taps_kernel(FinishBatch b)
-{
-    const int k = finish_item_of(b.tap_first, b.num, (int)blockIdx.x);
-    const FinishItem &it = b.item[k];
-    if (!it.b1_dev) return;
-    const int local = (int)blockIdx.x - b.tap_first[k];
-    b1_tap_sums_body(it.e3, it.tap_sums, (size_t)it.tap_stride, it.d.c_out, it.ho, it.wo, (size_t)it.pixels, it.pixels_per_block, it.bc,
-                     it.d, local % it.tap_grid_x, local / it.tap_grid_x);
-}
-
-__global__ void finish_sums_kernel(FinishBatch b)
-{
-    const int k = finish_item_of(b.fin_first, b.num, (int)blockIdx.x);
-    const FinishItem &it = b.item[k];
-    wgrad_finalize_body(it.parts, it.num_parts, it.groups, (size_t)it.n, it.acc, it.b1_dev ? it.tap_sums : nullptr,
-                        (size_t)it.tap_stride, 0, it.b1_dev, it.d.c_in, nullptr, it.max_cell, (int)blockIdx.x - b.fin_first[k],
-                        it.fin_blocks);
-}
-
-__global__ void finish_code_kernel(FinishBatch b, unsigned *status)
-{
-    const int k = finish_item_of(b.sq_first, b.num, (int)blockIdx.x);
-    const FinishItem &it = b.item[k];
-    sq_i64_body(it.acc, it.e3_exp, -7, (size_t)it.n, it.g, it.g_exp, *it.max_cell, status, (int)blockIdx.x - b.sq_first[k],
-                it.sq_blocks);
-}
-
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
@@ -1266,31 +993,6 @@ cudaError_t launch_sq_i32_scatter(const int32_t *src, const int32_t *src_exp, in
     return cudaGetLastError();
 }
 
-cudaError_t launch_sq_i64(const long long *src, const int32_t *src_exp, int exp_bias, size_t n, int8_t *dst,
-                          int32_t *dst_exp, long long *copy_out, const long long *tap_sums, size_t replica_stride,
-                          int32_t b1_c, const int32_t *b1_dev, int c_in, const int32_t *parts, int num_parts,
-                          DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook)
-{
-    const int groups = !parts ? 1 : (num_parts >= 32 ? 8 : (num_parts >= 8 ? 4 : 1));
-    const int bx = 256 / groups;
-    size_t blocks = (n + bx - 1) / bx;
-    if (blocks > (size_t)sm_count * 16) blocks = (size_t)sm_count * 16;
-    if (hook.fn) {
-        // replicas: local sums (b1 term included, it is linear in the error) -> all-reduce -> maximum of the global sums;
-        // the copy for the caller is taken from the global sums as well
-        wgrad_finalize_kernel<<<(unsigned)blocks, 256, 0, s>>>(parts, num_parts, groups, n, const_cast<long long *>(src), tap_sums,
-                                                               replica_stride, b1_c, b1_dev, c_in, nullptr, dev, 1);
-        hook(const_cast<long long *>(src), n, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
-        absmax_i64_kernel<<<grid_for(n, sm_count, 4), kThreads, 0, s>>>(src, n, dev);
-        if (copy_out) cudaMemcpyAsync(copy_out, src, n * sizeof(long long), cudaMemcpyDeviceToDevice, s);
-    } else {
-        wgrad_finalize_kernel<<<(unsigned)blocks, 256, 0, s>>>(parts, num_parts, groups, n, const_cast<long long *>(src), tap_sums,
-                                                               replica_stride, b1_c, b1_dev, c_in, copy_out, dev, 0);
-    }
-    sq_i64_kernel<<<grid_for(n, sm_count, 4), kThreads, 0, s>>>(src, src_exp, exp_bias, n, dst, dst_exp, dev);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_err_prescale(const int8_t *e0, const int32_t *e0_exp, const uint8_t *mask, const int16_t *x2,
                                 size_t n_el, int32_t gamma_c, const int32_t *gamma_dev, int8_t *e3, int32_t *e3_exp,
                                 long long *sum_e1, long long *sum_e1x2, DeviceState *dev, int sm_count, cudaStream_t s,
@@ -1367,65 +1069,6 @@ cudaError_t launch_b1_weight_table(const int8_t *w, int32_t *table, const eoq_co
 cudaError_t launch_weight_prep(const PrepBatch &b, cudaStream_t s)
 {
     weight_prep_kernel<<<b.first_block[b.num], 128, 0, s>>>(b);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_b1_error_sums(const int8_t *e3, long long *tap_sums, size_t replica_stride, const eoq_conv_desc_t &d, int ho,
-                                 int wo, const BorderClasses &bc, int sm_count, cudaStream_t s)
-{
-    // tap_sums was zeroed by the caller
-    const int classes = bc.nrc * bc.ncc;
-    const size_t pixels = (size_t)d.n * ho * wo;
-    const int slabs = (d.c_out + kClassSlab - 1) / kClassSlab;
-    int blocks = (sm_count + slabs - 1) / slabs;  // more blocks only add atomics on the per-tap cells
-    size_t ppb = (pixels + blocks - 1) / blocks;
-    if (ppb < 64) ppb = 64;
-    if (ppb > (1u << 23)) ppb = 1u << 23;  // keeps the int32 class sums exact
-    blocks = (int)((pixels + ppb - 1) / ppb);
-    dim3 grid(blocks, slabs);
-    b1_tap_sums_kernel<<<grid, 256, sizeof(int32_t) * classes * kClassSlab, s>>>(e3, tap_sums, replica_stride, d.c_out, ho, wo,
-                                                                               pixels, (int)ppb, bc, d);
-    return cudaGetLastError();
-}
-
-void plan_finish_item(FinishItem &it, int sm_count)
-{
-    // the b1 error sums: as launch_b1_error_sums lays them out
-    const int slabs = (it.d.c_out + kClassSlab - 1) / kClassSlab;
-    int blocks = (sm_count + slabs - 1) / slabs;
-    size_t ppb = ((size_t)it.pixels + blocks - 1) / blocks;
-    if (ppb < 64) ppb = 64;
-    if (ppb > (1u << 23)) ppb = 1u << 23;
-    it.pixels_per_block = (int)ppb;
-    it.tap_grid_x = (int)(((size_t)it.pixels + ppb - 1) / ppb);
-    it.tap_grid_y = slabs;
-    // slice sums and codes: as launch_sq_i64 sizes them, with a smaller cap (many tensors share the device)
-    it.groups = !it.parts ? 1 : (it.num_parts >= 32 ? 8 : (it.num_parts >= 8 ? 4 : 1));
-    const int bw = 256 / it.groups;
-    size_t fb = ((size_t)it.n + bw - 1) / bw;
-    if (fb > (size_t)sm_count * 4) fb = (size_t)sm_count * 4;
-    it.fin_blocks = (int)(fb < 1 ? 1 : fb);
-    size_t qb = ((size_t)it.n / 4 + kThreads - 1) / kThreads;
-    if (qb > (size_t)sm_count * 2) qb = (size_t)sm_count * 2;
-    it.sq_blocks = (int)(qb < 1 ? 1 : qb);
-}
-
-cudaError_t launch_wgrad_finish(const FinishBatch &b, unsigned *status, cudaStream_t s)
-{
-    int max_classes = 1;
-    for (int k = 0; k < b.num; ++k) {
-        const int c = b.item[k].bc.nrc * b.item[k].bc.ncc;
-        if (b.item[k].b1_dev && c > max_classes) max_classes = c;
-    }
-    const size_t smem = sizeof(int32_t) * max_classes * kClassSlab;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(finish_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    finish_zero_kernel<<<b.num, 256, 0, s>>>(b);
-    finish_taps_kernel<<<b.tap_first[b.num], 256, smem, s>>>(b);
-    finish_sums_kernel<<<b.fin_first[b.num], 256, 0, s>>>(b);
-    finish_code_kernel<<<b.sq_first[b.num], kThreads, 0, s>>>(b, status);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,499 @@
+// What follows the weight-gradient GEMM (arXiv 2105.13890, Sec. 3.2.1: g_w = Q_g(e3 * x1) with x1 = x0 + Q_b(b1)), for one
+// layer or for many layers in the same three launches: the b1 error sums (one pass over e3), the exact sums (split-K slices
+// or the GEMM's 64-bit sums, plus the b1 term) reduced to their maximum, and Q_g.  Blocks find their layer by their index.
+// The cells these kernels add into (tap sums, maximum) are cleared by the GEMM kernel in front.
+#include "eoq_device.cuh"
+#include "eoq_internal.h"
+
+namespace eoq {
+
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int kClassSlab = 128;   // channels one block of the error sums covers
+constexpr int kTapBytes = 32 * 1024;
+
+__device__ __forceinline__ int finish_item_of(const int *first, int num, int block)
+{
+    int k = 0;
+    while (k + 1 < num && block >= first[k + 1]) ++k;
+    return k;
+}
+
+__device__ __forceinline__ int finish_b1(const FinishItem &it)
+{
+    return it.b1_dev ? clampi(__ldg(it.b1_dev), -32768, 32767) : it.b1_c;
+}
+
+// Do the layer's sums fit 32 bits?  |G| <= pixels * 127 * (127 + |b1|).
+__device__ __forceinline__ bool finish_narrow(const FinishItem &it, int b1)
+{
+    return it.pixels < (1ull << 31) && (double)it.pixels * 127.0 * (127.0 + (double)abs(b1)) < 2147483647.0;
+}
+
+// ------------------------------------------------------------------ b1 error sums
+// tap_sums[oc][tap] += sum of e3[n,y,x,oc] over the pixels for which the tap falls inside the image (the weight gradient
+// adds b1 times this to every input channel).  Only border rows and columns ever fall outside a tap, so with T the sum over
+// all pixels, R_i and C_j those over the i-th border row and the j-th border column, and P_ij those over their crossings,
+//   tap sum = T - sum of R_i - sum of C_j + sum of P_ij   over the border rows and columns the tap does not take.
+// Every term is a plain sum over a regular set of pixels.  A block covers a range of rows and a slab of channels; a lane
+// keeps 16 channels (one 128-bit load per pixel, several in flight) in packed 16-bit halves (codes offset by 128, so that
+// no carry crosses; one instruction per code).  All warps sum T, then each takes its share of the border sets; the block
+// forms its tap sums in shared memory and adds each with one 64-bit atomic.
+// Bound by the latency of a few dependent rounds of loads.  With a border class and a 32-bit addition per byte the four
+// stages of ResNet-18 at batch 64 took 228 us (now 117 us, beside the backward chain), the 512-channel 7 x 7 layer alone
+// 11.1 us (8.8), the single 16-channel layer 5.3 us behind a memset (5.4 without one).
+struct PixelSum {
+    uint32_t even[4], odd[4];
+    int count;
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) even[q] = odd[q] = 0;
+        count = 0;
+    }
+    __device__ __forceinline__ void add(const int4 &v)
+    {
+        const uint32_t w[4] = {(uint32_t)v.x, (uint32_t)v.y, (uint32_t)v.z, (uint32_t)v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t u = w[q] ^ 0x80808080u;
+            even[q] += u & 0x00ff00ffu;
+            odd[q] += __byte_perm(u, 0u, 0x4341);
+        }
+    }
+    // Adds the warp's sums to the cells of a set: `dst` is the lane's first channel, `lanes` the lanes of a pixel.  Lanes
+    // that hold the same channels would queue at the cells (32 of them for 16 channels), so where `lanes` is a power of two
+    // they first halve their channels among each other, pairwise, and every channel is added once per warp.
+    __device__ __forceinline__ void flush(int32_t *dst, int lanes)
+    {
+        int v[16];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[4 * q] = (int)(even[q] & 0xffffu) - 128 * count;
+            v[4 * q + 1] = (int)(odd[q] & 0xffffu) - 128 * count;
+            v[4 * q + 2] = (int)(even[q] >> 16) - 128 * count;
+            v[4 * q + 3] = (int)(odd[q] >> 16) - 128 * count;
+        }
+        clear();
+        const int lane = threadIdx.x & 31;
+        if (lanes & (lanes - 1)) {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) atomicAdd(dst + c, v[c]);
+            return;
+        }
+        int have = 16, off = 0;
+#pragma unroll
+        for (int m = 16, half = 8; half >= 1; m >>= 1, half >>= 1)
+            if (m >= lanes) {
+                const bool up = (lane & m) != 0;
+#pragma unroll
+                for (int c = 0; c < half; ++c) {
+                    const int keep = up ? v[c + half] : v[c], send = up ? v[c] : v[c + half];
+                    v[c] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+                }
+                off += up ? half : 0;
+                have = half;
+            }
+        if (lanes == 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+        if (lanes > 1 || !(lane & 1))
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c < have) atomicAdd(dst + off + c, v[c]);
+    }
+    // adds kUnroll pixels (a zero one adds the offset alone); all lanes of the warp call it together
+    template <int kUnroll>
+    __device__ __forceinline__ void add_group(const int4 (&v)[kUnroll], int32_t *dst, int lanes)
+    {
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) add(v[u]);
+        count += kUnroll;
+        if (count > 256 - kUnroll) flush(dst, lanes);   // 255 * 257 is the most a half holds
+    }
+};
+
+// the i-th border row (column) of `extent` rows, and how many there are: all of them when no interior class exists
+__device__ __forceinline__ int border_count(int extent, int nlo, int nhi, int ncls) { return ncls == extent ? extent : nlo + nhi; }
+__device__ __forceinline__ int border_at(int i, int extent, int nlo, int nhi, int ncls)
+{
+    return (ncls == extent || i < nlo) ? i : extent - nhi + (i - nlo);
+}
+__device__ __forceinline__ bool tap_takes(int y, int k, int stride, int pad, int extent_in)
+{
+    const int src = y * stride - pad + k;
+    return src >= 0 && src < extent_in;
+}
+
+__global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_constant__ FinishBatch b)
+{
+    __shared__ unsigned long long rows_out[16], cols_out[16];  // per filter row / column: the border rows / columns it does not take
+    extern __shared__ int32_t sets[];  // [1 + border rows][1 + border columns][kClassSlab]; index 0 = all rows / columns
+    const int k = finish_item_of(b.tap_first, b.num, (int)blockIdx.x);
+    const FinishItem &it = b.item[k];
+    if (!it.use_b1) return;
+    const eoq_conv_desc_t &d = it.d;
+    const BorderClasses &bc = it.bc;
+    const int local = (int)blockIdx.x - b.tap_first[k], bx = local % it.tap_grid_x, by = local / it.tap_grid_x;
+    const int ho = it.ho, wo = it.wo, c_out = d.c_out;
+    const int nr = border_count(ho, bc.nlo_h, bc.nhi_h, bc.nrc), nc = border_count(wo, bc.nlo_w, bc.nhi_w, bc.ncc);
+    const int nsets = (1 + nr) * (1 + nc);
+    for (int i = threadIdx.x; i < nsets * kClassSlab; i += kThreads) sets[i] = 0;
+    if (threadIdx.x < d.kh) {
+        unsigned long long m = 0;
+        for (int i = 0; i < nr; ++i)
+            if (!tap_takes(border_at(i, ho, bc.nlo_h, bc.nhi_h, bc.nrc), threadIdx.x, d.stride, d.pad, d.h)) m |= 1ull << i;
+        rows_out[threadIdx.x] = m;
+    } else if (threadIdx.x >= 32 && threadIdx.x < 32 + d.kw) {
+        unsigned long long m = 0;
+        for (int i = 0; i < nc; ++i)
+            if (!tap_takes(border_at(i, wo, bc.nlo_w, bc.nhi_w, bc.ncc), threadIdx.x - 32, d.stride, d.pad, d.w)) m |= 1ull << i;
+        cols_out[threadIdx.x - 32] = m;
+    }
+    __syncthreads();
+    const int slab_ch = min(kClassSlab, c_out - by * kClassSlab);  // channels of this slab (multiple of 16)
+    const int lanes_per_pix = slab_ch / 16, pix_per_step = 32 / lanes_per_pix;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane % lanes_per_pix, slot = lane / lanes_per_pix;
+    const int r_begin = bx * it.rows_per_block, r_end = min(d.n * ho, r_begin + it.rows_per_block);
+    const int8_t *base = it.e3 + by * kClassSlab + sub * 16;
+    const int4 zero = make_int4(0, 0, 0, 0);
+    if (slot < pix_per_step) {
+        PixelSum acc;
+        acc.clear();
+        {   // T
+            constexpr int kUnroll = 8;
+            const size_t p_end = (size_t)r_end * wo;
+            const int step = (kThreads / 32) * pix_per_step;
+            for (size_t p0 = (size_t)r_begin * wo + warp * pix_per_step; p0 < p_end; p0 += kUnroll * step) {   // the same in all lanes
+                int4 v[kUnroll];
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) {
+                    const size_t p = p0 + slot + u * step;
+                    v[u] = p < p_end ? __ldg(reinterpret_cast<const int4 *>(base + p * c_out)) : zero;
+                }
+                acc.add_group(v, sets + sub * 16, lanes_per_pix);
+            }
+            if (acc.count) acc.flush(sets + sub * 16, lanes_per_pix);
+        }
+        for (int set = 1 + warp; set < nsets; set += kThreads / 32) {
+            constexpr int kUnroll = 4;
+            const int i = set / (1 + nc), j = set - i * (1 + nc);
+            int32_t *dst = sets + set * kClassSlab + sub * 16;
+            // rows first + q * row_step of the block's range, columns x0 .. x0 + cols - 1
+            int first = r_begin, row_step = 1, x0 = 0, cols = wo;
+            if (i > 0) {
+                const int y = border_at(i - 1, ho, bc.nlo_h, bc.nhi_h, bc.nrc);
+                row_step = ho;
+                first = r_begin + (y - r_begin % ho + ho) % ho;
+            }
+            if (j > 0) {
+                x0 = border_at(j - 1, wo, bc.nlo_w, bc.nhi_w, bc.ncc);
+                cols = 1;
+            }
+            const int rows = first < r_end ? (r_end - first + row_step - 1) / row_step : 0;
+            const int pixels = rows * cols;
+            for (int q0 = 0; q0 < pixels; q0 += kUnroll * pix_per_step) {
+                int4 v[kUnroll];
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) {
+                    const int q = q0 + slot + u * pix_per_step, rq = cols == 1 ? q : q / wo;
+                    const int r = first + rq * row_step, x = x0 + (q - rq * cols);
+                    v[u] = q < pixels ? __ldg(reinterpret_cast<const int4 *>(base + ((size_t)r * wo + x) * c_out)) : zero;
+                }
+                acc.add_group(v, dst, lanes_per_pix);
+            }
+            if (acc.count) acc.flush(dst, lanes_per_pix);
+        }
+    }
+    __syncthreads();
+    // the blocks spread their atomics over kTapReplicas copies
+    long long *tap_sums = it.tap_sums + (size_t)(bx % kTapReplicas) * it.tap_stride;
+    const int taps = d.kh * d.kw;
+    for (int i = threadIdx.x; i < taps * slab_ch; i += kThreads) {   // consecutive threads: neighbouring cells of [oc][tap]
+        const int c = i / taps, tap = i - c * taps, kh = tap / d.kw, kw = tap - kh * d.kw;
+        const unsigned long long rm = rows_out[kh], cm = cols_out[kw];
+        const int32_t *cell = sets + c;
+        auto over_columns = [&](const int32_t *row) {
+            int v = row[0];
+            for (unsigned long long m = cm; m; m &= m - 1) v -= row[__ffsll((long long)m) * kClassSlab];
+            return v;
+        };
+        int sum = over_columns(cell);
+        for (unsigned long long m = rm; m; m &= m - 1) sum -= over_columns(cell + __ffsll((long long)m) * (1 + nc) * kClassSlab);
+        if (sum)
+            atomicAdd(reinterpret_cast<unsigned long long *>(tap_sums + (size_t)(by * kClassSlab + c) * taps + tap),
+                      (unsigned long long)(long long)sum);
+    }
+}
+
+// ------------------------------------------------------------------ exact sums and their maximum
+// A thread owns four neighbouring weights (c_in is a multiple of 4: they share their (oc, tap)).  With more than
+// kDirectParts slices a block is (256 / groups) such quads x `groups` slice groups that meet in shared memory, and the sums
+// are written once, as int32 when they provably fit; with fewer slices, or 64-bit sums from the GEMM, nothing is written:
+// the coding pass forms them again, which costs fewer bytes than a round trip.  The 2.4 M weights of the 512-channel 3 x 3
+// layer: sums 18.9 -> 10.9 us, codes 7.8 -> 4.3 us against one weight per thread, four 64-bit tap sums read for each of
+// them and 64-bit sums written and read back.
+constexpr int kDirectParts = 2;
+
+// b1 term of the quad at weight index 4 q
+__device__ __forceinline__ long long finish_b1_term(const FinishItem &it, int b1, uint32_t q)
+{
+    const long long *t = it.tap_sums + (4u * q) / (uint32_t)it.d.c_in;
+    long long s = 0;
+#pragma unroll
+    for (int r = 0; r < kTapReplicas; ++r) s += __ldg(t + (size_t)r * it.tap_stride);
+    return (long long)b1 * s;
+}
+
+// the quad's sums without the b1 term, from at most kDirectParts slices or the 64-bit sums
+__device__ __forceinline__ void finish_direct(const FinishItem &it, uint32_t q, long long (&v)[4])
+{
+    if (it.parts) {
+        int4 a[kDirectParts];
+#pragma unroll
+        for (int s = 0; s < kDirectParts; ++s)
+            a[s] = s < it.num_parts ? __ldg(reinterpret_cast<const int4 *>(it.parts + (size_t)s * it.n) + q) : make_int4(0, 0, 0, 0);
+        v[0] = (long long)a[0].x + a[1].x;
+        v[1] = (long long)a[0].y + a[1].y;
+        v[2] = (long long)a[0].z + a[1].z;
+        v[3] = (long long)a[0].w + a[1].w;
+    } else {
+        const longlong2 lo = __ldg(reinterpret_cast<const longlong2 *>(it.acc) + 2 * (size_t)q);
+        const longlong2 hi = __ldg(reinterpret_cast<const longlong2 *>(it.acc) + 2 * (size_t)q + 1);
+        v[0] = lo.x;
+        v[1] = lo.y;
+        v[2] = hi.x;
+        v[3] = hi.y;
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) finish_sums_kernel(const __grid_constant__ FinishBatch b)
+{
+    __shared__ long long part[kThreads][4];
+    const int k = finish_item_of(b.fin_first, b.num, (int)blockIdx.x);
+    const FinishItem &it = b.item[k];
+    const int groups = it.groups, bw = kThreads / groups, tx = threadIdx.x % bw, ty = threadIdx.x / bw;
+    const uint32_t quads = (uint32_t)(it.n / 4);
+    const int b1 = it.use_b1 ? finish_b1(it) : 0;
+    const bool narrow = finish_narrow(it, b1);
+    unsigned long long mx = 0;
+    for (uint32_t base = (uint32_t)((int)blockIdx.x - b.fin_first[k]) * bw; base < quads; base += (uint32_t)it.fin_blocks * bw) {
+        const uint32_t q = base + tx;
+        const bool in = q < quads;
+        long long v[4] = {0, 0, 0, 0};
+        if (it.direct) {
+            if (in) finish_direct(it, q, v);
+        } else {
+            if (in) {
+                // four slices per round: their loads are independent and in flight together
+                const int4 *p = reinterpret_cast<const int4 *>(it.parts) + q;
+                int s = ty;
+                for (; s + 3 * groups < it.num_parts; s += 4 * groups) {
+                    int4 a[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) a[u] = __ldg(p + (size_t)(s + u * groups) * quads);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        v[0] += a[u].x;
+                        v[1] += a[u].y;
+                        v[2] += a[u].z;
+                        v[3] += a[u].w;
+                    }
+                }
+                for (; s < it.num_parts; s += groups) {
+                    const int4 a = __ldg(p + (size_t)s * quads);
+                    v[0] += a.x;
+                    v[1] += a.y;
+                    v[2] += a.z;
+                    v[3] += a.w;
+                }
+            }
+            if (groups > 1) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) part[threadIdx.x][c] = v[c];
+                __syncthreads();
+                if (ty == 0)
+                    for (int u = 1; u < groups; ++u)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) v[c] += part[u * bw + tx][c];
+                __syncthreads();
+            }
+        }
+        if (ty == 0 && in) {
+            if (it.use_b1) {
+                const long long t = finish_b1_term(it, b1, q);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[c] += t;
+            }
+            if (!it.direct || it.keep_sums) {
+                if (narrow && !it.keep_sums) {
+                    reinterpret_cast<int4 *>(it.acc)[q] = make_int4((int)v[0], (int)v[1], (int)v[2], (int)v[3]);
+                } else {
+                    longlong2 *o = reinterpret_cast<longlong2 *>(it.acc) + 2 * (size_t)q;
+                    o[0] = make_longlong2(v[0], v[1]);
+                    o[1] = make_longlong2(v[2], v[3]);
+                }
+            }
+            if (it.copy_out)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) it.copy_out[4 * (size_t)q + c] = v[c];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const unsigned long long a = (unsigned long long)(v[c] < 0 ? -v[c] : v[c]);
+                mx = a > mx ? a : mx;
+            }
+        }
+    }
+    mx = block_max_u64(mx);
+    if (threadIdx.x == 0 && mx && !it.keep_sums) atomicMax(it.max_cell, mx);
+}
+
+// max |.| of 64-bit sums that an all-reduce over replicas completed (keep_sums)
+__global__ void __launch_bounds__(kThreads) finish_max_kernel(const long long *__restrict__ src, size_t n, unsigned long long *max_cell)
+{
+    unsigned long long mx = 0;
+    for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kThreads) {
+        const long long v = src[i];
+        const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+        mx = a > mx ? a : mx;
+    }
+    mx = block_max_u64(mx);
+    if (threadIdx.x == 0 && mx) atomicMax(max_cell, mx);
+}
+
+// ------------------------------------------------------------------ Q_g
+
+__global__ void __launch_bounds__(kThreads) finish_code_kernel(const __grid_constant__ FinishBatch b, unsigned *status)
+{
+    const int k = finish_item_of(b.sq_first, b.num, (int)blockIdx.x);
+    const FinishItem &it = b.item[k];
+    const int bx = (int)blockIdx.x - b.sq_first[k];
+    const unsigned long long M = *it.max_cell;
+    const int b1 = it.use_b1 ? finish_b1(it) : 0;
+    const bool narrow = finish_narrow(it, b1);
+    const int t = M ? round_log2_u64(M) : 7;
+    if (bx == 0 && threadIdx.x == 0) {
+        const int p_in = __ldg(it.e3_exp) - 7;
+        *it.g_exp = M ? p_in + t - 7 : p_in;
+        if (!M) atomicOr(status, EOQ_DEV_SQ_ZERO);
+    }
+    // sums below 2^31 - 2^(t - 8): a right shift in four 32-bit operations (see sq_code32_shr)
+    const bool fast = t >= 8 && M < 0x7e000000ull;
+    const int sh = t - 7, half_m1 = fast ? (1 << (sh - 1)) - 1 : 0;
+    const uint32_t quads = (uint32_t)(it.n / 4);
+    const bool from_sums = !it.direct || it.keep_sums, narrow_sums = narrow && !it.keep_sums;
+    for (uint32_t q = (uint32_t)bx * kThreads + threadIdx.x; q < quads; q += (uint32_t)it.sq_blocks * kThreads) {
+        long long v[4];
+        if (from_sums && narrow_sums) {
+            const int4 a = __ldg(reinterpret_cast<const int4 *>(it.acc) + q);
+            v[0] = a.x;
+            v[1] = a.y;
+            v[2] = a.z;
+            v[3] = a.w;
+        } else if (from_sums) {
+            const longlong2 lo = __ldg(reinterpret_cast<const longlong2 *>(it.acc) + 2 * (size_t)q);
+            const longlong2 hi = __ldg(reinterpret_cast<const longlong2 *>(it.acc) + 2 * (size_t)q + 1);
+            v[0] = lo.x;
+            v[1] = lo.y;
+            v[2] = hi.x;
+            v[3] = hi.y;
+        } else {
+            finish_direct(it, q, v);
+            if (it.use_b1) {
+                const long long bt = finish_b1_term(it, b1, q);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[c] += bt;
+            }
+        }
+        int cd[4];
+        if (fast) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) cd[c] = sq_code32_shr((int32_t)v[c], sh, half_m1);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) cd[c] = sq_code64(v[c], t);
+        }
+        reinterpret_cast<uint32_t *>(it.g)[q] = pack4_sat(cd[0], cd[1], cd[2], cd[3]);
+    }
+}
+
+}  // namespace
+
+// The launch geometry of an item, from its sizes.
+static void plan_finish_item(FinishItem &it, int sm_count, bool alone)
+{
+    const int slabs = (it.d.c_out + kClassSlab - 1) / kClassSlab, rows = it.d.n * it.ho;
+    // Every block ends in one atomic per (channel, tap), so a block gets kTapBytes of e3 (the time of its reads then covers
+    // that of its atomics) as long as that leaves no more than one block per SM, and at least a row per warp.
+    const int slab_bytes_blocks = (int)(((long long)rows * it.wo * (it.d.c_out < kClassSlab ? it.d.c_out : kClassSlab) + kTapBytes - 1) / kTapBytes);
+    int blocks = (sm_count + slabs - 1) / slabs;
+    if (blocks > slab_bytes_blocks) blocks = slab_bytes_blocks;
+    int rpb = (rows + blocks - 1) / blocks;
+    if (rpb < kThreads / 32) rpb = kThreads / 32;
+    const int most = (1 << 23) / it.wo;           // keeps the int32 class sums exact
+    if (rpb > most) rpb = most < 1 ? 1 : most;
+    it.rows_per_block = rpb;
+    it.tap_grid_x = (rows + rpb - 1) / rpb;
+    it.tap_blocks = it.use_b1 ? it.tap_grid_x * slabs : 0;
+    it.direct = !it.parts || it.num_parts <= kDirectParts;
+    it.groups = it.direct ? 1 : (it.num_parts >= 32 ? 8 : (it.num_parts >= 8 ? 4 : 1));
+    const size_t quads = (size_t)it.n / 4, bw = kThreads / it.groups;
+    size_t fb = (quads + bw - 1) / bw;
+    const size_t cap = (size_t)sm_count * (alone ? 8 : 4);
+    it.fin_blocks = (int)(fb < 1 ? 1 : (fb > cap ? cap : fb));
+    size_t qb = (quads + kThreads - 1) / kThreads;
+    it.sq_blocks = (int)(qb < 1 ? 1 : (qb > cap ? cap : qb));
+}
+
+int finish_launches(const FinishItem *items, int num, const ReduceHook &hook)
+{
+    int n = 0;
+    for (int base = 0; base < num; base += kFinishChunk) {
+        bool taps = false;
+        for (int k = base; k < num && k < base + kFinishChunk; ++k) taps |= items[k].use_b1 != 0;
+        n += 2 + (taps ? 1 : 0) + (hook.fn ? 1 : 0);
+    }
+    return n;
+}
+
+cudaError_t launch_wgrad_finish(const FinishItem *items, int num, unsigned *status, int sm_count, cudaStream_t s, const ReduceHook &hook)
+{
+    for (int base = 0; base < num; base += kFinishChunk) {
+        FinishBatch b;
+        b.num = num - base < kFinishChunk ? num - base : kFinishChunk;
+        b.tap_first[0] = b.fin_first[0] = b.sq_first[0] = 0;
+        int max_sets = 1;
+        for (int k = 0; k < b.num; ++k) {
+            FinishItem &it = b.item[k];
+            it = items[base + k];
+            it.keep_sums = hook.fn != nullptr;
+            plan_finish_item(it, sm_count, num == 1);
+            b.tap_first[k + 1] = b.tap_first[k] + it.tap_blocks;
+            b.fin_first[k + 1] = b.fin_first[k] + it.fin_blocks;
+            b.sq_first[k + 1] = b.sq_first[k] + it.sq_blocks;
+            const int sets = (1 + it.bc.nrc) * (1 + it.bc.ncc);   // at least (1 + border rows)(1 + border columns)
+            if (it.use_b1 && sets > max_sets) max_sets = sets;
+        }
+        if (b.tap_first[b.num] > 0) {
+            const size_t smem = sizeof(int32_t) * max_sets * kClassSlab;
+            if (smem > 48 * 1024) {   // at most 64 classes: 130 sets
+                const cudaError_t e = cudaFuncSetAttribute(finish_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
+                if (e != cudaSuccess) return e;
+            }
+            finish_taps_kernel<<<b.tap_first[b.num], kThreads, smem, s>>>(b);
+        }
+        finish_sums_kernel<<<b.fin_first[b.num], kThreads, 0, s>>>(b);
+        if (hook.fn)
+            // replicas (one layer per call): local sums, b1 term included (it is linear in the error) -> all-reduce ->
+            // maximum of the global sums; the copy for the caller is taken from the global sums as well
+            for (int k = 0; k < b.num; ++k) {
+                const FinishItem &it = b.item[k];
+                hook(it.acc, (size_t)it.n, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
+                finish_max_kernel<<<it.fin_blocks, kThreads, 0, s>>>(it.acc, (size_t)it.n, it.max_cell);
+                if (it.copy_out) cudaMemcpyAsync(it.copy_out, it.acc, (size_t)it.n * sizeof(long long), cudaMemcpyDeviceToDevice, s);
+            }
+        finish_code_kernel<<<b.sq_first[b.num], kThreads, 0, s>>>(b, status);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace eoq

@@ -200,6 +200,8 @@ struct WgradParams {
     int row_window_kw;   // 0, or the filter width when an M tile is one filter row of 8 x 16 bytes (7 real taps of 8)
     unsigned char tap_dh[kMaxTaps], tap_dw[kMaxTaps];
     long long *acc;      // [c_out][taps][c_in] int64, zeroed before launch
+    int4 *zero;          // the cells of the kernels that follow (tap sums, maximum): cleared here, zero_n16 groups of 16 bytes
+    unsigned zero_n16;
     DeviceState *dev;
 };
 
@@ -229,6 +231,8 @@ struct WgradPatchPlan {
     int num_stages;
     int rows_total;      // taps * c_in
     int32_t *partials;   // [num_splits][c_out][taps][c_in]
+    int4 *zero;          // as in WgradParams
+    unsigned zero_n16;
     DeviceState *dev;
 };
 constexpr int kWgradPatchThreads = 192;  // warp 0 loads, warp 1 MMA + TMEM, warps 2..5 epilogue
@@ -265,13 +269,6 @@ cudaError_t launch_sq_i32(const int32_t *src, const int32_t *src_exp, int exp_bi
 cudaError_t launch_sq_i32_scatter(const int32_t *src, const int32_t *src_exp, int exp_bias, int n_img, int hh, int ww, int c,
                                   int stride, int hq, int wq, int8_t *dst, int32_t *dst_exp, long long *sum_codes,
                                   DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook);
-// b1 is b1_c, or the code at b1_dev when that is given.  Two kernels: slice sum + b1 term + max, then Q_g; the maximum
-// travels through the handle's absmax_u64 cell, which the second kernel puts back to zero.
-// tap_sums: kTapReplicas copies, `replica_stride` elements apart, whose sum is the b1 error sum per (oc, tap).
-cudaError_t launch_sq_i64(const long long *src, const int32_t *src_exp, int exp_bias, size_t n, int8_t *dst,
-                          int32_t *dst_exp, long long *copy_out, const long long *tap_sums, size_t replica_stride,
-                          int32_t b1_c, const int32_t *b1_dev, int c_in, const int32_t *parts, int num_parts,
-                          DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook);
 // gamma is gamma_c, or the code at gamma_dev when that is given.  force_timeout: self-test of the bounded wait.
 cudaError_t launch_err_prescale(const int8_t *e0, const int32_t *e0_exp, const uint8_t *mask, const int16_t *x2,
                                 size_t n_el, int32_t gamma_c, const int32_t *gamma_dev, int8_t *e3, int32_t *e3_exp,
@@ -300,9 +297,7 @@ struct BorderClasses {
 };
 cudaError_t launch_b1_weight_table(const int8_t *w, int32_t *table, const eoq_conv_desc_t &d, const BorderClasses &bc,
                                    cudaStream_t s);
-constexpr int kTapReplicas = 4;  // copies of the b1 error sums the blocks spread their atomics over
-cudaError_t launch_b1_error_sums(const int8_t *e3, long long *tap_sums, size_t replica_stride, const eoq_conv_desc_t &d, int ho,
-                                 int wo, const BorderClasses &bc, int sm_count, cudaStream_t s);
+constexpr int kTapReplicas = 4;  // copies of the b1 error sums of a weight gradient the blocks spread their atomics over
 constexpr int kMaxBorderClasses = 64;  // classes (rows x columns) the b1 kernels keep in shared memory
 
 // eoq_weight_prep: one launch derives the b1 tables (and the row-padded first-layer weights) of up to kPrepChunk layers
@@ -364,35 +359,40 @@ struct ScalarBatch {
     ScalarItem item[kScalarChunk];
     int num;
 };
-// Finish of the weight gradients of many layers in a few launches (eoq_wgrad_finish): per layer the b1 error sums,
-// the sum of the split-K slices plus the b1 term, and Q_g.  One item per layer; blocks find their item by their index.
+// What follows the weight-gradient GEMM (eoq_finish.cu), for one layer or for many in the same launches: the b1 error
+// sums, the exact sums with the b1 term, Q_g.  One item per layer; blocks find their item by their index.
 constexpr int kFinishChunk = 16;
 struct FinishItem {
     const int8_t *e3;
     const int32_t *e3_exp;
-    const int32_t *b1_dev;         // null: no b1 term (then the tap sums are neither formed nor read)
-    long long *tap_sums;           // kTapReplicas copies, tap_stride elements apart; zeroed by the finish itself
-    unsigned long long *max_cell;  // max |sum| of the layer (in the spare bytes behind the tap sums)
-    long long *acc;                // exact sums [oc][tap][ic]
+    const int32_t *b1_dev;         // b1 in device memory, or null: b1_c
+    int32_t b1_c;
+    int use_b1;                    // 0: no b1 term (then the tap sums are neither formed nor read)
+    long long *tap_sums;           // kTapReplicas copies, tap_stride elements apart; cleared by the GEMM kernel
+    unsigned long long *max_cell;  // max |sum| of the layer (behind the tap sums); cleared by the GEMM kernel
+    long long *acc;                // exact sums [oc][tap][ic]: the GEMM's (64-bit), or where the slices' sums go
     const int32_t *parts;          // int32 split-K slices, or null when the GEMM added into acc
+    long long *copy_out;           // the exact sums for the caller, or null
     int8_t *g;
     int32_t *g_exp;
     unsigned long long n;          // weights
-    unsigned long long tap_stride, zero_bytes;
+    unsigned long long tap_stride;
     unsigned long long pixels;
     eoq_conv_desc_t d;
     BorderClasses bc;
-    int ho, wo, pixels_per_block, tap_grid_x, tap_grid_y;
-    int num_parts, groups, fin_blocks, sq_blocks;
+    int ho, wo, num_parts;
+    // filled by launch_wgrad_finish
+    int rows_per_block, tap_grid_x, tap_blocks, groups, fin_blocks, sq_blocks;
+    int direct;                    // the sums are formed twice instead of being written and read back
+    int keep_sums;                 // reduce hook: the sums are completed by an all-reduce before their maximum is taken
 };
 struct FinishBatch {
     int num;
     int tap_first[kFinishChunk + 1], fin_first[kFinishChunk + 1], sq_first[kFinishChunk + 1];
     FinishItem item[kFinishChunk];
 };
-// fills the launch geometry of an item (tap grid, block counts) from its sizes
-void plan_finish_item(FinishItem &it, int sm_count);
-cudaError_t launch_wgrad_finish(const FinishBatch &b, unsigned *status, cudaStream_t s);
+cudaError_t launch_wgrad_finish(const FinishItem *items, int num, unsigned *status, int sm_count, cudaStream_t s, const ReduceHook &hook);
+int finish_launches(const FinishItem *items, int num, const ReduceHook &hook);
 
 // Batch normalisation behind the convolution (comparison case, eoq_bn.cu): per-channel record in the workspace
 struct BnChannel {

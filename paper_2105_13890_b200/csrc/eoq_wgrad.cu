@@ -77,6 +77,7 @@ wgrad_kernel(const __grid_constant__ WgradParams p, const __grid_constant__ CUte
         ptx::prefetch_tensormap(&map_x);
         ptx::prefetch_tensormap(&map_e);
     }
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < p.zero_n16; i += gridDim.x * blockDim.x) p.zero[i] = make_int4(0, 0, 0, 0);
     if (warp == 1) {
         ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), tmem_cols);
         ptx::tmem_relinquish();

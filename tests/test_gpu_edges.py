@@ -84,3 +84,24 @@ def test_head_error_sizes(n, c, hw):
         eoq.eoq_aux_head_error(G.handle(), G.dev(d), n, c, hw, e, pe, G.zeros(n * c * 4, torch.uint8))
         assert G.status_clear() == 0 and pe.item() == p
         assert all(np.array_equal(G.host(e)[:, i, :], codes.reshape(n, c)) for i in range(hw))
+
+
+@pytest.mark.parametrize("n,h,w,c_in,c_out,k,stride,pad", [
+    (3, 2, 2, 32, 32, 3, 1, 1),      # every row and column is a border one
+    (2, 9, 33, 32, 16, 3, 1, 1),     # one lane per pixel; two slices at most: sums formed twice
+    (5, 7, 7, 48, 80, 3, 2, 1),      # five lanes per pixel, strided borders
+    (40, 28, 28, 32, 160, 3, 1, 1),  # two channel slabs, the second ragged; many slices
+    (2, 11, 6, 16, 32, 5, 1, 2),     # two border rows and columns on each side
+])
+def test_weight_gradient_finish(n, h, w, c_in, c_out, k, stride, pad):
+    d = oracle.ConvDesc(n, h, w, c_in, c_out, k, k, stride, pad)
+    x, e3 = synth.relu_codes((n, h, w, c_in), 1550, 0), synth.normal_codes((n, d.ho, d.wo, c_out), 1550, 1)
+    b1 = -77
+    want, p, _ = oracle.sq_int(oracle.conv_wgrad_acc(d, e3, x, b1), -10 - 7)
+    g, pg = G.zeros((c_out, k, k, c_in), torch.int8), G.zeros(1, torch.int32)
+    gd = G.gdesc(d)
+    for _ in range(2):
+        eoq.eoq_conv_wgrad_dev(G.handle(), gd, G.dev(e3), G.dev(np.array([-10], dtype=np.int32)), G.dev(x),
+                               G.dev(np.array([b1], dtype=np.int32)), g, pg, G.workspace(gd, eoq.EOQ_PASS_WGRAD))
+        assert G.status_clear() == 0
+        assert np.array_equal(G.host(g).astype(np.int32).reshape(-1), np.asarray(want).reshape(-1)) and pg.item() == p
