@@ -214,6 +214,19 @@ inline int persistent_grid(int tiles, int sm_count)
     return (tiles + per_cta - 1) / per_cta;
 }
 
+// Tiles a CTA keeps in the epilogue at once.  One group of warps on one tile leaves every wait of that tile exposed (a
+// 128 x 64 tile took 2,250 cycles alone, 2,650 per tile with two of them, against about 1,100 of issue), so as many tiles as
+// the CTA gets and tensor memory holds are worked on side by side; a CTA with a single tile puts all its warps on it.
+void plan_epilogue(IgemmParams &p, int grid)
+{
+    const int tiles = p.num_m_tiles * p.num_n_tiles, per_cta = (tiles + grid - 1) / grid;
+    int cols = 32;
+    while (cols < p.tile_n) cols <<= 1;
+    const int buffer = p.tile_n <= 128 ? 2 * cols : cols;   // two partial accumulators up to 128 columns
+    p.ep_groups = per_cta >= 3 && 4 * buffer <= 512 ? 4 : (per_cta >= 2 && 2 * buffer <= 512 ? 2 : 1);
+    if (p.tile_n / 16 < 4 / p.ep_groups) p.ep_groups = p.tile_n >= 32 ? 2 : 4;   // at least one 16-column group per warp
+}
+
 // Shared tiling choices of the implicit GEMM: K sub-tiles, pipeline depth, column tile.
 void plan_igemm(IgemmParams &p, int src_channels, int ntaps, int sm_count)
 {
@@ -270,8 +283,14 @@ bool plan_patch(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, int
     p.hq = hq;
     p.wq = wq;
     p.num_m_tiles = n_img * tiles_per_img;
+    // 256 columns where that saves a wave of tiles: a 256-column MMA reads 12 KB of shared memory for twice the work of a
+    // 128-column one that reads 8 KB, and its tile costs about 1.4 times as much (256 channels, 14 x 14, batch 64: one wave of
+    // 128 wide tiles instead of two of narrow ones, 16.9 -> 13.6 us).
     int tn = n_cols < 256 ? n_cols : 256;
-    if (tn == 256 && (long long)p.num_m_tiles * ((n_cols + 255) / 256) < 2LL * sm_count) tn = 128;
+    if (tn == 256) {
+        auto waves = [&](int cols) { return ((long long)p.num_m_tiles * ((n_cols + cols - 1) / cols) + sm_count - 1) / sm_count; };
+        if (7 * waves(256) >= 5 * waves(128)) tn = 128;
+    }
     p.tile_n = tn;
     p.num_n_tiles = (n_cols + tn - 1) / tn;
     const size_t budget = 200 * 1024;
@@ -726,7 +745,9 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
         const int ptiles = p.num_m_tiles * p.num_n_tiles;
         count_launches(h, 1);
         ProfScope prof(h, EOQ_PROF_IGEMM_FWD, s);
-        return record(h, launch_igemm_patch(p, pl, map_a, map_b, persistent_grid(ptiles, h->gemm_ctas), s));
+        const int grid = persistent_grid(ptiles, h->gemm_ctas);
+        plan_epilogue(p, grid);
+        return record(h, launch_igemm_patch(p, pl, map_a, map_b, grid, s));
     }
     if (row_window) {
         if (!make_row_window_map(&map_a, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, g.wo, g.ho, d.stride, d.pad, kTileM) ||
@@ -740,7 +761,9 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
     const int tiles = p.num_m_tiles * p.num_n_tiles;
     count_launches(h, 1);
     ProfScope prof(h, EOQ_PROF_IGEMM_FWD, s);
-    return record(h, launch_igemm(p, map_a, map_b, persistent_grid(tiles, h->gemm_ctas), s));
+    const int grid = persistent_grid(tiles, h->gemm_ctas);
+    plan_epilogue(p, grid);
+    return record(h, launch_igemm(p, map_a, map_b, grid, s));
 }
 
 extern "C" int eoq_conv_fwd(eoq_handle_t handle, const eoq_conv_desc_t *desc, const int8_t *x, const int32_t *x_exp,
@@ -918,7 +941,9 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             count_launches(h, 1);
             {
                 ProfScope prof(h, EOQ_PROF_IGEMM_DGRAD, s);
-                e = launch_igemm_patch(p, pl, map_a, map_b, persistent_grid(ptiles, h->gemm_ctas), s);
+                const int grid = persistent_grid(ptiles, h->gemm_ctas);
+                plan_epilogue(p, grid);
+                e = launch_igemm_patch(p, pl, map_a, map_b, grid, s);
             }
             if (e != cudaSuccess || h->gemm_only) return record(h, e);
             {
@@ -1059,11 +1084,13 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
                 }
             }
             ++class_no;
+            const int grid = persistent_grid(tiles, ctas);
+            plan_epilogue(p, grid);
             if (side_by_side) {
-                e = launch_igemm(p, map_a, map_b, persistent_grid(tiles, ctas), cs);
+                e = launch_igemm(p, map_a, map_b, grid, cs);
             } else {
                 ProfScope prof(h, EOQ_PROF_IGEMM_DGRAD, cs);
-                e = launch_igemm(p, map_a, map_b, persistent_grid(tiles, ctas), cs);
+                e = launch_igemm(p, map_a, map_b, grid, cs);
             }
             if (e != cudaSuccess) {
                 launch_reset_cells(h->dev, s);  // GEMMs already queued have touched the maximum cell

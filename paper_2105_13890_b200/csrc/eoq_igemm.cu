@@ -5,7 +5,7 @@
 //              issue side by side, so the pipeline stages rotate over three producers
 //   warp 1       : owns tensor memory, issues tcgen05.mma kind::i8 (int8 x int8 -> int32 in TMEM)
 //   warps 4-19   : epilogue; read the accumulators with tcgen05.ld and apply the layer's quantizers in registers
-// Two accumulator buffers in TMEM let the epilogue of tile i overlap the main loop of tile i+1.
+// Up to four accumulator buffers in TMEM let the epilogue of a tile overlap the main loops of the next ones.
 // Every wait is bounded: when one runs out the CTA raises EOQ_DEV_TIMEOUT, drains and returns.
 #include "eoq_device.cuh"
 #include "eoq_epilogue.cuh"
@@ -18,12 +18,13 @@ namespace {
 constexpr int kMaxStages = 8;
 constexpr int kProducers = 3;
 
+template <int kEpi>   // EpilogueKind: forward and dgrad are kernels of their own (registers, code size)
 __global__ void __launch_bounds__(kGemmThreads, 1)
 igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUtensorMap map_a,
              const __grid_constant__ CUtensorMap map_b)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * kMaxStages + 5];
+    __shared__ __align__(8) uint64_t bars[2 * kMaxStages + 9];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile uint32_t abort_s;
 
@@ -35,8 +36,8 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (kMaxStages + s); };
     auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * kMaxStages + a); };
-    auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * kMaxStages + 2 + a); };
-    const uint32_t drain_bar = bar0 + 8u * (2 * kMaxStages + 4);
+    auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * kMaxStages + 4 + a); };
+    const uint32_t drain_bar = bar0 + 8u * (2 * kMaxStages + 8);
 
     uint32_t acc_stride = 32;
     while (acc_stride < (uint32_t)p.tile_n) acc_stride <<= 1;
@@ -44,16 +45,16 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     // exactly in the epilogue), which removes the wait of an MMA on its predecessor's write-back.
     const uint32_t nacc = (p.tile_n <= 128 && p.kc >= 32 && p.num_sub * (p.kc / 32) >= 2) ? 2u : 1u;
     const uint32_t buf_stride = nacc * acc_stride;
-    const uint32_t tmem_cols = 2 * buf_stride;
+    const uint32_t tmem_cols = p.ep_groups * buf_stride;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.num_stages; ++s) {
             ptx::mbar_init(full_bar(s), 1);
             ptx::mbar_init(empty_bar(s), 1);
         }
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < p.ep_groups; ++a) {
             ptx::mbar_init(tfull_bar(a), 1);
-            ptx::mbar_init(tempty_bar(a), kEpilogueWarps / 2);
+            ptx::mbar_init(tempty_bar(a), kEpilogueWarps / p.ep_groups);
         }
         ptx::mbar_init(drain_bar, 1);
         abort_s = 0;
@@ -74,6 +75,9 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     const int num_tiles = p.num_m_tiles * p.num_n_tiles;
     const int k_iters = (p.num_sub + p.subs_per_stage - 1) / p.subs_per_stage;
     const int pix_per_img = p.hq * p.wq;
+    // Every CTA walks the reduction from another starting point (the integer sums do not depend on the order): in step, all
+    // CTAs of a column tile would ask the same L2 slices for the same weights at the same time.
+    const int k_first = (int)(blockIdx.x % (unsigned)k_iters);
 
     if (warp == 0 || warp == 2 || warp == 3) {
         if (lane == 0) {
@@ -91,7 +95,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                 const int img = m0 / pix_per_img, rem = m0 % pix_per_img;
                 const int cw = (rem % p.wq) * p.src_stride_w + p.base_w;
                 const int ch = (rem / p.wq) * p.src_stride + p.base_h;
-                for (int kit = 0; kit < k_iters; ++kit) {
+                for (int step = 0, kit = k_first; step < k_iters; ++step, kit = kit + 1 == k_iters ? 0 : kit + 1) {
                     if (turn-- != 0) continue;
                     turn = kProducers - 1;
                     if (!(ok = wait_bar<32>(empty_bar(stage), phase ^ 1u, ctx))) break;
@@ -172,7 +176,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
             const uint32_t d_tmem = tmem_base + acc * buf_stride, d_other = nacc == 2 ? d_tmem + acc_stride : d_tmem;
             uint32_t accumulate = 0;
             uint32_t fresh0 = 1u, fresh1 = nacc == 2 ? 1u : 0u;
-            for (int kit = 0; kit < k_iters; ++kit) {
+            for (int step = 0, kit = k_first; step < k_iters; ++step, kit = kit + 1 == k_iters ? 0 : kit + 1) {
                 if (!(ok = __all_sync(0xffffffffu, wait_bar(full_bar(stage), phase, ctx)))) break;
                 ptx::tc_fence_after();
                 const int subs = min(p.subs_per_stage, p.num_sub - kit * p.subs_per_stage);
@@ -204,7 +208,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                 if (++stage == p.num_stages) { stage = 0; phase ^= 1u; }
             }
             if (ok) ptx::mma_commit(tfull_bar(acc), leader);
-            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            if (++acc == p.ep_groups) { acc = 0; acc_phase ^= 1u; }
         }
         if (!ok) {
             ptx::mma_commit(drain_bar, leader);
@@ -213,18 +217,16 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         }
     } else {
         // ---------------------------------------------------------------------- epilogue
-        // A warp may read the TMEM lanes of quadrant (warp % 4).  The four warps of a quadrant form two pairs;
-        // pair `grp` serves every second tile of this CTA (accumulator buffer `grp`), the two warps of a pair
-        // split the tile's columns, so that two tiles are in the epilogue at the same time.  Everything that does
-        // not depend on the sums is formed before the wait for the tile's MMAs.
+        // A warp may read the TMEM lanes of quadrant (warp % 4).  The four warps of a quadrant form ep_groups groups; group
+        // `grp` serves every ep_groups-th tile of this CTA (accumulator buffer `grp`) and its warps split the tile's columns.
+        // Everything that does not depend on the sums is formed before the wait for the tile's MMAs.
         const int quad = warp & 3;
         const int ew = (warp - 4) >> 2;
-        const int grp = ew & 1, part = ew >> 1;
+        const int parts = 4 / p.ep_groups, grp = ew / parts, part = ew - grp * parts;
         const int row = quad * 32 + lane;
         const int groups = p.tile_n / 16;                 // 16-column groups of the tile
-        constexpr int kParts = kEpilogueWarps / 8;
-        const int g_begin = (groups * part) / kParts, g_end = (groups * (part + 1)) / kParts;
-        const bool fwd = p.epilogue == kEpiForward;
+        const int g_begin = (groups * part) / parts, g_end = (groups * (part + 1)) / parts;
+        constexpr bool fwd = kEpi == kEpiForward;
         const FwdScalars fs = fwd ? load_fwd_scalars(p) : FwdScalars{0, 0, 0};
         // the b1 table of the whole layer goes to shared memory (behind the pipeline stages), once, times b1
         const int32_t *ts = fwd ? stage_b1_table(p, fs.b1, smem_raw + (smem_base - ptx::smem_u32(smem_raw)) + p.num_stages * stage_bytes,
@@ -238,10 +240,11 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                 shift = max(-16, min(31, shift));
             }
         }
+        const FwdShift sh = forward_shift(p, shift);
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
         const bool wide_out = (reinterpret_cast<uintptr_t>(p.acc_out) & 31) == 0;   // 256-bit stores of the exact sums
         bool ok = true;
-        for (int tile = blockIdx.x + grp * gridDim.x; tile < num_tiles && ok; tile += 2 * gridDim.x) {
+        for (int tile = blockIdx.x + grp * gridDim.x; tile < num_tiles && ok; tile += p.ep_groups * gridDim.x) {
             const int mt = tile / p.num_n_tiles, nt = tile % p.num_n_tiles;
             const int m = mt * kTileM + row;
             const bool valid = m < p.M;
@@ -281,23 +284,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                 }
                 if (valid && col < p.N) {
                     if (fwd) {
-                        if (shift == 7) {
-                            if (nacc == 2) {
-                                if (p.relu) forward_16<true, true, true>(p, fs, r, r2, off, tb, tg, sc, 7);
-                                else forward_16<true, false, true>(p, fs, r, r2, off, tb, tg, sc, 7);
-                            } else {
-                                if (p.relu) forward_16<true, true, false>(p, fs, r, r2, off, tb, tg, sc, 7);
-                                else forward_16<true, false, false>(p, fs, r, r2, off, tb, tg, sc, 7);
-                            }
-                        } else {
-                            // the generic shift (first layer behind the input quantizer) merges the partial sums itself
-                            if (nacc == 2) {
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) r[i] += r2[i];
-                            }
-                            if (p.relu) forward_16<false, true, false>(p, fs, r, r2, off, tb, tg, sc, shift);
-                            else forward_16<false, false, false>(p, fs, r, r2, off, tb, tg, sc, shift);
-                        }
+                        forward_group(p, fs, sh, r, r2, nacc, off, tb, tg, sc, shift);
                     } else {
                         mx = max(mx, wide_out ? dgrad_16<true>(p, r, off, mx_masked) : dgrad_16<false>(p, r, off, mx_masked));
                     }
@@ -311,7 +298,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
             if (lane == 0) ptx::mbar_arrive(tempty_bar(grp));
             acc_phase ^= 1u;
         }
-        if (p.epilogue == kEpiDgrad) {
+        if (!fwd) {
             mx = warp_max_u32(mx);
             if (lane == 0 && mx) atomicMax(&p.dev->absmax_u32, mx);
             if (p.next_mask) {
@@ -340,9 +327,10 @@ cudaError_t launch_igemm(const IgemmParams &p, const CUtensorMap &map_a, const C
                          cudaStream_t stream)
 {
     const size_t smem = igemm_smem_bytes(p);
-    cudaError_t e = cudaFuncSetAttribute(igemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    const auto kernel = p.epilogue == kEpiForward ? igemm_kernel<kEpiForward> : igemm_kernel<kEpiDgrad>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e != cudaSuccess) return e;
-    igemm_kernel<<<grid, kGemmThreads, smem, stream>>>(p, map_a, map_b);
+    kernel<<<grid, kGemmThreads, smem, stream>>>(p, map_a, map_b);
     return cudaGetLastError();
 }
 

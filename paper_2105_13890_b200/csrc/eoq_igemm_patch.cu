@@ -11,8 +11,8 @@
 // dropped.  Weights either stay resident in shared memory for the whole kernel (when the layer's weights fit) or
 // stream through their own ring.
 //
-// Roles: warp 0 patch loads, warp 1 TMEM owner + tcgen05.mma issuer, warp 2 weight loads, warps 4-19 epilogue
-// (four per TMEM lane quadrant: two pairs that take alternate tiles, the warps of a pair split the columns).
+// Roles: warp 0 patch loads, warp 1 TMEM owner + tcgen05.mma issuer, warps 2 and 3 weight loads, warps 4-19 epilogue
+// (four per TMEM lane quadrant, in one, two or four groups that take the CTA's tiles in turn).
 // All waits are bounded.
 #include "eoq_device.cuh"
 #include "eoq_epilogue.cuh"
@@ -24,12 +24,13 @@ namespace {
 
 constexpr int kMaxA = 4, kMaxB = 8;
 
+template <int kEpi>   // EpilogueKind: forward and dgrad are kernels of their own (registers, code size)
 __global__ void __launch_bounds__(kPatchThreads, 1)
 igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ PatchPlan pl,
                    const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * kMaxA + 2 * kMaxB + 5];
+    __shared__ __align__(8) uint64_t bars[2 * kMaxA + 2 * kMaxB + 9];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile uint32_t abort_s;
 
@@ -44,8 +45,8 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
     auto b_full = [&](int s) { return bar0 + 8u * (2 * kMaxA + s); };
     auto b_empty = [&](int s) { return bar0 + 8u * (2 * kMaxA + kMaxB + s); };
     auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * kMaxA + 2 * kMaxB + a); };
-    auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * kMaxA + 2 * kMaxB + 2 + a); };
-    const uint32_t drain_bar = bar0 + 8u * (2 * kMaxA + 2 * kMaxB + 4);
+    auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * kMaxA + 2 * kMaxB + 4 + a); };
+    const uint32_t drain_bar = bar0 + 8u * (2 * kMaxA + 2 * kMaxB + 8);
 
     uint32_t acc_stride = 32;
     while (acc_stride < (uint32_t)p.tile_n) acc_stride <<= 1;
@@ -53,7 +54,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
     // exactly in the epilogue), which removes the wait of an MMA on its predecessor's write-back.
     const uint32_t nacc = p.tile_n <= 128 ? 2u : 1u;
     const uint32_t buf_stride = nacc * acc_stride;
-    const uint32_t tmem_cols = 2 * buf_stride;
+    const uint32_t tmem_cols = p.ep_groups * buf_stride;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxA; ++s) {
@@ -64,9 +65,9 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
             ptx::mbar_init(b_full(s), 1);
             ptx::mbar_init(b_empty(s), 1);
         }
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < p.ep_groups; ++a) {
             ptx::mbar_init(tfull_bar(a), 1);
-            ptx::mbar_init(tempty_bar(a), kEpilogueWarps / 2);
+            ptx::mbar_init(tempty_bar(a), kEpilogueWarps / p.ep_groups);
         }
         ptx::mbar_init(drain_bar, 1);
         abort_s = 0;
@@ -112,7 +113,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
                         for (uint32_t i = 0; i < kSpinLimit; ++i)
                             if (ptx::mbar_try_wait(a_full(s), (inflight_parity >> s) & 1u)) break;
         }
-    } else if (warp == 2) {
+    } else if (warp == 2 || (warp == 3 && !pl.b_resident)) {
         if (lane == 0) {
             // ------------------------------------------------------------------ weight loads
             // One sub-tile = the weights of one tap for kc reduction channels and tile_n columns.  K-major: one box
@@ -133,19 +134,24 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
                         load_b(b_region + (c * taps + t) * b_sub, b_full(0), c, (int)p.tap_b[t], 0);
                 // completion is observed by the MMA thread, which every path out of this kernel waits for
             } else {
-                int ib = 0;
+                // Two loaders take turns: one thread gets a sub-tile out only every few hundred cycles (error back-propagation
+                // of the 256-channel 14 x 14 layer at batch 64: 25.4 -> 22.4 us).
+                int ib = warp - 2;
+                bool mine = warp == 2;
                 uint32_t phb = 0, inflight = 0, inflight_parity = 0;
                 bool ok = true;
                 for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
                     const int nt = tile % p.num_n_tiles;
                     for (int c = 0; c < pl.chunks && ok; ++c)
-                        for (int t = 0; t < taps; ++t) {
+                        for (int t = 0; t < taps; ++t, mine = !mine) {
+                            if (!mine) continue;
                             if (!(ok = wait_bar<64>(b_empty(ib), phb ^ 1u, ctx))) break;
                             ptx::mbar_expect_tx(b_full(ib), b_sub);
                             load_b(b_region + ib * b_sub, b_full(ib), c, (int)p.tap_b[t], nt * p.tile_n);
                             inflight |= 1u << ib;
                             inflight_parity = (inflight_parity & ~(1u << ib)) | (phb << ib);
-                            if (++ib == pl.num_b) { ib = 0; phb ^= 1u; }
+                            ib += 2;
+                            if (ib >= pl.num_b) { ib -= pl.num_b; phb ^= 1u; }   // (num_b is at least 2)
                         }
                 }
                 if (!ok)
@@ -241,7 +247,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
                 if (++ia == num_a) { ia = 0; pha ^= 1u; }
             }
             if (ok) ptx::mma_commit(tfull_bar(acc), leader);
-            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            if (++acc == p.ep_groups) { acc = 0; acc_phase ^= 1u; }
         }
         if (!ok) {
             ptx::mma_commit(drain_bar, leader);
@@ -253,32 +259,32 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
         }
     } else if (warp >= 4) {
         // ---------------------------------------------------------------------- epilogue
-        // The four warps of a TMEM lane quadrant form two pairs; pair `grp` serves every second tile of this CTA
-        // (the tiles whose sums sit in accumulator buffer `grp`), and the two warps of a pair split the columns.
-        // Two tiles are therefore in the epilogue at the same time: while one pair waits for tensor-memory loads
-        // or stores, the other has arithmetic to issue.  Everything that does not depend on the sums (pixel
-        // index, border class, b1 table row, shortcut codes) is formed before the wait for the tile's MMAs.
+        // The four warps of a TMEM lane quadrant form ep_groups groups; group `grp` serves every ep_groups-th tile of this
+        // CTA (the tiles whose sums sit in accumulator buffer `grp`), and its warps split the columns.  Several tiles are
+        // therefore in the epilogue at the same time: while one group waits for tensor-memory loads or stores, another has
+        // arithmetic to issue.  Everything that does not depend on the sums (pixel index, border class, b1 table row,
+        // shortcut codes) is formed before the wait for the tile's MMAs.
         const int quad = warp & 3;
         const int ew = (warp - 4) >> 2;
-        const int grp = ew & 1, part = ew >> 1;
+        const int parts = 4 / p.ep_groups, grp = ew / parts, part = ew - grp * parts;
         const int row = quad * 32 + lane;
         const int groups = p.tile_n / 16;
-        constexpr int kParts = kEpilogueWarps / 8;
-        const int g_begin = (groups * part) / kParts, g_end = (groups * (part + 1)) / kParts;
+        const int g_begin = (groups * part) / parts, g_end = (groups * (part + 1)) / parts;
         const int yl = row / pl.pw, xx = row % pl.pw;  // position of this thread's row in the patch raster
-        const bool fwd = p.epilogue == kEpiForward;
+        constexpr bool fwd = kEpi == kEpiForward;
         const FwdScalars fs = fwd ? load_fwd_scalars(p) : FwdScalars{0, 0, 0};
         // the b1 table of the whole layer goes to shared memory (behind the operand buffers), once, times b1
         const int32_t *ts = fwd ? stage_b1_table(p, fs.b1, smem_raw + (smem_base - ptx::smem_u32(smem_raw)) + table_off,
                                                  (int)threadIdx.x - 128, 32 * kEpilogueWarps)
                                 : nullptr;
+        const FwdShift sh = forward_shift(p, 7);
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
         const bool wide_out = (reinterpret_cast<uintptr_t>(p.acc_out) & 31) == 0;   // 256-bit stores of the exact sums
         bool ok = true;
         // (column tile, image, row tile in the image) of the current tile, carried from tile to tile: the step
         // between two tiles of this pair is constant, so its quotients are formed once instead of four integer
         // divisions per tile and warp
-        const int tile0 = blockIdx.x + grp * gridDim.x, step = 2 * gridDim.x;
+        const int tile0 = blockIdx.x + grp * gridDim.x, step = p.ep_groups * gridDim.x;
         int nt = tile0 % p.num_n_tiles, mt0 = tile0 / p.num_n_tiles;
         int img = mt0 / pl.tiles_per_img, ti = mt0 % pl.tiles_per_img;
         const int step_nt = step % p.num_n_tiles, step_mt = step / p.num_n_tiles;
@@ -320,13 +326,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
                 }
                 if (valid && col < p.N) {
                     if (fwd) {
-                        if (nacc == 2) {
-                            if (p.relu) forward_16<true, true, true>(p, fs, r, r2, off, tb, tg, sc, 7);
-                            else forward_16<true, false, true>(p, fs, r, r2, off, tb, tg, sc, 7);
-                        } else {
-                            if (p.relu) forward_16<true, true, false>(p, fs, r, r2, off, tb, tg, sc, 7);
-                            else forward_16<true, false, false>(p, fs, r, r2, off, tb, tg, sc, 7);
-                        }
+                        forward_group(p, fs, sh, r, r2, nacc, off, tb, tg, sc, 7);
                     }
                     else mx = max(mx, wide_out ? dgrad_16<true>(p, r, off, mx_masked) : dgrad_16<false>(p, r, off, mx_masked));
                 }
@@ -345,7 +345,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
             if (ti >= pl.tiles_per_img) { ti -= pl.tiles_per_img; ++img; }
             if (ti >= pl.tiles_per_img) { ti -= pl.tiles_per_img; ++img; }
         }
-        if (p.epilogue == kEpiDgrad) {
+        if (!fwd) {
             mx = warp_max_u32(mx);
             if (lane == 0 && mx) atomicMax(&p.dev->absmax_u32, mx);
             if (p.next_mask) {
@@ -374,9 +374,10 @@ size_t igemm_patch_smem_bytes(const IgemmParams &p, const PatchPlan &pl)
 cudaError_t launch_igemm_patch(const IgemmParams &p, const PatchPlan &pl, const CUtensorMap &map_a,
                                const CUtensorMap &map_b, int grid, cudaStream_t stream)
 {
-    cudaError_t e = cudaFuncSetAttribute(igemm_patch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    const auto kernel = p.epilogue == kEpiForward ? igemm_patch_kernel<kEpiForward> : igemm_patch_kernel<kEpiDgrad>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e != cudaSuccess) return e;
-    igemm_patch_kernel<<<grid, kPatchThreads, igemm_patch_smem_bytes(p, pl), stream>>>(p, pl, map_a, map_b);
+    kernel<<<grid, kPatchThreads, igemm_patch_smem_bytes(p, pl), stream>>>(p, pl, map_a, map_b);
     return cudaGetLastError();
 }
 

@@ -148,6 +148,9 @@ struct IgemmParams {
     // is [kc reduction rows][tile_n columns] made of tile_n / b_row atoms of b_row-byte rows, kc * b_row bytes apart
     int b_mn;
     int b_row;
+    // Tiles a CTA has in the epilogue at once (1, 2 or 4): as many accumulator buffers in tensor memory, each served by
+    // kEpilogueWarps / ep_groups warps (see plan_epilogue)
+    int ep_groups;
 };
 
 // Patch variant of the implicit GEMM for stride-1 filters (eoq_igemm_patch.cu): an M tile is `r_rows` output rows
@@ -166,7 +169,7 @@ struct PatchPlan {
     int num_a, num_b;   // ring depths (patches, weight sub-tiles)
     int b_resident;     // all weight sub-tiles of the layer stay in shared memory
 };
-constexpr int kPatchThreads = 128 + 32 * kEpilogueWarps;  // warps: 0 patch loads, 1 MMA + TMEM, 2 weight loads, 3 idle, then the epilogue
+constexpr int kPatchThreads = 128 + 32 * kEpilogueWarps;  // warps: 0 patch loads, 1 MMA + TMEM, 2 and 3 weight loads, then the epilogue
 
 size_t igemm_patch_smem_bytes(const IgemmParams &p, const PatchPlan &pl);
 cudaError_t launch_igemm_patch(const IgemmParams &p, const PatchPlan &pl, const CUtensorMap &map_a,

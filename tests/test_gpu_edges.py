@@ -105,3 +105,37 @@ def test_weight_gradient_finish(n, h, w, c_in, c_out, k, stride, pad):
                                G.dev(np.array([b1], dtype=np.int32)), g, pg, G.workspace(gd, eoq.EOQ_PASS_WGRAD))
         assert G.status_clear() == 0
         assert np.array_equal(G.host(g).astype(np.int32).reshape(-1), np.asarray(want).reshape(-1)) and pg.item() == p
+
+
+@pytest.mark.parametrize("d", [
+    oracle.ConvDesc(2, 9, 9, 64, 32, 1, 1, 1, 0),      # im2col kernel
+    oracle.ConvDesc(3, 14, 14, 64, 64, 3, 3, 1, 1),    # patch kernel, resident weights
+    oracle.ConvDesc(3, 14, 14, 256, 256, 3, 3, 1, 1),  # patch kernel, weights through the ring by two loaders
+    oracle.ConvDesc(2, 9, 9, 16, 16, 3, 3, 1, 1),      # one 16-column group: four tiles in the epilogue
+])
+@pytest.mark.parametrize("ctas", [1, 3, 0])            # four, two or one tile of a CTA in the epilogue at once
+def test_forward_rounding_and_tiles_in_the_epilogue(d, ctas):
+    """Every rounding shift of the forward chain on sums at ties and beyond 16 bits, and error back-propagation beside it."""
+    rng = np.random.Generator(np.random.Philox(key=[d.c_in, ctas]))
+    x0 = rng.choice(np.array((0, 64, -64, 127, 1), dtype=np.int8), size=(d.n, d.h, d.w, d.c_in))
+    w = rng.choice(np.array((0, 64, -64, 1), dtype=np.int8), size=(d.c_out, d.kh, d.kw, d.c_in))
+    w[::4] = 127
+    sc = rng.choice(np.array([-127, -1, 0, 1, 127], dtype=np.int8), size=(d.n, d.ho, d.wo, d.c_out))
+    gd, h = G.gdesc(d), eoq.eoq_create(0)
+    eoq.eoq_set_gemm_ctas(h, ctas)
+    for x_exp, relu in ((-15, True), (-14, True), (-13, False), (-10, True), (-8, False), (-7, True), (-7, False), (-6, True), (3, False)):
+        ref = oracle.layer_forward(d, x0, 5, w, -90, 7, sc, relu, x_exp=x_exp)
+        shape = ref["x5"].shape
+        x5, x2, mask = G.zeros(shape, torch.int8), G.zeros(shape, torch.int16), G.zeros((ref["x5"].size + 7) // 8, torch.uint8)
+        eoq.eoq_conv_fwd(h, gd, G.dev(x0), G.dev(np.array([x_exp], dtype=np.int32)), 5, G.dev(w), -90, 7, G.dev(sc), relu, x5, x2,
+                         mask, None, G.workspace(gd, eoq.EOQ_PASS_FWD))
+        assert np.array_equal(G.host(x2).astype(np.int32), ref["x2"]) and np.array_equal(G.host(x5), ref["x5"])
+        assert np.array_equal(G.unpack_mask(mask, shape), ref["mask"])
+    e3 = synth.normal_codes(shape, 1560, 0)
+    want, p, _ = oracle.sq_int(oracle.conv_dgrad_acc(d, e3, w), -9 - 7)
+    e4, pe = G.zeros(x0.shape, torch.int8), G.zeros(1, torch.int32)
+    eoq.eoq_conv_dgrad(h, gd, G.dev(e3), G.dev(np.array([-9], dtype=np.int32)), G.dev(w), e4, pe, None, None,
+                       G.workspace(gd, eoq.EOQ_PASS_DGRAD))
+    assert np.array_equal(G.host(e4).astype(np.int32), want) and pe.item() == p
+    assert eoq.eoq_last_status(h) == 0
+    eoq.eoq_destroy(h)
