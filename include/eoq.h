@@ -233,8 +233,8 @@ EOQ_API int eoq_conv_wgrad_dev(eoq_handle_t handle, const eoq_conv_desc_t *desc,
  *   untouched until the finish) and *num_parts (host) receives what the finish needs to read them.
  * eoq_wgrad_finish: for `num` layers at once (host arrays of length num; device pointers inside): the b1 error sums
  *   (b1_c[i]: the layer's code in device memory, or NULL for a layer without a bias in front of its convolution), the
- *   sum of the split-K slices plus the b1 term, and Q_g -> gq[i], *g_exp[i].  Four launches per 16 layers instead of
- *   four per layer.  workspace[i], workspace_bytes[i], num_parts[i]: as given to / returned by eoq_conv_wgrad_gemm
+ *   sum of the split-K slices plus the b1 term, and Q_g -> gq[i], *g_exp[i].  Three launches per 16 layers instead of
+ *   three per layer.  workspace[i], workspace_bytes[i], num_parts[i]: as given to / returned by eoq_conv_wgrad_gemm
  *   for that layer; descs[i], e3[i], e3_exp[i] likewise.  Results are those of eoq_conv_wgrad_dev, bit for bit.
  * EOQ_ERR_UNSUPPORTED while a reduce hook is installed (replicas exchange per layer).
  */

@@ -1,6 +1,7 @@
 // C ABI of libeoq: argument checks, TMA descriptors, launch plans.  Declarations and their contract: eoq.h.
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stddef.h>
 #include <stdio.h>
 #include <string.h>
@@ -55,6 +56,25 @@ int chunk_bytes(int c)
     for (int k = 128; k > 16; k >>= 1)
         if (c % k == 0) return k;
     return 16;
+}
+
+// Channel bytes of one K sub-tile of the patch kernels.  Their loads are tiled, so a chunk may reach past the last channel
+// (the rest arrives as zeros): an odd multiple of 16 channels takes the chunk with the least of patch loads (about 600 cycles
+// each, whatever the width) and MMAs (about 70 per tap and 32 channels), whichever bounds; 16 channels are one chunk of 32.
+int patch_chunk(int c, int taps)
+{
+    if (c % 32 == 0) return chunk_bytes(c);
+    int best = 32;
+    double best_cost = 0;
+    for (int kc = 32; kc <= 128; kc <<= 1) {
+        const int chunks = (c + kc - 1) / kc;
+        const double load = 600.0 * chunks, mma = 70.0 * taps * chunks * (kc / 32), cost = load > mma ? load : mma;
+        if (kc == 32 || cost < best_cost) {
+            best = kc;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
 
 // im2col view of an NHWC int8 tensor [n][h][w][c]: `pixels` consecutive positions of the walk that starts at
@@ -251,12 +271,11 @@ void plan_igemm(IgemmParams &p, int src_channels, int ntaps, int sm_count)
 
 // Plan of the patch variant for a stride-1 k x k correlation over a source [n][hs][ws][c_src] producing a
 // [n][hq][wq] grid with n_cols columns.  Returns false when the geometry does not suit it (then the per-tap
-// path is used): strided or 1x1 filters, fewer than 32 channels, rows too wide for a tile, or tiles that would
-// be mostly padding.
+// path is used): strided or 1x1 filters, rows too wide for a tile, or tiles that would be mostly padding.
 bool plan_patch(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, int wq, int k, int pad_src, int n_cols,
                 int sm_count)
 {
-    if (k < 2 || c_src % 32 || pad_src < 0 || pad_src > k - 1) return false;
+    if (k < 2 || c_src % 16 || pad_src < 0 || pad_src > k - 1) return false;
     const int pw = wq + k - 1;
     if (pw > kTileM) return false;
     int r = kTileM / pw;
@@ -269,8 +288,8 @@ bool plan_patch(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, int
     pl.pw = pw;
     pl.r_rows = r;
     pl.tiles_per_img = tiles_per_img;
-    p.kc = chunk_bytes(c_src);
-    pl.chunks = c_src / p.kc;
+    p.kc = patch_chunk(c_src, k * k);
+    pl.chunks = (c_src + p.kc - 1) / p.kc;
     p.chunks_per_tap = pl.chunks;
     p.ntaps = k * k;
     const int patch_rows = r + k - 1;
@@ -313,19 +332,19 @@ bool plan_patch(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, int
 // Plan of the patch variant of the weight gradient; false when the geometry does not suit it.
 bool plan_wgrad_patch(WgradPatchPlan &pl, const eoq_conv_desc_t &d, int ho, int wo, int target_ctas = kWgradTargetCtas)
 {
-    if (d.stride != 1 || d.kh != d.kw || d.kh < 2 || d.x_wmargin != 0 || d.c_in % 32 || d.c_out % 32) return false;
+    if (d.stride != 1 || d.kh != d.kw || d.kh < 2 || d.x_wmargin != 0 || d.c_in % 16 || d.c_out % 16) return false;
     if (d.pad > d.kh - 1) return false;
     memset(&pl, 0, sizeof(pl));
     pl.n_img = d.n; pl.ho = ho; pl.wo = wo; pl.c_in = d.c_in; pl.c_out = d.c_out;
     pl.kdim = d.kh; pl.pad = d.pad;
     pl.pw = wo + d.kh - 1;
     if (pl.pw > 256) return false;
-    pl.kc = chunk_bytes(d.c_in);
-    pl.chunks = d.c_in / pl.kc;
+    pl.kc = patch_chunk(d.c_in, d.kh * d.kw);
+    pl.chunks = (d.c_in + pl.kc - 1) / pl.kc;
     pl.apa = 128 / pl.kc;
     pl.accs_per_row = (d.kh + pl.apa - 1) / pl.apa;
-    pl.tile_n = chunk_bytes(d.c_out);
-    pl.n_tiles = d.c_out / pl.tile_n;
+    pl.tile_n = patch_chunk(d.c_out, d.kh * d.kw);
+    pl.n_tiles = (d.c_out + pl.tile_n - 1) / pl.tile_n;
     int rpg = 512 / (pl.tile_n * pl.accs_per_row);
     if (rpg * pl.accs_per_row > 8) rpg = 8 / pl.accs_per_row;
     if (rpg > d.kh) rpg = d.kh;
@@ -365,6 +384,116 @@ bool plan_wgrad_patch(WgradPatchPlan &pl, const eoq_conv_desc_t &d, int ho, int 
     pl.blocks_per_split = per;
     pl.num_splits = (total_blocks + per - 1) / per;
     return true;
+}
+
+// Plan of the per-tap weight gradient (strided and 1x1 filters, the filter-row path); false when the geometry is not
+// supported.  With fewer CTAs than the device has, no more splits than with all of them (the workspace holds that many).
+bool plan_wgrad(WgradParams &p, const eoq_conv_desc_t &d, const Geometry &g, int ctas)
+{
+    memset(&p, 0, sizeof(p));
+    p.P = d.n * g.ho * g.wo;
+    p.ho = g.ho;
+    p.wo = g.wo;
+    p.c_in = d.c_in;
+    p.c_out = d.c_out;
+    p.ntaps = g.taps;
+    const bool row_window = use_row_window(d, g.wo);
+    if (d.c_in == 8 && !row_window) return false;
+    p.kc = row_window ? 8 * d.c_in : chunk_bytes(d.c_in);
+    p.nc = chunk_bytes(d.c_out);
+    p.chunks_per_tap = row_window ? 1 : d.c_in / p.kc;
+    p.rows_total = g.taps * d.c_in;
+    p.subs_per_mtile = kTileM / p.kc;
+    // filter-row path: a filter row is 8 taps x c_in rows, 128 / (8 c_in) filter rows per M tile
+    p.num_m_tiles = row_window ? (d.kh * p.kc + kTileM - 1) / kTileM : (p.rows_total + kTileM - 1) / kTileM;
+    if (row_window) {
+        p.ntaps = d.kh;
+        p.row_window_kw = d.kw;
+    }
+    p.pixels_per_stage = 64;
+    const int px = p.pixels_per_stage;
+    const int total_stages = (p.P + px - 1) / px;
+    // a 64-pixel stage adds at most 64 * 127 * 127 to an int32 partial sum
+    const int max_stages_exact = 1024;
+    // Columns, M tiles side by side in one CTA (they share the stage's error tile) and splits of the pixel range are chosen
+    // together.  In SM cycles, as measured: a TMA row 3.1, an MMA 57 to 128, a column of an M tile in the epilogue 8; a slice
+    // is written and read back at 2,500 bytes per cycle of the whole device.  With 64-bit atomics into one buffer and at
+    // least 8 stages per CTA, the 1024 -> 256 layer of 14 x 14 pixels took 24.4 us at batch 32 (the atomics 17 of them).
+    // Twice the CTAs asked for, one per SM at most: the caps that callers set halve a GEMM that has a neighbour on the other
+    // SMs, and this kernel also ends the backward pass, alone.
+    const int cap = 2 * ctas < kWgradTargetCtas ? 2 * ctas : kWgradTargetCtas;
+    double best = 0;
+    int best_splits = 0;
+    for (int cuts = 1; cuts <= 8; cuts = cuts < 4 ? cuts + 1 : cuts * 2) {
+        const int tn = ((d.c_out + cuts - 1) / cuts + p.nc - 1) / p.nc * p.nc;
+        if (tn > 256) continue;
+        if (cuts > 1 && tn >= d.c_out) break;
+        const int n_tiles = (d.c_out + tn - 1) / tn, b_subs = tn / p.nc;
+        for (int mpc = 1; mpc <= 8 && mpc <= p.num_m_tiles && mpc * tn <= 512; ++mpc) {
+            const size_t stage_bytes = (size_t)px * (mpc * kTileM + tn);
+            if (mpc > 1 && 3 * stage_bytes > 200 * 1024) break;
+            const int groups = (p.num_m_tiles + mpc - 1) / mpc, tiles = groups * n_tiles;
+            const int waves = (tiles + cap - 1) / cap;
+            const double load = 3.1 * px * (mpc * p.subs_per_mtile + b_subs), mma = (px / 32) * mpc * (tn > 114 ? tn * 0.5 : 57.0);
+            const double per_stage = load > mma ? load : mma, per_slice = (double)p.rows_total * d.c_out * 8 / 2500.0;
+            // waves * (total / s) * per_stage + s * per_slice is smallest near s = sqrt(total * per_stage / per_slice)
+            const int most = tiles > cap ? 1 : cap / tiles;
+            int splits = (int)(sqrt((double)total_stages * per_stage / per_slice) + 0.5);
+            splits = splits < 1 ? 1 : (splits > most ? most : splits);
+            if (splits > total_stages) splits = total_stages;
+            int per = (total_stages + splits - 1) / splits;
+            if (per > max_stages_exact) per = max_stages_exact;
+            splits = (total_stages + per - 1) / per;
+            const double cost = waves * (per * per_stage + 8.0 * mpc * tn) + splits * per_slice;
+            if (best_splits == 0 || cost < best) {
+                best = cost;
+                best_splits = splits;
+                p.tile_n = tn;
+                p.num_n_tiles = n_tiles;
+                p.mtiles_per_cta = mpc;
+                p.num_m_groups = groups;
+                p.stages_per_split = per;
+                p.num_k_splits = splits;
+                const int stages = (int)(200 * 1024 / stage_bytes);
+                p.num_stages = stages > 8 ? 8 : (stages < 2 ? 2 : stages);
+            }
+        }
+    }
+    if (cap < kWgradTargetCtas) {
+        WgradParams full;
+        plan_wgrad(full, d, g, kWgradTargetCtas);
+        if (p.num_k_splits > full.num_k_splits) {
+            p.stages_per_split = full.stages_per_split;
+            p.num_k_splits = full.num_k_splits;
+        }
+    }
+    p.src_stride = d.stride;
+    p.base_h = -d.pad;
+    if (row_window) {
+        p.src_stride_w = 1;
+        p.base_w = 0;
+        for (int t = 0; t < d.kh; ++t) {
+            p.tap_dh[t] = (unsigned char)t;
+            p.tap_dw[t] = 0;
+        }
+    } else {
+        p.src_stride_w = d.stride;
+        p.base_w = d.x_wmargin - d.pad;
+        for (int t = 0; t < g.taps; ++t) {
+            p.tap_dh[t] = (unsigned char)(t / d.kw);
+            p.tap_dw[t] = (unsigned char)(t % d.kw);
+        }
+    }
+    return true;
+}
+
+// int32 slices of partial sums the weight-gradient GEMM leaves, at most
+int wgrad_slices(const eoq_conv_desc_t &d, const Geometry &g)
+{
+    WgradPatchPlan wp;
+    if (plan_wgrad_patch(wp, d, g.ho, g.wo)) return wp.num_splits;
+    WgradParams p;
+    return plan_wgrad(p, d, g, kWgradTargetCtas) ? p.num_k_splits : 0;
 }
 
 }  // namespace
@@ -610,8 +739,7 @@ extern "C" int eoq_workspace_size(const eoq_conv_desc_t *desc, int pass, size_t 
             *bytes = round256(g.w_elems) + round256(g.in_elems * sizeof(int32_t));
             return EOQ_OK;
         case EOQ_PASS_WGRAD: {  // per-tap error sums, reduction cell, int64 sums, split-K slices
-            WgradPatchPlan wp;
-            const size_t slices = plan_wgrad_patch(wp, *desc, g.ho, g.wo) ? (size_t)wp.num_splits * g.w_elems * sizeof(int32_t) : 0;
+            const size_t slices = (size_t)wgrad_slices(*desc, g) * g.w_elems * sizeof(int32_t);
             *bytes = kTapReplicas * round256((size_t)desc->c_out * g.taps * sizeof(long long)) + 256 +
                      round256(g.w_elems * sizeof(long long)) + round256(slices);
             return EOQ_OK;
@@ -668,7 +796,7 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
     memset(&p, 0, sizeof(p));
     PatchPlan pl;
     memset(&pl, 0, sizeof(pl));
-    const bool patch = d.stride == 1 && d.kh == d.kw && d.x_wmargin == 0 && !x_exp &&
+    const bool patch = d.stride == 1 && d.kh == d.kw && d.x_wmargin == 0 &&
                        plan_patch(p, pl, d.n, d.c_in, g.ho, g.wo, d.kh, d.pad, d.c_out, h->sm_count);
     p.M = d.n * g.ho * g.wo;
     p.N = d.c_out;
@@ -1194,7 +1322,7 @@ static FinishItem finish_item(const eoq_conv_desc_t &d, const Geometry &g, const
     it.max_cell = w.max_cell;
     it.acc = w.acc;
     it.num_parts = num_parts;
-    it.parts = num_parts > 0 ? w.parts : nullptr;
+    it.parts = w.parts;
     it.g = gq;
     it.g_exp = g_exp;
     it.n = g.w_elems;
@@ -1208,7 +1336,7 @@ static FinishItem finish_item(const eoq_conv_desc_t &d, const Geometry &g, const
 
 // Weight gradient behind eoq_conv_wgrad and eoq_conv_wgrad_dev: b1 is the host code b1_c, or the code at b1_dev.
 // num_parts_out (eoq_conv_wgrad_gemm): the GEMM alone; the sums stay in the workspace for eoq_wgrad_finish and
-// *num_parts_out tells it how many int32 slices there are (0: the GEMM added into the int64 sums).
+// *num_parts_out tells it how many int32 slices there are.
 static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const int8_t *e3, const int32_t *e3_exp,
                            const int8_t *x, int32_t b1_c, const int32_t *b1_dev, int8_t *gq, int32_t *g_exp,
                            int64_t *acc_dump, void *workspace, size_t workspace_bytes, void *stream, int *num_parts_out = nullptr)
@@ -1260,86 +1388,15 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     }
 
     WgradParams p;
-    memset(&p, 0, sizeof(p));
-    p.P = d.n * g.ho * g.wo;
-    p.ho = g.ho;
-    p.wo = g.wo;
-    p.c_in = d.c_in;
-    p.c_out = d.c_out;
-    p.ntaps = g.taps;
-    const bool row_window = use_row_window(d, g.wo);
-    if (d.c_in == 8 && !row_window) return EOQ_ERR_UNSUPPORTED;
+    if (!plan_wgrad(p, d, g, h->gemm_ctas)) return EOQ_ERR_UNSUPPORTED;
+    const bool row_window = p.row_window_kw != 0;
     const int w_mem = d.w + 2 * d.x_wmargin;
-    p.kc = row_window ? 8 * d.c_in : chunk_bytes(d.c_in);
-    p.nc = chunk_bytes(d.c_out);
-    p.chunks_per_tap = row_window ? 1 : d.c_in / p.kc;
-    p.rows_total = g.taps * d.c_in;
-    p.subs_per_mtile = kTileM / p.kc;
-    // filter-row path: a filter row is 8 taps x c_in rows, 128 / (8 c_in) filter rows per M tile
-    p.num_m_tiles = row_window ? (d.kh * p.kc + kTileM - 1) / kTileM : (p.rows_total + kTileM - 1) / kTileM;
-    if (row_window) {
-        p.ntaps = d.kh;
-        p.row_window_kw = d.kw;
-    }
-    p.tile_n = d.c_out < 256 ? d.c_out : 256;
-    if (p.tile_n % p.nc) p.tile_n = (p.tile_n / p.nc) * p.nc;
-    p.num_n_tiles = (d.c_out + p.tile_n - 1) / p.tile_n;
-    p.pixels_per_stage = 64;
-    // M tiles accumulated side by side by one CTA share the stage's error tile (fewer TMA rows per MMA): as many
-    // as tensor memory (512 columns) and three pipeline stages of shared memory allow
-    {
-        int mpc = 512 / p.tile_n;
-        const size_t a_mtile = (size_t)p.subs_per_mtile * p.pixels_per_stage * p.kc, b_tile = (size_t)p.tile_n * p.pixels_per_stage;
-        while (mpc > 1 && 3 * (mpc * a_mtile + b_tile) > 200 * 1024) --mpc;
-        if (mpc > p.num_m_tiles) mpc = p.num_m_tiles;
-        p.mtiles_per_cta = mpc < 1 ? 1 : mpc;
-        p.num_m_groups = (p.num_m_tiles + p.mtiles_per_cta - 1) / p.mtiles_per_cta;
-    }
-    const int total_stages = (p.P + p.pixels_per_stage - 1) / p.pixels_per_stage;
-    // a 64-pixel stage adds at most 64 * 127 * 255 to an int32 partial sum: cap the stages one CTA runs
-    const int max_stages_exact = 1024;
-    const int tiles = p.num_m_groups * p.num_n_tiles;
-    int splits = (2 * h->gemm_ctas + tiles - 1) / tiles;
-    const int max_splits = (total_stages + 7) / 8;  // at least 8 stages of work per CTA
-    if (splits > max_splits) splits = max_splits;
-    if (splits < 1) splits = 1;
-    int per = (total_stages + splits - 1) / splits;
-    if (per > max_stages_exact) per = max_stages_exact;
-    splits = (total_stages + per - 1) / per;
-    p.stages_per_split = per;
-    p.num_k_splits = splits;
-    const size_t stage_bytes = (size_t)p.mtiles_per_cta * p.subs_per_mtile * p.pixels_per_stage * p.kc +
-                               (size_t)p.tile_n * p.pixels_per_stage;
-    int stages = (int)((200 * 1024) / stage_bytes);
-    p.num_stages = stages > 8 ? 8 : (stages < 2 ? 2 : stages);
-    p.src_stride = d.stride;
-    p.base_h = -d.pad;
-    if (row_window) {
-        p.src_stride_w = 1;
-        p.base_w = 0;
-        for (int t = 0; t < d.kh; ++t) {
-            p.tap_dh[t] = (unsigned char)t;
-            p.tap_dw[t] = 0;
-        }
-    } else {
-        p.src_stride_w = d.stride;
-        p.base_w = d.x_wmargin - d.pad;
-        for (int t = 0; t < g.taps; ++t) {
-            p.tap_dh[t] = (unsigned char)(t / d.kw);
-            p.tap_dw[t] = (unsigned char)(t % d.kw);
-        }
-    }
-    p.acc = w.acc;
+    p.partials = w.parts;
     p.zero = reinterpret_cast<int4 *>(w.tap_sums);
     p.zero_n16 = (unsigned)(w.zero_bytes / 16);
     p.dev = h->dev;
 
-    cudaError_t e = cudaSuccess;
-    if (!h->gemm_only) {
-        ProfScope aux(h, EOQ_PROF_WGRAD_AUX, s);
-        e = cudaMemsetAsync(w.acc, 0, w.acc_bytes, s);  // the GEMM adds into the int64 sums with atomics
-    }
-    if (e != cudaSuccess) return record(h, e);
+    cudaError_t e;
     CUtensorMap map_x, map_e;
     if (!make_matrix_map(&map_e, e3, (size_t)p.P, d.c_out, p.nc, p.pixels_per_stage)) return EOQ_ERR_UNSUPPORTED;
     if (row_window ? !make_row_window_map(&map_x, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, g.wo, g.ho, d.stride, d.pad,
@@ -1352,9 +1409,9 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
         ProfScope prof(h, EOQ_PROF_WGRAD, s);
         e = launch_wgrad(p, map_x, map_e, s);
     }
-    if (num_parts_out) *num_parts_out = 0;
+    if (num_parts_out) *num_parts_out = p.num_k_splits;
     if (e != cudaSuccess || gemm_only) return record(h, e);
-    return finish(0);
+    return finish(p.num_k_splits);
 }
 
 extern "C" int eoq_conv_wgrad(eoq_handle_t handle, const eoq_conv_desc_t *desc, const int8_t *e3,
@@ -1393,7 +1450,7 @@ extern "C" int eoq_wgrad_finish(eoq_handle_t handle, int num, const eoq_conv_des
         Geometry g;
         int st = check_desc(&descs[i], &g);
         if (st != EOQ_OK) return st;
-        if (!e3[i] || !e3_exp[i] || !gq[i] || !g_exp[i] || num_parts[i] < 0) return EOQ_ERR_BAD_ARG;
+        if (!e3[i] || !e3_exp[i] || !gq[i] || !g_exp[i] || num_parts[i] < 1) return EOQ_ERR_BAD_ARG;
         if (!aligned16(e3[i]) || !aligned16(gq[i])) return EOQ_ERR_ALIGNMENT;
         if ((st = check_workspace(&descs[i], EOQ_PASS_WGRAD, workspace[i], workspace_bytes[i])) != EOQ_OK) return st;
         const BorderClasses bc = border_classes(descs[i], g);

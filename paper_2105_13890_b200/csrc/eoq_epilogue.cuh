@@ -122,6 +122,16 @@ __device__ __forceinline__ const int32_t *stage_b1_table(const IgemmParams &p, i
     return ts;
 }
 
+// The shift that brings a sum to exponent -14: 7, or what the exponent of an input behind the input quantizer asks for.
+__device__ __forceinline__ int input_shift(const IgemmParams &p)
+{
+    if (!p.x_exp) return 7;
+    const int shift = -__ldg(p.x_exp);
+    if (shift <= 31 && shift >= -16) return shift;
+    if (blockIdx.x == 0 && (threadIdx.x & 31) == 0) atomicOr(&p.dev->status, EOQ_DEV_RANGE);
+    return max(-16, min(31, shift));
+}
+
 // The rounding of x2 = R(acc / 2^shift) for shifts 0 to 7 (7: an input at exponent -7; less behind the input quantizer).
 struct FwdShift {
     bool ok;

@@ -1,6 +1,6 @@
 // What follows the weight-gradient GEMM (arXiv 2105.13890, Sec. 3.2.1: g_w = Q_g(e3 * x1) with x1 = x0 + Q_b(b1)), for one
 // layer or for many layers in the same three launches: the b1 error sums (one pass over e3), the exact sums (split-K slices
-// or the GEMM's 64-bit sums, plus the b1 term) reduced to their maximum, and Q_g.  Blocks find their layer by their index.
+// plus the b1 term) reduced to their maximum, and Q_g.  Blocks find their layer by their index.
 // The cells these kernels add into (tap sums, maximum) are cleared by the GEMM kernel in front.
 #include "eoq_device.cuh"
 #include "eoq_internal.h"
@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_cons
 // ------------------------------------------------------------------ exact sums and their maximum
 // A thread owns four neighbouring weights (c_in is a multiple of 4: they share their (oc, tap)).  With more than
 // kDirectParts slices a block is (256 / groups) such quads x `groups` slice groups that meet in shared memory, and the sums
-// are written once, as int32 when they provably fit; with fewer slices, or 64-bit sums from the GEMM, nothing is written:
-// the coding pass forms them again, which costs fewer bytes than a round trip.  The 2.4 M weights of the 512-channel 3 x 3
+// are written once, as int32 when they provably fit; with fewer slices nothing is written: the coding pass forms them again,
+// which costs fewer bytes than a round trip.  The 2.4 M weights of the 512-channel 3 x 3
 // layer: sums 18.9 -> 10.9 us, codes 7.8 -> 4.3 us against one weight per thread, four 64-bit tap sums read for each of
 // them and 64-bit sums written and read back.
 constexpr int kDirectParts = 2;
@@ -244,26 +244,17 @@ __device__ __forceinline__ long long finish_b1_term(const FinishItem &it, int b1
     return (long long)b1 * s;
 }
 
-// the quad's sums without the b1 term, from at most kDirectParts slices or the 64-bit sums
+// the quad's sums without the b1 term, from at most kDirectParts slices
 __device__ __forceinline__ void finish_direct(const FinishItem &it, uint32_t q, long long (&v)[4])
 {
-    if (it.parts) {
-        int4 a[kDirectParts];
+    int4 a[kDirectParts];
 #pragma unroll
-        for (int s = 0; s < kDirectParts; ++s)
-            a[s] = s < it.num_parts ? __ldg(reinterpret_cast<const int4 *>(it.parts + (size_t)s * it.n) + q) : make_int4(0, 0, 0, 0);
-        v[0] = (long long)a[0].x + a[1].x;
-        v[1] = (long long)a[0].y + a[1].y;
-        v[2] = (long long)a[0].z + a[1].z;
-        v[3] = (long long)a[0].w + a[1].w;
-    } else {
-        const longlong2 lo = __ldg(reinterpret_cast<const longlong2 *>(it.acc) + 2 * (size_t)q);
-        const longlong2 hi = __ldg(reinterpret_cast<const longlong2 *>(it.acc) + 2 * (size_t)q + 1);
-        v[0] = lo.x;
-        v[1] = lo.y;
-        v[2] = hi.x;
-        v[3] = hi.y;
-    }
+    for (int s = 0; s < kDirectParts; ++s)
+        a[s] = s < it.num_parts ? __ldg(reinterpret_cast<const int4 *>(it.parts + (size_t)s * it.n) + q) : make_int4(0, 0, 0, 0);
+    v[0] = (long long)a[0].x + a[1].x;
+    v[1] = (long long)a[0].y + a[1].y;
+    v[2] = (long long)a[0].z + a[1].z;
+    v[3] = (long long)a[0].w + a[1].w;
 }
 
 __global__ void __launch_bounds__(kThreads) finish_sums_kernel(const __grid_constant__ FinishBatch b)
@@ -434,7 +425,7 @@ static void plan_finish_item(FinishItem &it, int sm_count, bool alone)
     it.rows_per_block = rpb;
     it.tap_grid_x = (rows + rpb - 1) / rpb;
     it.tap_blocks = it.use_b1 ? it.tap_grid_x * slabs : 0;
-    it.direct = !it.parts || it.num_parts <= kDirectParts;
+    it.direct = it.num_parts <= kDirectParts;
     it.groups = it.direct ? 1 : (it.num_parts >= 32 ? 8 : (it.num_parts >= 8 ? 4 : 1));
     const size_t quads = (size_t)it.n / 4, bw = kThreads / it.groups;
     size_t fb = (quads + bw - 1) / bw;

@@ -232,14 +232,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         const int32_t *ts = fwd ? stage_b1_table(p, fs.b1, smem_raw + (smem_base - ptx::smem_u32(smem_raw)) + p.num_stages * stage_bytes,
                                                  (int)threadIdx.x - 128, 32 * kEpilogueWarps)
                                 : nullptr;
-        int shift = 7;
-        if (fwd && p.x_exp) {
-            shift = -__ldg(p.x_exp);
-            if (shift > 31 || shift < -16) {
-                if (lane == 0) atomicOr(&p.dev->status, EOQ_DEV_RANGE);
-                shift = max(-16, min(31, shift));
-            }
-        }
+        const int shift = input_shift(p);
         const FwdShift sh = forward_shift(p, shift);
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
         const bool wide_out = (reinterpret_cast<uintptr_t>(p.acc_out) & 31) == 0;   // 256-bit stores of the exact sums

@@ -277,7 +277,8 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
         const int32_t *ts = fwd ? stage_b1_table(p, fs.b1, smem_raw + (smem_base - ptx::smem_u32(smem_raw)) + table_off,
                                                  (int)threadIdx.x - 128, 32 * kEpilogueWarps)
                                 : nullptr;
-        const FwdShift sh = forward_shift(p, 7);
+        const int shift = fwd ? input_shift(p) : 7;
+        const FwdShift sh = forward_shift(p, shift);
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
         const bool wide_out = (reinterpret_cast<uintptr_t>(p.acc_out) & 31) == 0;   // 256-bit stores of the exact sums
         bool ok = true;
@@ -326,9 +327,8 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
                 }
                 if (valid && col < p.N) {
                     if (fwd) {
-                        forward_group(p, fs, sh, r, r2, nacc, off, tb, tg, sc, 7);
-                    }
-                    else mx = max(mx, wide_out ? dgrad_16<true>(p, r, off, mx_masked) : dgrad_16<false>(p, r, off, mx_masked));
+                        forward_group(p, fs, sh, r, r2, nacc, off, tb, tg, sc, shift);
+                    } else mx = max(mx, wide_out ? dgrad_16<true>(p, r, off, mx_masked) : dgrad_16<false>(p, r, off, mx_masked));
                 }
                 sc = sc_next;
                 if (tb) tb += 16;

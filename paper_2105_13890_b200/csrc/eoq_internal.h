@@ -163,7 +163,7 @@ struct PatchPlan {
     int pw;             // patch width = wq + kdim - 1
     int r_rows;         // output rows per tile
     int tiles_per_img;
-    int chunks;         // source channels / kc
+    int chunks;         // source channels / kc, rounded up
     int a_bytes;        // bytes of one patch buffer (multiple of 1024)
     int a_box_bytes;    // bytes one patch load delivers
     int num_a, num_b;   // ring depths (patches, weight sub-tiles)
@@ -202,7 +202,7 @@ struct WgradParams {
     int src_stride, src_stride_w, base_h, base_w;
     int row_window_kw;   // 0, or the filter width when an M tile is one filter row of 8 x 16 bytes (7 real taps of 8)
     unsigned char tap_dh[kMaxTaps], tap_dw[kMaxTaps];
-    long long *acc;      // [c_out][taps][c_in] int64, zeroed before launch
+    int32_t *partials;   // [num_k_splits][c_out][taps][c_in] partial sums, a slice per split
     int4 *zero;          // the cells of the kernels that follow (tap sums, maximum): cleared here, zero_n16 groups of 16 bytes
     unsigned zero_n16;
     DeviceState *dev;

@@ -3,7 +3,8 @@
 // The reduction runs over pixels, which is the slow axis of both NHWC operands, so both are fed to
 // tcgen05.mma as MN-major tiles: a TMA im2col load brings [pixels][channels] of the activation for one
 // filter tap, a tiled TMA load brings [pixels][channels] of the error.  The pixel range is split across
-// CTAs (split-K); int32 partial sums leave TMEM and are combined exactly with 64-bit atomics.
+// CTAs (split-K); each leaves its int32 partial sums in the slice of its split, and a finishing kernel adds the slices in
+// 64 bits.
 // Roles: warps 0, 2, 3 TMA producers (a thread gets a TMA instruction out only every few hundred cycles, threads
 // of different warps issue side by side: the loads of every stage are dealt out over three producers), warp 1
 // MMA issuer and TMEM owner, warps 4-7 epilogue.  All waits are bounded.
@@ -187,10 +188,13 @@ wgrad_kernel(const __grid_constant__ WgradParams p, const __grid_constant__ CUte
             for (uint32_t i = 0; i < kSpinLimit; ++i)
                 if (ptx::mbar_try_wait(done_bar, 0)) break;
     } else {
+        // Every lane has a row of the accumulator, neighbouring lanes neighbouring weights of one output channel: a store per
+        // column and warp, 128 bytes wide.
         const int quad = warp & 3;
-        bool ok = __all_sync(0xffffffffu, wait_bar(done_bar, 0, ctx));
-        if (ok && my_stages > 0) ptx::tc_fence_after();
-        for (int jm = 0; jm < my_mtiles && ok && my_stages > 0; ++jm) {
+        int32_t *slice = p.partials + (size_t)ks * p.c_out * p.rows_total;
+        const bool ok = __all_sync(0xffffffffu, wait_bar(done_bar, 0, ctx));
+        if (ok) ptx::tc_fence_after();
+        for (int jm = 0; jm < my_mtiles && ok; ++jm) {
             const int mt = mt0 + jm;
             int row = mt * kTileM + quad * 32 + lane;  // (tap, ic) flattened: tap * c_in + ic
             bool valid = row < p.rows_total;
@@ -204,20 +208,17 @@ wgrad_kernel(const __grid_constant__ WgradParams p, const __grid_constant__ CUte
             const uint32_t t_row = tmem_base + jm * p.tile_n + ((uint32_t)(quad * 32) << 16);
             for (int c0 = 0; c0 < p.tile_n; c0 += 32) {
                 uint32_t r[32];
-                const int ncol = min(32, p.tile_n - c0);
+                const int oc0 = nt * p.tile_n + c0;
+                const int ncol = min(min(32, p.tile_n - c0), p.c_out - oc0);   // (multiples of 16)
+                if (ncol <= 0) break;
                 if (ncol == 32) ptx::tmem_ld_32x32(t_row + c0, r);
                 else ptx::tmem_ld_32x16(t_row + c0, r);
                 ptx::tmem_ld_wait();
                 if (valid) {
+                    int32_t *dst = slice + (size_t)oc0 * p.rows_total + row;
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int oc = nt * p.tile_n + c0 + j;
-                        if (j < ncol && oc < p.c_out) {
-                            const long long v = (int32_t)r[j];
-                            if (v) atomicAdd(reinterpret_cast<unsigned long long *>(p.acc + (size_t)oc * p.rows_total + row),
-                                             (unsigned long long)v);
-                        }
-                    }
+                    for (int j = 0; j < 32; ++j)
+                        if (j < 16 || ncol == 32) dst[(size_t)j * p.rows_total] = (int32_t)r[j];
                 }
             }
         }

@@ -168,10 +168,10 @@ wgrad_patch_kernel(const __grid_constant__ WgradPatchPlan pl, const __grid_const
             ptx::tc_fence_after();
             for (int j = 0; j < num_acc; ++j) {
                 const int a = row0 + j / pl.accs_per_row, b = (j % pl.accs_per_row) * pl.apa + atom;
-                const bool valid = b < pl.kdim;
+                const bool valid = b < pl.kdim && c * pl.kc + ch < pl.c_in;   // (a chunk may reach past the last channel)
                 const size_t row = (size_t)(a * pl.kdim + b) * pl.c_in + c * pl.kc + ch;
                 const uint32_t t_row = tmem_base + j * pl.tile_n + ((uint32_t)(quad * 32) << 16);
-                for (int c0 = 0; c0 < pl.tile_n; c0 += 16) {
+                for (int c0 = 0; c0 < pl.tile_n && nt * pl.tile_n + c0 < pl.c_out; c0 += 16) {
                     uint32_t v[32];
                     if (my_blocks > 0) {
                         ptx::tmem_ld_32x16(t_row + c0, v);

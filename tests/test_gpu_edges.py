@@ -139,3 +139,40 @@ def test_forward_rounding_and_tiles_in_the_epilogue(d, ctas):
     assert np.array_equal(G.host(e4).astype(np.int32), want) and pe.item() == p
     assert eoq.eoq_last_status(h) == 0
     eoq.eoq_destroy(h)
+
+
+@pytest.mark.parametrize("d", [
+    oracle.ConvDesc(2, 12, 13, 16, 16, 3, 3, 1, 1),    # half a chunk of 32 channels
+    oracle.ConvDesc(3, 9, 12, 48, 80, 3, 3, 1, 1),     # chunks of 64 and 32 channels, the last one ragged
+    oracle.ConvDesc(2, 8, 9, 112, 144, 3, 3, 1, 1),    # chunks of 128 and 32
+    oracle.ConvDesc(1, 11, 10, 208, 272, 3, 3, 1, 1),  # several chunks, two column tiles
+    oracle.ConvDesc(2, 10, 11, 16, 48, 5, 5, 1, 2),
+    oracle.ConvDesc(2, 9, 8, 48, 80, 3, 3, 2, 1),      # one tap at a time: fewer pixels than a stage per split
+    oracle.ConvDesc(6, 14, 14, 256, 272, 1, 1, 1, 0),  # splits and column tiles chosen together, a ragged column tile
+    oracle.ConvDesc(9, 15, 13, 64, 528, 1, 1, 2, 0),
+], ids=lambda d: f"c{d.c_in}-{d.c_out}_k{d.kh}s{d.stride}")
+@pytest.mark.parametrize("ctas", [0, 5])
+def test_odd_channel_counts(d, ctas):
+    """Channel counts that are odd multiples of 16, all three passes; the weight gradient with all and with few CTAs."""
+    x, sc = synth.int8_uniform((d.n, d.h, d.w, d.c_in), 1570, 0), synth.int8_uniform((d.n, d.ho, d.wo, d.c_out), 1570, 1)
+    w, e3 = synth.int8_uniform((d.c_out, d.kh, d.kw, d.c_in), 1570, 2, -30, 30), synth.normal_codes((d.n, d.ho, d.wo, d.c_out), 1570, 3)
+    gd, h = G.gdesc(d), eoq.eoq_create(0)
+    eoq.eoq_set_gemm_ctas(h, ctas)
+    ref = oracle.layer_forward(d, x, -4, w, 90, 5, sc, True)
+    x5, x2, mask = G.zeros(sc.shape, torch.int8), G.zeros(sc.shape, torch.int16), G.zeros((sc.size + 7) // 8, torch.uint8)
+    eoq.eoq_conv_fwd(h, gd, G.dev(x), None, -4, G.dev(w), 90, 5, G.dev(sc), True, x5, x2, mask, None, G.workspace(gd, eoq.EOQ_PASS_FWD))
+    assert np.array_equal(G.host(x5), ref["x5"]) and np.array_equal(G.host(x2).astype(np.int32), ref["x2"])
+    assert np.array_equal(G.unpack_mask(mask, sc.shape), ref["mask"])
+    pe3 = G.dev(np.array([-9], dtype=np.int32))
+    want, p, _ = oracle.sq_int(oracle.conv_dgrad_acc(d, e3, w), -9 - 7)
+    e4, pe = G.zeros(x.shape, torch.int8), G.zeros(1, torch.int32)
+    eoq.eoq_conv_dgrad(h, gd, G.dev(e3), pe3, G.dev(w), e4, pe, None, None, G.workspace(gd, eoq.EOQ_PASS_DGRAD))
+    assert np.array_equal(G.host(e4).astype(np.int32), want) and pe.item() == p
+    want, p, _ = oracle.sq_int(oracle.conv_wgrad_acc(d, e3, x, -4), -9 - 7)
+    g, pg = G.zeros(w.shape, torch.int8), G.zeros(1, torch.int32)
+    ws = G.workspace(gd, eoq.EOQ_PASS_WGRAD)
+    ws.fill_(0x55)   # the slices need no clearing
+    eoq.eoq_conv_wgrad(h, gd, G.dev(e3), pe3, G.dev(x), -4, g, pg, None, ws)
+    assert np.array_equal(G.host(g).astype(np.int32), want) and pg.item() == p
+    assert eoq.eoq_last_status(h) == 0
+    eoq.eoq_destroy(h)
