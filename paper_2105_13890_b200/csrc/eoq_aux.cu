@@ -43,6 +43,7 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
                             const uint8_t *__restrict__ next_mask, const int16_t *__restrict__ next_x2, const int32_t *next_gamma,
                             int8_t *__restrict__ e3, int32_t *e3_exp, long long *sum_e1, long long *sum_e1x2, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     const JoinShift j = join_shift(__ldg(a_exp), __ldg(b_exp));
     unsigned long long mx = 0, mxm = 0;
     long long sum = 0, s1 = 0, s2 = 0;
@@ -129,6 +130,7 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
             }
         }
     }
+    ptx::grid_dep_launch();
     if (kPass == 0) {
         mx = block_max_u64(mx > mx32 ? mx : (unsigned long long)mx32);
         if (kNext) mxm = block_max_u64(mxm > mxm32 ? mxm : (unsigned long long)mxm32);
@@ -176,6 +178,7 @@ __device__ __forceinline__ unsigned long long mix64_aux(unsigned long long z)
 __global__ void scalar_update_kernel(const __grid_constant__ ScalarBatch b, int32_t lr_mant, int32_t lr_exp, int stochastic,
                                      unsigned long long seed, const unsigned long long *step_dev, unsigned long long step)
 {
+    ptx::grid_dep_wait_launch_small();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= b.num) return;
     const ScalarItem &it = b.item[i];
@@ -231,20 +234,20 @@ cudaError_t launch_join(const int8_t *a, const int32_t *a_exp, const int8_t *b, 
     const size_t n16 = n_el / 16;
     const int blocks = blocks_for(n16, sm_count, 8);
     if (e3) {
-        join_kernel<0, true><<<blocks, kThreads, 0, st>>>(a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, next_mask, next_x2,
+        launch_chained(join_kernel<0, true>, blocks, kThreads, 0, st, a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, next_mask, next_x2,
                                                           next_gamma, e3, e3_exp, sum_e1, sum_e1x2, dev);
         hook(&dev->absmax_u64, 1, EOQ_REDUCE_I64, EOQ_REDUCE_MAX, st);
         hook(&dev->absmax2_u64, 1, EOQ_REDUCE_I64, EOQ_REDUCE_MAX, st);
-        join_kernel<1, true><<<blocks, kThreads, 0, st>>>(a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, next_mask, next_x2,
+        launch_chained(join_kernel<1, true>, blocks, kThreads, 0, st, a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, next_mask, next_x2,
                                                           next_gamma, e3, e3_exp, sum_e1, sum_e1x2, dev);
         if (sum_out) hook(sum_out, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, st);
         if (sum_e1) hook(sum_e1, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, st);
         if (sum_e1x2) hook(sum_e1x2, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, st);
     } else {
-        join_kernel<0, false><<<blocks, kThreads, 0, st>>>(a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, nullptr, nullptr,
+        launch_chained(join_kernel<0, false>, blocks, kThreads, 0, st, a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, nullptr, nullptr,
                                                            nullptr, nullptr, nullptr, nullptr, nullptr, dev);
         hook(&dev->absmax_u64, 1, EOQ_REDUCE_I64, EOQ_REDUCE_MAX, st);
-        join_kernel<1, false><<<blocks, kThreads, 0, st>>>(a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, nullptr, nullptr,
+        launch_chained(join_kernel<1, false>, blocks, kThreads, 0, st, a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, nullptr, nullptr,
                                                            nullptr, nullptr, nullptr, nullptr, nullptr, dev);
         if (sum_out) hook(sum_out, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, st);
     }
@@ -258,10 +261,10 @@ cudaError_t launch_join_second(const int8_t *a, const int32_t *a_exp, const int8
     const size_t n16 = n_el / 16;
     const int blocks = blocks_for(n16, sm_count, 8);
     if (next)
-        join_kernel<1, true><<<blocks, kThreads, 0, st>>>(a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, next->mask, next->x2,
+        launch_chained(join_kernel<1, true>, blocks, kThreads, 0, st, a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, next->mask, next->x2,
                                                           next->gamma, next->e3, next->e3_exp, next->sum_e1, next->sum_e1x2, dev);
     else
-        join_kernel<1, false><<<blocks, kThreads, 0, st>>>(a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, nullptr, nullptr,
+        launch_chained(join_kernel<1, false>, blocks, kThreads, 0, st, a, a_exp, b, b_exp, mask_b, n16, out, out_exp, sum_out, nullptr, nullptr,
                                                            nullptr, nullptr, nullptr, nullptr, nullptr, dev);
     return cudaGetLastError();
 }
@@ -269,7 +272,7 @@ cudaError_t launch_join_second(const int8_t *a, const int32_t *a_exp, const int8
 cudaError_t launch_scalar_update(const ScalarBatch &b, int32_t lr_mant, int32_t lr_exp, int stochastic, uint64_t seed,
                                  const unsigned long long *step_dev, uint64_t step, cudaStream_t st)
 {
-    scalar_update_kernel<<<(b.num + 63) / 64, 64, 0, st>>>(b, lr_mant, lr_exp, stochastic, seed, step_dev, step);
+    launch_chained(scalar_update_kernel, (b.num + 63) / 64, 64, 0, st, b, lr_mant, lr_exp, stochastic, seed, step_dev, step);
     return cudaGetLastError();
 }
 

@@ -177,6 +177,20 @@ namespace ptx {
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// Chained launches (see launch_chained): the work of the kernels in front on the stream is complete and visible behind the
+// wait; the next kernel may be brought up once every block has called grid_dep_launch or ended.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// At the start of a kernel of many small blocks: a grid of at most one block per SM leaves room for its successor at once,
+// a larger one brings it up with its last blocks (or where it calls grid_dep_launch).  Brought up beside a full device, the
+// successor only keeps kernels of other streams away: ResNet-18 steps took 648 us at batch 1 without, 610 with it; 1697 us
+// at batch 64 without, 1730 with it in grids of any size.
+__device__ __forceinline__ void grid_dep_wait_launch_small()
+{
+    grid_dep_wait();
+    if (gridDim.x * gridDim.y <= 148) grid_dep_launch();
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

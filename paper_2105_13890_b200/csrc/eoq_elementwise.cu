@@ -43,6 +43,7 @@ __device__ __forceinline__ int round_log2_f32bits(uint32_t bits)
 
 __global__ void absmax_f32_kernel(const float *__restrict__ src, size_t n, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     uint32_t mx = 0;
     bool bad = false;
     const size_t n4 = n / 4;
@@ -111,6 +112,7 @@ template <int kMode>
 __global__ void __launch_bounds__(kThreads)
 quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     __shared__ uint32_t max_s;
     const size_t n4 = n / 4, base = (size_t)(gridDim.x - 1 - blockIdx.x) * kQuantTile + threadIdx.x;
     float4 v[kQuantLoads];
@@ -205,6 +207,7 @@ __global__ void __launch_bounds__(kThreads)
 quantize_image_kernel(const float *__restrict__ src, int rows, int w, int c_src, int c_dst, int wmargin, int8_t *dst, int32_t *dst_exp,
                       DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     __shared__ uint32_t max_s;
     const int groups = c_dst / kG, w_mem = w + 2 * wmargin, items = w_mem * groups;
     const int row0 = blockIdx.x * (kImageRows * blockDim.y) + threadIdx.y;
@@ -309,6 +312,7 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
                               int8_t *dst, int32_t *dst_exp, long long *sum_codes, NextHeadArgs next, JoinStatArgs join,
                               DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     const uint32_t M = dev->absmax_u32;
     const int t = M ? round_log2_u32(M) : 7;
     const int p_in = (src_exp ? *src_exp : 0) + exp_bias;
@@ -410,6 +414,7 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
                           (int)pack4(c3[8], c3[9], c3[10], c3[11]), (int)pack4(c3[12], c3[13], c3[14], c3[15]));
         }
     }
+    ptx::grid_dep_launch();
     if (!kNext && !kJoin)
         for (size_t i = n16 * 16 + (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
             const int c = sq_code32(src[i], t);
@@ -458,6 +463,7 @@ __global__ void sq_i32_scatter_kernel(const int32_t *__restrict__ src, const int
                                       int ww, int c, int stride, int hq, int wq, int8_t *dst, int32_t *dst_exp,
                                       long long *sum_codes, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     const uint32_t M = dev->absmax_u32;
     const int t = M ? round_log2_u32(M) : 7;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -783,6 +789,7 @@ __global__ void transpose_bytes_kernel(const int8_t *__restrict__ src, int8_t *_
 __global__ void weight_transpose_kernel(const int8_t *__restrict__ w, int8_t *__restrict__ wt, int c_out, int taps,
                                         int c_in)
 {
+    ptx::grid_dep_wait_launch_small();
     const size_t total = (size_t)c_out * taps * c_in;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int oc = (int)(i % c_out);
@@ -841,6 +848,7 @@ __global__ void b1_weight_table_kernel(const int8_t *__restrict__ w, int32_t *ta
 // [oc][kh][8][c_in] with zero taps.  One block per (layer, output channel).
 __global__ void weight_prep_kernel(const __grid_constant__ PrepBatch b)
 {
+    ptx::grid_dep_wait_launch_small();
     __shared__ int32_t tap_sum[kMaxTaps];
     int k = 0;
     while (k + 1 < b.num && (int)blockIdx.x >= b.first_block[k + 1]) ++k;
@@ -923,13 +931,13 @@ cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst,
         return cudaLaunchKernelEx(&cfg, quantize_sq_small_kernel, src, n, static_cast<int8_t *>(dst), dst_exp, dev);
     }
     if (mode == 2) {
-        absmax_f32_kernel<<<grid_for(n / 4 + 1, sm_count), kThreads, 0, s>>>(src, n, dev);
+        launch_chained(absmax_f32_kernel, grid_for(n / 4 + 1, sm_count), kThreads, 0, s, src, n, dev);
         hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);  // float bit patterns of |x| order like integers
     }
     const unsigned blocks = (unsigned)((n / 4 + kQuantTile - 1) / kQuantTile > 0 ? (n / 4 + kQuantTile - 1) / kQuantTile : 1);
-    if (mode == 0) quantize_f32_kernel<0><<<blocks, kThreads, 0, s>>>(src, n, dst, dst_exp, dev);
-    else if (mode == 1) quantize_f32_kernel<1><<<blocks, kThreads, 0, s>>>(src, n, dst, dst_exp, dev);
-    else quantize_f32_kernel<2><<<blocks, kThreads, 0, s>>>(src, n, dst, dst_exp, dev);
+    if (mode == 0) launch_chained(quantize_f32_kernel<0>, blocks, kThreads, 0, s, src, n, dst, dst_exp, dev);
+    else if (mode == 1) launch_chained(quantize_f32_kernel<1>, blocks, kThreads, 0, s, src, n, dst, dst_exp, dev);
+    else launch_chained(quantize_f32_kernel<2>, blocks, kThreads, 0, s, src, n, dst, dst_exp, dev);
     return cudaGetLastError();
 }
 
@@ -937,15 +945,15 @@ cudaError_t launch_quantize_image(const float *src, int n, int h, int w, int c_s
                                   int32_t *dst_exp, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook)
 {
     const size_t count = (size_t)n * h * w * c_src;
-    absmax_f32_kernel<<<grid_for(count / 4 + 1, sm_count), kThreads, 0, s>>>(src, count, dev);
+    launch_chained(absmax_f32_kernel, grid_for(count / 4 + 1, sm_count), kThreads, 0, s, src, count, dev);
     hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
     const int g = c_dst % 16 == 0 ? 16 : 8, items = (w + 2 * wmargin) * (c_dst / g), rows = n * h;
     int tx = 32;
     while (tx < items && tx < kThreads) tx *= 2;
     const dim3 block(tx, kThreads / tx);
     const unsigned grid = (unsigned)((rows + kImageRows * (int)block.y - 1) / (kImageRows * (int)block.y));
-    if (g == 16) quantize_image_kernel<16><<<grid, block, 0, s>>>(src, rows, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
-    else quantize_image_kernel<8><<<grid, block, 0, s>>>(src, rows, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
+    if (g == 16) launch_chained(quantize_image_kernel<16>, grid, block, 0, s, src, rows, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
+    else launch_chained(quantize_image_kernel<8>, grid, block, 0, s, src, rows, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
     return cudaGetLastError();
 }
 
@@ -966,15 +974,15 @@ cudaError_t launch_sq_i32(const int32_t *src, const int32_t *src_exp, int exp_bi
     const int grid = grid_for(n / 16 + 1, sm_count);
     if (join) {
         // (no hook in this form: callers with replicas take the separate calls)
-        sq_i32_kernel<false, true><<<grid, kThreads, 0, s>>>(src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, NextHeadArgs{}, *join, dev);
+        launch_chained(sq_i32_kernel<false, true>, grid, kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, NextHeadArgs{}, *join, dev);
     } else if (next) {
         // (only behind a GEMM whose epilogue reduced the masked maximum)
         hook(&dev->absmax_u64, 1, EOQ_REDUCE_I64, EOQ_REDUCE_MAX, s);
-        sq_i32_kernel<true, false><<<grid, kThreads, 0, s>>>(src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, *next, JoinStatArgs{}, dev);
+        launch_chained(sq_i32_kernel<true, false>, grid, kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, *next, JoinStatArgs{}, dev);
         if (next->sum_e1) hook(next->sum_e1, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
         if (next->sum_e1x2) hook(next->sum_e1x2, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
     } else {
-        sq_i32_kernel<false, false><<<grid, kThreads, 0, s>>>(src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, NextHeadArgs{},
+        launch_chained(sq_i32_kernel<false, false>, grid, kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, NextHeadArgs{},
                                                               JoinStatArgs{}, dev);
     }
     if (sum_codes) hook(sum_codes, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
@@ -987,7 +995,7 @@ cudaError_t launch_sq_i32_scatter(const int32_t *src, const int32_t *src_exp, in
 {
     const size_t items = (size_t)n_img * hh * ww * (c / 16);
     hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
-    sq_i32_scatter_kernel<<<grid_for(items, sm_count), kThreads, 0, s>>>(src, src_exp, exp_bias, n_img, hh, ww, c, stride, hq, wq,
+    launch_chained(sq_i32_scatter_kernel, grid_for(items, sm_count), kThreads, 0, s, src, src_exp, exp_bias, n_img, hh, ww, c, stride, hq, wq,
                                                                         dst, dst_exp, sum_codes, dev);
     if (sum_codes) hook(sum_codes, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
     return cudaGetLastError();
@@ -1054,7 +1062,7 @@ cudaError_t launch_weight_transpose(const int8_t *w, int8_t *wt, int c_out, int 
     const size_t total = (size_t)c_out * taps * c_in;
     int blocks = (int)((total + kThreads - 1) / kThreads);
     if (blocks > 148 * 16) blocks = 148 * 16;
-    weight_transpose_kernel<<<blocks, kThreads, 0, s>>>(w, wt, c_out, taps, c_in);
+    launch_chained(weight_transpose_kernel, blocks, kThreads, 0, s, w, wt, c_out, taps, c_in);
     return cudaGetLastError();
 }
 
@@ -1068,7 +1076,7 @@ cudaError_t launch_b1_weight_table(const int8_t *w, int32_t *table, const eoq_co
 
 cudaError_t launch_weight_prep(const PrepBatch &b, cudaStream_t s)
 {
-    weight_prep_kernel<<<b.first_block[b.num], 128, 0, s>>>(b);
+    launch_chained(weight_prep_kernel, b.first_block[b.num], 128, 0, s, b);
     return cudaGetLastError();
 }
 

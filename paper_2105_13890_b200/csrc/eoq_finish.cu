@@ -126,6 +126,7 @@ __device__ __forceinline__ bool tap_takes(int y, int k, int stride, int pad, int
 
 __global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_constant__ FinishBatch b)
 {
+    ptx::grid_dep_wait();
     __shared__ unsigned long long rows_out[16], cols_out[16];  // per filter row / column: the border rows / columns it does not take
     extern __shared__ int32_t sets[];  // [1 + border rows][1 + border columns][kClassSlab]; index 0 = all rows / columns
     const int k = finish_item_of(b.tap_first, b.num, (int)blockIdx.x);
@@ -259,6 +260,7 @@ __device__ __forceinline__ void finish_direct(const FinishItem &it, uint32_t q, 
 
 __global__ void __launch_bounds__(kThreads) finish_sums_kernel(const __grid_constant__ FinishBatch b)
 {
+    ptx::grid_dep_wait();
     __shared__ long long part[kThreads][4];
     const int k = finish_item_of(b.fin_first, b.num, (int)blockIdx.x);
     const FinishItem &it = b.item[k];
@@ -341,6 +343,7 @@ __global__ void __launch_bounds__(kThreads) finish_sums_kernel(const __grid_cons
 // max |.| of 64-bit sums that an all-reduce over replicas completed (keep_sums)
 __global__ void __launch_bounds__(kThreads) finish_max_kernel(const long long *__restrict__ src, size_t n, unsigned long long *max_cell)
 {
+    ptx::grid_dep_wait();
     unsigned long long mx = 0;
     for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kThreads) {
         const long long v = src[i];
@@ -355,6 +358,7 @@ __global__ void __launch_bounds__(kThreads) finish_max_kernel(const long long *_
 
 __global__ void __launch_bounds__(kThreads) finish_code_kernel(const __grid_constant__ FinishBatch b, unsigned *status)
 {
+    ptx::grid_dep_wait();
     const int k = finish_item_of(b.sq_first, b.num, (int)blockIdx.x);
     const FinishItem &it = b.item[k];
     const int bx = (int)blockIdx.x - b.sq_first[k];
@@ -470,19 +474,19 @@ cudaError_t launch_wgrad_finish(const FinishItem *items, int num, unsigned *stat
                 const cudaError_t e = cudaFuncSetAttribute(finish_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
                 if (e != cudaSuccess) return e;
             }
-            finish_taps_kernel<<<b.tap_first[b.num], kThreads, smem, s>>>(b);
+            launch_chained(finish_taps_kernel, b.tap_first[b.num], kThreads, smem, s, b);
         }
-        finish_sums_kernel<<<b.fin_first[b.num], kThreads, 0, s>>>(b);
+        launch_chained(finish_sums_kernel, b.fin_first[b.num], kThreads, 0, s, b);
         if (hook.fn)
             // replicas (one layer per call): local sums, b1 term included (it is linear in the error) -> all-reduce ->
             // maximum of the global sums; the copy for the caller is taken from the global sums as well
             for (int k = 0; k < b.num; ++k) {
                 const FinishItem &it = b.item[k];
                 hook(it.acc, (size_t)it.n, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
-                finish_max_kernel<<<it.fin_blocks, kThreads, 0, s>>>(it.acc, (size_t)it.n, it.max_cell);
+                launch_chained(finish_max_kernel, it.fin_blocks, kThreads, 0, s, it.acc, (size_t)it.n, it.max_cell);
                 if (it.copy_out) cudaMemcpyAsync(it.copy_out, it.acc, (size_t)it.n * sizeof(long long), cudaMemcpyDeviceToDevice, s);
             }
-        finish_code_kernel<<<b.sq_first[b.num], kThreads, 0, s>>>(b, status);
+        launch_chained(finish_code_kernel, b.sq_first[b.num], kThreads, 0, s, b, status);
     }
     return cudaGetLastError();
 }

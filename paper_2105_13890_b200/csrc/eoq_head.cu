@@ -16,6 +16,7 @@ constexpr int kThreads = 256;
 // sums[b][ch] = sum over the hw positions of x[b][.][ch]; one warp per (sample, 16-channel group)
 __global__ void __launch_bounds__(kThreads) avgpool_sum_kernel(const int8_t *__restrict__ x, int hw, int c, int items, int32_t *__restrict__ sums)
 {
+    ptx::grid_dep_wait_launch_small();
     const int groups = c / 16, item = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (item >= items) return;
     const int b = item / groups, g = item - b * groups;
@@ -78,6 +79,7 @@ __device__ __forceinline__ float pooled_of(int32_t sum, float fhw) { return __fd
 // pooled[b][k] = (float)sum * 2^-7 / hw
 __global__ void __launch_bounds__(kThreads) head_pooled_kernel(const int32_t *__restrict__ sums, int count, int hw, float *pooled)
 {
+    ptx::grid_dep_wait_launch_small();
     const int i = blockIdx.x * kThreads + threadIdx.x;
     if (i < count) pooled[i] = pooled_of(__ldg(sums + i), (float)hw);
 }
@@ -95,6 +97,7 @@ __global__ void __launch_bounds__(32 * kHeadWarps)
 head_logits_kernel(const int32_t *__restrict__ sums, int n, int c, int hw, int classes, const float *__restrict__ W,
                    const float *__restrict__ bias, float *pooled, float *__restrict__ logits)
 {
+    ptx::grid_dep_wait_launch_small();
     extern __shared__ float4 head_smem[];
     const int kc = min(c, kHeadK), ld = ((kc + 3) & ~3) + 4;
     float *ps = reinterpret_cast<float *>(head_smem), *ws = ps + 32 * ld;
@@ -167,6 +170,7 @@ template <bool kShared>
 __global__ void __launch_bounds__(kThreads)
 head_softmax_kernel(const float *__restrict__ logits, int n, int classes, const int32_t *__restrict__ labels, float *dl, double *loss_n)
 {
+    ptx::grid_dep_wait_launch_small();
     extern __shared__ float4 head_smem[];
     __shared__ float red[32];
     __shared__ float den_s;
@@ -236,6 +240,7 @@ __global__ void __launch_bounds__(kDpCh *kDpN)
 head_dpooled_kernel(const float *__restrict__ dl, const float *__restrict__ W, int n, int c, int classes, float *dpooled,
                     const double *loss_n, float *loss_out)
 {
+    ptx::grid_dep_wait_launch_small();
     extern __shared__ float4 head_smem[];
     DpStage *st = reinterpret_cast<DpStage *>(head_smem);
     if (blockIdx.y == gridDim.y - 1) {   // an extra row of blocks: the mean loss, in sample order, beside the chains
@@ -336,6 +341,7 @@ template <int kV>
 __global__ void __launch_bounds__(128)
 head_update_kernel(const float *__restrict__ dl, const float *__restrict__ pooled, int n, int c, int classes, float lr, float *W, float *bias)
 {
+    ptx::grid_dep_wait_launch_small();
     const int i = blockIdx.x * blockDim.x + threadIdx.x, cv = c / kV;
     if (i >= classes * cv) return;
     const int j = i / cv, k = (i - j * cv) * kV;
@@ -427,6 +433,7 @@ template <bool kScan>
 __global__ void __launch_bounds__(kSpreadThreads)
 head_error_spread_kernel(const float *__restrict__ dpooled, int n, int hw, int c, int8_t *e, int32_t *e_exp, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     __shared__ uint32_t max_s;
     const float fhw = (float)hw;
     uint32_t mbits;
@@ -484,7 +491,7 @@ head_error_spread_kernel(const float *__restrict__ dpooled, int n, int hw, int c
 cudaError_t launch_avgpool_sum(const int8_t *x, int n, int hw, int c, int32_t *sums, cudaStream_t st)
 {
     const int items = n * (c / 16);
-    avgpool_sum_kernel<<<(items + kThreads / 32 - 1) / (kThreads / 32), kThreads, 0, st>>>(x, hw, c, items, sums);
+    launch_chained(avgpool_sum_kernel, (items + kThreads / 32 - 1) / (kThreads / 32), kThreads, 0, st, x, hw, c, items, sums);
     return cudaGetLastError();
 }
 
@@ -493,8 +500,8 @@ cudaError_t launch_head_update(const float *dl, const float *pooled, int n, int 
 {
     const bool vec = c % 4 == 0 && ((reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(pooled)) & 15) == 0;
     const int items = classes * (vec ? c / 4 : c);
-    if (vec) head_update_kernel<4><<<(items + 127) / 128, 128, 0, st>>>(dl, pooled, n, c, classes, lr, W, bias);
-    else head_update_kernel<1><<<(items + 127) / 128, 128, 0, st>>>(dl, pooled, n, c, classes, lr, W, bias);
+    if (vec) launch_chained(head_update_kernel<4>, (items + 127) / 128, 128, 0, st, dl, pooled, n, c, classes, lr, W, bias);
+    else launch_chained(head_update_kernel<1>, (items + 127) / 128, 128, 0, st, dl, pooled, n, c, classes, lr, W, bias);
     return cudaGetLastError();
 }
 
@@ -513,15 +520,15 @@ cudaError_t launch_head(const int32_t *sums, int n, int c, int hw, int classes, 
     if (e != cudaSuccess) return e;
     const dim3 grid((classes + kHeadWarps - 1) / kHeadWarps, (n + 31) / 32);
     if (fold) {
-        head_logits_kernel<true><<<grid, 32 * kHeadWarps, logits_smem, st>>>(sums, n, c, hw, classes, W, bias, pooled, logits);
+        launch_chained(head_logits_kernel<true>, grid, 32 * kHeadWarps, logits_smem, st, sums, n, c, hw, classes, W, bias, pooled, logits);
     } else {
-        head_pooled_kernel<<<(n * c + kThreads - 1) / kThreads, kThreads, 0, st>>>(sums, n * c, hw, pooled);
-        head_logits_kernel<false><<<grid, 32 * kHeadWarps, logits_smem, st>>>(sums, n, c, hw, classes, W, bias, pooled, logits);
+        launch_chained(head_pooled_kernel, (n * c + kThreads - 1) / kThreads, kThreads, 0, st, sums, n * c, hw, pooled);
+        launch_chained(head_logits_kernel<false>, grid, 32 * kHeadWarps, logits_smem, st, sums, n, c, hw, classes, W, bias, pooled, logits);
     }
     const size_t soft_smem = ((size_t)classes * sizeof(float) + 15) & ~(size_t)15;
-    if (soft_smem <= 48 * 1024 - 256) head_softmax_kernel<true><<<n, kThreads, soft_smem, st>>>(logits, n, classes, labels, dl, loss_n);
-    else head_softmax_kernel<false><<<n, kThreads, 0, st>>>(logits, n, classes, labels, dl, loss_n);
-    head_dpooled_kernel<<<dim3((c + kDpCh - 1) / kDpCh, (n + kDpN - 1) / kDpN + 1), kDpCh * kDpN, dp_smem, st>>>(dl, W, n, c, classes, dpooled,
+    if (soft_smem <= 48 * 1024 - 256) launch_chained(head_softmax_kernel<true>, n, kThreads, soft_smem, st, logits, n, classes, labels, dl, loss_n);
+    else launch_chained(head_softmax_kernel<false>, n, kThreads, 0, st, logits, n, classes, labels, dl, loss_n);
+    launch_chained(head_dpooled_kernel, dim3((c + kDpCh - 1) / kDpCh, (n + kDpN - 1) / kDpN + 1), kDpCh * kDpN, dp_smem, st, dl, W, n, c, classes, dpooled,
                                                                                                    loss_n, loss_out);
     if (lr != 0.0f) return launch_head_update(dl, pooled, n, c, classes, lr, W, bias, st);
     return cudaGetLastError();
@@ -533,13 +540,13 @@ cudaError_t launch_head_error(const float *dpooled, int n, int c, int hw, int8_t
                               cudaStream_t st, const ReduceHook &hook)
 {
     if (head_error_is_single(n, c, hook)) {
-        head_error_spread_kernel<true><<<n, kSpreadThreads, 0, st>>>(dpooled, n, hw, c, e, e_exp, dev);
+        launch_chained(head_error_spread_kernel<true>, n, kSpreadThreads, 0, st, dpooled, n, hw, c, e, e_exp, dev);
         return cudaGetLastError();
     }
     const int blocks = (n * c + kThreads - 1) / kThreads;
     head_error_max_kernel<<<blocks < sm_count ? blocks : sm_count, kThreads, 0, st>>>(dpooled, n * c, hw, dev);
     hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, st);
-    head_error_spread_kernel<false><<<n, kSpreadThreads, 0, st>>>(dpooled, n, hw, c, e, e_exp, dev);
+    launch_chained(head_error_spread_kernel<false>, n, kSpreadThreads, 0, st, dpooled, n, hw, c, e, e_exp, dev);
     return cudaGetLastError();
 }
 

@@ -82,6 +82,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    ptx::grid_dep_wait();   // everything up to here touched no global memory
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, p.dev};
 
@@ -249,6 +250,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
             if (ok) ptx::mma_commit(tfull_bar(acc), leader);
             if (++acc == p.ep_groups) { acc = 0; acc_phase ^= 1u; }
         }
+        ptx::grid_dep_launch();   // what remains is the epilogue of the last tiles
         if (!ok) {
             ptx::mma_commit(drain_bar, leader);
             for (uint32_t i = 0; i < kSpinLimit; ++i)
@@ -377,8 +379,7 @@ cudaError_t launch_igemm_patch(const IgemmParams &p, const PatchPlan &pl, const 
     const auto kernel = p.epilogue == kEpiForward ? igemm_patch_kernel<kEpiForward> : igemm_patch_kernel<kEpiDgrad>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e != cudaSuccess) return e;
-    kernel<<<grid, kPatchThreads, igemm_patch_smem_bytes(p, pl), stream>>>(p, pl, map_a, map_b);
-    return cudaGetLastError();
+    return launch_chained(kernel, grid, kPatchThreads, igemm_patch_smem_bytes(p, pl), stream, p, pl, map_a, map_b);
 }
 
 }  // namespace eoq

@@ -16,6 +16,26 @@ constexpr int kWgradThreads = 256;  // weight gradient: warps 0, 2, 3 TMA, warp 
 constexpr uint32_t kSpinLimit = 1u << 22;  // polls before a wait gives up (normal waits end within microseconds)
 
 // Device state a handle owns.
+// Launches a kernel that may be brought up while its predecessor on the stream still runs (programmatic dependent launch):
+// the predecessor allows it with ptx::grid_dep_launch (or by ending), and the kernel calls ptx::grid_dep_wait before it
+// touches global memory, in every block.  Launch latency and prologue, about 1.5 us per kernel in a captured chain, then
+// overlap the predecessor's last microseconds.
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
+}
+
 struct DeviceState {
     unsigned status;       // EOQ_DEV_* bits
     unsigned absmax_u32;   // reduction cell for |.| maxima (int32 sources, float bit patterns)

@@ -34,6 +34,7 @@ __global__ void __launch_bounds__(kThreads)
 maxpool_fwd_kernel(const int8_t *__restrict__ x, uint32_t items, int h, int w, int c, int k_rt, int s, int p, int ho, int wo,
                    int8_t *__restrict__ y, uint8_t *__restrict__ arg)
 {
+    ptx::grid_dep_wait_launch_small();
     const int groups = c / 16, k = kK ? kK : k_rt;
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
     if (i >= items) return;
@@ -284,6 +285,7 @@ maxpool_bwd_quad_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, cons
                         int c, int ho, int wo, int8_t *__restrict__ e_in, int32_t *e_in_exp, const uint8_t *__restrict__ next_mask,
                         const int32_t *next_gamma, int8_t *__restrict__ e3, int32_t *e3_exp, long long *sum_e1, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
     const bool live = i < items;
     const int groups = c / 16;
@@ -435,8 +437,8 @@ cudaError_t launch_maxpool_fwd(const int8_t *x, int n, int h, int w, int c, int 
     const int ho = (h + 2 * p - k) / s + 1, wo = (w + 2 * p - k) / s + 1;
     const uint32_t items = (uint32_t)n * ho * wo * (c / 16);   // below 2^31 (checked by the caller)
     const unsigned blocks = (items + kThreads - 1) / kThreads;
-    if (k == 3) maxpool_fwd_kernel<3><<<blocks, kThreads, 0, st>>>(x, items, h, w, c, k, s, p, ho, wo, y, arg);
-    else maxpool_fwd_kernel<0><<<blocks, kThreads, 0, st>>>(x, items, h, w, c, k, s, p, ho, wo, y, arg);
+    if (k == 3) launch_chained(maxpool_fwd_kernel<3>, blocks, kThreads, 0, st, x, items, h, w, c, k, s, p, ho, wo, y, arg);
+    else launch_chained(maxpool_fwd_kernel<0>, blocks, kThreads, 0, st, x, items, h, w, c, k, s, p, ho, wo, y, arg);
     return cudaGetLastError();
 }
 
@@ -453,7 +455,7 @@ cudaError_t launch_maxpool_bwd(const int8_t *e, const int32_t *e_exp, const uint
     const unsigned grid = quads ? (qitems + kThreads - 1) / kThreads : (unsigned)blocks;
     auto pass = [&](auto kernel, auto quad_kernel) {
         if (quads)
-            quad_kernel<<<grid, kThreads, 0, st>>>(e, e_exp, arg, qitems, h, w, c, ho, wo, e_in, e_in_exp, next_mask, next_gamma, e3, e3_exp,
+            launch_chained(quad_kernel, grid, kThreads, 0, st, e, e_exp, arg, qitems, h, w, c, ho, wo, e_in, e_in_exp, next_mask, next_gamma, e3, e3_exp,
                                                    sum_e1, dev);
         else
             kernel<<<grid, kThreads, 0, st>>>(e, e_exp, arg, n, h, w, c, k, s, p, ho, wo, e_in, e_in_exp, next_mask, next_gamma, e3, e3_exp,

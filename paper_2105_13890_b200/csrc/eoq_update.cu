@@ -67,6 +67,7 @@ struct AbsMax16 {
 // with packed 16-bit ones.
 __global__ void __launch_bounds__(kThreads) update_absmax_kernel(const __grid_constant__ UpdateBatch b, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     const int k = find_tensor(b, blockIdx.x);
     const UpdateTensor &T = b.t[k];
     const size_t begin = (size_t)(blockIdx.x - b.first_block[k]) * kUpdElemsPerBlock;
@@ -215,6 +216,7 @@ __global__ void __launch_bounds__(kThreads)
 update_apply_kernel(const __grid_constant__ UpdateBatch b, int32_t lr_mant, int32_t lr_exp, int stochastic, unsigned long long seed,
                     unsigned long long step, unsigned long long *step_dev, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     __shared__ unsigned long long step_s;
     __shared__ uint32_t max_s;
     const int k = find_tensor(b, blockIdx.x);
@@ -248,6 +250,7 @@ __global__ void __launch_bounds__(kSmallThreads)
 update_small_kernel(const __grid_constant__ UpdateBatch b, int32_t lr_mant, int32_t lr_exp, int stochastic, unsigned long long seed,
                     unsigned long long step, unsigned long long *step_dev, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     __shared__ unsigned long long step_s;
     const UpdateTensor &T = b.t[blockIdx.x];
     const int g_exp = __ldg(T.g_exp);
@@ -286,6 +289,7 @@ __global__ void update_wide_apply_kernel(const __grid_constant__ UpdateBatch b, 
                                          int stochastic, unsigned long long seed, unsigned long long step,
                                          unsigned long long *step_dev, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
     __shared__ unsigned long long step_s;
     __shared__ uint32_t max_s;
     const int k = find_tensor(b, blockIdx.x);
@@ -379,12 +383,12 @@ cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32
     if (!small)
         for (int base = 0; base < num; base += kUpdChunk) {
             const int blocks = fill_batch(b, t, num, base);
-            update_absmax_kernel<<<blocks, kThreads, 0, s>>>(b, dev);
+            launch_chained(update_absmax_kernel, blocks, kThreads, 0, s, b, dev);
         }
     for (int base = 0; base < num; base += kUpdChunk) {
         const int blocks = fill_batch(b, t, num, base);
-        if (small) update_small_kernel<<<b.num, kSmallThreads, 0, s>>>(b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
-        else update_apply_kernel<<<blocks, kThreads, 0, s>>>(b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
+        if (small) launch_chained(update_small_kernel, b.num, kSmallThreads, 0, s, b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
+        else launch_chained(update_apply_kernel, blocks, kThreads, 0, s, b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
     }
     return cudaGetLastError();
 }
@@ -396,8 +400,8 @@ cudaError_t launch_update_wide(const UpdateTensor *t, int num, int32_t lr_mant, 
     for (int pass = 0; pass < 2; ++pass)
         for (int base = 0; base < num; base += kUpdChunk) {
             const int blocks = fill_batch(b, t, num, base);
-            if (pass == 0) update_absmax_kernel<<<blocks, kThreads, 0, s>>>(b, dev);
-            else update_wide_apply_kernel<<<blocks, kThreads, 0, s>>>(b, lr_mant, lr_exp, k_u, k_m, stochastic, seed, step, step_dev, dev);
+            if (pass == 0) launch_chained(update_absmax_kernel, blocks, kThreads, 0, s, b, dev);
+            else launch_chained(update_wide_apply_kernel, blocks, kThreads, 0, s, b, lr_mant, lr_exp, k_u, k_m, stochastic, seed, step, step_dev, dev);
         }
     return cudaGetLastError();
 }

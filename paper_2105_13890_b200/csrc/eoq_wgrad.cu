@@ -78,7 +78,6 @@ wgrad_kernel(const __grid_constant__ WgradParams p, const __grid_constant__ CUte
         ptx::prefetch_tensormap(&map_x);
         ptx::prefetch_tensormap(&map_e);
     }
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < p.zero_n16; i += gridDim.x * blockDim.x) p.zero[i] = make_int4(0, 0, 0, 0);
     if (warp == 1) {
         ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), tmem_cols);
         ptx::tmem_relinquish();
@@ -86,6 +85,8 @@ wgrad_kernel(const __grid_constant__ WgradParams p, const __grid_constant__ CUte
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    ptx::grid_dep_wait();   // everything up to here touched no global memory
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < p.zero_n16; i += gridDim.x * blockDim.x) p.zero[i] = make_int4(0, 0, 0, 0);
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, p.dev};
 
@@ -246,8 +247,7 @@ cudaError_t launch_wgrad(const WgradParams &p, const CUtensorMap &map_x, const C
     cudaError_t e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024);
     if (e != cudaSuccess) return e;
     const int grid = p.num_m_groups * p.num_n_tiles * p.num_k_splits;
-    wgrad_kernel<<<grid, kWgradThreads, wgrad_smem_bytes(p), stream>>>(p, map_x, map_e);
-    return cudaGetLastError();
+    return launch_chained(wgrad_kernel, grid, kWgradThreads, wgrad_smem_bytes(p), stream, p, map_x, map_e);
 }
 
 }  // namespace eoq

@@ -80,7 +80,6 @@ wgrad_patch_kernel(const __grid_constant__ WgradPatchPlan pl, const __grid_const
         ptx::prefetch_tensormap(&map_x);
         ptx::prefetch_tensormap(&map_e);
     }
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < pl.zero_n16; i += gridDim.x * blockDim.x) pl.zero[i] = make_int4(0, 0, 0, 0);
     if (warp == 1) {
         ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), tmem_cols);
         ptx::tmem_relinquish();
@@ -88,6 +87,8 @@ wgrad_patch_kernel(const __grid_constant__ WgradPatchPlan pl, const __grid_const
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    ptx::grid_dep_wait();   // everything up to here touched no global memory
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < pl.zero_n16; i += gridDim.x * blockDim.x) pl.zero[i] = make_int4(0, 0, 0, 0);
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, pl.dev};
 
@@ -212,9 +213,8 @@ cudaError_t launch_wgrad_patch(const WgradPatchPlan &pl, const CUtensorMap &map_
 {
     cudaError_t e = cudaFuncSetAttribute(wgrad_patch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024);
     if (e != cudaSuccess) return e;
-    wgrad_patch_kernel<<<pl.num_groups * pl.num_splits, kWgradPatchThreads, wgrad_patch_smem_bytes(pl), stream>>>(pl, map_x,
+    return launch_chained(wgrad_patch_kernel, pl.num_groups * pl.num_splits, kWgradPatchThreads, wgrad_patch_smem_bytes(pl), stream, pl, map_x,
                                                                                                                  map_e);
-    return cudaGetLastError();
 }
 
 }  // namespace eoq
