@@ -239,6 +239,10 @@ inline int persistent_grid(int tiles, int sm_count)
 // the CTA gets and tensor memory holds are worked on side by side; a CTA with a single tile puts all its warps on it.
 void plan_epilogue(IgemmParams &p, int grid)
 {
+    if (p.split > 1) {   // every epilogue warp takes part in the exchange
+        p.ep_groups = 1;
+        return;
+    }
     const int tiles = p.num_m_tiles * p.num_n_tiles, per_cta = (tiles + grid - 1) / grid;
     int cols = 32;
     while (cols < p.tile_n) cols <<= 1;
@@ -264,9 +268,45 @@ void plan_igemm(IgemmParams &p, int src_channels, int ntaps, int sm_count)
     if (tn == 256 && (long long)p.num_m_tiles * ((p.N + 255) / 256) < 2LL * sm_count) tn = 128;
     p.tile_n = tn;
     p.num_n_tiles = (p.N + tn - 1) / tn;
+    p.split = 1;
+    p.a_rows = kTileM;   // a problem of fewer pixels loads no more of them (TMA time goes by rows; the rest of the tile is never stored)
+    while (p.a_rows > 16 && p.M <= p.a_rows / 2) p.a_rows /= 2;
     const size_t stage = (size_t)p.subs_per_stage * (kTileM + tn) * p.kc;
     int stages = (int)((200 * 1024) / stage);
     p.num_stages = stages > 8 ? 8 : (stages < 2 ? 2 : stages);
+}
+
+// SM cycles of one K iteration of the im2col kernel: a TMA row takes 3.1
+double igemm_iteration_cycles(const IgemmParams &p)
+{
+    return 3.1 * p.subs_per_stage * (p.a_rows + (p.b_mn ? p.kc * (p.tile_n / p.b_row) : p.tile_n));
+}
+
+// CTAs that share a tile (see igemm_kernel): a cluster of 2, 4 or 8 where few tiles leave at least half of the `ctas` CTAs idle
+// and the shorter reductions save more than a sixth of the kernel; the exchange costs about 4,000 cycles.  Wants every CTA to
+// have a K iteration and its part of the columns.  Returns the estimated cycles.
+double plan_split(IgemmParams &p, int ctas)
+{
+    const int tiles = p.num_m_tiles * p.num_n_tiles, groups = p.tile_n / 16;
+    const int k_iters = (p.num_sub + p.subs_per_stage - 1) / p.subs_per_stage;
+    const double per_iter = igemm_iteration_cycles(p), whole = k_iters * per_iter;
+    double best = whole;
+    p.split = 1;
+    if (p.kc < 64 || p.tile_n > 128) return whole;
+    for (int s = 2; s <= 8; s *= 2) {
+        if (groups % s || groups / s > 4 || k_iters < s || tiles * s > ctas / 2) continue;
+        const double cost = (k_iters + s - 1) / s * per_iter + 4000.0;
+        if (cost < best && 6 * cost < 5 * whole + 6000.0) {   // (6,000: what a kernel spends beside its reduction)
+            best = cost;
+            p.split = s;
+        }
+    }
+    if (p.split > 1) {   // the exchange takes a tile's worth of shared memory from the stages
+        const size_t stage = (size_t)p.subs_per_stage * (kTileM + p.tile_n) * p.kc;
+        const int stages = (int)((200 * 1024 - (size_t)kTileM * p.tile_n * sizeof(int32_t)) / stage);
+        p.num_stages = stages > 8 ? 8 : (stages < 2 ? 2 : stages);
+    }
+    return best;
 }
 
 // Plan of the patch variant for a stride-1 k x k correlation over a source [n][hs][ws][c_src] producing a
@@ -327,6 +367,23 @@ bool plan_patch(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, int
         pl.num_b = nb > 8 ? 8 : (int)nb;
     }
     return pl.num_a >= 2 || (pl.b_resident && pl.num_a >= 1);
+}
+
+// Is a cluster per tile in the im2col kernel faster than the patch kernel's plan?  (A patch tile costs its MMAs, about 1.45
+// times 57 cycles each, 100 beyond 64 columns, with what surrounds them.)  Only problems of few tiles get a split.
+bool split_beats_patch(const IgemmParams &patch, int c_src, bool b_mn, int ctas)
+{
+    if (patch.num_m_tiles * patch.num_n_tiles > ctas / 4) return false;
+    IgemmParams q;
+    memset(&q, 0, sizeof(q));
+    q.M = patch.M;
+    q.N = patch.N;
+    plan_igemm(q, c_src, patch.ntaps, ctas);
+    q.b_mn = b_mn ? 1 : 0;
+    q.b_row = chunk_bytes(q.tile_n);
+    const double split = plan_split(q, ctas);
+    const double mmas = (double)patch.ntaps * patch.chunks_per_tap * patch.kc / 32;
+    return q.split > 1 && split < 1.45 * mmas * (patch.tile_n <= 64 ? 57.0 : 100.0);
 }
 
 // Plan of the patch variant of the weight gradient; false when the geometry does not suit it.
@@ -797,7 +854,8 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
     PatchPlan pl;
     memset(&pl, 0, sizeof(pl));
     const bool patch = d.stride == 1 && d.kh == d.kw && d.x_wmargin == 0 &&
-                       plan_patch(p, pl, d.n, d.c_in, g.ho, g.wo, d.kh, d.pad, d.c_out, h->sm_count);
+                       plan_patch(p, pl, d.n, d.c_in, g.ho, g.wo, d.kh, d.pad, d.c_out, h->sm_count) &&
+                       !split_beats_patch(p, d.c_in, false, h->gemm_ctas);
     p.M = d.n * g.ho * g.wo;
     p.N = d.c_out;
     p.hq = g.ho;
@@ -834,6 +892,7 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
             p.tap_dw[t] = (unsigned char)(t % d.kw);
             p.tap_b[t] = (unsigned char)t;
         }
+        plan_split(p, h->gemm_ctas);
     }
     p.out_h = g.ho;
     p.out_w = g.wo;
@@ -878,11 +937,11 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
         return record(h, launch_igemm_patch(p, pl, map_a, map_b, grid, s));
     }
     if (row_window) {
-        if (!make_row_window_map(&map_a, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, g.wo, g.ho, d.stride, d.pad, kTileM) ||
+        if (!make_row_window_map(&map_a, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, g.wo, g.ho, d.stride, d.pad, p.a_rows) ||
             !make_weight_map(&map_b, w_rows, d.c_out, d.kh, 8 * d.c_in, 8 * d.c_in, p.tile_n))
             return EOQ_ERR_UNSUPPORTED;
     } else if (!make_im2col_map(&map_a, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, -d.pad, g.wo, g.ho, d.stride, p.kc,
-                                kTileM) ||
+                                p.a_rows) ||
                !make_weight_map(&map_b, w, d.c_out, g.taps, d.c_in, p.kc, p.tile_n)) {
         return EOQ_ERR_UNSUPPORTED;
     }
@@ -891,7 +950,7 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
     ProfScope prof(h, EOQ_PROF_IGEMM_FWD, s);
     const int grid = persistent_grid(tiles, h->gemm_ctas);
     plan_epilogue(p, grid);
-    return record(h, launch_igemm(p, map_a, map_b, grid, s));
+    return record(h, launch_igemm(p, map_a, map_b, grid * p.split, s));
 }
 
 extern "C" int eoq_conv_fwd(eoq_handle_t handle, const eoq_conv_desc_t *desc, const int8_t *x, const int32_t *x_exp,
@@ -1047,7 +1106,8 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
         memset(&p, 0, sizeof(p));
         PatchPlan pl;
         memset(&pl, 0, sizeof(pl));
-        if (plan_patch(p, pl, d.n, d.c_out, d.h, d.w, d.kh, d.kh - 1 - d.pad, d.c_in, h->sm_count)) {
+        if (plan_patch(p, pl, d.n, d.c_out, d.h, d.w, d.kh, d.kh - 1 - d.pad, d.c_in, h->sm_count) &&
+            !split_beats_patch(p, d.c_out, true, h->gemm_ctas)) {
             for (int a = 0; a < d.kh; ++a)
                 for (int b = 0; b < d.kw; ++b) p.tap_b[a * d.kw + b] = (unsigned char)((d.kh - 1 - a) * d.kw + (d.kw - 1 - b));
             p.out_h = d.h;
@@ -1191,7 +1251,7 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
                 p.b_mn = 1;
                 p.b_row = chunk_bytes(p.tile_n);
             }
-            if (!make_im2col_map(&map_a, e3, d.n, g.ho, g.wo, d.c_out, min_w, min_h, wq, hq, 1, p.kc, kTileM) ||
+            if (!make_im2col_map(&map_a, e3, d.n, g.ho, g.wo, d.c_out, min_w, min_h, wq, hq, 1, p.kc, p.a_rows) ||
                 !(weights_in_place ? make_weight_map(&map_b, w, d.c_out, g.taps, d.c_in, p.b_row, p.kc)
                                    : make_weight_map(&map_b, wt, d.c_in, g.taps, d.c_out, p.kc, p.tile_n)))
                 return EOQ_ERR_UNSUPPORTED;
@@ -1212,13 +1272,14 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
                 }
             }
             ++class_no;
+            plan_split(p, ctas);
             const int grid = persistent_grid(tiles, ctas);
             plan_epilogue(p, grid);
             if (side_by_side) {
-                e = launch_igemm(p, map_a, map_b, grid, cs);
+                e = launch_igemm(p, map_a, map_b, grid * p.split, cs);
             } else {
                 ProfScope prof(h, EOQ_PROF_IGEMM_DGRAD, cs);
-                e = launch_igemm(p, map_a, map_b, grid, cs);
+                e = launch_igemm(p, map_a, map_b, grid * p.split, cs);
             }
             if (e != cudaSuccess) {
                 launch_reset_cells(h->dev, s);  // GEMMs already queued have touched the maximum cell
@@ -1525,7 +1586,8 @@ extern "C" int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *des
     buf[0] = 0;
     if (pass == EOQ_PASS_FWD) {
         if (d.stride == 1 && d.kh == d.kw && d.x_wmargin == 0 &&
-            plan_patch(p, pl, d.n, d.c_in, g.ho, g.wo, d.kh, d.pad, d.c_out, h->sm_count)) {
+            plan_patch(p, pl, d.n, d.c_in, g.ho, g.wo, d.kh, d.pad, d.c_out, h->sm_count) &&
+            !split_beats_patch(p, d.c_in, false, h->gemm_ctas)) {
             snprintf(buf, buf_bytes, "kernel=igemm_patch tile_n=%d accumulators=%d m_tiles=%d n_tiles=%d weights=%s", p.tile_n,
                      p.tile_n <= 128 ? 2 : 1, p.num_m_tiles, p.num_n_tiles, pl.b_resident ? "resident" : "streamed");
             return EOQ_OK;
@@ -1534,13 +1596,15 @@ extern "C" int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *des
         p.N = d.c_out;
         const bool rw = use_row_window(d, g.wo);
         plan_igemm(p, rw ? 8 * d.c_in : d.c_in, rw ? d.kh : g.taps, h->sm_count);
-        snprintf(buf, buf_bytes, "kernel=igemm%s tile_n=%d m_tiles=%d n_tiles=%d kc=%d stages=%d", rw ? "_filter_rows" : "",
-                 p.tile_n, p.num_m_tiles, p.num_n_tiles, p.kc, p.num_stages);
+        if (!rw) plan_split(p, h->gemm_ctas);
+        snprintf(buf, buf_bytes, "kernel=igemm%s tile_n=%d m_tiles=%d n_tiles=%d kc=%d stages=%d split=%d", rw ? "_filter_rows" : "",
+                 p.tile_n, p.num_m_tiles, p.num_n_tiles, p.kc, p.num_stages, p.split);
         return EOQ_OK;
     }
     if (pass == EOQ_PASS_DGRAD) {
         if (d.stride == 1 && d.kh == d.kw && d.kh - 1 - d.pad >= 0 &&
-            plan_patch(p, pl, d.n, d.c_out, d.h, d.w, d.kh, d.kh - 1 - d.pad, d.c_in, h->sm_count)) {
+            plan_patch(p, pl, d.n, d.c_out, d.h, d.w, d.kh, d.kh - 1 - d.pad, d.c_in, h->sm_count) &&
+            !split_beats_patch(p, d.c_out, true, h->gemm_ctas)) {
             snprintf(buf, buf_bytes, "kernel=igemm_patch tile_n=%d accumulators=%d m_tiles=%d n_tiles=%d weights=%s", p.tile_n,
                      p.tile_n <= 128 ? 2 : 1, p.num_m_tiles, p.num_n_tiles, pl.b_resident ? "resident" : "streamed");
             return EOQ_OK;

@@ -18,7 +18,11 @@ namespace {
 constexpr int kMaxStages = 8;
 constexpr int kProducers = 3;
 
-template <int kEpi>   // EpilogueKind: forward and dgrad are kernels of their own (registers, code size)
+// kEpi: EpilogueKind; forward and dgrad are kernels of their own (registers, code size).
+// kSplit: a cluster of p.split CTAs shares one tile.  Each runs its part of the reduction, hands every other CTA the partial
+// sums of that CTA's columns through distributed shared memory, and takes the epilogue of its own columns.  Small batches
+// leave a handful of tiles with long reductions: the 512-channel 7 x 7 layer at batch 1 took 13.3 us on 4 CTAs.
+template <int kEpi, bool kSplit>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUtensorMap map_a,
              const __grid_constant__ CUtensorMap map_b)
@@ -47,6 +51,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     const uint32_t buf_stride = nacc * acc_stride;
     const uint32_t tmem_cols = p.ep_groups * buf_stride;
 
+    if (kSplit) ptx::cluster_arrive();   // met below: the other blocks must have started before their shared memory is written
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.num_stages; ++s) {
             ptx::mbar_init(full_bar(s), 1);
@@ -69,6 +74,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    if (kSplit) ptx::cluster_wait();
     ptx::grid_dep_wait();   // everything up to here touched no global memory
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, p.dev};
@@ -78,7 +84,11 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     const int pix_per_img = p.hq * p.wq;
     // Every CTA walks the reduction from another starting point (the integer sums do not depend on the order): in step, all
     // CTAs of a column tile would ask the same L2 slices for the same weights at the same time.
-    const int k_first = (int)(blockIdx.x % (unsigned)k_iters);
+    // A cluster divides the iterations instead.
+    const int rank = kSplit ? (int)(blockIdx.x % (unsigned)p.split) : 0;
+    const int k_first = kSplit ? k_iters * rank / p.split : (int)(blockIdx.x % (unsigned)k_iters);
+    const int k_count = kSplit ? k_iters * (rank + 1) / p.split - k_first : k_iters;
+    const int tile_first = kSplit ? (int)blockIdx.x / p.split : (int)blockIdx.x;   // (a cluster has one tile)
 
     if (warp == 0 || warp == 2 || warp == 3) {
         if (lane == 0) {
@@ -90,13 +100,13 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
             int turn = q;  // slots until this producer's next one
             uint32_t inflight = 0, inflight_parity = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+            for (int tile = tile_first; tile < num_tiles && ok; tile += gridDim.x) {
                 const int mt = tile / p.num_n_tiles, nt = tile % p.num_n_tiles;
                 const int m0 = mt * kTileM;
                 const int img = m0 / pix_per_img, rem = m0 % pix_per_img;
                 const int cw = (rem % p.wq) * p.src_stride_w + p.base_w;
                 const int ch = (rem / p.wq) * p.src_stride + p.base_h;
-                for (int step = 0, kit = k_first; step < k_iters; ++step, kit = kit + 1 == k_iters ? 0 : kit + 1) {
+                for (int step = 0, kit = k_first; step < k_count; ++step, kit = kit + 1 == k_iters ? 0 : kit + 1) {
                     if (turn-- != 0) continue;
                     turn = kProducers - 1;
                     if (!(ok = wait_bar<32>(empty_bar(stage), phase ^ 1u, ctx))) break;
@@ -104,7 +114,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                     const int subs = min(p.subs_per_stage, p.num_sub - s0);
                     const uint32_t a_dst = smem_base + stage * stage_bytes;
                     const uint32_t b_dst = a_dst + p.subs_per_stage * a_sub;
-                    ptx::mbar_expect_tx(full_bar(stage), subs * (a_sub + b_sub));
+                    ptx::mbar_expect_tx(full_bar(stage), subs * ((uint32_t)p.a_rows * p.kc + b_sub));
                     for (int j = 0; j < subs; ++j) {
                         const int s = s0 + j;
                         const int sd = min(s, p.real_sub - 1);  // a padding sub-tile re-reads real data; its weights are zero
@@ -137,6 +147,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                             if (ptx::mbar_try_wait(full_bar(s), (inflight_parity >> s) & 1u)) break;
             }
         }
+        if (kSplit) ptx::cluster_sync();
     } else if (warp == 1) {
         // the whole warp runs the issue loop; one elected lane issues the MMAs and commits (see elect_one)
         const uint32_t leader = elect_one();
@@ -171,13 +182,13 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+        for (int tile = tile_first; tile < num_tiles && ok; tile += gridDim.x) {
             if (!(ok = __all_sync(0xffffffffu, wait_bar(tempty_bar(acc), acc_phase ^ 1u, ctx)))) break;
             ptx::tc_fence_after();
             const uint32_t d_tmem = tmem_base + acc * buf_stride, d_other = nacc == 2 ? d_tmem + acc_stride : d_tmem;
             uint32_t accumulate = 0;
             uint32_t fresh0 = 1u, fresh1 = nacc == 2 ? 1u : 0u;
-            for (int step = 0, kit = k_first; step < k_iters; ++step, kit = kit + 1 == k_iters ? 0 : kit + 1) {
+            for (int step = 0, kit = k_first; step < k_count; ++step, kit = kit + 1 == k_iters ? 0 : kit + 1) {
                 if (!(ok = __all_sync(0xffffffffu, wait_bar(full_bar(stage), phase, ctx)))) break;
                 ptx::tc_fence_after();
                 const int subs = min(p.subs_per_stage, p.num_sub - kit * p.subs_per_stage);
@@ -217,6 +228,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
             for (uint32_t i = 0; i < kSpinLimit; ++i)
                 if (ptx::mbar_try_wait(drain_bar, 0)) break;
         }
+        if (kSplit) ptx::cluster_sync();
     } else {
         // ---------------------------------------------------------------------- epilogue
         // A warp may read the TMEM lanes of quadrant (warp % 4).  The four warps of a quadrant form ep_groups groups; group
@@ -224,10 +236,14 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         // Everything that does not depend on the sums is formed before the wait for the tile's MMAs.
         const int quad = warp & 3;
         const int ew = (warp - 4) >> 2;
-        const int parts = 4 / p.ep_groups, grp = ew / parts, part = ew - grp * parts;
+        // (In a cluster all of them are one group, whatever the number of columns: each must reach the cluster's barrier.)
+        const int parts = kSplit ? 4 : 4 / p.ep_groups, grp = kSplit ? 0 : ew / parts, part = ew - grp * parts;
         const int row = quad * 32 + lane;
         const int groups = p.tile_n / 16;                 // 16-column groups of the tile
-        const int g_begin = (groups * part) / parts, g_end = (groups * (part + 1)) / parts;
+        const int own = kSplit ? groups / p.split : 1;    // groups whose epilogue is this CTA's (at most four)
+        const int g_begin = kSplit ? rank * own + part : (groups * part) / parts;
+        const int g_end = kSplit ? g_begin + (part < own ? 1 : 0) : (groups * (part + 1)) / parts;
+        const uint32_t red_base = smem_base + p.num_stages * stage_bytes + kTableSmemBytes;   // [source CTA][own group][4][row] x 16 bytes
         constexpr bool fwd = kEpi == kEpiForward;
         const FwdScalars fs = fwd ? load_fwd_scalars(p) : FwdScalars{0, 0, 0};
         // the b1 table of the whole layer goes to shared memory (behind the pipeline stages), once, times b1
@@ -239,7 +255,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
         const bool wide_out = (reinterpret_cast<uintptr_t>(p.acc_out) & 31) == 0;   // 256-bit stores of the exact sums
         bool ok = true;
-        for (int tile = blockIdx.x + grp * gridDim.x; tile < num_tiles && ok; tile += p.ep_groups * gridDim.x) {
+        for (int tile = tile_first + grp * gridDim.x; tile < num_tiles && ok; tile += p.ep_groups * gridDim.x) {
             const int mt = tile / p.num_n_tiles, nt = tile % p.num_n_tiles;
             const int m = mt * kTileM + row;
             const bool valid = m < p.M;
@@ -260,26 +276,61 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
             int4 sc = (fwd && valid && col < p.N && p.shortcut) ? __ldg(reinterpret_cast<const int4 *>(p.shortcut + off)) : zero4;
             const int32_t *tb = ts ? ts + cls * p.N + col : nullptr;
             const int32_t *tg = (!ts && p.b1_table) ? p.b1_table + (size_t)cls * p.N + col : nullptr;
-            if (!(ok = __all_sync(0xffffffffu, wait_bar(tfull_bar(grp), acc_phase, ctx)))) break;  // warp-uniform
+            ok = __all_sync(0xffffffffu, wait_bar(tfull_bar(grp), acc_phase, ctx));  // warp-uniform
             ptx::tc_fence_after();
             const uint32_t t_row = tmem_base + grp * buf_stride + ((uint32_t)(quad * 32) << 16);
+            if (kSplit) {
+#pragma unroll 1
+                for (int g = part; g < groups && ok; g += 4) {
+                    uint32_t r[32], r2[32];
+                    ptx::tmem_ld_32x16(t_row + g * 16, r);
+                    if (nacc == 2) ptx::tmem_ld_32x16(t_row + acc_stride + g * 16, r2);
+                    ptx::tmem_ld_wait();
+                    if (nacc == 2) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) r[i] += r2[i];
+                    }
+                    const uint32_t dst = ptx::cluster_addr(red_base + (((rank * own + g % own) * 4) * kTileM + row) * 16, g / own);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        ptx::st_cluster_128(dst + c * kTileM * 16, r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+                }
+                ptx::cluster_sync();
+            }
+            if (!ok) break;
             for (int g = g_begin; g < g_end; ++g, col += 16, off += 16) {
                 uint32_t r[32];
-                ptx::tmem_ld_32x16(t_row + g * 16, r);
                 uint32_t r2[32];
-                if (nacc == 2) ptx::tmem_ld_32x16(t_row + acc_stride + g * 16, r2);
+                if (kSplit) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) r[i] = 0;
+#pragma unroll 1
+                    for (int src = 0; src < p.split; ++src) {
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const int4 v = ptx::ld_shared_128(red_base + (((src * own + part) * 4 + c) * kTileM + row) * 16);
+                            r[4 * c] += v.x;
+                            r[4 * c + 1] += v.y;
+                            r[4 * c + 2] += v.z;
+                            r[4 * c + 3] += v.w;
+                        }
+                    }
+                } else {
+                    ptx::tmem_ld_32x16(t_row + g * 16, r);
+                    if (nacc == 2) ptx::tmem_ld_32x16(t_row + acc_stride + g * 16, r2);
+                }
                 // the next group's shortcut codes travel while this group is computed
                 int4 sc_next = zero4;
                 if (g + 1 < g_end && fwd && valid && col + 16 < p.N && p.shortcut)
                     sc_next = __ldg(reinterpret_cast<const int4 *>(p.shortcut + off + 16));
-                ptx::tmem_ld_wait();
-                if (nacc == 2 && !fwd) {
+                if (!kSplit) ptx::tmem_ld_wait();
+                if (nacc == 2 && !fwd && !kSplit) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) r[i] += r2[i];  // the two partial accumulators of the tile
                 }
                 if (valid && col < p.N) {
                     if (fwd) {
-                        forward_group(p, fs, sh, r, r2, nacc, off, tb, tg, sc, shift);
+                        forward_group(p, fs, sh, r, r2, kSplit ? 1u : nacc, off, tb, tg, sc, shift);
                     } else {
                         mx = max(mx, wide_out ? dgrad_16<true>(p, r, off, mx_masked) : dgrad_16<false>(p, r, off, mx_masked));
                     }
@@ -315,17 +366,19 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
 
 size_t igemm_smem_bytes(const IgemmParams &p)
 {
-    return (size_t)p.num_stages * p.subs_per_stage * ((size_t)kTileM + p.tile_n) * p.kc + 1024 + kTableSmemBytes;
+    return (size_t)p.num_stages * p.subs_per_stage * ((size_t)kTileM + p.tile_n) * p.kc + 1024 + kTableSmemBytes +
+           (p.split > 1 ? (size_t)kTileM * p.tile_n * sizeof(int32_t) : 0);
 }
 
 cudaError_t launch_igemm(const IgemmParams &p, const CUtensorMap &map_a, const CUtensorMap &map_b, int grid,
                          cudaStream_t stream)
 {
     const size_t smem = igemm_smem_bytes(p);
-    const auto kernel = p.epilogue == kEpiForward ? igemm_kernel<kEpiForward> : igemm_kernel<kEpiDgrad>;
+    const auto kernel = p.split > 1 ? (p.epilogue == kEpiForward ? igemm_kernel<kEpiForward, true> : igemm_kernel<kEpiDgrad, true>)
+                                    : (p.epilogue == kEpiForward ? igemm_kernel<kEpiForward, false> : igemm_kernel<kEpiDgrad, false>);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e != cudaSuccess) return e;
-    return launch_chained(kernel, grid, kGemmThreads, smem, stream, p, map_a, map_b);
+    return launch_chained_clusters(p.split, kernel, grid, kGemmThreads, smem, stream, p, map_a, map_b);
 }
 
 }  // namespace eoq

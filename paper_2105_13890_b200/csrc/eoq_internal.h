@@ -21,19 +21,28 @@ constexpr uint32_t kSpinLimit = 1u << 22;  // polls before a wait gives up (norm
 // touches global memory, in every block.  Launch latency and prologue, about 1.5 us per kernel in a captured chain, then
 // overlap the predecessor's last microseconds.
 template <typename... P, typename... A>
-inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A &&...args)
+inline cudaError_t launch_chained_clusters(int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                           A &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A &&...args)
+{
+    return launch_chained_clusters(1, kernel, grid, block, smem, stream, static_cast<A &&>(args)...);
 }
 
 struct DeviceState {
@@ -171,6 +180,8 @@ struct IgemmParams {
     // Tiles a CTA has in the epilogue at once (1, 2 or 4): as many accumulator buffers in tensor memory, each served by
     // kEpilogueWarps / ep_groups warps (see plan_epilogue)
     int ep_groups;
+    int a_rows;   // pixels of an activation load: 128, or less when the whole problem has fewer
+    int split;    // CTAs (a cluster) that share a tile's reduction and its columns in the epilogue; 1: one CTA per tile
 };
 
 // Patch variant of the implicit GEMM for stride-1 filters (eoq_igemm_patch.cu): an M tile is `r_rows` output rows

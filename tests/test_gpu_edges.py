@@ -176,3 +176,32 @@ def test_odd_channel_counts(d, ctas):
     assert np.array_equal(G.host(g).astype(np.int32), want) and pg.item() == p
     assert eoq.eoq_last_status(h) == 0
     eoq.eoq_destroy(h)
+
+
+@pytest.mark.parametrize("d", [
+    oracle.ConvDesc(1, 7, 7, 512, 512, 3, 3, 1, 1),    # 49 pixels, eight CTAs a tile
+    oracle.ConvDesc(1, 14, 14, 256, 256, 3, 3, 1, 1),  # a ragged second row tile
+    oracle.ConvDesc(1, 4, 4, 512, 128, 3, 3, 1, 1),    # exactly 16 pixels
+    oracle.ConvDesc(1, 1, 17, 512, 128, 1, 1, 1, 0),   # 17 pixels
+    oracle.ConvDesc(2, 8, 8, 576, 192, 3, 3, 1, 1),    # 64-channel sub-tiles, two column tiles of 12 groups
+    oracle.ConvDesc(3, 7, 7, 512, 1040, 1, 1, 1, 0),   # columns that end inside a tile
+    oracle.ConvDesc(2, 6, 6, 512, 32, 3, 3, 1, 1),     # two 16-column groups: fewer than the warps of a quadrant
+    oracle.ConvDesc(2, 14, 14, 256, 512, 3, 3, 2, 1),  # residue classes with their own splits
+], ids=lambda d: f"n{d.n}_{d.h}x{d.w}_c{d.c_in}-{d.c_out}_k{d.kh}s{d.stride}")
+@pytest.mark.parametrize("b1", [0, 3])
+def test_reduction_shared_by_a_cluster(d, b1):
+    x, sc = synth.relu_codes((d.n, d.h, d.w, d.c_in), 1580, 0), synth.int8_uniform((d.n, d.ho, d.wo, d.c_out), 1580, 1)
+    w, e3 = synth.int8_uniform((d.c_out, d.kh, d.kw, d.c_in), 1580, 2, -30, 30), synth.normal_codes((d.n, d.ho, d.wo, d.c_out), 1580, 3)
+    gd, h = G.gdesc(d), G.handle()
+    ref = oracle.layer_forward(d, x, b1, w, 90, 5, sc, True)
+    want, p, _ = oracle.sq_int(oracle.conv_dgrad_acc(d, e3, w), -9 - 7)
+    x5, x2, mask = G.zeros(sc.shape, torch.int8), G.zeros(sc.shape, torch.int16), G.zeros((sc.size + 7) // 8, torch.uint8)
+    e4, pe = G.zeros(x.shape, torch.int8), G.zeros(1, torch.int32)
+    for _ in range(2):
+        eoq.eoq_conv_fwd(h, gd, G.dev(x), None, b1, G.dev(w), 90, 5, G.dev(sc), True, x5, x2, mask, None, G.workspace(gd, eoq.EOQ_PASS_FWD))
+        eoq.eoq_conv_dgrad(h, gd, G.dev(e3), G.dev(np.array([-9], dtype=np.int32)), G.dev(w), e4, pe, None, None,
+                           G.workspace(gd, eoq.EOQ_PASS_DGRAD))
+        assert np.array_equal(G.host(x5), ref["x5"]) and np.array_equal(G.host(x2).astype(np.int32), ref["x2"])
+        assert np.array_equal(G.unpack_mask(mask, sc.shape), ref["mask"])
+        assert np.array_equal(G.host(e4).astype(np.int32), want) and pe.item() == p
+        assert G.status_clear() == 0
