@@ -13,11 +13,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ uint32_t pack4(int a, int b, int c, int d)
-{
-    return (uint32_t)(a & 0xff) | ((uint32_t)(b & 0xff) << 8) | ((uint32_t)(c & 0xff) << 16) | ((uint32_t)(d & 0xff) << 24);
-}
-
 inline int blocks_for(size_t items, int sm_count, int per_sm = 8)
 {
     size_t b = (items + kThreads - 1) / kThreads, cap = (size_t)sm_count * per_sm;
@@ -26,13 +21,6 @@ inline int blocks_for(size_t items, int sm_count, int per_sm = 8)
 }
 
 // ------------------------------------------------------------------ join of two error streams + Q_e
-
-__device__ __forceinline__ void unpack16(const int4 &v, int (&o)[16])
-{
-    const int8_t *b = reinterpret_cast<const int8_t *>(&v);
-#pragma unroll
-    for (int k = 0; k < 16; ++k) o[k] = b[k];
-}
 
 // pass = 0: max |S| into the handle's 64-bit cell; pass = 1: codes of SQ(S), their sum, exponent; cells back to zero.
 // kNext: the error head of the layer that consumes the joined error rides along (see NextHead): pass 0 also reduces
@@ -49,8 +37,9 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
     long long sum = 0, s1 = 0, s2 = 0;
     int t = 7;
     NextHead nh = {};
+    unsigned long long M = 0;
     if (kPass == 1) {
-        const unsigned long long M = dev->absmax_u64;
+        M = dev->absmax_u64;
         t = M ? round_log2_u64(M) : 7;
         const int p0 = M ? j.p + t - 7 : j.p;
         if (kNext) {
@@ -67,66 +56,70 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
     const bool narrow = j.sa >= 0 && j.sb >= 0 && j.sa <= 23 && j.sb <= 23;
     const int ma = 1 << (j.sa < 0 ? 0 : min(j.sa, 23)), mb = 1 << (j.sb < 0 ? 0 : min(j.sb, 23));
     uint32_t mx32 = 0, mxm32 = 0;
+    // sums below 2^31 - 2^(t - 8): a right shift in few 32-bit operations (see sq_pack4_shr)
+    const int sh = t - 7;
+    const bool fast = narrow && sh >= 1 && M < 0x7e000000ull;
+    const int32_t half_m1 = fast ? (1 << (sh - 1)) - 1 : 0, lo = fast ? -(127 << sh) : 0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
-        int av[16], bv[16];
-        unpack16(__ldg(reinterpret_cast<const int4 *>(a) + i), av);
-        unpack16(__ldg(reinterpret_cast<const int4 *>(b) + i), bv);
+        const int4 a4 = __ldg(reinterpret_cast<const int4 *>(a) + i), b4 = __ldg(reinterpret_cast<const int4 *>(b) + i);
         const uint32_t m = mask_b ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(mask_b) + i) : 0xffffu;
         const uint32_t nm = kNext ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(next_mask) + i) : 0u;
-        int c[16];
-        if (narrow) {
+        const uint32_t aw[4] = {(uint32_t)a4.x, (uint32_t)a4.y, (uint32_t)a4.z, (uint32_t)a4.w};
+        const uint32_t bw[4] = {(uint32_t)b4.x, (uint32_t)b4.y, (uint32_t)b4.z, (uint32_t)b4.w};
+        uint32_t cw[4];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const int s32 = av[q] * ma + (((m >> q) & 1u) ? bv[q] : 0) * mb;
-                if (kPass == 0) {
-                    const uint32_t v = (uint32_t)abs(s32);
-                    mx32 = max(mx32, v);
-                    if (kNext && ((nm >> q) & 1u)) mxm32 = max(mxm32, v);
-                } else {
-                    c[q] = sq_code32(s32, t);
-                }
-            }
-        } else {
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t g = bw[q] & bits_to_bytes(m >> (4 * q));
+            const int av[4] = {sbyte<0>(aw[q]), sbyte<1>(aw[q]), sbyte<2>(aw[q]), sbyte<3>(aw[q])};
+            const int bv[4] = {sbyte<0>(g), sbyte<1>(g), sbyte<2>(g), sbyte<3>(g)};
+            if (narrow) {
+                int s32[4];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const long long s = join_one(av[q], ((m >> q) & 1u) ? bv[q] : 0, j);
-                if (kPass == 0) {
-                    const unsigned long long u = (unsigned long long)(s < 0 ? -s : s);
-                    mx = u > mx ? u : mx;
-                    if (kNext && ((nm >> q) & 1u)) mxm = u > mxm ? u : mxm;
-                } else {
-                    c[q] = sq_code64(s, t);
+                for (int k = 0; k < 4; ++k) {
+                    s32[k] = av[k] * ma + bv[k] * mb;
+                    if (kPass == 0) {
+                        const uint32_t v = (uint32_t)abs(s32[k]);
+                        mx32 = max(mx32, v);
+                        if (kNext && ((nm >> (4 * q + k)) & 1u)) mxm32 = max(mxm32, v);
+                    }
                 }
+                if (kPass == 1)
+                    cw[q] = fast ? sq_pack4_shr(s32, sh, half_m1, lo)
+                                 : pack4_sat(sq_code32(s32[0], t), sq_code32(s32[1], t), sq_code32(s32[2], t), sq_code32(s32[3], t));
+            } else {
+                int c[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const long long s = join_one(av[k], bv[k], j);
+                    if (kPass == 0) {
+                        const unsigned long long u = (unsigned long long)(s < 0 ? -s : s);
+                        mx = u > mx ? u : mx;
+                        if (kNext && ((nm >> (4 * q + k)) & 1u)) mxm = u > mxm ? u : mxm;
+                    } else {
+                        c[k] = sq_code64(s, t);
+                    }
+                }
+                if (kPass == 1) cw[q] = pack4_sat(c[0], c[1], c[2], c[3]);
             }
         }
         if (kPass == 1) {
-            int sum32 = 0;
+            int sum16 = 0;
 #pragma unroll
-            for (int q = 0; q < 16; ++q) sum32 += c[q];
-            sum += sum32;
-            reinterpret_cast<int4 *>(out)[i] = make_int4((int)pack4(c[0], c[1], c[2], c[3]), (int)pack4(c[4], c[5], c[6], c[7]),
-                                                          (int)pack4(c[8], c[9], c[10], c[11]), (int)pack4(c[12], c[13], c[14], c[15]));
+            for (int q = 0; q < 4; ++q) sum16 = __dp4a((int)cw[q], 0x01010101, sum16);
+            sum += sum16;
+            reinterpret_cast<int4 *>(out)[i] = make_int4((int)cw[0], (int)cw[1], (int)cw[2], (int)cw[3]);
             if (kNext) {
-                int e1[16], c3[16], a1 = 0;
+                uint32_t e1[4], c3[4];
+                int a1 = 0;
 #pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    e1[q] = ((nm >> q) & 1u) ? c[q] : 0;
-                    a1 += e1[q];
-                    c3[q] = next_head_code(nh, e1[q]);
+                for (int q = 0; q < 4; ++q) {
+                    e1[q] = cw[q] & bits_to_bytes(nm >> (4 * q));
+                    a1 = __dp4a((int)e1[q], 0x01010101, a1);
+                    c3[q] = next_head_codes(nh, e1[q]);
                 }
                 s1 += a1;
-                if (next_x2) {
-                    const int4 lo = __ldg(reinterpret_cast<const int4 *>(next_x2) + 2 * i);
-                    const int4 hi = __ldg(reinterpret_cast<const int4 *>(next_x2) + 2 * i + 1);
-                    const int16_t *pl = reinterpret_cast<const int16_t *>(&lo), *ph = reinterpret_cast<const int16_t *>(&hi);
-                    int a2 = 0;  // |e1 * x2| < 2^22, 16 terms
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) a2 += e1[q] * pl[q] + e1[8 + q] * ph[q];
-                    s2 += a2;
-                }
-                reinterpret_cast<int4 *>(e3)[i] =
-                    make_int4((int)pack4(c3[0], c3[1], c3[2], c3[3]), (int)pack4(c3[4], c3[5], c3[6], c3[7]),
-                              (int)pack4(c3[8], c3[9], c3[10], c3[11]), (int)pack4(c3[12], c3[13], c3[14], c3[15]));
+                if (next_x2) s2 += dot16_s8_s16(e1, reinterpret_cast<const int4 *>(next_x2) + 2 * i);
+                reinterpret_cast<int4 *>(e3)[i] = make_int4((int)c3[0], (int)c3[1], (int)c3[2], (int)c3[3]);
             }
         }
     }
@@ -139,17 +132,12 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
             if (kNext && mxm) atomicMax(&dev->absmax2_u64, mxm);
         }
     } else {
-        if (sum_out) {
-            sum = block_sum_i64(sum);
-            if (threadIdx.x == 0 && sum) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)sum);
-        }
-        if (kNext) {
-            s1 = block_sum_i64(s1);
-            s2 = block_sum_i64(s2);
-            if (threadIdx.x == 0) {
-                if (s1) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum1), (unsigned long long)s1);
-                if (s2) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum2), (unsigned long long)s2);
-            }
+        long long v[3] = {sum, s1, s2};
+        block_sums_i64(v);
+        if (threadIdx.x == 0) {
+            if (sum_out && v[0]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)v[0]);
+            if (kNext && v[1]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum1), (unsigned long long)v[1]);
+            if (kNext && v[2]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum2), (unsigned long long)v[2]);
         }
         if (last_block_done(dev)) {
             if (sum_out) *sum_out = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum0), 0ull);

@@ -38,6 +38,16 @@ __device__ __forceinline__ uint32_t pack4_sat(int c0, int c1, int c2, int c3)
     return r;
 }
 
+// byte k of w, sign-extended
+template <int k>
+__device__ __forceinline__ int32_t sbyte(uint32_t w)
+{
+    // prmt selector digit 8 + k replicates the sign bit of byte k (the __byte_perm intrinsic drops that bit)
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %1, %2;" : "=r"(r) : "r"(w), "n"(((8 + k) << 12) | ((8 + k) << 8) | ((8 + k) << 4) | k));
+    return (int32_t)r;
+}
+
 // R(log2 M) for M >= 1: floor(log2 M) plus one when M^2 >= 2^(2f+1).
 __device__ __forceinline__ int round_log2_u32(uint32_t M)
 {
@@ -69,6 +79,35 @@ __device__ __forceinline__ int32_t sq_code32(int32_t a, int t)
 __device__ __forceinline__ int32_t sq_code32_shr(int32_t a, int s, int32_t half_m1)
 {
     return clampi((a + half_m1 + ((a >> s) & 1)) >> s, -127, 127);
+}
+
+// Four such codes in a word: the lower clamp rides on the addition (`lo` = -127 * 2^s), the pack saturates at 127.
+__device__ __forceinline__ uint32_t sq_pack4_shr(const int32_t *a, int s, int32_t half_m1, int32_t lo)
+{
+    int32_t v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = (__viaddmax_s32(a[k], half_m1, lo) + ((a[k] >> s) & 1)) >> s;
+    return pack4_sat(v[0], v[1], v[2], v[3]);
+}
+
+// Expands 4 mask bits into 4 byte masks (0x00 / 0xff).
+__device__ __forceinline__ uint32_t bits_to_bytes(uint32_t nibble)
+{
+    return (((nibble & 0xfu) * 0x00204081u) & 0x01010101u) * 0xffu;
+}
+
+// sum of the 16 products of the codes in e with 16-bit values at x (32 bytes): below 2^26
+__device__ __forceinline__ int dot16_s8_s16(const uint32_t (&e)[4], const int4 *x)
+{
+    const int4 lo = __ldg(x), hi = __ldg(x + 1);
+    int s = __dp2a_lo(lo.x, (int)e[0], 0);
+    s = __dp2a_hi(lo.y, (int)e[0], s);
+    s = __dp2a_lo(lo.z, (int)e[1], s);
+    s = __dp2a_hi(lo.w, (int)e[1], s);
+    s = __dp2a_lo(hi.x, (int)e[2], s);
+    s = __dp2a_hi(hi.y, (int)e[2], s);
+    s = __dp2a_lo(hi.z, (int)e[3], s);
+    return __dp2a_hi(hi.w, (int)e[3], s);
 }
 
 __device__ __forceinline__ int32_t sq_code64(long long a, int t)
@@ -169,6 +208,23 @@ __device__ __forceinline__ long long block_sum_i64(long long v)
     if (warp == 0) v = warp_sum_i64(lane < nw ? red_sum[lane] : 0ll);
     __syncthreads();
     return v;
+}
+
+// kN sums over the block behind one barrier, valid in thread 0 (and once per kernel: the cells are not free again)
+template <int kN>
+__device__ __forceinline__ void block_sums_i64(long long (&v)[kN])
+{
+    __shared__ long long red_sums[kN][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+        v[i] = warp_sum_i64(v[i]);
+        if (lane == 0) red_sums[i][warp] = v[i];
+    }
+    __syncthreads();
+    if (warp == 0)
+#pragma unroll
+        for (int i = 0; i < kN; ++i) v[i] = warp_sum_i64(lane < nw ? red_sums[i][lane] : 0ll);
 }
 
 // ------------------------------------------------------------------ PTX: shared-memory barriers and TMA

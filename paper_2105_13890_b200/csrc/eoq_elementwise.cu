@@ -340,10 +340,12 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
     }
     // the maximum bounds every element, so |a| + 2^(sh-1) cannot wrap as long as M + M / 2^7 < 2^31
     const bool fast = sh >= 1 && M < 0x7e000000u;
-    const int32_t half_m1 = fast ? (1 << (sh - 1)) - 1 : 0;
+    const int32_t half_m1 = fast ? (1 << (sh - 1)) - 1 : 0, lo = fast ? -(127 << sh) : 0;
+    uint32_t jm32 = 0, jmm32 = 0;
     const bool wide_in = (reinterpret_cast<uintptr_t>(src) & 31) == 0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
-        int c[16], a[16];
+        int a[16];
+        uint32_t cw[4];   // four codes per word
         if (wide_in) {   // two 256-bit loads: whole 32-byte sectors per lane
             ld_global_256_stream(src + i * 16, a);
             ld_global_256_stream(src + i * 16 + 8, a + 8);
@@ -357,61 +359,53 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
                 a[4 * k + 3] = v.w;
             }
         }
-        if (fast) {
+        int sum16 = 0;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) c[k] = sq_code32_shr(a[k], sh, half_m1);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 16; ++k) c[k] = sq_code32(a[k], t);
+        for (int q = 0; q < 4; ++q) {
+            cw[q] = fast ? sq_pack4_shr(a + 4 * q, sh, half_m1, lo)
+                         : pack4_sat(sq_code32(a[4 * q], t), sq_code32(a[4 * q + 1], t), sq_code32(a[4 * q + 2], t), sq_code32(a[4 * q + 3], t));
+            sum16 = __dp4a((int)cw[q], 0x01010101, sum16);
         }
-        int s = 0;
-#pragma unroll
-        for (int k = 0; k < 16; ++k) s += c[k];
-        sum += s;
-        reinterpret_cast<int4 *>(dst)[i] =
-            make_int4((int)pack4(c[0], c[1], c[2], c[3]), (int)pack4(c[4], c[5], c[6], c[7]),
-                      (int)pack4(c[8], c[9], c[10], c[11]), (int)pack4(c[12], c[13], c[14], c[15]));
+        sum += sum16;
+        reinterpret_cast<int4 *>(dst)[i] = make_int4((int)cw[0], (int)cw[1], (int)cw[2], (int)cw[3]);
         if (kJoin) {
             const int4 bq = __ldg(reinterpret_cast<const int4 *>(join.b) + i);
-            const int8_t *bb = reinterpret_cast<const int8_t *>(&bq);
             const uint32_t gate = join.mask_b ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(join.mask_b) + i) : 0xffffu;
             const uint32_t nm = join.next_mask ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(join.next_mask) + i) : 0u;
+            const uint32_t bw[4] = {(uint32_t)bq.x, (uint32_t)bq.y, (uint32_t)bq.z, (uint32_t)bq.w};
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const int bv = ((gate >> k) & 1u) ? (int)bb[k] : 0;
-                unsigned long long u;
-                if (j_narrow) {
-                    u = (unsigned long long)(uint32_t)abs(c[k] * j_ma + bv * j_mb);
-                } else {
-                    const long long v = join_one(c[k], bv, js);
-                    u = (unsigned long long)(v < 0 ? -v : v);
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t g = bw[q] & bits_to_bytes(gate >> (4 * q)), m = nm >> (4 * q);
+                const int bv[4] = {sbyte<0>(g), sbyte<1>(g), sbyte<2>(g), sbyte<3>(g)};
+                const int cv[4] = {sbyte<0>(cw[q]), sbyte<1>(cw[q]), sbyte<2>(cw[q]), sbyte<3>(cw[q])};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (j_narrow) {
+                        const uint32_t u = (uint32_t)abs(cv[k] * j_ma + bv[k] * j_mb);
+                        jm32 = max(jm32, u);
+                        if (m & (1u << k)) jmm32 = max(jmm32, u);
+                    } else {
+                        const long long v = join_one(cv[k], bv[k], js);
+                        const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
+                        jmx = u > jmx ? u : jmx;
+                        if (m & (1u << k)) jmxm = u > jmxm ? u : jmxm;
+                    }
                 }
-                jmx = u > jmx ? u : jmx;
-                if ((nm >> k) & 1u) jmxm = u > jmxm ? u : jmxm;
             }
         }
         if (kNext) {
             const uint32_t bits = (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(next.mask) + i);
-            int e1[16], c3[16], a1 = 0;
+            uint32_t e1[4], c3[4];
+            int a1 = 0;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                e1[k] = ((bits >> k) & 1u) ? c[k] : 0;
-                a1 += e1[k];
-                c3[k] = next_head_code(nh, e1[k]);
+            for (int q = 0; q < 4; ++q) {
+                e1[q] = cw[q] & bits_to_bytes(bits >> (4 * q));
+                a1 = __dp4a((int)e1[q], 0x01010101, a1);
+                c3[q] = next_head_codes(nh, e1[q]);
             }
             s1 += a1;
-            if (next.x2) {
-                const int4 lo = __ldg(reinterpret_cast<const int4 *>(next.x2) + 2 * i);
-                const int4 hi = __ldg(reinterpret_cast<const int4 *>(next.x2) + 2 * i + 1);
-                const int16_t *pl = reinterpret_cast<const int16_t *>(&lo), *ph = reinterpret_cast<const int16_t *>(&hi);
-                int a2 = 0;  // |e1 * x2| < 2^22, 16 terms
-#pragma unroll
-                for (int k = 0; k < 8; ++k) a2 += e1[k] * pl[k] + e1[8 + k] * ph[k];
-                s2 += a2;
-            }
-            reinterpret_cast<int4 *>(next.e3)[i] =
-                make_int4((int)pack4(c3[0], c3[1], c3[2], c3[3]), (int)pack4(c3[4], c3[5], c3[6], c3[7]),
-                          (int)pack4(c3[8], c3[9], c3[10], c3[11]), (int)pack4(c3[12], c3[13], c3[14], c3[15]));
+            if (next.x2) s2 += dot16_s8_s16(e1, reinterpret_cast<const int4 *>(next.x2) + 2 * i);
+            reinterpret_cast<int4 *>(next.e3)[i] = make_int4((int)c3[0], (int)c3[1], (int)c3[2], (int)c3[3]);
         }
     }
     ptx::grid_dep_launch();
@@ -421,22 +415,24 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
             sum += c;
             dst[i] = (int8_t)c;
         }
-    if (sum_codes) {
-        sum = block_sum_i64(sum);
-        if (threadIdx.x == 0 && sum) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)sum);
-    }
-    if (kNext) {
-        s1 = block_sum_i64(s1);
-        s2 = block_sum_i64(s2);
+    {
+        long long v[kNext ? 3 : 1];
+        v[0] = sum;
+        if (kNext) {
+            v[kNext ? 1 : 0] = s1;
+            v[kNext ? 2 : 0] = s2;
+        }
+        if (kNext || sum_codes) block_sums_i64(v);
         if (threadIdx.x == 0) {
-            if (s1) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum1), (unsigned long long)s1);
-            if (s2) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum2), (unsigned long long)s2);
+            if (sum_codes && v[0]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)v[0]);
+            if (kNext && v[kNext ? 1 : 0]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum1), (unsigned long long)v[kNext ? 1 : 0]);
+            if (kNext && v[kNext ? 2 : 0]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum2), (unsigned long long)v[kNext ? 2 : 0]);
         }
     }
     if (kJoin) {
         // the join's second pass (the next kernel on the stream) reads these cells and puts them back to zero
-        jmx = block_max_u64(jmx);
-        jmxm = block_max_u64(jmxm);
+        jmx = block_max_u64(jmx > jm32 ? jmx : (unsigned long long)jm32);
+        jmxm = block_max_u64(jmxm > jmm32 ? jmxm : (unsigned long long)jmm32);
         if (threadIdx.x == 0) {
             if (jmx) atomicMax(&dev->absmax_u64, jmx);
             if (jmxm) atomicMax(&dev->absmax2_u64, jmxm);
@@ -513,12 +509,6 @@ __global__ void sq_i32_scatter_kernel(const int32_t *__restrict__ src, const int
 // ------------------------------------------------------------------ head of the error chain
 
 // Pass 1: max |e1| and the sums behind g_b2 and g_gamma, with e1 = e0 * [x4 > 0].
-// Expands 4 mask bits into 4 byte masks (0x00 / 0xff).
-__device__ __forceinline__ uint32_t bits_to_bytes(uint32_t nibble)
-{
-    return (((nibble & 0xfu) * 0x00204081u) & 0x01010101u) * 0xffu;
-}
-
 __global__ void prescale_reduce_kernel(const int8_t *__restrict__ e0, const uint8_t *__restrict__ mask,
                                        const int16_t *__restrict__ x2, size_t n16, DeviceState *dev)
 {
@@ -691,22 +681,15 @@ prescale_fused_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, cons
             }
             s1 += a1;
             const size_t i = i0 + u * stride;
-            if (x2 && i < n16) {
-                const int4 lo = __ldg(reinterpret_cast<const int4 *>(x2) + 2 * i);
-                const int4 hi = __ldg(reinterpret_cast<const int4 *>(x2) + 2 * i + 1);
-                const int16_t *pl = reinterpret_cast<const int16_t *>(&lo), *ph = reinterpret_cast<const int16_t *>(&hi);
-                const int8_t *eb = reinterpret_cast<const int8_t *>(e1w[u]);
-                int a2 = 0;  // |e1 * x2| < 2^22, 16 terms
-#pragma unroll
-                for (int k = 0; k < 8; ++k) a2 += (int)eb[k] * pl[k] + (int)eb[8 + k] * ph[k];
-                s2 += a2;
-            }
+            if (x2 && i < n16) s2 += dot16_s8_s16(e1w[u], reinterpret_cast<const int4 *>(x2) + 2 * i);
         }
     }
     uint32_t mx = max(max(mx4 & 0xffu, (mx4 >> 8) & 0xffu), max((mx4 >> 16) & 0xffu, mx4 >> 24));
-    mx = (uint32_t)block_max_u64(mx);
-    s1 = block_sum_i64(s1);
-    s2 = block_sum_i64(s2);
+    mx = block_max_u32(mx);
+    long long sums[2] = {s1, s2};
+    block_sums_i64(sums);
+    s1 = sums[0];
+    s2 = sums[1];
     if (threadIdx.x == 0) {
         if (mx) atomicMax(&dev->absmax_u32, mx);
         if (s1) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)s1);
@@ -737,26 +720,18 @@ prescale_fused_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, cons
         if (sum_e1x2) *sum_e1x2 = *reinterpret_cast<volatile long long *>(&dev->sum1);
     }
     // same rounding as prescale_apply_kernel: R(gamma * e1 * 2^(7-t)) with one FMA
-    constexpr uint32_t kMagic = 0x4B400000u;
-    const float scale = __int_as_float((127 + 7 - t) << 23);
-    const float rest = 12582912.0f - 12582912.0f * scale;
-    const uint32_t g = (uint32_t)gamma_c;
+    NextHead nh;
+    nh.g = (uint32_t)gamma_c;
+    nh.scale = __int_as_float((127 + 7 - t) << 23);
+    nh.rest = 12582912.0f - 12582912.0f * nh.scale;
 #pragma unroll
     for (int u = 0; u < kFusedGroups; ++u) {
         const size_t i = i0 + u * stride;
         if (i >= n16) continue;
-        int c[16];
+        uint32_t c3[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int32_t e1 = (int32_t)(int8_t)(e1w[u][q] >> (8 * k));
-                const uint32_t r = __float_as_uint(__fmaf_rn(__uint_as_float(g * (uint32_t)e1 + kMagic), scale, rest));
-                c[4 * q + k] = clampi((int32_t)(r - kMagic), -127, 127);
-            }
-        reinterpret_cast<int4 *>(e3)[i] =
-            make_int4((int)pack4(c[0], c[1], c[2], c[3]), (int)pack4(c[4], c[5], c[6], c[7]),
-                      (int)pack4(c[8], c[9], c[10], c[11]), (int)pack4(c[12], c[13], c[14], c[15]));
+        for (int q = 0; q < 4; ++q) c3[q] = next_head_codes(nh, e1w[u][q]);
+        reinterpret_cast<int4 *>(e3)[i] = make_int4((int)c3[0], (int)c3[1], (int)c3[2], (int)c3[3]);
     }
     if (last_block_done(dev)) {
         dev->absmax_u32 = 0;

@@ -47,16 +47,6 @@ __device__ __forceinline__ uint32_t rne7_magic(uint32_t biased)
     return __float_as_uint(__fmaf_rn(__uint_as_float(biased), 0.0078125f, kMagicRest));
 }
 
-// byte k of w, sign-extended
-template <int k>
-__device__ __forceinline__ int32_t sbyte(uint32_t w)
-{
-    // prmt selector digit 8 + k replicates the sign bit of byte k (the __byte_perm intrinsic drops that bit)
-    uint32_t r;
-    asm("prmt.b32 %0, %1, %1, %2;" : "=r"(r) : "r"(w), "n"(((8 + k) << 12) | ((8 + k) << 8) | ((8 + k) << 4) | k));
-    return (int32_t)r;
-}
-
 // Forward chain on 16 consecutive output channels of one pixel (Sec. 3.2.1: x2 = Q_a1(conv), x3 = gamma x2,
 // x4 = x3 + b2 [+ shortcut], x5 = Q_a2(relu(x4)); mask = [x4 > 0]).
 // The integer pipe bounds this code (an instruction every two cycles and scheduler), so clamps are moved in front of the

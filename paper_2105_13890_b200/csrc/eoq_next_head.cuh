@@ -39,6 +39,20 @@ __device__ __forceinline__ int next_head_code(const NextHead &nh, int e1)
     return v < -127 ? -127 : (v > 127 ? 127 : v);
 }
 
+// the codes of four errors: the subtraction of the magic number and the lower clamp are one instruction, the pack saturates
+// at 127
+__device__ __forceinline__ uint32_t next_head_codes(const NextHead &nh, uint32_t e1)
+{
+    const int32_t e[4] = {sbyte<0>(e1), sbyte<1>(e1), sbyte<2>(e1), sbyte<3>(e1)};
+    int32_t v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t biased = nh.g * (uint32_t)e[k] + kHeadMagic;
+        v[k] = __viaddmax_s32((int32_t)__float_as_uint(__fmaf_rn(__uint_as_float(biased), nh.scale, nh.rest)), -(int32_t)kHeadMagic, -127);
+    }
+    return pack4_sat(v[0], v[1], v[2], v[3]);
+}
+
 // exponent of e3 given the exponent p0 of e (the head sees e at p0 - 7 after the multiplication by gamma's grid)
 __device__ __forceinline__ void next_head_exponent(const NextHead &nh, int p0, int32_t *e3_exp, DeviceState *dev)
 {
