@@ -376,7 +376,8 @@ cudaError_t launch_igemm(const IgemmParams &p, const CUtensorMap &map_a, const C
     const size_t smem = igemm_smem_bytes(p);
     const auto kernel = p.split > 1 ? (p.epilogue == kEpiForward ? igemm_kernel<kEpiForward, true> : igemm_kernel<kEpiDgrad, true>)
                                     : (p.epilogue == kEpiForward ? igemm_kernel<kEpiForward, false> : igemm_kernel<kEpiDgrad, false>);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    static std::atomic<unsigned long long> allowed[2][2];
+    const cudaError_t e = allow_smem((const void *)kernel, 226 * 1024, allowed[p.split > 1][p.epilogue == kEpiForward]);
     if (e != cudaSuccess) return e;
     return launch_chained_clusters(p.split, kernel, grid, kGemmThreads, smem, stream, p, map_a, map_b);
 }

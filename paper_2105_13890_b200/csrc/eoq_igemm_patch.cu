@@ -377,7 +377,8 @@ cudaError_t launch_igemm_patch(const IgemmParams &p, const PatchPlan &pl, const 
                                const CUtensorMap &map_b, int grid, cudaStream_t stream)
 {
     const auto kernel = p.epilogue == kEpiForward ? igemm_patch_kernel<kEpiForward> : igemm_patch_kernel<kEpiDgrad>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    static std::atomic<unsigned long long> allowed[2];
+    const cudaError_t e = allow_smem((const void *)kernel, 226 * 1024, allowed[p.epilogue == kEpiForward]);
     if (e != cudaSuccess) return e;
     return launch_chained(kernel, grid, kPatchThreads, igemm_patch_smem_bytes(p, pl), stream, p, pl, map_a, map_b);
 }

@@ -1,5 +1,6 @@
 // Internal declarations shared by the translation units of libeoq (not part of the public ABI).
 #pragma once
+#include <atomic>
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -16,6 +17,20 @@ constexpr int kWgradThreads = 256;  // weight gradient: warps 0, 2, 3 TMA, warp 
 constexpr uint32_t kSpinLimit = 1u << 22;  // polls before a wait gives up (normal waits end within microseconds)
 
 // Device state a handle owns.
+// Lets a kernel have `bytes` of dynamic shared memory; asked once per kernel and device (`done`: a bit per device), since the
+// runtime call costs as much host time as a quarter of a launch.
+inline cudaError_t allow_smem(const void *kernel, int bytes, std::atomic<unsigned long long> &done)
+{
+    int device = 0;
+    const cudaError_t got = cudaGetDevice(&device);
+    if (got != cudaSuccess) return got;
+    const unsigned long long bit = device < 64 ? 1ull << device : 0ull;
+    if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
+
 // Launches a kernel that may be brought up while its predecessor on the stream still runs (programmatic dependent launch):
 // the predecessor allows it with ptx::grid_dep_launch (or by ending), and the kernel calls ptx::grid_dep_wait before it
 // touches global memory, in every block.  Launch latency and prologue, about 1.5 us per kernel in a captured chain, then

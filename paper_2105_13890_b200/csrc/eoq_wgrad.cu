@@ -244,7 +244,8 @@ size_t wgrad_smem_bytes(const WgradParams &p)
 
 cudaError_t launch_wgrad(const WgradParams &p, const CUtensorMap &map_x, const CUtensorMap &map_e, cudaStream_t stream)
 {
-    cudaError_t e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024);
+    static std::atomic<unsigned long long> allowed;
+    const cudaError_t e = allow_smem((const void *)wgrad_kernel, 208 * 1024, allowed);
     if (e != cudaSuccess) return e;
     const int grid = p.num_m_groups * p.num_n_tiles * p.num_k_splits;
     return launch_chained(wgrad_kernel, grid, kWgradThreads, wgrad_smem_bytes(p), stream, p, map_x, map_e);

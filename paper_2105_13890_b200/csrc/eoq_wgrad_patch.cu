@@ -211,7 +211,8 @@ size_t wgrad_patch_smem_bytes(const WgradPatchPlan &pl)
 cudaError_t launch_wgrad_patch(const WgradPatchPlan &pl, const CUtensorMap &map_x, const CUtensorMap &map_e,
                                cudaStream_t stream)
 {
-    cudaError_t e = cudaFuncSetAttribute(wgrad_patch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024);
+    static std::atomic<unsigned long long> allowed;
+    const cudaError_t e = allow_smem((const void *)wgrad_patch_kernel, 208 * 1024, allowed);
     if (e != cudaSuccess) return e;
     return launch_chained(wgrad_patch_kernel, pl.num_groups * pl.num_splits, kWgradPatchThreads, wgrad_patch_smem_bytes(pl), stream, pl, map_x,
                                                                                                                  map_e);

@@ -1,4 +1,5 @@
-"""Thin ctypes binding over libeoq.so (the C ABI declared in include/eoq.h).
+"""Thin binding over libeoq.so (the C ABI declared in include/eoq.h): ctypes, and a native module (csrc/eoq_bind.c) for the
+entry points that a program calls for every layer and step.
 
 Each function has the name and argument order of its C counterpart and only
 marshals arguments: torch tensors (device memory owned by the caller) become raw
@@ -14,6 +15,7 @@ from typing import Optional, Sequence
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libeoq.so")
+BIND_PATH = os.path.join(_HERE, "_eoqbind.so")
 
 EOQ_OK, EOQ_ERR_BAD_ARG, EOQ_ERR_ALIGNMENT, EOQ_ERR_UNSUPPORTED, EOQ_ERR_WORKSPACE, EOQ_ERR_RANGE, EOQ_ERR_CUDA = range(7)
 EOQ_DEV_TIMEOUT, EOQ_DEV_NONFINITE, EOQ_DEV_SQ_ZERO, EOQ_DEV_RANGE = 1, 2, 4, 8
@@ -139,6 +141,22 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_native = None
+
+
+def native():
+    """Loads the native module for the entry points called per layer and step; raises if it has not been built."""
+    global _native
+    if _native is None:
+        lib()   # the module links against the same library
+        if not os.path.exists(BIND_PATH):
+            raise RuntimeError(f"{BIND_PATH} is missing: build it with `python -m paper_2105_13890_b200.build`")
+        from . import _eoqbind
+
+        _native = _eoqbind
+    return _native
+
+
 def status_string(status: int) -> str:
     return lib().eoq_status_string(int(status)).decode()
 
@@ -155,9 +173,20 @@ def _ptr(t) -> Optional[int]:
 def _stream(stream) -> Optional[int]:
     if stream is not None:
         return stream if isinstance(stream, int) else stream.cuda_stream
+    return _current_stream()
+
+
+def _current_stream() -> int:
+    """The current stream of torch's current device.  The first call sets torch up and puts its two getters in place of the
+    stream object that torch.cuda.current_stream() builds each time (2 us)."""
+    global _current_stream
     import torch
 
-    return torch.cuda.current_stream().cuda_stream
+    value = torch.cuda.current_stream().cuda_stream
+    get_stream, get_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+    _current_stream = lambda: get_stream(get_device())  # noqa: E731
+    return value
 
 
 def _nbytes(t) -> int:
@@ -199,8 +228,7 @@ def eoq_conv_fwd(handle, desc, x, x_exp, b1_c, w, gamma_c, b2_c, shortcut, relu,
 
 def eoq_conv_dgrad(handle, desc, e3, e3_exp, w, e4, e4_exp, sum_e4=None, acc_dump=None, workspace=None, stream=None,
                    check: bool = True) -> int:
-    st = lib().eoq_conv_dgrad(handle, C.byref(desc), _ptr(e3), _ptr(e3_exp), _ptr(w), _ptr(e4), _ptr(e4_exp),
-                              _ptr(sum_e4), _ptr(acc_dump), _ptr(workspace), _nbytes(workspace), _stream(stream))
+    st = (_native or native()).conv_dgrad(handle, desc, e3, e3_exp, w, e4, e4_exp, sum_e4, acc_dump, workspace, _stream(stream))
     if check:
         _check(st, "eoq_conv_dgrad")
     return st
@@ -217,8 +245,7 @@ def eoq_conv_wgrad(handle, desc, e3, e3_exp, x, b1_c, g, g_exp, acc_dump=None, w
 
 def eoq_quantize(handle, mode, src, src_is_float, src_exp, n, dst, dst_exp=None, workspace=None, stream=None,
                  check: bool = True) -> int:
-    st = lib().eoq_quantize(handle, int(mode), _ptr(src), 1 if src_is_float else 0, _ptr(src_exp), int(n), _ptr(dst),
-                            _ptr(dst_exp), _ptr(workspace), _nbytes(workspace), _stream(stream))
+    st = (_native or native()).quantize(handle, mode, src, 1 if src_is_float else 0, src_exp, n, dst, dst_exp, workspace, _stream(stream))
     if check:
         _check(st, "eoq_quantize")
     return st
@@ -305,8 +332,8 @@ def eoq_conv_dgrad_static(desc, e3, e3_exp, w, e4, e4_exp, sum_e4=None, status_o
 def eoq_conv_fwd_dev(handle, desc, x, x_exp, scalars, w, w_prep, shortcut, relu, x5, x2=None, relu_mask=None, stream=None,
                      check: bool = True) -> int:
     """eoq_conv_fwd with the scalars {b1_c, gamma_c, b2_c} in device memory and prepared weights (eoq_weight_prep)."""
-    st = lib().eoq_conv_fwd_dev(handle, C.byref(desc), _ptr(x), _ptr(x_exp), _ptr(scalars), _ptr(w), _ptr(w_prep),
-                                _ptr(shortcut), 1 if relu else 0, _ptr(x5), _ptr(x2), _ptr(relu_mask), _stream(stream))
+    st = (_native or native()).conv_fwd_dev(handle, desc, x, x_exp, scalars, w, w_prep, shortcut, 1 if relu else 0, x5, x2, relu_mask,
+                                            _stream(stream))
     if check:
         _check(st, "eoq_conv_fwd_dev")
     return st
@@ -320,11 +347,7 @@ def eoq_weight_prep_size(desc: eoq_conv_desc_t) -> int:
 
 def eoq_weight_prep(handle, descs: Sequence[eoq_conv_desc_t], w: Sequence, prep: Sequence, stream=None,
                     check: bool = True) -> int:
-    num = len(descs)
-    darr = (eoq_conv_desc_t * num)(*descs)
-    arr = C.c_void_p * num
-    st = lib().eoq_weight_prep(handle, num, darr, arr(*[_ptr(t) for t in w]), arr(*[_ptr(t) for t in prep]),
-                               _stream(stream))
+    st = (_native or native()).weight_prep(handle, descs, w, prep, _stream(stream))
     if check:
         _check(st, "eoq_weight_prep")
     return st
@@ -350,8 +373,7 @@ def eoq_wgrad_finish(handle, descs: Sequence[eoq_conv_desc_t], e3: Sequence, e3_
 
 
 def eoq_conv_wgrad_dev(handle, desc, e3, e3_exp, x, b1_c, g, g_exp, workspace=None, stream=None, check: bool = True) -> int:
-    st = lib().eoq_conv_wgrad_dev(handle, C.byref(desc), _ptr(e3), _ptr(e3_exp), _ptr(x), _ptr(b1_c), _ptr(g),
-                                  _ptr(g_exp), _ptr(workspace), _nbytes(workspace), _stream(stream))
+    st = (_native or native()).conv_wgrad_dev(handle, desc, e3, e3_exp, x, b1_c, g, g_exp, workspace, _stream(stream))
     if check:
         _check(st, "eoq_conv_wgrad_dev")
     return st
@@ -359,8 +381,8 @@ def eoq_conv_wgrad_dev(handle, desc, e3, e3_exp, x, b1_c, g, g_exp, workspace=No
 
 def eoq_err_prescale_dev(handle, e0, e0_exp, relu_mask, x2, n_el, gamma_c, e3, e3_exp, sum_e1=None, sum_e1x2=None,
                          stream=None, check: bool = True) -> int:
-    st = lib().eoq_err_prescale_dev(handle, _ptr(e0), _ptr(e0_exp), _ptr(relu_mask), _ptr(x2), int(n_el), _ptr(gamma_c),
-                                    _ptr(e3), _ptr(e3_exp), _ptr(sum_e1), _ptr(sum_e1x2), _stream(stream))
+    st = (_native or native()).err_prescale_dev(handle, e0, e0_exp, relu_mask, x2, n_el, gamma_c, e3, e3_exp, sum_e1, sum_e1x2,
+                                                _stream(stream))
     if check:
         _check(st, "eoq_err_prescale_dev")
     return st
@@ -369,12 +391,7 @@ def eoq_err_prescale_dev(handle, e0, e0_exp, relu_mask, x2, n_el, gamma_c, e3, e
 def eoq_update_dev(handle, w: Sequence, g: Sequence, g_exp: Sequence, lr_mant: int, lr_exp: int, round_mode: int, seed: int,
                    step, stream=None, check: bool = True) -> int:
     """eoq_update with the step counter in device memory (a one-element int64/uint64 tensor, bumped by the call)."""
-    num = len(w)
-    arr = C.c_void_p * num
-    sizes = (C.c_size_t * num)(*[t.numel() for t in w])
-    st = lib().eoq_update_dev(handle, num, arr(*[_ptr(t) for t in w]), arr(*[_ptr(t) for t in g]),
-                              arr(*[_ptr(t) for t in g_exp]), sizes, int(lr_mant), int(lr_exp), int(round_mode), int(seed),
-                              _ptr(step), _stream(stream))
+    st = (_native or native()).update_dev(handle, w, g, g_exp, lr_mant, lr_exp, round_mode, seed, step, _stream(stream))
     if check:
         _check(st, "eoq_update_dev")
     return st
