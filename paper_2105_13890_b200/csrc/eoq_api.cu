@@ -410,7 +410,10 @@ bool plan_wgrad_patch(WgradPatchPlan &pl, const eoq_conv_desc_t &d, int ho, int 
     pl.row_groups = (d.kh + rpg - 1) / rpg;
     pl.num_groups = pl.n_tiles * pl.chunks * pl.row_groups;
     pl.rows_total = d.kh * d.kw * d.c_in;
-    // rows per pixel block: as many as keep one stage near 64 KB (three stages in flight)
+    // Rows per pixel block: as many as keep one stage near 64 KB (three stages in flight).  Layers of one 32-channel chunk take
+    // half: the error back-propagation of such layers leaves the other half of an SM's shared memory, and the two then share
+    // SMs (ResNet-20 step at batch 128: 659 -> 647 us; wider layers fill the SM anyway and only load more halo rows).
+    const int smem_kb = pl.kc <= 32 && pl.tile_n <= 32 ? 100 : 200;
     int r = ho < 32 ? ho : 32;
     for (; r >= 1; --r) {
         const int kp = (r * pl.pw + 31) / 32 * 32;
@@ -420,14 +423,14 @@ bool plan_wgrad_patch(WgradPatchPlan &pl, const eoq_conv_desc_t &d, int ho, int 
         pl.x_bytes = (x_rows * pl.kc + 1023) / 1024 * 1024;
         pl.e_bytes = (kp * pl.tile_n + 1023) / 1024 * 1024;
         pl.kp = kp;
-        if (pl.x_bytes + pl.e_bytes <= 66 * 1024) break;
+        if (pl.x_bytes + pl.e_bytes <= smem_kb / 3 * 1024) break;
     }
     if (r < 1) return false;
     pl.r_rows = r;
     pl.blocks_per_img = (ho + r - 1) / r;
     pl.x_box_bytes = pl.kc * pl.pw * (r + d.kh - 1);
     pl.e_box_bytes = pl.tile_n * pl.pw * r;
-    int stages = (200 * 1024) / (pl.x_bytes + pl.e_bytes);
+    int stages = (smem_kb * 1024) / (pl.x_bytes + pl.e_bytes);
     pl.num_stages = stages > 4 ? 4 : stages;
     if (pl.num_stages < 2) return false;
     const int total_blocks = d.n * pl.blocks_per_img;

@@ -47,6 +47,23 @@ __device__ __forceinline__ uint32_t rne7_magic(uint32_t biased)
     return __float_as_uint(__fmaf_rn(__uint_as_float(biased), 0.0078125f, kMagicRest));
 }
 
+// R(x / 2^7) for an integer x in [0, 2^22) without a bias: x read as a float is the denormal x 2^-149, and one fused
+// multiply-add forms x 2^-22 + 1.5 * 2^8, whose unit of rounding is 2^-15.  Returns kDenormalBits + R(x / 2^7).
+constexpr uint32_t kDenormalBits = 0x43C00000u;   // 1.5 * 2^8 as a float
+__device__ __forceinline__ uint32_t rne7_denormal(uint32_t x)
+{
+    return __float_as_uint(__fmaf_rn(__uint_as_float(x), __int_as_float((127 + 127) << 23), __uint_as_float(kDenormalBits)));
+}
+
+// sum of the products of four signed bytes with four unsigned ones, plus c: with one byte of b set to 128 it scales and adds
+// one code without the byte extraction, which would go to the busier pipe
+__device__ __forceinline__ uint32_t dot4_s8_u8(uint32_t a, uint32_t b, uint32_t c)
+{
+    uint32_t d;
+    asm("dp4a.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
 // Forward chain on 16 consecutive output channels of one pixel (Sec. 3.2.1: x2 = Q_a1(conv), x3 = gamma x2,
 // x4 = x3 + b2 [+ shortcut], x5 = Q_a2(relu(x4)); mask = [x4 > 0]).
 // The integer pipe bounds this code (an instruction every two cycles and scheduler), so clamps are moved in front of the
@@ -205,15 +222,11 @@ __device__ __forceinline__ void forward_16(const IgemmParams &p, const FwdScalar
     const uint32_t base = ((uint32_t)fs.b2 << 7) - g * kMagicBits - 1u;
     uint32_t add[16];
     if (p.shortcut) {
-        const int4 v = sc;
-        const uint32_t w[4] = {(uint32_t)v.x, (uint32_t)v.y, (uint32_t)v.z, (uint32_t)v.w};
+        const uint32_t w[4] = {(uint32_t)sc.x, (uint32_t)sc.y, (uint32_t)sc.z, (uint32_t)sc.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            add[4 * i + 0] = base + (uint32_t)sbyte<0>(w[i]) * 128u;
-            add[4 * i + 1] = base + (uint32_t)sbyte<1>(w[i]) * 128u;
-            add[4 * i + 2] = base + (uint32_t)sbyte<2>(w[i]) * 128u;
-            add[4 * i + 3] = base + (uint32_t)sbyte<3>(w[i]) * 128u;
-        }
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) add[4 * i + k] = dot4_s8_u8(w[i], 128u << (8 * k), base);
     } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) add[i] = base;
@@ -226,14 +239,21 @@ __device__ __forceinline__ void forward_16(const IgemmParams &p, const FwdScalar
     for (int i = 15; i >= 0; --i) {
         const int32_t w = (int32_t)(g * q[i] + add[i]);  // x4 - 1
         nbits = __funnelshift_l((uint32_t)w, nbits, 1);
-        if (kRelu) r[i] = rne7_magic((uint32_t)__viaddmin_s32_relu(w, 1, 16319) | kMagicBits);
+        if (kRelu) r[i] = rne7_denormal((uint32_t)__viaddmin_s32_relu(w, 1, 16319));
         else r[i] = rne7_magic((uint32_t)max(__viaddmin_s32(w, 1, 16319), -16319) + kMagicBits);
     }
     int4 o;
-    o.x = (int)__byte_perm(__byte_perm(r[0], r[1], 0x0040), __byte_perm(r[2], r[3], 0x0040), 0x5410);
-    o.y = (int)__byte_perm(__byte_perm(r[4], r[5], 0x0040), __byte_perm(r[6], r[7], 0x0040), 0x5410);
-    o.z = (int)__byte_perm(__byte_perm(r[8], r[9], 0x0040), __byte_perm(r[10], r[11], 0x0040), 0x5410);
-    o.w = (int)__byte_perm(__byte_perm(r[12], r[13], 0x0040), __byte_perm(r[14], r[15], 0x0040), 0x5410);
+    if (kRelu) {
+        // codes 0 to 127 above a constant: shifted and added on the multiply-add pipe, the constants taken off at the end
+        constexpr uint32_t kRest = kDenormalBits * 0x01010101u;
+        auto pack = [&](int i) { return (int)(((r[i + 3] * 256u + r[i + 2]) * 256u + r[i + 1]) * 256u + r[i] - kRest); };
+        o = make_int4(pack(0), pack(4), pack(8), pack(12));
+    } else {
+        o.x = (int)__byte_perm(__byte_perm(r[0], r[1], 0x0040), __byte_perm(r[2], r[3], 0x0040), 0x5410);
+        o.y = (int)__byte_perm(__byte_perm(r[4], r[5], 0x0040), __byte_perm(r[6], r[7], 0x0040), 0x5410);
+        o.z = (int)__byte_perm(__byte_perm(r[8], r[9], 0x0040), __byte_perm(r[10], r[11], 0x0040), 0x5410);
+        o.w = (int)__byte_perm(__byte_perm(r[12], r[13], 0x0040), __byte_perm(r[14], r[15], 0x0040), 0x5410);
+    }
     *reinterpret_cast<int4 *>(p.x5 + off) = o;
     if (p.relu_mask) *reinterpret_cast<uint16_t *>(p.relu_mask + (off >> 3)) = (uint16_t)~nbits;
     if (p.x2) {
