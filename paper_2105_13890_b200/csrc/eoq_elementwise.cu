@@ -652,7 +652,7 @@ prescale_fused_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, cons
                       int32_t *e3_exp, long long *sum_e1, long long *sum_e1x2, DeviceState *dev, unsigned expected_blocks,
                       uint32_t spin_limit)
 {
-    ptx::grid_dep_wait_launch_small();
+    if (gridDim.x <= 148) ptx::grid_dep_launch();   // (its successor may come up beside it)
     __shared__ unsigned go_s;
     gamma_c = load_gamma(gamma_c, gamma_dev, dev);
     const size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -1004,9 +1004,12 @@ cudaError_t launch_err_prescale(const int8_t *e0, const int32_t *e0_exp, const u
         // self-test of the bounded wait: one arrival more than there are blocks and a short limit
         unsigned expected = (unsigned)need_blocks + (force_timeout ? 1u : 0u);
         uint32_t spin_limit = force_timeout ? 2048u : kSpinLimit;
-        const cudaError_t e = launch_chained_cooperative(prescale_fused_kernel, dim3((unsigned)need_blocks), dim3(kThreads), s, e0, e0_exp,
-                                                         mask, x2, n16, gamma_c, gamma_dev, e3, e3_exp, sum_e1, sum_e1x2, dev, expected,
-                                                         spin_limit);
+        void *args[] = {(void *)&e0, (void *)&e0_exp, (void *)&mask, (void *)&x2, (void *)&n16, (void *)&gamma_c,
+                        (void *)&gamma_dev, (void *)&e3, (void *)&e3_exp, (void *)&sum_e1, (void *)&sum_e1x2, (void *)&dev,
+                        (void *)&expected, (void *)&spin_limit};
+        // (not a chained launch: together with the cooperative attribute that takes about 2 us more than it saves)
+        const cudaError_t e = cudaLaunchCooperativeKernel((const void *)prescale_fused_kernel, dim3((unsigned)need_blocks),
+                                                          dim3(kThreads), args, 0, s);
         if (e != cudaErrorCooperativeLaunchTooLarge) {
             *kernels = 1;
             return e;

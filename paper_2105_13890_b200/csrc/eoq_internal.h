@@ -54,23 +54,6 @@ inline cudaError_t launch_chained_clusters(int cluster, void (*kernel)(P...), di
     cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
 }
-// all blocks resident at once (kernels with a barrier over the grid)
-template <typename... P, typename... A>
-inline cudaError_t launch_chained_cooperative(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A &&...args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2] = {};
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeCooperative;
-    attr[1].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
-}
 template <typename... P, typename... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A &&...args)
 {
