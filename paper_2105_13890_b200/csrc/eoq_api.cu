@@ -1101,6 +1101,13 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     int32_t *sums = acc_dump ? acc_dump : reinterpret_cast<int32_t *>(reinterpret_cast<char *>(workspace) + round256(g.w_elems));
     cudaError_t e;
 
+    // sums that the kernels behind the GEMM add into; it clears them (one the caller also names for the join or the head is
+    // written there: the later value counts)
+    if (sum_e4 && jc && (void *)sum_e4 == (void *)jc->sum_out) sum_e4 = nullptr;
+    const NextHeadArgs *const any_next = jc ? jc->next : next;
+    long long *const zero_sums[4] = {reinterpret_cast<long long *>(sum_e4), jc ? jc->sum_out : nullptr, any_next ? any_next->sum_e1 : nullptr,
+                                     any_next ? any_next->sum_e1x2 : nullptr};
+
     // One GEMM per residue class (y mod stride, x mod stride) of the input pixels: within a class the taps
     // kh with (y + pad - kh) divisible by the stride form a unit-stride correlation over e3.
     if (d.stride == 1 && d.kh == d.kw && d.kh - 1 - d.pad >= 0) {
@@ -1117,6 +1124,7 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.out_w = d.w;
             p.out_step = 1;
             p.epilogue = kEpiDgrad;
+            memcpy(p.zero_sums, zero_sums, sizeof(zero_sums));
             p.acc_out = sums;
             p.dev = h->dev;
             p.next_mask = next ? next->mask : nullptr;
@@ -1246,6 +1254,7 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.out_off_h = py;
             p.out_off_w = px;
             p.epilogue = kEpiDgrad;
+            memcpy(p.zero_sums, zero_sums, sizeof(zero_sums));
             p.acc_out = sums;
             p.dev = h->dev;
             p.next_mask = next ? next->mask : nullptr;
@@ -1298,6 +1307,9 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     delete group;  // closes the group's bracket on `s`, behind the joins
     group = nullptr;
     if (h->gemm_only) return EOQ_OK;
+    if (class_no == 0)   // no tap reaches any pixel: no GEMM ran
+        for (long long *z : zero_sums)
+            if (z && (e = cudaMemsetAsync(z, 0, sizeof(*z), s)) != cudaSuccess) return record(h, e);
     // Q_e over the whole tensor: the maximum is complete only now
     {
         ProfScope prof(h, EOQ_PROF_DGRAD_AUX, s);

@@ -32,18 +32,41 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
                             int8_t *__restrict__ e3, int32_t *e3_exp, long long *sum_e1, long long *sum_e1x2, DeviceState *dev)
 {
     ptx::grid_dep_wait_launch_small();
+    const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (kPass == 1 && first < n16) {   // on their way while the maxima are read
+        ptx::prefetch_l1(a + first * 16);
+        ptx::prefetch_l1(b + first * 16);
+        if (mask_b) ptx::prefetch_l1(mask_b + first * 2);
+        if (kNext) {
+            ptx::prefetch_l1(next_mask + first * 2);
+            if (next_x2) ptx::prefetch_l1(next_x2 + first * 16);
+        }
+    }
     const JoinShift j = join_shift(__ldg(a_exp), __ldg(b_exp));
     unsigned long long mx = 0, mxm = 0;
     long long sum = 0, s1 = 0, s2 = 0;
     int t = 7;
     NextHead nh = {};
     unsigned long long M = 0;
+    bool last = false;
+    if (kPass == 0 && blockIdx.x == 0 && threadIdx.x == 0) {   // the second pass adds to the sums where the caller wants them
+        if (sum_out) *sum_out = 0;
+        if (kNext && sum_e1) *sum_e1 = 0;
+        if (kNext && sum_e1x2) *sum_e1x2 = 0;
+    }
     if (kPass == 1) {
-        M = dev->absmax_u64;
+        __shared__ unsigned long long cell_s[2];   // (the protocol of sq_i32_kernel)
+        if (threadIdx.x == 0) {
+            cell_s[0] = *(volatile unsigned long long *)&dev->absmax_u64;
+            cell_s[1] = *(volatile unsigned long long *)&dev->absmax2_u64;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) last = last_reader(dev);
+        M = cell_s[0];
         t = M ? round_log2_u64(M) : 7;
         const int p0 = M ? j.p + t - 7 : j.p;
         if (kNext) {
-            const unsigned long long Mm = dev->absmax2_u64;
+            const unsigned long long Mm = cell_s[1];
             nh = next_head_setup(next_gamma, (uint32_t)abs(sq_code64((long long)Mm, t)), dev);
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -135,21 +158,16 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
         long long v[3] = {sum, s1, s2};
         block_sums_i64(v);
         if (threadIdx.x == 0) {
-            if (sum_out && v[0]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)v[0]);
-            if (kNext && v[1]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum1), (unsigned long long)v[1]);
-            if (kNext && v[2]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum2), (unsigned long long)v[2]);
-        }
-        if (last_block_done(dev)) {
-            if (sum_out) *sum_out = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum0), 0ull);
-            dev->absmax_u64 = 0;
+            auto add = [](long long *dst, long long x) {
+                if (dst && x) atomicAdd(reinterpret_cast<unsigned long long *>(dst), (unsigned long long)x);
+            };
+            add(sum_out, v[0]);
             if (kNext) {
-                dev->absmax2_u64 = 0;
-                const long long t1 = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum1), 0ull);
-                const long long t2 = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum2), 0ull);
-                if (sum_e1) *sum_e1 = t1;
-                if (sum_e1x2) *sum_e1x2 = t2;
+                add(sum_e1, v[1]);
+                add(sum_e1x2, v[2]);
             }
         }
+        if (last) dev->absmax_u64 = dev->absmax2_u64 = 0;
     }
 }
 

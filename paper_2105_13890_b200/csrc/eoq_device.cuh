@@ -237,6 +237,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)_
 // wait; the next kernel may be brought up once every block has called grid_dep_launch or ended.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A line that the thread will read behind a barrier: its latency runs beside that of the values the barrier waits for.
+__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
 // Thread-block clusters: a barrier over all their threads (the writes in front of it, to shared memory of any of the blocks,
 // are visible behind it), the address of a shared-memory location in another block, and a 16-byte store there.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }

@@ -313,20 +313,62 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
                               DeviceState *dev)
 {
     ptx::grid_dep_wait_launch_small();
-    const uint32_t M = dev->absmax_u32;
+    // The maxima go through one thread per block and shared memory; that thread counts the block as a reader, and the last
+    // one puts the cells back to zero at its end.  The sums are added to where the caller wants them (cleared by the kernel
+    // in front): with a ticket, a fence and the publication of the sums by the last block, these kernels took about 2 us more
+    // on the few hundred KB of a small batch.
+    __shared__ uint32_t cell_s[2];
+    const size_t n16 = n / 16;
+    const bool wide_in = (reinterpret_cast<uintptr_t>(src) & 31) == 0;
+    auto load16 = [&](size_t i, int (&a)[16]) {
+        if (wide_in) {   // two 256-bit loads: whole 32-byte sectors per lane
+            ld_global_256_stream(src + i * 16, a);
+            ld_global_256_stream(src + i * 16 + 8, a + 8);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int4 v = __ldcs(reinterpret_cast<const int4 *>(src) + i * 4 + k);
+                a[4 * k + 0] = v.x;
+                a[4 * k + 1] = v.y;
+                a[4 * k + 2] = v.z;
+                a[4 * k + 3] = v.w;
+            }
+        }
+    };
+    // the first group of every thread is on its way while the maxima are read
+    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int a[16];
+    if (i < n16) {
+        load16(i, a);
+        if (kJoin) {
+            ptx::prefetch_l1(join.b + i * 16);
+            if (join.mask_b) ptx::prefetch_l1(join.mask_b + i * 2);
+            if (join.next_mask) ptx::prefetch_l1(join.next_mask + i * 2);
+        }
+        if (kNext) {
+            ptx::prefetch_l1(next.mask + i * 2);
+            if (next.x2) ptx::prefetch_l1(next.x2 + i * 16);
+        }
+    }
+    bool last = false;
+    if (threadIdx.x == 0) {
+        cell_s[0] = *(volatile unsigned *)&dev->absmax_u32;
+        if (kNext) cell_s[1] = (uint32_t)*(volatile unsigned long long *)&dev->absmax_u64;
+    }
+    const int p_in = (src_exp ? __ldg(src_exp) : 0) + exp_bias;
+    __syncthreads();
+    if (threadIdx.x == 0) last = last_reader(dev);
+    const uint32_t M = cell_s[0];
     const int t = M ? round_log2_u32(M) : 7;
-    const int p_in = (src_exp ? *src_exp : 0) + exp_bias;
     const int p0 = M ? p_in + t - 7 : p_in;
     NextHead nh = {};
-    if (kNext) nh = next_head_setup(next.gamma, (uint32_t)abs(sq_code32((int32_t)dev->absmax_u64, t)), dev);
+    if (kNext) nh = next_head_setup(next.gamma, (uint32_t)abs(sq_code32((int32_t)cell_s[1], t)), dev);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *dst_exp = p0;
         if (!M) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
         if (kNext) next_head_exponent(nh, p0, next.e3_exp, dev);
     }
     long long sum = 0, s1 = 0, s2 = 0;
-    const size_t n16 = n / 16;
-    const int4 *s4 = reinterpret_cast<const int4 *>(src);
     const int sh = t - 7;
     JoinShift js = {0, 0, 0};
     bool j_narrow = true;
@@ -342,23 +384,8 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
     const bool fast = sh >= 1 && M < 0x7e000000u;
     const int32_t half_m1 = fast ? (1 << (sh - 1)) - 1 : 0, lo = fast ? -(127 << sh) : 0;
     uint32_t jm32 = 0, jmm32 = 0;
-    const bool wide_in = (reinterpret_cast<uintptr_t>(src) & 31) == 0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
-        int a[16];
+    while (i < n16) {
         uint32_t cw[4];   // four codes per word
-        if (wide_in) {   // two 256-bit loads: whole 32-byte sectors per lane
-            ld_global_256_stream(src + i * 16, a);
-            ld_global_256_stream(src + i * 16 + 8, a + 8);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int4 v = __ldcs(s4 + i * 4 + k);
-                a[4 * k + 0] = v.x;
-                a[4 * k + 1] = v.y;
-                a[4 * k + 2] = v.z;
-                a[4 * k + 3] = v.w;
-            }
-        }
         int sum16 = 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -407,6 +434,8 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
             if (next.x2) s2 += dot16_s8_s16(e1, reinterpret_cast<const int4 *>(next.x2) + 2 * i);
             reinterpret_cast<int4 *>(next.e3)[i] = make_int4((int)c3[0], (int)c3[1], (int)c3[2], (int)c3[3]);
         }
+        i += (size_t)gridDim.x * blockDim.x;
+        if (i < n16) load16(i, a);
     }
     ptx::grid_dep_launch();
     if (!kNext && !kJoin)
@@ -424,9 +453,14 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
         }
         if (kNext || sum_codes) block_sums_i64(v);
         if (threadIdx.x == 0) {
-            if (sum_codes && v[0]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)v[0]);
-            if (kNext && v[kNext ? 1 : 0]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum1), (unsigned long long)v[kNext ? 1 : 0]);
-            if (kNext && v[kNext ? 2 : 0]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum2), (unsigned long long)v[kNext ? 2 : 0]);
+            auto add = [](long long *dst, long long x) {
+                if (dst && x) atomicAdd(reinterpret_cast<unsigned long long *>(dst), (unsigned long long)x);
+            };
+            add(sum_codes, v[0]);
+            if (kNext) {
+                add(next.sum_e1, v[kNext ? 1 : 0]);
+                add(next.sum_e1x2, v[kNext ? 2 : 0]);
+            }
         }
     }
     if (kJoin) {
@@ -438,16 +472,9 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
             if (jmxm) atomicMax(&dev->absmax2_u64, jmxm);
         }
     }
-    if (last_block_done(dev)) {
-        if (sum_codes) *sum_codes = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum0), 0ull);
+    if (last) {
         dev->absmax_u32 = 0;
-        if (kNext) {
-            dev->absmax_u64 = 0;
-            const long long t1 = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum1), 0ull);
-            const long long t2 = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum2), 0ull);
-            if (next.sum_e1) *next.sum_e1 = t1;
-            if (next.sum_e1x2) *next.sum_e1x2 = t2;
-        }
+        if (kNext) dev->absmax_u64 = 0;
     }
 }
 
@@ -460,7 +487,12 @@ __global__ void sq_i32_scatter_kernel(const int32_t *__restrict__ src, const int
                                       long long *sum_codes, DeviceState *dev)
 {
     ptx::grid_dep_wait_launch_small();
-    const uint32_t M = dev->absmax_u32;
+    __shared__ uint32_t cell_s;   // (the protocol of sq_i32_kernel)
+    bool last = false;
+    if (threadIdx.x == 0) cell_s = *(volatile unsigned *)&dev->absmax_u32;
+    __syncthreads();
+    if (threadIdx.x == 0) last = last_reader(dev);
+    const uint32_t M = cell_s;
     const int t = M ? round_log2_u32(M) : 7;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const int p_in = (src_exp ? *src_exp : 0) + exp_bias;
@@ -497,13 +529,11 @@ __global__ void sq_i32_scatter_kernel(const int32_t *__restrict__ src, const int
         reinterpret_cast<int4 *>(dst)[i] = out;
     }
     if (sum_codes) {
-        sum = block_sum_i64(sum);
-        if (threadIdx.x == 0 && sum) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)sum);
+        long long v[1] = {sum};
+        block_sums_i64(v);
+        if (threadIdx.x == 0 && v[0]) atomicAdd(reinterpret_cast<unsigned long long *>(sum_codes), (unsigned long long)v[0]);
     }
-    if (last_block_done(dev)) {
-        if (sum_codes) *sum_codes = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum0), 0ull);
-        dev->absmax_u32 = 0;
-    }
+    if (last) dev->absmax_u32 = 0;
 }
 
 // ------------------------------------------------------------------ head of the error chain

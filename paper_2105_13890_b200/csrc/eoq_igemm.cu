@@ -76,6 +76,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     ptx::tc_fence_after();
     if (kSplit) ptx::cluster_wait();
     ptx::grid_dep_wait();   // everything up to here touched no global memory
+    if (kEpi == kEpiDgrad && blockIdx.x == 0 && threadIdx.x < 4 && p.zero_sums[threadIdx.x]) *p.zero_sums[threadIdx.x] = 0;
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, p.dev};
 

@@ -66,13 +66,12 @@ struct DeviceState {
     unsigned long long absmax_u64;
     long long sum0, sum1;  // reduction cells for integer sums
     unsigned long long absmax2_u64;  // second maximum of a call that also serves its consumer's error head (masked |.|)
-    long long sum2;                  // third sum of such a call
     unsigned tensor_absmax[256];  // per-tensor maxima of the multi-tensor update (zero between calls)
     unsigned ticket;       // blocks of the kernel that consumes the cells last count themselves here (see last_block_done)
     unsigned arrivals;     // grid-wide barrier of the one-kernel error head (cooperative launch)
     unsigned long long probe_cycles;  // eoq_probe_mma_i8: longest issue loop of the last launch, in SM clock cycles
 };
-// Invariant: absmax_u32, absmax_u64, absmax2_u64, sum0, sum1, sum2, ticket and arrivals are zero whenever no call is in flight on the handle.
+// Invariant: absmax_u32, absmax_u64, absmax2_u64, sum0, sum1, ticket and arrivals are zero whenever no call is in flight on the handle.
 // The kernel that reads a call's reductions last puts the cells it used back to zero (its last block does), so
 // no call starts with a memset.  A kernel that gave up on a wait (EOQ_DEV_TIMEOUT) may leave them dirty:
 // eoq_last_status clears them again when it reports that bit.
@@ -196,6 +195,7 @@ struct IgemmParams {
     // kEpilogueWarps / ep_groups warps (see plan_epilogue)
     int ep_groups;
     int a_rows;   // pixels of an activation load: 128, or less when the whole problem has fewer
+    long long *zero_sums[4];   // sums that the kernels behind this one add into: cleared here (null entries are skipped)
     int split;    // CTAs (a cluster) that share a tile's reduction and its columns in the epilogue; 1: one CTA per tile
 };
 

@@ -205,3 +205,25 @@ def test_reduction_shared_by_a_cluster(d, b1):
         assert np.array_equal(G.unpack_mask(mask, sc.shape), ref["mask"])
         assert np.array_equal(G.host(e4).astype(np.int32), want) and pe.item() == p
         assert G.status_clear() == 0
+
+
+@pytest.mark.parametrize("d", [
+    oracle.ConvDesc(2, 1, 1, 32, 32, 1, 1, 2, 1),      # no tap reaches a pixel: every error is zero, and no GEMM runs
+    oracle.ConvDesc(1, 4, 3, 32, 32, 3, 3, 1, 1),      # one block
+    oracle.ConvDesc(3, 37, 29, 48, 32, 3, 3, 1, 1),    # several blocks, the last one ragged
+    oracle.ConvDesc(17, 56, 56, 64, 32, 1, 1, 1, 0),   # several groups per thread
+    oracle.ConvDesc(2, 9, 11, 32, 32, 1, 1, 2, 0),     # scattered codes
+], ids=lambda d: f"n{d.n}_{d.h}x{d.w}_k{d.kh}s{d.stride}p{d.pad}")
+def test_error_sums_are_written_whole(d):
+    """The sum of the codes is formed where the caller wants it: whatever was there before, and on every call."""
+    e3, w = synth.normal_codes((d.n, d.ho, d.wo, d.c_out), 1600, 0), synth.int8_uniform((d.c_out, d.kh, d.kw, d.c_in), 1600, 1, -30, 30)
+    want, p, _ = oracle.sq_int(oracle.conv_dgrad_acc(d, e3, w), -9 - 7)
+    gd = G.gdesc(d)
+    total = torch.full((1,), 12345, dtype=torch.int64, device="cuda:0")
+    for _ in range(2):
+        e4, pe = G.zeros((d.n, d.h, d.w, d.c_in), torch.int8), G.zeros(1, torch.int32)
+        eoq.eoq_conv_dgrad(G.handle(), gd, G.dev(e3), G.dev(np.array([-9], dtype=np.int32)), G.dev(w), e4, pe, total, None,
+                           G.workspace(gd, eoq.EOQ_PASS_DGRAD))
+        assert G.status_clear() in ((0,) if want.any() else (eoq.EOQ_DEV_SQ_ZERO,))
+        assert np.array_equal(G.host(e4).astype(np.int32).reshape(-1), np.asarray(want).reshape(-1)) and pe.item() == p
+        assert total.item() == int(np.asarray(want, dtype=np.int64).sum())
