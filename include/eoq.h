@@ -289,6 +289,15 @@ EOQ_API int eoq_update(eoq_handle_t handle, int num, int8_t *const *w, const int
 EOQ_API int eoq_update_dev(eoq_handle_t handle, int num, int8_t *const *w, const int8_t *const *g,
                    const int32_t *const *g_exp, const size_t *n, int32_t lr_mant, int32_t lr_exp, int round_mode,
                    uint64_t seed, uint64_t *step, void *stream);
+/*
+ * Part of eoq_update_dev, for loops that update the weights of a stage while the backward pass of the stages in front still
+ * runs: the `num` tensors are numbers first, first + 1, ... of the whole list (what the stochastic rounding counts by;
+ * first + num <= 256), and *step is moved on only by the part with last != 0, which must come behind all others.  The parts
+ * together give the results of one eoq_update_dev on the whole list, bit for bit.
+ */
+EOQ_API int eoq_update_part(eoq_handle_t handle, int first, int last, int num, int8_t *const *w, const int8_t *const *g,
+                    const int32_t *const *g_exp, const size_t *n, int32_t lr_mant, int32_t lr_exp, int round_mode,
+                    uint64_t seed, uint64_t *step, void *stream);
 
 /*
  * The update at other widths (Sec. 3.2.3 sets the paper's 8-bit update against the 24-bit update of earlier integer

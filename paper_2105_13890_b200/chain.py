@@ -249,20 +249,33 @@ class ChainedStep:
             else:
                 wgrad_call(h, u, b1_dev, ws)
 
-        def finish(us) -> None:
-            """b1 sums, slice sums and Q_g of the units whose GEMMs have been issued: a few launches for all of them,
-            behind those GEMMs on a side stream (so that they run beside the rest of the backward chain)."""
+        def finish(us, hh, last=False) -> None:
+            """b1 sums, slice sums and Q_g of the units whose GEMMs have been issued, a few launches for all of them; then
+            their update and the preparation of the new weights."""
+            eoq.eoq_wgrad_finish(hh, [u.desc for u in us], [u.e3 for u in us], [u.e3_exp for u in us], [u.b1_dev for u in us],
+                                 [u.g for u in us], [u.g_exp for u in us], [u.wgrad_ws for u in us], [u.wgrad_parts for u in us])
+            if overlap:   # the error chain must be through with the old weights; every other part of the update with the step counter
+                torch.cuda.current_stream(self.dev).wait_stream(main)
+                if last:
+                    for side in self.sides:
+                        main.wait_stream(side)
+            us = sorted(us, key=lambda u: u.index)
+            eoq.eoq_update_part(hh, us[0].index, last, [u.w for u in us], [u.g for u in us], [u.g_exp for u in us], self.lr_mant,
+                                self.lr_exp, self.round_mode, self.seed, self.step_dev)
+            eoq.eoq_weight_prep(hh, [u.desc for u in us], [u.w for u in us], [u.prep for u in us])
+
+        def stage_done(us) -> None:
+            """A stage of the network is through: its gradients are finished and its weights updated together, behind its
+            GEMMs on a side stream, beside the backward chain of the stages in front."""
             if not self.finish_together or not us:
                 return
-            args = ([u.desc for u in us], [u.e3 for u in us], [u.e3_exp for u in us], [u.b1_dev for u in us], [u.g for u in us],
-                    [u.g_exp for u in us], [u.wgrad_ws for u in us], [u.wgrad_parts for u in us])
             if overlap:
                 for side in self.sides[1:]:
                     self.sides[0].wait_stream(side)
                 with torch.cuda.stream(self.sides[0]):
-                    eoq.eoq_wgrad_finish(self.h_sides[0], *args)
+                    finish(us, self.h_sides[0])
             else:
-                eoq.eoq_wgrad_finish(h, *args)
+                finish(us, h)
 
         e_out, e_exp = self.e_head, self.e_head_exp
         head_done = False   # the error head of this block's last unit already ran inside the join of the block behind it
@@ -272,7 +285,7 @@ class ChainedStep:
             blk = self.blocks[i]
             a, b, pr = blk.a, blk.b, blk.proj
             if stage is not None and a.layer.name.split(".")[0] != stage:
-                finish(pending)     # a stage of the network is through: its gradients are finished together
+                stage_done(pending)
                 pending = []
             stage = a.layer.name.split(".")[0]
             pending += [b, a] + ([pr] if pr else [])
@@ -304,7 +317,7 @@ class ChainedStep:
                                              blk.e_in_exp, blk.sum_join, workspace=ws)
                 head_done = False
             e_out, e_exp = blk.e_in, blk.e_in_exp
-        finish(pending)
+        stage_done(pending)
         if self.pool:
             k, s, p = self.pool
             # pool backward and the first layer's error head in one pair of kernels; the error between them (51 MB at
@@ -315,15 +328,29 @@ class ChainedStep:
         elif not head_done:
             eoq.eoq_err_prescale_dev(h, e_out, e_exp, stem.mask, None, stem.n_out, stem.scal[1:2], stem.e3, stem.e3_exp, stem.sum_e1,
                                      None)
+        it = self.items
+
+        def scalar_update(hh) -> None:
+            eoq.eoq_aux_scalar_update(hh, [i[0] for i in it], [i[1] for i in it], [i[2] for i in it], [i[3] for i in it],
+                                      [i[4] for i in it], [i[5] for i in it], [i[6] for i in it], self.lr_mant, self.lr_exp,
+                                      self.round_mode, self.seed, self.step_dev)
+
+        if self.finish_together:
+            # the first layer's weight gradient ends the chain; the scalars are updated beside it, behind the last reader of b1
+            if overlap:
+                self.sides[0].wait_stream(main)
+                with torch.cuda.stream(self.sides[0]):
+                    scalar_update(self.h_sides[0])
+            else:
+                scalar_update(h)
+            wgrad_call(h, stem, None, ws)
+            finish([stem], h, last=True)
+            return
         wgrad(stem, None)
-        finish([stem])
         if overlap:
             for side in self.sides:
                 main.wait_stream(side)
-        it = self.items
-        eoq.eoq_aux_scalar_update(h, [i[0] for i in it], [i[1] for i in it], [i[2] for i in it], [i[3] for i in it],
-                                  [i[4] for i in it], [i[5] for i in it], [i[6] for i in it], self.lr_mant, self.lr_exp,
-                                  self.round_mode, self.seed, self.step_dev)
+        scalar_update(h)
         eoq.eoq_update_dev(h, [u.w for u in self.units], [u.g for u in self.units], [u.g_exp for u in self.units],
                            self.lr_mant, self.lr_exp, self.round_mode, self.seed, self.step_dev)
         self.weight_prep()

@@ -1712,11 +1712,12 @@ extern "C" int eoq_debug_force_wait_timeout(eoq_handle_t handle)
 
 static int update_impl(eoq_handle_t handle, int num, int8_t *const *w, const int8_t *const *g,
                        const int32_t *const *g_exp, const size_t *n, int32_t lr_mant, int32_t lr_exp, int round_mode,
-                       uint64_t seed, uint64_t step, uint64_t *step_dev, void *stream)
+                       uint64_t seed, uint64_t step, uint64_t *step_dev, void *stream, int first = 0, bool last = true)
 {
     Handle *h = reinterpret_cast<Handle *>(handle);
     if (!h || num <= 0 || !w || !g || !g_exp || !n) return EOQ_ERR_BAD_ARG;
-    if (num > 256) return EOQ_ERR_UNSUPPORTED;
+    if (first < 0) return EOQ_ERR_BAD_ARG;
+    if (num > 256 || first > 256 - num) return EOQ_ERR_UNSUPPORTED;
     if (lr_mant < 1 || lr_mant > 255 || lr_exp < -64 || lr_exp > 64) return EOQ_ERR_RANGE;
     if (round_mode != EOQ_ROUND_RNE && round_mode != EOQ_ROUND_STOCHASTIC) return EOQ_ERR_BAD_ARG;
     UpdateTensor t[256];
@@ -1732,7 +1733,7 @@ static int update_impl(eoq_handle_t handle, int num, int8_t *const *w, const int
     count_launches(h, update_launches(t, num, false));
     ProfScope prof(h, EOQ_PROF_UPDATE, s);
     return record(h, launch_update(t, num, lr_mant, lr_exp, round_mode == EOQ_ROUND_STOCHASTIC, seed, step,
-                                   reinterpret_cast<unsigned long long *>(step_dev), h->dev, s));
+                                   reinterpret_cast<unsigned long long *>(step_dev), h->dev, s, first, last));
 }
 
 extern "C" int eoq_update(eoq_handle_t handle, int num, int8_t *const *w, const int8_t *const *g,
@@ -1748,6 +1749,14 @@ extern "C" int eoq_update_dev(eoq_handle_t handle, int num, int8_t *const *w, co
 {
     if (!step || (reinterpret_cast<uintptr_t>(step) & 7)) return EOQ_ERR_BAD_ARG;
     return update_impl(handle, num, w, g, g_exp, n, lr_mant, lr_exp, round_mode, seed, 0, step, stream);
+}
+
+extern "C" int eoq_update_part(eoq_handle_t handle, int first, int last, int num, int8_t *const *w, const int8_t *const *g,
+                               const int32_t *const *g_exp, const size_t *n, int32_t lr_mant, int32_t lr_exp, int round_mode,
+                               uint64_t seed, uint64_t *step, void *stream)
+{
+    if (!step || (reinterpret_cast<uintptr_t>(step) & 7)) return EOQ_ERR_BAD_ARG;
+    return update_impl(handle, num, w, g, g_exp, n, lr_mant, lr_exp, round_mode, seed, 0, step, stream, first, last != 0);
 }
 
 extern "C" int eoq_update_wide(eoq_handle_t handle, int num, int32_t *const *master, int8_t *const *w, const int8_t *const *g,

@@ -332,7 +332,8 @@ struct UpdateTensor {
 };
 // step_dev (device, optional): the step counter is read from it and it is incremented behind the update.
 cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32_t lr_exp, int stochastic, uint64_t seed,
-                          uint64_t step, unsigned long long *step_dev, DeviceState *dev, cudaStream_t s);
+                          uint64_t step, unsigned long long *step_dev, DeviceState *dev, cudaStream_t s, int first = 0,
+                          bool last = true);
 int update_launches(const UpdateTensor *t, int num, bool wide);  // kernels the call above (wide: the one below) launches
 // The same update with a k_u-bit update quantizer on k_m-bit master codes (t[i].master); t[i].w receives Q_w(master).
 cudaError_t launch_update_wide(const UpdateTensor *t, int num, int32_t lr_mant, int32_t lr_exp, int k_u, int k_m, int stochastic,

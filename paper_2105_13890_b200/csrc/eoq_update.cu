@@ -23,7 +23,7 @@ struct UpdateBatch {
     int first_block[kUpdChunk + 1];
     int num;
     int tensor_base;  // index of t[0] in the whole call (cell of its maximum, counter of the hash)
-    int last;         // the call's last launch: its last block moves the step counter on
+    int last;         // the last launch for a step: its last block moves the step counter on
 };
 
 __device__ __forceinline__ int find_tensor(const UpdateBatch &b, int block)
@@ -350,11 +350,12 @@ __global__ void update_wide_apply_kernel(const __grid_constant__ UpdateBatch b, 
 }
 
 // The tensors [base, base + kUpdChunk) of a call as one launch's batch; returns its block count.
-int fill_batch(UpdateBatch &b, const UpdateTensor *t, int num, int base)
+// `first`: index of t[0] in the list that the rounding counts by; `last`: the call ends a step.
+int fill_batch(UpdateBatch &b, const UpdateTensor *t, int num, int base, int first, bool last)
 {
     b.num = num - base < kUpdChunk ? num - base : kUpdChunk;
-    b.tensor_base = base;
-    b.last = base + b.num == num;
+    b.tensor_base = first + base;
+    b.last = last && base + b.num == num;
     int blocks = 0;
     for (int k = 0; k < b.num; ++k) {
         b.t[k] = t[base + k];
@@ -375,18 +376,18 @@ int update_launches(const UpdateTensor *t, int num, bool wide)
 }
 
 cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32_t lr_exp, int stochastic, uint64_t seed,
-                          uint64_t step, unsigned long long *step_dev, DeviceState *dev, cudaStream_t s)
+                          uint64_t step, unsigned long long *step_dev, DeviceState *dev, cudaStream_t s, int first, bool last)
 {
     const int chunks = (num + kUpdChunk - 1) / kUpdChunk;
     const bool small = update_launches(t, num, false) == chunks;
     UpdateBatch b;
     if (!small)
         for (int base = 0; base < num; base += kUpdChunk) {
-            const int blocks = fill_batch(b, t, num, base);
+            const int blocks = fill_batch(b, t, num, base, first, last);
             launch_chained(update_absmax_kernel, blocks, kThreads, 0, s, b, dev);
         }
     for (int base = 0; base < num; base += kUpdChunk) {
-        const int blocks = fill_batch(b, t, num, base);
+        const int blocks = fill_batch(b, t, num, base, first, last);
         if (small) launch_chained(update_small_kernel, b.num, kSmallThreads, 0, s, b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
         else launch_chained(update_apply_kernel, blocks, kThreads, 0, s, b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
     }
@@ -399,7 +400,7 @@ cudaError_t launch_update_wide(const UpdateTensor *t, int num, int32_t lr_mant, 
     UpdateBatch b;
     for (int pass = 0; pass < 2; ++pass)
         for (int base = 0; base < num; base += kUpdChunk) {
-            const int blocks = fill_batch(b, t, num, base);
+            const int blocks = fill_batch(b, t, num, base, 0, true);
             if (pass == 0) launch_chained(update_absmax_kernel, blocks, kThreads, 0, s, b, dev);
             else launch_chained(update_wide_apply_kernel, blocks, kThreads, 0, s, b, lr_mant, lr_exp, k_u, k_m, stochastic, seed, step, step_dev, dev);
         }

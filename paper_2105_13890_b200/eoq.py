@@ -28,7 +28,7 @@ EXPORTS = [
     "eoq_quantize", "eoq_quantize_image", "eoq_err_prescale", "eoq_update", "eoq_layout_convert", "eoq_last_status",
     "eoq_last_cuda_error", "eoq_status_string", "eoq_profile_start", "eoq_profile_stop", "eoq_launch_count", "eoq_set_gemm_ctas",
     "eoq_conv_dgrad_static", "eoq_conv_fwd_dev", "eoq_weight_prep_size", "eoq_weight_prep", "eoq_conv_wgrad_dev",
-    "eoq_err_prescale_dev", "eoq_update_dev", "eoq_describe_plan", "eoq_debug_force_wait_timeout", "eoq_probe_mma_i8", "eoq_profile_gemm_only", "eoq_aux_maxpool_fwd", "eoq_aux_maxpool_bwd",
+    "eoq_err_prescale_dev", "eoq_update_dev", "eoq_update_part", "eoq_describe_plan", "eoq_debug_force_wait_timeout", "eoq_probe_mma_i8", "eoq_profile_gemm_only", "eoq_aux_maxpool_fwd", "eoq_aux_maxpool_bwd",
     "eoq_aux_maxpool_bwd_head", "eoq_aux_avgpool_sum", "eoq_aux_join", "eoq_aux_join_head", "eoq_conv_dgrad_head", "eoq_conv_dgrad_join_head", "eoq_conv_wgrad_gemm", "eoq_wgrad_finish", "eoq_aux_head_workspace_size", "eoq_aux_head", "eoq_aux_head_update", "eoq_aux_head_error", "eoq_aux_scalar_update", "eoq_update_wide", "eoq_set_reduce_hook", "eoq_bn_workspace_size", "eoq_bn_fwd", "eoq_bn_bwd",
 ]
 EOQ_STATIC_SCRATCH_BYTES = 16 << 20
@@ -103,6 +103,8 @@ def lib() -> C.CDLL:
         L.eoq_err_prescale_dev.argtypes = [vp, vp, vp, vp, vp, sz, vp, vp, vp, vp, vp, vp]
         L.eoq_update_dev.argtypes = [vp, C.c_int, C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), C.POINTER(sz), i32, i32,
                                      C.c_int, u64, vp, vp]
+        L.eoq_update_part.argtypes = [vp, C.c_int, C.c_int, C.c_int, C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), C.POINTER(sz), i32, i32,
+                                      C.c_int, u64, vp, vp]
         L.eoq_update_wide.argtypes = [vp, C.c_int, C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), C.POINTER(sz), i32, i32,
                                       C.c_int, C.c_int, C.c_int, u64, u64, vp, vp]
         L.eoq_set_reduce_hook.argtypes = [vp, REDUCE_FN, vp]
@@ -395,6 +397,17 @@ def eoq_update_dev(handle, w: Sequence, g: Sequence, g_exp: Sequence, lr_mant: i
     if check:
         _check(st, "eoq_update_dev")
     return st
+
+
+def eoq_update_part(handle, first: int, last: bool, w: Sequence, g: Sequence, g_exp: Sequence, lr_mant: int, lr_exp: int,
+                    round_mode: int, seed: int, step, stream=None) -> None:
+    """eoq_update_dev on the tensors first, first + 1, ... of a longer list; the part with `last` moves the step counter on."""
+    num = len(w)
+    arr = C.c_void_p * num
+    sizes = (C.c_size_t * num)(*[t.numel() for t in w])
+    _check(lib().eoq_update_part(handle, int(first), 1 if last else 0, num, arr(*[_ptr(t) for t in w]), arr(*[_ptr(t) for t in g]),
+                                 arr(*[_ptr(t) for t in g_exp]), sizes, int(lr_mant), int(lr_exp), int(round_mode), int(seed),
+                                 _ptr(step), _stream(stream)), "eoq_update_part")
 
 
 def eoq_describe_plan(handle, desc, pass_: int) -> str:

@@ -227,3 +227,23 @@ def test_error_sums_are_written_whole(d):
         assert G.status_clear() in ((0,) if want.any() else (eoq.EOQ_DEV_SQ_ZERO,))
         assert np.array_equal(G.host(e4).astype(np.int32).reshape(-1), np.asarray(want).reshape(-1)) and pe.item() == p
         assert total.item() == int(np.asarray(want, dtype=np.int64).sum())
+
+
+@pytest.mark.parametrize("cut", [1, 3, 5])
+@pytest.mark.parametrize("mode", [eoq.EOQ_ROUND_RNE, eoq.EOQ_ROUND_STOCHASTIC])
+def test_update_in_parts(cut, mode):
+    """Two parts of a list, the later one first, against one call on the whole list; the counter moves once."""
+    sizes = [144, 65536, 65537, 9408, 300007, 16]
+    w = [synth.int8_uniform(n, 1610, i) for i, n in enumerate(sizes)]
+    g, pg = [G.dev(synth.normal_codes(n, 1611, i)) for i, n in enumerate(sizes)], [G.dev(np.array([-9 - i], dtype=np.int32)) for i in range(6)]
+    whole, parts = [G.dev(x) for x in w], [G.dev(x) for x in w]
+    step, step_parts, h = torch.full((1,), 7, dtype=torch.int64, device="cuda:0"), torch.full((1,), 7, dtype=torch.int64, device="cuda:0"), G.handle()
+    for k in range(2):
+        eoq.eoq_update_dev(h, whole, g, pg, 37, -6, mode, 5, step)
+        eoq.eoq_update_part(h, cut, False, parts[cut:], g[cut:], pg[cut:], 37, -6, mode, 5, step_parts)
+        assert step_parts.item() == 7 + k
+        eoq.eoq_update_part(h, 0, True, parts[:cut], g[:cut], pg[:cut], 37, -6, mode, 5, step_parts)
+        assert all(torch.equal(a, b) for a, b in zip(whole, parts)) and step.item() == step_parts.item() == 8 + k
+    with pytest.raises(eoq.EoqError):
+        eoq.eoq_update_part(h, 255, True, parts[:2], g[:2], pg[:2], 37, -6, mode, 5, step_parts)
+    assert G.status_clear() == 0
