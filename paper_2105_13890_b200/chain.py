@@ -141,12 +141,13 @@ class ChainedStep:
         ws = max(ws, n * self.c_last * 4)
         self.workspace = torch.empty(ws, dtype=torch.uint8, device=dev)
         dev_index = dev.index if dev.index is not None else 0
-        self.h_sides = [eoq.eoq_create(dev_index) for _ in range(side_streams)]
+        self.h_sides = [eoq.eoq_create(dev_index) for _ in range(side_streams + 1)]   # the last: finishing and updating stages
         self.workspace_sides = [torch.empty(ws, dtype=torch.uint8, device=dev) for _ in range(side_streams)]
         half = torch.cuda.get_device_properties(dev).multi_processor_count // 2
         for hs in self.h_sides:
             eoq.eoq_set_gemm_ctas(hs, half)
-        self.sides = [torch.cuda.Stream(device=dev) for _ in range(side_streams)]
+        self.sides = [torch.cuda.Stream(device=dev) for _ in range(side_streams + 1)]
+        self.wgrad_sides = side_streams
         if finish_together:
             for u in self.units:
                 u.wgrad_ws = torch.empty(max(256, eoq.eoq_workspace_size(u.desc, eoq.EOQ_PASS_WGRAD)), dtype=torch.uint8, device=dev)
@@ -241,7 +242,7 @@ class ChainedStep:
 
         def wgrad(u: UnitBuffers, b1_dev) -> None:
             if overlap:
-                k = side_no[0] % len(self.sides)
+                k = side_no[0] % self.wgrad_sides
                 side_no[0] += 1
                 self.sides[k].wait_stream(main)
                 with torch.cuda.stream(self.sides[k]):
@@ -249,33 +250,36 @@ class ChainedStep:
             else:
                 wgrad_call(h, u, b1_dev, ws)
 
-        def finish(us, hh, last=False) -> None:
-            """b1 sums, slice sums and Q_g of the units whose GEMMs have been issued, a few launches for all of them; then
-            their update and the preparation of the new weights."""
+        def finish(us, hh) -> None:
+            """b1 sums, slice sums and Q_g of the units whose GEMMs have been issued, a few launches for all of them."""
             eoq.eoq_wgrad_finish(hh, [u.desc for u in us], [u.e3 for u in us], [u.e3_exp for u in us], [u.b1_dev for u in us],
                                  [u.g for u in us], [u.g_exp for u in us], [u.wgrad_ws for u in us], [u.wgrad_parts for u in us])
-            if overlap:   # the error chain must be through with the old weights; every other part of the update with the step counter
-                torch.cuda.current_stream(self.dev).wait_stream(main)
-                if last:
-                    for side in self.sides:
-                        main.wait_stream(side)
+
+        def update(us, hh, last) -> None:
             us = sorted(us, key=lambda u: u.index)
             eoq.eoq_update_part(hh, us[0].index, last, [u.w for u in us], [u.g for u in us], [u.g_exp for u in us], self.lr_mant,
                                 self.lr_exp, self.round_mode, self.seed, self.step_dev)
             eoq.eoq_weight_prep(hh, [u.desc for u in us], [u.w for u in us], [u.prep for u in us])
 
-        def stage_done(us) -> None:
+        def stage_done(us, front: bool) -> None:
             """A stage of the network is through: its gradients are finished and its weights updated together, behind its
-            GEMMs on a side stream, beside the backward chain of the stages in front."""
-            if not self.finish_together or not us:
+            GEMMs on a side stream, beside the backward chain of the stages in front.  (The front stage is updated with the
+            first layer.)"""
+            if not self.finish_together:
                 return
-            if overlap:
-                for side in self.sides[1:]:
-                    self.sides[0].wait_stream(side)
-                with torch.cuda.stream(self.sides[0]):
-                    finish(us, self.h_sides[0])
-            else:
+            if not overlap:
                 finish(us, h)
+                if not front:
+                    update(us, h, False)
+                return
+            fin, h_fin = self.sides[-1], self.h_sides[-1]
+            for side in self.sides[:-1]:
+                fin.wait_stream(side)
+            with torch.cuda.stream(fin):
+                finish(us, h_fin)
+                if not front:
+                    fin.wait_stream(main)   # the error chain is through with the old weights
+                    update(us, h_fin, False)
 
         e_out, e_exp = self.e_head, self.e_head_exp
         head_done = False   # the error head of this block's last unit already ran inside the join of the block behind it
@@ -285,7 +289,7 @@ class ChainedStep:
             blk = self.blocks[i]
             a, b, pr = blk.a, blk.b, blk.proj
             if stage is not None and a.layer.name.split(".")[0] != stage:
-                stage_done(pending)
+                stage_done(pending, False)
                 pending = []
             stage = a.layer.name.split(".")[0]
             pending += [b, a] + ([pr] if pr else [])
@@ -317,7 +321,7 @@ class ChainedStep:
                                              blk.e_in_exp, blk.sum_join, workspace=ws)
                 head_done = False
             e_out, e_exp = blk.e_in, blk.e_in_exp
-        stage_done(pending)
+        stage_done(pending, True)
         if self.pool:
             k, s, p = self.pool
             # pool backward and the first layer's error head in one pair of kernels; the error between them (51 MB at
@@ -338,13 +342,17 @@ class ChainedStep:
         if self.finish_together:
             # the first layer's weight gradient ends the chain; the scalars are updated beside it, behind the last reader of b1
             if overlap:
-                self.sides[0].wait_stream(main)
-                with torch.cuda.stream(self.sides[0]):
-                    scalar_update(self.h_sides[0])
+                self.sides[-1].wait_stream(main)
+                with torch.cuda.stream(self.sides[-1]):
+                    scalar_update(self.h_sides[-1])
             else:
                 scalar_update(h)
             wgrad_call(h, stem, None, ws)
-            finish([stem], h, last=True)
+            finish([stem], h)
+            if overlap:
+                for side in self.sides:
+                    main.wait_stream(side)
+            update(pending + [stem], h, True)
             return
         wgrad(stem, None)
         if overlap:
