@@ -259,6 +259,10 @@ __device__ __forceinline__ void st_cluster_128(uint32_t addr, uint32_t a, uint32
 {
     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+__device__ __forceinline__ void st_cluster_32(uint32_t addr, uint32_t v)
+{
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 __device__ __forceinline__ int4 ld_shared_128(uint32_t addr)
 {
     int4 v;

@@ -851,48 +851,68 @@ __global__ void b1_weight_table_kernel(const int8_t *__restrict__ w, int32_t *ta
 
 // What eoq_weight_prep derives from the weights of several layers in one launch: the b1 table of every layer
 // (as b1_weight_table_kernel builds it) and, for a first layer on the filter-row path, the weights re-packed as
-// [oc][kh][8][c_in] with zero taps.  One block per (layer, output channel).
+// [oc][kh][8][c_in] with zero taps.  One block per (layer, output channel), bound by latency: all chunks of a channel are
+// loaded at once and added to their tap's cell, while the taps that each border class takes are worked out.
 __global__ void weight_prep_kernel(const __grid_constant__ PrepBatch b)
 {
     ptx::grid_dep_wait_launch_small();
     __shared__ int32_t tap_sum[kMaxTaps];
     int k = 0;
-    while (k + 1 < b.num && (int)blockIdx.x >= b.first_block[k + 1]) ++k;
+    for (int hi = b.num - 1; k < hi;) {
+        const int mid = (k + hi + 1) >> 1;
+        if ((int)blockIdx.x >= b.first_block[mid]) k = mid;
+        else hi = mid - 1;
+    }
     const PrepItem &it = b.item[k];
     const eoq_conv_desc_t &d = it.d;
     const BorderClasses &bc = it.bc;
     const int oc = blockIdx.x - b.first_block[k];
-    const int taps = d.kh * d.kw;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    for (int t = warp; t < taps; t += nwarps) {
-        const int8_t *p = it.w + ((size_t)oc * taps + t) * d.c_in;
-        int sum = 0;
-        for (int i = lane; i < d.c_in / 16; i += 32) {
-            const int4 v = __ldg(reinterpret_cast<const int4 *>(p) + i);
-            sum = __dp4a(v.x, 0x01010101, sum);
-            sum = __dp4a(v.y, 0x01010101, sum);
-            sum = __dp4a(v.z, 0x01010101, sum);
-            sum = __dp4a(v.w, 0x01010101, sum);
-        }
-        if (d.c_in == 8 && lane == 0) {
-            const int2 v = __ldg(reinterpret_cast<const int2 *>(p));
-            sum = __dp4a(v.x, 0x01010101, sum);
-            sum = __dp4a(v.y, 0x01010101, sum);
-        }
+    const int taps = d.kh * d.kw, width = d.c_in == 8 ? 8 : 16, per_tap = d.c_in / width, chunks = taps * per_tap;
+    const int8_t *w = it.w + (size_t)oc * taps * d.c_in;
+    auto load = [&](int i) {
+        if (width == 16) return __ldg(reinterpret_cast<const int4 *>(w) + i);
+        const int2 v = __ldg(reinterpret_cast<const int2 *>(w) + i);   // the 8-channel first layer: one 8-byte pixel per tap
+        return make_int4(v.x, v.y, 0, 0);
+    };
+    constexpr int kAhead = 3;   // 3 x 3 filters of up to 640 channels in one round
+    int4 v[kAhead];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (lane == 0) tap_sum[t] = sum;
+    for (int u = 0; u < kAhead; ++u) {
+        const int i = threadIdx.x + u * blockDim.x;
+        if (i < chunks) v[u] = load(i);
+    }
+    for (int t = threadIdx.x; t < taps; t += blockDim.x) tap_sum[t] = 0;
+    const int classes = bc.nrc * bc.ncc;   // at most kMaxBorderClasses, fewer than threads
+    unsigned long long takes = 0;          // the taps of this thread's class that fall inside the image
+    if ((int)threadIdx.x < classes) {
+        const int rc = threadIdx.x / bc.ncc, cc = threadIdx.x - rc * bc.ncc;
+        unsigned long long row = 0;
+        for (int kw = 0; kw < d.kw; ++kw)
+            if (tap_valid(cc, kw, it.wo, d.w, bc.nlo_w, bc.nhi_w, bc.ncc, d.stride, d.pad)) row |= 1ull << kw;
+        for (int kh = 0; kh < d.kh; ++kh)
+            if (tap_valid(rc, kh, it.ho, d.h, bc.nlo_h, bc.nhi_h, bc.nrc, d.stride, d.pad)) takes |= row << (kh * d.kw);
     }
     __syncthreads();
-    for (int cls = threadIdx.x; cls < bc.nrc * bc.ncc; cls += blockDim.x) {
-        const int rc = cls / bc.ncc, cc = cls % bc.ncc;
-        int32_t sum = 0;
-        for (int kh = 0; kh < d.kh; ++kh) {
-            if (!tap_valid(rc, kh, it.ho, d.h, bc.nlo_h, bc.nhi_h, bc.nrc, d.stride, d.pad)) continue;
-            for (int kw = 0; kw < d.kw; ++kw)
-                if (tap_valid(cc, kw, it.wo, d.w, bc.nlo_w, bc.nhi_w, bc.ncc, d.stride, d.pad)) sum += tap_sum[kh * d.kw + kw];
+    auto add = [&](int i, const int4 &q) {
+        const int s = __dp4a(q.x, 0x01010101, __dp4a(q.y, 0x01010101, __dp4a(q.z, 0x01010101, __dp4a(q.w, 0x01010101, 0))));
+        if (per_tap % 32 == 0) {   // a warp's chunks belong to one tap (and `chunks` is a multiple of 32)
+            const int sum = __reduce_add_sync(0xffffffffu, s);
+            if ((threadIdx.x & 31) == 0) atomicAdd(&tap_sum[i / per_tap], sum);
+        } else {
+            atomicAdd(&tap_sum[i / per_tap], s);
         }
-        it.table[(size_t)cls * d.c_out + oc] = sum;
+    };
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+        const int i = threadIdx.x + u * blockDim.x;
+        if (i < chunks) add(i, v[u]);
+    }
+    for (int i = threadIdx.x + kAhead * blockDim.x; i < chunks; i += blockDim.x) add(i, load(i));
+    __syncthreads();
+    if ((int)threadIdx.x < classes) {
+        int32_t sum = 0;
+        for (unsigned long long m = takes; m; m &= m - 1) sum += tap_sum[__ffsll((long long)m) - 1];
+        it.table[(size_t)threadIdx.x * d.c_out + oc] = sum;
     }
     if (it.w_rows) {
         // this output channel's filter rows, each widened to 8 taps (c_in is 16 or 8: 4 or 2 words per tap)

@@ -12,10 +12,13 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kUpdChunk = 64;            // tensors per launch
 constexpr int kUpdElemsPerBlock = 8192;  // elements one block covers
-// Tensors up to this size are updated by one block each, which keeps the gradient codes in registers between the two
-// passes (64 codes per thread): every weight tensor of the CIFAR-shaped networks (at most 36,864 codes).
+// Tensors up to kSmallElems are updated by one block or one cluster each, in one launch: every weight tensor of the
+// CIFAR-shaped networks (at most 36,864 codes).  Beyond kSmallPart codes stochastic rounding takes one block too long
+// (36,864 codes: 11 us, a cluster of eight 6 us).
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallGroups = 4;          // 16-code groups per thread
+constexpr size_t kSmallPart = 8192;
+constexpr int kSmallMostParts = 8;
 constexpr size_t kSmallElems = (size_t)kSmallThreads * kSmallGroups * 16;
 
 struct UpdateBatch {
@@ -243,41 +246,58 @@ update_apply_kernel(const __grid_constant__ UpdateBatch b, int32_t lr_mant, int3
     }
 }
 
-// Both passes of one small tensor in one block (see kSmallElems).  Bound by latency: one read of g, one block reduction,
-// one read and one write of w.  2,304 weights: 3.5 us, where a cleared cell, two passes and the step counter's own kernel
-// took four launches and 8.8 us.
+// Both passes of one small tensor in one block, or in a cluster of `parts` blocks that exchange their maxima through
+// distributed shared memory (see kSmallElems and kSmallPart).  Bound by latency: one read of g, one reduction, one read and
+// one write of w.  2,304 weights: 3.5 us, where a cleared cell, two passes and the step counter's own kernel took four launches
+// and 8.8 us.
 __global__ void __launch_bounds__(kSmallThreads)
-update_small_kernel(const __grid_constant__ UpdateBatch b, int32_t lr_mant, int32_t lr_exp, int stochastic, unsigned long long seed,
-                    unsigned long long step, unsigned long long *step_dev, DeviceState *dev)
+update_small_kernel(const __grid_constant__ UpdateBatch b, int parts, int32_t lr_mant, int32_t lr_exp, int stochastic,
+                    unsigned long long seed, unsigned long long step, unsigned long long *step_dev, DeviceState *dev)
 {
-    ptx::grid_dep_wait_launch_small();
     __shared__ unsigned long long step_s;
-    const UpdateTensor &T = b.t[blockIdx.x];
+    __shared__ __align__(16) uint32_t max_s[kSmallMostParts];
+    const int k = (int)blockIdx.x / parts, part = (int)blockIdx.x - k * parts;
+    if (parts > 1) ptx::cluster_arrive();   // met below: the other blocks have started before their shared memory is written
+    ptx::grid_dep_wait_launch_small();
+    const UpdateTensor &T = b.t[k];
     const int g_exp = __ldg(T.g_exp);
     if (threadIdx.x == 0) step_s = step_dev ? *reinterpret_cast<volatile unsigned long long *>(step_dev) : step;
-    const size_t n = (size_t)T.n;
+    const size_t n = (size_t)T.n, slice = ((n + parts - 1) / parts + 15) / 16 * 16;
+    const size_t begin = min(n, part * slice), end = min(n, begin + slice);
     const bool vec = (reinterpret_cast<uintptr_t>(T.g) & 15) == 0;
     AbsMax16 am;
     if (vec) {
 #pragma unroll
         for (int q = 0; q < kSmallGroups; ++q) {
-            const size_t i = ((size_t)q * kSmallThreads + threadIdx.x) * 16;
-            if (i + 16 <= n) am.add(__ldg(reinterpret_cast<const int4 *>(T.g + i)));
+            const size_t i = begin + ((size_t)q * kSmallThreads + threadIdx.x) * 16;
+            if (i + 16 <= end) am.add(__ldg(reinterpret_cast<const int4 *>(T.g + i)));
         }
     }
     uint32_t mx = am.value();
-    for (size_t j = (vec ? n / 16 * 16 : 0) + threadIdx.x; j < n; j += kSmallThreads) mx = max(mx, (uint32_t)abs((int)T.g[j]));
+    for (size_t j = (vec ? begin + (end - begin) / 16 * 16 : begin) + threadIdx.x; j < end; j += kSmallThreads)
+        mx = max(mx, (uint32_t)abs((int)T.g[j]));
     mx = block_max_u32(mx);
-    __shared__ uint32_t max_s;
-    if (threadIdx.x == 0) max_s = mx;
-    __syncthreads();
+    if (parts > 1) {
+        ptx::cluster_wait();
+        if (threadIdx.x < 32) {
+            mx = __shfl_sync(0xffffffffu, mx, 0);
+            if ((int)threadIdx.x < parts) ptx::st_cluster_32(ptx::cluster_addr(ptx::smem_u32(&max_s[part]), threadIdx.x), mx);
+        }
+        ptx::cluster_sync();
+        mx = 0;
+        for (int i = 0; i < parts; ++i) mx = max(mx, max_s[i]);
+    } else {
+        if (threadIdx.x == 0) max_s[0] = mx;
+        __syncthreads();
+        mx = max_s[0];
+    }
     bool last = false;
     if (threadIdx.x == 0) last = last_reader(dev);
-    const uint32_t M = max_s * (uint32_t)lr_mant;
+    const uint32_t M = mx * (uint32_t)lr_mant;
     if (M != 0) {
-        const UpdateRule r = update_rule(M, g_exp, lr_mant, lr_exp, stochastic, seed, step_s, b.tensor_base + blockIdx.x);
-        update_range(update_mode(r, stochastic), T, 0, n, r);
-    } else if (threadIdx.x == 0) {
+        const UpdateRule r = update_rule(M, g_exp, lr_mant, lr_exp, stochastic, seed, step_s, b.tensor_base + k);
+        update_range(update_mode(r, stochastic), T, begin, end, r);
+    } else if (threadIdx.x == 0 && part == 0) {
         atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
     }
     if (last && b.last && step_dev) *step_dev = step_s + 1ull;
@@ -380,6 +400,9 @@ cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32
 {
     const int chunks = (num + kUpdChunk - 1) / kUpdChunk;
     const bool small = update_launches(t, num, false) == chunks;
+    int parts = 1;
+    for (int i = 0; i < num; ++i)
+        if (stochastic && t[i].n > kSmallPart) parts = kSmallMostParts;   // (the hash is what takes the time)
     UpdateBatch b;
     if (!small)
         for (int base = 0; base < num; base += kUpdChunk) {
@@ -388,7 +411,7 @@ cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32
         }
     for (int base = 0; base < num; base += kUpdChunk) {
         const int blocks = fill_batch(b, t, num, base, first, last);
-        if (small) launch_chained(update_small_kernel, b.num, kSmallThreads, 0, s, b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
+        if (small) launch_chained_clusters(parts, update_small_kernel, b.num * parts, kSmallThreads, 0, s, b, parts, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
         else launch_chained(update_apply_kernel, blocks, kThreads, 0, s, b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
     }
     return cudaGetLastError();

@@ -229,7 +229,7 @@ def test_error_sums_are_written_whole(d):
         assert total.item() == int(np.asarray(want, dtype=np.int64).sum())
 
 
-@pytest.mark.parametrize("cut", [1, 3, 5])
+@pytest.mark.parametrize("cut", [1, 2, 3, 5])
 @pytest.mark.parametrize("mode", [eoq.EOQ_ROUND_RNE, eoq.EOQ_ROUND_STOCHASTIC])
 def test_update_in_parts(cut, mode):
     """Two parts of a list, the later one first, against one call on the whole list; the counter moves once."""
@@ -247,3 +247,19 @@ def test_update_in_parts(cut, mode):
     with pytest.raises(eoq.EoqError):
         eoq.eoq_update_part(h, 255, True, parts[:2], g[:2], pg[:2], 37, -6, mode, 5, step_parts)
     assert G.status_clear() == 0
+
+
+@pytest.mark.parametrize("d", [
+    oracle.ConvDesc(1, 5, 6, 704, 32, 3, 3, 1, 1),    # more chunks than one round of loads
+    oracle.ConvDesc(2, 8, 8, 16, 16, 7, 7, 1, 3),     # every row and column has its own class: 64 of them
+    oracle.ConvDesc(1, 9, 9, 48, 16, 8, 8, 1, 3),     # 64 taps
+    oracle.ConvDesc(2, 6, 6, 32, 48, 1, 1, 2, 0),     # one tap
+], ids=lambda d: f"{d.h}x{d.w}_c{d.c_in}_k{d.kh}")
+def test_prepared_weights(d):
+    x, w = synth.relu_codes((d.n, d.h, d.w, d.c_in), 1620, 0), synth.int8_uniform((d.c_out, d.kh, d.kw, d.c_in), 1620, 1, -30, 30)
+    ref, gd, h = oracle.layer_forward(d, x, -6, w, 90, 5, None, True), G.gdesc(d), G.handle()
+    prep = torch.full((max(256, eoq.eoq_weight_prep_size(gd)),), 0x55, dtype=torch.uint8, device="cuda:0")
+    wd, x5 = G.dev(w), G.zeros(ref["x5"].shape, torch.int8)
+    eoq.eoq_weight_prep(h, [gd], [wd], [prep])
+    eoq.eoq_conv_fwd_dev(h, gd, G.dev(x), None, G.dev(np.array([-6, 90, 5], dtype=np.int32)), wd, prep, None, True, x5)
+    assert G.status_clear() == 0 and np.array_equal(G.host(x5), ref["x5"])
