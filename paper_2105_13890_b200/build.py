@@ -11,7 +11,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libeoq.so")
 BIND = os.path.join(HERE, "_eoqbind.so")
-SOURCES = ["eoq_api.cu", "eoq_igemm.cu", "eoq_igemm_patch.cu", "eoq_wgrad_patch.cu", "eoq_wgrad.cu", "eoq_finish.cu", "eoq_elementwise.cu", "eoq_update.cu", "eoq_static.cu", "eoq_probe.cu", "eoq_aux.cu", "eoq_pool.cu", "eoq_head.cu", "eoq_bn.cu"]
+SOURCES = ["eoq_api.cu", "eoq_igemm.cu", "eoq_igemm_patch.cu", "eoq_wgrad_patch.cu", "eoq_wgrad.cu", "eoq_wgrad_rows.cu", "eoq_finish.cu", "eoq_elementwise.cu", "eoq_update.cu", "eoq_static.cu", "eoq_probe.cu", "eoq_aux.cu", "eoq_pool.cu", "eoq_head.cu", "eoq_bn.cu"]
 HEADERS = ["eoq_internal.h", "eoq_cells.cuh", "eoq_device.cuh", "eoq_epilogue.cuh", "eoq_next_head.cuh", os.path.join(ROOT, "include", "eoq.h")]
 
 

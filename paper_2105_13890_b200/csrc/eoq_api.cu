@@ -547,11 +547,51 @@ bool plan_wgrad(WgradParams &p, const eoq_conv_desc_t &d, const Geometry &g, int
     return true;
 }
 
+// Plan of the filter-row weight gradient with its window rows in a ring; false when the geometry does not suit it (16 channels,
+// or rows so wide that the ring does not hold two output rows: the per-tap kernel).
+bool plan_wgrad_rows(WgradRowsPlan &pl, const eoq_conv_desc_t &d, const Geometry &g, int ctas)
+{
+    if (!use_row_window(d, g.wo) || d.c_in != 8 || g.wo > 256) return false;
+    memset(&pl, 0, sizeof(pl));
+    pl.n_img = d.n; pl.ho = g.ho; pl.wo = g.wo; pl.kh = d.kh; pl.kw = d.kw; pl.stride = d.stride; pl.pad = d.pad;
+    pl.c_in = d.c_in; pl.c_out = d.c_out;
+    pl.kc = 8 * d.c_in;
+    pl.nc = chunk_bytes(d.c_out);
+    const int per_tile = kTileM / pl.kc;
+    pl.mtiles = (d.kh + per_tile - 1) / per_tile;
+    if (pl.nc < 32 || d.c_out > 256 || pl.mtiles * d.c_out > 512) return false;
+    pl.kp = (g.wo + 31) / 32 * 32;
+    pl.span = pl.mtiles * per_tile;
+    pl.rows_total = g.taps * d.c_in;
+    const int most = pl.span > d.stride ? pl.span : d.stride;   // what the ring advances at the start of an image
+    for (int stages = 4; stages >= 2; --stages) {
+        // `stages` output rows in flight, with one start of an image among them (or each its own, in images of few rows)
+        const int advance = g.ho >= stages - 1 ? (stages - 2) * d.stride + most : (stages - 1) * most;
+        int slots = (200 * 1024 - stages * pl.kp * d.c_out) / (pl.kp * pl.kc);
+        slots -= slots % per_tile;
+        if (slots < advance + pl.span) continue;
+        pl.num_stages = stages;
+        pl.slots = advance + pl.span + per_tile - 1;
+        pl.slots -= pl.slots % per_tile;
+        break;
+    }
+    if (!pl.num_stages) return false;
+    // as plan_wgrad: twice the CTAs asked for, one per SM at most; a row adds at most wo * 127 * 127 to an int32 sum
+    const int cap = 2 * ctas < kWgradTargetCtas ? 2 * ctas : kWgradTargetCtas, rows = d.n * g.ho, exact = 130000 / g.wo;
+    int per = (rows + cap - 1) / cap;
+    if (per > exact) per = exact;
+    pl.rows_per_split = per;
+    pl.num_splits = (rows + per - 1) / per;
+    return true;
+}
+
 // int32 slices of partial sums the weight-gradient GEMM leaves, at most
 int wgrad_slices(const eoq_conv_desc_t &d, const Geometry &g)
 {
     WgradPatchPlan wp;
     if (plan_wgrad_patch(wp, d, g.ho, g.wo)) return wp.num_splits;
+    WgradRowsPlan rp;
+    if (plan_wgrad_rows(rp, d, g, kWgradTargetCtas)) return rp.num_splits;
     WgradParams p;
     return plan_wgrad(p, d, g, kWgradTargetCtas) ? p.num_k_splits : 0;
 }
@@ -1463,10 +1503,31 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
         return finish(wp.num_splits);
     }
 
+    const int w_mem = d.w + 2 * d.x_wmargin;
+    WgradRowsPlan rp;
+    if (plan_wgrad_rows(rp, d, g, h->gemm_ctas)) {
+        rp.partials = w.parts;
+        rp.zero = reinterpret_cast<int4 *>(w.tap_sums);
+        rp.zero_n16 = (unsigned)(w.zero_bytes / 16);
+        rp.dev = h->dev;
+        CUtensorMap map_x, map_e;
+        if (!make_matrix_map(&map_e, e3, (size_t)d.n * g.ho * g.wo, d.c_out, rp.nc, g.wo) ||
+            !make_row_window_map(&map_x, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, g.wo, g.ho, d.stride, d.pad, g.wo))
+            return EOQ_ERR_UNSUPPORTED;
+        count_launches(h, 1);
+        if (num_parts_out) *num_parts_out = rp.num_splits;
+        cudaError_t e;
+        {
+            ProfScope prof(h, EOQ_PROF_WGRAD, s);
+            e = launch_wgrad_rows(rp, map_x, map_e, s);
+        }
+        if (e != cudaSuccess || gemm_only) return record(h, e);
+        return finish(rp.num_splits);
+    }
+
     WgradParams p;
     if (!plan_wgrad(p, d, g, h->gemm_ctas)) return EOQ_ERR_UNSUPPORTED;
     const bool row_window = p.row_window_kw != 0;
-    const int w_mem = d.w + 2 * d.x_wmargin;
     p.partials = w.parts;
     p.zero = reinterpret_cast<int4 *>(w.tap_sums);
     p.zero_n16 = (unsigned)(w.zero_bytes / 16);

@@ -287,6 +287,23 @@ struct WgradPatchPlan {
 constexpr int kWgradPatchThreads = 192;  // warp 0 loads, warp 1 MMA + TMEM, warps 2..5 epilogue
 constexpr int kWgradTargetCtas = 148;    // CTAs the split count aims at (one per SM of a 148-SM part; shared memory allows one)
 
+// Weight gradient of a first layer on the filter-row path with its window rows in a ring (eoq_wgrad_rows.cu)
+struct WgradRowsPlan {
+    int n_img, ho, wo, kh, kw, stride, pad, c_in, c_out;
+    int kc, nc;          // bytes of a window (8 pixels) and of an error sub-tile row
+    int kp;              // wo rounded up to 32
+    int slots, span;     // window rows in the ring (even), and of one output row rounded up to whole M tiles
+    int mtiles;          // M tiles of 128 / kc filter rows
+    int num_stages;      // output rows in flight
+    int rows_per_split, num_splits;
+    int rows_total;      // kh * kw * c_in
+    int32_t *partials;   // [num_splits][c_out][kh][kw][c_in]
+    int4 *zero;          // as in WgradParams
+    unsigned zero_n16;
+    DeviceState *dev;
+};
+cudaError_t launch_wgrad_rows(const WgradRowsPlan &pl, const CUtensorMap &map_x, const CUtensorMap &map_e, cudaStream_t stream);
+
 size_t wgrad_patch_smem_bytes(const WgradPatchPlan &pl);
 cudaError_t launch_wgrad_patch(const WgradPatchPlan &pl, const CUtensorMap &map_x, const CUtensorMap &map_e,
                                cudaStream_t stream);

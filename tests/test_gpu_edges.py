@@ -263,3 +263,30 @@ def test_prepared_weights(d):
     eoq.eoq_weight_prep(h, [gd], [wd], [prep])
     eoq.eoq_conv_fwd_dev(h, gd, G.dev(x), None, G.dev(np.array([-6, 90, 5], dtype=np.int32)), wd, prep, None, True, x5)
     assert G.status_clear() == 0 and np.array_equal(G.host(x5), ref["x5"])
+
+
+@pytest.mark.parametrize("d,m", [
+    (oracle.ConvDesc(5, 20, 20, 8, 64, 7, 7, 2, 3), 5),     # ring restarts at every image
+    (oracle.ConvDesc(2, 9, 226, 8, 64, 7, 7, 2, 3), 5),     # 113 pixels a row: 15 pixels of padding
+    (oracle.ConvDesc(9, 3, 64, 8, 128, 7, 7, 2, 3), 5),     # two output rows an image, 128 columns
+    (oracle.ConvDesc(7, 1, 24, 8, 32, 5, 5, 2, 2), 4),      # one output row an image, 5 x 5
+    (oracle.ConvDesc(2, 31, 30, 8, 64, 7, 7, 4, 3), 7),     # stride 4
+    (oracle.ConvDesc(1, 40, 66, 8, 32, 8, 8, 2, 3), 9),     # 8 x 8: no padding tap
+    (oracle.ConvDesc(1, 8, 512, 8, 64, 7, 7, 2, 3), 5),     # rows too wide for the ring
+    (oracle.ConvDesc(2, 12, 20, 8, 48, 7, 7, 2, 3), 5),     # 16-byte error sub-tiles: one tap at a time
+], ids=lambda v: f"n{v.n}_{v.h}x{v.w}_c{v.c_out}_k{v.kh}s{v.stride}" if isinstance(v, oracle.ConvDesc) else None)
+@pytest.mark.parametrize("ctas", [0, 1])
+def test_first_layer_weight_gradient(d, m, ctas):
+    """Window rows in a ring, over every wrap and restart; with two CTAs each walks many output rows."""
+    x, e3 = synth.int8_uniform((d.n, d.h, d.w, d.c_in), 1630, 0), synth.normal_codes((d.n, d.ho, d.wo, d.c_out), 1630, 1)
+    want = oracle.conv_wgrad_acc(d, e3, x, 0)
+    gd, h = eoq.conv_desc(d.n, d.h, d.w, d.c_in, d.c_out, d.kh, d.kw, d.stride, d.pad, m), eoq.eoq_create(0)
+    eoq.eoq_set_gemm_ctas(h, ctas)
+    xm = G.dev(np.pad(x, ((0, 0), (0, 0), (m, m), (0, 0))))
+    ws = G.workspace(gd, eoq.EOQ_PASS_WGRAD)
+    ws.fill_(0x55)
+    g, pg, acc = G.zeros(want.shape, torch.int8), G.zeros(1, torch.int32), G.zeros(want.shape, torch.int64)
+    for _ in range(2):
+        eoq.eoq_conv_wgrad(h, gd, G.dev(e3), G.dev(np.array([-9], dtype=np.int32)), xm, 0, g, pg, acc, ws)
+        assert eoq.eoq_last_status(h) == 0 and np.array_equal(G.host(acc), want)
+    eoq.eoq_destroy(h)
