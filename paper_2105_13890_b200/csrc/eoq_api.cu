@@ -414,8 +414,7 @@ bool plan_wgrad_patch(WgradPatchPlan &pl, const eoq_conv_desc_t &d, int ho, int 
     // half: the error back-propagation of such layers leaves the other half of an SM's shared memory, and the two then share
     // SMs (ResNet-20 step at batch 128: 659 -> 647 us; wider layers fill the SM anyway and only load more halo rows).
     const int smem_kb = pl.kc <= 32 && pl.tile_n <= 32 ? 100 : 200;
-    int r = ho < 32 ? ho : 32;
-    for (; r >= 1; --r) {
+    auto set_rows = [&](int r) {
         const int kp = (r * pl.pw + 31) / 32 * 32;
         int x_rows = (r + d.kh - 1) * pl.pw;
         const int x_read = (d.kh - 1) * (pl.pw + 1) + pl.apa + kp;
@@ -423,26 +422,49 @@ bool plan_wgrad_patch(WgradPatchPlan &pl, const eoq_conv_desc_t &d, int ho, int 
         pl.x_bytes = (x_rows * pl.kc + 1023) / 1024 * 1024;
         pl.e_bytes = (kp * pl.tile_n + 1023) / 1024 * 1024;
         pl.kp = kp;
+        pl.r_rows = r;
+        pl.blocks_per_img = (ho + r - 1) / r;
+        pl.x_box_bytes = pl.kc * pl.pw * (r + d.kh - 1);
+        pl.e_box_bytes = pl.tile_n * pl.pw * r;
+        const int stages = (smem_kb * 1024) / (pl.x_bytes + pl.e_bytes);
+        pl.num_stages = stages > 4 ? 4 : stages;
+        const int total_blocks = d.n * pl.blocks_per_img;
+        int splits = target_ctas / pl.num_groups;  // rounded down: a few CTAs beyond one wave would double the kernel's time
+        if (splits > total_blocks) splits = total_blocks;
+        if (splits < 1) splits = 1;
+        int per = (total_blocks + splits - 1) / splits;
+        const int max_per = 130000 / kp;  // keeps a CTA's int32 partial sums exact: rows * 127 * 128 < 2^31
+        if (per > max_per) per = max_per;
+        pl.blocks_per_split = per;
+        pl.num_splits = per > 0 ? (total_blocks + per - 1) / per : 0;
+    };
+    int r = ho < 32 ? ho : 32;
+    for (; r >= 1; --r) {
+        set_rows(r);
         if (pl.x_bytes + pl.e_bytes <= smem_kb / 3 * 1024) break;
     }
-    if (r < 1) return false;
-    pl.r_rows = r;
-    pl.blocks_per_img = (ho + r - 1) / r;
-    pl.x_box_bytes = pl.kc * pl.pw * (r + d.kh - 1);
-    pl.e_box_bytes = pl.tile_n * pl.pw * r;
-    int stages = (smem_kb * 1024) / (pl.x_bytes + pl.e_bytes);
-    pl.num_stages = stages > 4 ? 4 : stages;
-    if (pl.num_stages < 2) return false;
-    const int total_blocks = d.n * pl.blocks_per_img;
-    int splits = target_ctas / pl.num_groups;  // rounded down: a few CTAs beyond one wave would double the kernel's time
-    if (splits > total_blocks) splits = total_blocks;
-    if (splits < 1) splits = 1;
-    int per = (total_blocks + splits - 1) / splits;
-    const int max_per = 130000 / pl.kp;  // keeps a CTA's int32 partial sums exact: rows * 127 * 128 < 2^31
-    if (max_per < 1) return false;
-    if (per > max_per) per = max_per;
-    pl.blocks_per_split = per;
-    pl.num_splits = (total_blocks + per - 1) / per;
+    if (r < 1 || pl.num_stages < 2 || pl.blocks_per_split < 1) return false;
+    // Small batches leave fewer blocks than CTAs: shorter blocks then, as long as the time a CTA saves is not spent on more
+    // slices.  In SM cycles: a TMA row 4.5, an MMA 57 to 64; a slice is written and read back at 2,500 bytes per cycle.
+    auto cost = [&]() {
+        const double load = 4.5 * pl.pw * (2 * pl.r_rows + d.kh - 1);
+        const double mma = pl.kp / 32 * pl.rows_per_group * pl.accs_per_row * (pl.tile_n > 114 ? 64.0 : 57.0);
+        return pl.blocks_per_split * (load > mma ? load : mma) + (double)pl.num_splits * d.c_out * pl.rows_total * 8 / 2500.0;
+    };
+    int best_r = r;
+    double best = cost();
+    for (int rr = (r + 1) / 2; rr >= 1; rr = (rr + 1) / 2) {
+        set_rows(rr);
+        if (pl.num_stages >= 2 && pl.blocks_per_split >= 1 && cost() < 0.9 * best) {
+            best = cost();
+            best_r = rr;
+        }
+        if (rr == 1) break;
+    }
+    set_rows(best_r);
+    // with fewer CTAs no more slices than with all of them (the workspace holds that many)
+    WgradPatchPlan full;
+    if (target_ctas < kWgradTargetCtas && plan_wgrad_patch(full, d, ho, wo) && pl.num_splits > full.num_splits) pl = full;
     return true;
 }
 

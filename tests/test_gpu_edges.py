@@ -92,6 +92,8 @@ def test_head_error_sizes(n, c, hw):
     (5, 7, 7, 48, 80, 3, 2, 1),      # five lanes per pixel, strided borders
     (40, 28, 28, 32, 160, 3, 1, 1),  # two channel slabs, the second ragged; many slices
     (2, 11, 6, 16, 32, 5, 1, 2),     # two border rows and columns on each side
+    (1, 32, 32, 16, 16, 3, 1, 1),    # short pixel blocks: a slice per output row
+    (2, 30, 17, 64, 64, 3, 1, 1),    # short blocks, the last one of an image ragged
 ])
 def test_weight_gradient_finish(n, h, w, c_in, c_out, k, stride, pad):
     d = oracle.ConvDesc(n, h, w, c_in, c_out, k, k, stride, pad)
