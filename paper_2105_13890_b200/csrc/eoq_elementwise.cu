@@ -684,6 +684,8 @@ prescale_fused_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, cons
 {
     if (gridDim.x <= 148) ptx::grid_dep_launch();   // (its successor may come up beside it)
     __shared__ unsigned go_s;
+    __shared__ uint32_t max_s;
+    __shared__ long long total_s[2];
     gamma_c = load_gamma(gamma_c, gamma_dev, dev);
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -738,17 +740,22 @@ prescale_fused_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, cons
         if (!ok) atomicOr(&dev->status, EOQ_DEV_TIMEOUT);
         __threadfence();
         go_s = ok;
+        max_s = *reinterpret_cast<volatile unsigned *>(&dev->absmax_u32);
+        total_s[0] = *reinterpret_cast<volatile long long *>(&dev->sum0);
+        total_s[1] = *reinterpret_cast<volatile long long *>(&dev->sum1);
     }
     __syncthreads();
     if (!go_s) return;
-    const uint32_t M = *reinterpret_cast<volatile unsigned *>(&dev->absmax_u32) * (uint32_t)abs(gamma_c);
+    bool last = false;
+    if (threadIdx.x == 0) last = last_reader(dev);   // the last block to have read the cells clears them at its end
+    const uint32_t M = max_s * (uint32_t)abs(gamma_c);
     const int t = M ? round_log2_u32(M) : 7;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const int p_in = *e0_exp - 7;
         *e3_exp = M ? p_in + t - 7 : p_in;
         if (!M) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-        if (sum_e1) *sum_e1 = *reinterpret_cast<volatile long long *>(&dev->sum0);
-        if (sum_e1x2) *sum_e1x2 = *reinterpret_cast<volatile long long *>(&dev->sum1);
+        if (sum_e1) *sum_e1 = total_s[0];
+        if (sum_e1x2) *sum_e1x2 = total_s[1];
     }
     // same rounding as prescale_apply_kernel: R(gamma * e1 * 2^(7-t)) with one FMA
     NextHead nh;
@@ -764,7 +771,7 @@ prescale_fused_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, cons
         for (int q = 0; q < 4; ++q) c3[q] = next_head_codes(nh, e1w[u][q]);
         reinterpret_cast<int4 *>(e3)[i] = make_int4((int)c3[0], (int)c3[1], (int)c3[2], (int)c3[3]);
     }
-    if (last_block_done(dev)) {
+    if (last) {
         dev->absmax_u32 = 0;
         dev->sum0 = 0;
         dev->sum1 = 0;

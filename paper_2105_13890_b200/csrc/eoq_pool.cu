@@ -286,6 +286,7 @@ maxpool_bwd_quad_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, cons
                         const int32_t *next_gamma, int8_t *__restrict__ e3, int32_t *e3_exp, long long *sum_e1, DeviceState *dev)
 {
     ptx::grid_dep_wait_launch_small();
+    if (kPass == 0 && kNext && blockIdx.x == 0 && threadIdx.x == 0 && sum_e1) *sum_e1 = 0;   // pass 1 adds to it
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
     const bool live = i < items;
     const int groups = c / 16;
@@ -371,6 +372,8 @@ maxpool_bwd_quad_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, cons
             sum_s = 0;
         }
         __syncthreads();
+        bool last = false;
+        if (threadIdx.x == 0) last = last_reader(dev);   // the last block to have read the maxima clears them at its end
         const uint32_t M = m_s[0];
         const int t = M ? round_log2_u32(M) : 7;
         NextHead nh = {};
@@ -418,14 +421,11 @@ maxpool_bwd_quad_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, cons
             s1 = __reduce_add_sync(0xffffffffu, s1);
             if ((threadIdx.x & 31) == 0 && s1) atomicAdd(&sum_s, s1);
             __syncthreads();
-            if (threadIdx.x == 0 && sum_s) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)(long long)sum_s);
+            if (threadIdx.x == 0 && sum_s) atomicAdd(reinterpret_cast<unsigned long long *>(sum_e1), (unsigned long long)(long long)sum_s);
         }
-        if (last_block_done(dev)) {
+        if (last) {
             dev->absmax_u32 = 0;
-            if (kNext) {
-                dev->absmax_u64 = 0;
-                if (sum_e1) *sum_e1 = (long long)atomicExch(reinterpret_cast<unsigned long long *>(&dev->sum0), 0ull);
-            }
+            if (kNext) dev->absmax_u64 = 0;
         }
     }
 }
