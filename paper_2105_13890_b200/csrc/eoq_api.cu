@@ -1245,7 +1245,7 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     }
     // The classes write disjoint pixels, so their GEMMs are independent: with more than one class and branch streams
     // at hand they are issued side by side (fork on `s`, one stream per class, joins before Q_e), each with a
-    // share of the CTAs in proportion to its taps, instead of one after the other at full width.
+    // share of the CTAs in proportion to its work, instead of one after the other at full width.
     int total_taps = 0, live_classes = 0;
     for (int py = 0; py < d.stride && py < d.h; ++py)
         for (int px = 0; px < d.stride && px < d.w; ++px) {
@@ -1334,7 +1334,8 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             cudaStream_t cs = s;
             int ctas = h->gemm_ctas;
             if (side_by_side) {
-                ctas = (int)((long long)h->gemm_ctas * (nh * nw) / total_taps);
+                // a tile costs its taps and, about half of one, its sums: by taps alone the class of one tap ended last
+                ctas = (int)((long long)h->gemm_ctas * (2 * nh * nw + 1) / (2 * total_taps + live_classes));
                 if (ctas < 1) ctas = 1;
                 if (class_no > 0) {
                     const int k = (class_no - 1) % kClassBranches;
