@@ -11,11 +11,12 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from importlib.machinery import EXTENSION_SUFFIXES
 from typing import Optional, Sequence
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libeoq.so")
-BIND_PATH = os.path.join(_HERE, "_eoqbind.so")
+BIND_PATH = os.path.join(_HERE, "_eoqbind" + EXTENSION_SUFFIXES[0])   # of this interpreter
 
 EOQ_OK, EOQ_ERR_BAD_ARG, EOQ_ERR_ALIGNMENT, EOQ_ERR_UNSUPPORTED, EOQ_ERR_WORKSPACE, EOQ_ERR_RANGE, EOQ_ERR_CUDA = range(7)
 EOQ_DEV_TIMEOUT, EOQ_DEV_NONFINITE, EOQ_DEV_SQ_ZERO, EOQ_DEV_RANGE = 1, 2, 4, 8

@@ -1,4 +1,7 @@
 """The native part of the Python binding marshals arguments like the C ABI expects them (no GPU: calls that are refused)."""
+import os
+import sysconfig
+
 import pytest
 
 from paper_2105_13890_b200 import build, eoq
@@ -40,3 +43,18 @@ def test_statuses_and_argument_errors():
         eoq.eoq_conv_dgrad(0, m, m, m, m, m, m, stream=0)
     with pytest.raises(ValueError):
         eoq.eoq_update_dev(0, [m, m], [m], [m, m], 1, -6, 0, 1, m, stream=0)
+
+
+def test_module_is_the_one_of_this_interpreter(tmp_path, monkeypatch):
+    """A module built for another interpreter, however new, neither counts as built nor is loaded."""
+    tag = sysconfig.get_config_var("EXT_SUFFIX")
+    assert "cpython" in tag and os.path.basename(build.BIND) == "_eoqbind" + tag
+    assert eoq.BIND_PATH == build.BIND and os.path.samefile(eoq.native().__file__, build.BIND)
+    # one for another interpreter lies beside the library (newer than the sources): this one's is built all the same
+    os.symlink(build.LIB, tmp_path / "libeoq.so")
+    other = tmp_path / "_eoqbind.so"
+    other.write_bytes(b"built for another interpreter")
+    monkeypatch.setattr(build, "HERE", str(tmp_path))
+    monkeypatch.setattr(build, "BIND", str(tmp_path / os.path.basename(build.BIND)))
+    assert build.build_bind() == build.BIND and os.path.getsize(build.BIND) > 1000
+    assert other.read_bytes() == b"built for another interpreter"
