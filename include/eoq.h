@@ -476,12 +476,14 @@ EOQ_API int eoq_profile_gemm_only(eoq_handle_t handle, int on);
 typedef void (*eoq_reduce_fn)(void *user, void *device_buffer, size_t count, int dtype, int op, void *stream);
 EOQ_API int eoq_set_reduce_hook(eoq_handle_t handle, eoq_reduce_fn fn, void *user);
 
-/* Caps the CTAs (one per SM) that the GEMM launches of this handle use; 0 = one per SM of the device (the
- * default).  Every GEMM kernel is persistent: with fewer CTAs a launch walks more tiles per CTA and leaves the
- * other SMs free, so that GEMMs issued through two handles on two streams run side by side instead of one after
- * the other (in the training step of Sec. 3.2.1 the error back-propagation of a layer and its weight gradient are
- * independent once e3 exists).  Results do not depend on the setting.  Host-side state only; applies to the calls
- * made after it. */
+/* Caps the CTAs (one per SM) that each GEMM call of this handle uses; 0 = one per SM of the device (the default).
+ * With fewer CTAs each of them does more of the work (forward and dgrad kernels walk more tiles, a weight gradient
+ * splits its pixels into fewer ranges) and the other SMs are left free, so that GEMMs issued through two handles on
+ * two streams run side by side instead of one after the other (in the training step of Sec. 3.2.1 the error
+ * back-propagation of a layer and its weight gradient are independent once e3 exists).  A call never takes fewer CTAs
+ * than it has parts that need one each: a tile of the gradient (times the pixel ranges that keep int32 partial sums
+ * exact), a residue class of a strided dgrad.  Results do not depend on the setting.  Host-side state only; applies
+ * to the calls made after it. */
 EOQ_API int eoq_set_gemm_ctas(eoq_handle_t handle, int ctas);
 
 /*

@@ -144,7 +144,7 @@ class ChainedStep:
         self.h_sides = [eoq.eoq_create(dev_index) for _ in range(side_streams + 1)]   # the last: finishing and updating stages
         self.workspace_sides = [torch.empty(ws, dtype=torch.uint8, device=dev) for _ in range(side_streams)]
         # a third of the SMs for each of the weight-gradient GEMMs, so that the error chain finds free ones (ResNet-18 step at
-        # batch 64: 1588 us with all SMs, 1512 with half, 1502 with a third; fewer changes little)
+        # batch 64: 1576 us with all SMs, 1502 with half, 1474 with a third, 1480 with a quarter; at batch 13: 769, 727, 717, 715)
         third = torch.cuda.get_device_properties(dev).multi_processor_count // 3
         for hs in self.h_sides:
             eoq.eoq_set_gemm_ctas(hs, third)

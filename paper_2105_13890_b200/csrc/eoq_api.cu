@@ -501,9 +501,7 @@ bool plan_wgrad(WgradParams &p, const eoq_conv_desc_t &d, const Geometry &g, int
     // together.  In SM cycles, as measured: a TMA row 3.1, an MMA 57 to 128, a column of an M tile in the epilogue 8; a slice
     // is written and read back at 2,500 bytes per cycle of the whole device.  With 64-bit atomics into one buffer and at
     // least 8 stages per CTA, the 1024 -> 256 layer of 14 x 14 pixels took 24.4 us at batch 32 (the atomics 17 of them).
-    // Twice the CTAs asked for, one per SM at most: the caps that callers set halve a GEMM that has a neighbour on the other
-    // SMs, and this kernel also ends the backward pass, alone.
-    const int cap = 2 * ctas < kWgradTargetCtas ? 2 * ctas : kWgradTargetCtas;
+    const int cap = ctas < kWgradTargetCtas ? ctas : kWgradTargetCtas;
     double best = 0;
     int best_splits = 0;
     for (int cuts = 1; cuts <= 8; cuts = cuts < 4 ? cuts + 1 : cuts * 2) {
@@ -598,8 +596,8 @@ bool plan_wgrad_rows(WgradRowsPlan &pl, const eoq_conv_desc_t &d, const Geometry
         break;
     }
     if (!pl.num_stages) return false;
-    // as plan_wgrad: twice the CTAs asked for, one per SM at most; a row adds at most wo * 127 * 127 to an int32 sum
-    const int cap = 2 * ctas < kWgradTargetCtas ? 2 * ctas : kWgradTargetCtas, rows = d.n * g.ho, exact = 130000 / g.wo;
+    // a row adds at most wo * 127 * 127 to an int32 sum
+    const int cap = ctas < kWgradTargetCtas ? ctas : kWgradTargetCtas, rows = d.n * g.ho, exact = 130000 / g.wo;
     int per = (rows + cap - 1) / cap;
     if (per > exact) per = exact;
     pl.rows_per_split = per;

@@ -97,7 +97,8 @@ class TrainStep:
         self.h_sides = [eoq.eoq_create(dev_index) for _ in range(side_streams)]
         self.workspace_sides = [torch.empty(ws, dtype=torch.uint8, device=self.dev) for _ in range(side_streams)]
         # the weight-gradient GEMMs of the side streams take half of the SMs each: two of them then run side by side
-        # (and beside the helper kernels of the main chain) instead of one after the other
+        # (and beside the helper kernels of the main chain) instead of one after the other (ResNet-18 step at batch 64: 1420 us
+        # with all SMs, 1385 with half, 1412 with a third)
         half = torch.cuda.get_device_properties(self.dev).multi_processor_count // 2
         for hs in self.h_sides:
             eoq.eoq_set_gemm_ctas(hs, half)

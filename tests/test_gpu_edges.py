@@ -279,7 +279,7 @@ def test_prepared_weights(d):
 ], ids=lambda v: f"n{v.n}_{v.h}x{v.w}_c{v.c_out}_k{v.kh}s{v.stride}" if isinstance(v, oracle.ConvDesc) else None)
 @pytest.mark.parametrize("ctas", [0, 1])
 def test_first_layer_weight_gradient(d, m, ctas):
-    """Window rows in a ring, over every wrap and restart; with two CTAs each walks many output rows."""
+    """Window rows in a ring, over every wrap and restart; one CTA alone walks all output rows."""
     x, e3 = synth.int8_uniform((d.n, d.h, d.w, d.c_in), 1630, 0), synth.normal_codes((d.n, d.ho, d.wo, d.c_out), 1630, 1)
     want = oracle.conv_wgrad_acc(d, e3, x, 0)
     gd, h = eoq.conv_desc(d.n, d.h, d.w, d.c_in, d.c_out, d.kh, d.kw, d.stride, d.pad, m), eoq.eoq_create(0)
@@ -291,4 +291,27 @@ def test_first_layer_weight_gradient(d, m, ctas):
     for _ in range(2):
         eoq.eoq_conv_wgrad(h, gd, G.dev(e3), G.dev(np.array([-9], dtype=np.int32)), xm, 0, g, pg, acc, ws)
         assert eoq.eoq_last_status(h) == 0 and np.array_equal(G.host(acc), want)
+    eoq.eoq_destroy(h)
+
+
+@pytest.mark.parametrize("d,m", [
+    (oracle.ConvDesc(4, 24, 24, 32, 32, 3, 3, 1, 1), 0),   # patch kernel
+    (oracle.ConvDesc(8, 28, 28, 64, 64, 1, 1, 2, 0), 0),   # one tap at a time
+    (oracle.ConvDesc(3, 32, 40, 8, 32, 7, 7, 2, 3), 5),    # window rows in a ring
+], ids=["patch", "taps", "rows"])
+@pytest.mark.parametrize("ctas", [1, 5, 11])
+def test_weight_gradient_keeps_to_the_cta_cap(d, m, ctas):
+    """A gradient of one tile takes as many CTAs as it leaves slices: no more than eoq_set_gemm_ctas allows, in every kernel."""
+    x, e3 = synth.int8_uniform((d.n, d.h, d.w, d.c_in), 1640, 0), synth.normal_codes((d.n, d.ho, d.wo, d.c_out), 1640, 1)
+    want, p, _ = oracle.sq_int(oracle.conv_wgrad_acc(d, e3, x, 0), -9 - 7)
+    gd, h = eoq.conv_desc(d.n, d.h, d.w, d.c_in, d.c_out, d.kh, d.kw, d.stride, d.pad, m), eoq.eoq_create(0)
+    xm, e3_d, pe = G.dev(np.pad(x, ((0, 0), (0, 0), (m, m), (0, 0)))), G.dev(e3), G.dev(np.array([-9], dtype=np.int32))
+    ws, g, pg = G.workspace(gd, eoq.EOQ_PASS_WGRAD), G.zeros(want.shape, torch.int8), G.zeros(1, torch.int32)
+    assert eoq.eoq_conv_wgrad_gemm(h, gd, e3_d, pe, xm, ws) > 11   # without a cap there are more
+    eoq.eoq_set_gemm_ctas(h, ctas)
+    parts = eoq.eoq_conv_wgrad_gemm(h, gd, e3_d, pe, xm, ws)
+    assert 1 <= parts <= ctas
+    eoq.eoq_wgrad_finish(h, [gd], [e3_d], [pe], [None], [g], [pg], [ws], [parts])
+    assert np.array_equal(G.host(g).astype(np.int32), want) and pg.item() == p
+    assert eoq.eoq_last_status(h) == 0
     eoq.eoq_destroy(h)
