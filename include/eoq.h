@@ -439,12 +439,12 @@ EOQ_API int eoq_last_status(eoq_handle_t handle, void *stream, unsigned *bits);
 #define EOQ_PROF_WGRAD 2         /* the weight-gradient GEMM kernel */
 #define EOQ_PROF_ERR_HEAD 3      /* eoq_err_prescale (one kernel; two for tensors beyond the one-kernel capacity) */
 #define EOQ_PROF_DGRAD_AUX 4     /* Q_e phase 2; weight transpose (only layers with fewer than 32 output channels) */
-#define EOQ_PROF_WGRAD_AUX 5     /* slice sum + b1 term + Q_g behind the weight-gradient GEMM (and the memset in front of it) */
+#define EOQ_PROF_WGRAD_AUX 5     /* slice sum + b1 term + Q_g behind the weight-gradient GEMM */
 #define EOQ_PROF_FWD_AUX 6       /* b1 weight table, weight row padding (eoq_weight_prep, or per call without it) */
 #define EOQ_PROF_OTHER 7         /* eoq_quantize, eoq_bn_fwd, eoq_bn_bwd */
 #define EOQ_PROF_UPDATE 8        /* eoq_update */
 #define EOQ_PROF_INPUT_Q 9       /* eoq_quantize_image */
-#define EOQ_PROF_WGRAD_TAPS 10   /* b1 error sums of the weight gradient */
+#define EOQ_PROF_WGRAD_TAPS 10   /* b1 error sums of the weight gradient (none for a layer without a bias in front) */
 #define EOQ_PROF_GLUE 11         /* eoq_aux_*: pooling, error join, float head, scalar updates */
 #define EOQ_PROF_KINDS 12
 EOQ_API int eoq_profile_start(eoq_handle_t handle);

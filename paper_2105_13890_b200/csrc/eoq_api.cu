@@ -1470,6 +1470,22 @@ static FinishItem finish_item(const eoq_conv_desc_t &d, const Geometry &g, const
     return it;
 }
 
+// b1 error sums, sums and Q_g of up to kFinishChunk layers whose GEMMs are in front on the stream.
+static int finish_items(Handle *h, const FinishItem *items, int num, cudaStream_t s)
+{
+    FinishBatch b;
+    plan_finish(b, items, num, h->sm_count, h->hook);
+    if (b.tap_first[num] > 0) {
+        ProfScope prof(h, EOQ_PROF_WGRAD_TAPS, s);
+        count_launches(h, 1);
+        const cudaError_t e = launch_finish_taps(b, s);
+        if (e != cudaSuccess) return record(h, e);
+    }
+    ProfScope prof(h, EOQ_PROF_WGRAD_AUX, s);
+    count_launches(h, h->hook.fn ? 2 + num : 2);
+    return record(h, launch_finish_sums(b, &h->dev->status, s, h->hook));
+}
+
 // Weight gradient behind eoq_conv_wgrad and eoq_conv_wgrad_dev: b1 is the host code b1_c, or the code at b1_dev.
 // num_parts_out (eoq_conv_wgrad_gemm): the GEMM alone; the sums stay in the workspace for eoq_wgrad_finish and
 // *num_parts_out tells it how many int32 slices there are.
@@ -1497,9 +1513,7 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     auto finish = [&](int num_parts) -> int {
         FinishItem it = finish_item(d, g, w, e3, e3_exp, b1_c, b1_dev, gq, g_exp, num_parts);
         it.copy_out = reinterpret_cast<long long *>(acc_dump);
-        ProfScope prof_q(h, EOQ_PROF_WGRAD_AUX, s);
-        count_launches(h, finish_launches(&it, 1, h->hook));
-        return record(h, launch_wgrad_finish(&it, 1, &h->dev->status, h->sm_count, s, h->hook));
+        return finish_items(h, &it, 1, s);
     };
 
     WgradPatchPlan wp;
@@ -1623,10 +1637,8 @@ extern "C" int eoq_wgrad_finish(eoq_handle_t handle, int num, const eoq_conv_des
             items[k] = finish_item(d, g, wgrad_space(d, g, workspace[base + k]), e3[base + k], e3_exp[base + k], 0, b1_c[base + k],
                                    gq[base + k], g_exp[base + k], num_parts[base + k]);
         }
-        ProfScope prof(h, EOQ_PROF_WGRAD_AUX, s);
-        count_launches(h, finish_launches(items, count, h->hook));
-        const cudaError_t e = launch_wgrad_finish(items, count, &h->dev->status, h->sm_count, s, h->hook);
-        if (e != cudaSuccess) return record(h, e);
+        const int st = finish_items(h, items, count, s);
+        if (st != EOQ_OK) return st;
     }
     return EOQ_OK;
 }

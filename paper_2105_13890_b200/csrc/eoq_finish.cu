@@ -439,55 +439,51 @@ static void plan_finish_item(FinishItem &it, int sm_count, bool alone)
     it.sq_blocks = (int)(qb < 1 ? 1 : (qb > cap ? cap : qb));
 }
 
-int finish_launches(const FinishItem *items, int num, const ReduceHook &hook)
+void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, const ReduceHook &hook)
 {
-    int n = 0;
-    for (int base = 0; base < num; base += kFinishChunk) {
-        bool taps = false;
-        for (int k = base; k < num && k < base + kFinishChunk; ++k) taps |= items[k].use_b1 != 0;
-        n += 2 + (taps ? 1 : 0) + (hook.fn ? 1 : 0);
+    b.num = num;
+    b.tap_first[0] = b.fin_first[0] = b.sq_first[0] = 0;
+    for (int k = 0; k < num; ++k) {
+        FinishItem &it = b.item[k];
+        it = items[k];
+        it.keep_sums = hook.fn != nullptr;
+        plan_finish_item(it, sm_count, num == 1);
+        b.tap_first[k + 1] = b.tap_first[k] + it.tap_blocks;
+        b.fin_first[k + 1] = b.fin_first[k] + it.fin_blocks;
+        b.sq_first[k + 1] = b.sq_first[k] + it.sq_blocks;
     }
-    return n;
 }
 
-cudaError_t launch_wgrad_finish(const FinishItem *items, int num, unsigned *status, int sm_count, cudaStream_t s, const ReduceHook &hook)
+cudaError_t launch_finish_taps(const FinishBatch &b, cudaStream_t s)
 {
-    for (int base = 0; base < num; base += kFinishChunk) {
-        FinishBatch b;
-        b.num = num - base < kFinishChunk ? num - base : kFinishChunk;
-        b.tap_first[0] = b.fin_first[0] = b.sq_first[0] = 0;
-        int max_sets = 1;
-        for (int k = 0; k < b.num; ++k) {
-            FinishItem &it = b.item[k];
-            it = items[base + k];
-            it.keep_sums = hook.fn != nullptr;
-            plan_finish_item(it, sm_count, num == 1);
-            b.tap_first[k + 1] = b.tap_first[k] + it.tap_blocks;
-            b.fin_first[k + 1] = b.fin_first[k] + it.fin_blocks;
-            b.sq_first[k + 1] = b.sq_first[k] + it.sq_blocks;
-            const int sets = (1 + it.bc.nrc) * (1 + it.bc.ncc);   // at least (1 + border rows)(1 + border columns)
-            if (it.use_b1 && sets > max_sets) max_sets = sets;
-        }
-        if (b.tap_first[b.num] > 0) {
-            const size_t smem = sizeof(int32_t) * max_sets * kClassSlab;
-            if (smem > 48 * 1024) {   // at most 64 classes: 130 sets
-                const cudaError_t e = cudaFuncSetAttribute(finish_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
-                if (e != cudaSuccess) return e;
-            }
-            launch_chained(finish_taps_kernel, b.tap_first[b.num], kThreads, smem, s, b);
-        }
-        launch_chained(finish_sums_kernel, b.fin_first[b.num], kThreads, 0, s, b);
-        if (hook.fn)
-            // replicas (one layer per call): local sums, b1 term included (it is linear in the error) -> all-reduce ->
-            // maximum of the global sums; the copy for the caller is taken from the global sums as well
-            for (int k = 0; k < b.num; ++k) {
-                const FinishItem &it = b.item[k];
-                hook(it.acc, (size_t)it.n, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
-                launch_chained(finish_max_kernel, it.fin_blocks, kThreads, 0, s, it.acc, (size_t)it.n, it.max_cell);
-                if (it.copy_out) cudaMemcpyAsync(it.copy_out, it.acc, (size_t)it.n * sizeof(long long), cudaMemcpyDeviceToDevice, s);
-            }
-        launch_chained(finish_code_kernel, b.sq_first[b.num], kThreads, 0, s, b, status);
+    int max_sets = 1;
+    for (int k = 0; k < b.num; ++k) {
+        const FinishItem &it = b.item[k];
+        const int sets = (1 + it.bc.nrc) * (1 + it.bc.ncc);   // at least (1 + border rows)(1 + border columns)
+        if (it.use_b1 && sets > max_sets) max_sets = sets;
     }
+    const size_t smem = sizeof(int32_t) * max_sets * kClassSlab;
+    if (smem > 48 * 1024) {   // at most 64 classes: 130 sets
+        const cudaError_t e = cudaFuncSetAttribute(finish_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
+        if (e != cudaSuccess) return e;
+    }
+    launch_chained(finish_taps_kernel, b.tap_first[b.num], kThreads, smem, s, b);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_finish_sums(const FinishBatch &b, unsigned *status, cudaStream_t s, const ReduceHook &hook)
+{
+    launch_chained(finish_sums_kernel, b.fin_first[b.num], kThreads, 0, s, b);
+    if (hook.fn)
+        // replicas (one layer per call): local sums, b1 term included (it is linear in the error) -> all-reduce ->
+        // maximum of the global sums; the copy for the caller is taken from the global sums as well
+        for (int k = 0; k < b.num; ++k) {
+            const FinishItem &it = b.item[k];
+            hook(it.acc, (size_t)it.n, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
+            launch_chained(finish_max_kernel, it.fin_blocks, kThreads, 0, s, it.acc, (size_t)it.n, it.max_cell);
+            if (it.copy_out) cudaMemcpyAsync(it.copy_out, it.acc, (size_t)it.n * sizeof(long long), cudaMemcpyDeviceToDevice, s);
+        }
+    launch_chained(finish_code_kernel, b.sq_first[b.num], kThreads, 0, s, b, status);
     return cudaGetLastError();
 }
 

@@ -448,7 +448,7 @@ struct FinishItem {
     eoq_conv_desc_t d;
     BorderClasses bc;
     int ho, wo, num_parts;
-    // filled by launch_wgrad_finish
+    // filled by plan_finish
     int rows_per_block, tap_grid_x, tap_blocks, groups, fin_blocks, sq_blocks;
     int direct;                    // the sums are formed twice instead of being written and read back
     int keep_sums;                 // reduce hook: the sums are completed by an all-reduce before their maximum is taken
@@ -458,8 +458,11 @@ struct FinishBatch {
     int tap_first[kFinishChunk + 1], fin_first[kFinishChunk + 1], sq_first[kFinishChunk + 1];
     FinishItem item[kFinishChunk];
 };
-cudaError_t launch_wgrad_finish(const FinishItem *items, int num, unsigned *status, int sm_count, cudaStream_t s, const ReduceHook &hook);
-int finish_launches(const FinishItem *items, int num, const ReduceHook &hook);
+// Lays out the launches of up to kFinishChunk items; then, in this order on one stream, the b1 error sums (only where an item
+// has a b1 term: tap_first[num] > 0) and the sums with Q_g (two kernels, a third per item under a reduce hook).
+void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, const ReduceHook &hook);
+cudaError_t launch_finish_taps(const FinishBatch &b, cudaStream_t s);
+cudaError_t launch_finish_sums(const FinishBatch &b, unsigned *status, cudaStream_t s, const ReduceHook &hook);
 
 // Batch normalisation behind the convolution (comparison case, eoq_bn.cu): per-channel record in the workspace
 struct BnChannel {

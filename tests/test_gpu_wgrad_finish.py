@@ -74,3 +74,26 @@ def test_a_zero_error_gives_zero_gradients_and_the_flag():
     assert not G.host(g).any() and pg.item() == -19
     assert eoq.eoq_last_status(hd) == eoq.EOQ_DEV_SQ_ZERO
     G.status_clear()
+
+
+@pytest.mark.parametrize("b1", [None, -3])
+def test_profile_groups_of_a_weight_gradient(b1):
+    """The GEMM, the b1 error sums and what follows them are timed as kinds of their own, per call and in two parts."""
+    d, e3, x0, _, g_o, pg_o = make((2, 12, 12, 32, 32, 3, 1, 1, b1), 9100)
+    gd, h = G.gdesc(d), eoq.eoq_create(0)
+    e3_d, x_d, pe = G.dev(e3), G.dev(x0), G.dev(np.array([-12], dtype=np.int32))
+    b1_d = None if b1 is None else G.dev(np.array([b1], dtype=np.int32))
+    ws, g, pg = G.workspace(gd, eoq.EOQ_PASS_WGRAD), G.zeros(g_o.shape, torch.int8), G.zeros(1, torch.int32)
+    kinds = dict.fromkeys(eoq.EOQ_PROF_NAMES, 0)
+    kinds.update(wgrad_gemm=2, wgrad_aux=2, wgrad_taps=0 if b1 is None else 2)
+    before = eoq.eoq_launch_count(h)
+    eoq.eoq_profile_start(h)
+    eoq.eoq_conv_wgrad_dev(h, gd, e3_d, pe, x_d, b1_d, g, pg, ws)
+    parts = eoq.eoq_conv_wgrad_gemm(h, gd, e3_d, pe, x_d, ws)
+    eoq.eoq_wgrad_finish(h, [gd], [e3_d], [pe], [b1_d], [g], [pg], [ws], [parts])
+    n, ms = eoq.eoq_profile_stop(h)
+    assert dict(zip(eoq.EOQ_PROF_NAMES, n)) == kinds
+    assert all((t > 0) == (k > 0) for k, t in zip(n, ms))
+    assert eoq.eoq_launch_count(h) - before == 6 + kinds["wgrad_taps"]
+    assert np.array_equal(G.host(g), g_o) and pg.item() == pg_o and eoq.eoq_last_status(h) == 0
+    eoq.eoq_destroy(h)
