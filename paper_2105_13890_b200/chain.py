@@ -259,6 +259,8 @@ class ChainedStep:
 
         def update(us, hh, last) -> None:
             us = sorted(us, key=lambda u: u.index)
+            # a part is a run of the whole list: pending units come from consecutive blocks, whatever their stages are called
+            assert [u.index for u in us] == list(range(us[0].index, us[0].index + len(us)))
             eoq.eoq_update_part(hh, us[0].index, last, [u.w for u in us], [u.g for u in us], [u.g_exp for u in us], self.lr_mant,
                                 self.lr_exp, self.round_mode, self.seed, self.step_dev)
             eoq.eoq_weight_prep(hh, [u.desc for u in us], [u.w for u in us], [u.prep for u in us])

@@ -2,6 +2,8 @@
 scalar and weight updates) against the oracle's closed-loop step: every intermediate tensor of every unit, the
 head's results and every updated parameter, bit for bit (the reported loss within 1e-6 relative: its logarithm is
 each side's library routine)."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -95,6 +97,31 @@ def test_chained_step_matches_the_oracle_on_every_tensor(name, batch, mode):
         u = next(x for x, ou in zip(st.units, net.units) if ou.name == uname)
         assert host(u.sgrad[which[w]]).tolist() == [code, p], (uname, w)
     compare_parameters(st, net, "after the step")
+
+
+@pytest.mark.parametrize("order", [(0, 0, 0, 1, 1, 1, 2, 2, 2), (0, 1, 0, 2, 1, 1, 0, 2, 2)], ids=["stages", "interleaved"])
+def test_parts_of_the_update_count_like_the_whole(order):
+    """Stochastic rounding counts the tensors of the whole network: stages that are updated one by one beside the backward pass,
+    consecutive or interleaved, give the weights of one update at the end."""
+    wl = workloads.resnet20(2)
+    names = {f"stage{b // 3 + 1}.{b % 3}": f"s{order[b]}.{b}" for b in range(9)}
+    layers = [l if l.name == "stem" else dataclasses.replace(l, name=names[l.name.rsplit(".", 1)[0]] + "." + l.name.rsplit(".", 1)[1])
+              for l in wl.layers]
+    wl = dataclasses.replace(wl, layers=layers)
+    steps = [ChainedStep(wl, eoq.eoq_create(0), lr_mant=3, lr_exp=-4, classes=10, round_mode=eoq.EOQ_ROUND_STOCHASTIC, seed=SEED,
+                         finish_together=together) for together in (True, True, False)]
+    start = [host(u.w) for u in steps[0].units]
+    for k in range(2):
+        for st, overlap in zip(steps, (True, False, False)):
+            feed(st, k)
+            st.run(overlap)
+    torch.cuda.synchronize()
+    assert any((host(u.w) != w0).any() for u, w0 in zip(steps[0].units, start))
+    for st in steps[:2]:
+        assert st.step_dev.item() == steps[2].step_dev.item() == 2
+        for u, v in zip(st.units, steps[2].units):
+            assert np.array_equal(host(u.w), host(v.w)), u.layer.name
+            assert np.array_equal(host(u.scal), host(v.scal)), u.layer.name
 
 
 def test_closed_loop_step_at_the_benchmark_size():
