@@ -173,13 +173,6 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
 
 // ------------------------------------------------------------------ scalar parameters (Sec. 3.2.3 on a single value)
 
-__device__ __forceinline__ unsigned long long mix64_aux(unsigned long long z)
-{
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
 // One thread per scalar: g = Q_g({total}) (SQ of a single value), u = Q_u(lr g), theta <- Q(theta - u) saturated to 16 bits.
 __global__ void scalar_update_kernel(const __grid_constant__ ScalarBatch b, int32_t lr_mant, int32_t lr_exp, int stochastic,
                                      unsigned long long seed, const unsigned long long *step_dev, unsigned long long step)
@@ -216,9 +209,7 @@ __global__ void scalar_update_kernel(const __grid_constant__ ScalarBatch b, int3
             if (!stochastic) {
                 next = rne_shr64(v, s);
             } else {
-                unsigned long long key = mix64_aux(seed + 0x9E3779B97F4A7C15ull * (step + 1));
-                key = mix64_aux(key + 0x9E3779B97F4A7C15ull * ((unsigned long long)it.tensor_id + 1));
-                const unsigned long long r = mix64_aux(key + 0x9E3779B97F4A7C15ull) & ((1ull << s) - 1ull);  // element index 0
+                const unsigned long long r = rounding_bits(rounding_key(seed, step, (unsigned long long)it.tensor_id), 0) & ((1ull << s) - 1ull);
                 next = (v + (long long)r) >> s;
             }
         }

@@ -38,6 +38,12 @@ __device__ __forceinline__ uint32_t pack4_sat(int c0, int c1, int c2, int c3)
     return r;
 }
 
+// the same of values whose low bytes are the codes already
+__device__ __forceinline__ uint32_t pack4(int a, int b, int c, int d)
+{
+    return (uint32_t)(a & 0xff) | ((uint32_t)(b & 0xff) << 8) | ((uint32_t)(c & 0xff) << 16) | ((uint32_t)(d & 0xff) << 24);
+}
+
 // byte k of w, sign-extended
 template <int k>
 __device__ __forceinline__ int32_t sbyte(uint32_t w)
@@ -56,12 +62,42 @@ __device__ __forceinline__ int round_log2_u32(uint32_t M)
     return f + (sq >= (1ull << (2 * f + 1)) ? 1 : 0);
 }
 
+// ... of a positive finite float given by its bit pattern
+__device__ __forceinline__ int round_log2_f32bits(uint32_t bits)
+{
+    const int eb = (int)((bits >> 23) & 0xffu);
+    const uint32_t frac = bits & 0x7fffffu;
+    if (eb == 0) return round_log2_u32(frac) - 149;  // subnormal: frac * 2^-149
+    const unsigned long long m = (1ull << 23) | frac;  // M = m * 2^(eb - 150), m in [2^23, 2^24)
+    return (eb - 127) + ((m * m >= (1ull << 47)) ? 1 : 0);
+}
+
 __device__ __forceinline__ int round_log2_u64(unsigned long long M)
 {
     if (M < (1ull << 32)) return round_log2_u32((uint32_t)M);
     int f = 63 - __clzll(M);
     unsigned long long hi = __umul64hi(M, M);  // M^2 >= 2^(2f+1) with 2f+1 >= 65
     return f + (hi >= (1ull << (2 * f + 1 - 64)) ? 1 : 0);
+}
+
+// ------------------------------------------------------------------ stochastic rounding (an extension, not in the paper)
+
+// SplitMix64 output function (Steele, Lea, Flood 2014) as a counter hash.
+__device__ __forceinline__ unsigned long long mix64(unsigned long long z)
+{
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+constexpr unsigned long long kGolden = 0x9E3779B97F4A7C15ull;
+// The bits of one element: a hash of (seed, step, tensor), then of the element's index.
+__device__ __forceinline__ unsigned long long rounding_key(unsigned long long seed, unsigned long long step, unsigned long long tensor)
+{
+    return mix64(mix64(seed + kGolden * (step + 1)) + kGolden * (tensor + 1));
+}
+__device__ __forceinline__ unsigned long long rounding_bits(unsigned long long key, unsigned long long element)
+{
+    return mix64(key + kGolden * (element + 1));
 }
 
 // Code of SQ for an integer a once t = R(log2 max) is known: sat(R(a * 2^(7-t)), -127, 127).

@@ -15,11 +15,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ uint32_t pack4(int a, int b, int c, int d)
-{
-    return (uint32_t)(a & 0xff) | ((uint32_t)(b & 0xff) << 8) | ((uint32_t)(c & 0xff) << 16) | ((uint32_t)(d & 0xff) << 24);
-}
-
 inline int grid_for(size_t work_items, int sm_count, int per_sm = 8)
 {
     size_t blocks = (work_items + kThreads - 1) / kThreads;
@@ -30,16 +25,6 @@ inline int grid_for(size_t work_items, int sm_count, int per_sm = 8)
 }
 
 // ------------------------------------------------------------------ fp32 -> Q / CQ / SQ
-
-// R(log2 M) for a positive finite float given by its bit pattern.
-__device__ __forceinline__ int round_log2_f32bits(uint32_t bits)
-{
-    const int eb = (int)((bits >> 23) & 0xffu);
-    const uint32_t frac = bits & 0x7fffffu;
-    if (eb == 0) return round_log2_u32(frac) - 149;  // subnormal: frac * 2^-149
-    const unsigned long long m = (1ull << 23) | frac;  // M = m * 2^(eb - 150), m in [2^23, 2^24)
-    return (eb - 127) + ((m * m >= (1ull << 47)) ? 1 : 0);
-}
 
 __global__ void absmax_f32_kernel(const float *__restrict__ src, size_t n, DeviceState *dev)
 {

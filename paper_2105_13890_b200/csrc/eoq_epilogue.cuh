@@ -27,11 +27,6 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const Ro
     return false;
 }
 
-__device__ __forceinline__ uint32_t pack4(int a, int b, int c, int d)
-{
-    return (uint32_t)(a & 0xff) | ((uint32_t)(b & 0xff) << 8) | ((uint32_t)(c & 0xff) << 16) | ((uint32_t)(d & 0xff) << 24);
-}
-
 // R(a / 2^7) with ties to even in four integer operations: adding 63 plus the parity of the quotient carries
 // into bit 7 exactly when the remainder exceeds one half, or equals it with an odd quotient.
 __device__ __forceinline__ int32_t rne7(int32_t a) { return (a + 63 + ((a >> 7) & 1)) >> 7; }

@@ -400,15 +400,6 @@ head_update_kernel(const float *__restrict__ dl, const float *__restrict__ poole
 
 // ------------------------------------------------------------------ error handed back by the head
 
-__device__ __forceinline__ int round_log2_f32bits(uint32_t bits)
-{
-    const int eb = (int)((bits >> 23) & 0xffu);
-    const uint32_t frac = bits & 0x7fffffu;
-    if (eb == 0) return round_log2_u32(frac) - 149;
-    const unsigned long long m = (1ull << 23) | frac;
-    return (eb - 127) + ((m * m >= (1ull << 47)) ? 1 : 0);
-}
-
 // max |dpooled| / hw (as float bit patterns; the division is monotonic) into the handle's cell
 __global__ void __launch_bounds__(kThreads) head_error_max_kernel(const float *__restrict__ dpooled, int count, int hw, DeviceState *dev)
 {

@@ -93,15 +93,6 @@ __global__ void __launch_bounds__(kThreads) update_absmax_kernel(const __grid_co
     if (threadIdx.x == 0 && mx) atomicMax(&dev->tensor_absmax[b.tensor_base + k], mx);
 }
 
-// SplitMix64 output function (Steele, Lea, Flood 2014) as a counter hash.
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z)
-{
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-constexpr unsigned long long kGolden = 0x9E3779B97F4A7C15ull;
-
 // What the update of one tensor needs, the same for all its elements.
 struct UpdateRule {
     int mul, sh, half_m1;  // u = sat(R(mul * g / 2^sh))
@@ -120,8 +111,7 @@ __device__ __forceinline__ UpdateRule update_rule(uint32_t M, int g_exp, int lr_
     r.d = (g_exp + lr_exp + t - 7) + 7;
     r.key = 0;
     if (stochastic) {
-        r.key = mix64(seed + kGolden * (step + 1));
-        r.key = mix64(r.key + kGolden * ((unsigned long long)tensor + 1));
+        r.key = rounding_key(seed, step, (unsigned long long)tensor);
     }
     return r;
 }
@@ -329,10 +319,7 @@ __global__ void update_wide_apply_kernel(const __grid_constant__ UpdateBatch b, 
         const int d = (__ldg(T.g_exp) + lr_exp + su) + (k_m - 1);      // exponent of u relative to the master grid
         const long long lim_u = (1ll << (k_u - 1)) - 1, lim_m = (1ll << (k_m - 1)) - 1;
         unsigned long long key = 0;
-        if (stochastic) {
-            key = mix64(seed + kGolden * (step + 1));
-            key = mix64(key + kGolden * ((unsigned long long)(b.tensor_base + k) + 1));
-        }
+        if (stochastic) key = rounding_key(seed, step, (unsigned long long)(b.tensor_base + k));
         const size_t begin = (size_t)(blockIdx.x - b.first_block[k]) * kUpdElemsPerBlock;
         const size_t end = min((size_t)T.n, begin + kUpdElemsPerBlock);
         for (size_t j = begin + threadIdx.x; j < end; j += blockDim.x) {
@@ -351,7 +338,7 @@ __global__ void update_wide_apply_kernel(const __grid_constant__ UpdateBatch b, 
                 if (!stochastic) {
                     next = rne_shr64(v, s);
                 } else {
-                    const unsigned long long r = mix64(key + kGolden * (j + 1)) & ((1ull << s) - 1ull);
+                    const unsigned long long r = rounding_bits(key, j) & ((1ull << s) - 1ull);
                     next = (v + (long long)r) >> s;
                 }
             }
