@@ -1221,7 +1221,7 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     if (!weights_in_place) {
         {
             ProfScope prof(h, EOQ_PROF_DGRAD_AUX, s);
-            e = launch_weight_transpose(w, wt, d.c_out, g.taps, d.c_in, s);
+            e = launch_weight_transpose(w, wt, d.c_out, g.taps, d.c_in, h->sm_count, s);
         }
         if (e != cudaSuccess) return record(h, e);
         count_launches(h, 1);

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "eoq_internal.h"
+
 namespace eoq {
 
 // ------------------------------------------------------------------ integer rounding (Sec. 3.2.2)
@@ -309,11 +311,12 @@ __device__ __forceinline__ int4 ld_shared_128(uint32_t addr)
 // At the start of a kernel of many small blocks: a grid of at most one block per SM leaves room for its successor at once,
 // a larger one brings it up with its last blocks (or where it calls grid_dep_launch).  Brought up beside a full device, the
 // successor only keeps kernels of other streams away: ResNet-18 steps took 648 us at batch 1 without, 610 with it; 1697 us
-// at batch 64 without, 1730 with it in grids of any size.
+// at batch 64 without, 1730 with it in grids of any size.  (The limit is that of the whole part; on a slice of it kernels come
+// up in another order, with the same results.)
 __device__ __forceinline__ void grid_dep_wait_launch_small()
 {
     grid_dep_wait();
-    if (gridDim.x * gridDim.y <= 148) grid_dep_launch();
+    if (gridDim.x * gridDim.y <= kPartSms) grid_dep_launch();
 }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)

@@ -667,7 +667,7 @@ prescale_fused_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, cons
                       int32_t *e3_exp, long long *sum_e1, long long *sum_e1x2, DeviceState *dev, unsigned expected_blocks,
                       uint32_t spin_limit)
 {
-    if (gridDim.x <= 148) ptx::grid_dep_launch();   // (its successor may come up beside it)
+    if (gridDim.x <= kPartSms) ptx::grid_dep_launch();   // (its successor may come up beside it)
     __shared__ unsigned go_s;
     __shared__ uint32_t max_s;
     __shared__ long long total_s[2];
@@ -1076,11 +1076,9 @@ cudaError_t launch_layout_convert(const int8_t *src, int8_t *dst, int n, int c, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_weight_transpose(const int8_t *w, int8_t *wt, int c_out, int taps, int c_in, cudaStream_t s)
+cudaError_t launch_weight_transpose(const int8_t *w, int8_t *wt, int c_out, int taps, int c_in, int sm_count, cudaStream_t s)
 {
-    const size_t total = (size_t)c_out * taps * c_in;
-    int blocks = (int)((total + kThreads - 1) / kThreads);
-    if (blocks > 148 * 16) blocks = 148 * 16;
+    const int blocks = grid_for((size_t)c_out * taps * c_in, sm_count, 16);
     launch_chained(weight_transpose_kernel, blocks, kThreads, 0, s, w, wt, c_out, taps, c_in);
     return cudaGetLastError();
 }

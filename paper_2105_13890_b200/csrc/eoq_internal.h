@@ -10,6 +10,9 @@
 namespace eoq {
 
 constexpr int kMaxTaps = 64;        // kh * kw of any supported filter
+// SMs of the part that the kernels are written for.  Limits that were measured on it are stated with this number; what has to
+// hold on any part (resident grids, CTA caps, grid sizes) goes by the handle's count.
+constexpr int kPartSms = 148;
 constexpr int kTileM = 128;         // GEMM rows per CTA tile (TMEM lanes)
 constexpr int kEpilogueWarps = 16;  // implicit GEMM: four epilogue warps per scheduler hide the latency of the integer chain
 constexpr int kGemmThreads = 128 + 32 * kEpilogueWarps;  // warps 0, 2, 3: TMA, warp 1: MMA + TMEM owner, then the epilogue
@@ -285,7 +288,7 @@ struct WgradPatchPlan {
     DeviceState *dev;
 };
 constexpr int kWgradPatchThreads = 192;  // warp 0 loads, warp 1 MMA + TMEM, warps 2..5 epilogue
-constexpr int kWgradTargetCtas = 148;    // CTAs the split count aims at (one per SM of a 148-SM part; shared memory allows one)
+constexpr int kWgradTargetCtas = kPartSms;  // CTAs the split count aims at (one per SM; shared memory allows one); workspaces hold as many slices
 
 // Weight gradient of a first layer on the filter-row path with its window rows in a ring (eoq_wgrad_rows.cu)
 struct WgradRowsPlan {
@@ -357,7 +360,7 @@ cudaError_t launch_update_wide(const UpdateTensor *t, int num, int32_t lr_mant, 
                                uint64_t seed, uint64_t step, unsigned long long *step_dev, DeviceState *dev, cudaStream_t s);
 cudaError_t launch_layout_convert(const int8_t *src, int8_t *dst, int n, int c, int h, int w, int to_nhwc,
                                   cudaStream_t s);
-cudaError_t launch_weight_transpose(const int8_t *w, int8_t *wt, int c_out, int taps, int c_in, cudaStream_t s);
+cudaError_t launch_weight_transpose(const int8_t *w, int8_t *wt, int c_out, int taps, int c_in, int sm_count, cudaStream_t s);
 // b1 support: class tables of weight sums (forward) and of error sums (weight gradient)
 struct BorderClasses {
     int nlo_h, nhi_h, nrc, nlo_w, nhi_w, ncc;
