@@ -77,8 +77,6 @@ int patch_chunk(int c, int taps)
     return best;
 }
 
-// im2col view of an NHWC int8 tensor [n][h][w][c]: `pixels` consecutive positions of the walk that starts at
-// (lower_w, lower_h) and advances by `stride`, `box_c` channels each.  count_w/h = positions per row/column.
 // View for the filter-row path: the pixel of the walk is a 128-byte window of 8 adjacent 16-channel pixels that
 // starts at memory column (first_col + k * stride) of a row w_mem pixels long, so consecutive windows overlap
 // (the W stride of the view is smaller than its inner extent).  Rows are walked with zero fill above and below.
@@ -99,6 +97,8 @@ bool make_row_window_map(CUtensorMap *map, const void *ptr, int n, int h, int w_
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// im2col view of an NHWC int8 tensor [n][h][w][c]: `pixels` consecutive positions of the walk that starts at
+// (lower_w, lower_h) and advances by `stride`, `box_c` channels each.  count_w/h = positions per row/column.
 bool make_im2col_map(CUtensorMap *map, const void *ptr, int n, int h, int w, int c, int lower_w, int lower_h,
                      int count_w, int count_h, int stride, int box_c, int pixels)
 {
@@ -638,7 +638,7 @@ extern "C" int eoq_create(eoq_handle_t *handle, int device)
     h->hook = ReduceHook{nullptr, nullptr};
     h->num_records = 0;
     h->records = nullptr;
-    h->fork_ev = h->join_ev = nullptr;
+    h->fork_ev = nullptr;
     for (int k = 0; k < kClassBranches; ++k) {
         h->class_branch[k] = nullptr;
         h->class_join[k] = nullptr;
@@ -657,7 +657,6 @@ extern "C" int eoq_create(eoq_handle_t *handle, int device)
     }
     if (e == cudaSuccess) e = cudaMemset(h->dev, 0, sizeof(DeviceState));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->join_ev, cudaEventDisableTiming);
     for (int k = 0; k < kClassBranches && e == cudaSuccess; ++k) {
         e = cudaStreamCreateWithFlags(&h->class_branch[k], cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->class_join[k], cudaEventDisableTiming);
@@ -668,7 +667,6 @@ extern "C" int eoq_create(eoq_handle_t *handle, int device)
             if (h->class_join[k]) cudaEventDestroy(h->class_join[k]);
             if (h->class_branch[k]) cudaStreamDestroy(h->class_branch[k]);
         }
-        if (h->join_ev) cudaEventDestroy(h->join_ev);
         if (h->fork_ev) cudaEventDestroy(h->fork_ev);
         if (h->dev) cudaFree(h->dev);
         delete h;
@@ -688,7 +686,6 @@ extern "C" int eoq_destroy(eoq_handle_t handle)
         if (h->class_join[k]) cudaEventDestroy(h->class_join[k]);
         if (h->class_branch[k]) cudaStreamDestroy(h->class_branch[k]);
     }
-    if (h->join_ev) cudaEventDestroy(h->join_ev);
     if (h->fork_ev) cudaEventDestroy(h->fork_ev);
     if (h->dev) cudaFree(h->dev);
     if (h->records) {

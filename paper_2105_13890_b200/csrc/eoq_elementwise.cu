@@ -1,7 +1,7 @@
 // Bandwidth-bound kernels of the EOQ layer (arXiv 2105.13890): the standalone quantizers Q / CQ / SQ
 // (Sec. 3.2.2), the second phase of the scale quantizer after a convolution, the head of the error
 // chain (Sec. 3.2.1) and small layout helpers.
-// Reductions run warp-shuffle -> one atomic per warp; 16 elements per thread with 128-bit accesses.
+// Reductions run warp-shuffle -> shared memory -> one atomic per block; 16 elements per thread with 128-bit accesses.
 #include <cooperative_groups.h>
 
 #include "eoq_cells.cuh"

@@ -19,7 +19,6 @@ constexpr int kGemmThreads = 128 + 32 * kEpilogueWarps;  // warps 0, 2, 3: TMA, 
 constexpr int kWgradThreads = 256;  // weight gradient: warps 0, 2, 3 TMA, warp 1 MMA, warps 4..7 epilogue
 constexpr uint32_t kSpinLimit = 1u << 22;  // polls before a wait gives up (normal waits end within microseconds)
 
-// Device state a handle owns.
 // Lets a kernel have `bytes` of dynamic shared memory; asked once per kernel and device (`done`: a bit per device), since the
 // runtime call costs as much host time as a quarter of a launch.
 inline cudaError_t allow_smem(const void *kernel, int bytes, std::atomic<unsigned long long> &done)
@@ -63,6 +62,7 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
     return launch_chained_clusters(1, kernel, grid, block, smem, stream, static_cast<A &&>(args)...);
 }
 
+// Device state a handle owns.
 struct DeviceState {
     unsigned status;       // EOQ_DEV_* bits
     unsigned absmax_u32;   // reduction cell for |.| maxima (int32 sources, float bit patterns)
@@ -79,8 +79,6 @@ struct DeviceState {
 // no call starts with a memset.  A kernel that gave up on a wait (EOQ_DEV_TIMEOUT) may leave them dirty:
 // eoq_last_status clears them again when it reports that bit.
 
-// eoq_set_reduce_hook: called on the host between the kernel that forms a value reduced over the batch and the kernel
-// that consumes it; it enqueues an all-reduce of the device buffer on the stream (no-op when no hook is set).
 // The error head of the layer that consumes an error tensor, fused into the second pass of the kernel that produces it
 // (eoq_conv_dgrad_head, eoq_aux_join_head, eoq_aux_maxpool_bwd_head).
 struct NextHeadArgs {
@@ -101,6 +99,8 @@ struct JoinStatArgs {
     const uint8_t *next_mask;  // ReLU mask of the layer that consumes the joined error, or null
 };
 
+// eoq_set_reduce_hook: called on the host between the kernel that forms a value reduced over the batch and the kernel
+// that consumes it; it enqueues an all-reduce of the device buffer on the stream (no-op when no hook is set).
 struct ReduceHook {
     eoq_reduce_fn fn;
     void *user;
@@ -129,12 +129,11 @@ struct Handle {
     bool force_timeout;           // self-test: the next error-head call makes its grid-wide wait run out
     int num_records;
     ProfRecord *records;          // kMaxProfRecords entries, allocated on first eoq_profile_start
-    // Fork and join events of the calls that issue independent kernels on the class_branch streams (null branch
-    // streams: everything stays on the caller's stream).  Under stream capture they become graph edges.
-    int gemm_ctas;                // most CTAs a GEMM launch of this handle may use (eoq_set_gemm_ctas; default: one per SM)
-    cudaEvent_t fork_ev, join_ev;
-    // further branch streams: the per-class GEMMs of a strided error back-propagation write disjoint pixels and
-    // run side by side, each with its share of the CTAs
+    int gemm_ctas;                // most CTAs a GEMM call of this handle may use (eoq_set_gemm_ctas; default: one per SM)
+    // Branch streams with their fork and join events: the per-class GEMMs of a strided error back-propagation write disjoint
+    // pixels and run side by side, each with its share of the CTAs (null streams, as on the path without a handle: everything
+    // stays on the caller's stream).  Under stream capture the events become graph edges.
+    cudaEvent_t fork_ev;
     cudaStream_t class_branch[kClassBranches];
     cudaEvent_t class_join[kClassBranches];
 };
@@ -333,8 +332,8 @@ cudaError_t launch_sq_i32(const int32_t *src, const int32_t *src_exp, int exp_bi
                           int32_t *dst_exp, long long *sum_codes, bool max_already_reduced, DeviceState *dev,
                           int sm_count, cudaStream_t s, const ReduceHook &hook, const NextHeadArgs *next = nullptr,
                           const JoinStatArgs *join = nullptr);
-// Q_g of the exact sums.  `src` holds int64 sums; when `parts` is given the sums are first formed from
-// `num_parts` int32 slices of n elements each (and written to src).
+// SQ of the compact sums [n][hq][wq][c] of a strided 1 x 1 filter, scattered onto the stride grid of an [n][hh][ww][c] tensor
+// that is zero elsewhere.
 cudaError_t launch_sq_i32_scatter(const int32_t *src, const int32_t *src_exp, int exp_bias, int n_img, int hh, int ww, int c,
                                   int stride, int hq, int wq, int8_t *dst, int32_t *dst_exp, long long *sum_codes,
                                   DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook);
@@ -389,7 +388,7 @@ cudaError_t launch_weight_prep(const PrepBatch &b, cudaStream_t s);
 
 
 // ---------------------------------------------------------------------------------------------
-// Network glue (eoq_aux.cu)
+// Network glue (eoq_pool.cu, eoq_aux.cu, eoq_head.cu)
 // ---------------------------------------------------------------------------------------------
 cudaError_t launch_maxpool_fwd(const int8_t *x, int n, int h, int w, int c, int k, int s, int p, int8_t *y, uint8_t *arg,
                                cudaStream_t st);
@@ -440,8 +439,8 @@ struct FinishItem {
     int use_b1;                    // 0: no b1 term (then the tap sums are neither formed nor read)
     long long *tap_sums;           // kTapReplicas copies, tap_stride elements apart; cleared by the GEMM kernel
     unsigned long long *max_cell;  // max |sum| of the layer (behind the tap sums); cleared by the GEMM kernel
-    long long *acc;                // exact sums [oc][tap][ic]: the GEMM's (64-bit), or where the slices' sums go
-    const int32_t *parts;          // int32 split-K slices, or null when the GEMM added into acc
+    long long *acc;                // where the slices' sums [oc][tap][ic] go: 64-bit, or int32 when they provably fit
+    const int32_t *parts;          // int32 split-K slices of the GEMM
     long long *copy_out;           // the exact sums for the caller, or null
     int8_t *g;
     int32_t *g_exp;

@@ -91,7 +91,7 @@ extern "C" int eoq_conv_dgrad_static(const eoq_conv_desc_t *desc, const int8_t *
     h.num_records = 0;
     h.records = nullptr;
     h.gemm_ctas = pd.sm_count;
-    h.fork_ev = h.join_ev = nullptr;
+    h.fork_ev = nullptr;
     for (int k = 0; k < kClassBranches; ++k) {
         h.class_branch[k] = nullptr;
         h.class_join[k] = nullptr;

@@ -416,7 +416,7 @@ def test_strided_1x1_dgrad_without_sum_dump(d):
 # ------------------------------------------------------------------ paths that only large problems take
 
 WIDE_CASES = [
-    # (geometry, pass, expected fragment of the plan): a 256-column tile needs at least twice as many tiles as SMs
+    # (geometry, pass, expected fragment of the plan): im2col kernel: twice as many tiles as SMs; patch kernel: a wave saved
     (ConvDesc(13, 56, 56, 64, 256, 1, 1, 1, 0), eoq.EOQ_PASS_FWD, "kernel=igemm tile_n=256"),
     (ConvDesc(13, 56, 56, 256, 64, 1, 1, 1, 0), eoq.EOQ_PASS_DGRAD, "kernel=igemm classes=1 tile_n=256"),
     (ConvDesc(148, 14, 14, 256, 256, 3, 3, 1, 1), eoq.EOQ_PASS_FWD, "kernel=igemm_patch tile_n=256 accumulators=1"),
@@ -426,8 +426,8 @@ WIDE_CASES = [
 
 @pytest.mark.parametrize("d,pass_,plan", WIDE_CASES, ids=["igemm_fwd", "igemm_dgrad", "patch_fwd", "patch_dgrad"])
 def test_256_column_tiles(d, pass_, plan):
-    """Both implicit-GEMM kernels with 256-column tiles (one accumulator per tile), which only problems with at
-    least 2 x SMs row tiles take; the plan report confirms the path before the results are compared."""
+    """Both implicit-GEMM kernels with 256-column tiles (one accumulator per tile), which only large
+    problems take; the plan report confirms the path before the results are compared."""
     gd = G.gdesc(d)
     assert plan in eoq.eoq_describe_plan(G.handle(), gd, pass_)
     x0, w, sc, e3 = layer_data(d, 7300 + d.c_in, wrange=12)
@@ -534,8 +534,7 @@ def test_update_with_device_step_counter():
 
 
 def test_wgrad_two_kernel_finish_path():
-    """A weight tensor too large for the one-kernel slice sum + Q_g (more sums than a resident grid keeps in
-    registers) takes the finalize + Q_g pair."""
+    """The largest weight tensor of the suite: tap sums, slice sums and Q_g behind the GEMM, twice on the same handle."""
     d = ConvDesc(1, 6, 6, 1024, 1024, 3, 3, 1, 1)   # 9.4 M weights
     x0, _, _, e3 = layer_data(d, 8400)
     Gacc = oracle.conv_wgrad_acc(d, e3, x0, -2)
@@ -548,7 +547,7 @@ def test_wgrad_two_kernel_finish_path():
         eoq.eoq_conv_wgrad(h, gd, G.dev(e3), G.dev(np.array([-9], dtype=np.int32)), G.dev(x0), -2, g_d, g_exp, None,
                            G.workspace(gd, eoq.EOQ_PASS_WGRAD))
         assert G.status_clear() == 0
-        assert eoq.eoq_launch_count(h) - before == 4  # tap sums, GEMM, finalize, Q_g
+        assert eoq.eoq_launch_count(h) - before == 4  # GEMM, tap sums, slice sums, Q_g
         assert np.array_equal(G.host(g_d).astype(np.int32), g) and g_exp.item() == pg
 
 

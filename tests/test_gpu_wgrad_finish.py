@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 LAYERS = [  # n, h, w, c_in, c_out, k, stride, pad, b1 (None: no bias in front of the convolution)
     (2, 12, 12, 32, 32, 3, 1, 1, -2),       # patch kernel, int32 slices
     (3, 7, 7, 64, 128, 3, 1, 1, 5),
-    (2, 10, 10, 32, 64, 3, 2, 1, 3),        # strided: per-tap kernel, int64 sums
+    (2, 10, 10, 32, 64, 3, 2, 1, 3),        # strided: per-tap kernel
     (2, 9, 11, 48, 32, 1, 1, 0, -7),
     (2, 16, 16, 16, 32, 7, 2, 3, None),     # a first-layer shape
     (1, 20, 20, 64, 64, 5, 1, 2, 0),        # b1 present and zero
