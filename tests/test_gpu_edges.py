@@ -315,3 +315,23 @@ def test_weight_gradient_keeps_to_the_cta_cap(d, m, ctas):
     assert np.array_equal(G.host(g).astype(np.int32), want) and pg.item() == p
     assert eoq.eoq_last_status(h) == 0
     eoq.eoq_destroy(h)
+
+
+@pytest.mark.parametrize("d,m", [
+    (oracle.ConvDesc(9, 128, 128, 16, 16, 3, 3, 1, 1), 0),  # patch kernel
+    (oracle.ConvDesc(9, 128, 128, 16, 16, 1, 1, 1, 0), 0),  # one tap at a time
+    (oracle.ConvDesc(9, 256, 256, 8, 32, 7, 7, 2, 3), 5),   # window rows in a ring
+], ids=["patch", "taps", "rows"])
+def test_weight_gradient_slices_stay_exact_in_few_ctas(d, m):
+    """147,456 pixels of extreme operands: more than one int32 sum holds, so a cap of one CTA still leaves several slices."""
+    x, e3 = np.full((d.n, d.h, d.w, d.c_in), 127, dtype=np.int8), np.full((d.n, d.ho, d.wo, d.c_out), -127, dtype=np.int8)
+    want = oracle.conv_wgrad_acc(d, e3, x, 0)
+    assert abs(want).max() > 2 ** 31
+    gd, h = eoq.conv_desc(d.n, d.h, d.w, d.c_in, d.c_out, d.kh, d.kw, d.stride, d.pad, m), eoq.eoq_create(0)
+    eoq.eoq_set_gemm_ctas(h, 1)
+    xm, e3_d, pe = G.dev(np.pad(x, ((0, 0), (0, 0), (m, m), (0, 0)))), G.dev(e3), G.dev(np.array([0], dtype=np.int32))
+    ws, g, pg, acc = G.workspace(gd, eoq.EOQ_PASS_WGRAD), G.zeros(want.shape, torch.int8), G.zeros(1, torch.int32), G.zeros(want.shape, torch.int64)
+    assert 2 <= eoq.eoq_conv_wgrad_gemm(h, gd, e3_d, pe, xm, ws) <= 3
+    eoq.eoq_conv_wgrad(h, gd, e3_d, pe, xm, 0, g, pg, acc, ws)
+    assert eoq.eoq_last_status(h) == 0 and np.array_equal(G.host(acc), want)
+    eoq.eoq_destroy(h)
