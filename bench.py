@@ -266,8 +266,8 @@ def run_gpu(args):
         step = TrainStep(wl, handle, f"cuda:{local}", scalars=Scalars(), round_mode=round_mode)
     stream = torch.cuda.current_stream()
 
-    # One step = one replay of a CUDA graph of the whole path (the weight-gradient chain of each layer on a side
-    # stream next to its dgrad chain); --eager launches call by call on one stream instead.
+    # One step = one replay of a CUDA graph of the whole path (weight gradients, and in the closed loop the updates of the
+    # stages, on side streams next to the dgrad chain); --eager launches call by call on one stream instead.
     if args.eager:
         do_step = step.run
     else:
@@ -411,7 +411,9 @@ def run_gpu(args):
                        "scalars": "b1=-2 gamma=118 b2=3 codes at the start, device-resident",
                        "update": "stochastic rounding (extension)" if args.stochastic else "round to nearest even (Sec. 3.2.2)",
                        "parallelism": f"replicas x{world}",
-                       "launch": "eager, one stream" if args.eager else "CUDA graph replay, wgrad chains on two side streams"},
+                       "launch": "eager, one stream" if args.eager else
+                                 "CUDA graph replay, weight-gradient GEMMs on two side streams, stages finished and updated on a third" if chained
+                                 else "CUDA graph replay, wgrad chains on two side streams"},
             "clocks": clocks,
             "e2e": {"value": tops_e2e, "unit": "TOPS", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "ms_per_step": ms_e2e / args.steps},

@@ -72,8 +72,8 @@ class ChainedStep:
                  image_channels: int = 3, side_streams: int = 2, keep_pool_error: bool = False, finish_together: bool = True):
         self.wl, self.h, self.dev = workload, handle, torch.device(device)
         self.keep_pool_error = keep_pool_error   # also write the error between the pool and the first layer's head
-        # weight gradients: only the GEMMs run per layer beside the backward chain; the b1 sums, slice sums and Q_g of all
-        # layers follow in four launches at the end (each layer then keeps its sums in a workspace of its own)
+        # weight gradients: only the GEMMs run per layer beside the backward chain; the b1 sums, slice sums and Q_g of a
+        # stage's layers follow in three launches (each layer then keeps its sums in a workspace of its own)
         self.finish_together = finish_together
         self.sc = scalars or Scalars()
         self.lr_mant, self.lr_exp, self.head_lr, self.classes = lr_mant, lr_exp, head_lr, classes
