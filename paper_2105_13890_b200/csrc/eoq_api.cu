@@ -1156,7 +1156,14 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
     int8_t *wt = reinterpret_cast<int8_t *>(workspace);
-    int32_t *sums = acc_dump ? acc_dump : reinterpret_cast<int32_t *>(reinterpret_cast<char *>(workspace) + round256(g.w_elems));
+    // the GEMMs leave their sums as 16-bit words in the workspace, or as int32 where the caller wants them
+    uint16_t *const sums16 = acc_dump ? nullptr : reinterpret_cast<uint16_t *>(static_cast<char *>(workspace) + round256(g.w_elems));
+    auto code_sums = [&](cudaStream_t st) {   // Q_e over the whole tensor, behind the GEMMs
+        return acc_dump ? launch_sq_i32(acc_dump, e3_exp, -7, g.in_elems, e4, e4_exp, reinterpret_cast<long long *>(sum_e4), true, h->dev,
+                                        h->sm_count, st, h->hook)
+                        : launch_sq_sums(sums16, e3_exp, -7, g.in_elems, e4, e4_exp, reinterpret_cast<long long *>(sum_e4), h->dev,
+                                         h->sm_count, st, h->hook, next, jstat_p);
+    };
     cudaError_t e;
 
     // sums that the kernels behind the GEMM add into; it clears them (one the caller also names for the join or the head is
@@ -1183,7 +1190,8 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.out_step = 1;
             p.epilogue = kEpiDgrad;
             memcpy(p.zero_sums, zero_sums, sizeof(zero_sums));
-            p.acc_out = sums;
+            p.acc_out = acc_dump;
+            p.sums16 = sums16;
             p.dev = h->dev;
             p.next_mask = next ? next->mask : nullptr;
             // the weights are read where they are, [c_out][tap][c_in]: the reduction (c_out) is their slow axis, so
@@ -1205,8 +1213,7 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             if (e != cudaSuccess || h->gemm_only) return record(h, e);
             {
                 ProfScope prof(h, EOQ_PROF_DGRAD_AUX, s);
-                e = launch_sq_i32(sums, e3_exp, -7, g.in_elems, e4, e4_exp, reinterpret_cast<long long *>(sum_e4), true,
-                                  h->dev, h->sm_count, s, h->hook, next, jstat_p);
+                e = code_sums(s);
             }
             count_launches(h, 1);
             return join_after(e, s);
@@ -1236,7 +1243,8 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     const bool compact = d.kh == 1 && d.kw == 1 && d.pad == 0 && d.stride > 1 && !acc_dump &&
                          (size_t)d.n * d.h * d.w * (d.c_in / 16) <= 0xffffffffull;
     if (any_empty && !compact) {
-        e = cudaMemsetAsync(sums, 0, g.in_elems * sizeof(int32_t), s);
+        e = acc_dump ? cudaMemsetAsync(acc_dump, 0, g.in_elems * sizeof(int32_t), s)
+                     : cudaMemsetAsync(sums16, 0, g.in_elems * sizeof(uint16_t), s);
         if (e != cudaSuccess) return record(h, e);
     }
     // The classes write disjoint pixels, so their GEMMs are independent: with more than one class and branch streams
@@ -1312,7 +1320,8 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.out_off_w = px;
             p.epilogue = kEpiDgrad;
             memcpy(p.zero_sums, zero_sums, sizeof(zero_sums));
-            p.acc_out = sums;
+            p.acc_out = acc_dump;
+            p.sums16 = sums16;
             p.dev = h->dev;
             p.next_mask = next ? next->mask : nullptr;
             CUtensorMap map_a, map_b;
@@ -1372,12 +1381,11 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     {
         ProfScope prof(h, EOQ_PROF_DGRAD_AUX, s);
         if (compact)
-            e = launch_sq_i32_scatter(sums, e3_exp, -7, d.n, d.h, d.w, d.c_in, d.stride, (d.h + d.stride - 1) / d.stride,
-                                      (d.w + d.stride - 1) / d.stride, e4, e4_exp, reinterpret_cast<long long *>(sum_e4),
-                                      h->dev, h->sm_count, s, h->hook);
+            e = launch_sq_sums_scatter(sums16, e3_exp, -7, d.n, d.h, d.w, d.c_in, d.stride, (d.h + d.stride - 1) / d.stride,
+                                       (d.w + d.stride - 1) / d.stride, e4, e4_exp, reinterpret_cast<long long *>(sum_e4),
+                                       h->dev, h->sm_count, s, h->hook);
         else
-            e = launch_sq_i32(sums, e3_exp, -7, g.in_elems, e4, e4_exp, reinterpret_cast<long long *>(sum_e4), true, h->dev,
-                              h->sm_count, s, h->hook, next, jstat_p);
+            e = code_sums(s);
     }
     count_launches(h, 1);
     return join_after(e, s);

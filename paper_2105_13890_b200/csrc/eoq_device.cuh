@@ -128,6 +128,94 @@ __device__ __forceinline__ uint32_t sq_pack4_shr(const int32_t *a, int s, int32_
     return pack4_sat(v[0], v[1], v[2], v[3]);
 }
 
+// ------------------------------------------------------------------ sums on their way to Q_e
+// The sums of an error back-propagation travel from its GEMM to the kernel that codes them as 16-bit words: 16 consecutive
+// channels of a pixel are 32 bytes instead of 64.  Nothing that Q_e can see is lost.  Sums below 2^14 stand as they are; in a
+// group with a larger one, all 16 lose their low s bits (s = bits of the largest - 14) and what was cut off is or-ed into the
+// lowest bit that stays.  Q_e rounds at bit S = R(log2 max) - 7 of the tensor's maximum, and a group's largest |sum| is at most
+// that maximum, so S >= s + 6: the bit Q_e rounds at and all above it are kept, and the or-ed bit tells a remainder of exactly
+// one half from one beside it.  Either way a word has 15 significant bits, so bit 15 repeats bit 14, and that is where a group
+// with s > 0 is marked (word 0) and carries s (words 1 to 5): bits flipped, no space beside the sums.
+
+// `mx` = the largest magnitude among the 16 sums
+__device__ __forceinline__ void sums_pack_16(const uint32_t *acc, uint32_t mx, uint32_t (&w)[8])
+{
+    if (mx < (1u << 14)) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = __byte_perm(acc[2 * i], acc[2 * i + 1], 0x5410);
+        return;
+    }
+    const int s = 18 - __clz(mx);
+    const int32_t rest = (1 << s) - 1;
+    uint32_t m[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) m[i] = (uint32_t)(((int32_t)acc[i] >> s) | (((int32_t)acc[i] & rest) ? 1 : 0));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = __byte_perm(m[2 * i], m[2 * i + 1], 0x5410);
+    w[0] ^= 0x8000u | (uint32_t)(s & 1) << 31;
+    w[1] ^= (uint32_t)(s & 2) << 14 | (uint32_t)(s & 4) << 29;
+    w[2] ^= (uint32_t)(s & 8) << 12 | (uint32_t)(s & 16) << 27;
+}
+
+// Was the group shortened?
+__device__ __forceinline__ bool sums_shortened(uint32_t w0) { return ((w0 ^ (w0 << 1)) & 0x8000u) != 0; }
+
+// The sums of a shortened group, their lost bits zero but for the or-ed one.
+__device__ __forceinline__ void sums_restore_16(const uint32_t (&w)[8], int32_t (&a)[16])
+{
+    const uint32_t d0 = w[0] ^ (w[0] << 1), d1 = w[1] ^ (w[1] << 1), d2 = w[2] ^ (w[2] << 1);
+    const int s = (int)((d0 >> 31) | (d1 >> 14 & 2u) | (d1 >> 29 & 4u) | (d2 >> 12 & 8u) | (d2 >> 27 & 16u));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        a[2 * i] = (int32_t)((uint32_t)((int32_t)(w[i] << 17) >> 17) << s);
+        a[2 * i + 1] = (int32_t)((uint32_t)((int32_t)(w[i] << 1) >> 17) << s);
+    }
+}
+
+// Codes of SQ for 16 sums under a shift s known to the whole kernel.  Sums that were not shortened go to their codes on the
+// floating-point pipe: 2^23 + (sum + 2^15) is a float whose bits are put together from the word, and one fused multiply-add
+// forms 1.5 * 2^23 + sum / 2^s, rounded to nearest even at unit spacing (every constant is exact for -7 <= s <= 15; a larger s
+// leaves only zeros, as 15 does).
+struct SumCode {
+    int t, sh;
+    float scale, rest;
+    int32_t half_m1, lo;   // of sq_pack4_shr, for shortened groups (their tensor's shift is at least 7)
+};
+__device__ __forceinline__ SumCode sum_code_setup(int t)
+{
+    SumCode c;
+    c.t = t;
+    c.sh = t - 7;
+    c.scale = __int_as_float((127 - min(c.sh, 15)) << 23);
+    c.rest = 12582912.0f - 8421376.0f * c.scale;
+    const int sh = max(c.sh, 1);
+    c.half_m1 = (1 << (sh - 1)) - 1;
+    c.lo = -(127 << sh);
+    return c;
+}
+__device__ __forceinline__ void sum_codes_16(const SumCode &c, const uint32_t (&w)[8], uint32_t (&cw)[4])
+{
+    if (!sums_shortened(w[0])) {
+        auto code = [&](uint32_t u, uint32_t sel) {
+            const float f = __fmaf_rn(__uint_as_float(__byte_perm(u, 0x4B00u, sel)), c.scale, c.rest);
+            return __viaddmax_s32((int32_t)__float_as_uint(f), -0x4B400000, -127);
+        };
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t u0 = w[2 * q] ^ 0x80008000u, u1 = w[2 * q + 1] ^ 0x80008000u;
+            cw[q] = pack4_sat(code(u0, 0x5410), code(u0, 0x5432), code(u1, 0x5410), code(u1, 0x5432));
+        }
+        return;
+    }
+    int32_t a[16];
+    sums_restore_16(w, a);
+    const bool fits = c.t <= 30;   // (sq_pack4_shr wants the largest sum and half a step to stay below 2^31)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        cw[q] = fits ? sq_pack4_shr(a + 4 * q, c.sh, c.half_m1, c.lo)
+                     : pack4_sat(sq_code32(a[4 * q], c.t), sq_code32(a[4 * q + 1], c.t), sq_code32(a[4 * q + 2], c.t), sq_code32(a[4 * q + 3], c.t));
+}
+
 // Expands 4 mask bits into 4 byte masks (0x00 / 0xff).
 __device__ __forceinline__ uint32_t bits_to_bytes(uint32_t nibble)
 {

@@ -280,7 +280,7 @@ __global__ void absmax_i32_kernel(const int32_t *__restrict__ src, size_t n, Dev
 }
 
 // One 256-bit streaming load (sm_100); ptr must be 32-byte aligned.
-__device__ __forceinline__ void ld_global_256_stream(const int32_t *ptr, int *v)
+__device__ __forceinline__ void ld_global_256_stream(const void *ptr, uint32_t *v)
 {
     asm volatile("ld.global.cs.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
@@ -292,8 +292,10 @@ __device__ __forceinline__ void ld_global_256_stream(const int32_t *ptr, int *v)
 // come out of the same pass.  n must then be a multiple of 16.
 // kJoin: dst is the first operand of an error join; the join's first pass rides along: max |dst * 2^sa + b * 2^sb|
 // over all positions (64-bit cell) and over those the consumer's ReLU lets through (second 64-bit cell).
-template <bool kNext, bool kJoin>
-__global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *src_exp, int exp_bias, size_t n,
+// kPacked: src holds the sums of an error back-propagation as 16-bit words (sums_pack_16; 32-byte aligned, n a multiple of 16);
+// int32 otherwise.
+template <bool kPacked, bool kNext, bool kJoin>
+__global__ void sq_i32_kernel(const void *__restrict__ src_any, const int32_t *src_exp, int exp_bias, size_t n,
                               int8_t *dst, int32_t *dst_exp, long long *sum_codes, NextHeadArgs next, JoinStatArgs join,
                               DeviceState *dev)
 {
@@ -304,27 +306,30 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
     // on the few hundred KB of a small batch.
     __shared__ uint32_t cell_s[2];
     const size_t n16 = n / 16;
+    const int32_t *const src = static_cast<const int32_t *>(src_any);
+    uint32_t raw[kPacked ? 8 : 16];   // a group of 16 sums
     const bool wide_in = (reinterpret_cast<uintptr_t>(src) & 31) == 0;
-    auto load16 = [&](size_t i, int (&a)[16]) {
-        if (wide_in) {   // two 256-bit loads: whole 32-byte sectors per lane
-            ld_global_256_stream(src + i * 16, a);
-            ld_global_256_stream(src + i * 16 + 8, a + 8);
+    auto load16 = [&](size_t i) {
+        if constexpr (kPacked) {
+            ld_global_256_stream(static_cast<const uint16_t *>(src_any) + i * 16, raw);
+        } else if (wide_in) {   // two 256-bit loads: whole 32-byte sectors per lane
+            ld_global_256_stream(src + i * 16, raw);
+            ld_global_256_stream(src + i * 16 + 8, raw + 8);
         } else {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int4 v = __ldcs(reinterpret_cast<const int4 *>(src) + i * 4 + k);
-                a[4 * k + 0] = v.x;
-                a[4 * k + 1] = v.y;
-                a[4 * k + 2] = v.z;
-                a[4 * k + 3] = v.w;
+                raw[4 * k + 0] = v.x;
+                raw[4 * k + 1] = v.y;
+                raw[4 * k + 2] = v.z;
+                raw[4 * k + 3] = v.w;
             }
         }
     };
     // the first group of every thread is on its way while the maxima are read
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int a[16];
     if (i < n16) {
-        load16(i, a);
+        load16(i);
         if (kJoin) {
             ptx::prefetch_l1(join.b + i * 16);
             if (join.mask_b) ptx::prefetch_l1(join.mask_b + i * 2);
@@ -368,16 +373,22 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
     // the maximum bounds every element, so |a| + 2^(sh-1) cannot wrap as long as M + M / 2^7 < 2^31
     const bool fast = sh >= 1 && M < 0x7e000000u;
     const int32_t half_m1 = fast ? (1 << (sh - 1)) - 1 : 0, lo = fast ? -(127 << sh) : 0;
+    const SumCode sc = sum_code_setup(t);
     uint32_t jm32 = 0, jmm32 = 0;
     while (i < n16) {
         uint32_t cw[4];   // four codes per word
+        if constexpr (kPacked) {
+            sum_codes_16(sc, raw, cw);
+        } else {
+            const int32_t *a = reinterpret_cast<const int32_t *>(raw);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                cw[q] = fast ? sq_pack4_shr(a + 4 * q, sh, half_m1, lo)
+                             : pack4_sat(sq_code32(a[4 * q], t), sq_code32(a[4 * q + 1], t), sq_code32(a[4 * q + 2], t), sq_code32(a[4 * q + 3], t));
+        }
         int sum16 = 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            cw[q] = fast ? sq_pack4_shr(a + 4 * q, sh, half_m1, lo)
-                         : pack4_sat(sq_code32(a[4 * q], t), sq_code32(a[4 * q + 1], t), sq_code32(a[4 * q + 2], t), sq_code32(a[4 * q + 3], t));
-            sum16 = __dp4a((int)cw[q], 0x01010101, sum16);
-        }
+        for (int q = 0; q < 4; ++q) sum16 = __dp4a((int)cw[q], 0x01010101, sum16);
         sum += sum16;
         reinterpret_cast<int4 *>(dst)[i] = make_int4((int)cw[0], (int)cw[1], (int)cw[2], (int)cw[3]);
         if (kJoin) {
@@ -420,10 +431,10 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
             reinterpret_cast<int4 *>(next.e3)[i] = make_int4((int)c3[0], (int)c3[1], (int)c3[2], (int)c3[3]);
         }
         i += (size_t)gridDim.x * blockDim.x;
-        if (i < n16) load16(i, a);
+        if (i < n16) load16(i);
     }
     ptx::grid_dep_launch();
-    if (!kNext && !kJoin)
+    if (!kPacked)
         for (size_t i = n16 * 16 + (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
             const int c = sq_code32(src[i], t);
             sum += c;
@@ -464,10 +475,10 @@ __global__ void sq_i32_kernel(const int32_t *__restrict__ src, const int32_t *sr
 }
 
 // Q_e for a strided 1x1 filter: only the pixels (y, x) with y and x multiples of the stride receive an error, the
-// others are exactly zero.  The GEMM leaves its sums compact, [n][hq][wq][c]; this kernel writes the full tensor
-// [n][h][w][c], codes on the grid and zeros elsewhere, so neither a cleared full-size int32 tensor nor a pass over
+// others are exactly zero.  The GEMM leaves its sums (16-bit words) compact, [n][hq][wq][c]; this kernel writes the full tensor
+// [n][h][w][c], codes on the grid and zeros elsewhere, so neither a cleared full-size tensor of sums nor a pass over
 // it is needed.  A thread writes 16 channels of one pixel.
-__global__ void sq_i32_scatter_kernel(const int32_t *__restrict__ src, const int32_t *src_exp, int exp_bias, int n_img, int hh,
+__global__ void sq_sums_scatter_kernel(const uint16_t *__restrict__ src, const int32_t *src_exp, int exp_bias, int n_img, int hh,
                                       int ww, int c, int stride, int hq, int wq, int8_t *dst, int32_t *dst_exp,
                                       long long *sum_codes, DeviceState *dev)
 {
@@ -484,6 +495,7 @@ __global__ void sq_i32_scatter_kernel(const int32_t *__restrict__ src, const int
         *dst_exp = M ? p_in + t - 7 : p_in;
         if (!M) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
     }
+    const SumCode code = sum_code_setup(t);
     long long sum = 0;
     const uint32_t groups = (uint32_t)c / 16u;
     const size_t items = (size_t)n_img * hh * ww * groups;  // fits 32 bits (checked by the launcher)
@@ -494,22 +506,14 @@ __global__ void sq_i32_scatter_kernel(const int32_t *__restrict__ src, const int
         int4 out = make_int4(0, 0, 0, 0);
         if (y % (uint32_t)stride == 0 && x % (uint32_t)stride == 0) {
             const size_t q = (((size_t)img * hq + y / (uint32_t)stride) * wq + x / (uint32_t)stride) * c + g * 16u;
-            const int4 *s4 = reinterpret_cast<const int4 *>(src + q);
-            int cdes[16];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int4 v = __ldcs(s4 + k);
-                cdes[4 * k + 0] = sq_code32(v.x, t);
-                cdes[4 * k + 1] = sq_code32(v.y, t);
-                cdes[4 * k + 2] = sq_code32(v.z, t);
-                cdes[4 * k + 3] = sq_code32(v.w, t);
-            }
+            uint32_t raw[8], cw[4];
+            ld_global_256_stream(src + q, raw);
+            sum_codes_16(code, raw, cw);
             int sc = 0;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) sc += cdes[k];
+            for (int k = 0; k < 4; ++k) sc = __dp4a((int)cw[k], 0x01010101, sc);
             sum += sc;
-            out = make_int4((int)pack4(cdes[0], cdes[1], cdes[2], cdes[3]), (int)pack4(cdes[4], cdes[5], cdes[6], cdes[7]),
-                            (int)pack4(cdes[8], cdes[9], cdes[10], cdes[11]), (int)pack4(cdes[12], cdes[13], cdes[14], cdes[15]));
+            out = make_int4((int)cw[0], (int)cw[1], (int)cw[2], (int)cw[3]);
         }
         reinterpret_cast<int4 *>(dst)[i] = out;
     }
@@ -985,36 +989,47 @@ cudaError_t launch_weight_pad_rows(const int8_t *w, int8_t *wp, int c_out, int k
 
 cudaError_t launch_sq_i32(const int32_t *src, const int32_t *src_exp, int exp_bias, size_t n, int8_t *dst,
                           int32_t *dst_exp, long long *sum_codes, bool max_already_reduced, DeviceState *dev,
-                          int sm_count, cudaStream_t s, const ReduceHook &hook, const NextHeadArgs *next, const JoinStatArgs *join)
+                          int sm_count, cudaStream_t s, const ReduceHook &hook)
 {
     if (!max_already_reduced) absmax_i32_kernel<<<grid_for(n / 4 + 1, sm_count), kThreads, 0, s>>>(src, n, dev);
+    hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
+    launch_chained(sq_i32_kernel<false, false, false>, grid_for(n / 16 + 1, sm_count), kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp,
+                   sum_codes, NextHeadArgs{}, JoinStatArgs{}, dev);
+    if (sum_codes) hook(sum_codes, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sq_sums(const uint16_t *src, const int32_t *src_exp, int exp_bias, size_t n, int8_t *dst, int32_t *dst_exp,
+                           long long *sum_codes, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook,
+                           const NextHeadArgs *next, const JoinStatArgs *join)
+{
     hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
     const int grid = grid_for(n / 16 + 1, sm_count);
     if (join) {
         // (no hook in this form: callers with replicas take the separate calls)
-        launch_chained(sq_i32_kernel<false, true>, grid, kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, NextHeadArgs{}, *join, dev);
+        launch_chained(sq_i32_kernel<true, false, true>, grid, kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, NextHeadArgs{}, *join, dev);
     } else if (next) {
         // (only behind a GEMM whose epilogue reduced the masked maximum)
         hook(&dev->absmax_u64, 1, EOQ_REDUCE_I64, EOQ_REDUCE_MAX, s);
-        launch_chained(sq_i32_kernel<true, false>, grid, kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, *next, JoinStatArgs{}, dev);
+        launch_chained(sq_i32_kernel<true, true, false>, grid, kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, *next, JoinStatArgs{}, dev);
         if (next->sum_e1) hook(next->sum_e1, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
         if (next->sum_e1x2) hook(next->sum_e1x2, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
     } else {
-        launch_chained(sq_i32_kernel<false, false>, grid, kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, NextHeadArgs{},
-                                                              JoinStatArgs{}, dev);
+        launch_chained(sq_i32_kernel<true, false, false>, grid, kThreads, 0, s, src, src_exp, exp_bias, n, dst, dst_exp, sum_codes, NextHeadArgs{},
+                       JoinStatArgs{}, dev);
     }
     if (sum_codes) hook(sum_codes, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sq_i32_scatter(const int32_t *src, const int32_t *src_exp, int exp_bias, int n_img, int hh, int ww, int c,
-                                  int stride, int hq, int wq, int8_t *dst, int32_t *dst_exp, long long *sum_codes,
-                                  DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook)
+cudaError_t launch_sq_sums_scatter(const uint16_t *src, const int32_t *src_exp, int exp_bias, int n_img, int hh, int ww, int c,
+                                   int stride, int hq, int wq, int8_t *dst, int32_t *dst_exp, long long *sum_codes,
+                                   DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook)
 {
     const size_t items = (size_t)n_img * hh * ww * (c / 16);
     hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
-    launch_chained(sq_i32_scatter_kernel, grid_for(items, sm_count), kThreads, 0, s, src, src_exp, exp_bias, n_img, hh, ww, c, stride, hq, wq,
-                                                                        dst, dst_exp, sum_codes, dev);
+    launch_chained(sq_sums_scatter_kernel, grid_for(items, sm_count), kThreads, 0, s, src, src_exp, exp_bias, n_img, hh, ww, c, stride, hq, wq,
+                   dst, dst_exp, sum_codes, dev);
     if (sum_codes) hook(sum_codes, 1, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);
     return cudaGetLastError();
 }

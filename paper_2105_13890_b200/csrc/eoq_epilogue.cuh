@@ -317,10 +317,10 @@ __device__ __forceinline__ void forward_group(const IgemmParams &p, const FwdSca
     }
 }
 
-// Error back-propagation: keep the exact int32 sums (the scale quantizer needs the maximum over the whole
-// tensor before any element can be coded) and track max |.|.
-// kWide: the destination is 32-byte aligned (the launch checks the base; off is a multiple of 16 elements)
-template <bool kWide>
+// Error back-propagation: keep the exact sums (the scale quantizer needs the maximum over the whole tensor before any element can
+// be coded) and track max |.|.  They are kept as 16-bit words that lose nothing Q_e can see (sums_pack_16), one 32-byte sector per
+// lane and 16 columns: this launch is bound by its stores.  A caller who asks for the int32 sums gets those instead
+// (p.sums16 == null).
 __device__ __forceinline__ uint32_t dgrad_16(const IgemmParams &p, const uint32_t *acc, size_t off, uint32_t &mx_masked)
 {
     uint32_t mx = 0;
@@ -340,9 +340,10 @@ __device__ __forceinline__ uint32_t dgrad_16(const IgemmParams &p, const uint32_
             mx_masked = max(mx_masked, (b4 & 8u) ? a3 : 0u);
         }
     }
-    if (kWide) {
-        st_global_256(p.acc_out + off, acc);
-        st_global_256(p.acc_out + off + 8, acc + 8);
+    if (p.sums16) {
+        uint32_t w[8];
+        sums_pack_16(acc, mx, w);
+        st_global_256(p.sums16 + off, w);   // (a workspace: aligned to 256 bytes)
     } else {
         int4 *d = reinterpret_cast<int4 *>(p.acc_out + off);
 #pragma unroll

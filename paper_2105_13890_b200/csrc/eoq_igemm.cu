@@ -254,7 +254,6 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         const int shift = input_shift(p);
         const FwdShift sh = forward_shift(p, shift);
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
-        const bool wide_out = (reinterpret_cast<uintptr_t>(p.acc_out) & 31) == 0;   // 256-bit stores of the exact sums
         bool ok = true;
         for (int tile = tile_first + grp * gridDim.x; tile < num_tiles && ok; tile += p.ep_groups * gridDim.x) {
             const int mt = tile / p.num_n_tiles, nt = tile % p.num_n_tiles;
@@ -333,7 +332,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                     if (fwd) {
                         forward_group(p, fs, sh, r, r2, kSplit ? 1u : nacc, off, tb, tg, sc, shift);
                     } else {
-                        mx = max(mx, wide_out ? dgrad_16<true>(p, r, off, mx_masked) : dgrad_16<false>(p, r, off, mx_masked));
+                        mx = max(mx, dgrad_16(p, r, off, mx_masked));
                     }
                 }
                 sc = sc_next;

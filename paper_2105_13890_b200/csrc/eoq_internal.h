@@ -187,7 +187,8 @@ struct IgemmParams {
     int8_t *x5;
     int16_t *x2;
     uint8_t *relu_mask;
-    int32_t *acc_out;         // forward: optional dump; dgrad: the int32 scratch (required)
+    int32_t *acc_out;         // forward: optional dump; dgrad: the int32 sums when the caller wants them
+    uint16_t *sums16;         // dgrad: else the sums as 16-bit words for the kernel that codes them (sums_pack_16; 32-byte aligned)
     DeviceState *dev;
     // B operand read MN-major (patch kernel, error back-propagation): the weights stay [c_out][tap][c_in], a sub-tile
     // is [kc reduction rows][tile_n columns] made of tile_n / b_row atoms of b_row-byte rows, kc * b_row bytes apart
@@ -330,13 +331,16 @@ cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst,
                                 int sm_count, cudaStream_t s, const ReduceHook &hook);
 cudaError_t launch_sq_i32(const int32_t *src, const int32_t *src_exp, int exp_bias, size_t n, int8_t *dst,
                           int32_t *dst_exp, long long *sum_codes, bool max_already_reduced, DeviceState *dev,
-                          int sm_count, cudaStream_t s, const ReduceHook &hook, const NextHeadArgs *next = nullptr,
-                          const JoinStatArgs *join = nullptr);
+                          int sm_count, cudaStream_t s, const ReduceHook &hook);
+// ... of the 16-bit words that the GEMMs of an error back-propagation leave (n a multiple of 16); the maximum is in the cell
+cudaError_t launch_sq_sums(const uint16_t *src, const int32_t *src_exp, int exp_bias, size_t n, int8_t *dst, int32_t *dst_exp,
+                           long long *sum_codes, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook,
+                           const NextHeadArgs *next = nullptr, const JoinStatArgs *join = nullptr);
 // SQ of the compact sums [n][hq][wq][c] of a strided 1 x 1 filter, scattered onto the stride grid of an [n][hh][ww][c] tensor
-// that is zero elsewhere.
-cudaError_t launch_sq_i32_scatter(const int32_t *src, const int32_t *src_exp, int exp_bias, int n_img, int hh, int ww, int c,
-                                  int stride, int hq, int wq, int8_t *dst, int32_t *dst_exp, long long *sum_codes,
-                                  DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook);
+// (n * hh * ww * c / 16 below 2^32)
+cudaError_t launch_sq_sums_scatter(const uint16_t *src, const int32_t *src_exp, int exp_bias, int n_img, int hh, int ww, int c,
+                                   int stride, int hq, int wq, int8_t *dst, int32_t *dst_exp, long long *sum_codes,
+                                   DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook);
 // gamma is gamma_c, or the code at gamma_dev when that is given.  force_timeout: self-test of the bounded wait.
 cudaError_t launch_err_prescale(const int8_t *e0, const int32_t *e0_exp, const uint8_t *mask, const int16_t *x2,
                                 size_t n_el, int32_t gamma_c, const int32_t *gamma_dev, int8_t *e3, int32_t *e3_exp,
