@@ -1,8 +1,8 @@
 // Implicit-GEMM convolution kernel for sm_100a: forward pass and error back-propagation of the EOQ layer
 // (arXiv 2105.13890, Sec. 3.2.1).  One persistent CTA per SM walks 128-row output tiles:
 //   warps 0, 2, 3: TMA producers (im2col loads of the activation/error operand, tiled loads of the weights); a
-//              thread gets a TMA instruction out only every few hundred cycles, but threads of different warps
-//              issue side by side, so the pipeline stages rotate over three producers
+//              thread gets a TMA instruction out only every few hundred cycles, most of them address arithmetic, but
+//              threads issue side by side: the pipeline stages rotate over three warps, a stage's loads over their lanes
 //   warp 1       : owns tensor memory, issues tcgen05.mma kind::i8 (int8 x int8 -> int32 in TMEM)
 //   warps 4-19   : epilogue; read the accumulators with tcgen05.ld and apply the layer's quantizers in registers
 // Up to four accumulator buffers in TMEM let the epilogue of a tile overlap the main loops of the next ones.
@@ -71,15 +71,6 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), tmem_cols);
         ptx::tmem_relinquish();
     }
-    ptx::tc_fence_before();
-    __syncthreads();
-    ptx::tc_fence_after();
-    if (kSplit) ptx::cluster_wait();
-    ptx::grid_dep_wait();   // everything up to here touched no global memory
-    if (kEpi == kEpiDgrad && blockIdx.x == 0 && threadIdx.x < 4 && p.zero_sums[threadIdx.x]) *p.zero_sums[threadIdx.x] = 0;
-    const uint32_t tmem_base = tmem_base_s;
-    const RoleCtx ctx{&abort_s, p.dev};
-
     const int num_tiles = p.num_m_tiles * p.num_n_tiles;
     const int k_iters = (p.num_sub + p.subs_per_stage - 1) / p.subs_per_stage;
     const int pix_per_img = p.hq * p.wq;
@@ -91,62 +82,82 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     const int k_count = kSplit ? k_iters * (rank + 1) / p.split - k_first : k_iters;
     const int tile_first = kSplit ? (int)blockIdx.x / p.split : (int)blockIdx.x;   // (a cluster has one tile)
 
-    if (warp == 0 || warp == 2 || warp == 3) {
-        if (lane == 0) {
-            // ------------------------------------------------------------------ TMA producers
-            // producer q fills the pipeline slots q, q + 3, q + 6, ... of the CTA's sequence of (tile, k iteration)
-            const int q = warp == 0 ? 0 : warp - 1;
-            int stage = q % p.num_stages;
-            uint32_t phase = (uint32_t)(q / p.num_stages) & 1u;
-            int turn = q;  // slots until this producer's next one
-            uint32_t inflight = 0, inflight_parity = 0;
-            bool ok = true;
-            for (int tile = tile_first; tile < num_tiles && ok; tile += gridDim.x) {
-                const int mt = tile / p.num_n_tiles, nt = tile % p.num_n_tiles;
-                const int m0 = mt * kTileM;
-                const int img = m0 / pix_per_img, rem = m0 % pix_per_img;
-                const int cw = (rem % p.wq) * p.src_stride_w + p.base_w;
-                const int ch = (rem / p.wq) * p.src_stride + p.base_h;
-                for (int step = 0, kit = k_first; step < k_count; ++step, kit = kit + 1 == k_iters ? 0 : kit + 1) {
-                    if (turn-- != 0) continue;
-                    turn = kProducers - 1;
-                    if (!(ok = wait_bar<32>(empty_bar(stage), phase ^ 1u, ctx))) break;
-                    const int s0 = kit * p.subs_per_stage;
-                    const int subs = min(p.subs_per_stage, p.num_sub - s0);
-                    const uint32_t a_dst = smem_base + stage * stage_bytes;
-                    const uint32_t b_dst = a_dst + p.subs_per_stage * a_sub;
-                    ptx::mbar_expect_tx(full_bar(stage), subs * ((uint32_t)p.a_rows * p.kc + b_sub));
-                    for (int j = 0; j < subs; ++j) {
-                        const int s = s0 + j;
-                        const int sd = min(s, p.real_sub - 1);  // a padding sub-tile re-reads real data; its weights are zero
-                        const int tap = sd / p.chunks_per_tap, chunk = sd % p.chunks_per_tap;
-                        ptx::tma_load_im2col_4d(a_dst + j * a_sub, &map_a, full_bar(stage), chunk * p.kc, cw, ch, img,
+    // where a tile's loads start; of the first tile while the kernels in front still run
+    struct Source {
+        int nt, img, cw, ch;
+    };
+    auto source_of = [&](int tile) {
+        const int mt = tile / p.num_n_tiles, m0 = mt * kTileM, img = m0 / pix_per_img, rem = m0 - img * pix_per_img, y = rem / p.wq;
+        return Source{tile - mt * p.num_n_tiles, img, (rem - y * p.wq) * p.src_stride_w + p.base_w, y * p.src_stride + p.base_h};
+    };
+    const bool producer = warp == 0 || warp == 2 || warp == 3;
+    Source at = {};
+    if (producer) at = source_of(tile_first);
+
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    if (kSplit) ptx::cluster_wait();
+    ptx::grid_dep_wait();   // everything up to here touched no global memory
+    if (kEpi == kEpiDgrad && blockIdx.x == 0 && threadIdx.x < 4 && p.zero_sums[threadIdx.x]) *p.zero_sums[threadIdx.x] = 0;
+    const uint32_t tmem_base = tmem_base_s;
+    const RoleCtx ctx{&abort_s, p.dev};
+
+    if (producer) {
+        // ------------------------------------------------------------------ TMA producers
+        // producer q fills the pipeline slots q, q + 3, q + 6, ... of the CTA's sequence of (tile, k iteration); the loads of a slot
+        // are spread over its lanes (what a thread computes between two loads is most of a load's time)
+        const int q = warp == 0 ? 0 : warp - 1;
+        const int atoms = p.b_mn ? p.tile_n / p.b_row : 1;
+        int stage = q % p.num_stages;
+        uint32_t phase = (uint32_t)(q / p.num_stages) & 1u;
+        int turn = q;  // slots until this producer's next one
+        uint32_t inflight = 0, inflight_parity = 0;
+        bool ok = true;
+        for (int tile = tile_first; tile < num_tiles && ok;) {
+            for (int step = 0, kit = k_first; step < k_count; ++step, kit = kit + 1 == k_iters ? 0 : kit + 1) {
+                if (turn-- != 0) continue;
+                turn = kProducers - 1;
+                if (!(ok = __all_sync(0xffffffffu, wait_bar<32>(empty_bar(stage), phase ^ 1u, ctx)))) break;
+                const int s0 = kit * p.subs_per_stage;
+                const int subs = min(p.subs_per_stage, p.num_sub - s0);
+                const uint32_t a_dst = smem_base + stage * stage_bytes;
+                const uint32_t b_dst = a_dst + p.subs_per_stage * a_sub;
+                if (lane == 0) ptx::mbar_expect_tx(full_bar(stage), subs * ((uint32_t)p.a_rows * p.kc + b_sub));
+                __syncwarp();
+                for (int i = lane; i < subs * (1 + atoms); i += 32) {
+                    const int j = i < subs ? i : (i - subs) / atoms;
+                    const int s = s0 + j;
+                    const int sd = min(s, p.real_sub - 1);  // a padding sub-tile re-reads real data; its weights are zero
+                    const int tap = sd / p.chunks_per_tap, chunk = sd - tap * p.chunks_per_tap;
+                    if (i < subs) {
+                        ptx::tma_load_im2col_4d(a_dst + j * a_sub, &map_a, full_bar(stage), chunk * p.kc, at.cw, at.ch, at.img,
                                                 (uint16_t)p.tap_dw[tap], (uint16_t)p.tap_dh[tap]);
-                        if (p.b_mn) {
-                            // weights in place, [reduction rows][tap][columns]: tile_n / b_row atoms of [kc rows][b_row bytes]
-                            const uint32_t atom = (uint32_t)p.kc * p.b_row;
-                            for (int a = 0, na = p.tile_n / p.b_row; a < na; ++a)
-                                ptx::tma_load_3d(b_dst + j * b_sub + a * atom, &map_b, full_bar(stage),
-                                                 nt * p.tile_n + a * p.b_row, (int)p.tap_b[tap], chunk * p.kc);
-                        } else {
-                            // tap coordinate p.ntaps lies outside the weight tensor: the padding sub-tile is zero-filled
-                            ptx::tma_load_3d(b_dst + j * b_sub, &map_b, full_bar(stage), chunk * p.kc,
-                                             s < p.real_sub ? (int)p.tap_b[tap] : 0x7fff, nt * p.tile_n);
-                        }
+                    } else if (p.b_mn) {
+                        // weights in place, [reduction rows][tap][columns]: tile_n / b_row atoms of [kc rows][b_row bytes]
+                        const int a = i - subs - j * atoms;
+                        ptx::tma_load_3d(b_dst + j * b_sub + a * (uint32_t)p.kc * p.b_row, &map_b, full_bar(stage),
+                                         at.nt * p.tile_n + a * p.b_row, (int)p.tap_b[tap], chunk * p.kc);
+                    } else {
+                        // tap coordinate p.ntaps lies outside the weight tensor: the padding sub-tile is zero-filled
+                        ptx::tma_load_3d(b_dst + j * b_sub, &map_b, full_bar(stage), chunk * p.kc,
+                                         s < p.real_sub ? (int)p.tap_b[tap] : 0x7fff, at.nt * p.tile_n);
                     }
-                    inflight |= 1u << stage;
-                    inflight_parity = (inflight_parity & ~(1u << stage)) | (phase << stage);
-                    stage += kProducers;
-                    while (stage >= p.num_stages) { stage -= p.num_stages; phase ^= 1u; }
                 }
+                inflight |= 1u << stage;
+                inflight_parity = (inflight_parity & ~(1u << stage)) | (phase << stage);
+                stage += kProducers;
+                while (stage >= p.num_stages) { stage -= p.num_stages; phase ^= 1u; }
             }
-            if (!ok) {
-                // wait, bounded, for the copies this thread still has in flight
-                for (int s = 0; s < p.num_stages; ++s)
-                    if (inflight & (1u << s))
-                        for (uint32_t i = 0; i < kSpinLimit; ++i)
-                            if (ptx::mbar_try_wait(full_bar(s), (inflight_parity >> s) & 1u)) break;
-            }
+            tile += gridDim.x;
+            if (tile < num_tiles) at = source_of(tile);
+        }
+        if (!ok && lane == 0) {
+            // wait, bounded, for the copies this warp still has in flight
+            for (int s = 0; s < p.num_stages; ++s)
+                if (inflight & (1u << s))
+                    for (uint32_t i = 0; i < kSpinLimit; ++i)
+                        if (ptx::mbar_try_wait(full_bar(s), (inflight_parity >> s) & 1u)) break;
         }
         if (kSplit) ptx::cluster_sync();
     } else if (warp == 1) {

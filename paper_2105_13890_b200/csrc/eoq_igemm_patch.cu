@@ -11,7 +11,7 @@
 // dropped.  Weights either stay resident in shared memory for the whole kernel (when the layer's weights fit) or
 // stream through their own ring.
 //
-// Roles: warp 0 patch loads, warp 1 TMEM owner + tcgen05.mma issuer, warps 2 and 3 weight loads, warps 4-19 epilogue
+// Roles: warp 0 patch loads, warp 1 TMEM owner + tcgen05.mma issuer, warp 2 weight loads, warps 4-19 epilogue
 // (four per TMEM lane quadrant, in one, two or four groups that take the CTA's tiles in turn).
 // All waits are bounded.
 #include "eoq_device.cuh"
@@ -22,7 +22,27 @@ namespace eoq {
 
 namespace {
 
-constexpr int kMaxA = 4, kMaxB = 8;
+constexpr int kMaxA = 6, kMaxB = 8;
+
+// Column tile, image and row tile in the image.  A role carries them from tile to tile: its step between two tiles is constant, so
+// the quotients are formed once instead of per tile.
+struct TilePos {
+    int nt, img, ti;
+    __device__ __forceinline__ void advance(const TilePos &by, int num_n_tiles, int tiles_per_img)
+    {
+        nt += by.nt;
+        ti += by.ti;
+        if (nt >= num_n_tiles) { nt -= num_n_tiles; ++ti; }
+        img += by.img;
+        if (ti >= tiles_per_img) { ti -= tiles_per_img; ++img; }
+        if (ti >= tiles_per_img) { ti -= tiles_per_img; ++img; }
+    }
+};
+__device__ __forceinline__ TilePos tile_pos(int tile, int num_n_tiles, int tiles_per_img)
+{
+    const int mt = tile / num_n_tiles, img = mt / tiles_per_img;
+    return TilePos{tile - mt * num_n_tiles, img, mt - img * tiles_per_img};
+}
 
 template <int kEpi>   // EpilogueKind: forward and dgrad are kernels of their own (registers, code size)
 __global__ void __launch_bounds__(kPatchThreads, 1)
@@ -79,6 +99,12 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
         ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), tmem_cols);
         ptx::tmem_relinquish();
     }
+    // the patch loader's first tile and its step from tile to tile (formed while the kernels in front still run)
+    TilePos pos = {}, by = {};
+    if (warp == 0) {
+        pos = tile_pos((int)blockIdx.x, p.num_n_tiles, pl.tiles_per_img);
+        by = tile_pos((int)gridDim.x, p.num_n_tiles, pl.tiles_per_img);
+    }
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
@@ -97,17 +123,17 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
             uint32_t pha = 0, inflight = 0, inflight_parity = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-                const int mt = tile / p.num_n_tiles;
-                const int img = mt / pl.tiles_per_img, y0 = (mt % pl.tiles_per_img) * pl.r_rows;
+                const int y0 = pos.ti * pl.r_rows;
                 for (int c = 0; c < pl.chunks; ++c) {
-                    if (!(ok = wait_bar<64>(a_empty(ia), pha ^ 1u, ctx))) break;
+                    if (!(ok = wait_bar<32>(a_empty(ia), pha ^ 1u, ctx))) break;
                     ptx::mbar_expect_tx(a_full(ia), (uint32_t)pl.a_box_bytes);
                     // source columns -pad .. -pad + pw - 1, rows y0 - pad .. : out-of-image pixels arrive as zeros
-                    ptx::tma_load_4d(smem_base + ia * pl.a_bytes, &map_a, a_full(ia), c * p.kc, -pl.pad, y0 - pl.pad, img);
+                    ptx::tma_load_4d(smem_base + ia * pl.a_bytes, &map_a, a_full(ia), c * p.kc, -pl.pad, y0 - pl.pad, pos.img);
                     inflight |= 1u << ia;
                     inflight_parity = (inflight_parity & ~(1u << ia)) | (pha << ia);
                     if (++ia == pl.num_a) { ia = 0; pha ^= 1u; }
                 }
+                pos.advance(by, p.num_n_tiles, pl.tiles_per_img);
             }
             if (!ok)
                 for (int s = 0; s < pl.num_a; ++s)
@@ -115,53 +141,70 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
                         for (uint32_t i = 0; i < kSpinLimit; ++i)
                             if (ptx::mbar_try_wait(a_full(s), (inflight_parity >> s) & 1u)) break;
         }
-    } else if (warp == 2 || (warp == 3 && !pl.b_resident)) {
-        if (lane == 0) {
-            // ------------------------------------------------------------------ weight loads
-            // One sub-tile = the weights of one tap for kc reduction channels and tile_n columns.  K-major: one box
-            // [tile_n rows][kc bytes].  MN-major: tile_n / b_row boxes [kc rows][b_row bytes], one per atom.
-            auto load_b = [&](uint32_t dst, uint32_t bar, int chunk, int tap, int n0) {
-                if (!p.b_mn) {
-                    ptx::tma_load_3d(dst, &map_b, bar, chunk * p.kc, tap, n0);
-                } else {
-                    const uint32_t atom = (uint32_t)p.kc * p.b_row;
-                    for (int a = 0, na = p.tile_n / p.b_row; a < na; ++a)
-                        ptx::tma_load_3d(dst + a * atom, &map_b, bar, n0 + a * p.b_row, tap, chunk * p.kc);
-                }
-            };
-            if (pl.b_resident) {
-                ptx::mbar_expect_tx(b_full(0), (uint32_t)pl.chunks * taps * b_sub);
-                for (int c = 0; c < pl.chunks; ++c)
-                    for (int t = 0; t < taps; ++t)
-                        load_b(b_region + (c * taps + t) * b_sub, b_full(0), c, (int)p.tap_b[t], 0);
-                // completion is observed by the MMA thread, which every path out of this kernel waits for
+    } else if (warp == 2) {
+        // ---------------------------------------------------------------------- weight loads
+        // One sub-tile = the weights of one tap for kc reduction channels and tile_n columns.  K-major: one box
+        // [tile_n rows][kc bytes].  MN-major: tile_n / b_row boxes [kc rows][b_row bytes], one per atom.
+        auto load_b = [&](uint32_t dst, uint32_t bar, int chunk, int tap, int n0) {
+            if (!p.b_mn) {
+                ptx::tma_load_3d(dst, &map_b, bar, chunk * p.kc, tap, n0);
             } else {
-                // Two loaders take turns: one thread gets a sub-tile out only every few hundred cycles (error back-propagation
-                // of the 256-channel 14 x 14 layer at batch 64: 25.4 -> 22.4 us).
-                int ib = warp - 2;
-                bool mine = warp == 2;
-                uint32_t phb = 0, inflight = 0, inflight_parity = 0;
-                bool ok = true;
-                for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-                    const int nt = tile % p.num_n_tiles;
-                    for (int c = 0; c < pl.chunks && ok; ++c)
-                        for (int t = 0; t < taps; ++t, mine = !mine) {
-                            if (!mine) continue;
-                            if (!(ok = wait_bar<64>(b_empty(ib), phb ^ 1u, ctx))) break;
-                            ptx::mbar_expect_tx(b_full(ib), b_sub);
-                            load_b(b_region + ib * b_sub, b_full(ib), c, (int)p.tap_b[t], nt * p.tile_n);
-                            inflight |= 1u << ib;
-                            inflight_parity = (inflight_parity & ~(1u << ib)) | (phb << ib);
-                            ib += 2;
-                            if (ib >= pl.num_b) { ib -= pl.num_b; phb ^= 1u; }   // (num_b is at least 2)
-                        }
-                }
-                if (!ok)
-                    for (int s = 0; s < pl.num_b; ++s)
-                        if (inflight & (1u << s))
-                            for (uint32_t i = 0; i < kSpinLimit; ++i)
-                                if (ptx::mbar_try_wait(b_full(s), (inflight_parity >> s) & 1u)) break;
+                const uint32_t atom = (uint32_t)p.kc * p.b_row;
+                for (int a = 0, na = p.tile_n / p.b_row; a < na; ++a)
+                    ptx::tma_load_3d(dst + a * atom, &map_b, bar, n0 + a * p.b_row, tap, chunk * p.kc);
             }
+        };
+        if (pl.b_resident) {
+            // a lane per sub-tile: what a thread computes between two loads is most of a load's time
+            const int subs = pl.chunks * taps;
+            if (lane == 0) ptx::mbar_expect_tx(b_full(0), (uint32_t)subs * b_sub);
+            __syncwarp();
+            for (int i = lane; i < subs; i += 32) {
+                const int c = i / taps, t = i - c * taps;
+                load_b(b_region + i * b_sub, b_full(0), c, (int)p.tap_b[t], 0);
+            }
+            // completion is observed by the MMA thread, which every path out of this kernel waits for
+        } else {
+            // A lane per ring slot, each filling its own as it falls free: a single thread gets a sub-tile out only every few hundred
+            // cycles.
+            const int per_tile = pl.chunks * taps;
+            const int left = num_tiles > (int)blockIdx.x ? (num_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+            const int total = left * per_tile;
+            int seq = lane < pl.num_b ? lane : total, tile = blockIdx.x;
+            int c = lane / taps, t = lane - c * taps;
+            for (; c >= pl.chunks; c -= pl.chunks) tile += gridDim.x;
+            int nt = tile % p.num_n_tiles;
+            uint32_t ph = 0, polls = 0;
+            bool loaded = false, ok = true;
+            while (__any_sync(0xffffffffu, ok && seq < total)) {
+                bool filled = false;
+                if (ok && seq < total) {
+                    if (ptx::mbar_test_wait(b_empty(lane), ph ^ 1u)) {
+                        ptx::mbar_expect_tx(b_full(lane), b_sub);
+                        load_b(b_region + lane * b_sub, b_full(lane), c, (int)p.tap_b[t], nt * p.tile_n);
+                        filled = loaded = true;
+                        ph ^= 1u;
+                        seq += pl.num_b;
+                        t += pl.num_b;
+                        while (t >= taps) { t -= taps; ++c; }
+                        if (c >= pl.chunks) {
+                            for (; c >= pl.chunks; c -= pl.chunks) tile += gridDim.x;
+                            nt = tile % p.num_n_tiles;
+                        }
+                        polls = 0;
+                    } else if (*ctx.abort_flag) {
+                        ok = false;
+                    } else if (++polls >= kSpinLimit) {
+                        *ctx.abort_flag = 1u;
+                        atomicOr(&p.dev->status, EOQ_DEV_TIMEOUT);
+                        ok = false;
+                    }
+                }
+                if (!__any_sync(0xffffffffu, filled)) __nanosleep(32);
+            }
+            if (!ok && loaded)   // wait, bounded, for the slot's copy in flight
+                for (uint32_t i = 0; i < kSpinLimit; ++i)
+                    if (ptx::mbar_try_wait(b_full(lane), ph ^ 1u)) break;
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------------- MMA issuer (whole warp, see elect_one)
@@ -284,26 +327,21 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
         const FwdShift sh = forward_shift(p, shift);
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
         bool ok = true;
-        // (column tile, image, row tile in the image) of the current tile, carried from tile to tile: the step
-        // between two tiles of this pair is constant, so its quotients are formed once instead of four integer
-        // divisions per tile and warp
         const int tile0 = blockIdx.x + grp * gridDim.x, step = p.ep_groups * gridDim.x;
-        int nt = tile0 % p.num_n_tiles, mt0 = tile0 / p.num_n_tiles;
-        int img = mt0 / pl.tiles_per_img, ti = mt0 % pl.tiles_per_img;
-        const int step_nt = step % p.num_n_tiles, step_mt = step / p.num_n_tiles;
-        const int step_img = step_mt / pl.tiles_per_img, step_ti = step_mt % pl.tiles_per_img;
+        TilePos at = tile_pos(tile0, p.num_n_tiles, pl.tiles_per_img);
+        const TilePos at_step = tile_pos(step, p.num_n_tiles, pl.tiles_per_img);
         for (int tile = tile0; tile < num_tiles && ok; tile += step) {
-            const int y = ti * pl.r_rows + yl;
+            const int y = at.ti * pl.r_rows + yl;
             const bool valid = yl < pl.r_rows && xx < p.wq && y < p.hq;
             size_t pix = 0;
             int cls = 0;
             if (valid) {
-                pix = ((size_t)img * p.hq + y) * p.wq + xx;
+                pix = ((size_t)at.img * p.hq + y) * p.wq + xx;
                 if (p.b1_table)
                     cls = border_class(y, p.hq, p.b1_nlo_h, p.b1_nhi_h, p.b1_nrc) * p.b1_ncc +
                           border_class(xx, p.wq, p.b1_nlo_w, p.b1_nhi_w, p.b1_ncc);
             }
-            int col = nt * p.tile_n + g_begin * 16;
+            int col = at.nt * p.tile_n + g_begin * 16;
             size_t off = pix * p.N + col;
             const int4 zero4 = make_int4(0, 0, 0, 0);
             // the shortcut codes do not depend on the sums: the first group's are requested before the wait for the MMAs
@@ -340,12 +378,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(tempty_bar(grp));
             acc_phase ^= 1u;
-            nt += step_nt;
-            ti += step_ti;
-            if (nt >= p.num_n_tiles) { nt -= p.num_n_tiles; ++ti; }
-            img += step_img;
-            if (ti >= pl.tiles_per_img) { ti -= pl.tiles_per_img; ++img; }
-            if (ti >= pl.tiles_per_img) { ti -= pl.tiles_per_img; ++img; }
+            at.advance(at_step, p.num_n_tiles, pl.tiles_per_img);
         }
         if (!fwd) {
             mx = warp_max_u32(mx);

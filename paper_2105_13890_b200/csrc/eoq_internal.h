@@ -218,7 +218,7 @@ struct PatchPlan {
     int num_a, num_b;   // ring depths (patches, weight sub-tiles)
     int b_resident;     // all weight sub-tiles of the layer stay in shared memory
 };
-constexpr int kPatchThreads = 128 + 32 * kEpilogueWarps;  // warps: 0 patch loads, 1 MMA + TMEM, 2 and 3 weight loads, then the epilogue
+constexpr int kPatchThreads = 128 + 32 * kEpilogueWarps;  // warps: 0 patch loads, 1 MMA + TMEM, 2 weight loads, then the epilogue
 
 size_t igemm_patch_smem_bytes(const IgemmParams &p, const PatchPlan &pl);
 cudaError_t launch_igemm_patch(const IgemmParams &p, const PatchPlan &pl, const CUtensorMap &map_a,
