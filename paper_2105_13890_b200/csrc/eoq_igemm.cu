@@ -204,8 +204,10 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                 if (!(ok = __all_sync(0xffffffffu, wait_bar(full_bar(stage), phase, ctx)))) break;
                 ptx::tc_fence_after();
                 const int subs = min(p.subs_per_stage, p.num_sub - kit * p.subs_per_stage);
-                uint32_t a_lo = ((smem_base + stage * stage_bytes) >> 4) | a_lead;
-                uint32_t b_lo = (((smem_base + stage * stage_bytes) >> 4) + p.subs_per_stage * a_sub16) | b_lead;
+                // (a descriptor's address has 14 bits; in a cluster, shared-memory addresses carry the CTA's rank above them)
+                const uint32_t stage16 = ((smem_base + stage * stage_bytes) >> 4) & 0x3FFFu;
+                uint32_t a_lo = stage16 | a_lead;
+                uint32_t b_lo = (stage16 + p.subs_per_stage * a_sub16) | b_lead;
                 if (wide && k_steps >= 2) {
                     // 2 or 4 MMAs per sub-tile, alternating between the two partial accumulators
                     for (int j = 0; j < subs; ++j) {
