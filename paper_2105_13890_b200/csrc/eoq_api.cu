@@ -251,7 +251,20 @@ void plan_epilogue(IgemmParams &p, int grid)
     if (p.tile_n / 16 < 4 / p.ep_groups) p.ep_groups = p.tile_n >= 32 ? 2 : 4;   // at least one 16-column group per warp
 }
 
-// Shared tiling choices of the implicit GEMM: K sub-tiles, pipeline depth, column tile.
+// Columns of a tile and CTAs that share one, with what follows from them.
+void set_columns(IgemmParams &p, int tile_n, int split)
+{
+    p.tile_n = tile_n;
+    p.num_n_tiles = (p.N + tile_n - 1) / tile_n;
+    p.split = split;
+    p.b_row = p.b_mn ? chunk_bytes(tile_n) : 0;
+    const size_t stage = (size_t)p.subs_per_stage * (kTileM + tile_n) * p.kc;
+    // (a split's exchange takes a tile's worth of shared memory from the stages)
+    const int stages = (int)((200 * 1024 - (split > 1 ? (size_t)kTileM * tile_n * sizeof(int32_t) : 0)) / stage);
+    p.num_stages = stages > 8 ? 8 : (stages < 2 ? 2 : stages);
+}
+
+// Shared tiling choices of the implicit GEMM: K sub-tiles, pipeline depth, column tile.  (p.b_mn is set before.)
 void plan_igemm(IgemmParams &p, int src_channels, int ntaps, int sm_count)
 {
     p.kc = chunk_bytes(src_channels);
@@ -266,54 +279,66 @@ void plan_igemm(IgemmParams &p, int src_channels, int ntaps, int sm_count)
     // up, so tiles stay 128 wide even when that leaves some SMs without one; 256 when there are tiles to spare.
     int tn = p.N < 256 ? p.N : 256;
     if (tn == 256 && (long long)p.num_m_tiles * ((p.N + 255) / 256) < 2LL * sm_count) tn = 128;
-    p.tile_n = tn;
-    p.num_n_tiles = (p.N + tn - 1) / tn;
-    p.split = 1;
+    set_columns(p, tn, 1);
     p.a_rows = kTileM;   // a problem of fewer pixels loads no more of them (TMA time goes by rows; the rest of the tile is never stored)
     while (p.a_rows > 16 && p.M <= p.a_rows / 2) p.a_rows /= 2;
-    const size_t stage = (size_t)p.subs_per_stage * (kTileM + tn) * p.kc;
-    int stages = (int)((200 * 1024) / stage);
-    p.num_stages = stages > 8 ? 8 : (stages < 2 ? 2 : stages);
 }
 
-// SM cycles of one K iteration of the im2col kernel: a TMA row takes 3.1
-double igemm_iteration_cycles(const IgemmParams &p)
-{
-    return 3.1 * p.subs_per_stage * (p.a_rows + (p.b_mn ? p.kc * (p.tile_n / p.b_row) : p.tile_n));
-}
+// ---- problems of few tiles (small batches)
+// Where the tiles leave at least half of the CTAs idle, everything runs at once and the time of one tile counts: narrower tiles then
+// (shorter epilogues, fewer weights per CTA), several CTAs per tile (a cluster, see igemm_kernel), and whichever of the two kernels
+// is faster.  The estimates are in microseconds of a kernel in a chain of its like, fitted to layers of 1 to 13 images; what they
+// choose against the wide tiles before: 128 channels 28 x 28, one image: 6.1 -> 4.3 (32 columns, patch kernel); 256 channels
+// 14 x 14: 7.1 -> 5.3; 512 channels 7 x 7: 7.6 -> 5.8 (128 columns, 8 CTAs a tile), 3.6 of which any kernel takes.
+constexpr double kFewPerCta = 0.0025;   // a CTA more to bring up
+// bytes of a TMA row: its time
+double few_row(int bytes) { return 0.0004 + 3.4e-6 * bytes; }
 
-// CTAs that share a tile (see igemm_kernel): a cluster of 2, 4 or 8 where few tiles leave at least half of the `ctas` CTAs idle
-// and the shorter reductions save more than a sixth of the kernel; the exchange costs about 4,000 cycles.  Wants every CTA to
-// have a K iteration and its part of the columns.  Returns the estimated cycles.
-double plan_split(IgemmParams &p, int ctas)
+double few_igemm_time(const IgemmParams &p)
 {
-    const int tiles = p.num_m_tiles * p.num_n_tiles, groups = p.tile_n / 16;
     const int k_iters = (p.num_sub + p.subs_per_stage - 1) / p.subs_per_stage;
-    const double per_iter = igemm_iteration_cycles(p), whole = k_iters * per_iter;
-    double best = whole;
-    p.split = 1;
-    if (p.kc < 64 || p.tile_n > 128) return whole;
-    for (int s = 2; s <= 8; s *= 2) {
-        if (groups % s || groups / s > 4 || k_iters < s || tiles * s > ctas / 2) continue;
-        const double cost = (k_iters + s - 1) / s * per_iter + 4000.0;
-        if (cost < best && 6 * cost < 5 * whole + 6000.0) {   // (6,000: what a kernel spends beside its reduction)
-            best = cost;
-            p.split = s;
+    const int iters = (k_iters + p.split - 1) / p.split, rows = p.M < kTileM ? p.M : kTileM;
+    const double load = 0.0009 * p.subs_per_stage * (p.a_rows + (p.b_mn ? p.kc * (p.tile_n / p.b_row) : p.tile_n));
+    const double mma = 0.0485 * p.subs_per_stage * (p.kc < 32 ? 0.5 : p.kc / 32);   // (92 cycles each, with their waits and commits)
+    double t = 3.6 + iters * (load > mma ? load : mma) + 6e-5 * rows * p.tile_n / p.split +
+               kFewPerCta * p.num_m_tiles * p.num_n_tiles * p.split;
+    if (p.split > 1) t += 0.3 + 0.025 * rows * p.tile_n * 4 / 1024.0;   // the exchange
+    return t;
+}
+
+// Columns per tile and CTAs per tile of the im2col kernel.  Clusters take at most half of the CTAs (beyond that many, some wait for
+// room: 512 channels 7 x 7, one image: 64 CTAs 5.9 us, 128 CTAs 6.7) and want every CTA to have a K iteration of at least two MMAs.
+void plan_few_tiles(IgemmParams &p, int ctas)
+{
+    if (2 * p.num_m_tiles * p.num_n_tiles > ctas) return;
+    const int k_iters = (p.num_sub + p.subs_per_stage - 1) / p.subs_per_stage;
+    IgemmParams best = p;
+    double best_time = few_igemm_time(p);
+    for (int cuts = 1; cuts <= 32; cuts *= 2) {
+        const int tn = ((p.N + cuts - 1) / cuts + 15) / 16 * 16;
+        if (tn > 128) continue;
+        for (int split = 1; split <= 8; split *= 2) {
+            if (split > 1 && (p.kc < 64 || k_iters < split || tn / 16 > 4 * split)) continue;
+            IgemmParams q = p;
+            set_columns(q, tn, split);
+            if (q.num_m_tiles * q.num_n_tiles * split > (split > 1 ? ctas / 2 : ctas)) continue;
+            const double time = few_igemm_time(q);
+            if (time < 0.97 * best_time) {
+                best = q;
+                best_time = time;
+            }
         }
+        if (tn == 16) break;
     }
-    if (p.split > 1) {   // the exchange takes a tile's worth of shared memory from the stages
-        const size_t stage = (size_t)p.subs_per_stage * (kTileM + p.tile_n) * p.kc;
-        const int stages = (int)((200 * 1024 - (size_t)kTileM * p.tile_n * sizeof(int32_t)) / stage);
-        p.num_stages = stages > 8 ? 8 : (stages < 2 ? 2 : stages);
-    }
-    return best;
+    p = best;
 }
 
 // Plan of the patch variant for a stride-1 k x k correlation over a source [n][hs][ws][c_src] producing a
 // [n][hq][wq] grid with n_cols columns.  Returns false when the geometry does not suit it (then the per-tap
 // path is used): strided or 1x1 filters, rows too wide for a tile, or tiles that would be mostly padding.
+// `ctas`: that the launch may use; `columns`: of a tile, 0 for the plan's own choice.
 bool plan_patch(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, int wq, int k, int pad_src, int n_cols,
-                int sm_count)
+                int sm_count, int ctas, int columns = 0)
 {
     if (k < 2 || c_src % 16 || pad_src < 0 || pad_src > k - 1) return false;
     const int pw = wq + k - 1;
@@ -350,12 +375,18 @@ bool plan_patch(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, int
         auto waves = [&](int cols) { return ((long long)p.num_m_tiles * ((n_cols + cols - 1) / cols) + sm_count - 1) / sm_count; };
         if (7 * waves(256) >= 5 * waves(128)) tn = 128;
     }
+    if (columns) tn = columns;
     p.tile_n = tn;
     p.num_n_tiles = (n_cols + tn - 1) / tn;
+    p.b_row = p.b_mn ? chunk_bytes(tn) : 0;
     const size_t budget = 200 * 1024;
     const size_t b_sub = (size_t)tn * p.kc;
     const size_t b_all = b_sub * pl.chunks * p.ntaps;
-    pl.b_resident = (p.num_n_tiles == 1 && b_all + 2 * (size_t)pl.a_bytes <= budget && b_all < (1u << 20)) ? 1 : 0;
+    // resident where the tiles of a CTA share their weights: one column tile, or one tile per CTA (which needs one patch buffer, two
+    // if it has several chunks)
+    const bool one_tile = (long long)p.num_m_tiles * p.num_n_tiles <= ctas;
+    pl.b_resident = ((p.num_n_tiles == 1 || one_tile) && b_all + (one_tile && pl.chunks == 1 ? 1 : 2) * (size_t)pl.a_bytes <= budget &&
+                     b_all < (1u << 20)) ? 1 : 0;
     if (pl.b_resident) {
         size_t na = (budget - b_all) / pl.a_bytes;
         // 64 channels 56 x 56, batch 512: 152 us with at most 4 patches in flight, 140 with 6, 145 with 8
@@ -370,21 +401,45 @@ bool plan_patch(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, int
     return pl.num_a >= 2 || (pl.b_resident && pl.num_a >= 1);
 }
 
-// Is a cluster per tile in the im2col kernel faster than the patch kernel's plan?  (A patch tile costs its MMAs, about 1.45
-// times 57 cycles each, 100 beyond 64 columns, with what surrounds them.)  Only problems of few tiles get a split.
-bool split_beats_patch(const IgemmParams &patch, int c_src, bool b_mn, int ctas)
+double few_patch_time(const IgemmParams &p, const PatchPlan &pl)
 {
-    if (patch.num_m_tiles * patch.num_n_tiles > ctas / 4) return false;
-    IgemmParams q;
-    memset(&q, 0, sizeof(q));
-    q.M = patch.M;
-    q.N = patch.N;
-    plan_igemm(q, c_src, patch.ntaps, ctas);
-    q.b_mn = b_mn ? 1 : 0;
-    q.b_row = chunk_bytes(q.tile_n);
-    const double split = plan_split(q, ctas);
-    const double mmas = (double)patch.ntaps * patch.chunks_per_tap * patch.kc / 32;
-    return q.split > 1 && split < 1.45 * mmas * (patch.tile_n <= 64 ? 57.0 : 100.0);
+    const int subs = pl.chunks * p.ntaps, mmas = subs * (p.kc / 32);
+    const double weights = p.b_mn ? p.kc * (p.tile_n / p.b_row) * few_row(p.b_row) : p.tile_n * few_row(p.kc);
+    // weights through the ring: about 0.3 us a sub-tile, with its wait and commit; resident ones arrive in front of the MMAs
+    const double body = pl.b_resident ? subs * weights + mmas * (p.tile_n > 114 ? 0.034 : 0.028) : subs * 0.3;
+    return 3.0 + body + 4e-5 * kTileM * p.tile_n + kFewPerCta * p.num_m_tiles * p.num_n_tiles;
+}
+
+// Plan of a stride-1 k x k correlation (p.b_mn says how the weights are read); false: the im2col kernel takes it.
+bool plan_stride1(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, int wq, int k, int pad_src, int n_cols, int sm_count,
+                  int ctas)
+{
+    if (!plan_patch(p, pl, n_img, c_src, hq, wq, k, pad_src, n_cols, sm_count, ctas)) return false;
+    if (2 * p.num_m_tiles * p.num_n_tiles > ctas) return true;
+    double time = few_patch_time(p, pl);
+    for (int cuts = 2; cuts <= 32; cuts *= 2) {
+        const int tn = ((n_cols + cuts - 1) / cuts + 15) / 16 * 16;
+        IgemmParams q = p;
+        PatchPlan ql = pl;
+        if (!plan_patch(q, ql, n_img, c_src, hq, wq, k, pad_src, n_cols, sm_count, ctas, tn)) continue;
+        if (q.num_m_tiles * q.num_n_tiles > ctas) break;
+        const double t = few_patch_time(q, ql);
+        if (t < 0.97 * time) {
+            time = t;
+            p = q;
+            pl = ql;
+        }
+        if (tn == 16) break;
+    }
+    IgemmParams g;
+    memset(&g, 0, sizeof(g));
+    g.M = p.M;
+    g.N = p.N;
+    g.b_mn = p.b_mn;
+    plan_igemm(g, c_src, p.ntaps, sm_count);
+    plan_few_tiles(g, ctas);
+    // (with fewer than 32 channels per chunk the im2col kernel reads a transposed copy of the weights: a kernel more)
+    return few_igemm_time(g) + (p.b_mn && c_src % 32 ? 3.0 : 0.0) > 0.97 * time;
 }
 
 // Plan of the patch variant of the weight gradient; false when the geometry does not suit it.
@@ -916,8 +971,7 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
     PatchPlan pl;
     memset(&pl, 0, sizeof(pl));
     const bool patch = d.stride == 1 && d.kh == d.kw && d.x_wmargin == 0 &&
-                       plan_patch(p, pl, d.n, d.c_in, g.ho, g.wo, d.kh, d.pad, d.c_out, h->sm_count) &&
-                       !split_beats_patch(p, d.c_in, false, h->gemm_ctas);
+                       plan_stride1(p, pl, d.n, d.c_in, g.ho, g.wo, d.kh, d.pad, d.c_out, h->sm_count, h->gemm_ctas);
     p.M = d.n * g.ho * g.wo;
     p.N = d.c_out;
     p.hq = g.ho;
@@ -954,7 +1008,7 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
             p.tap_dw[t] = (unsigned char)(t % d.kw);
             p.tap_b[t] = (unsigned char)t;
         }
-        plan_split(p, h->gemm_ctas);
+        plan_few_tiles(p, h->gemm_ctas);
     }
     p.out_h = g.ho;
     p.out_w = g.wo;
@@ -1182,8 +1236,10 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
         memset(&p, 0, sizeof(p));
         PatchPlan pl;
         memset(&pl, 0, sizeof(pl));
-        if (plan_patch(p, pl, d.n, d.c_out, d.h, d.w, d.kh, d.kh - 1 - d.pad, d.c_in, h->sm_count) &&
-            !split_beats_patch(p, d.c_out, true, h->gemm_ctas)) {
+        // the weights are read where they are, [c_out][tap][c_in]: the reduction (c_out) is their slow axis, so
+        // they reach the MMA as MN-major atoms of b_row input channels
+        p.b_mn = 1;
+        if (plan_stride1(p, pl, d.n, d.c_out, d.h, d.w, d.kh, d.kh - 1 - d.pad, d.c_in, h->sm_count, h->gemm_ctas)) {
             for (int a = 0; a < d.kh; ++a)
                 for (int b = 0; b < d.kw; ++b) p.tap_b[a * d.kw + b] = (unsigned char)((d.kh - 1 - a) * d.kw + (d.kw - 1 - b));
             p.out_h = d.h;
@@ -1195,10 +1251,6 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.sums16 = sums16;
             p.dev = h->dev;
             p.next_mask = next ? next->mask : nullptr;
-            // the weights are read where they are, [c_out][tap][c_in]: the reduction (c_out) is their slow axis, so
-            // they reach the MMA as MN-major atoms of b_row input channels
-            p.b_mn = 1;
-            p.b_row = chunk_bytes(p.tile_n);
             CUtensorMap map_a, map_b;
             if (!make_patch_map(&map_a, e3, d.n, g.ho, g.wo, d.c_out, p.kc, pl.pw, pl.r_rows + d.kh - 1) ||
                 !make_weight_map(&map_b, w, d.c_out, g.taps, d.c_in, p.b_row, p.kc))
@@ -1301,6 +1353,7 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.N = d.c_in;
             p.hq = hq;
             p.wq = wq;
+            p.b_mn = weights_in_place ? 1 : 0;
             plan_igemm(p, d.c_out, nh * nw, h->sm_count);
             p.src_stride = 1;
             p.src_stride_w = 1;
@@ -1325,35 +1378,28 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.sums16 = sums16;
             p.dev = h->dev;
             p.next_mask = next ? next->mask : nullptr;
+            // a tile costs its taps and, about half of one, its sums: by taps alone the class of one tap ended last
+            int ctas = h->gemm_ctas;
+            if (side_by_side) ctas = (int)((long long)h->gemm_ctas * (2 * nh * nw + 1) / (2 * total_taps + live_classes));
+            if (ctas < 1) ctas = 1;
+            plan_few_tiles(p, ctas);
             CUtensorMap map_a, map_b;
-            if (weights_in_place) {
-                p.b_mn = 1;
-                p.b_row = chunk_bytes(p.tile_n);
-            }
             if (!make_im2col_map(&map_a, e3, d.n, g.ho, g.wo, d.c_out, min_w, min_h, wq, hq, 1, p.kc, p.a_rows) ||
                 !(weights_in_place ? make_weight_map(&map_b, w, d.c_out, g.taps, d.c_in, p.b_row, p.kc)
                                    : make_weight_map(&map_b, wt, d.c_in, g.taps, d.c_out, p.kc, p.tile_n)))
                 return EOQ_ERR_UNSUPPORTED;
-            const int tiles = p.num_m_tiles * p.num_n_tiles;
             count_launches(h, 1);
             cudaStream_t cs = s;
-            int ctas = h->gemm_ctas;
-            if (side_by_side) {
-                // a tile costs its taps and, about half of one, its sums: by taps alone the class of one tap ended last
-                ctas = (int)((long long)h->gemm_ctas * (2 * nh * nw + 1) / (2 * total_taps + live_classes));
-                if (ctas < 1) ctas = 1;
-                if (class_no > 0) {
-                    const int k = (class_no - 1) % kClassBranches;
-                    cs = h->class_branch[k];
-                    // a stream that already carries a class of this call simply queues the next one behind it
-                    if (!(joins & (1u << k))) e = cudaStreamWaitEvent(cs, h->fork_ev, 0);
-                    if (e != cudaSuccess) return record(h, e);
-                    joins |= 1u << k;
-                }
+            if (side_by_side && class_no > 0) {
+                const int k = (class_no - 1) % kClassBranches;
+                cs = h->class_branch[k];
+                // a stream that already carries a class of this call simply queues the next one behind it
+                if (!(joins & (1u << k))) e = cudaStreamWaitEvent(cs, h->fork_ev, 0);
+                if (e != cudaSuccess) return record(h, e);
+                joins |= 1u << k;
             }
             ++class_no;
-            plan_split(p, ctas);
-            const int grid = persistent_grid(tiles, ctas);
+            const int grid = persistent_grid(p.num_m_tiles * p.num_n_tiles, ctas);
             plan_epilogue(p, grid);
             if (side_by_side) {
                 e = launch_igemm(p, map_a, map_b, grid * p.split, cs);
@@ -1701,8 +1747,7 @@ extern "C" int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *des
     buf[0] = 0;
     if (pass == EOQ_PASS_FWD) {
         if (d.stride == 1 && d.kh == d.kw && d.x_wmargin == 0 &&
-            plan_patch(p, pl, d.n, d.c_in, g.ho, g.wo, d.kh, d.pad, d.c_out, h->sm_count) &&
-            !split_beats_patch(p, d.c_in, false, h->gemm_ctas)) {
+            plan_stride1(p, pl, d.n, d.c_in, g.ho, g.wo, d.kh, d.pad, d.c_out, h->sm_count, h->gemm_ctas)) {
             snprintf(buf, buf_bytes, "kernel=igemm_patch tile_n=%d accumulators=%d m_tiles=%d n_tiles=%d weights=%s", p.tile_n,
                      p.tile_n <= 128 ? 2 : 1, p.num_m_tiles, p.num_n_tiles, pl.b_resident ? "resident" : "streamed");
             return EOQ_OK;
@@ -1711,15 +1756,15 @@ extern "C" int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *des
         p.N = d.c_out;
         const bool rw = use_row_window(d, g.wo);
         plan_igemm(p, rw ? 8 * d.c_in : d.c_in, rw ? d.kh : g.taps, h->sm_count);
-        if (!rw) plan_split(p, h->gemm_ctas);
+        if (!rw) plan_few_tiles(p, h->gemm_ctas);
         snprintf(buf, buf_bytes, "kernel=igemm%s tile_n=%d m_tiles=%d n_tiles=%d kc=%d stages=%d split=%d", rw ? "_filter_rows" : "",
                  p.tile_n, p.num_m_tiles, p.num_n_tiles, p.kc, p.num_stages, p.split);
         return EOQ_OK;
     }
     if (pass == EOQ_PASS_DGRAD) {
+        p.b_mn = 1;
         if (d.stride == 1 && d.kh == d.kw && d.kh - 1 - d.pad >= 0 &&
-            plan_patch(p, pl, d.n, d.c_out, d.h, d.w, d.kh, d.kh - 1 - d.pad, d.c_in, h->sm_count) &&
-            !split_beats_patch(p, d.c_out, true, h->gemm_ctas)) {
+            plan_stride1(p, pl, d.n, d.c_out, d.h, d.w, d.kh, d.kh - 1 - d.pad, d.c_in, h->sm_count, h->gemm_ctas)) {
             snprintf(buf, buf_bytes, "kernel=igemm_patch tile_n=%d accumulators=%d m_tiles=%d n_tiles=%d weights=%s", p.tile_n,
                      p.tile_n <= 128 ? 2 : 1, p.num_m_tiles, p.num_n_tiles, pl.b_resident ? "resident" : "streamed");
             return EOQ_OK;
@@ -1727,9 +1772,11 @@ extern "C" int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *des
         const int hq = (d.h + d.stride - 1) / d.stride, wq = (d.w + d.stride - 1) / d.stride;
         p.M = d.n * hq * wq;
         p.N = d.c_in;
+        p.b_mn = d.c_out % 32 == 0;
         plan_igemm(p, d.c_out, ((d.kh + d.stride - 1) / d.stride) * ((d.kw + d.stride - 1) / d.stride), h->sm_count);
-        snprintf(buf, buf_bytes, "kernel=igemm classes=%d tile_n=%d m_tiles=%d n_tiles=%d kc=%d", d.stride * d.stride, p.tile_n,
-                 p.num_m_tiles, p.num_n_tiles, p.kc);
+        if (d.stride == 1) plan_few_tiles(p, h->gemm_ctas);
+        snprintf(buf, buf_bytes, "kernel=igemm classes=%d tile_n=%d m_tiles=%d n_tiles=%d kc=%d split=%d", d.stride * d.stride, p.tile_n,
+                 p.num_m_tiles, p.num_n_tiles, p.kc, p.split);
         return EOQ_OK;
     }
     if (pass == EOQ_PASS_WGRAD) {

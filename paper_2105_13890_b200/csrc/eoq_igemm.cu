@@ -20,8 +20,10 @@ constexpr int kProducers = 3;
 
 // kEpi: EpilogueKind; forward and dgrad are kernels of their own (registers, code size).
 // kSplit: a cluster of p.split CTAs shares one tile.  Each runs its part of the reduction, hands every other CTA the partial
-// sums of that CTA's columns through distributed shared memory, and takes the epilogue of its own columns.  Small batches
-// leave a handful of tiles with long reductions: the 512-channel 7 x 7 layer at batch 1 took 13.3 us on 4 CTAs.
+// sums of that CTA's share of the (column group, pixel) pairs through distributed shared memory, and takes the epilogue of its own
+// share.  Small batches leave a handful of tiles with long reductions: the 512-channel 7 x 7 layer at batch 1 took 13.3 us on
+// 4 CTAs.  The exchange is the price, bound by distributed shared memory: with whole tiles of 128 rows exchanged by columns it was
+// 3.5 us of that layer's 7.4 on 32 CTAs; of the 49 pixels that exist it takes about 1 us.
 template <int kEpi, bool kSplit>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUtensorMap map_a,
@@ -252,12 +254,22 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         const int ew = (warp - 4) >> 2;
         // (In a cluster all of them are one group, whatever the number of columns: each must reach the cluster's barrier.)
         const int parts = kSplit ? 4 : 4 / p.ep_groups, grp = kSplit ? 0 : ew / parts, part = ew - grp * parts;
-        const int row = quad * 32 + lane;
         const int groups = p.tile_n / 16;                 // 16-column groups of the tile
-        const int own = kSplit ? groups / p.split : 1;    // groups whose epilogue is this CTA's (at most four)
-        const int g_begin = kSplit ? rank * own + part : (groups * part) / parts;
-        const int g_end = kSplit ? g_begin + (part < own ? 1 : 0) : (groups * (part + 1)) / parts;
-        const uint32_t red_base = smem_base + p.num_stages * stage_bytes + kTableSmemBytes;   // [source CTA][own group][4][row] x 16 bytes
+        int row = quad * 32 + lane;
+        int g_begin = (groups * part) / parts, g_end = (groups * (part + 1)) / parts;
+        // A cluster deals out its tile's (column group, pixel) pairs, pixels that exist only, in equal shares: one pair per epilogue
+        // thread.  Cells of the exchange: [source CTA][4][pair of the share] x 16 bytes.
+        const int rows_in = kSplit ? min(kTileM, p.M - tile_first / p.num_n_tiles * kTileM) : kTileM;
+        const int share = kSplit ? (groups * rows_in + p.split - 1) / p.split : 0;
+        const uint32_t red_base = smem_base + p.num_stages * stage_bytes + kTableSmemBytes;
+        bool mine = true;
+        if (kSplit) {
+            const int tid = (int)threadIdx.x - 128, pair = rank * share + tid;
+            mine = tid < share && pair < groups * rows_in;
+            g_begin = mine ? pair / rows_in : 0;
+            g_end = g_begin + 1;
+            row = mine ? pair - g_begin * rows_in : 0;
+        }
         constexpr bool fwd = kEpi == kEpiForward;
         const FwdScalars fs = fwd ? load_fwd_scalars(p) : FwdScalars{0, 0, 0};
         // the b1 table of the whole layer goes to shared memory (behind the pipeline stages), once, times b1
@@ -271,7 +283,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         for (int tile = tile_first + grp * gridDim.x; tile < num_tiles && ok; tile += p.ep_groups * gridDim.x) {
             const int mt = tile / p.num_n_tiles, nt = tile % p.num_n_tiles;
             const int m = mt * kTileM + row;
-            const bool valid = m < p.M;
+            const bool valid = m < p.M && mine;
             size_t pix = 0;
             int cls = 0;
             if (valid) {
@@ -293,8 +305,9 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
             ptx::tc_fence_after();
             const uint32_t t_row = tmem_base + grp * buf_stride + ((uint32_t)(quad * 32) << 16);
             if (kSplit) {
+                const int r_own = quad * 32 + lane;   // the tensor-memory lane of this thread
 #pragma unroll 1
-                for (int g = part; g < groups && ok; g += 4) {
+                for (int g = part; g < groups && ok && quad * 32 < rows_in; g += 4) {
                     uint32_t r[32], r2[32];
                     ptx::tmem_ld_32x16(t_row + g * 16, r);
                     if (nacc == 2) ptx::tmem_ld_32x16(t_row + acc_stride + g * 16, r2);
@@ -303,10 +316,13 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
 #pragma unroll
                         for (int i = 0; i < 16; ++i) r[i] += r2[i];
                     }
-                    const uint32_t dst = ptx::cluster_addr(red_base + (((rank * own + g % own) * 4) * kTileM + row) * 16, g / own);
+                    if (r_own < rows_in) {
+                        const int pair = g * rows_in + r_own, owner = pair / share, slot = pair - owner * share;
+                        const uint32_t dst = ptx::cluster_addr(red_base + (rank * 4 * share + slot) * 16, owner);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        ptx::st_cluster_128(dst + c * kTileM * 16, r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+                        for (int c = 0; c < 4; ++c)
+                            ptx::st_cluster_128(dst + c * share * 16, r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+                    }
                 }
                 ptx::cluster_sync();
             }
@@ -317,17 +333,18 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                 if (kSplit) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) r[i] = 0;
-#pragma unroll 1
-                    for (int src = 0; src < p.split; ++src) {
+                    if (mine)
+#pragma unroll 2
+                        for (int src = 0; src < p.split; ++src) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const int4 v = ptx::ld_shared_128(red_base + (((src * own + part) * 4 + c) * kTileM + row) * 16);
-                            r[4 * c] += v.x;
-                            r[4 * c + 1] += v.y;
-                            r[4 * c + 2] += v.z;
-                            r[4 * c + 3] += v.w;
+                            for (int c = 0; c < 4; ++c) {
+                                const int4 v = ptx::ld_shared_128(red_base + ((src * 4 + c) * share + (int)threadIdx.x - 128) * 16);
+                                r[4 * c] += v.x;
+                                r[4 * c + 1] += v.y;
+                                r[4 * c + 2] += v.z;
+                                r[4 * c + 3] += v.w;
+                            }
                         }
-                    }
                 } else {
                     ptx::tmem_ld_32x16(t_row + g * 16, r);
                     if (nacc == 2) ptx::tmem_ld_32x16(t_row + acc_stride + g * 16, r2);
@@ -380,7 +397,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
 size_t igemm_smem_bytes(const IgemmParams &p)
 {
     return (size_t)p.num_stages * p.subs_per_stage * ((size_t)kTileM + p.tile_n) * p.kc + 1024 + kTableSmemBytes +
-           (p.split > 1 ? (size_t)kTileM * p.tile_n * sizeof(int32_t) : 0);
+           (p.split > 1 ? (size_t)kTileM * p.tile_n * sizeof(int32_t) + 64 * p.split : 0);   // (shares are rounded up)
 }
 
 cudaError_t launch_igemm(const IgemmParams &p, const CUtensorMap &map_a, const CUtensorMap &map_b, int grid,

@@ -8,7 +8,7 @@
 // is loaded ONCE per channel chunk; filter tap (a, b) is the same shared-memory tile read through a descriptor
 // whose start address is (a * pw + b) rows further (the swizzle is a function of the address, so a row shift
 // keeps operand and descriptor consistent).  Output rows that fall in the (k - 1) extra columns are computed and
-// dropped.  Weights either stay resident in shared memory for the whole kernel (when the layer's weights fit) or
+// dropped.  Weights either stay resident in shared memory for the whole kernel (when those of the CTA's column tile fit) or
 // stream through their own ring.
 //
 // Roles: warp 0 patch loads, warp 1 TMEM owner + tcgen05.mma issuer, warp 2 weight loads, warps 4-19 epilogue
@@ -155,13 +155,14 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
             }
         };
         if (pl.b_resident) {
-            // a lane per sub-tile: what a thread computes between two loads is most of a load's time
-            const int subs = pl.chunks * taps;
+            // a lane per sub-tile: what a thread computes between two loads is most of a load's time (all tiles of this CTA lie in
+            // one column tile)
+            const int subs = pl.chunks * taps, n0 = (int)(blockIdx.x % (unsigned)p.num_n_tiles) * p.tile_n;
             if (lane == 0) ptx::mbar_expect_tx(b_full(0), (uint32_t)subs * b_sub);
             __syncwarp();
             for (int i = lane; i < subs; i += 32) {
                 const int c = i / taps, t = i - c * taps;
-                load_b(b_region + i * b_sub, b_full(0), c, (int)p.tap_b[t], 0);
+                load_b(b_region + i * b_sub, b_full(0), c, (int)p.tap_b[t], n0);
             }
             // completion is observed by the MMA thread, which every path out of this kernel waits for
         } else {

@@ -216,7 +216,7 @@ struct PatchPlan {
     int a_bytes;        // bytes of one patch buffer (multiple of 1024)
     int a_box_bytes;    // bytes one patch load delivers
     int num_a, num_b;   // ring depths (patches, weight sub-tiles)
-    int b_resident;     // all weight sub-tiles of the layer stay in shared memory
+    int b_resident;     // all weight sub-tiles of a column tile stay in shared memory (then a CTA's tiles all lie in one)
 };
 constexpr int kPatchThreads = 128 + 32 * kEpilogueWarps;  // warps: 0 patch loads, 1 MMA + TMEM, 2 weight loads, then the epilogue
 
