@@ -277,7 +277,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                                                  (int)threadIdx.x - 128, 32 * kEpilogueWarps)
                                 : nullptr;
         const int shift = input_shift(p);
-        const FwdShift sh = forward_shift(p, shift);
+        const FwdShift sh = forward_shift(p, fs, shift);
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
         bool ok = true;
         for (int tile = tile_first + grp * gridDim.x; tile < num_tiles && ok; tile += p.ep_groups * gridDim.x) {

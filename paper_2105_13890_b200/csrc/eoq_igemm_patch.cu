@@ -40,7 +40,7 @@ struct TilePos {
 };
 __device__ __forceinline__ TilePos tile_pos(int tile, int num_n_tiles, int tiles_per_img)
 {
-    const int mt = tile / num_n_tiles, img = mt / tiles_per_img;
+    const int mt = num_n_tiles == 1 ? tile : tile / num_n_tiles, img = mt / tiles_per_img;
     return TilePos{tile - mt * num_n_tiles, img, mt - img * tiles_per_img};
 }
 
@@ -99,12 +99,9 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
         ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), tmem_cols);
         ptx::tmem_relinquish();
     }
-    // the patch loader's first tile and its step from tile to tile (formed while the kernels in front still run)
-    TilePos pos = {}, by = {};
-    if (warp == 0) {
-        pos = tile_pos((int)blockIdx.x, p.num_n_tiles, pl.tiles_per_img);
-        by = tile_pos((int)gridDim.x, p.num_n_tiles, pl.tiles_per_img);
-    }
+    // the patch loader's first tile (formed while the kernels in front still run)
+    TilePos pos = {};
+    if (warp == 0) pos = tile_pos((int)blockIdx.x, p.num_n_tiles, pl.tiles_per_img);
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
@@ -122,6 +119,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
             int ia = 0;
             uint32_t pha = 0, inflight = 0, inflight_parity = 0;
             bool ok = true;
+            TilePos by = {};   // formed behind the first loads
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
                 const int y0 = pos.ti * pl.r_rows;
                 for (int c = 0; c < pl.chunks; ++c) {
@@ -133,6 +131,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
                     inflight_parity = (inflight_parity & ~(1u << ia)) | (pha << ia);
                     if (++ia == pl.num_a) { ia = 0; pha ^= 1u; }
                 }
+                if (tile == (int)blockIdx.x) by = tile_pos((int)gridDim.x, p.num_n_tiles, pl.tiles_per_img);
                 pos.advance(by, p.num_n_tiles, pl.tiles_per_img);
             }
             if (!ok)
@@ -155,14 +154,21 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
             }
         };
         if (pl.b_resident) {
-            // a lane per sub-tile: what a thread computes between two loads is most of a load's time (all tiles of this CTA lie in
-            // one column tile)
+            // A CTA of one tile waits for the last of its weights: a lane per sub-tile then, since what a thread computes between two
+            // loads is most of a load's time (128 channels 28 x 28, one image: 4.9 -> 4.4 us).  With several tiles the weights keep
+            // out of the way of the patches behind the first (16 channels 32 x 32, batch 128: 9.8 -> 9.3 us).
+            // (All tiles of a CTA lie in one column tile.)
             const int subs = pl.chunks * taps, n0 = (int)(blockIdx.x % (unsigned)p.num_n_tiles) * p.tile_n;
             if (lane == 0) ptx::mbar_expect_tx(b_full(0), (uint32_t)subs * b_sub);
             __syncwarp();
-            for (int i = lane; i < subs; i += 32) {
-                const int c = i / taps, t = i - c * taps;
-                load_b(b_region + i * b_sub, b_full(0), c, (int)p.tap_b[t], n0);
+            if ((int)gridDim.x >= num_tiles) {
+                for (int i = lane; i < subs; i += 32) {
+                    const int c = i / taps, t = i - c * taps;
+                    load_b(b_region + i * b_sub, b_full(0), c, (int)p.tap_b[t], n0);
+                }
+            } else if (lane == 0) {
+                for (int c = 0; c < pl.chunks; ++c)
+                    for (int t = 0; t < taps; ++t) load_b(b_region + (c * taps + t) * b_sub, b_full(0), c, (int)p.tap_b[t], n0);
             }
             // completion is observed by the MMA thread, which every path out of this kernel waits for
         } else {
@@ -325,7 +331,7 @@ igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant_
                                                  (int)threadIdx.x - 128, 32 * kEpilogueWarps)
                                 : nullptr;
         const int shift = fwd ? input_shift(p) : 7;
-        const FwdShift sh = forward_shift(p, shift);
+        const FwdShift sh = forward_shift(p, fs, shift);
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
         bool ok = true;
         const int tile0 = blockIdx.x + grp * gridDim.x, step = p.ep_groups * gridDim.x;

@@ -44,3 +44,21 @@ def test_few_tiles(d, relu):
     if relu:
         assert np.array_equal(G.unpack_mask(mask, out), ref["mask"])
     assert np.array_equal(G.host(e4), want) and e4_exp.item() == p and total.item() == int(want.astype(np.int64).sum())
+
+
+@pytest.mark.parametrize("b2", [0, 3, -5, 16384, -16384, 16385, -32768, 32767])
+@pytest.mark.parametrize("relu", [True, False])
+def test_unit_gamma_without_shortcut(relu, b2):
+    """gamma = 1 and no shortcut: x5 comes from one rounding, with b2 in its limits (|b2| <= 2^14) or by the general chain; ties at both parities."""
+    d = oracle.ConvDesc(2, 9, 20, 32, 48, 3, 3, 1, 1)
+    x0, w = synth.int8_uniform((d.n, d.h, d.w, d.c_in), 2710, 1), synth.normal_codes((d.c_out, d.kh, d.kw, d.c_in), 2711, 2, std_codes=40 if abs(b2) > 100 else 2)
+    x0 = (x0 // 16 * 16).astype(np.int8)   # sums in steps of 16: every eighth is a tie
+    ref = oracle.layer_forward(d, x0, -2, w, 128, b2, None, relu)
+    out = (d.n, d.ho, d.wo, d.c_out)
+    gd = G.gdesc(d)
+    for keep in (False, True):   # without x2, and with it (the general chain)
+        x5, mask = G.zeros(out, torch.int8), G.zeros((ref["x5"].size + 7) // 8, torch.uint8)
+        x2 = G.zeros(out, torch.int16) if keep else None
+        eoq.eoq_conv_fwd(G.handle(), gd, G.dev(x0), None, -2, G.dev(w), 128, b2, None, relu, x5, x2, mask, None, G.workspace(gd, eoq.EOQ_PASS_FWD))
+        assert G.status_clear() == 0
+        assert np.array_equal(G.host(x5), ref["x5"]) and np.array_equal(G.unpack_mask(mask, out), ref["mask"])
