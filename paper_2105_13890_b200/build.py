@@ -14,7 +14,7 @@ LIB = os.path.join(HERE, "libeoq.so")
 # Tagged with the interpreter it is built for: CPython's ABI changes between versions, and another interpreter then builds a
 # module of its own instead of loading this one.
 BIND = os.path.join(HERE, "_eoqbind" + EXTENSION_SUFFIXES[0])
-SOURCES = ["eoq_api.cu", "eoq_igemm.cu", "eoq_igemm_patch.cu", "eoq_wgrad_patch.cu", "eoq_wgrad.cu", "eoq_wgrad_rows.cu", "eoq_finish.cu", "eoq_elementwise.cu", "eoq_update.cu", "eoq_static.cu", "eoq_probe.cu", "eoq_aux.cu", "eoq_pool.cu", "eoq_head.cu", "eoq_bn.cu"]
+SOURCES = ["eoq_api.cu", "eoq_igemm.cu", "eoq_igemm_patch.cu", "eoq_igemm_rows.cu", "eoq_wgrad_patch.cu", "eoq_wgrad.cu", "eoq_wgrad_rows.cu", "eoq_finish.cu", "eoq_elementwise.cu", "eoq_update.cu", "eoq_static.cu", "eoq_probe.cu", "eoq_aux.cu", "eoq_pool.cu", "eoq_head.cu", "eoq_bn.cu"]
 HEADERS = ["eoq_internal.h", "eoq_cells.cuh", "eoq_device.cuh", "eoq_epilogue.cuh", "eoq_next_head.cuh", os.path.join(ROOT, "include", "eoq.h")]
 
 

@@ -129,6 +129,19 @@ bool make_patch_map(CUtensorMap *map, const void *ptr, int n, int h, int w, int 
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Tiled view of the rows of an NHWC int8 tensor, `row_bytes` each (a multiple of 16), in 8-byte units: a box of `box8` units of
+// `box_rows` rows.
+bool make_input_rows_map(CUtensorMap *map, const void *ptr, int n, int h, size_t row_bytes, int box8, int box_rows)
+{
+    cuuint64_t dims[3] = {(cuuint64_t)row_bytes / 8, (cuuint64_t)h, (cuuint64_t)n};
+    cuuint64_t strides[2] = {(cuuint64_t)row_bytes, (cuuint64_t)row_bytes * h};
+    cuuint32_t box[3] = {(cuuint32_t)box8, (cuuint32_t)box_rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<void *>(ptr), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Tiled view of a [rows][taps][c] int8 tensor with a (box_c, 1, box_rows) box.
 bool make_weight_map(CUtensorMap *map, const void *ptr, int rows, int taps, int c, int box_c, int box_rows)
 {
@@ -440,6 +453,56 @@ bool plan_stride1(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, i
     plan_few_tiles(g, ctas);
     // (with fewer than 32 channels per chunk the im2col kernel reads a transposed copy of the weights: a kernel more)
     return few_igemm_time(g) + (p.b_mn && c_src % 32 ? 3.0 : 0.0) > 0.97 * time;
+}
+
+// Plan of the input-row forward kernel for a filter-row layer (see use_row_window); false: the im2col kernel takes it.
+bool plan_rows(IgemmParams &p, RowsPlan &pl, const eoq_conv_desc_t &d, const Geometry &g, int ctas)
+{
+    if (d.stride * d.c_in != 16 || d.c_out > 128 || (d.w + 2 * d.x_wmargin) * d.c_in % 16 || (d.x_wmargin - d.pad) * d.c_in % 16) return false;
+    memset(&pl, 0, sizeof(pl));
+    pl.n_img = d.n;
+    pl.stride = d.stride;
+    pl.pad = d.pad;
+    // a box row has at most 256 units of 8 bytes: 125 windows of 8 channels, 121 of 16
+    const int most_px = (2048 - 8 * d.c_in) / 16 + 1;
+    pl.x_tiles = (g.wo + most_px - 1) / most_px;
+    pl.tile_px = (g.wo + pl.x_tiles - 1) / pl.x_tiles;
+    pl.first_col8 = (d.x_wmargin - d.pad) * d.c_in / 8;
+    pl.row_pitch = 16 * (pl.tile_px - 1) + 8 * d.c_in;
+    pl.slack = (16 * (kTileM - 1) + 8 * d.c_in - pl.row_pitch + 127) / 128 * 128;
+    p.kc = 8 * d.c_in;
+    p.ntaps = d.kh;
+    p.tile_n = d.c_out;
+    p.num_n_tiles = 1;
+    p.split = 1;
+    const long long budget = 200 * 1024 - (long long)p.ntaps * p.tile_n * p.kc - pl.slack;
+    // Output rows per patch: a CTA's rows at about 1,100 cycles each and 150 per patch, and the load of its first patch (35 bytes a
+    // cycle) in front of them.
+    double best = 0;
+    for (int r = 1; r <= 16 && r <= g.ho; ++r) {
+        const int rows_in = (r - 1) * d.stride + d.kh;
+        const long long bytes = ((long long)rows_in * pl.row_pitch + 127) / 128 * 128;
+        if (rows_in > 256 || 2 * bytes > budget) break;
+        const int blocks = (g.ho + r - 1) / r;
+        const long long patches = (long long)d.n * blocks * pl.x_tiles;
+        const int per_cta = (int)((patches + ctas - 1) / ctas);
+        const double load = rows_in * pl.row_pitch / 35.0, rows = r * 1100.0 + 150.0;
+        const double cost = load + per_cta * (rows > load ? rows : load);
+        if (pl.r_rows == 0 || cost < best) {
+            best = cost;
+            pl.r_rows = r;
+            pl.row_blocks = blocks;
+            pl.a_box_bytes = rows_in * pl.row_pitch;
+            pl.a_bytes = (int)bytes;
+            const long long na = budget / bytes;
+            pl.num_a = na > 4 ? 4 : (int)na;
+        }
+    }
+    if (!pl.r_rows) return false;
+    const long long patches = (long long)d.n * pl.row_blocks * pl.x_tiles;
+    if (patches > 0x7fffffff) return false;
+    p.num_m_tiles = (int)patches;   // (for the grid; the epilogue's groups go by output rows)
+    return true;
 }
 
 // Plan of the patch variant of the weight gradient; false when the geometry does not suit it.
@@ -979,11 +1042,14 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
     p.src_stride = d.stride;
     p.base_h = -d.pad;
     int8_t *w_rows = nullptr;
+    RowsPlan rp;
+    bool by_rows = false;
     if (patch) {
         for (int t = 0; t < g.taps; ++t) p.tap_b[t] = (unsigned char)t;
     } else if (row_window) {
         // K sub-tile = one filter row (8 pixels x c_in channels); the map's W axis already steps by the stride
-        plan_igemm(p, 8 * d.c_in, d.kh, h->sm_count);
+        by_rows = plan_rows(p, rp, d, g, h->gemm_ctas);
+        if (!by_rows) plan_igemm(p, 8 * d.c_in, d.kh, h->sm_count);
         p.src_stride_w = 1;
         p.base_w = 0;
         for (int t = 0; t < d.kh; ++t) {
@@ -1051,6 +1117,17 @@ static int conv_fwd_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const
         const int grid = persistent_grid(ptiles, h->gemm_ctas);
         plan_epilogue(p, grid);
         return record(h, launch_igemm_patch(p, pl, map_a, map_b, grid, s));
+    }
+    if (by_rows) {
+        if (!make_input_rows_map(&map_a, x, d.n, d.h, (size_t)w_mem * d.c_in, rp.row_pitch / 8, (rp.r_rows - 1) * d.stride + d.kh) ||
+            !make_weight_map(&map_b, w_rows, d.c_out, d.kh, 8 * d.c_in, 8 * d.c_in, p.tile_n))
+            return EOQ_ERR_UNSUPPORTED;
+        count_launches(h, 1);
+        ProfScope prof(h, EOQ_PROF_IGEMM_FWD, s);
+        const int grid = persistent_grid(p.num_m_tiles, h->gemm_ctas), rows = (p.num_m_tiles + grid - 1) / grid * rp.r_rows;
+        p.ep_groups = rows >= 3 && p.tile_n <= 64 ? 4 : (rows >= 2 || p.tile_n < 64 ? 2 : 1);
+        if (p.tile_n / 16 < 4 / p.ep_groups) p.ep_groups = p.tile_n >= 32 ? 2 : 4;   // at least one 16-column group per warp
+        return record(h, launch_igemm_rows(p, rp, map_a, map_b, grid, s));
     }
     if (row_window) {
         if (!make_row_window_map(&map_a, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, g.wo, g.ho, d.stride, d.pad, p.a_rows) ||
@@ -1755,6 +1832,12 @@ extern "C" int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *des
         p.M = d.n * g.ho * g.wo;
         p.N = d.c_out;
         const bool rw = use_row_window(d, g.wo);
+        RowsPlan rp;
+        if (rw && plan_rows(p, rp, d, g, h->gemm_ctas)) {
+            snprintf(buf, buf_bytes, "kernel=igemm_input_rows tile_n=%d rows_per_patch=%d patches=%d pixels=%d", p.tile_n, rp.r_rows, p.num_m_tiles,
+                     rp.tile_px);
+            return EOQ_OK;
+        }
         plan_igemm(p, rw ? 8 * d.c_in : d.c_in, rw ? d.kh : g.taps, h->sm_count);
         if (!rw) plan_few_tiles(p, h->gemm_ctas);
         snprintf(buf, buf_bytes, "kernel=igemm%s tile_n=%d m_tiles=%d n_tiles=%d kc=%d stages=%d split=%d", rw ? "_filter_rows" : "",

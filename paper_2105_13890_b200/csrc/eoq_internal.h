@@ -224,6 +224,22 @@ size_t igemm_patch_smem_bytes(const IgemmParams &p, const PatchPlan &pl);
 cudaError_t launch_igemm_patch(const IgemmParams &p, const PatchPlan &pl, const CUtensorMap &map_a,
                                const CUtensorMap &map_b, int grid, cudaStream_t stream);
 
+// Forward of a first layer whose windows start 16 bytes apart (eoq_igemm_rows.cu): an M tile is one output row, of tile_px pixels
+// where it is wider; a patch of input rows serves r_rows of them.
+struct RowsPlan {
+    int n_img, stride, pad;
+    int r_rows;       // output rows per patch
+    int row_blocks;   // patches down an image
+    int x_tiles, tile_px;
+    int first_col8;   // where the first window starts in an input row, in 8-byte units
+    int row_pitch;    // bytes of an input row of the patch
+    int a_bytes, a_box_bytes, num_a;   // a patch buffer, what a load delivers, buffers
+    int slack;        // bytes behind the last buffer that its last pixels' windows may reach into (their sums are dropped)
+};
+size_t igemm_rows_smem_bytes(const IgemmParams &p, const RowsPlan &pl);
+cudaError_t launch_igemm_rows(const IgemmParams &p, const RowsPlan &pl, const CUtensorMap &map_a, const CUtensorMap &map_b, int grid,
+                              cudaStream_t stream);
+
 size_t igemm_smem_bytes(const IgemmParams &p);
 cudaError_t launch_igemm(const IgemmParams &p, const CUtensorMap &map_a, const CUtensorMap &map_b, int grid,
                          cudaStream_t stream);
