@@ -56,6 +56,15 @@ __device__ __forceinline__ int32_t sbyte(uint32_t w)
     return (int32_t)r;
 }
 
+// sum of the products of four signed bytes with four unsigned ones, plus c: with one byte of b set to 128 it scales and adds
+// one code without the byte extraction, which would go to the busier pipe
+__device__ __forceinline__ uint32_t dot4_s8_u8(uint32_t a, uint32_t b, uint32_t c)
+{
+    uint32_t d;
+    asm("dp4a.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
 // R(log2 M) for M >= 1: floor(log2 M) plus one when M^2 >= 2^(2f+1).
 __device__ __forceinline__ int round_log2_u32(uint32_t M)
 {
@@ -160,60 +169,33 @@ __device__ __forceinline__ void sums_pack_16(const uint32_t *acc, uint32_t mx, u
 // Was the group shortened?
 __device__ __forceinline__ bool sums_shortened(uint32_t w0) { return ((w0 ^ (w0 << 1)) & 0x8000u) != 0; }
 
-// The sums of a shortened group, their lost bits zero but for the or-ed one.
-__device__ __forceinline__ void sums_restore_16(const uint32_t (&w)[8], int32_t (&a)[16])
+// s of a shortened group; its marked words get their bit 15 back.
+__device__ __forceinline__ int sums_unmark(uint32_t (&w)[8])
 {
     const uint32_t d0 = w[0] ^ (w[0] << 1), d1 = w[1] ^ (w[1] << 1), d2 = w[2] ^ (w[2] << 1);
-    const int s = (int)((d0 >> 31) | (d1 >> 14 & 2u) | (d1 >> 29 & 4u) | (d2 >> 12 & 8u) | (d2 >> 27 & 16u));
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        a[2 * i] = (int32_t)((uint32_t)((int32_t)(w[i] << 17) >> 17) << s);
-        a[2 * i + 1] = (int32_t)((uint32_t)((int32_t)(w[i] << 1) >> 17) << s);
-    }
+    for (int i = 0; i < 3; ++i) w[i] = (w[i] & 0x7fff7fffu) | ((w[i] << 1) & 0x80008000u);
+    return (int)((d0 >> 31) | (d1 >> 14 & 2u) | (d1 >> 29 & 4u) | (d2 >> 12 & 8u) | (d2 >> 27 & 16u));
 }
 
-// Codes of SQ for 16 sums under a shift s known to the whole kernel.  Sums that were not shortened go to their codes on the
-// floating-point pipe: 2^23 + (sum + 2^15) is a float whose bits are put together from the word, and one fused multiply-add
-// forms 1.5 * 2^23 + sum / 2^s, rounded to nearest even at unit spacing (every constant is exact for -7 <= s <= 15; a larger s
-// leaves only zeros, as 15 does).
-struct SumCode {
-    int t, sh;
-    float scale, rest;
-    int32_t half_m1, lo;   // of sq_pack4_shr, for shortened groups (their tensor's shift is at least 7)
-};
-__device__ __forceinline__ SumCode sum_code_setup(int t)
+// Codes of SQ for 16 sums under a shift known to the whole kernel (t = R(log2 max)), on the floating-point pipe: 2^23 + (word +
+// 2^15) is a float whose bits are put together from the word, and one fused multiply-add forms 1.5 * 2^23 + word / 2^n, rounded to
+// nearest even at unit spacing.  n = t - 7, less s in a shortened group.  Every constant is exact for -7 <= n <= 15; a larger n
+// leaves only zeros, as 15 does (-2^14 / 2^15 is a tie and goes to 0).
+__device__ __forceinline__ void sum_codes_16(int t, uint32_t (&w)[8], uint32_t (&cw)[4])
 {
-    SumCode c;
-    c.t = t;
-    c.sh = t - 7;
-    c.scale = __int_as_float((127 - min(c.sh, 15)) << 23);
-    c.rest = 12582912.0f - 8421376.0f * c.scale;
-    const int sh = max(c.sh, 1);
-    c.half_m1 = (1 << (sh - 1)) - 1;
-    c.lo = -(127 << sh);
-    return c;
-}
-__device__ __forceinline__ void sum_codes_16(const SumCode &c, const uint32_t (&w)[8], uint32_t (&cw)[4])
-{
-    if (!sums_shortened(w[0])) {
-        auto code = [&](uint32_t u, uint32_t sel) {
-            const float f = __fmaf_rn(__uint_as_float(__byte_perm(u, 0x4B00u, sel)), c.scale, c.rest);
-            return __viaddmax_s32((int32_t)__float_as_uint(f), -0x4B400000, -127);
-        };
+    int n = t - 7;
+    if (sums_shortened(w[0])) n -= sums_unmark(w);
+    const float scale = __int_as_float((127 - min(n, 15)) << 23), rest = 12582912.0f - 8421376.0f * scale;
+    auto code = [&](uint32_t u, uint32_t sel) {
+        const float f = __fmaf_rn(__uint_as_float(__byte_perm(u, 0x4B00u, sel)), scale, rest);
+        return __viaddmax_s32((int32_t)__float_as_uint(f), -0x4B400000, -127);
+    };
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t u0 = w[2 * q] ^ 0x80008000u, u1 = w[2 * q + 1] ^ 0x80008000u;
-            cw[q] = pack4_sat(code(u0, 0x5410), code(u0, 0x5432), code(u1, 0x5410), code(u1, 0x5432));
-        }
-        return;
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t u0 = w[2 * q] ^ 0x80008000u, u1 = w[2 * q + 1] ^ 0x80008000u;
+        cw[q] = pack4_sat(code(u0, 0x5410), code(u0, 0x5432), code(u1, 0x5410), code(u1, 0x5432));
     }
-    int32_t a[16];
-    sums_restore_16(w, a);
-    const bool fits = c.t <= 30;   // (sq_pack4_shr wants the largest sum and half a step to stay below 2^31)
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        cw[q] = fits ? sq_pack4_shr(a + 4 * q, c.sh, c.half_m1, c.lo)
-                     : pack4_sat(sq_code32(a[4 * q], c.t), sq_code32(a[4 * q + 1], c.t), sq_code32(a[4 * q + 2], c.t), sq_code32(a[4 * q + 3], c.t));
 }
 
 // Expands 4 mask bits into 4 byte masks (0x00 / 0xff).

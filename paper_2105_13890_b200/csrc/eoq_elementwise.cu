@@ -307,38 +307,41 @@ __global__ void sq_i32_kernel(const void *__restrict__ src_any, const int32_t *s
     __shared__ uint32_t cell_s[2];
     const size_t n16 = n / 16;
     const int32_t *const src = static_cast<const int32_t *>(src_any);
-    uint32_t raw[kPacked ? 8 : 16];   // a group of 16 sums
+    // a group of 16 sums, and what a join wants beside it
+    struct Group {
+        uint32_t raw[kPacked ? 8 : 16];
+        int4 b;
+        uint32_t gate, nm;
+    } cur = {};
     const bool wide_in = (reinterpret_cast<uintptr_t>(src) & 31) == 0;
-    auto load16 = [&](size_t i) {
+    auto load16 = [&](size_t i, Group &to) {
         if constexpr (kPacked) {
-            ld_global_256_stream(static_cast<const uint16_t *>(src_any) + i * 16, raw);
+            ld_global_256_stream(static_cast<const uint16_t *>(src_any) + i * 16, to.raw);
         } else if (wide_in) {   // two 256-bit loads: whole 32-byte sectors per lane
-            ld_global_256_stream(src + i * 16, raw);
-            ld_global_256_stream(src + i * 16 + 8, raw + 8);
+            ld_global_256_stream(src + i * 16, to.raw);
+            ld_global_256_stream(src + i * 16 + 8, to.raw + 8);
         } else {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int4 v = __ldcs(reinterpret_cast<const int4 *>(src) + i * 4 + k);
-                raw[4 * k + 0] = v.x;
-                raw[4 * k + 1] = v.y;
-                raw[4 * k + 2] = v.z;
-                raw[4 * k + 3] = v.w;
+                to.raw[4 * k + 0] = v.x;
+                to.raw[4 * k + 1] = v.y;
+                to.raw[4 * k + 2] = v.z;
+                to.raw[4 * k + 3] = v.w;
             }
         }
+        if (kJoin) {
+            to.b = __ldg(reinterpret_cast<const int4 *>(join.b) + i);
+            to.gate = join.mask_b ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(join.mask_b) + i) : 0xffffu;
+            to.nm = join.next_mask ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(join.next_mask) + i) : 0u;
+        }
+        if (kNext) to.nm = (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(next.mask) + i);
     };
     // the first group of every thread is on its way while the maxima are read
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n16) {
-        load16(i);
-        if (kJoin) {
-            ptx::prefetch_l1(join.b + i * 16);
-            if (join.mask_b) ptx::prefetch_l1(join.mask_b + i * 2);
-            if (join.next_mask) ptx::prefetch_l1(join.next_mask + i * 2);
-        }
-        if (kNext) {
-            ptx::prefetch_l1(next.mask + i * 2);
-            if (next.x2) ptx::prefetch_l1(next.x2 + i * 16);
-        }
+        load16(i, cur);
+        if (kNext && next.x2) ptx::prefetch_l1(next.x2 + i * 16);
     }
     bool last = false;
     if (threadIdx.x == 0) {
@@ -361,26 +364,28 @@ __global__ void sq_i32_kernel(const void *__restrict__ src_any, const int32_t *s
     long long sum = 0, s1 = 0, s2 = 0;
     const int sh = t - 7;
     JoinShift js = {0, 0, 0};
-    bool j_narrow = true;
-    int j_ma = 1, j_mb = 1;
+    JoinMul jm = {};
     unsigned long long jmx = 0, jmxm = 0;
     if (kJoin) {
         js = join_shift(p0, __ldg(join.b_exp));
-        j_narrow = js.sa >= 0 && js.sb >= 0 && js.sa <= 23 && js.sb <= 23;
-        j_ma = 1 << (js.sa < 0 ? 0 : min(js.sa, 23));
-        j_mb = 1 << (js.sb < 0 ? 0 : min(js.sb, 23));
+        jm = join_mul(js);
     }
     // the maximum bounds every element, so |a| + 2^(sh-1) cannot wrap as long as M + M / 2^7 < 2^31
     const bool fast = sh >= 1 && M < 0x7e000000u;
     const int32_t half_m1 = fast ? (1 << (sh - 1)) - 1 : 0, lo = fast ? -(127 << sh) : 0;
-    const SumCode sc = sum_code_setup(t);
     uint32_t jm32 = 0, jmm32 = 0;
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
     while (i < n16) {
+        Group ahead = {};   // the thread's next group travels while this one is worked on
+        if (i + stride < n16) {
+            load16(i + stride, ahead);
+            if (kNext && next.x2) ptx::prefetch_l1(next.x2 + (i + stride) * 16);
+        }
         uint32_t cw[4];   // four codes per word
         if constexpr (kPacked) {
-            sum_codes_16(sc, raw, cw);
+            sum_codes_16(t, cur.raw, cw);
         } else {
-            const int32_t *a = reinterpret_cast<const int32_t *>(raw);
+            const int32_t *a = reinterpret_cast<const int32_t *>(cur.raw);
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 cw[q] = fast ? sq_pack4_shr(a + 4 * q, sh, half_m1, lo)
@@ -392,22 +397,31 @@ __global__ void sq_i32_kernel(const void *__restrict__ src_any, const int32_t *s
         sum += sum16;
         reinterpret_cast<int4 *>(dst)[i] = make_int4((int)cw[0], (int)cw[1], (int)cw[2], (int)cw[3]);
         if (kJoin) {
-            const int4 bq = __ldg(reinterpret_cast<const int4 *>(join.b) + i);
-            const uint32_t gate = join.mask_b ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(join.mask_b) + i) : 0xffffu;
-            const uint32_t nm = join.next_mask ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(join.next_mask) + i) : 0u;
-            const uint32_t bw[4] = {(uint32_t)bq.x, (uint32_t)bq.y, (uint32_t)bq.z, (uint32_t)bq.w};
+            const uint32_t bw[4] = {(uint32_t)cur.b.x, (uint32_t)cur.b.y, (uint32_t)cur.b.z, (uint32_t)cur.b.w};
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const uint32_t g = bw[q] & bits_to_bytes(gate >> (4 * q)), m = nm >> (4 * q);
-                const int bv[4] = {sbyte<0>(g), sbyte<1>(g), sbyte<2>(g), sbyte<3>(g)};
-                const int cv[4] = {sbyte<0>(cw[q]), sbyte<1>(cw[q]), sbyte<2>(cw[q]), sbyte<3>(cw[q])};
+                const uint32_t g = bw[q] & bits_to_bytes(cur.gate >> (4 * q)), m = cur.nm >> (4 * q);
+                if (!jm.wide) {
+                    int32_t v[4];
+                    if (jm.near) {
+                        uint32_t u[4];
+                        join_near(jm, cw[q], g, 0u, u);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (j_narrow) {
-                        const uint32_t u = (uint32_t)abs(cv[k] * j_ma + bv[k] * j_mb);
-                        jm32 = max(jm32, u);
-                        if (m & (1u << k)) jmm32 = max(jmm32, u);
+                        for (int k = 0; k < 4; ++k) v[k] = (int32_t)u[k];
                     } else {
+                        join_narrow(jm, cw[q], g, v);
+                    }
+                    const uint32_t u0 = (uint32_t)abs(v[0]), u1 = (uint32_t)abs(v[1]), u2 = (uint32_t)abs(v[2]), u3 = (uint32_t)abs(v[3]);
+                    jm32 = max(max(jm32, u0), max(u1, max(u2, u3)));
+                    if (m & 1u) jmm32 = max(jmm32, u0);
+                    if (m & 2u) jmm32 = max(jmm32, u1);
+                    if (m & 4u) jmm32 = max(jmm32, u2);
+                    if (m & 8u) jmm32 = max(jmm32, u3);
+                } else {
+                    const int bv[4] = {sbyte<0>(g), sbyte<1>(g), sbyte<2>(g), sbyte<3>(g)};
+                    const int cv[4] = {sbyte<0>(cw[q]), sbyte<1>(cw[q]), sbyte<2>(cw[q]), sbyte<3>(cw[q])};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
                         const long long v = join_one(cv[k], bv[k], js);
                         const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
                         jmx = u > jmx ? u : jmx;
@@ -417,7 +431,7 @@ __global__ void sq_i32_kernel(const void *__restrict__ src_any, const int32_t *s
             }
         }
         if (kNext) {
-            const uint32_t bits = (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(next.mask) + i);
+            const uint32_t bits = cur.nm;
             uint32_t e1[4], c3[4];
             int a1 = 0;
 #pragma unroll
@@ -430,8 +444,8 @@ __global__ void sq_i32_kernel(const void *__restrict__ src_any, const int32_t *s
             if (next.x2) s2 += dot16_s8_s16(e1, reinterpret_cast<const int4 *>(next.x2) + 2 * i);
             reinterpret_cast<int4 *>(next.e3)[i] = make_int4((int)c3[0], (int)c3[1], (int)c3[2], (int)c3[3]);
         }
-        i += (size_t)gridDim.x * blockDim.x;
-        if (i < n16) load16(i);
+        i += stride;
+        cur = ahead;
     }
     ptx::grid_dep_launch();
     if (!kPacked)
@@ -495,7 +509,6 @@ __global__ void sq_sums_scatter_kernel(const uint16_t *__restrict__ src, const i
         *dst_exp = M ? p_in + t - 7 : p_in;
         if (!M) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
     }
-    const SumCode code = sum_code_setup(t);
     long long sum = 0;
     const uint32_t groups = (uint32_t)c / 16u;
     const size_t items = (size_t)n_img * hh * ww * groups;  // fits 32 bits (checked by the launcher)
@@ -508,7 +521,7 @@ __global__ void sq_sums_scatter_kernel(const uint16_t *__restrict__ src, const i
             const size_t q = (((size_t)img * hq + y / (uint32_t)stride) * wq + x / (uint32_t)stride) * c + g * 16u;
             uint32_t raw[8], cw[4];
             ld_global_256_stream(src + q, raw);
-            sum_codes_16(code, raw, cw);
+            sum_codes_16(t, raw, cw);
             int sc = 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k) sc = __dp4a((int)cw[k], 0x01010101, sc);

@@ -50,15 +50,6 @@ __device__ __forceinline__ uint32_t rne7_denormal(uint32_t x)
     return __float_as_uint(__fmaf_rn(__uint_as_float(x), __int_as_float((127 + 127) << 23), __uint_as_float(kDenormalBits)));
 }
 
-// sum of the products of four signed bytes with four unsigned ones, plus c: with one byte of b set to 128 it scales and adds
-// one code without the byte extraction, which would go to the busier pipe
-__device__ __forceinline__ uint32_t dot4_s8_u8(uint32_t a, uint32_t b, uint32_t c)
-{
-    uint32_t d;
-    asm("dp4a.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-    return d;
-}
-
 // Forward chain on 16 consecutive output channels of one pixel (Sec. 3.2.1: x2 = Q_a1(conv), x3 = gamma x2,
 // x4 = x3 + b2 [+ shortcut], x5 = Q_a2(relu(x4)); mask = [x4 > 0]).
 // The integer pipe bounds this code (an instruction every two cycles and scheduler), so clamps are moved in front of the

@@ -43,12 +43,19 @@ __device__ __forceinline__ int next_head_code(const NextHead &nh, int e1)
 // at 127
 __device__ __forceinline__ uint32_t next_head_codes(const NextHead &nh, uint32_t e1)
 {
-    const int32_t e[4] = {sbyte<0>(e1), sbyte<1>(e1), sbyte<2>(e1), sbyte<3>(e1)};
+    uint32_t biased[4];
+    if (nh.g < 256u) {   // gamma below 2 (codes below 256): a byte dot product takes its code out of the word and scales it
+#pragma unroll
+        for (int k = 0; k < 4; ++k) biased[k] = dot4_s8_u8(e1, nh.g << (8 * k), kHeadMagic);
+    } else {
+        const int32_t e[4] = {sbyte<0>(e1), sbyte<1>(e1), sbyte<2>(e1), sbyte<3>(e1)};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) biased[k] = nh.g * (uint32_t)e[k] + kHeadMagic;
+    }
     int32_t v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const uint32_t biased = nh.g * (uint32_t)e[k] + kHeadMagic;
-        v[k] = __viaddmax_s32((int32_t)__float_as_uint(__fmaf_rn(__uint_as_float(biased), nh.scale, nh.rest)), -(int32_t)kHeadMagic, -127);
+        v[k] = __viaddmax_s32((int32_t)__float_as_uint(__fmaf_rn(__uint_as_float(biased[k]), nh.scale, nh.rest)), -(int32_t)kHeadMagic, -127);
     }
     return pack4_sat(v[0], v[1], v[2], v[3]);
 }
@@ -76,6 +83,39 @@ __device__ __forceinline__ JoinShift join_shift(int pa, int pb)
     if (j.sa > 31) { j.sb = -1; j.sa = 0; j.p = pa; }        // b lies more than 31 octaves below a
     else if (j.sb > 31) { j.sa = -1; j.sb = 0; j.p = pb; }
     return j;
+}
+// The sums in 32 bits: a factor per operand (0: dropped), unless the exponents lie 24 to 31 octaves apart (`wide`: join_one).
+// `near`: both factors at most 128, so that a byte dot product forms a sum of less than 2^14.
+struct JoinMul {
+    bool wide, near;
+    int ma, mb;
+    uint32_t pair;   // ma | mb << 8
+};
+__device__ __forceinline__ JoinMul join_mul(const JoinShift &j)
+{
+    JoinMul m;
+    m.wide = j.sa > 23 || j.sb > 23;
+    m.near = j.sa <= 7 && j.sb <= 7;
+    m.ma = j.sa < 0 ? 0 : 1 << min(j.sa, 23);
+    m.mb = j.sb < 0 ? 0 : 1 << min(j.sb, 23);
+    m.pair = (uint32_t)(m.ma & 255) | (uint32_t)(m.mb & 255) << 8;
+    return m;
+}
+// four sums of near operands, each plus `bias` (codes of a and b in a word each)
+__device__ __forceinline__ void join_near(const JoinMul &m, uint32_t a, uint32_t b, uint32_t bias, uint32_t (&s)[4])
+{
+    const uint32_t lo = __byte_perm(a, b, 0x5140), hi = __byte_perm(a, b, 0x7362);   // a0 b0 a1 b1, a2 b2 a3 b3
+    s[0] = dot4_s8_u8(lo, m.pair, bias);
+    s[1] = dot4_s8_u8(lo, m.pair << 16, bias);
+    s[2] = dot4_s8_u8(hi, m.pair, bias);
+    s[3] = dot4_s8_u8(hi, m.pair << 16, bias);
+}
+__device__ __forceinline__ void join_narrow(const JoinMul &m, uint32_t a, uint32_t b, int32_t (&s)[4])
+{
+    s[0] = sbyte<0>(a) * m.ma + sbyte<0>(b) * m.mb;
+    s[1] = sbyte<1>(a) * m.ma + sbyte<1>(b) * m.mb;
+    s[2] = sbyte<2>(a) * m.ma + sbyte<2>(b) * m.mb;
+    s[3] = sbyte<3>(a) * m.ma + sbyte<3>(b) * m.mb;
 }
 __device__ __forceinline__ long long join_one(int a, int b, const JoinShift &j)
 {
