@@ -155,12 +155,10 @@ __device__ __forceinline__ void sums_pack_16(const uint32_t *acc, uint32_t mx, u
         return;
     }
     const int s = 18 - __clz(mx);
-    const int32_t rest = (1 << s) - 1;
-    uint32_t m[16];
+    const uint32_t rest = (1u << s) - 1u;
+    auto cut = [&](uint32_t v) { return (uint32_t)((int32_t)(v | ((v & rest) + rest)) >> s); };   // (the sum carries into bit s if any bit is lost)
 #pragma unroll
-    for (int i = 0; i < 16; ++i) m[i] = (uint32_t)(((int32_t)acc[i] >> s) | (((int32_t)acc[i] & rest) ? 1 : 0));
-#pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = __byte_perm(m[2 * i], m[2 * i + 1], 0x5410);
+    for (int i = 0; i < 8; ++i) w[i] = __byte_perm(cut(acc[2 * i]), cut(acc[2 * i + 1]), 0x5410);
     w[0] ^= 0x8000u | (uint32_t)(s & 1) << 31;
     w[1] ^= (uint32_t)(s & 2) << 14 | (uint32_t)(s & 4) << 29;
     w[2] ^= (uint32_t)(s & 8) << 12 | (uint32_t)(s & 16) << 27;
