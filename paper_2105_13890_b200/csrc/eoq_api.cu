@@ -1603,6 +1603,10 @@ static FinishItem finish_item(const eoq_conv_desc_t &d, const Geometry &g, const
 // b1 error sums, sums and Q_g of up to kFinishChunk layers whose GEMMs are in front on the stream.
 static int finish_items(Handle *h, const FinishItem *items, int num, cudaStream_t s)
 {
+    if (num == 1 && !h->profiling && finish_is_small(items[0], h->hook)) {   // (a profile brackets the b1 sums as a kind of their own)
+        count_launches(h, 1);
+        return record(h, launch_finish_small(items[0], &h->dev->status, h->sm_count, s));
+    }
     FinishBatch b;
     plan_finish(b, items, num, h->sm_count, h->hook);
     if (b.tap_first[num] > 0) {

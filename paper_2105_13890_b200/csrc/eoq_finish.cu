@@ -124,21 +124,18 @@ __device__ __forceinline__ bool tap_takes(int y, int k, int stride, int pad, int
     return src >= 0 && src < extent_in;
 }
 
-__global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_constant__ FinishBatch b)
+// Block `local` of the item's tap blocks.  sets: [1 + border rows][1 + border columns][kClassSlab]; index 0 = all rows / columns.
+template <int kT>   // threads of the block
+__device__ __forceinline__ void finish_taps_block(const FinishItem &it, int local, int32_t *sets)
 {
-    ptx::grid_dep_wait();
     __shared__ unsigned long long rows_out[16], cols_out[16];  // per filter row / column: the border rows / columns it does not take
-    extern __shared__ int32_t sets[];  // [1 + border rows][1 + border columns][kClassSlab]; index 0 = all rows / columns
-    const int k = finish_item_of(b.tap_first, b.num, (int)blockIdx.x);
-    const FinishItem &it = b.item[k];
-    if (!it.use_b1) return;
     const eoq_conv_desc_t &d = it.d;
     const BorderClasses &bc = it.bc;
-    const int local = (int)blockIdx.x - b.tap_first[k], bx = local % it.tap_grid_x, by = local / it.tap_grid_x;
+    const int bx = local % it.tap_grid_x, by = local / it.tap_grid_x;
     const int ho = it.ho, wo = it.wo, c_out = d.c_out;
     const int nr = border_count(ho, bc.nlo_h, bc.nhi_h, bc.nrc), nc = border_count(wo, bc.nlo_w, bc.nhi_w, bc.ncc);
     const int nsets = (1 + nr) * (1 + nc);
-    for (int i = threadIdx.x; i < nsets * kClassSlab; i += kThreads) sets[i] = 0;
+    for (int i = threadIdx.x; i < nsets * kClassSlab; i += kT) sets[i] = 0;
     if (threadIdx.x < d.kh) {
         unsigned long long m = 0;
         for (int i = 0; i < nr; ++i)
@@ -163,7 +160,7 @@ __global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_cons
         {   // T
             constexpr int kUnroll = 8;
             const size_t p_end = (size_t)r_end * wo;
-            const int step = (kThreads / 32) * pix_per_step;
+            const int step = (kT / 32) * pix_per_step;
             for (size_t p0 = (size_t)r_begin * wo + warp * pix_per_step; p0 < p_end; p0 += kUnroll * step) {   // the same in all lanes
                 int4 v[kUnroll];
 #pragma unroll
@@ -175,7 +172,7 @@ __global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_cons
             }
             if (acc.count) acc.flush(sets + sub * 16, lanes_per_pix);
         }
-        for (int set = 1 + warp; set < nsets; set += kThreads / 32) {
+        for (int set = 1 + warp; set < nsets; set += kT / 32) {
             constexpr int kUnroll = 4;
             const int i = set / (1 + nc), j = set - i * (1 + nc);
             int32_t *dst = sets + set * kClassSlab + sub * 16;
@@ -209,7 +206,7 @@ __global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_cons
     // the blocks spread their atomics over kTapReplicas copies
     long long *tap_sums = it.tap_sums + (size_t)(bx % kTapReplicas) * it.tap_stride;
     const int taps = d.kh * d.kw;
-    for (int i = threadIdx.x; i < taps * slab_ch; i += kThreads) {   // consecutive threads: neighbouring cells of [oc][tap]
+    for (int i = threadIdx.x; i < taps * slab_ch; i += kT) {   // consecutive threads: neighbouring cells of [oc][tap]
         const int c = i / taps, tap = i - c * taps, kh = tap / d.kw, kw = tap - kh * d.kw;
         const unsigned long long rm = rows_out[kh], cm = cols_out[kw];
         const int32_t *cell = sets + c;
@@ -224,6 +221,14 @@ __global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_cons
             atomicAdd(reinterpret_cast<unsigned long long *>(tap_sums + (size_t)(by * kClassSlab + c) * taps + tap),
                       (unsigned long long)(long long)sum);
     }
+}
+
+__global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_constant__ FinishBatch b)
+{
+    ptx::grid_dep_wait();
+    extern __shared__ int32_t sets[];
+    const int k = finish_item_of(b.tap_first, b.num, (int)blockIdx.x);
+    if (b.item[k].use_b1) finish_taps_block<kThreads>(b.item[k], (int)blockIdx.x - b.tap_first[k], sets);
 }
 
 // ------------------------------------------------------------------ exact sums and their maximum
@@ -411,6 +416,129 @@ __global__ void __launch_bounds__(kThreads) finish_code_kernel(const __grid_cons
     }
 }
 
+// ------------------------------------------------------------------ all of it in one cluster
+// The three steps for one small layer in one launch of a cluster: tap sums into the cells, slice sums into shared memory, their
+// maximum through distributed shared memory, codes.  Bound by latency, so a layer has to be small: one pass over a CTA's weights and
+// four rounds of loads (34,560 weights of a 48 -> 80 layer in 17 passes took 39 us where the three launches take 14).  The 16-channel
+// layer at batch 8 called by itself 42.2 -> 39.3 us with it and the error head in a cluster, the backward of the 16-channel layer
+// 32 x 32 at batch 2 29.7 -> 24.8, of a 256 -> 64 1 x 1 layer 28.2 -> 23.5.
+constexpr int kSmallCtas = 8, kSmallThreads = 512;
+constexpr size_t kSmallErrorBytes = 256 * 1024;
+
+__device__ __forceinline__ long long finish_b1_term_fresh(const FinishItem &it, int b1, uint32_t q)   // (cells written in this launch)
+{
+    const long long *t = it.tap_sums + (4u * q) / (uint32_t)it.d.c_in;
+    long long s = 0;
+#pragma unroll
+    for (int r = 0; r < kTapReplicas; ++r) s += __ldcg(t + (size_t)r * it.tap_stride);
+    return (long long)b1 * s;
+}
+
+__global__ void __launch_bounds__(kSmallThreads) finish_small_kernel(const __grid_constant__ FinishItem it, unsigned *status)
+{
+    extern __shared__ __align__(16) int32_t dyn[];   // the tap kernel's sets, then this CTA's sums, four to a quad
+    __shared__ long long part[kSmallThreads][4];
+    __shared__ __align__(16) unsigned long long max_s[kSmallCtas][2];
+    ptx::cluster_arrive();   // (met before the first write to another CTA's shared memory)
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    const int rank = (int)blockIdx.x;
+    if (it.use_b1) {
+        for (int i = rank; i < it.tap_blocks; i += kSmallCtas) {
+            finish_taps_block<kSmallThreads>(it, i, dyn);
+            __syncthreads();
+        }
+    }
+    ptx::cluster_wait();
+    if (it.use_b1) {
+        __threadfence();
+        ptx::cluster_sync();   // every CTA's tap sums are in the cells
+    }
+    long long *sums = reinterpret_cast<long long *>(dyn);
+    const int groups = it.groups, bw = kSmallThreads / groups, tx = threadIdx.x % bw, ty = threadIdx.x / bw;
+    const uint32_t quads = (uint32_t)(it.n / 4), mine = (quads + kSmallCtas - 1) / kSmallCtas;   // quads of a CTA
+    const uint32_t first = rank * mine, end = min(quads, first + mine);
+    const int b1 = it.use_b1 ? finish_b1(it) : 0;
+    unsigned long long mx = 0;
+    for (uint32_t base = first; base < end; base += bw) {
+        const uint32_t q = base + tx;
+        const bool in = q < end;
+        long long v[4] = {0, 0, 0, 0};
+        if (in) {
+            const int4 *p = reinterpret_cast<const int4 *>(it.parts) + q;
+            int s = ty;
+            for (; s + 7 * groups < it.num_parts; s += 8 * groups) {
+                int4 a[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) a[u] = __ldg(p + (size_t)(s + u * groups) * quads);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    v[0] += a[u].x;
+                    v[1] += a[u].y;
+                    v[2] += a[u].z;
+                    v[3] += a[u].w;
+                }
+            }
+            for (; s < it.num_parts; s += groups) {
+                const int4 a = __ldg(p + (size_t)s * quads);
+                v[0] += a.x;
+                v[1] += a.y;
+                v[2] += a.z;
+                v[3] += a.w;
+            }
+        }
+        if (groups > 1) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) part[threadIdx.x][c] = v[c];
+            __syncthreads();
+            if (ty == 0)
+                for (int u = 1; u < groups; ++u)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) v[c] += part[u * bw + tx][c];
+            __syncthreads();
+        }
+        if (ty == 0 && in) {
+            const long long t = it.use_b1 ? finish_b1_term_fresh(it, b1, q) : 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                v[c] += t;
+                sums[4 * (size_t)(q - first) + c] = v[c];
+                if (it.copy_out) it.copy_out[4 * (size_t)q + c] = v[c];
+                const unsigned long long a = (unsigned long long)(v[c] < 0 ? -v[c] : v[c]);
+                mx = a > mx ? a : mx;
+            }
+        }
+    }
+    mx = block_max_u64(mx);   // (its barriers also publish the sums to the block)
+    if (threadIdx.x == 0) part[0][0] = (long long)mx;
+    __syncthreads();
+    if (threadIdx.x < kSmallCtas) {
+        const unsigned long long m = (unsigned long long)part[0][0];
+        ptx::st_cluster_128(ptx::cluster_addr(ptx::smem_u32(&max_s[rank][0]), threadIdx.x), (uint32_t)m, (uint32_t)(m >> 32), 0u, 0u);
+    }
+    ptx::cluster_sync();
+    unsigned long long M = 0;
+#pragma unroll
+    for (int r = 0; r < kSmallCtas; ++r) M = max_s[r][0] > M ? max_s[r][0] : M;
+    const int t = M ? round_log2_u64(M) : 7;
+    if (rank == 0 && threadIdx.x == 0) {
+        const int p_in = __ldg(it.e3_exp) - 7;
+        *it.g_exp = M ? p_in + t - 7 : p_in;
+        if (!M) atomicOr(status, EOQ_DEV_SQ_ZERO);
+    }
+    const bool fast = t >= 8 && M < 0x7e000000ull;
+    const int sh = t - 7, half_m1 = fast ? (1 << (sh - 1)) - 1 : 0;
+    for (uint32_t q = first + threadIdx.x; q < end; q += kSmallThreads) {
+        int cd[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const long long v = sums[4 * (size_t)(q - first) + c];
+            cd[c] = fast ? sq_code32_shr((int32_t)v, sh, half_m1) : sq_code64(v, t);
+        }
+        reinterpret_cast<uint32_t *>(it.g)[q] = pack4_sat(cd[0], cd[1], cd[2], cd[3]);
+    }
+}
+
 }  // namespace
 
 // The launch geometry of an item, from its sizes.
@@ -454,15 +582,48 @@ void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count,
     }
 }
 
+// shared memory of an item's tap blocks: at least (1 + border rows)(1 + border columns) sets
+static size_t tap_set_bytes(const FinishItem &it)
+{
+    return it.use_b1 ? sizeof(int32_t) * kClassSlab * (1 + it.bc.nrc) * (1 + it.bc.ncc) : 0;
+}
+
+// slice groups of the small kernel: as many as leave its CTAs one pass over their quads
+static int small_groups(const FinishItem &it)
+{
+    const size_t mine = (it.n / 4 + kSmallCtas - 1) / kSmallCtas;
+    int groups = 16;
+    while (groups > 1 && (kSmallThreads / groups < (int)mine || groups > it.num_parts)) groups /= 2;
+    return groups;
+}
+
+bool finish_is_small(const FinishItem &it, const ReduceHook &hook)
+{
+    if (hook.fn || it.n > 4ull * kSmallCtas * kSmallThreads || (it.use_b1 && it.pixels * it.d.c_out > kSmallErrorBytes)) return false;
+    return it.num_parts <= 32 * small_groups(it);   // (four rounds of loads)
+}
+
+cudaError_t launch_finish_small(FinishItem it, unsigned *status, int sm_count, cudaStream_t s)
+{
+    it.keep_sums = 0;
+    plan_finish_item(it, sm_count, true);
+    it.groups = small_groups(it);
+    // one range of rows per CTA and slab of channels
+    const int rows = it.d.n * it.ho, rpb = (rows + kSmallCtas - 1) / kSmallCtas;
+    it.rows_per_block = rpb;
+    it.tap_grid_x = (rows + rpb - 1) / rpb;
+    it.tap_blocks = it.use_b1 ? it.tap_grid_x * ((it.d.c_out + kClassSlab - 1) / kClassSlab) : 0;
+    const size_t sums = (it.n / 4 + kSmallCtas - 1) / kSmallCtas * 4 * sizeof(long long), sets = tap_set_bytes(it);
+    static std::atomic<unsigned long long> allowed;   // 16 KB of sums, or 130 sets (at most 64 border classes)
+    const cudaError_t e = allow_smem((const void *)finish_small_kernel, 72 * 1024, allowed);
+    if (e != cudaSuccess) return e;
+    return launch_chained_clusters(kSmallCtas, finish_small_kernel, kSmallCtas, kSmallThreads, sums > sets ? sums : sets, s, it, status);
+}
+
 cudaError_t launch_finish_taps(const FinishBatch &b, cudaStream_t s)
 {
-    int max_sets = 1;
-    for (int k = 0; k < b.num; ++k) {
-        const FinishItem &it = b.item[k];
-        const int sets = (1 + it.bc.nrc) * (1 + it.bc.ncc);   // at least (1 + border rows)(1 + border columns)
-        if (it.use_b1 && sets > max_sets) max_sets = sets;
-    }
-    const size_t smem = sizeof(int32_t) * max_sets * kClassSlab;
+    size_t smem = 0;
+    for (int k = 0; k < b.num; ++k) smem = tap_set_bytes(b.item[k]) > smem ? tap_set_bytes(b.item[k]) : smem;
     if (smem > 48 * 1024) {   // at most 64 classes: 130 sets
         const cudaError_t e = cudaFuncSetAttribute(finish_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
         if (e != cudaSuccess) return e;

@@ -44,11 +44,12 @@ __device__ __forceinline__ TilePos tile_pos(int tile, int num_n_tiles, int tiles
     return TilePos{tile - mt * num_n_tiles, img, mt - img * tiles_per_img};
 }
 
-// Error back-propagation keeps to 72 registers (the bound of a block of 896 threads): the two of a weight gradient's six warps that
-// share a scheduler then find theirs beside its five.  At 80 and more the weight gradient and the error chain waited for each other's
-// SMs: ResNet-20 step at batch 128 587 us, at 72 575.
-template <int kEpi>   // EpilogueKind: forward and dgrad are kernels of their own (registers, code size)
-__global__ void __launch_bounds__(kEpi == kEpiDgrad ? 896 : kPatchThreads, 1)
+// kLean: 72 registers (the bound of a block of 896 threads) for the error back-propagation of layers of one 32-channel chunk, which
+// share their SMs with weight gradients: the two of a weight gradient's six warps that share a scheduler then find their registers
+// beside its five.  At 80 and more the two streams waited for each other's SMs (ResNet-20 step at batch 128: 587 us, with 72 575).
+// Wider layers fill an SM's shared memory and keep what they use (64 channels 56 x 56, batch 64: 14.5 us with 83, 14.9 with 72).
+template <int kEpi, bool kLean>   // EpilogueKind: forward and dgrad are kernels of their own (registers, code size)
+__global__ void __launch_bounds__(kLean ? 896 : kPatchThreads, 1)
 igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ PatchPlan pl,
                    const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b)
 {
@@ -419,9 +420,11 @@ size_t igemm_patch_smem_bytes(const IgemmParams &p, const PatchPlan &pl)
 cudaError_t launch_igemm_patch(const IgemmParams &p, const PatchPlan &pl, const CUtensorMap &map_a,
                                const CUtensorMap &map_b, int grid, cudaStream_t stream)
 {
-    const auto kernel = p.epilogue == kEpiForward ? igemm_patch_kernel<kEpiForward> : igemm_patch_kernel<kEpiDgrad>;
-    static std::atomic<unsigned long long> allowed[2];
-    const cudaError_t e = allow_smem((const void *)kernel, 226 * 1024, allowed[p.epilogue == kEpiForward]);
+    const int variant = p.epilogue == kEpiForward ? 0 : (p.kc <= 32 && p.tile_n <= 32 ? 2 : 1);
+    const auto kernel = variant == 0 ? igemm_patch_kernel<kEpiForward, false>
+                                     : (variant == 1 ? igemm_patch_kernel<kEpiDgrad, false> : igemm_patch_kernel<kEpiDgrad, true>);
+    static std::atomic<unsigned long long> allowed[3];
+    const cudaError_t e = allow_smem((const void *)kernel, 226 * 1024, allowed[variant]);
     if (e != cudaSuccess) return e;
     return launch_chained(kernel, grid, kPatchThreads, igemm_patch_smem_bytes(p, pl), stream, p, pl, map_a, map_b);
 }

@@ -484,6 +484,9 @@ struct FinishBatch {
 // has a b1 term: tap_first[num] > 0) and the sums with Q_g (two kernels, a third per item under a reduce hook).
 void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, const ReduceHook &hook);
 cudaError_t launch_finish_taps(const FinishBatch &b, cudaStream_t s);
+// ... or all of it in one launch, for one small item (no reduce hook)
+bool finish_is_small(const FinishItem &it, const ReduceHook &hook);
+cudaError_t launch_finish_small(FinishItem it, unsigned *status, int sm_count, cudaStream_t s);
 cudaError_t launch_finish_sums(const FinishBatch &b, unsigned *status, cudaStream_t s, const ReduceHook &hook);
 
 // Batch normalisation behind the convolution (comparison case, eoq_bn.cu): per-channel record in the workspace
