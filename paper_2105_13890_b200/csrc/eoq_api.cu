@@ -1551,7 +1551,6 @@ extern "C" int eoq_conv_dgrad_head(eoq_handle_t handle, const eoq_conv_desc_t *d
 // The weight-gradient workspace: [tap sums][256 bytes with the maximum cell][int64 sums][split-K slices].
 struct WgradSpace {
     long long *tap_sums;
-    size_t tap_stride;            // one copy of the tap sums, in elements
     unsigned long long *max_cell;
     size_t zero_bytes;            // tap sums and maximum cell: cleared by the GEMM kernel
     long long *acc;
@@ -1562,8 +1561,7 @@ static WgradSpace wgrad_space(const eoq_conv_desc_t &d, const Geometry &g, void 
 {
     WgradSpace w;
     char *ws = static_cast<char *>(workspace);
-    w.tap_stride = round256((size_t)d.c_out * g.taps * sizeof(long long)) / sizeof(long long);
-    const size_t tap_bytes = kTapReplicas * w.tap_stride * sizeof(long long);
+    const size_t tap_bytes = kTapReplicas * round256((size_t)d.c_out * g.taps * sizeof(long long));   // (also 16-byte aligned cells)
     w.tap_sums = reinterpret_cast<long long *>(ws);
     w.max_cell = reinterpret_cast<unsigned long long *>(ws + tap_bytes);
     w.zero_bytes = tap_bytes + 256;
@@ -1584,7 +1582,6 @@ static FinishItem finish_item(const eoq_conv_desc_t &d, const Geometry &g, const
     it.b1_c = b1_c;
     it.use_b1 = b1_dev != nullptr || b1_c != 0;   // a device-resident b1 may be anything: its term is always formed
     it.tap_sums = w.tap_sums;
-    it.tap_stride = w.tap_stride;
     it.max_cell = w.max_cell;
     it.acc = w.acc;
     it.num_parts = num_parts;

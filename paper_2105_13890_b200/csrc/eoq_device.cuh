@@ -269,25 +269,20 @@ __device__ __forceinline__ long long warp_sum_i64(long long v)
 
 // Block-wide reductions (every thread of the block must call; the result is valid in thread 0).  Thousands of
 // warps hitting one global cell with an atomic serialise at the L2, so each block sends one.
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)   // the upper words decide, then the lower ones
+{
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32));
+    const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0u);
+    return (unsigned long long)hi << 32 | lo;
+}
 __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v)
 {
     __shared__ unsigned long long red_max[32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, v, o);
-        v = other > v ? other : v;
-    }
+    v = warp_max_u64(v);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
     if (lane == 0) red_max[warp] = v;
     __syncthreads();
-    if (warp == 0) {
-        v = lane < nw ? red_max[lane] : 0ull;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, v, o);
-            v = other > v ? other : v;
-        }
-    }
+    if (warp == 0) v = warp_max_u64(lane < nw ? red_max[lane] : 0ull);
     __syncthreads();
     return v;
 }

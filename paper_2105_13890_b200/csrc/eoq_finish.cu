@@ -203,8 +203,8 @@ __device__ __forceinline__ void finish_taps_block(const FinishItem &it, int loca
         }
     }
     __syncthreads();
-    // the blocks spread their atomics over kTapReplicas copies
-    long long *tap_sums = it.tap_sums + (size_t)(bx % kTapReplicas) * it.tap_stride;
+    // the blocks spread their atomics over the kTapReplicas copies of a cell
+    long long *tap_sums = it.tap_sums + bx % kTapReplicas;
     const int taps = d.kh * d.kw;
     for (int i = threadIdx.x; i < taps * slab_ch; i += kT) {   // consecutive threads: neighbouring cells of [oc][tap]
         const int c = i / taps, tap = i - c * taps, kh = tap / d.kw, kw = tap - kh * d.kw;
@@ -218,7 +218,7 @@ __device__ __forceinline__ void finish_taps_block(const FinishItem &it, int loca
         int sum = over_columns(cell);
         for (unsigned long long m = rm; m; m &= m - 1) sum -= over_columns(cell + __ffsll((long long)m) * (1 + nc) * kClassSlab);
         if (sum)
-            atomicAdd(reinterpret_cast<unsigned long long *>(tap_sums + (size_t)(by * kClassSlab + c) * taps + tap),
+            atomicAdd(reinterpret_cast<unsigned long long *>(tap_sums + ((size_t)(by * kClassSlab + c) * taps + tap) * kTapReplicas),
                       (unsigned long long)(long long)sum);
     }
 }
@@ -232,115 +232,110 @@ __global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_cons
 }
 
 // ------------------------------------------------------------------ exact sums and their maximum
-// A thread owns four neighbouring weights (c_in is a multiple of 4: they share their (oc, tap)).  With more than
-// kDirectParts slices a block is (256 / groups) such quads x `groups` slice groups that meet in shared memory, and the sums
-// are written once, as int32 when they provably fit; with fewer slices nothing is written: the coding pass forms them again,
-// which costs fewer bytes than a round trip.  The 2.4 M weights of the 512-channel 3 x 3
-// layer: sums 18.9 -> 10.9 us, codes 7.8 -> 4.3 us against one weight per thread, four 64-bit tap sums read for each of
-// them and 64-bit sums written and read back.
-constexpr int kDirectParts = 2;
+// A thread owns four neighbouring weights (c_in is a multiple of 4: they share their (oc, tap)); a block is (256 / groups) such
+// quads x `groups` slice groups that meet in shared memory.  The sums are written once, as int32 where they provably fit.
+// Bound by the latency of a round of loads, so a launch is one wave (kSumBlocks blocks of 48 registers to an SM) whose threads
+// keep up to four slices in flight, the last and incomplete round too.  With a serial remainder, more blocks than an SM holds and
+// 64-bit sums throughout: the layer of 512 channels with three slices 11.1 us, 256 channels with eleven 11.4, 128 with 43 8.6;
+// now 6.6, 7.0 and 6.1.  The coding pass reads the written sums: forming them again from one or two slices costs it 6.4 us
+// instead of 4.5 at 512 channels and saves this pass 0.1.
+constexpr int kSumBlocks = 5;
 
-// b1 term of the quad at weight index 4 q
+// b1 term of the quad at weight index 4 q; the copies of a cell are neighbours (one 32-byte sector)
 __device__ __forceinline__ long long finish_b1_term(const FinishItem &it, int b1, uint32_t q)
 {
-    const long long *t = it.tap_sums + (4u * q) / (uint32_t)it.d.c_in;
-    long long s = 0;
-#pragma unroll
-    for (int r = 0; r < kTapReplicas; ++r) s += __ldg(t + (size_t)r * it.tap_stride);
-    return (long long)b1 * s;
+    static_assert(kTapReplicas == 4, "two 16-byte loads hold a cell's copies");
+    const longlong2 *t = reinterpret_cast<const longlong2 *>(it.tap_sums) + (size_t)((4u * q) / (uint32_t)it.d.c_in) * 2;
+    const longlong2 lo = __ldg(t), hi = __ldg(t + 1);
+    return (long long)b1 * (lo.x + lo.y + hi.x + hi.y);
 }
 
-// the quad's sums without the b1 term, from at most kDirectParts slices
-__device__ __forceinline__ void finish_direct(const FinishItem &it, uint32_t q, long long (&v)[4])
+// Adds slices s, s + groups, ... of quad q, four of them (or what is left) in flight together.  Sum: long long, or int where the
+// layer's sums provably fit 32 bits (the slices' sums and the b1 term then fit by themselves).
+template <typename Sum>
+__device__ __forceinline__ void finish_add_slices(const FinishItem &it, uint32_t q, uint32_t quads, int s, int groups, Sum (&v)[4])
 {
-    int4 a[kDirectParts];
+    const int4 *p = reinterpret_cast<const int4 *>(it.parts) + q;
+    for (; s < it.num_parts; s += 4 * groups) {
+        int4 a[4];
 #pragma unroll
-    for (int s = 0; s < kDirectParts; ++s)
-        a[s] = s < it.num_parts ? __ldg(reinterpret_cast<const int4 *>(it.parts + (size_t)s * it.n) + q) : make_int4(0, 0, 0, 0);
-    v[0] = (long long)a[0].x + a[1].x;
-    v[1] = (long long)a[0].y + a[1].y;
-    v[2] = (long long)a[0].z + a[1].z;
-    v[3] = (long long)a[0].w + a[1].w;
+        for (int u = 0; u < 4; ++u)
+            a[u] = s + u * groups < it.num_parts ? __ldg(p + (size_t)(s + u * groups) * quads) : make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[0] += a[u].x;
+            v[1] += a[u].y;
+            v[2] += a[u].z;
+            v[3] += a[u].w;
+        }
+    }
 }
 
-__global__ void __launch_bounds__(kThreads) finish_sums_kernel(const __grid_constant__ FinishBatch b)
+// Sums of the block's quads, written where the coding pass will read them; returns the thread's maximum.
+template <typename Sum>
+__device__ __forceinline__ unsigned long long finish_sums_block(const FinishItem &it, int block, int b1, Sum (*part)[4])
 {
-    ptx::grid_dep_wait();
-    __shared__ long long part[kThreads][4];
-    const int k = finish_item_of(b.fin_first, b.num, (int)blockIdx.x);
-    const FinishItem &it = b.item[k];
+    constexpr bool kNarrow = sizeof(Sum) == 4;
     const int groups = it.groups, bw = kThreads / groups, tx = threadIdx.x % bw, ty = threadIdx.x / bw;
     const uint32_t quads = (uint32_t)(it.n / 4);
-    const int b1 = it.use_b1 ? finish_b1(it) : 0;
-    const bool narrow = finish_narrow(it, b1);
     unsigned long long mx = 0;
-    for (uint32_t base = (uint32_t)((int)blockIdx.x - b.fin_first[k]) * bw; base < quads; base += (uint32_t)it.fin_blocks * bw) {
+    for (uint32_t base = (uint32_t)block * bw; base < quads; base += (uint32_t)it.fin_blocks * bw) {
         const uint32_t q = base + tx;
         const bool in = q < quads;
-        long long v[4] = {0, 0, 0, 0};
-        if (it.direct) {
-            if (in) finish_direct(it, q, v);
-        } else {
-            if (in) {
-                // four slices per round: their loads are independent and in flight together
-                const int4 *p = reinterpret_cast<const int4 *>(it.parts) + q;
-                int s = ty;
-                for (; s + 3 * groups < it.num_parts; s += 4 * groups) {
-                    int4 a[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) a[u] = __ldg(p + (size_t)(s + u * groups) * quads);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        v[0] += a[u].x;
-                        v[1] += a[u].y;
-                        v[2] += a[u].z;
-                        v[3] += a[u].w;
-                    }
-                }
-                for (; s < it.num_parts; s += groups) {
-                    const int4 a = __ldg(p + (size_t)s * quads);
-                    v[0] += a.x;
-                    v[1] += a.y;
-                    v[2] += a.z;
-                    v[3] += a.w;
-                }
-            }
-            if (groups > 1) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) part[threadIdx.x][c] = v[c];
-                __syncthreads();
-                if (ty == 0)
-                    for (int u = 1; u < groups; ++u)
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) v[c] += part[u * bw + tx][c];
-                __syncthreads();
-            }
-        }
-        if (ty == 0 && in) {
-            if (it.use_b1) {
-                const long long t = finish_b1_term(it, b1, q);
+        Sum v[4] = {0, 0, 0, 0};
+        if (in) {
+            finish_add_slices(it, q, quads, ty, groups, v);
+            if (ty == 0 && it.use_b1) {
+                const Sum t = (Sum)finish_b1_term(it, b1, q);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) v[c] += t;
             }
-            if (!it.direct || it.keep_sums) {
-                if (narrow && !it.keep_sums) {
-                    reinterpret_cast<int4 *>(it.acc)[q] = make_int4((int)v[0], (int)v[1], (int)v[2], (int)v[3]);
-                } else {
-                    longlong2 *o = reinterpret_cast<longlong2 *>(it.acc) + 2 * (size_t)q;
-                    o[0] = make_longlong2(v[0], v[1]);
-                    o[1] = make_longlong2(v[2], v[3]);
-                }
+        }
+        if (groups > 1) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) part[threadIdx.x][c] = v[c];
+            __syncthreads();
+            if (ty == 0)
+                for (int u = 1; u < groups; ++u)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) v[c] += part[u * bw + tx][c];
+            __syncthreads();
+        }
+        if (ty == 0 && in) {
+            if (kNarrow) {
+                reinterpret_cast<int4 *>(it.acc)[q] = make_int4((int)v[0], (int)v[1], (int)v[2], (int)v[3]);
+            } else {
+                longlong2 *o = reinterpret_cast<longlong2 *>(it.acc) + 2 * (size_t)q;
+                o[0] = make_longlong2(v[0], v[1]);
+                o[1] = make_longlong2(v[2], v[3]);
             }
             if (it.copy_out)
 #pragma unroll
                 for (int c = 0; c < 4; ++c) it.copy_out[4 * (size_t)q + c] = v[c];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const unsigned long long a = (unsigned long long)(v[c] < 0 ? -v[c] : v[c]);
-                mx = a > mx ? a : mx;
+                if (kNarrow) {
+                    mx = max((uint32_t)mx, (uint32_t)abs((int)v[c]));
+                } else {
+                    const unsigned long long a = (unsigned long long)(v[c] < 0 ? -v[c] : v[c]);
+                    mx = a > mx ? a : mx;
+                }
             }
         }
     }
+    return mx;
+}
+
+__global__ void __launch_bounds__(kThreads, kSumBlocks) finish_sums_kernel(const __grid_constant__ FinishBatch b)
+{
+    ptx::grid_dep_wait();
+    __shared__ __align__(16) long long part[kThreads][4];
+    const int k = finish_item_of(b.fin_first, b.num, (int)blockIdx.x);
+    const FinishItem &it = b.item[k];
+    const int b1 = it.use_b1 ? finish_b1(it) : 0, block = (int)blockIdx.x - b.fin_first[k];
+    unsigned long long mx;
+    if (finish_narrow(it, b1) && !it.keep_sums) mx = finish_sums_block<int>(it, block, b1, reinterpret_cast<int (*)[4]>(part));
+    else mx = finish_sums_block<long long>(it, block, b1, part);
     mx = block_max_u64(mx);
     if (threadIdx.x == 0 && mx && !it.keep_sums) atomicMax(it.max_cell, mx);
 }
@@ -368,8 +363,7 @@ __global__ void __launch_bounds__(kThreads) finish_code_kernel(const __grid_cons
     const FinishItem &it = b.item[k];
     const int bx = (int)blockIdx.x - b.sq_first[k];
     const unsigned long long M = *it.max_cell;
-    const int b1 = it.use_b1 ? finish_b1(it) : 0;
-    const bool narrow = finish_narrow(it, b1);
+    const bool narrow = finish_narrow(it, it.use_b1 ? finish_b1(it) : 0) && !it.keep_sums;   // how the sums were written
     const int t = M ? round_log2_u64(M) : 7;
     if (bx == 0 && threadIdx.x == 0) {
         const int p_in = __ldg(it.e3_exp) - 7;
@@ -380,29 +374,21 @@ __global__ void __launch_bounds__(kThreads) finish_code_kernel(const __grid_cons
     const bool fast = t >= 8 && M < 0x7e000000ull;
     const int sh = t - 7, half_m1 = fast ? (1 << (sh - 1)) - 1 : 0;
     const uint32_t quads = (uint32_t)(it.n / 4);
-    const bool from_sums = !it.direct || it.keep_sums, narrow_sums = narrow && !it.keep_sums;
     for (uint32_t q = (uint32_t)bx * kThreads + threadIdx.x; q < quads; q += (uint32_t)it.sq_blocks * kThreads) {
         long long v[4];
-        if (from_sums && narrow_sums) {
+        if (narrow) {
             const int4 a = __ldg(reinterpret_cast<const int4 *>(it.acc) + q);
             v[0] = a.x;
             v[1] = a.y;
             v[2] = a.z;
             v[3] = a.w;
-        } else if (from_sums) {
+        } else {
             const longlong2 lo = __ldg(reinterpret_cast<const longlong2 *>(it.acc) + 2 * (size_t)q);
             const longlong2 hi = __ldg(reinterpret_cast<const longlong2 *>(it.acc) + 2 * (size_t)q + 1);
             v[0] = lo.x;
             v[1] = lo.y;
             v[2] = hi.x;
             v[3] = hi.y;
-        } else {
-            finish_direct(it, q, v);
-            if (it.use_b1) {
-                const long long bt = finish_b1_term(it, b1, q);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) v[c] += bt;
-            }
         }
         int cd[4];
         if (fast) {
@@ -427,11 +413,9 @@ constexpr size_t kSmallErrorBytes = 256 * 1024;
 
 __device__ __forceinline__ long long finish_b1_term_fresh(const FinishItem &it, int b1, uint32_t q)   // (cells written in this launch)
 {
-    const long long *t = it.tap_sums + (4u * q) / (uint32_t)it.d.c_in;
-    long long s = 0;
-#pragma unroll
-    for (int r = 0; r < kTapReplicas; ++r) s += __ldcg(t + (size_t)r * it.tap_stride);
-    return (long long)b1 * s;
+    const longlong2 *t = reinterpret_cast<const longlong2 *>(it.tap_sums) + (size_t)((4u * q) / (uint32_t)it.d.c_in) * 2;
+    const longlong2 lo = __ldcg(t), hi = __ldcg(t + 1);
+    return (long long)b1 * (lo.x + lo.y + hi.x + hi.y);
 }
 
 __global__ void __launch_bounds__(kSmallThreads) finish_small_kernel(const __grid_constant__ FinishItem it, unsigned *status)
@@ -557,12 +541,11 @@ static void plan_finish_item(FinishItem &it, int sm_count, bool alone)
     it.rows_per_block = rpb;
     it.tap_grid_x = (rows + rpb - 1) / rpb;
     it.tap_blocks = it.use_b1 ? it.tap_grid_x * slabs : 0;
-    it.direct = it.num_parts <= kDirectParts;
-    it.groups = it.direct ? 1 : (it.num_parts >= 32 ? 8 : (it.num_parts >= 8 ? 4 : 1));
+    it.groups = it.num_parts >= 64 ? 16 : (it.num_parts >= 32 ? 8 : (it.num_parts >= 8 ? 4 : 1));
     const size_t quads = (size_t)it.n / 4, bw = kThreads / it.groups;
     size_t fb = (quads + bw - 1) / bw;
-    const size_t cap = (size_t)sm_count * (alone ? 8 : 4);
-    it.fin_blocks = (int)(fb < 1 ? 1 : (fb > cap ? cap : fb));
+    const size_t fin_cap = (size_t)sm_count * (alone ? kSumBlocks : 4), cap = (size_t)sm_count * (alone ? 8 : 4);
+    it.fin_blocks = (int)(fb < 1 ? 1 : (fb > fin_cap ? fin_cap : fb));
     size_t qb = (quads + kThreads - 1) / kThreads;
     it.sq_blocks = (int)(qb < 1 ? 1 : (qb > cap ? cap : qb));
 }

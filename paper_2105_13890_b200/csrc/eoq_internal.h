@@ -457,7 +457,7 @@ struct FinishItem {
     const int32_t *b1_dev;         // b1 in device memory, or null: b1_c
     int32_t b1_c;
     int use_b1;                    // 0: no b1 term (then the tap sums are neither formed nor read)
-    long long *tap_sums;           // kTapReplicas copies, tap_stride elements apart; cleared by the GEMM kernel
+    long long *tap_sums;           // [oc][tap][kTapReplicas copies]; cleared by the GEMM kernel
     unsigned long long *max_cell;  // max |sum| of the layer (behind the tap sums); cleared by the GEMM kernel
     long long *acc;                // where the slices' sums [oc][tap][ic] go: 64-bit, or int32 when they provably fit
     const int32_t *parts;          // int32 split-K slices of the GEMM
@@ -465,14 +465,12 @@ struct FinishItem {
     int8_t *g;
     int32_t *g_exp;
     unsigned long long n;          // weights
-    unsigned long long tap_stride;
     unsigned long long pixels;
     eoq_conv_desc_t d;
     BorderClasses bc;
     int ho, wo, num_parts;
     // filled by plan_finish
     int rows_per_block, tap_grid_x, tap_blocks, groups, fin_blocks, sq_blocks;
-    int direct;                    // the sums are formed twice instead of being written and read back
     int keep_sums;                 // reduce hook: the sums are completed by an all-reduce before their maximum is taken
 };
 struct FinishBatch {

@@ -97,3 +97,33 @@ def test_profile_groups_of_a_weight_gradient(b1):
     assert eoq.eoq_launch_count(h) - before == 6 + kinds["wgrad_taps"]
     assert np.array_equal(G.host(g), g_o) and pg.item() == pg_o and eoq.eoq_last_status(h) == 0
     eoq.eoq_destroy(h)
+
+
+# from one slice of the GEMM to about one per SM: an incomplete round of loads, several rounds, groups of slices
+SLICES = [
+    oracle.ConvDesc(1, 7, 7, 128, 128, 3, 3, 1, 1),
+    oracle.ConvDesc(2, 9, 9, 256, 256, 1, 1, 1, 0),
+    oracle.ConvDesc(9, 7, 7, 256, 256, 3, 3, 1, 1),
+    oracle.ConvDesc(16, 14, 14, 256, 256, 3, 3, 1, 1),
+    oracle.ConvDesc(16, 28, 28, 128, 128, 3, 3, 1, 1),
+    oracle.ConvDesc(64, 32, 32, 16, 16, 3, 3, 1, 1),
+    oracle.ConvDesc(6, 56, 56, 64, 64, 3, 3, 1, 1),
+]
+
+
+@pytest.mark.parametrize("d", SLICES, ids=lambda d: "n%d_%dx%d_%d_%d" % (d.n, d.h, d.w, d.c_in, d.c_out))
+@pytest.mark.parametrize("b1", [0, 3, -30000])
+def test_sums_of_slices(d, b1):
+    """32-bit sums, and 64-bit ones where pixels * 127 * (127 + |b1|) does not fit."""
+    x0, e3 = synth.int8_uniform((d.n, d.h, d.w, d.c_in), 2960, d.c_in), synth.normal_codes((d.n, d.ho, d.wo, d.c_out), 2961, d.c_out, std_codes=30)
+    acc = oracle.conv_wgrad_acc(d, e3, x0, b1)
+    want, p, _ = oracle.sq_int(acc, -16)
+    gd = G.gdesc(d)
+    ws = G.workspace(gd, eoq.EOQ_PASS_WGRAD)
+    ws.fill_(0x5a)
+    for dump in (None, G.zeros(acc.shape, torch.int64)):
+        g, ex = G.empty(acc.shape, torch.int8), G.zeros(1, torch.int32)
+        eoq.eoq_conv_wgrad(G.handle(), gd, G.dev(e3), torch.tensor([-9], dtype=torch.int32, device="cuda:0"), G.dev(x0), b1, g, ex, dump, ws)
+        assert G.status_clear() == 0
+        assert np.array_equal(G.host(g), want) and ex.item() == p
+    assert np.array_equal(G.host(dump), acc)
