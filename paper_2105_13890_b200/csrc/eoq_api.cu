@@ -1597,19 +1597,19 @@ static FinishItem finish_item(const eoq_conv_desc_t &d, const Geometry &g, const
     return it;
 }
 
-// b1 error sums, sums and Q_g of up to kFinishChunk layers whose GEMMs are in front on the stream.
-static int finish_items(Handle *h, const FinishItem *items, int num, cudaStream_t s)
+// b1 error sums, sums and Q_g of up to kFinishChunk layers whose GEMMs are in front on the stream (beside: directly, and one layer).
+static int finish_items(Handle *h, const FinishItem *items, int num, bool beside, cudaStream_t s)
 {
     if (num == 1 && !h->profiling && finish_is_small(items[0], h->hook)) {   // (a profile brackets the b1 sums as a kind of their own)
         count_launches(h, 1);
-        return record(h, launch_finish_small(items[0], &h->dev->status, h->sm_count, s));
+        return record(h, launch_finish_small(items[0], &h->dev->status, h->sm_count, beside, s));
     }
     FinishBatch b;
     plan_finish(b, items, num, h->sm_count, h->hook);
     if (b.tap_first[num] > 0) {
         ProfScope prof(h, EOQ_PROF_WGRAD_TAPS, s);
         count_launches(h, 1);
-        const cudaError_t e = launch_finish_taps(b, s);
+        const cudaError_t e = launch_finish_taps(b, beside, s);
         if (e != cudaSuccess) return record(h, e);
     }
     ProfScope prof(h, EOQ_PROF_WGRAD_AUX, s);
@@ -1644,7 +1644,7 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     auto finish = [&](int num_parts) -> int {
         FinishItem it = finish_item(d, g, w, e3, e3_exp, b1_c, b1_dev, gq, g_exp, num_parts);
         it.copy_out = reinterpret_cast<long long *>(acc_dump);
-        return finish_items(h, &it, 1, s);
+        return finish_items(h, &it, 1, true, s);
     };
 
     WgradPatchPlan wp;
@@ -1652,6 +1652,7 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
         wp.partials = w.parts;
         wp.zero = reinterpret_cast<int4 *>(w.tap_sums);
         wp.zero_n16 = (unsigned)(w.zero_bytes / 16);
+        wp.launch_early = use_b1 && !gemm_only;
         wp.dev = h->dev;
         CUtensorMap map_x, map_e;
         if (!make_patch_map(&map_x, x, d.n, d.h, d.w, d.c_in, wp.kc, wp.pw, wp.r_rows + d.kh - 1) ||
@@ -1696,6 +1697,7 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     p.partials = w.parts;
     p.zero = reinterpret_cast<int4 *>(w.tap_sums);
     p.zero_n16 = (unsigned)(w.zero_bytes / 16);
+    p.launch_early = use_b1 && !gemm_only;
     p.dev = h->dev;
 
     cudaError_t e;
@@ -1768,7 +1770,7 @@ extern "C" int eoq_wgrad_finish(eoq_handle_t handle, int num, const eoq_conv_des
             items[k] = finish_item(d, g, wgrad_space(d, g, workspace[base + k]), e3[base + k], e3_exp[base + k], 0, b1_c[base + k],
                                    gq[base + k], g_exp[base + k], num_parts[base + k]);
         }
-        const int st = finish_items(h, items, count, s);
+        const int st = finish_items(h, items, count, false, s);
         if (st != EOQ_OK) return st;
     }
     return EOQ_OK;

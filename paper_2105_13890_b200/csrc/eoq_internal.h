@@ -270,6 +270,7 @@ struct WgradParams {
     int32_t *partials;   // [num_k_splits][c_out][taps][c_in] partial sums, a slice per split
     int4 *zero;          // the cells of the kernels that follow (tap sums, maximum): cleared here, zero_n16 groups of 16 bytes
     unsigned zero_n16;
+    int launch_early;    // the next kernel on the stream starts beside this one (see launch_finish_taps)
     DeviceState *dev;
 };
 
@@ -301,6 +302,7 @@ struct WgradPatchPlan {
     int32_t *partials;   // [num_splits][c_out][taps][c_in]
     int4 *zero;          // as in WgradParams
     unsigned zero_n16;
+    int launch_early;
     DeviceState *dev;
 };
 constexpr int kWgradPatchThreads = 192;  // warp 0 loads, warp 1 MMA + TMEM, warps 2..5 epilogue
@@ -480,11 +482,13 @@ struct FinishBatch {
 };
 // Lays out the launches of up to kFinishChunk items; then, in this order on one stream, the b1 error sums (only where an item
 // has a b1 term: tap_first[num] > 0) and the sums with Q_g (two kernels, a third per item under a reduce hook).
+// beside: the launch in front on the stream is the item's GEMM, which lets its successor start once e3 is complete
+// (launch_early); the error sums are then formed beside it, and wait for its end only before they go into the cells.
 void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, const ReduceHook &hook);
-cudaError_t launch_finish_taps(const FinishBatch &b, cudaStream_t s);
+cudaError_t launch_finish_taps(const FinishBatch &b, bool beside, cudaStream_t s);
 // ... or all of it in one launch, for one small item (no reduce hook)
 bool finish_is_small(const FinishItem &it, const ReduceHook &hook);
-cudaError_t launch_finish_small(FinishItem it, unsigned *status, int sm_count, cudaStream_t s);
+cudaError_t launch_finish_small(FinishItem it, unsigned *status, int sm_count, bool beside, cudaStream_t s);
 cudaError_t launch_finish_sums(const FinishBatch &b, unsigned *status, cudaStream_t s, const ReduceHook &hook);
 
 // Batch normalisation behind the convolution (comparison case, eoq_bn.cu): per-channel record in the workspace

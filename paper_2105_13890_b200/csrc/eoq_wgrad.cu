@@ -103,6 +103,7 @@ wgrad_kernel(const __grid_constant__ WgradParams p, const __grid_constant__ CUte
     __syncthreads();
     ptx::tc_fence_after();
     ptx::grid_dep_wait();   // everything up to here touched no global memory
+    if (p.launch_early) ptx::grid_dep_launch();
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < p.zero_n16; i += gridDim.x * blockDim.x) p.zero[i] = make_int4(0, 0, 0, 0);
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, p.dev};

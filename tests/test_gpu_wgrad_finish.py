@@ -127,3 +127,29 @@ def test_sums_of_slices(d, b1):
         assert G.status_clear() == 0
         assert np.array_equal(G.host(g), want) and ex.item() == p
     assert np.array_equal(G.host(dump), acc)
+
+
+@pytest.mark.parametrize("d", [oracle.ConvDesc(4, 16, 16, 16, 16, 3, 3, 1, 1), oracle.ConvDesc(8, 28, 28, 64, 128, 3, 3, 1, 1),
+                               oracle.ConvDesc(5, 17, 15, 32, 48, 3, 3, 2, 1)], ids=lambda d: "n%d_%d_%d_s%d" % (d.n, d.c_in, d.c_out, d.stride))
+def test_error_sums_beside_the_gemm(d):
+    """The error sums start beside the GEMM: errors that the kernel in front of it wrote, over and over into one buffer and one
+    workspace, have to be the ones they see."""
+    hd, rounds = G.handle(), 12
+    shape = (d.n, d.ho, d.wo, d.c_out)
+    n = int(np.prod(shape))
+    x0 = synth.int8_uniform((d.n, d.h, d.w, d.c_in), 2970, d.c_in)
+    e0s = [synth.normal_codes(shape, 2971, i, std_codes=10 + 6 * i) for i in range(rounds)]
+    gd = G.gdesc(d)
+    ws = G.workspace(gd, eoq.EOQ_PASS_WGRAD)
+    e3, pe, gamma, p_in = G.empty(shape, torch.int8), G.zeros(1, torch.int32), torch.tensor([128], dtype=torch.int32, device="cuda:0"), G.zeros(1, torch.int32)
+    b1, x, mask = torch.tensor([-37], dtype=torch.int32, device="cuda:0"), G.dev(x0), G.dev(G.pack_mask(np.ones(n, np.uint8)))
+    ins = [G.dev(e) for e in e0s]
+    outs = [(G.empty((d.c_out, d.kh, d.kw, d.c_in), torch.int8), G.zeros(1, torch.int32)) for _ in e0s]
+    for e0, (g, pg) in zip(ins, outs):
+        eoq.eoq_err_prescale_dev(hd, e0, p_in, mask, None, n, gamma, e3, pe, G.zeros(1, torch.int64), None)
+        eoq.eoq_conv_wgrad_dev(hd, gd, e3, pe, x, b1, g, pg, ws)
+    assert G.status_clear() == 0
+    for e0, (g, pg) in zip(e0s, outs):
+        e3_o, p3, _ = oracle.sq_int(e0.astype(np.int64) * 128, -7)
+        want, p, _ = oracle.sq_int(oracle.conv_wgrad_acc(d, e3_o, x0, -37), p3 - 7)
+        assert np.array_equal(G.host(g), want) and pg.item() == p
