@@ -334,6 +334,84 @@ head_dpooled_kernel(const float *__restrict__ dl, const float *__restrict__ W, i
     if (k < c && b < n) dpooled[(size_t)b * c + k] = acc;
 }
 
+// The same with the block's columns of W whole in shared memory (up to kDpMost classes; W in 16-byte pieces): they are fetched
+// beside the softmax kernel.  That one starts its successor only after its own wait, behind which the logits kernel and all in
+// front of it are complete, so W is; past the L1 it is read as they left it.  What remains behind the wait is the latency of
+// dl and the chain itself, without a barrier in it.  Head without its update, 512 channels and 1000 classes, against the kernel
+// above: 15.1 us for 19.0 at batch 1, 27.2 for 35.4 at 64, 44.9 for 51.9 at 128 (two waves of blocks, of which an SM holds one);
+// in more waves the other one, three blocks to an SM, covers its loads better (81.5 for 77.6 at 256, 61.7 for 60.2 with 1536
+// channels at 64).
+constexpr int kDpMost = 1344;
+static size_t dp_resident_bytes(int classes) { return ((size_t)(classes + 8) * kDpCh + (size_t)kDpN * (((classes + 3) & ~3) + 12)) * sizeof(float); }
+__global__ void __launch_bounds__(kDpCh *kDpN)
+head_dpooled_resident_kernel(const float *__restrict__ dl, const float *__restrict__ W, int n, int c, int classes, float *dpooled,
+                             const double *loss_n, float *loss_out)
+{
+    extern __shared__ float4 head_smem[];
+    float *ws = reinterpret_cast<float *>(head_smem), *ds = ws + (size_t)(classes + 8) * kDpCh;
+    const int cl = threadIdx.x % kDpCh, nl = threadIdx.x / kDpCh;
+    const int k0 = blockIdx.x * kDpCh, b = blockIdx.y * kDpN + nl;
+    const bool chains = blockIdx.y < gridDim.y - 1;
+    if (chains)
+        for (int i = threadIdx.x; i < classes * (kDpCh / 4); i += kDpCh * kDpN) {
+            const int j = i / (kDpCh / 4), q = (i % (kDpCh / 4)) * 4;
+            const bool in = k0 + q < c;   // (c is a multiple of 4)
+            cp_async_16(ws + j * kDpCh + q, in ? W + (size_t)j * c + k0 + q : W, in);
+        }
+    ptx::grid_dep_wait_launch_small();
+    if (!chains) {   // an extra row of blocks: the mean loss, in sample order, beside the chains
+        if (blockIdx.x == 0 && threadIdx.x == 0 && loss_out) {
+            double s = 0.0;
+#pragma unroll 8
+            for (int i = 0; i < n; ++i) s += __ldg(loss_n + i);
+            *loss_out = (float)(s / n);
+        }
+        return;
+    }
+    float *d = ds + (size_t)nl * (((classes + 3) & ~3) + 12);
+    if (b < n) {   // a warp fetches its own sample's row
+        const float *src = dl + (size_t)b * classes;
+        if (classes % 4 == 0 && (reinterpret_cast<uintptr_t>(dl) & 15) == 0)
+            for (int j = cl * 4; j < classes; j += kDpCh * 4) cp_async_16(d + j, src + j, true);
+        else
+            for (int j = cl; j < classes; j += kDpCh) cp_async_4(d + j, src + j, true);
+    }
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    if (b >= n) return;
+    const float *w = ws + cl;
+    float acc = 0.0f;
+    int j = 0;
+    // eight links while the operands of the next eight come out of shared memory (the last round reads up to eight rows and
+    // values past the end: the buffers have them to spare)
+    float4 da = *reinterpret_cast<const float4 *>(d), db = *reinterpret_cast<const float4 *>(d + 4);
+    float wa[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) wa[q] = w[q * kDpCh];
+#pragma unroll 4
+    for (; j + 8 <= classes; j += 8) {
+        const float4 d0 = da, d1 = db;
+        float w0[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) w0[q] = wa[q];
+        da = *reinterpret_cast<const float4 *>(d + j + 8);
+        db = *reinterpret_cast<const float4 *>(d + j + 12);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) wa[q] = w[(j + 8 + q) * kDpCh];
+        acc = __fmaf_rn(d0.x, w0[0], acc);
+        acc = __fmaf_rn(d0.y, w0[1], acc);
+        acc = __fmaf_rn(d0.z, w0[2], acc);
+        acc = __fmaf_rn(d0.w, w0[3], acc);
+        acc = __fmaf_rn(d1.x, w0[4], acc);
+        acc = __fmaf_rn(d1.y, w0[5], acc);
+        acc = __fmaf_rn(d1.z, w0[6], acc);
+        acc = __fmaf_rn(d1.w, w0[7], acc);
+    }
+    for (; j < classes; ++j) acc = __fmaf_rn(d[j], w[j * kDpCh], acc);
+    if (k0 + cl < c) dpooled[(size_t)b * c + k0 + cl] = acc;
+}
+
 // W[j][k] <- fma(-lr, sum_b fma(dl[b][j], pooled[b][k], .), W[j][k]), b ascending; bias[j] alike (thread k == 0).
 // kV = 4: a thread owns four adjacent channels, so that a link of its four chains costs one and a quarter loads
 // instead of eight (64 samples, 1000 x 512 weights: 18 -> 14.5 us beside the backward pass).
@@ -507,7 +585,12 @@ cudaError_t launch_head(const int32_t *sums, int n, int c, int hw, int classes, 
     const bool fold = head_folds_pooling(n);
     cudaError_t e = cudaFuncSetAttribute(fold ? head_logits_kernel<true> : head_logits_kernel<false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(((32 + kHeadWarps) * (kHeadK + 4) + 16) * sizeof(float)));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(head_dpooled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dp_smem);
+    const dim3 dp_grid((c + kDpCh - 1) / kDpCh, (n + kDpN - 1) / kDpN + 1);
+    const bool resident = c % 4 == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0 && classes <= kDpMost &&
+                          dp_grid.x * dp_grid.y <= 2u * kPartSms;
+    if (e == cudaSuccess)
+        e = resident ? cudaFuncSetAttribute(head_dpooled_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dp_resident_bytes(kDpMost))
+                     : cudaFuncSetAttribute(head_dpooled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dp_smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((classes + kHeadWarps - 1) / kHeadWarps, (n + 31) / 32);
     if (fold) {
@@ -519,8 +602,9 @@ cudaError_t launch_head(const int32_t *sums, int n, int c, int hw, int classes, 
     const size_t soft_smem = ((size_t)classes * sizeof(float) + 15) & ~(size_t)15;
     if (soft_smem <= 48 * 1024 - 256) launch_chained(head_softmax_kernel<true>, n, kThreads, soft_smem, st, logits, n, classes, labels, dl, loss_n);
     else launch_chained(head_softmax_kernel<false>, n, kThreads, 0, st, logits, n, classes, labels, dl, loss_n);
-    launch_chained(head_dpooled_kernel, dim3((c + kDpCh - 1) / kDpCh, (n + kDpN - 1) / kDpN + 1), kDpCh * kDpN, dp_smem, st, dl, W, n, c, classes, dpooled,
-                                                                                                   loss_n, loss_out);
+    if (resident)
+        launch_chained(head_dpooled_resident_kernel, dp_grid, kDpCh * kDpN, dp_resident_bytes(classes), st, dl, W, n, c, classes, dpooled, loss_n, loss_out);
+    else launch_chained(head_dpooled_kernel, dp_grid, kDpCh * kDpN, dp_smem, st, dl, W, n, c, classes, dpooled, loss_n, loss_out);
     if (lr != 0.0f) return launch_head_update(dl, pooled, n, c, classes, lr, W, bias, st);
     return cudaGetLastError();
 }

@@ -291,3 +291,26 @@ def test_dgrad_join_and_head_in_one_call(n, h, w, c_in, c_out, k, stride, pad, p
     eoq.eoq_aux_join(hd, e4b, p4b, G.dev(b), i32(pb), G.dev(G.pack_mask(gate01)) if gated else None, b.size, out2, pout2, None)
     torch.cuda.synchronize()
     assert np.array_equal(G.host(out2), out_o) and pout2.item() == pout_o
+
+
+@pytest.mark.parametrize("n,c,classes", [(1, 16, 1), (1, 16, 7), (9, 48, 8), (7, 80, 1001), (8, 512, 1000), (3, 96, 1344), (3, 96, 1345), (128, 512, 40),
+                                         (144, 512, 9)])
+def test_head_gradient_sizes(n, c, classes):
+    """Both kernels of the gradient of the pooled activations (up to 1344 classes in up to 296 blocks of 32 channels x 8 samples,
+    or beyond), with a weight matrix that the step of the call before has just changed."""
+    hd, hw = G.handle(), 49
+    sums = (synth.relu_codes((n, c), 8600 + classes, 0).astype(np.int64) * hw) // 3
+    W = (synth.normal_f32((classes, c), 8600 + classes, 1) / np.float32(np.sqrt(c))).astype(np.float32)
+    bias = np.zeros(classes, np.float32)
+    labels = synth.labels(n, classes, 8600 + classes, 3).astype(np.int32)
+    W_d, bias_d, s_d, l_d = G.dev(W), G.dev(bias), G.dev(sums.astype(np.int32)), G.dev(labels)
+    ws = G.zeros(eoq.eoq_aux_head_workspace_size(n, c, classes), torch.uint8)
+    outs = [(G.zeros(1, torch.float32), G.zeros((n, c), torch.float32), G.zeros((n, classes), torch.float32)) for _ in range(3)]
+    for loss, dpooled, logits in outs:
+        eoq.eoq_aux_head(hd, s_d, n, c, hw, classes, W_d, bias_d, l_d, 0.25, loss, dpooled, logits, ws)
+    torch.cuda.synchronize()
+    for loss, dpooled, logits in outs:
+        loss_o, dpooled_o, logits_o = oracle.head(sums, hw, W, bias, labels, 0.25)
+        assert np.array_equal(G.host(logits), logits_o) and np.array_equal(G.host(dpooled), dpooled_o)
+        assert loss.item() == pytest.approx(loss_o, rel=1e-6, abs=1e-6)
+    assert np.array_equal(G.host(W_d), W) and np.array_equal(G.host(bias_d), bias)
