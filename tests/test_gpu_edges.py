@@ -335,3 +335,31 @@ def test_weight_gradient_slices_stay_exact_in_few_ctas(d, m):
     eoq.eoq_conv_wgrad(h, gd, e3_d, pe, xm, 0, g, pg, acc, ws)
     assert eoq.eoq_last_status(h) == 0 and np.array_equal(G.host(acc), want)
     eoq.eoq_destroy(h)
+
+
+@pytest.mark.parametrize("loads,extra", [(8, 0), (8, 3), (8, 4), (9, 5), (15, -1), (22, 0), (22, 3), (22, 4)])
+@pytest.mark.parametrize("kind", ["normal", "zero", "inf", "captured"])
+def test_quantize_float_held_on_the_device(loads, extra, kind):
+    """SQ around the sizes whose share of a thread (1024 per SM, four floats to a load) no longer fits its registers (8 loads) or its
+    registers and shared memory (22): one launch between them, two outside."""
+    n = loads * 4096 * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    x = torch.zeros(n) if kind == "zero" else torch.from_numpy(synth.normal_f32(n, 2980 + loads, extra + 1))
+    if kind == "inf":
+        x[n - 1] = float("inf")
+    hd, x_d, out, ex = G.handle(), x.cuda(), G.empty((n,), torch.int8), G.zeros(1, torch.int32)
+    run = lambda: eoq.eoq_quantize(hd, eoq.EOQ_SQ, x_d, True, None, n, out, ex)
+    if kind == "captured":
+        stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            eoq.eoq_quantize(hd, eoq.EOQ_SQ, x_d, True, None, n, out, ex, stream=torch.cuda.current_stream().cuda_stream)
+        run = graph.replay
+    for _ in range(2):   # (the first call has to leave the handle's cells clean)
+        out.fill_(77)
+        run()
+        torch.cuda.synchronize()
+        assert G.status_clear() == {"zero": eoq.EOQ_DEV_SQ_ZERO, "inf": eoq.EOQ_DEV_NONFINITE}.get(kind, 0)
+        if kind == "inf":   # flagged; the codes are those at an exponent of -7
+            c, p = np.clip(np.rint(x.numpy() * np.float32(128)), -127, 127).astype(np.int8), -7
+        else:
+            c, p, _ = oracle.quantize_f32(oracle.MODE_SQ, x.numpy())
+        assert np.array_equal(G.host(out), c) and ex.item() == p
