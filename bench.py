@@ -230,7 +230,7 @@ def bandwidth_bytes(wl, chained=False):
         elif l.name.endswith(".a"):
             dq += n_out * (1 + 0.125)                                       # e3 out and mask bits, on the Q_e pass of unit B
         if l.has_dgrad:
-            dq += l.n * l.h * l.w * l.c_in * (4 + 1)                        # exact int32 sums in, e4 codes out
+            dq += l.n * l.h * l.w * l.c_in * (2 + 1)                        # sums in as 16-bit words, e4 codes out
         fin += l.weight_elems * (4 + 1)                                     # exact sums in, g codes out
         upd += l.weight_elems * 3                                           # g in, w in, w out
     f = wl.layers[0]
