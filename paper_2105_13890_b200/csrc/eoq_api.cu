@@ -1891,14 +1891,10 @@ extern "C" int eoq_quantize(eoq_handle_t handle, int mode, const void *src, int 
     if (mode == EOQ_SQ && !dst_exp) return EOQ_ERR_BAD_ARG;
     if (!aligned16(src) || !aligned16(dst)) return EOQ_ERR_ALIGNMENT;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    count_launches(h, mode == EOQ_SQ && !(src_is_float && quantize_is_small(mode, n, h->hook)) ? 2 : 1);
     ProfScope prof(h, EOQ_PROF_OTHER, s);
-    if (src_is_float) {
-        int kernels = 0;
-        const cudaError_t e = launch_quantize_f32(mode, reinterpret_cast<const float *>(src), n, dst, dst_exp, h->dev, h->sm_count, s, h->hook, &kernels);
-        count_launches(h, kernels);
-        return record(h, e);
-    }
-    count_launches(h, mode == EOQ_SQ ? 2 : 1);
+    if (src_is_float)
+        return record(h, launch_quantize_f32(mode, reinterpret_cast<const float *>(src), n, dst, dst_exp, h->dev, h->sm_count, s, h->hook));
     if (mode != EOQ_SQ || !src_exp) return EOQ_ERR_UNSUPPORTED;
     return record(h, launch_sq_i32(reinterpret_cast<const int32_t *>(src), src_exp, 0, n, reinterpret_cast<int8_t *>(dst),
                                    dst_exp, nullptr, false, h->dev, h->sm_count, s, h->hook));

@@ -181,91 +181,6 @@ quantize_sq_small_kernel(const float *__restrict__ src, size_t n, int8_t *dst, i
     cluster.sync();  // no block leaves while another may still read its maximum
 }
 
-// SQ in one launch for tensors that the device can hold: every thread keeps its share, the first kHeldRegs loads in registers and
-// the others in shared memory, where asynchronous copies bring them with everything in flight at once; between reduction and codes
-// all blocks meet at a grid-wide barrier (see prescale_fused_kernel), so the tensor is read once.  The launch is cooperative, one
-// block to an SM; its wait is bounded, and a kernel that gives up flags it and writes nothing.
-// The cooperative launch and its barrier cost 6.2 us where two chained launches cost 4.9, so tensors that fit the registers alone
-// keep the two passes (4.0 M floats 8.2 us here, 7.6 there); 6.0 M floats 11.2 -> 10.3, 12.8 M floats 20.0 -> 18.5.
-constexpr int kHeldThreads = 1024, kHeldRegs = 8, kHeldSmem = 14;
-__global__ void __launch_bounds__(kHeldThreads, 1)
-quantize_sq_held_kernel(const float *__restrict__ src, size_t n, int8_t *dst, int32_t *dst_exp, DeviceState *dev, int smem_loads,
-                        uint32_t spin_limit)
-{
-    extern __shared__ float4 held[];
-    __shared__ uint32_t max_s;
-    __shared__ unsigned go_s;
-    const float4 *s4 = reinterpret_cast<const float4 *>(src);
-    const size_t n4 = n / 4, base = (size_t)blockIdx.x * kHeldThreads + threadIdx.x, step = (size_t)gridDim.x * kHeldThreads;
-    for (int u = 0; u < smem_loads; ++u) {   // (a thread reads only what it copied itself)
-        const size_t i = base + (kHeldRegs + u) * step;
-        const bool in = i < n4;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(held + u * kHeldThreads + threadIdx.x)), "l"(in ? s4 + i : s4),
-                     "r"(in ? 16 : 0) : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    float4 v[kHeldRegs];
-#pragma unroll
-    for (int u = 0; u < kHeldRegs; ++u) {
-        const size_t i = base + u * step;
-        v[u] = i < n4 ? __ldg(s4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const size_t ti = n4 * 4 + threadIdx.x;
-    const bool has_tail = blockIdx.x == 0 && ti < n;
-    const float tail = has_tail ? src[ti] : 0.0f;
-    uint32_t mx = __float_as_uint(tail) & 0x7fffffffu;
-    auto add = [&](const float4 &x) {
-        mx = max(max(mx, max(__float_as_uint(x.x) & 0x7fffffffu, __float_as_uint(x.y) & 0x7fffffffu)),
-                 max(__float_as_uint(x.z) & 0x7fffffffu, __float_as_uint(x.w) & 0x7fffffffu));
-    };
-#pragma unroll
-    for (int u = 0; u < kHeldRegs; ++u) add(v[u]);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    for (int u = 0; u < smem_loads; ++u) add(held[u * kHeldThreads + threadIdx.x]);
-    mx = block_max_u32(mx);
-    if (threadIdx.x == 0) {
-        if (mx) atomicMax(&dev->absmax_u32, mx);
-        __threadfence();
-        atomicAdd(&dev->arrivals, 1u);
-        unsigned ok = 0;
-        for (uint32_t it = 0; it < spin_limit; ++it) {
-            if (*reinterpret_cast<volatile unsigned *>(&dev->arrivals) >= gridDim.x) { ok = 1; break; }
-            __nanosleep(40);
-        }
-        if (!ok) atomicOr(&dev->status, EOQ_DEV_TIMEOUT);
-        __threadfence();
-        go_s = ok;
-        max_s = *reinterpret_cast<volatile uint32_t *>(&dev->absmax_u32);
-    }
-    __syncthreads();
-    if (!go_s) return;
-    const uint32_t M = max_s;
-    bool last = false;
-    if (threadIdx.x == 0) last = last_reader(dev);   // the last block to have read the cells clears them at its end
-    const int up = sq_up(M);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *dst_exp = -up;
-        if (M == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-        if (M >= 0x7f800000u) atomicOr(&dev->status, EOQ_DEV_NONFINITE);
-    }
-    const Pow2Scale sc = pow2_scale(up);
-#pragma unroll
-    for (int u = 0; u < kHeldRegs; ++u) {
-        const size_t i = base + u * step;
-        if (i < n4) quantize_store4<2>(dst, i, sc, v[u]);
-    }
-#pragma unroll 2
-    for (int u = 0; u < smem_loads; ++u) {
-        const size_t i = base + (kHeldRegs + u) * step;
-        if (i < n4) quantize_store4<2>(dst, i, sc, held[u * kHeldThreads + threadIdx.x]);
-    }
-    if (has_tail) dst[ti] = (int8_t)quantize_code<2>(sc, tail);
-    if (last) {
-        dev->absmax_u32 = 0;
-        dev->arrivals = 0;
-    }
-}
-
 // SQ of an fp32 image under the already reduced maximum: c_src channels in, c_dst (zero-padded) channels out,
 // rows widened by `wmargin` zero pixels at both ends.  A thread writes kG = 16 or 8 channels of a pixel.
 // Bound by memory (12 B in, 8 or 16 B out per RGB pixel).  A block is tx pixels x ty rows and a thread takes its pixel in
@@ -1123,17 +1038,12 @@ cudaError_t launch_reset_cells(DeviceState *dev, cudaStream_t s)
                            offsetof(DeviceState, tensor_absmax) - offsetof(DeviceState, absmax_u32), s);
 }
 
-static bool cooperative_launch_allowed()
-{
-    int dev_id = 0, can = 0;
-    return cudaGetDevice(&dev_id) == cudaSuccess && cudaDeviceGetAttribute(&can, cudaDevAttrCooperativeLaunch, dev_id) == cudaSuccess && can;
-}
+bool quantize_is_small(int mode, size_t n, const ReduceHook &hook) { return mode == 2 && !hook.fn && n <= kSmallElems * kSmallCluster; }
 
 cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev,
-                                int sm_count, cudaStream_t s, const ReduceHook &hook, int *kernels)
+                                int sm_count, cudaStream_t s, const ReduceHook &hook)
 {
-    if (mode == 2 && !hook.fn && n <= kSmallElems * kSmallCluster) {
-        *kernels = 1;
+    if (quantize_is_small(mode, n, hook)) {
         int blocks = 1;
         while ((size_t)blocks * kSmallElems < n) blocks *= 2;
         cudaLaunchConfig_t cfg{};
@@ -1147,23 +1057,6 @@ cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst,
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, quantize_sq_small_kernel, src, n, static_cast<int8_t *>(dst), dst_exp, dev);
     }
-    const size_t n4 = n / 4, per_load = (size_t)sm_count * kHeldThreads, loads = (n4 + per_load - 1) / per_load;
-    if (mode == 2 && !hook.fn && loads > kHeldRegs && loads <= kHeldRegs + kHeldSmem && cooperative_launch_allowed()) {
-        int smem_loads = (int)loads - kHeldRegs;
-        const size_t smem = (size_t)smem_loads * kHeldThreads * sizeof(float4);
-        static std::atomic<unsigned long long> allowed;
-        cudaError_t e = allow_smem((const void *)quantize_sq_held_kernel, kHeldSmem * kHeldThreads * (int)sizeof(float4), allowed);
-        if (e != cudaSuccess) return e;
-        uint32_t spin_limit = kSpinLimit;
-        void *args[] = {(void *)&src, (void *)&n, (void *)&dst, (void *)&dst_exp, (void *)&dev, (void *)&smem_loads, (void *)&spin_limit};
-        e = cudaLaunchCooperativeKernel((const void *)quantize_sq_held_kernel, dim3(sm_count), dim3(kHeldThreads), args, smem, s);
-        if (e != cudaErrorCooperativeLaunchTooLarge) {
-            *kernels = 1;
-            return e;
-        }
-        (void)cudaGetLastError();  // fewer SMs at hand than at start-up (e.g. a partitioned device): two kernels instead
-    }
-    *kernels = mode == 2 ? 2 : 1;
     if (mode == 2) {
         launch_chained(absmax_f32_kernel, grid_for(n / 4 + 1, sm_count), kThreads, 0, s, src, n, dev);
         hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);  // float bit patterns of |x| order like integers

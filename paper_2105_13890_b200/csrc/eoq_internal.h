@@ -344,9 +344,9 @@ cudaError_t launch_quantize_image(const float *src, int n, int h, int w, int c_s
                                   int32_t *dst_exp, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook);
 // w[oc][kh][kw][16] -> wp[oc][kh][8][16], zero in the taps kw..7 (weights of the filter-row path)
 cudaError_t launch_weight_pad_rows(const int8_t *w, int8_t *wp, int c_out, int kh, int kw, int c_in, cudaStream_t s);
-// *kernels: how many were launched
+bool quantize_is_small(int mode, size_t n, const ReduceHook &hook);  // one launch instead of two
 cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev,
-                                int sm_count, cudaStream_t s, const ReduceHook &hook, int *kernels);
+                                int sm_count, cudaStream_t s, const ReduceHook &hook);
 cudaError_t launch_sq_i32(const int32_t *src, const int32_t *src_exp, int exp_bias, size_t n, int8_t *dst,
                           int32_t *dst_exp, long long *sum_codes, bool max_already_reduced, DeviceState *dev,
                           int sm_count, cudaStream_t s, const ReduceHook &hook);

@@ -339,9 +339,9 @@ def test_weight_gradient_slices_stay_exact_in_few_ctas(d, m):
 
 @pytest.mark.parametrize("loads,extra", [(8, 0), (8, 3), (8, 4), (9, 5), (15, -1), (22, 0), (22, 3), (22, 4)])
 @pytest.mark.parametrize("kind", ["normal", "zero", "inf", "captured"])
-def test_quantize_float_held_on_the_device(loads, extra, kind):
-    """SQ around the sizes whose share of a thread (1024 per SM, four floats to a load) no longer fits its registers (8 loads) or its
-    registers and shared memory (22): one launch between them, two outside."""
+def test_quantize_float_of_whole_device_shares(loads, extra, kind):
+    """SQ of as many floats as all threads of the device (1024 per SM, four floats to a load) take in whole rounds, and a few more or
+    less: remainders modulo 4 behind 4.8 to 13.3 M floats."""
     n = loads * 4096 * torch.cuda.get_device_properties(0).multi_processor_count + extra
     x = torch.zeros(n) if kind == "zero" else torch.from_numpy(synth.normal_f32(n, 2980 + loads, extra + 1))
     if kind == "inf":
@@ -363,3 +363,41 @@ def test_quantize_float_held_on_the_device(loads, extra, kind):
         else:
             c, p, _ = oracle.quantize_f32(oracle.MODE_SQ, x.numpy())
         assert np.array_equal(G.host(out), c) and ex.item() == p
+
+
+@pytest.mark.parametrize("n", [262144, 6000001, 64 * 56 * 56 * 64 + 1])
+def test_quantize_float_runs_beside_a_long_kernel(n):
+    """SQ needs no SM for itself alone: it ends while a kernel of another stream still occupies one (a convolution capped to one CTA,
+    whose shared memory fills its SM for several milliseconds)."""
+    d = eoq.conv_desc(128, 56, 56, 64, 64, 3, 3, 1, 1)
+    hold, h = eoq.eoq_create(0), eoq.eoq_create(0)
+    eoq.eoq_set_gemm_ctas(hold, 1)
+    x, w = G.zeros((128, 56, 56, 64), torch.int8), G.zeros((64, 3, 3, 64), torch.int8)
+    x5, scal, prep = G.empty(x.shape, torch.int8), torch.tensor([0, 128, 0], dtype=torch.int32, device="cuda:0"), G.zeros(eoq.eoq_weight_prep_size(d), torch.uint8)
+    eoq.eoq_weight_prep(hold, [d], [w], [prep])
+    src = synth.normal_f32(n, 3010, 0)
+    c, p, _ = oracle.quantize_f32(oracle.MODE_SQ, src)
+    src_d, out, ex = G.dev(src), G.zeros(n, torch.int8), G.zeros(1, torch.int32)
+    s_hold, s = torch.cuda.Stream(), torch.cuda.Stream()
+
+    def convolution():
+        eoq.eoq_conv_fwd_dev(hold, d, x, None, scal, w, prep, None, True, x5, None, None, stream=s_hold.cuda_stream)
+
+    def quantizer():
+        eoq.eoq_quantize(h, eoq.EOQ_SQ, src_d, True, None, n, out, ex, stream=s.cuda_stream)
+
+    convolution()   # (first launches load their kernels)
+    quantizer()
+    torch.cuda.synchronize()
+    out.zero_()
+    torch.cuda.synchronize()
+    convolution()
+    held = torch.cuda.Event()
+    held.record(s_hold)
+    quantizer()
+    s.synchronize()
+    assert not held.query()
+    assert np.array_equal(G.host(out), c) and ex.item() == p
+    assert eoq.eoq_last_status(h) == 0 and eoq.eoq_last_status(hold) == 0
+    eoq.eoq_destroy(h)
+    eoq.eoq_destroy(hold)
