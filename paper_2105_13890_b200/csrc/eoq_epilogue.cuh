@@ -352,7 +352,8 @@ __device__ __forceinline__ void forward_group(const IgemmParams &p, const FwdSca
 // Error back-propagation: keep the exact sums (the scale quantizer needs the maximum over the whole tensor before any element can
 // be coded) and track max |.|.  They are kept as 16-bit words that lose nothing Q_e can see (sums_pack_16), one 32-byte sector per
 // lane and 16 columns: this launch is bound by its stores.  A caller who asks for the int32 sums gets those instead
-// (p.sums16 == null).
+// (p.sums16 == null), two 32-byte sectors at a time where the buffer allows it: with four 16-byte stores of half a sector each, 64
+// channels 56 x 56 take 163 us instead of 103 at batch 512 (79 as words), 22.0 instead of 16.7 at batch 64.
 __device__ __forceinline__ uint32_t dgrad_16(const IgemmParams &p, const uint32_t *acc, size_t off, uint32_t &mx_masked)
 {
     uint32_t mx = 0;
@@ -376,6 +377,9 @@ __device__ __forceinline__ uint32_t dgrad_16(const IgemmParams &p, const uint32_
         uint32_t w[8];
         sums_pack_16(acc, mx, w);
         st_global_256(p.sums16 + off, w);   // (a workspace: aligned to 256 bytes)
+    } else if ((reinterpret_cast<uintptr_t>(p.acc_out) & 31) == 0) {   // (off is a multiple of 16: one answer for a launch)
+        st_global_256(p.acc_out + off, acc);
+        st_global_256(p.acc_out + off + 8, acc + 8);
     } else {
         int4 *d = reinterpret_cast<int4 *>(p.acc_out + off);
 #pragma unroll

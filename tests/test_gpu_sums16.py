@@ -85,3 +85,24 @@ def test_halves_and_neighbours_of_halves_in_shortened_groups():
     eoq.eoq_conv_dgrad(G.handle(), desc, G.dev(e3), torch.tensor([-9], dtype=torch.int32, device="cuda:0"), G.dev(w), e4, e4_exp, None, None,
                        G.workspace(desc, eoq.EOQ_PASS_DGRAD))
     assert np.array_equal(G.host(e4), want) and e4_exp.item() == p
+
+
+@pytest.mark.parametrize("first", [0, 4, 8])
+@pytest.mark.parametrize("name", ["patch", "taps, strided", "1x1", "cluster"])
+def test_dumped_sums_at_every_alignment(name, first):
+    """The int32 sums for a caller, 32 bytes to a store where their buffer starts at a multiple of 32 bytes and 16 where it does not
+    (`first` elements behind an allocation): all of them, and nothing beside them."""
+    d = GEOMETRIES[name]
+    e3 = _errors("large", (d.n, d.ho, d.wo, d.c_out), 40 + first)
+    w = synth.int8_uniform((d.c_out, d.kh, d.kw, d.c_in), 2602, first)
+    acc = oracle.conv_dgrad_acc(d, e3, w)
+    want, p, _ = oracle.sq_int(acc, -9 - 7)
+    buf = torch.full((first + acc.size + 8,), 77, dtype=torch.int32, device="cuda:0")
+    dump = buf[first:first + acc.size]
+    assert dump.data_ptr() % 32 == 4 * first % 32
+    e4, e4_exp, desc = G.empty(acc.shape, torch.int8), G.zeros(1, torch.int32), G.gdesc(d)
+    eoq.eoq_conv_dgrad(G.handle(), desc, G.dev(e3), torch.tensor([-9], dtype=torch.int32, device="cuda:0"), G.dev(w), e4, e4_exp, None, dump,
+                       G.workspace(desc, eoq.EOQ_PASS_DGRAD))
+    assert G.status_clear() == 0
+    assert np.array_equal(G.host(dump).reshape(acc.shape), acc) and (G.host(buf[:first]) == 77).all() and (G.host(buf[first + acc.size:]) == 77).all()
+    assert np.array_equal(G.host(e4), want) and e4_exp.item() == p
