@@ -1848,11 +1848,13 @@ extern "C" int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *des
         return EOQ_OK;
     }
     if (pass == EOQ_PASS_DGRAD) {
+        p.epilogue = kEpiDgrad;
         p.b_mn = 1;
         if (d.stride == 1 && d.kh == d.kw && d.kh - 1 - d.pad >= 0 &&
             plan_stride1(p, pl, d.n, d.c_out, d.h, d.w, d.kh, d.kh - 1 - d.pad, d.c_in, h->sm_count, h->gemm_ctas)) {
-            snprintf(buf, buf_bytes, "kernel=igemm_patch tile_n=%d accumulators=%d m_tiles=%d n_tiles=%d weights=%s", p.tile_n,
-                     p.tile_n <= 128 ? 2 : 1, p.num_m_tiles, p.num_n_tiles, pl.b_resident ? "resident" : "streamed");
+            snprintf(buf, buf_bytes, "kernel=igemm_patch tile_n=%d accumulators=%d m_tiles=%d n_tiles=%d weights=%s%s", p.tile_n,
+                     p.tile_n <= 128 ? 2 : 1, p.num_m_tiles, p.num_n_tiles, pl.b_resident ? "resident" : "streamed",
+                     igemm_patch_lean(p, pl) ? " registers=72" : "");
             return EOQ_OK;
         }
         const int hq = (d.h + d.stride - 1) / d.stride, wq = (d.w + d.stride - 1) / d.stride;

@@ -44,10 +44,13 @@ __device__ __forceinline__ TilePos tile_pos(int tile, int num_n_tiles, int tiles
     return TilePos{tile - mt * num_n_tiles, img, mt - img * tiles_per_img};
 }
 
-// kLean: 72 registers (the bound of a block of 896 threads) for the error back-propagation of layers of one 32-channel chunk, which
-// share their SMs with weight gradients: the two of a weight gradient's six warps that share a scheduler then find their registers
-// beside its five.  At 80 and more the two streams waited for each other's SMs (ResNet-20 step at batch 128: 587 us, with 72 575).
-// Wider layers fill an SM's shared memory and keep what they use (64 channels 56 x 56, batch 64: 14.5 us with 83, 14.9 with 72).
+// kLean: 72 registers (the bound of a block of 896 threads; 16 bytes of it are spilled) for error back-propagations whose reduction
+// is one chunk of at most 32 channels and whose column tile is at most 32 wide (igemm_patch_lean).  They leave an SM's shared memory
+// half free for a weight gradient of the same layer, and the two of a weight gradient's six warps that share a scheduler find their
+// registers beside its five; at 80 and more the two streams wait for each other's SMs.  ResNet-20 step at batch 128: stochastic
+// 591 -> 583 us, nearest 580 -> 580, at batch 64 and below no difference beyond the noise; alone the two variants take the same time
+// (16 channels 32 x 32, batch 128: 9.5 us).  Layers of several chunks and wider column tiles fill an SM's shared memory and keep the
+// 96 that they use (64 channels 56 x 56, batch 64: 14.7 us, 14.9 with 72).
 template <int kEpi, bool kLean>   // EpilogueKind: forward and dgrad are kernels of their own (registers, code size)
 __global__ void __launch_bounds__(kLean ? 896 : kPatchThreads, 1)
 igemm_patch_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ PatchPlan pl,
@@ -417,10 +420,12 @@ size_t igemm_patch_smem_bytes(const IgemmParams &p, const PatchPlan &pl)
     return (size_t)pl.num_a * pl.a_bytes + b + 1024 + kTableSmemBytes;
 }
 
+bool igemm_patch_lean(const IgemmParams &p, const PatchPlan &pl) { return p.epilogue == kEpiDgrad && pl.chunks == 1 && p.kc <= 32 && p.tile_n <= 32; }
+
 cudaError_t launch_igemm_patch(const IgemmParams &p, const PatchPlan &pl, const CUtensorMap &map_a,
                                const CUtensorMap &map_b, int grid, cudaStream_t stream)
 {
-    const int variant = p.epilogue == kEpiForward ? 0 : (p.kc <= 32 && p.tile_n <= 32 ? 2 : 1);
+    const int variant = p.epilogue == kEpiForward ? 0 : (igemm_patch_lean(p, pl) ? 2 : 1);
     const auto kernel = variant == 0 ? igemm_patch_kernel<kEpiForward, false>
                                      : (variant == 1 ? igemm_patch_kernel<kEpiDgrad, false> : igemm_patch_kernel<kEpiDgrad, true>);
     static std::atomic<unsigned long long> allowed[3];

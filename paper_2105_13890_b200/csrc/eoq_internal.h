@@ -221,6 +221,7 @@ struct PatchPlan {
 constexpr int kPatchThreads = 128 + 32 * kEpilogueWarps;  // warps: 0 patch loads, 1 MMA + TMEM, 2 weight loads, then the epilogue
 
 size_t igemm_patch_smem_bytes(const IgemmParams &p, const PatchPlan &pl);
+bool igemm_patch_lean(const IgemmParams &p, const PatchPlan &pl);   // error back-propagation by the kernel of 72 registers
 cudaError_t launch_igemm_patch(const IgemmParams &p, const PatchPlan &pl, const CUtensorMap &map_a,
                                const CUtensorMap &map_b, int grid, cudaStream_t stream);
 

@@ -62,3 +62,24 @@ def test_unit_gamma_without_shortcut(relu, b2):
         eoq.eoq_conv_fwd(G.handle(), gd, G.dev(x0), None, -2, G.dev(w), 128, b2, None, relu, x5, x2, mask, None, G.workspace(gd, eoq.EOQ_PASS_FWD))
         assert G.status_clear() == 0
         assert np.array_equal(G.host(x5), ref["x5"]) and np.array_equal(G.unpack_mask(mask, out), ref["mask"])
+
+
+@pytest.mark.parametrize("c_in,c_out", [(16, 16), (32, 32), (16, 32), (48, 32), (32, 48), (32, 96), (96, 96), (160, 160)])
+@pytest.mark.parametrize("n", [1, 8])
+def test_error_back_propagation_in_72_registers(n, c_in, c_out):
+    """The kernel of fewer registers is for a reduction of one 32-channel chunk into a column tile of at most 32: no layer of several
+    chunks takes it, however narrow its column tiles are."""
+    d = oracle.ConvDesc(n, 16, 16, c_in, c_out, 3, 3, 1, 1)
+    gd = G.gdesc(d)
+    plan = eoq.eoq_describe_plan(G.handle(), gd, eoq.EOQ_PASS_DGRAD)
+    narrow = int(plan.split("tile_n=")[1].split()[0]) <= 32
+    assert ("registers=72" in plan) == ("kernel=igemm_patch" in plan and c_out <= 32 and narrow)
+    assert c_out > 32 or "kernel=igemm_patch" in plan
+    e3, w = synth.normal_codes((n, 16, 16, c_out), 2720, c_in, std_codes=24), synth.normal_codes((c_out, 3, 3, c_in), 2721, c_out, std_codes=6)
+    acc = oracle.conv_dgrad_acc(d, e3, w)
+    want, p, _ = oracle.sq_int(acc, -9 - 7)
+    e4, e4_exp, total = G.zeros(acc.shape, torch.int8), G.zeros(1, torch.int32), G.zeros(1, torch.int64)
+    eoq.eoq_conv_dgrad(G.handle(), gd, G.dev(e3), torch.tensor([-9], dtype=torch.int32, device="cuda:0"), G.dev(w), e4, e4_exp, total, None,
+                       G.workspace(gd, eoq.EOQ_PASS_DGRAD))
+    assert G.status_clear() == 0
+    assert np.array_equal(G.host(e4), want) and e4_exp.item() == p and total.item() == int(want.astype(np.int64).sum())
