@@ -106,3 +106,36 @@ def test_dumped_sums_at_every_alignment(name, first):
     assert G.status_clear() == 0
     assert np.array_equal(G.host(dump).reshape(acc.shape), acc) and (G.host(buf[:first]) == 77).all() and (G.host(buf[first + acc.size:]) == 77).all()
     assert np.array_equal(G.host(e4), want) and e4_exp.item() == p
+
+
+@pytest.mark.parametrize("c_out,cut", [(3000, 12), (20000, 15), (40000, 16), (80000, 17), (100000, 17)])
+def test_sums_cut_by_the_most_bits(c_out, cut):
+    """Reductions so long that groups lose `cut` bits, up to the 17 that a 32-bit sum can (16 and above need every bit of the count that a
+    group carries): halves of a code step, their neighbours, and short groups beside them."""
+    c_out = c_out // 16 * 16
+    e3, w = np.zeros((1, 1, 40, c_out), np.int8), np.zeros((c_out, 1, 1, 32), np.int8)
+    v = np.concatenate([np.array([127, -127, 120, -120, 112, -112, 104, 96, -96, 80, 64, 48, 32, 16, 8, 4]), np.arange(1, 25)])
+    e3[0, 0, :, :c_out - 16] = v[:, None]
+    e3[0, 0, :, c_out - 1] = np.arange(40) % 3 - 1    # (one beside the multiples)
+    ones = 1 << int(np.log2(c_out - 16))
+    w[:, 0, 0, 0] = 127
+    for i in range(1, 8):   # ones << k in all: sums of v << (log2(ones) + k)
+        w[:ones, 0, 0, i] = -(1 << (i - 1)) if i == 3 else 1 << (i - 1)
+    w[:, 0, 0, 8:16] = synth.int8_uniform((c_out, 8), 2610, c_out)
+    w[:100, 0, 0, 16:] = synth.int8_uniform((100, 16), 2611, c_out)   # the other group of a pixel
+    w[c_out - 1] = 1
+    d = oracle.ConvDesc(1, 1, 40, 32, c_out, 1, 1, 1, 0)
+    acc = oracle.conv_dgrad_acc(d, e3, w)
+    largest = np.abs(acc.astype(np.int64)).reshape(-1, 16).max(axis=1)
+    assert largest.max().item().bit_length() - 14 == cut and len(set(x.item().bit_length() for x in largest)) > 5
+    want, p, _ = oracle.sq_int(acc, -9 - 7)
+    step = p - (-9 - 7)   # log2 of a code step
+    rest = np.abs(acc.astype(np.int64)) & ((1 << step) - 1)
+    for beside in (-1, 0, 1):
+        assert (rest == (1 << (step - 1)) + beside).any()
+    desc = G.gdesc(d)
+    e4, e4_exp, total = G.empty(acc.shape, torch.int8), G.zeros(1, torch.int32), G.zeros(1, torch.int64)
+    eoq.eoq_conv_dgrad(G.handle(), desc, G.dev(e3), torch.tensor([-9], dtype=torch.int32, device="cuda:0"), G.dev(w), e4, e4_exp, total, None,
+                       G.workspace(desc, eoq.EOQ_PASS_DGRAD))
+    assert G.status_clear() == 0
+    assert np.array_equal(G.host(e4), want) and e4_exp.item() == p and total.item() == int(want.astype(np.int64).sum())
