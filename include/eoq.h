@@ -189,7 +189,7 @@ EOQ_API int eoq_conv_dgrad_join_head(eoq_handle_t handle, const eoq_conv_desc_t 
  * device, a plugin loaded into a host application that forbids cudaMalloc after start-up, or a real-time loop
  * where an allocation's implicit synchronisation is not acceptable.  Such callers cannot use eoq_create (it
  * allocates the handle's device state) nor supply a workspace.  This entry point needs neither: every byte of
- * scratch -- reduction cells, transposed weights, int32 sums -- sits in one static device array of
+ * scratch -- reduction cells, transposed weights, sums -- sits in one static device array of
  * EOQ_STATIC_SCRATCH_BYTES (+4 KiB of cells) that is part of the library image, so each GPU that loads the
  * library carries it until the process exits.  It calls no cudaMalloc, cudaFree or allocating library routine.
  *

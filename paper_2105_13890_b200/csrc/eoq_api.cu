@@ -972,7 +972,9 @@ extern "C" int eoq_workspace_size(const eoq_conv_desc_t *desc, int pass, size_t 
             *bytes = round256((size_t)bc.nrc * bc.ncc * desc->c_out * sizeof(int32_t)) +
                      (use_row_window(*desc, g.wo) ? round256((size_t)desc->c_out * desc->kh * 8 * desc->c_in) : 0);
             return EOQ_OK;
-        case EOQ_PASS_DGRAD:  // transposed weights + int32 sums
+        // transposed weights + sums.  The room is that of int32 sums; as 16-bit words they fill half of it.  The size is part of
+        // the interface: callers keep buffers of it, and the allocation-free entry point accepts geometries by it.
+        case EOQ_PASS_DGRAD:
             *bytes = round256(g.w_elems) + round256(g.in_elems * sizeof(int32_t));
             return EOQ_OK;
         case EOQ_PASS_WGRAD: {  // per-tap error sums, reduction cell, int64 sums, split-K slices

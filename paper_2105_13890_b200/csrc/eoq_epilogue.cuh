@@ -52,11 +52,13 @@ __device__ __forceinline__ uint32_t rne7_denormal(uint32_t x)
 
 // Forward chain on 16 consecutive output channels of one pixel (Sec. 3.2.1: x2 = Q_a1(conv), x3 = gamma x2,
 // x4 = x3 + b2 [+ shortcut], x5 = Q_a2(relu(x4)); mask = [x4 > 0]).
-// The integer pipe bounds this code (an instruction every two cycles and scheduler), so clamps are moved in front of the
+// The integer pipe (an instruction every two cycles and scheduler) is the busiest of this code, so clamps are moved in front of the
 // roundings (both are monotonic, the clamp limits are chosen so that the rounded result is unchanged), roundings run as one
 // FMA each, and the constant offsets of that trick are folded into the multiply-add that forms x4.  (The chain on floats
 // alone, with conversions and saturating additions, has fewer instructions but a longer dependent sequence: 25.7 us where
-// this takes 20.4 us for the 64-channel 56 x 56 layer at batch 64.)
+// this takes 20.4 us for the 64-channel 56 x 56 layer at batch 64.)  No pipe is full: with shortcut and x2, 64 channels 56 x 56 at
+// batch 512 take 133 us of which the integer pipe is busy 46% (9.4 of 26 instructions per element), the issue slots 63% and memory
+// 3.6 TB/s; the largest stall is the wait for tensor memory and the shortcut.
 //
 // The b1 term (b1 times the sum of the weights whose taps fall inside the image, per border class and output
 // channel) is read from shared memory, already multiplied by b1: the epilogue warps copy the table there once per
@@ -255,7 +257,7 @@ __device__ __forceinline__ void forward_16(const IgemmParams &p, const FwdScalar
 // The chain where gamma = 1 (unit A of a block, the first layer, projections) and x2 is not kept: x4 = x2 + b2 in whole codes, so
 // Q_a2 rounds nothing and x5 = clamp(R(acc / 2^shift) + b2).  Both clamps move in front of the one rounding, where b2 shifts their
 // limits (|b2| <= 2^14: the 16-bit saturation of x2 lies outside them), and mask = [x4 > 0] = [x5 > 0].  About 7 instructions per
-// element, 3.5 of them on the integer pipe that bounds the general form (20 and 8.5): 64 channels 56 x 56,
+// element, 3.5 of them on the integer pipe, the busiest of the general form (20 and 8.5): 64 channels 56 x 56,
 // batch 64: 17.0 -> 15.7 us; 128 channels 28 x 28: 13.6 -> 12.3; 512 -> 256 channels 1 x 1, batch 32: 10.8 -> 9.9.
 template <bool kRelu>
 __device__ __forceinline__ void forward_unit_16(const IgemmParams &p, const FwdScalars &fs, const FwdShift &sh, const uint32_t (&acc)[32],

@@ -239,8 +239,9 @@ __global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_cons
 // ------------------------------------------------------------------ exact sums and their maximum
 // A thread owns four neighbouring weights (c_in is a multiple of 4: they share their (oc, tap)); a block is (256 / groups) such
 // quads x `groups` slice groups that meet in shared memory.  The sums are written once, as int32 where they provably fit.
-// Bound by the latency of a round of loads, so a launch is one wave (kSumBlocks blocks of 48 registers to an SM) whose threads
-// keep up to four slices in flight, the last and incomplete round too.  With a serial remainder, more blocks than an SM holds and
+// Bound by the latency of a round of loads, so the launch for one layer is one wave (kSumBlocks blocks of 48 registers to an SM) whose
+// threads keep up to four slices in flight, the last and incomplete round too.  In a launch for several layers each of them has up to
+// four blocks per SM for itself, several waves in all (plan_finish_item).  With a serial remainder, more blocks than an SM holds and
 // 64-bit sums throughout: the layer of 512 channels with three slices 11.1 us, 256 channels with eleven 11.4, 128 with 43 8.6;
 // now 6.6, 7.0 and 6.1.  The coding pass reads the written sums: forming them again from one or two slices costs it 6.4 us
 // instead of 4.5 at 512 channels and saves this pass 0.1.

@@ -6,7 +6,8 @@
 // apart in an input row, which is just the distance between the rows of a core matrix without swizzle: eight pixels' 16-byte chunks
 // are 128 contiguous bytes, the next chunk of the same pixels starts 16 bytes further.  So a descriptor with a leading offset of 16
 // and a stride offset of 128 bytes reads the windows out of the input row as it lies in memory, overlaps and all, and a patch of
-// (r - 1) * stride + kh input rows, one TMA box, serves r output rows.  An M tile is one output row (of 125 pixels at most).  What
+// (r - 1) * stride + kh input rows, one TMA box, serves r output rows.  An M tile is one output row; rows of
+// more than 125 pixels (8 channels; 121 with 16) are cut into several tiles (plan_rows; at most 128 output channels).  What
 // bounds it now is the MMAs (two per filter row and tile, about 60 cycles each) and the epilogue: 224 x 224 images at batch 64
 // 77.8 -> 35.0 us, 178 x 178 at batch 13 14.5 -> 9.7, one 224 x 224 image 5.6 -> 4.2 (back to back).
 //

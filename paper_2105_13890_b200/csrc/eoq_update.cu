@@ -202,9 +202,10 @@ __device__ __forceinline__ void update_range(UpdateMode mode, const UpdateTensor
     }
 }
 
-// w <- Q_w(w - Q_u(lr * g)).  Bound by instruction issue under stochastic rounding (the 64-bit hash is about 20 of the 30
-// instructions of an element), else by memory (3 B per weight).  Every rounding mode is a loop of its own on 32-bit
-// values: the 21 M weights of ResNet-34 take 37 us under stochastic rounding, 58 us with one 64-bit sequence for all modes.
+// w <- Q_w(w - Q_u(lr * g)).  Bound by the integer pipe under stochastic rounding: 43 instructions a weight, most of them the 64-bit
+// hash's, 24 of which go to the pipe that takes one every two cycles and scheduler: 27.5 of the 37 us that the 21 M weights of
+// ResNet-34 take (the pipe is 79% busy while an SM has work).  Rounding to nearest takes 14 instructions and 15 us; its largest stall
+// is that of its loads.  Every rounding mode is a loop of its own on 32-bit values: one 64-bit sequence for all modes took 58 us.
 __global__ void __launch_bounds__(kThreads)
 update_apply_kernel(const __grid_constant__ UpdateBatch b, int32_t lr_mant, int32_t lr_exp, int stochastic, unsigned long long seed,
                     unsigned long long step, unsigned long long *step_dev, DeviceState *dev)
