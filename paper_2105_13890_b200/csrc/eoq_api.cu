@@ -772,9 +772,10 @@ extern "C" int eoq_create(eoq_handle_t *handle, int device)
             delete h;
             return EOQ_ERR_UNSUPPORTED;  // the kernels are sm_100a only
         }
-        e = cudaMalloc(reinterpret_cast<void **>(&h->dev), sizeof(DeviceState));
+        e = cudaMalloc(reinterpret_cast<void **>(&h->dev), round256(sizeof(DeviceState)) + kSqTiles * sizeof(int16_t));
     }
     if (e == cudaSuccess) e = cudaMemset(h->dev, 0, sizeof(DeviceState));
+    h->tile_shift = reinterpret_cast<int16_t *>(reinterpret_cast<char *>(h->dev) + round256(sizeof(DeviceState)));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming);
     for (int k = 0; k < kClassBranches && e == cudaSuccess; ++k) {
         e = cudaStreamCreateWithFlags(&h->class_branch[k], cudaStreamNonBlocking);
@@ -1898,7 +1899,8 @@ extern "C" int eoq_quantize(eoq_handle_t handle, int mode, const void *src, int 
     count_launches(h, mode == EOQ_SQ && !(src_is_float && quantize_is_small(mode, n, h->hook)) ? 2 : 1);
     ProfScope prof(h, EOQ_PROF_OTHER, s);
     if (src_is_float)
-        return record(h, launch_quantize_f32(mode, reinterpret_cast<const float *>(src), n, dst, dst_exp, h->dev, h->sm_count, s, h->hook));
+        return record(h, launch_quantize_f32(mode, reinterpret_cast<const float *>(src), n, dst, dst_exp, h->tile_shift, h->dev,
+                                             h->sm_count, s, h->hook));
     if (mode != EOQ_SQ || !src_exp) return EOQ_ERR_UNSUPPORTED;
     return record(h, launch_sq_i32(reinterpret_cast<const int32_t *>(src), src_exp, 0, n, reinterpret_cast<int8_t *>(dst),
                                    dst_exp, nullptr, false, h->dev, h->sm_count, s, h->hook));
@@ -2042,7 +2044,7 @@ extern "C" int eoq_quantize_image(eoq_handle_t handle, const float *src, int n, 
     if ((c_dst % 16 && c_dst != 8) || c_dst > 64 || !aligned16(src) || !aligned16(dst)) return EOQ_ERR_ALIGNMENT;
     count_launches(h, 2);
     ProfScope prof(h, EOQ_PROF_INPUT_Q, reinterpret_cast<cudaStream_t>(stream));
-    return record(h, launch_quantize_image(src, n, hh, ww, c_src, c_dst, wmargin, dst, dst_exp, h->dev, h->sm_count,
+    return record(h, launch_quantize_image(src, n, hh, ww, c_src, c_dst, wmargin, dst, dst_exp, h->tile_shift, h->dev, h->sm_count,
                                            reinterpret_cast<cudaStream_t>(stream), h->hook));
 }
 

@@ -26,36 +26,6 @@ inline int grid_for(size_t work_items, int sm_count, int per_sm = 8)
 
 // ------------------------------------------------------------------ fp32 -> Q / CQ / SQ
 
-__global__ void absmax_f32_kernel(const float *__restrict__ src, size_t n, DeviceState *dev)
-{
-    ptx::grid_dep_wait_launch_small();
-    uint32_t mx = 0;
-    bool bad = false;
-    const size_t n4 = n / 4;
-    const float4 *s4 = reinterpret_cast<const float4 *>(src);
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-        float4 v = __ldg(s4 + i);
-        uint32_t b[4] = {__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            uint32_t a = b[k] & 0x7fffffffu;
-            bad |= a >= 0x7f800000u;
-            mx = max(mx, a);
-        }
-    }
-    for (size_t i = n4 * 4 + (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        uint32_t a = __float_as_uint(src[i]) & 0x7fffffffu;
-        bad |= a >= 0x7f800000u;
-        mx = max(mx, a);
-    }
-    mx = (uint32_t)block_max_u64(mx);
-    bad = __syncthreads_or(bad);
-    if (threadIdx.x == 0) {
-        if (mx) atomicMax(&dev->absmax_u32, mx);
-        if (bad) atomicOr(&dev->status, EOQ_DEV_NONFINITE);
-    }
-}
-
 // x * 2^up, exact wherever the code depends on it (a result too small for a normal number codes to 0 either way).
 // 2^up itself may exceed the float range for a tensor of subnormal size, hence two factors.
 struct Pow2Scale {
@@ -87,37 +57,23 @@ __device__ __forceinline__ void quantize_store4(void *dst, size_t i, const Pow2S
     else reinterpret_cast<uint32_t *>(dst)[i] = pack4_sat(a, b, c, d);
 }
 
-// kMode 0: Q -> int16, 1: CQ -> int8, 2: SQ -> int8 under the already reduced maximum.
-// Bound by memory: 4 B in (from L2 where the maximum's pass left it: the tiles are walked backwards), 1 or 2 B out.  A
-// block takes one tile of kQuantTile float4; eight independent, coalesced loads per thread are in flight before the
-// maximum is needed.  12.8 M floats: 18.1 us with 64 strided bytes per thread and a general power-of-two function per
-// element, 7.7 us so.
+// kMode 0: Q -> int16, 1: CQ -> int8.  Bound by memory: 4 B in, 1 or 2 B out.  A block takes one tile of kQuantTile float4, eight
+// independent, coalesced loads per thread.
 constexpr int kQuantLoads = 8, kQuantTile = kThreads * kQuantLoads;
 template <int kMode>
 __global__ void __launch_bounds__(kThreads)
-quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev)
+quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp)
 {
     ptx::grid_dep_wait_launch_small();
-    __shared__ uint32_t max_s;
-    const size_t n4 = n / 4, base = (size_t)(gridDim.x - 1 - blockIdx.x) * kQuantTile + threadIdx.x;
+    const size_t n4 = n / 4, base = (size_t)blockIdx.x * kQuantTile + threadIdx.x;
     float4 v[kQuantLoads];
 #pragma unroll
     for (int u = 0; u < kQuantLoads; ++u) {
         const size_t i = base + (size_t)u * kThreads;
         if (i < n4) v[u] = __ldg(reinterpret_cast<const float4 *>(src) + i);
     }
-    int up = 7;
-    bool last = false;
-    if (kMode == 2) {
-        if (threadIdx.x == 0) max_s = *reinterpret_cast<volatile uint32_t *>(&dev->absmax_u32);
-        __syncthreads();
-        up = sq_up(max_s);
-        if (threadIdx.x == 0) last = last_reader(dev);
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0 && dst_exp) {
-        *dst_exp = -up;
-        if (kMode == 2 && max_s == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-    }
+    constexpr int up = 7;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && dst_exp) *dst_exp = -up;
     const Pow2Scale sc = pow2_scale(up);
 #pragma unroll
     for (int u = 0; u < kQuantLoads; ++u) {
@@ -130,7 +86,140 @@ quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t 
         if (kMode == 0) reinterpret_cast<int16_t *>(dst)[i] = (int16_t)c;
         else reinterpret_cast<int8_t *>(dst)[i] = (int8_t)c;
     }
+}
+
+// ------------------------------------------------------------------ SQ of a tensor beyond one cluster
+// The codes of SQ depend on the tensor's maximum through R(log2 max) alone, and a tile of a few thousand elements mostly has the
+// tensor's R(log2 max) already.  So the first pass reads the tensor once, codes every tile under the larger of its own maximum
+// and what other blocks have reduced by then, and leaves the shift it used; the second pass, under the whole maximum, codes again
+// the tiles whose shift was another one, and returns where there are none.  Bound by memory.  12.8 M normal floats from memory: 13.1
+// us for a maximum's pass and 8.2 for the codes before; now 12.3 + 3.7, of which the second returns at once, and 12.6 + 6.4 where every
+// tile was wrong (one element beyond all others).  4 M floats: 6.3 + 3.9 before, 6.2 + 3.1 now, 6.0 + 6.0 at worst.
+
+// shift of a tile: what its codes were formed under, or one of
+constexpr int kTileAny = 0x7fff;     // all of it is zero: codes 0 under any shift
+constexpr int kTileMixed = 0x7ffe;   // parts under different shifts
+constexpr int kAgainPerSm = 5;       // blocks of the second pass on an SM
+
+// The block's guess for one part of its tile (all threads, `tid` in the block; one barrier): `mx` is the thread's maximum.
+struct TileGuess {
+    uint32_t own = 0;        // largest |x| of the tile so far (bit pattern)
+    int shift = kTileAny;    // of the tile so far
+    int turn = 0;
+    __device__ __forceinline__ int part(uint32_t mx, int tid, DeviceState *dev)
+    {
+        __shared__ __align__(16) uint32_t warp_s[2][kThreads / 32];
+        __shared__ uint32_t seen_s;
+        uint32_t *w = warp_s[turn & 1];
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (turn == 0 && tid == 0) seen_s = *reinterpret_cast<volatile uint32_t *>(&dev->absmax_u32);
+        if ((tid & 31) == 0) w[tid >> 5] = mx;
+        __syncthreads();
+        uint32_t m = 0;
+#pragma unroll
+        for (int i = 0; i < kThreads / 32; ++i) m = max(m, w[i]);
+        own = max(own, m);
+        const int up = sq_up(max(own, seen_s));
+        if (m) shift = shift == kTileAny || shift == up ? up : kTileMixed;
+        ++turn;
+        return up;
+    }
+    __device__ __forceinline__ void publish(int tid, int16_t *tile_shift, DeviceState *dev) const
+    {
+        if (tid != 0) return;
+        *tile_shift = (int16_t)shift;
+        if (own) atomicMax(&dev->absmax_u32, own);
+        if (own >= 0x7f800000u) atomicOr(&dev->status, EOQ_DEV_NONFINITE);
+    }
+};
+
+// Second pass: calls again(tile, scale) in all threads of a block for those of its tiles that need it; tiles are dealt out from the
+// tensor's end, which the first pass read last.  `owner`: the thread that writes the exponent.
+template <typename Again>
+__device__ __forceinline__ void recode_tiles(const int16_t *tile_shift, int tiles, int tid, int32_t *dst_exp, DeviceState *dev, Again again)
+{
+    __shared__ uint32_t max_s;
+    __shared__ uint8_t wrong_s[kThreads];
+    bool last = false;
+    if (tid == 0) max_s = *reinterpret_cast<volatile uint32_t *>(&dev->absmax_u32);
+    for (int first = blockIdx.x; first < tiles; first += gridDim.x * kThreads) {   // (one round)
+        const int t = first + tid * (int)gridDim.x, used = t < tiles ? tile_shift[tiles - 1 - t] : kTileAny;
+        __syncthreads();
+        const int up = sq_up(max_s);
+        const bool wrong = used != kTileAny && used != up;
+        wrong_s[tid] = wrong;
+        if (first == (int)blockIdx.x && tid == 0) {
+            last = last_reader(dev);
+            if (blockIdx.x == 0) {
+                *dst_exp = -up;
+                if (max_s == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
+            }
+        }
+        if (!__syncthreads_or(wrong)) continue;
+        const Pow2Scale sc = pow2_scale(up);
+        for (int k = 0, t = first; k < kThreads && t < tiles; ++k, t += gridDim.x)
+            if (wrong_s[k]) again(tiles - 1 - t, sc);
+    }
     if (last) dev->absmax_u32 = 0;
+}
+
+// Part `p` of the tensor is kQuantTile float4; a tile is `reps` of them.
+__device__ __forceinline__ void load_part(const float *src, size_t n4, size_t p, float4 (&v)[kQuantLoads])
+{
+#pragma unroll
+    for (int u = 0; u < kQuantLoads; ++u) {
+        const size_t i = p * kQuantTile + (size_t)u * kThreads + threadIdx.x;
+        v[u] = i < n4 ? __ldg(reinterpret_cast<const float4 *>(src) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+__device__ __forceinline__ void store_part(int8_t *dst, size_t n4, size_t p, const Pow2Scale &sc, const float4 (&v)[kQuantLoads])
+{
+#pragma unroll
+    for (int u = 0; u < kQuantLoads; ++u) {
+        const size_t i = p * kQuantTile + (size_t)u * kThreads + threadIdx.x;
+        if (i < n4) quantize_store4<2>(dst, i, sc, v[u]);
+    }
+}
+__device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+
+__global__ void __launch_bounds__(kThreads)
+quantize_sq_kernel(const float *__restrict__ src, size_t n, int8_t *dst, int16_t *tile_shift, int reps, DeviceState *dev)
+{
+    ptx::grid_dep_wait_launch_small();
+    const size_t n4 = n / 4;
+    TileGuess guess;
+    for (int r = 0; r < reps; ++r) {
+        const size_t p = (size_t)blockIdx.x * reps + r;
+        float4 v[kQuantLoads];
+        load_part(src, n4, p, v);
+        uint32_t mx = 0;
+        // (the up to three elements behind the last float4 are coded by the second pass)
+        if (blockIdx.x == 0 && r == 0 && threadIdx.x < (n & 3)) mx = abs_bits(src[n4 * 4 + threadIdx.x]);
+#pragma unroll
+        for (int u = 0; u < kQuantLoads; ++u)
+            mx = max(max(mx, max(abs_bits(v[u].x), abs_bits(v[u].y))), max(abs_bits(v[u].z), abs_bits(v[u].w)));
+        store_part(dst, n4, p, pow2_scale(guess.part(mx, threadIdx.x, dev)), v);
+    }
+    guess.publish(threadIdx.x, tile_shift + blockIdx.x, dev);
+}
+
+__global__ void __launch_bounds__(kThreads, kAgainPerSm)
+quantize_sq_again_kernel(const float *__restrict__ src, size_t n, int8_t *dst, int32_t *dst_exp, const int16_t *tile_shift, int tiles, int reps,
+                         DeviceState *dev)
+{
+    ptx::grid_dep_wait_launch_small();
+    const size_t n4 = n / 4;
+    if (blockIdx.x == 0 && threadIdx.x < (n & 3)) {
+        const size_t i = n4 * 4 + threadIdx.x;
+        dst[i] = (int8_t)quantize_code<2>(pow2_scale(sq_up(*reinterpret_cast<volatile uint32_t *>(&dev->absmax_u32))), src[i]);
+    }
+    recode_tiles(tile_shift, tiles, threadIdx.x, dst_exp, dev, [&](int tile, const Pow2Scale &sc) {
+        for (int r = 0; r < reps; ++r) {
+            float4 v[kQuantLoads];
+            load_part(src, n4, (size_t)tile * reps + r, v);
+            store_part(dst, n4, (size_t)tile * reps + r, sc, v);
+        }
+    });
 }
 
 // SQ in one launch for tensors that one cluster can hold in registers (kSmallElems codes per block, up to
@@ -181,73 +270,140 @@ quantize_sq_small_kernel(const float *__restrict__ src, size_t n, int8_t *dst, i
     cluster.sync();  // no block leaves while another may still read its maximum
 }
 
-// SQ of an fp32 image under the already reduced maximum: c_src channels in, c_dst (zero-padded) channels out,
-// rows widened by `wmargin` zero pixels at both ends.  A thread writes kG = 16 or 8 channels of a pixel.
+// SQ of an fp32 image: c_src channels in, c_dst (zero-padded) channels out, rows widened by `wmargin` zero pixels at both ends.  A
+// thread writes kG = 16 or 8 channels of a pixel.  The same two passes: a part is kImageRows * blockDim.y rows, a tile `reps` of them.
 // Bound by memory (12 B in, 8 or 16 B out per RGB pixel).  A block is tx pixels x ty rows and a thread takes its pixel in
-// kImageRows rows, all loads issued before the maximum is needed, no divisions: 3.2 M pixels took 30.4 us with one
-// pixel at a time behind three of them.
+// kImageRows rows, all loads issued before the maximum is needed, no divisions.  64 images 224 x 224: 10.7 us for the maximum and 13.4
+// for the codes before; now 16.0 + 2.8, and 16.0 + 13.6 where every tile was wrong.
 constexpr int kImageRows = 4;
+struct ImageShape {
+    int rows, w, c_src, c_dst, wmargin;
+};
+// 16 or 8 codes of an output pixel from the values of its channels (`more`: those beyond the first four, read again)
 template <int kG>
-__global__ void __launch_bounds__(kThreads)
-quantize_image_kernel(const float *__restrict__ src, int rows, int w, int c_src, int c_dst, int wmargin, int8_t *dst, int32_t *dst_exp,
-                      DeviceState *dev)
+__device__ __forceinline__ void image_store(int8_t *dst, size_t o, const Pow2Scale &sc, const float (&v)[4], const float *more, int nch)
 {
-    ptx::grid_dep_wait_launch_small();
-    __shared__ uint32_t max_s;
-    const int groups = c_dst / kG, w_mem = w + 2 * wmargin, items = w_mem * groups;
-    const int row0 = blockIdx.x * (kImageRows * blockDim.y) + threadIdx.y;
-    const bool t0 = threadIdx.x == 0 && threadIdx.y == 0;
-    int up = 7;
-    bool last = false;
-    for (int x0 = 0; x0 < items; x0 += blockDim.x) {   // one round unless a row is wider than the block
+    int c[kG];
+#pragma unroll
+    for (int k = 0; k < kG; ++k) c[k] = k < 4 ? quantize_code<2>(sc, v[k & 3]) : (more && k < nch ? quantize_code<2>(sc, __ldg(more + k)) : 0);
+    if (kG == 16)
+        reinterpret_cast<uint4 *>(dst)[o] = make_uint4(pack4_sat(c[0], c[1], c[2], c[3]), pack4_sat(c[4], c[5], c[6], c[7]),
+                                                       pack4_sat(c[8 % kG], c[9 % kG], c[10 % kG], c[11 % kG]),
+                                                       pack4_sat(c[12 % kG], c[13 % kG], c[14 % kG], c[15 % kG]));
+    else
+        reinterpret_cast<uint2 *>(dst)[o] = make_uint2(pack4_sat(c[0], c[1], c[2], c[3]), pack4_sat(c[4], c[5], c[6], c[7]));
+}
+
+// One part (`first_row`: the thread's first): scale_of(maximum of the thread's channels) gives the scale, once per round of a row
+// (one unless a row is wider than the block).
+template <int kG, typename ScaleOf>
+__device__ __forceinline__ void image_part(const float *__restrict__ src, const ImageShape &s, int first_row, int8_t *dst, ScaleOf scale_of)
+{
+    const int groups = s.c_dst / kG, items = (s.w + 2 * s.wmargin) * groups;
+    for (int x0 = 0; x0 < items; x0 += blockDim.x) {
         const int it = x0 + threadIdx.x;
-        const int xp = groups == 1 ? it : it / groups, g = groups == 1 ? 0 : it - xp * groups, xm = xp - wmargin;
-        const int nch = min(kG, c_src - g * kG);       // real channels of this group (none or fewer beyond c_src)
-        const bool in = it < items && xm >= 0 && xm < w;
-        float v[kImageRows][4];                        // the first four channels; more are read when they are coded
+        const int xp = groups == 1 ? it : it / groups, g = groups == 1 ? 0 : it - xp * groups, xm = xp - s.wmargin;
+        const int nch = min(kG, s.c_src - g * kG);       // real channels of this group (none or fewer beyond c_src)
+        const bool in = it < items && xm >= 0 && xm < s.w;
+        float v[kImageRows][4];
+        uint32_t mx = 0;
 #pragma unroll
         for (int u = 0; u < kImageRows; ++u) {
-            const int row = row0 + u * blockDim.y;
-            const float *p = src + ((size_t)row * w + xm) * c_src + g * kG;
+            const int row = first_row + u * blockDim.y;
+            const float *p = src + ((size_t)row * s.w + xm) * s.c_src + g * kG;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) v[u][k] = (in && row < rows && k < nch) ? __ldg(p + k) : 0.0f;
+            for (int k = 0; k < 4; ++k) v[u][k] = (in && row < s.rows && k < nch) ? __ldg(p + k) : 0.0f;
+            if (in && row < s.rows)
+                for (int k = 4; k < nch; ++k) mx = max(mx, abs_bits(__ldg(p + k)));
         }
-        if (x0 == 0) {
-            if (t0) max_s = *reinterpret_cast<volatile uint32_t *>(&dev->absmax_u32);
-            __syncthreads();
-            up = sq_up(max_s);
-            if (t0) {
-                last = last_reader(dev);
-                if (blockIdx.x == 0) {
-                    *dst_exp = -up;
-                    if (max_s == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-                }
-            }
-        }
-        const Pow2Scale sc = pow2_scale(up);
+#pragma unroll
+        for (int u = 0; u < kImageRows; ++u)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) mx = max(mx, abs_bits(v[u][k]));
+        const Pow2Scale sc = scale_of(mx);
 #pragma unroll
         for (int u = 0; u < kImageRows; ++u) {
-            const int row = row0 + u * blockDim.y;
-            if (it >= items || row >= rows) continue;
-            int c[kG];
-#pragma unroll
-            for (int k = 0; k < kG; ++k) c[k] = k < 4 ? quantize_code<2>(sc, v[u][k & 3]) : 0;
-            if (in && nch > 4) {
-                const float *p = src + ((size_t)row * w + xm) * c_src + g * kG;
-#pragma unroll
-                for (int k = 4; k < kG; ++k)
-                    if (k < nch) c[k] = quantize_code<2>(sc, __ldg(p + k));
-            }
-            const size_t o = (size_t)row * items + it;
-            if (kG == 16)
-                reinterpret_cast<uint4 *>(dst)[o] = make_uint4(pack4_sat(c[0], c[1], c[2], c[3]), pack4_sat(c[4], c[5], c[6], c[7]),
-                                                               pack4_sat(c[8 % kG], c[9 % kG], c[10 % kG], c[11 % kG]),
-                                                               pack4_sat(c[12 % kG], c[13 % kG], c[14 % kG], c[15 % kG]));
-            else
-                reinterpret_cast<uint2 *>(dst)[o] = make_uint2(pack4_sat(c[0], c[1], c[2], c[3]), pack4_sat(c[4], c[5], c[6], c[7]));
+            const int row = first_row + u * blockDim.y;
+            if (it >= items || row >= s.rows) continue;
+            image_store<kG>(dst, (size_t)row * items + it, sc, v[u], in && nch > 4 ? src + ((size_t)row * s.w + xm) * s.c_src + g * kG : nullptr, nch);
         }
     }
-    if (last) dev->absmax_u32 = 0;
+}
+
+// First pass over images of up to four channels in one group, no row wider than the block: a part is then a run of at most
+// 4 * kThreads pixels, which the block reads as float4 and hands out through shared memory (a pixel's channels read one by one, 64
+// images 224 x 224: 19.7 us, 16.0 so).
+template <int kG>
+__device__ __forceinline__ void image_part_staged(const float *__restrict__ src, const ImageShape &s, int part, int tid, TileGuess &guess, int8_t *dst,
+                                                  DeviceState *dev)
+{
+    __shared__ __align__(16) float stage[4 * kImageRows * kThreads];
+    const int part_rows = kImageRows * blockDim.y, row0 = part * part_rows, rows = min(part_rows, s.rows - row0);
+    const int count = rows > 0 ? rows * s.w * s.c_src : 0;
+    const float *p = src + (size_t)row0 * s.w * s.c_src;   // (16-byte aligned: part_rows is a multiple of 4)
+    float4 v[kImageRows];
+    uint32_t mx = 0;
+#pragma unroll
+    for (int u = 0; u < kImageRows; ++u) {
+        const int i = u * kThreads + tid;
+        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (4 * i + 3 < count) v[u] = __ldg(reinterpret_cast<const float4 *>(p) + i);
+        else if (4 * i < count) {
+            v[u].x = __ldg(p + 4 * i);
+            if (4 * i + 1 < count) v[u].y = __ldg(p + 4 * i + 1);
+            if (4 * i + 2 < count) v[u].z = __ldg(p + 4 * i + 2);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kImageRows; ++u) {
+        mx = max(max(mx, max(abs_bits(v[u].x), abs_bits(v[u].y))), max(abs_bits(v[u].z), abs_bits(v[u].w)));
+        reinterpret_cast<float4 *>(stage)[u * kThreads + tid] = v[u];
+    }
+    const Pow2Scale sc = pow2_scale(guess.part(mx, tid, dev));   // (its barrier also publishes the stage)
+    const int w_mem = s.w + 2 * s.wmargin, xm = (int)threadIdx.x - s.wmargin;
+    const bool in = xm >= 0 && xm < s.w;
+#pragma unroll
+    for (int u = 0; u < kImageRows; ++u) {
+        const int r = threadIdx.y + u * blockDim.y;
+        if ((int)threadIdx.x >= w_mem || r >= rows) continue;
+        const float *q = stage + (r * s.w + xm) * s.c_src;
+        float f[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) f[k] = in && k < s.c_src ? q[k] : 0.0f;
+        image_store<kG>(dst, (size_t)(row0 + r) * w_mem + threadIdx.x, sc, f, nullptr, 0);
+    }
+}
+
+template <int kG, bool kStaged>
+__global__ void __launch_bounds__(kThreads)
+quantize_image_kernel(const float *__restrict__ src, ImageShape s, int8_t *dst, int16_t *tile_shift, int reps, DeviceState *dev)
+{
+    ptx::grid_dep_wait_launch_small();
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    TileGuess guess;
+    for (int r = 0; r < reps; ++r) {
+        const int part = (int)blockIdx.x * reps + r;
+        if (kStaged) {
+            if (r > 0) __syncthreads();   // (the stage is read)
+            image_part_staged<kG>(src, s, part, tid, guess, dst, dev);
+        } else {
+            image_part<kG>(src, s, part * kImageRows * (int)blockDim.y + threadIdx.y, dst, [&](uint32_t mx) { return pow2_scale(guess.part(mx, tid, dev)); });
+        }
+    }
+    guess.publish(tid, tile_shift + blockIdx.x, dev);
+}
+
+template <int kG>
+__global__ void __launch_bounds__(kThreads, kAgainPerSm)
+quantize_image_again_kernel(const float *__restrict__ src, ImageShape s, int8_t *dst, int32_t *dst_exp, const int16_t *tile_shift, int tiles,
+                            int reps, DeviceState *dev)
+{
+    ptx::grid_dep_wait_launch_small();
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x, part_rows = kImageRows * blockDim.y;
+    recode_tiles(tile_shift, tiles, tid, dst_exp, dev, [&](int tile, const Pow2Scale &sc) {
+        for (int r = 0; r < reps; ++r)
+            image_part<kG>(src, s, (tile * reps + r) * part_rows + threadIdx.y, dst, [&](uint32_t) { return sc; });
+    });
 }
 
 // w[oc][kh][kw][c] -> wp[oc][kh][8][c] with zeros in the unused taps; c = 16 (Pixel = int4) or 8 (int2)
@@ -1040,7 +1196,22 @@ cudaError_t launch_reset_cells(DeviceState *dev, cudaStream_t s)
 
 bool quantize_is_small(int mode, size_t n, const ReduceHook &hook) { return mode == 2 && !hook.fn && n <= kSmallElems * kSmallCluster; }
 
-cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev,
+// Tiles of the two-pass SQ: `reps` parts each, more than one only where the handle has no cell for every part; the second pass's
+// blocks look after at most kThreads tiles each.
+struct TileSplit {
+    int reps, tiles, again_blocks;
+};
+static TileSplit split_tiles(size_t parts, int sm_count)
+{
+    TileSplit t;
+    t.reps = (int)((parts + kSqTiles - 1) / kSqTiles);
+    t.tiles = (int)((parts + t.reps - 1) / t.reps);
+    const int least = (t.tiles + kThreads - 1) / kThreads, most = kAgainPerSm * sm_count;
+    t.again_blocks = t.tiles < most ? t.tiles : (least > most ? least : most);
+    return t;
+}
+
+cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst, int32_t *dst_exp, int16_t *tile_shift, DeviceState *dev,
                                 int sm_count, cudaStream_t s, const ReduceHook &hook)
 {
     if (quantize_is_small(mode, n, hook)) {
@@ -1057,30 +1228,36 @@ cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst,
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, quantize_sq_small_kernel, src, n, static_cast<int8_t *>(dst), dst_exp, dev);
     }
-    if (mode == 2) {
-        launch_chained(absmax_f32_kernel, grid_for(n / 4 + 1, sm_count), kThreads, 0, s, src, n, dev);
+    const size_t parts = (n / 4 + kQuantTile - 1) / kQuantTile > 0 ? (n / 4 + kQuantTile - 1) / kQuantTile : 1;
+    if (mode == 0) launch_chained(quantize_f32_kernel<0>, (unsigned)parts, kThreads, 0, s, src, n, dst, dst_exp);
+    else if (mode == 1) launch_chained(quantize_f32_kernel<1>, (unsigned)parts, kThreads, 0, s, src, n, dst, dst_exp);
+    else {
+        const TileSplit t = split_tiles(parts, sm_count);
+        launch_chained(quantize_sq_kernel, t.tiles, kThreads, 0, s, src, n, static_cast<int8_t *>(dst), tile_shift, t.reps, dev);
         hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);  // float bit patterns of |x| order like integers
+        launch_chained(quantize_sq_again_kernel, t.again_blocks, kThreads, 0, s, src, n, static_cast<int8_t *>(dst), dst_exp,
+                       (const int16_t *)tile_shift, t.tiles, t.reps, dev);
     }
-    const unsigned blocks = (unsigned)((n / 4 + kQuantTile - 1) / kQuantTile > 0 ? (n / 4 + kQuantTile - 1) / kQuantTile : 1);
-    if (mode == 0) launch_chained(quantize_f32_kernel<0>, blocks, kThreads, 0, s, src, n, dst, dst_exp, dev);
-    else if (mode == 1) launch_chained(quantize_f32_kernel<1>, blocks, kThreads, 0, s, src, n, dst, dst_exp, dev);
-    else launch_chained(quantize_f32_kernel<2>, blocks, kThreads, 0, s, src, n, dst, dst_exp, dev);
     return cudaGetLastError();
 }
 
-cudaError_t launch_quantize_image(const float *src, int n, int h, int w, int c_src, int c_dst, int wmargin, int8_t *dst,
-                                  int32_t *dst_exp, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook)
+cudaError_t launch_quantize_image(const float *src, int n, int h, int w, int c_src, int c_dst, int wmargin, int8_t *dst, int32_t *dst_exp,
+                                  int16_t *tile_shift, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook)
 {
-    const size_t count = (size_t)n * h * w * c_src;
-    launch_chained(absmax_f32_kernel, grid_for(count / 4 + 1, sm_count), kThreads, 0, s, src, count, dev);
-    hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
-    const int g = c_dst % 16 == 0 ? 16 : 8, items = (w + 2 * wmargin) * (c_dst / g), rows = n * h;
+    const int g = c_dst % 16 == 0 ? 16 : 8, items = (w + 2 * wmargin) * (c_dst / g);
+    const ImageShape shape{n * h, w, c_src, c_dst, wmargin};
     int tx = 32;
     while (tx < items && tx < kThreads) tx *= 2;
     const dim3 block(tx, kThreads / tx);
-    const unsigned grid = (unsigned)((rows + kImageRows * (int)block.y - 1) / (kImageRows * (int)block.y));
-    if (g == 16) launch_chained(quantize_image_kernel<16>, grid, block, 0, s, src, rows, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
-    else launch_chained(quantize_image_kernel<8>, grid, block, 0, s, src, rows, w, c_src, c_dst, wmargin, dst, dst_exp, dev);
+    const int part_rows = kImageRows * (int)block.y;
+    const TileSplit t = split_tiles((size_t)(shape.rows + part_rows - 1) / part_rows, sm_count);
+    const bool staged = c_src <= 4 && c_dst == g && items <= kThreads;
+    const auto first = staged ? (g == 16 ? quantize_image_kernel<16, true> : quantize_image_kernel<8, true>)
+                              : (g == 16 ? quantize_image_kernel<16, false> : quantize_image_kernel<8, false>);
+    launch_chained(first, t.tiles, block, 0, s, src, shape, dst, tile_shift, t.reps, dev);
+    hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
+    launch_chained(g == 16 ? quantize_image_again_kernel<16> : quantize_image_again_kernel<8>, t.again_blocks, block, 0, s, src, shape, dst,
+                   dst_exp, (const int16_t *)tile_shift, t.tiles, t.reps, dev);
     return cudaGetLastError();
 }
 

@@ -110,6 +110,7 @@ struct ReduceHook {
     }
 };
 
+constexpr int kSqTiles = 32768;
 constexpr int kClassBranches = 3;
 
 struct ProfRecord {
@@ -122,6 +123,7 @@ struct Handle {
     int sm_count;
     int last_cuda_error;
     DeviceState *dev;
+    int16_t *tile_shift;          // kSqTiles cells behind the device state: the shifts under which the first pass of SQ coded its tiles
     unsigned long long launches;  // kernels launched through this handle
     bool profiling;
     ReduceHook hook;              // all-reduce between the phases of every batch-wide reduction (data-parallel replicas)
@@ -341,12 +343,13 @@ cudaError_t launch_probe_mma_i8(int n_cols, int iters, int grid, DeviceState *de
 // Elementwise / reduction kernels
 // ---------------------------------------------------------------------------------------------
 cudaError_t launch_reset_cells(DeviceState *dev, cudaStream_t s);
-cudaError_t launch_quantize_image(const float *src, int n, int h, int w, int c_src, int c_dst, int wmargin, int8_t *dst,
-                                  int32_t *dst_exp, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook);
+cudaError_t launch_quantize_image(const float *src, int n, int h, int w, int c_src, int c_dst, int wmargin, int8_t *dst, int32_t *dst_exp,
+                                  int16_t *tile_shift, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook);
 // w[oc][kh][kw][16] -> wp[oc][kh][8][16], zero in the taps kw..7 (weights of the filter-row path)
 cudaError_t launch_weight_pad_rows(const int8_t *w, int8_t *wp, int c_out, int kh, int kw, int c_in, cudaStream_t s);
 bool quantize_is_small(int mode, size_t n, const ReduceHook &hook);  // one launch instead of two
-cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev,
+// tile_shift: kSqTiles cells of the handle (written by the first pass of SQ, read by the second)
+cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst, int32_t *dst_exp, int16_t *tile_shift, DeviceState *dev,
                                 int sm_count, cudaStream_t s, const ReduceHook &hook);
 cudaError_t launch_sq_i32(const int32_t *src, const int32_t *src_exp, int exp_bias, size_t n, int8_t *dst,
                           int32_t *dst_exp, long long *sum_codes, bool max_already_reduced, DeviceState *dev,

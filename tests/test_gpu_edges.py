@@ -365,6 +365,62 @@ def test_quantize_float_of_whole_device_shares(loads, extra, kind):
         assert np.array_equal(G.host(out), c) and ex.item() == p
 
 
+@pytest.mark.parametrize("kind", ["rising", "falling", "one tile", "zero tiles", "nan"])
+@pytest.mark.parametrize("n", [262145, 262144 + 8192, 1000003, 1 << 23])
+def test_quantize_float_whose_parts_have_other_scales(n, kind):
+    """SQ codes parts of the tensor before its maximum is known: parts whose own maximum asks for another shift than the whole
+    tensor's, parts of zeros, and a maximum that only the last part holds."""
+    x = synth.normal_f32(n, 3040, 0)
+    part = np.arange(n) // 8192
+    if kind in ("rising", "falling"):
+        steps = part if kind == "rising" else part[::-1]
+        x *= np.exp2(steps % 97 - 40).astype(np.float32)
+    elif kind == "one tile":
+        x[n - 1] = 3000.0
+    elif kind == "zero tiles":
+        x[(part % 3) != 1] = -0.0
+    else:
+        x[n // 2] = np.nan
+    h, out, ex = G.handle(), G.empty((n,), torch.int8), G.zeros(1, torch.int32)
+    eoq.eoq_quantize(h, eoq.EOQ_SQ, G.dev(x), True, None, n, out, ex)
+    assert G.status_clear() == (eoq.EOQ_DEV_NONFINITE if kind == "nan" else 0)
+    if kind == "nan":   # flagged; the codes are those at an exponent of -7
+        c, p = np.clip(np.rint(np.nan_to_num(x) * np.float32(128)), -127, 127).astype(np.int8), -7
+    else:
+        c, p, _ = oracle.quantize_f32(oracle.MODE_SQ, x)
+    assert ex.item() == p and np.array_equal(G.host(out), c)
+
+
+@pytest.mark.parametrize("scales", ["even", "one row"])
+@pytest.mark.parametrize("shape,c_dst,margin", [((1100, 1000, 1, 3), 8, 0), ((5, 37, 300, 3), 8, 2), ((3, 50, 41, 11), 16, 1), ((2, 9, 40, 20), 48, 0)])
+def test_quantize_image_whose_rows_have_other_scales(shape, c_dst, margin, scales):
+    """The same for images: more parts than the handle has cells for, rows wider than a block, channels beyond the first four."""
+    n, h, w, c = shape
+    x = synth.normal_f32(shape, 3041, c)
+    if scales == "one row":
+        x[n - 1, h - 1] *= np.float32(1000.0)
+    x[0, : h // 2] *= np.float32(0.01)
+    codes, p, _ = oracle.quantize_f32(eoq.EOQ_SQ, x.reshape(-1))
+    out, ex = G.empty((n, h, w + 2 * margin, c_dst), torch.int8), G.zeros(1, torch.int32)
+    eoq.eoq_quantize_image(G.handle(), G.dev(x), n, h, w, c, c_dst, margin, out, ex)
+    want = np.zeros((n, h, w + 2 * margin, c_dst), dtype=np.int8)
+    want[:, :, margin:margin + w, :c] = codes.reshape(shape)
+    assert G.status_clear() == 0 and ex.item() == p and np.array_equal(G.host(out), want)
+
+
+def test_quantize_float_of_more_parts_than_cells():
+    """A tensor of more than 2^28 floats, whose blocks take several parts each: repetitions of one run of floats."""
+    run, times = 1000003, 269
+    x = synth.normal_f32(run, 3042, 0)
+    x[7] = 20.0
+    codes, p, _ = oracle.quantize_f32(oracle.MODE_SQ, x)
+    src = torch.from_numpy(x).cuda().repeat(times)
+    out, ex = G.empty((run * times,), torch.int8), G.zeros(1, torch.int32)
+    eoq.eoq_quantize(G.handle(), eoq.EOQ_SQ, src, True, None, run * times, out, ex)
+    assert G.status_clear() == 0 and ex.item() == p
+    assert bool((out.view(times, run) == torch.from_numpy(codes).cuda()).all())
+
+
 @pytest.mark.parametrize("n", [262144, 6000001, 64 * 56 * 56 * 64 + 1])
 def test_quantize_float_runs_beside_a_long_kernel(n):
     """SQ needs no SM for itself alone: it ends while a kernel of another stream still occupies one (a convolution capped to one CTA,
