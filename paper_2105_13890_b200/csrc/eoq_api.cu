@@ -319,6 +319,31 @@ double few_igemm_time(const IgemmParams &p)
     return t;
 }
 
+// The fastest column tile at `split` CTAs per tile within `ctas` (false: none).
+bool narrow_tiles(const IgemmParams &p, int split, int ctas, IgemmParams &best, double &best_time)
+{
+    const int k_iters = (p.num_sub + p.subs_per_stage - 1) / p.subs_per_stage;
+    bool found = false;
+    for (int cuts = 1; cuts <= 32; cuts *= 2) {
+        const int tn = ((p.N + cuts - 1) / cuts + 15) / 16 * 16;
+        if (tn > 128) continue;
+        if (!(split > 1 && (p.kc < 64 || k_iters < split || tn / 16 > 4 * split))) {
+            IgemmParams q = p;
+            set_columns(q, tn, split);
+            if (q.num_m_tiles * q.num_n_tiles * split <= (split > 1 ? ctas / 2 : ctas)) {
+                const double time = few_igemm_time(q);
+                if (!found || time < 0.97 * best_time) {
+                    best = q;
+                    best_time = time;
+                    found = true;
+                }
+            }
+        }
+        if (tn == 16) break;
+    }
+    return found;
+}
+
 // Columns per tile and CTAs per tile of the im2col kernel.  Clusters take at most half of the CTAs (beyond that many, some wait for
 // room: 512 channels 7 x 7, one image: 64 CTAs 5.9 us, 128 CTAs 6.7) and want every CTA to have a K iteration of at least two MMAs.
 void plan_few_tiles(IgemmParams &p, int ctas)
@@ -344,6 +369,67 @@ void plan_few_tiles(IgemmParams &p, int ctas)
         if (tn == 16) break;
     }
     p = best;
+}
+
+// Tiles and CTAs of the residue classes that share a launch (cl.num of them, planned by plan_igemm).
+// CTAs: the fewest per class with which the class that takes longest is done first.  A tile costs its taps and, about half of one, its
+// sums: by taps alone the class of one tap ended last.
+// Few tiles: as plan_few_tiles, each class within its share of the CTAs, with one split for all of them.
+void plan_classes(IgemmClasses &cl, int ctas)
+{
+    if (cl.num == 1) {
+        plan_few_tiles(cl.p[0], ctas);
+    } else {
+        int share[kMaxClasses], total = 0;
+        for (int k = 0; k < cl.num; ++k) total += 2 * cl.p[k].ntaps + 1;
+        bool few = true;
+        for (int k = 0; k < cl.num; ++k) {
+            share[k] = ctas * (2 * cl.p[k].ntaps + 1) / total;
+            if (share[k] < 1) share[k] = 1;
+            few = few && 2 * cl.p[k].num_m_tiles * cl.p[k].num_n_tiles <= share[k];
+        }
+        double best_time = 0;
+        IgemmParams best[kMaxClasses];
+        for (int split = 1; few && split <= 8; split *= 2) {
+            IgemmParams q[kMaxClasses];
+            double slowest = 0;
+            bool ok = true;
+            for (int k = 0; k < cl.num && ok; ++k) {
+                double time = 0;
+                ok = narrow_tiles(cl.p[k], split, share[k], q[k], time);
+                if (time > slowest) slowest = time;
+            }
+            if (ok && (split == 1 || slowest < 0.97 * best_time)) {
+                best_time = slowest;
+                memcpy(best, q, sizeof(IgemmParams) * cl.num);
+            }
+        }
+        if (best_time > 0) memcpy(cl.p, best, sizeof(IgemmParams) * cl.num);
+    }
+    int cost[kMaxClasses], tiles[kMaxClasses];
+    long long work = 0;
+    for (int k = 0; k < cl.num; ++k) {
+        tiles[k] = cl.p[k].num_m_tiles * cl.p[k].num_n_tiles;
+        cost[k] = 2 * cl.p[k].ntaps + 1;
+        work += (long long)tiles[k] * cost[k];
+    }
+    // (a time of all tiles on a single CTA each is always enough: the search ends)
+    for (long long time = work / ctas;; ++time) {
+        int used = 0;
+        bool fits = true;
+        cl.first[0] = 0;
+        for (int k = 0; k < cl.num; ++k) {
+            const long long per_cta = cl.p[0].split > 1 ? 1 : time / cost[k];   // (a cluster has one tile)
+            if (per_cta < 1) {
+                fits = false;
+                break;
+            }
+            used += (int)((tiles[k] + per_cta - 1) / per_cta);
+            cl.first[k + 1] = used * cl.p[0].split;
+        }
+        if (fits && (used <= ctas || used <= cl.num)) break;
+    }
+    for (int k = 0; k < cl.num; ++k) plan_epilogue(cl.p[k], (cl.first[k + 1] - cl.first[k]) / cl.p[0].split);
 }
 
 // Plan of the patch variant for a stride-1 k x k correlation over a source [n][hs][ws][c_src] producing a
@@ -757,11 +843,6 @@ extern "C" int eoq_create(eoq_handle_t *handle, int device)
     h->hook = ReduceHook{nullptr, nullptr};
     h->num_records = 0;
     h->records = nullptr;
-    h->fork_ev = nullptr;
-    for (int k = 0; k < kClassBranches; ++k) {
-        h->class_branch[k] = nullptr;
-        h->class_join[k] = nullptr;
-    }
     // two attributes: cudaGetDeviceProperties took 2.5 of the call's 3.1 ms, and a training step creates four handles
     int major = 0;
     cudaError_t e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, device);
@@ -776,18 +857,8 @@ extern "C" int eoq_create(eoq_handle_t *handle, int device)
     }
     if (e == cudaSuccess) e = cudaMemset(h->dev, 0, sizeof(DeviceState));
     h->tile_shift = reinterpret_cast<int16_t *>(reinterpret_cast<char *>(h->dev) + round256(sizeof(DeviceState)));
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming);
-    for (int k = 0; k < kClassBranches && e == cudaSuccess; ++k) {
-        e = cudaStreamCreateWithFlags(&h->class_branch[k], cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->class_join[k], cudaEventDisableTiming);
-    }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
-        for (int k = 0; k < kClassBranches; ++k) {
-            if (h->class_join[k]) cudaEventDestroy(h->class_join[k]);
-            if (h->class_branch[k]) cudaStreamDestroy(h->class_branch[k]);
-        }
-        if (h->fork_ev) cudaEventDestroy(h->fork_ev);
         if (h->dev) cudaFree(h->dev);
         delete h;
         return EOQ_ERR_CUDA;
@@ -802,11 +873,6 @@ extern "C" int eoq_destroy(eoq_handle_t handle)
     if (!h) return EOQ_ERR_BAD_ARG;
     cudaSetDevice(h->device);
     cudaDeviceSynchronize();
-    for (int k = 0; k < kClassBranches; ++k) {
-        if (h->class_join[k]) cudaEventDestroy(h->class_join[k]);
-        if (h->class_branch[k]) cudaStreamDestroy(h->class_branch[k]);
-    }
-    if (h->fork_ev) cudaEventDestroy(h->fork_ev);
     if (h->dev) cudaFree(h->dev);
     if (h->records) {
         for (int i = 0; i < h->num_records; ++i) {
@@ -1380,37 +1446,33 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
                      : cudaMemsetAsync(sums16, 0, g.in_elems * sizeof(uint16_t), s);
         if (e != cudaSuccess) return record(h, e);
     }
-    // The classes write disjoint pixels, so their GEMMs are independent: with more than one class and branch streams
-    // at hand they are issued side by side (fork on `s`, one stream per class, joins before Q_e), each with a
-    // share of the CTAs in proportion to its work, instead of one after the other at full width.
-    int total_taps = 0, live_classes = 0;
-    for (int py = 0; py < d.stride && py < d.h; ++py)
-        for (int px = 0; px < d.stride && px < d.w; ++px) {
-            int nh = 0, nw = 0;
-            for (int kh = 0; kh < d.kh; ++kh) nh += (py + d.pad - kh) % d.stride == 0;
-            for (int kw = 0; kw < d.kw; ++kw) nw += (px + d.pad - kw) % d.stride == 0;
-            total_taps += nh * nw;
-            live_classes += nh * nw > 0;
+    // The classes write disjoint pixels: up to kMaxClasses of them share a launch, each with its share of the CTAs.
+    IgemmClasses cl;
+    cl.num = 0;
+    int dw_of[kMaxClasses], dh_of[kMaxClasses];
+    auto launch_classes = [&]() -> int {
+        if (cl.num == 0) return EOQ_OK;
+        plan_classes(cl, h->gemm_ctas);
+        for (int k = 0; k < cl.num; ++k) {
+            const IgemmParams &p = cl.p[k];
+            if (!make_im2col_map(&cl.map_a[k], e3, d.n, g.ho, g.wo, d.c_out, dw_of[k], dh_of[k], p.wq, p.hq, 1, p.kc, p.a_rows) ||
+                !(weights_in_place ? make_weight_map(&cl.map_b[k], w, d.c_out, g.taps, d.c_in, p.b_row, p.kc)
+                                   : make_weight_map(&cl.map_b[k], wt, d.c_in, g.taps, d.c_out, p.kc, p.tile_n)))
+                return EOQ_ERR_UNSUPPORTED;
         }
-    // (also where a class alone would keep the device busy: one launch's ramp and last wave hide behind the others; 64 channels
-    // 56 x 56 at batch 64: 40.0 -> 35.0 us with its quantizer)
-    const bool side_by_side = live_classes > 1 && h->class_branch[0] != nullptr;
-    // timed as one group on `s` (fork to join): the brackets of kernels that run side by side would overlap
-    ProfScope *group = side_by_side ? new (std::nothrow) ProfScope(h, EOQ_PROF_IGEMM_DGRAD, s) : nullptr;
-    struct GroupEnd {
-        ProfScope *&g;
-        ~GroupEnd() { delete g; }
-    } group_end{group};
-    if (side_by_side) {
-        e = cudaEventRecord(h->fork_ev, s);
-        if (e != cudaSuccess) return record(h, e);
-    }
+        count_launches(h, 1);
+        ProfScope prof(h, EOQ_PROF_IGEMM_DGRAD, s);
+        e = cl.num == 1 ? launch_igemm(cl.p[0], cl.map_a[0], cl.map_b[0], cl.first[1], s) : launch_igemm_classes(cl, s);
+        cl.num = 0;
+        if (e != cudaSuccess) {
+            launch_reset_cells(h->dev, s);  // GEMMs already queued have touched the maximum cell
+            return record(h, e);
+        }
+        return EOQ_OK;
+    };
     int class_no = 0;
-    unsigned joins = 0;
     for (int py = 0; py < d.stride && py < d.h; ++py)
         for (int px = 0; px < d.stride && px < d.w; ++px) {
-            IgemmParams p;
-            memset(&p, 0, sizeof(p));
             int dh[16], dw[16], kh_of[16], kw_of[16], nh = 0, nw = 0, min_h = 0, min_w = 0;
             for (int kh = 0; kh < d.kh; ++kh)
                 if ((py + d.pad - kh) % d.stride == 0) {
@@ -1429,6 +1491,12 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
                 }
             const int hq = (d.h - py + d.stride - 1) / d.stride, wq = (d.w - px + d.stride - 1) / d.stride;
             if (nh == 0 || nw == 0) continue;  // no tap reaches this class: its sums stay zero
+            if (cl.num == kMaxClasses && (st = launch_classes()) != EOQ_OK) return st;
+            dh_of[cl.num] = min_h;
+            dw_of[cl.num] = min_w;
+            IgemmParams &p = cl.p[cl.num++];
+            memset(&p, 0, sizeof(p));
+            ++class_no;
             p.M = d.n * hq * wq;
             p.N = d.c_in;
             p.hq = hq;
@@ -1458,48 +1526,8 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.sums16 = sums16;
             p.dev = h->dev;
             p.next_mask = next ? next->mask : nullptr;
-            // a tile costs its taps and, about half of one, its sums: by taps alone the class of one tap ended last
-            int ctas = h->gemm_ctas;
-            if (side_by_side) ctas = (int)((long long)h->gemm_ctas * (2 * nh * nw + 1) / (2 * total_taps + live_classes));
-            if (ctas < 1) ctas = 1;
-            plan_few_tiles(p, ctas);
-            CUtensorMap map_a, map_b;
-            if (!make_im2col_map(&map_a, e3, d.n, g.ho, g.wo, d.c_out, min_w, min_h, wq, hq, 1, p.kc, p.a_rows) ||
-                !(weights_in_place ? make_weight_map(&map_b, w, d.c_out, g.taps, d.c_in, p.b_row, p.kc)
-                                   : make_weight_map(&map_b, wt, d.c_in, g.taps, d.c_out, p.kc, p.tile_n)))
-                return EOQ_ERR_UNSUPPORTED;
-            count_launches(h, 1);
-            cudaStream_t cs = s;
-            if (side_by_side && class_no > 0) {
-                const int k = (class_no - 1) % kClassBranches;
-                cs = h->class_branch[k];
-                // a stream that already carries a class of this call simply queues the next one behind it
-                if (!(joins & (1u << k))) e = cudaStreamWaitEvent(cs, h->fork_ev, 0);
-                if (e != cudaSuccess) return record(h, e);
-                joins |= 1u << k;
-            }
-            ++class_no;
-            const int grid = persistent_grid(p.num_m_tiles * p.num_n_tiles, ctas);
-            plan_epilogue(p, grid);
-            if (side_by_side) {
-                e = launch_igemm(p, map_a, map_b, grid * p.split, cs);
-            } else {
-                ProfScope prof(h, EOQ_PROF_IGEMM_DGRAD, cs);
-                e = launch_igemm(p, map_a, map_b, grid * p.split, cs);
-            }
-            if (e != cudaSuccess) {
-                launch_reset_cells(h->dev, s);  // GEMMs already queued have touched the maximum cell
-                return record(h, e);
-            }
         }
-    for (int k = 0; k < kClassBranches; ++k)
-        if (joins & (1u << k)) {
-            e = cudaEventRecord(h->class_join[k], h->class_branch[k]);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->class_join[k], 0);
-            if (e != cudaSuccess) return record(h, e);
-        }
-    delete group;  // closes the group's bracket on `s`, behind the joins
-    group = nullptr;
+    if ((st = launch_classes()) != EOQ_OK) return st;
     if (h->gemm_only) return EOQ_OK;
     if (class_no == 0)   // no tap reaches any pixel: no GEMM ran
         for (long long *z : zero_sums)

@@ -24,10 +24,9 @@ constexpr int kProducers = 3;
 // share.  Small batches leave a handful of tiles with long reductions: the 512-channel 7 x 7 layer at batch 1 took 13.3 us on
 // 4 CTAs.  The exchange is the price, bound by distributed shared memory: with whole tiles of 128 rows exchanged by columns it was
 // 3.5 us of that layer's 7.4 on 32 CTAs; of the 49 pixels that exist it takes about 1 us.
+// `block` of `grid`: the calling CTA among those that walk this GEMM's tiles.
 template <int kEpi, bool kSplit>
-__global__ void __launch_bounds__(kGemmThreads, 1)
-igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUtensorMap map_a,
-             const __grid_constant__ CUtensorMap map_b)
+__device__ __forceinline__ void igemm_body(const IgemmParams &p, const CUtensorMap &map_a, const CUtensorMap &map_b, const int block, const int grid)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bars[2 * kMaxStages + 9];
@@ -79,10 +78,10 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     // Every CTA walks the reduction from another starting point (the integer sums do not depend on the order): in step, all
     // CTAs of a column tile would ask the same L2 slices for the same weights at the same time.
     // A cluster divides the iterations instead.
-    const int rank = kSplit ? (int)(blockIdx.x % (unsigned)p.split) : 0;
-    const int k_first = kSplit ? k_iters * rank / p.split : (int)(blockIdx.x % (unsigned)k_iters);
+    const int rank = kSplit ? (int)((unsigned)block % (unsigned)p.split) : 0;
+    const int k_first = kSplit ? k_iters * rank / p.split : (int)((unsigned)block % (unsigned)k_iters);
     const int k_count = kSplit ? k_iters * (rank + 1) / p.split - k_first : k_iters;
-    const int tile_first = kSplit ? (int)blockIdx.x / p.split : (int)blockIdx.x;   // (a cluster has one tile)
+    const int tile_first = kSplit ? block / p.split : block;   // (a cluster has one tile)
 
     // where a tile's loads start; of the first tile while the kernels in front still run
     struct Source {
@@ -151,7 +150,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
                 stage += kProducers;
                 while (stage >= p.num_stages) { stage -= p.num_stages; phase ^= 1u; }
             }
-            tile += gridDim.x;
+            tile += grid;
             if (tile < num_tiles) at = source_of(tile);
         }
         if (!ok && lane == 0) {
@@ -196,7 +195,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
         bool ok = true;
-        for (int tile = tile_first; tile < num_tiles && ok; tile += gridDim.x) {
+        for (int tile = tile_first; tile < num_tiles && ok; tile += grid) {
             if (!(ok = __all_sync(0xffffffffu, wait_bar(tempty_bar(acc), acc_phase ^ 1u, ctx)))) break;
             ptx::tc_fence_after();
             const uint32_t d_tmem = tmem_base + acc * buf_stride, d_other = nacc == 2 ? d_tmem + acc_stride : d_tmem;
@@ -280,7 +279,7 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
         const FwdShift sh = forward_shift(p, fs, shift);
         uint32_t acc_phase = 0, mx = 0, mx_masked = 0;
         bool ok = true;
-        for (int tile = tile_first + grp * gridDim.x; tile < num_tiles && ok; tile += p.ep_groups * gridDim.x) {
+        for (int tile = tile_first + grp * grid; tile < num_tiles && ok; tile += p.ep_groups * grid) {
             const int mt = tile / p.num_n_tiles, nt = tile % p.num_n_tiles;
             const int m = mt * kTileM + row;
             const bool valid = m < p.M && mine;
@@ -392,6 +391,25 @@ igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUte
     }
 }
 
+template <int kEpi, bool kSplit>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+igemm_kernel(const __grid_constant__ IgemmParams p, const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b)
+{
+    igemm_body<kEpi, kSplit>(p, map_a, map_b, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// The GEMMs of a strided error back-propagation's residue classes, which write disjoint pixels, in one launch: a class has a range of
+// CTAs.  Bound as igemm_kernel.  On branch streams of their own, with fork and join, the 48 -> 80 channel layer 37 x 29 at batch 5 called
+// by itself took 36.8 us (28.6 so), and at batch 1 the four GEMMs of 256 -> 512 channels 14 x 14 ended 12.6 us behind the kernel in
+// front (8.5 so); ResNet-20 step at batch 128 576 -> 567 us.
+template <bool kSplit>
+__global__ void __launch_bounds__(kGemmThreads, 1) igemm_classes_kernel(const __grid_constant__ IgemmClasses c)
+{
+    int k = 0;
+    while (k + 1 < c.num && (int)blockIdx.x >= c.first[k + 1]) ++k;
+    igemm_body<kEpiDgrad, kSplit>(c.p[k], c.map_a[k], c.map_b[k], (int)blockIdx.x - c.first[k], c.first[k + 1] - c.first[k]);
+}
+
 }  // namespace
 
 size_t igemm_smem_bytes(const IgemmParams &p)
@@ -410,6 +428,18 @@ cudaError_t launch_igemm(const IgemmParams &p, const CUtensorMap &map_a, const C
     const cudaError_t e = allow_smem((const void *)kernel, 226 * 1024, allowed[p.split > 1][p.epilogue == kEpiForward]);
     if (e != cudaSuccess) return e;
     return launch_chained_clusters(p.split, kernel, grid, kGemmThreads, smem, stream, p, map_a, map_b);
+}
+
+cudaError_t launch_igemm_classes(const IgemmClasses &c, cudaStream_t stream)
+{
+    size_t smem = 0;
+    for (int k = 0; k < c.num; ++k) smem = igemm_smem_bytes(c.p[k]) > smem ? igemm_smem_bytes(c.p[k]) : smem;
+    const int split = c.p[0].split;   // (of all classes: a launch has one cluster size)
+    const auto kernel = split > 1 ? igemm_classes_kernel<true> : igemm_classes_kernel<false>;
+    static std::atomic<unsigned long long> allowed[2];
+    const cudaError_t e = allow_smem((const void *)kernel, 226 * 1024, allowed[split > 1]);
+    if (e != cudaSuccess) return e;
+    return launch_chained_clusters(split, kernel, c.first[c.num], kGemmThreads, smem, stream, c);
 }
 
 }  // namespace eoq

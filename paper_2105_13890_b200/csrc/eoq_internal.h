@@ -111,7 +111,6 @@ struct ReduceHook {
 };
 
 constexpr int kSqTiles = 32768;
-constexpr int kClassBranches = 3;
 
 struct ProfRecord {
     int kind;
@@ -132,12 +131,6 @@ struct Handle {
     int num_records;
     ProfRecord *records;          // kMaxProfRecords entries, allocated on first eoq_profile_start
     int gemm_ctas;                // most CTAs a GEMM call of this handle may use (eoq_set_gemm_ctas; default: one per SM)
-    // Branch streams with their fork and join events: the per-class GEMMs of a strided error back-propagation write disjoint
-    // pixels and run side by side, each with its share of the CTAs (null streams, as on the path without a handle: everything
-    // stays on the caller's stream).  Under stream capture the events become graph edges.
-    cudaEvent_t fork_ev;
-    cudaStream_t class_branch[kClassBranches];
-    cudaEvent_t class_join[kClassBranches];
 };
 constexpr int kMaxProfRecords = 8192;
 int static_path_last_cuda_error();  // last cudaError_t of eoq_conv_dgrad_static (eoq_static.cu)
@@ -246,6 +239,16 @@ cudaError_t launch_igemm_rows(const IgemmParams &p, const RowsPlan &pl, const CU
 size_t igemm_smem_bytes(const IgemmParams &p);
 cudaError_t launch_igemm(const IgemmParams &p, const CUtensorMap &map_a, const CUtensorMap &map_b, int grid,
                          cudaStream_t stream);
+
+// Several GEMMs of one error back-propagation in a launch: class k has the CTAs [first[k], first[k + 1]).  All have the same split.
+constexpr int kMaxClasses = 4;
+struct IgemmClasses {
+    CUtensorMap map_a[kMaxClasses], map_b[kMaxClasses];
+    IgemmParams p[kMaxClasses];
+    int num;
+    int first[kMaxClasses + 1];
+};
+cudaError_t launch_igemm_classes(const IgemmClasses &c, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------------------------
 // Weight-gradient kernel: D[(tap, ic), oc] = sum over pixels of x1[pixel + tap, ic] * e3[pixel, oc]

@@ -91,11 +91,6 @@ extern "C" int eoq_conv_dgrad_static(const eoq_conv_desc_t *desc, const int8_t *
     h.num_records = 0;
     h.records = nullptr;
     h.gemm_ctas = pd.sm_count;
-    h.fork_ev = nullptr;
-    for (int k = 0; k < kClassBranches; ++k) {
-        h.class_branch[k] = nullptr;
-        h.class_join[k] = nullptr;
-    }
     st = eoq_conv_dgrad(reinterpret_cast<eoq_handle_t>(&h), desc, e3, e3_exp, w, e4, e4_exp, sum_e4, nullptr,
                         pd.scratch + kStaticHeaderBytes, kStaticScratchBytes, stream);
     if (st != EOQ_OK) {

@@ -1,0 +1,41 @@
+"""Strided error back-propagation: the residue classes of the input pixels share launches of up to four GEMMs."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2105_13890_b200 import eoq, synth
+import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+
+GEOMETRIES = [
+    oracle.ConvDesc(1, 14, 14, 256, 512, 3, 3, 2, 1),    # one split for four classes of 1 to 4 taps
+    oracle.ConvDesc(2, 17, 13, 64, 128, 3, 3, 2, 1),     # classes of other sizes
+    oracle.ConvDesc(9, 30, 30, 32, 64, 3, 3, 2, 1),      # many tiles to a CTA under a cap
+    oracle.ConvDesc(3, 11, 11, 32, 96, 5, 5, 3, 2),      # nine classes in three launches
+    oracle.ConvDesc(2, 13, 9, 48, 80, 7, 7, 4, 3),       # sixteen classes, transposed weights
+    oracle.ConvDesc(2, 1, 9, 32, 32, 3, 3, 2, 1),        # no odd rows
+    oracle.ConvDesc(2, 8, 8, 32, 64, 1, 1, 3, 0),        # eight classes without a tap
+    oracle.ConvDesc(2, 9, 9, 32, 64, 2, 2, 3, 0),        # some without
+]
+
+
+@pytest.mark.parametrize("cap", [0, 1, 7])
+@pytest.mark.parametrize("d", GEOMETRIES, ids=lambda d: "n%d_%dx%d_%d_%d_k%ds%d" % (d.n, d.h, d.w, d.c_in, d.c_out, d.kh, d.stride))
+def test_strided_classes(d, cap):
+    """With and without the dump of the sums, whatever share of the CTAs a class gets."""
+    gd, h = G.gdesc(d), eoq.eoq_create(0)
+    if cap:
+        eoq.eoq_set_gemm_ctas(h, cap)
+    e3, w = synth.normal_codes((d.n, d.ho, d.wo, d.c_out), 2730, d.h, std_codes=24), synth.normal_codes((d.c_out, d.kh, d.kw, d.c_in), 2731, d.w, std_codes=6)
+    acc = oracle.conv_dgrad_acc(d, e3, w)
+    want, p, _ = oracle.sq_int(acc, -9 - 7)
+    e3_d, w_d, exp, ws = G.dev(e3), G.dev(w), torch.tensor([-9], dtype=torch.int32, device="cuda:0"), G.workspace(gd, eoq.EOQ_PASS_DGRAD)
+    for dump in (None, G.empty(acc.shape, torch.int32)):
+        e4, e4_exp, total = G.empty(acc.shape, torch.int8), G.zeros(1, torch.int32), G.empty(1, torch.int64)
+        eoq.eoq_conv_dgrad(h, gd, e3_d, exp, w_d, e4, e4_exp, total, dump, ws)
+        assert eoq.eoq_last_status(h) == 0
+        assert np.array_equal(G.host(e4), want) and e4_exp.item() == p and total.item() == int(want.astype(np.int64).sum())
+        assert dump is None or np.array_equal(G.host(dump), acc)
+    eoq.eoq_destroy(h)
