@@ -189,7 +189,7 @@ EOQ_API int eoq_conv_dgrad_join_head(eoq_handle_t handle, const eoq_conv_desc_t 
  * device, a plugin loaded into a host application that forbids cudaMalloc after start-up, or a real-time loop
  * where an allocation's implicit synchronisation is not acceptable.  Such callers cannot use eoq_create (it
  * allocates the handle's device state) nor supply a workspace.  This entry point needs neither: every byte of
- * scratch -- reduction cells, transposed weights, sums -- sits in one static device array of
+ * scratch -- reduction cells, sums -- sits in one static device array of
  * EOQ_STATIC_SCRATCH_BYTES (+4 KiB of cells) that is part of the library image, so each GPU that loads the
  * library carries it until the process exits.  It calls no cudaMalloc, cudaFree or allocating library routine.
  *
@@ -438,7 +438,7 @@ EOQ_API int eoq_last_status(eoq_handle_t handle, void *stream, unsigned *bits);
 #define EOQ_PROF_IGEMM_DGRAD 1   /* the dgrad implicit-GEMM kernel, one launch per group */
 #define EOQ_PROF_WGRAD 2         /* the weight-gradient GEMM kernel */
 #define EOQ_PROF_ERR_HEAD 3      /* eoq_err_prescale (one kernel; two for tensors beyond the one-kernel capacity) */
-#define EOQ_PROF_DGRAD_AUX 4     /* Q_e phase 2; weight transpose (only layers with fewer than 32 output channels) */
+#define EOQ_PROF_DGRAD_AUX 4     /* Q_e phase 2 */
 #define EOQ_PROF_WGRAD_AUX 5     /* slice sum + b1 term + Q_g behind the weight-gradient GEMM */
 #define EOQ_PROF_FWD_AUX 6       /* b1 weight table, weight row padding (eoq_weight_prep, or per call without it) */
 #define EOQ_PROF_OTHER 7         /* eoq_quantize, eoq_bn_fwd, eoq_bn_bwd */

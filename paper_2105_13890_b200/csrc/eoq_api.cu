@@ -537,8 +537,7 @@ bool plan_stride1(IgemmParams &p, PatchPlan &pl, int n_img, int c_src, int hq, i
     g.b_mn = p.b_mn;
     plan_igemm(g, c_src, p.ntaps, sm_count);
     plan_few_tiles(g, ctas);
-    // (with fewer than 32 channels per chunk the im2col kernel reads a transposed copy of the weights: a kernel more)
-    return few_igemm_time(g) + (p.b_mn && c_src % 32 ? 3.0 : 0.0) > 0.97 * time;
+    return few_igemm_time(g) > 0.97 * time;
 }
 
 // Plan of the input-row forward kernel for a filter-row layer (see use_row_window); false: the im2col kernel takes it.
@@ -1039,7 +1038,7 @@ extern "C" int eoq_workspace_size(const eoq_conv_desc_t *desc, int pass, size_t 
             *bytes = round256((size_t)bc.nrc * bc.ncc * desc->c_out * sizeof(int32_t)) +
                      (use_row_window(*desc, g.wo) ? round256((size_t)desc->c_out * desc->kh * 8 * desc->c_in) : 0);
             return EOQ_OK;
-        // transposed weights + sums.  The room is that of int32 sums; as 16-bit words they fill half of it.  The size is part of
+        // a copy of the weights (no kernel makes one any more) + sums.  The room is that of int32 sums; as 16-bit words they fill half of it.  The size is part of
         // the interface: callers keep buffers of it, and the allocation-free entry point accepts geometries by it.
         case EOQ_PASS_DGRAD:
             *bytes = round256(g.w_elems) + round256(g.in_elems * sizeof(int32_t));
@@ -1356,7 +1355,6 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     const eoq_conv_desc_t &d = *desc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
-    int8_t *wt = reinterpret_cast<int8_t *>(workspace);
     // the GEMMs leave their sums as 16-bit words in the workspace, or as int32 where the caller wants them
     uint16_t *const sums16 = acc_dump ? nullptr : reinterpret_cast<uint16_t *>(static_cast<char *>(workspace) + round256(g.w_elems));
     auto code_sums = [&](cudaStream_t st) {   // Q_e over the whole tensor, behind the GEMMs
@@ -1418,17 +1416,6 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             return join_after(e, s);
         }
     }
-    // With at least 32 output channels per K chunk the per-class GEMMs read the weights in place as MN-major atoms
-    // (as the patch kernel does); narrower layers read a K-major transposed copy [c_in][tap][c_out].
-    const bool weights_in_place = d.c_out % 32 == 0;
-    if (!weights_in_place) {
-        {
-            ProfScope prof(h, EOQ_PROF_DGRAD_AUX, s);
-            e = launch_weight_transpose(w, wt, d.c_out, g.taps, d.c_in, h->sm_count, s);
-        }
-        if (e != cudaSuccess) return record(h, e);
-        count_launches(h, 1);
-    }
     // a class no tap reaches (e.g. the odd pixels of a strided 1x1 filter) keeps zero sums: clear first
     bool any_empty = false;
     for (int r = 0; r < d.stride; ++r) {
@@ -1456,8 +1443,7 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
         for (int k = 0; k < cl.num; ++k) {
             const IgemmParams &p = cl.p[k];
             if (!make_im2col_map(&cl.map_a[k], e3, d.n, g.ho, g.wo, d.c_out, dw_of[k], dh_of[k], p.wq, p.hq, 1, p.kc, p.a_rows) ||
-                !(weights_in_place ? make_weight_map(&cl.map_b[k], w, d.c_out, g.taps, d.c_in, p.b_row, p.kc)
-                                   : make_weight_map(&cl.map_b[k], wt, d.c_in, g.taps, d.c_out, p.kc, p.tile_n)))
+                !make_weight_map(&cl.map_b[k], w, d.c_out, g.taps, d.c_in, p.b_row, p.kc))
                 return EOQ_ERR_UNSUPPORTED;
         }
         count_launches(h, 1);
@@ -1501,7 +1487,7 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             p.N = d.c_in;
             p.hq = hq;
             p.wq = wq;
-            p.b_mn = weights_in_place ? 1 : 0;
+            p.b_mn = 1;   // (the weights stay where they are, as for the patch kernel)
             plan_igemm(p, d.c_out, nh * nw, h->sm_count);
             p.src_stride = 1;
             p.src_stride_w = 1;
@@ -1891,7 +1877,6 @@ extern "C" int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *des
         const int hq = (d.h + d.stride - 1) / d.stride, wq = (d.w + d.stride - 1) / d.stride;
         p.M = d.n * hq * wq;
         p.N = d.c_in;
-        p.b_mn = d.c_out % 32 == 0;
         plan_igemm(p, d.c_out, ((d.kh + d.stride - 1) / d.stride) * ((d.kw + d.stride - 1) / d.stride), h->sm_count);
         if (d.stride == 1) plan_few_tiles(p, h->gemm_ctas);
         snprintf(buf, buf_bytes, "kernel=igemm classes=%d tile_n=%d m_tiles=%d n_tiles=%d kc=%d split=%d", d.stride * d.stride, p.tile_n,

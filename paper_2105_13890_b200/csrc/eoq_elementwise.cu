@@ -1048,20 +1048,6 @@ __global__ void transpose_bytes_kernel(const int8_t *__restrict__ src, int8_t *_
     }
 }
 
-// w[oc][tap][ic] -> wt[ic][tap][oc]
-__global__ void weight_transpose_kernel(const int8_t *__restrict__ w, int8_t *__restrict__ wt, int c_out, int taps,
-                                        int c_in)
-{
-    ptx::grid_dep_wait_launch_small();
-    const size_t total = (size_t)c_out * taps * c_in;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int oc = (int)(i % c_out);
-        const int tap = (int)((i / c_out) % taps);
-        const int ic = (int)(i / ((size_t)c_out * taps));
-        wt[i] = w[((size_t)oc * taps + tap) * c_in + ic];
-    }
-}
-
 // ------------------------------------------------------------------ b1 support
 
 // table[class][oc] = sum over the taps valid for the class, and over ic, of w[oc][tap][ic]  (the forward
@@ -1379,13 +1365,6 @@ cudaError_t launch_layout_convert(const int8_t *src, int8_t *dst, int n, int c, 
     const int rows = to_nhwc ? c : h * w, cols = to_nhwc ? h * w : c;
     dim3 grid((cols + 31) / 32, (rows + 31) / 32, n), block(32, 8);
     transpose_bytes_kernel<<<grid, block, 0, s>>>(src, dst, rows, cols);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_weight_transpose(const int8_t *w, int8_t *wt, int c_out, int taps, int c_in, int sm_count, cudaStream_t s)
-{
-    const int blocks = grid_for((size_t)c_out * taps * c_in, sm_count, 16);
-    launch_chained(weight_transpose_kernel, blocks, kThreads, 0, s, w, wt, c_out, taps, c_in);
     return cudaGetLastError();
 }
 

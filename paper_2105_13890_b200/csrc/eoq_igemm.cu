@@ -37,6 +37,11 @@ __device__ __forceinline__ void igemm_body(const IgemmParams &p, const CUtensorM
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t a_sub = (uint32_t)kTileM * p.kc, b_sub = (uint32_t)p.tile_n * p.kc;
     const uint32_t stage_bytes = (uint32_t)p.subs_per_stage * (a_sub + b_sub);
+    // Weights read MN-major: a sub-tile is atoms of kc rows of b_row bytes, `b_atom` bytes apart along the columns, and the next
+    // sub-tile lies `b_next` bytes further.  With 16 rows an MMA spans two sub-tiles, so those of a stage share their atoms (rows of
+    // one sub-tile behind those of the other) and the K groups of an MMA keep one distance.
+    const bool b_shared = p.b_mn && p.kc == 16;
+    const uint32_t b_atom = (uint32_t)(b_shared ? p.subs_per_stage * 16 : p.kc) * p.b_row, b_next = b_shared ? 16u * p.b_row : b_sub;
     const uint32_t bar0 = ptx::smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (kMaxStages + s); };
@@ -135,10 +140,11 @@ __device__ __forceinline__ void igemm_body(const IgemmParams &p, const CUtensorM
                         ptx::tma_load_im2col_4d(a_dst + j * a_sub, &map_a, full_bar(stage), chunk * p.kc, at.cw, at.ch, at.img,
                                                 (uint16_t)p.tap_dw[tap], (uint16_t)p.tap_dh[tap]);
                     } else if (p.b_mn) {
-                        // weights in place, [reduction rows][tap][columns]: tile_n / b_row atoms of [kc rows][b_row bytes]
+                        // weights in place, [reduction rows][tap][columns]: tile_n / b_row atoms of [kc rows][b_row bytes]; zeros
+                        // for a padding sub-tile, as below
                         const int a = i - subs - j * atoms;
-                        ptx::tma_load_3d(b_dst + j * b_sub + a * (uint32_t)p.kc * p.b_row, &map_b, full_bar(stage),
-                                         at.nt * p.tile_n + a * p.b_row, (int)p.tap_b[tap], chunk * p.kc);
+                        ptx::tma_load_3d(b_dst + j * b_next + a * b_atom, &map_b, full_bar(stage), at.nt * p.tile_n + a * p.b_row,
+                                         s < p.real_sub ? (int)p.tap_b[tap] : 0x7fff, chunk * p.kc);
                     } else {
                         // tap coordinate p.ntaps lies outside the weight tensor: the padding sub-tile is zero-filled
                         ptx::tma_load_3d(b_dst + j * b_sub, &map_b, full_bar(stage), chunk * p.kc,
@@ -173,21 +179,19 @@ __device__ __forceinline__ void igemm_body(const IgemmParams &p, const CUtensorM
         // (two taps): the second half of K sits one sub-tile further (leading offset), 8-row groups 128 B apart.
         const bool wide = p.kc >= 32;
         const uint32_t hi = wide ? smem_desc_hi(8u * p.kc, layout_type_for(p.kc)) : smem_desc_hi(128, 0);
-        const uint32_t a_sub16 = a_sub >> 4, b_sub16 = b_sub >> 4;
+        const uint32_t a_sub16 = a_sub >> 4, b_sub16 = b_next >> 4;
         const uint32_t a_lead = wide ? 0u : (a_sub16 << 16);
         uint32_t b_lead = wide ? 0u : (b_sub16 << 16);
-        // B read MN-major (only with kc >= 32): atoms kc * b_row apart along the columns (leading offset), 8-row
-        // groups 8 * b_row apart (stride offset); 16-byte rows carry no swizzle and the two offsets swap roles; a
-        // 32-deep K step is 32 rows of an atom
+        // B read MN-major: atoms b_atom apart along the columns (leading offset), 8-row groups 8 * b_row apart (stride
+        // offset); 16-byte rows carry no swizzle and the two offsets swap roles; a 32-deep K step is 32 rows of an atom
         uint32_t b_hi = hi, b_k16 = 2u;
         if (p.b_mn) {
-            const uint32_t atom = (uint32_t)p.kc * p.b_row;
             if (p.b_row == 16) {
-                b_hi = smem_desc_hi(atom, 0);
+                b_hi = smem_desc_hi(b_atom, 0);
                 b_lead = (128u >> 4) << 16;
             } else {
                 b_hi = smem_desc_hi(8u * p.b_row, layout_type_for(p.b_row));
-                b_lead = ((atom >> 4) & 0x3FFFu) << 16;
+                b_lead = ((b_atom >> 4) & 0x3FFFu) << 16;
             }
             b_k16 = (32u * p.b_row) >> 4;
         }

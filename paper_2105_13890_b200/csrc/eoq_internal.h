@@ -388,7 +388,6 @@ cudaError_t launch_update_wide(const UpdateTensor *t, int num, int32_t lr_mant, 
                                uint64_t seed, uint64_t step, unsigned long long *step_dev, DeviceState *dev, cudaStream_t s);
 cudaError_t launch_layout_convert(const int8_t *src, int8_t *dst, int n, int c, int h, int w, int to_nhwc,
                                   cudaStream_t s);
-cudaError_t launch_weight_transpose(const int8_t *w, int8_t *wt, int c_out, int taps, int c_in, int sm_count, cudaStream_t s);
 // b1 support: class tables of weight sums (forward) and of error sums (weight gradient)
 struct BorderClasses {
     int nlo_h, nhi_h, nrc, nlo_w, nhi_w, ncc;

@@ -1,5 +1,5 @@
 // eoq_conv_dgrad_static: error back-propagation for callers that cannot allocate device memory.
-// All scratch (the reduction cells, the transposed weights, the sums) lives in one file-scope device
+// All scratch (the reduction cells, the sums) lives in one file-scope device
 // array that every GPU loading the library carries until the process exits.
 #include <cuda_runtime.h>
 #include <stdint.h>

@@ -1,4 +1,5 @@
-"""Strided error back-propagation: the residue classes of the input pixels share launches of up to four GEMMs."""
+"""Error back-propagation by the im2col kernel: the residue classes of a strided layer share launches of up to four GEMMs, and the
+weights are read where they are whatever the number of channels."""
 import numpy as np
 import pytest
 import torch
@@ -10,11 +11,19 @@ import gpu_util as G
 pytestmark = pytest.mark.gpu
 
 GEOMETRIES = [
+    # reductions over odd multiples of 16 channels, whose MMAs span two sub-tiles, padded ones among them; column atoms of 16 to 128 bytes
+    oracle.ConvDesc(3, 9, 10, 16, 16, 1, 1, 1, 0),
+    oracle.ConvDesc(2, 9, 10, 48, 48, 1, 1, 1, 0),
+    oracle.ConvDesc(2, 12, 9, 64, 80, 1, 1, 1, 0),
+    oracle.ConvDesc(40, 14, 14, 256, 112, 1, 1, 1, 0),
+    oracle.ConvDesc(5, 37, 29, 48, 80, 3, 3, 2, 1),
+    oracle.ConvDesc(2, 15, 16, 160, 48, 3, 3, 2, 1),
+    oracle.ConvDesc(3, 7, 7, 128, 144, 3, 3, 1, 1),
     oracle.ConvDesc(1, 14, 14, 256, 512, 3, 3, 2, 1),    # one split for four classes of 1 to 4 taps
     oracle.ConvDesc(2, 17, 13, 64, 128, 3, 3, 2, 1),     # classes of other sizes
     oracle.ConvDesc(9, 30, 30, 32, 64, 3, 3, 2, 1),      # many tiles to a CTA under a cap
     oracle.ConvDesc(3, 11, 11, 32, 96, 5, 5, 3, 2),      # nine classes in three launches
-    oracle.ConvDesc(2, 13, 9, 48, 80, 7, 7, 4, 3),       # sixteen classes, transposed weights
+    oracle.ConvDesc(2, 13, 9, 48, 80, 7, 7, 4, 3),       # sixteen classes, 16 channels to a chunk
     oracle.ConvDesc(2, 1, 9, 32, 32, 3, 3, 2, 1),        # no odd rows
     oracle.ConvDesc(2, 8, 8, 32, 64, 1, 1, 3, 0),        # eight classes without a tap
     oracle.ConvDesc(2, 9, 9, 32, 64, 2, 2, 3, 0),        # some without
