@@ -1569,7 +1569,6 @@ extern "C" int eoq_conv_dgrad_head(eoq_handle_t handle, const eoq_conv_desc_t *d
 struct WgradSpace {
     long long *tap_sums;
     unsigned long long *max_cell;
-    size_t zero_bytes;            // tap sums and maximum cell: cleared by the GEMM kernel
     long long *acc;
     size_t acc_bytes;
     int32_t *parts;
@@ -1581,10 +1580,9 @@ static WgradSpace wgrad_space(const eoq_conv_desc_t &d, const Geometry &g, void 
     const size_t tap_bytes = kTapReplicas * round256((size_t)d.c_out * g.taps * sizeof(long long));   // (also 16-byte aligned cells)
     w.tap_sums = reinterpret_cast<long long *>(ws);
     w.max_cell = reinterpret_cast<unsigned long long *>(ws + tap_bytes);
-    w.zero_bytes = tap_bytes + 256;
-    w.acc = reinterpret_cast<long long *>(ws + w.zero_bytes);
+    w.acc = reinterpret_cast<long long *>(ws + tap_bytes + 256);
     w.acc_bytes = round256(g.w_elems * sizeof(long long));
-    w.parts = reinterpret_cast<int32_t *>(ws + w.zero_bytes + w.acc_bytes);
+    w.parts = reinterpret_cast<int32_t *>(ws + tap_bytes + 256 + w.acc_bytes);
     return w;
 }
 
@@ -1614,23 +1612,19 @@ static FinishItem finish_item(const eoq_conv_desc_t &d, const Geometry &g, const
     return it;
 }
 
-// b1 error sums, sums and Q_g of up to kFinishChunk layers whose GEMMs are in front on the stream (beside: directly, and one layer).
-static int finish_items(Handle *h, const FinishItem *items, int num, bool beside, cudaStream_t s)
+// The b1 error sums of the batch (let_in: see launch_finish_taps).
+static int finish_taps(Handle *h, const FinishBatch &b, bool let_in, cudaStream_t s)
 {
-    if (num == 1 && !h->profiling && finish_is_small(items[0], h->hook)) {   // (a profile brackets the b1 sums as a kind of their own)
-        count_launches(h, 1);
-        return record(h, launch_finish_small(items[0], &h->dev->status, h->sm_count, beside, s));
-    }
-    FinishBatch b;
-    plan_finish(b, items, num, h->sm_count, h->hook);
-    if (b.tap_first[num] > 0) {
-        ProfScope prof(h, EOQ_PROF_WGRAD_TAPS, s);
-        count_launches(h, 1);
-        const cudaError_t e = launch_finish_taps(b, beside, s);
-        if (e != cudaSuccess) return record(h, e);
-    }
+    ProfScope prof(h, EOQ_PROF_WGRAD_TAPS, s);
+    count_launches(h, 1);
+    return record(h, launch_finish_taps(b, let_in, s));
+}
+
+// Sums and Q_g of the batch, whose GEMMs and b1 error sums are in front on the stream.
+static int finish_sums(Handle *h, const FinishBatch &b, cudaStream_t s)
+{
     ProfScope prof(h, EOQ_PROF_WGRAD_AUX, s);
-    count_launches(h, h->hook.fn ? 2 + num : 2);
+    count_launches(h, h->hook.fn ? 2 + b.num : 2);
     return record(h, launch_finish_sums(b, &h->dev->status, s, h->hook));
 }
 
@@ -1657,64 +1651,77 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     const bool use_b1 = b1_dev != nullptr || b1_c != 0;
     if (use_b1 && bc.nrc * bc.ncc > kMaxBorderClasses) return EOQ_ERR_UNSUPPORTED;
     const WgradSpace w = wgrad_space(d, g, workspace);
+    // A layer's b1 error sums go in front of its GEMM, which they let in and which runs beside them; a small layer is finished by one
+    // launch behind it, which forms them too and runs beside it up to there.
+    FinishItem item = finish_item(d, g, w, e3, e3_exp, b1_c, b1_dev, gq, g_exp, 0);
+    item.copy_out = reinterpret_cast<long long *>(acc_dump);
+    FinishBatch batch;
+    bool small = false, taps_first = false;
+    auto begin = [&](int num_parts, bool beside) -> int {   // beside: the GEMM's kernel can run beside its neighbours
+        if (num_parts_out) *num_parts_out = num_parts;
+        if (gemm_only) return EOQ_OK;
+        item.num_parts = num_parts;
+        small = !h->profiling && finish_is_small(item, h->hook);   // (a profile brackets the b1 sums as a kind of their own)
+        if (small) return EOQ_OK;
+        plan_finish(batch, &item, 1, h->sm_count, h->hook);
+        if (!use_b1) return EOQ_OK;
+        taps_first = beside;
+        return finish_taps(h, batch, beside, s);
+    };
     // behind the GEMM (whose kernel leaves sums as [oc][tap][ic], the layout of g)
-    auto finish = [&](int num_parts) -> int {
-        FinishItem it = finish_item(d, g, w, e3, e3_exp, b1_c, b1_dev, gq, g_exp, num_parts);
-        it.copy_out = reinterpret_cast<long long *>(acc_dump);
-        return finish_items(h, &it, 1, true, s);
+    auto finish = [&](cudaError_t e) -> int {
+        if (e != cudaSuccess || gemm_only) return record(h, e);
+        if (!small) return finish_sums(h, batch, s);
+        count_launches(h, 1);
+        return record(h, launch_finish_small(item, &h->dev->status, h->sm_count, use_b1, s));
     };
 
     WgradPatchPlan wp;
     if (plan_wgrad_patch(wp, d, g.ho, g.wo, h->gemm_ctas < kWgradTargetCtas ? h->gemm_ctas : kWgradTargetCtas)) {
         wp.partials = w.parts;
-        wp.zero = reinterpret_cast<int4 *>(w.tap_sums);
-        wp.zero_n16 = (unsigned)(w.zero_bytes / 16);
-        wp.launch_early = use_b1 && !gemm_only;
+        wp.zero = w.max_cell;
         wp.dev = h->dev;
         CUtensorMap map_x, map_e;
         if (!make_patch_map(&map_x, x, d.n, d.h, d.w, d.c_in, wp.kc, wp.pw, wp.r_rows + d.kh - 1) ||
             !make_patch_map(&map_e, e3, d.n, g.ho, g.wo, d.c_out, wp.tile_n, wp.pw, wp.r_rows))
             return EOQ_ERR_UNSUPPORTED;
+        if ((st = begin(wp.num_splits, true)) != EOQ_OK) return st;
+        wp.launch_early = small && use_b1;
+        wp.wait_late = taps_first;
         count_launches(h, 1);
-        if (num_parts_out) *num_parts_out = wp.num_splits;
         cudaError_t e;
         {
             ProfScope prof(h, EOQ_PROF_WGRAD, s);
             e = launch_wgrad_patch(wp, map_x, map_e, s);
         }
-        if (e != cudaSuccess || gemm_only) return record(h, e);
-        return finish(wp.num_splits);
+        return finish(e);
     }
 
     const int w_mem = d.w + 2 * d.x_wmargin;
     WgradRowsPlan rp;
     if (plan_wgrad_rows(rp, d, g, h->gemm_ctas)) {
         rp.partials = w.parts;
-        rp.zero = reinterpret_cast<int4 *>(w.tap_sums);
-        rp.zero_n16 = (unsigned)(w.zero_bytes / 16);
+        rp.zero = w.max_cell;
         rp.dev = h->dev;
         CUtensorMap map_x, map_e;
         if (!make_matrix_map(&map_e, e3, (size_t)d.n * g.ho * g.wo, d.c_out, rp.nc, g.wo) ||
             !make_row_window_map(&map_x, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, g.wo, g.ho, d.stride, d.pad, g.wo))
             return EOQ_ERR_UNSUPPORTED;
+        if ((st = begin(rp.num_splits, false)) != EOQ_OK) return st;
         count_launches(h, 1);
-        if (num_parts_out) *num_parts_out = rp.num_splits;
         cudaError_t e;
         {
             ProfScope prof(h, EOQ_PROF_WGRAD, s);
             e = launch_wgrad_rows(rp, map_x, map_e, s);
         }
-        if (e != cudaSuccess || gemm_only) return record(h, e);
-        return finish(rp.num_splits);
+        return finish(e);
     }
 
     WgradParams p;
     if (!plan_wgrad(p, d, g, h->gemm_ctas)) return EOQ_ERR_UNSUPPORTED;
     const bool row_window = p.row_window_kw != 0;
     p.partials = w.parts;
-    p.zero = reinterpret_cast<int4 *>(w.tap_sums);
-    p.zero_n16 = (unsigned)(w.zero_bytes / 16);
-    p.launch_early = use_b1 && !gemm_only;
+    p.zero = w.max_cell;
     p.dev = h->dev;
 
     cudaError_t e;
@@ -1725,14 +1732,15 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
                    : !make_im2col_map(&map_x, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, -d.pad, g.wo, g.ho, d.stride,
                                       p.kc, p.pixels_per_stage))
         return EOQ_ERR_UNSUPPORTED;
+    if ((st = begin(p.num_k_splits, true)) != EOQ_OK) return st;
+    p.launch_early = small && use_b1;
+    p.wait_late = taps_first;
     count_launches(h, 1);
     {
         ProfScope prof(h, EOQ_PROF_WGRAD, s);
         e = launch_wgrad(p, map_x, map_e, s);
     }
-    if (num_parts_out) *num_parts_out = p.num_k_splits;
-    if (e != cudaSuccess || gemm_only) return record(h, e);
-    return finish(p.num_k_splits);
+    return finish(e);
 }
 
 extern "C" int eoq_conv_wgrad(eoq_handle_t handle, const eoq_conv_desc_t *desc, const int8_t *e3,
@@ -1787,7 +1795,16 @@ extern "C" int eoq_wgrad_finish(eoq_handle_t handle, int num, const eoq_conv_des
             items[k] = finish_item(d, g, wgrad_space(d, g, workspace[base + k]), e3[base + k], e3_exp[base + k], 0, b1_c[base + k],
                                    gq[base + k], g_exp[base + k], num_parts[base + k]);
         }
-        const int st = finish_items(h, items, count, false, s);
+        if (count == 1 && !h->profiling && finish_is_small(items[0], h->hook)) {
+            count_launches(h, 1);
+            const int st = record(h, launch_finish_small(items[0], &h->dev->status, h->sm_count, false, s));
+            if (st != EOQ_OK) return st;
+            continue;
+        }
+        FinishBatch b;
+        plan_finish(b, items, count, h->sm_count, h->hook);
+        int st = b.tap_first[count] > 0 ? finish_taps(h, b, false, s) : EOQ_OK;
+        if (st == EOQ_OK) st = finish_sums(h, b, s);
         if (st != EOQ_OK) return st;
     }
     return EOQ_OK;

@@ -1,7 +1,7 @@
 // What follows the weight-gradient GEMM (arXiv 2105.13890, Sec. 3.2.1: g_w = Q_g(e3 * x1) with x1 = x0 + Q_b(b1)), for one
 // layer or for many layers in the same three launches: the b1 error sums (one pass over e3), the exact sums (split-K slices
 // plus the b1 term) reduced to their maximum, and Q_g.  Blocks find their layer by their index.
-// The cells these kernels add into (tap sums, maximum) are cleared by the GEMM kernel in front.
+// The maximum's cell is cleared by the GEMM kernel.
 #include "eoq_device.cuh"
 #include "eoq_internal.h"
 
@@ -10,8 +10,9 @@ namespace eoq {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kClassSlab = 128;   // channels one block of the error sums covers
-constexpr int kTapBytes = 32 * 1024;
+constexpr int kTapSlab = 32;      // channels one block of the error sums covers: a 32-byte sector of a pixel
+constexpr int kTapThreads = 512;
+constexpr int kTapMostCluster = 8;
 
 __device__ __forceinline__ int finish_item_of(const int *first, int num, int block)
 {
@@ -32,21 +33,19 @@ __device__ __forceinline__ bool finish_narrow(const FinishItem &it, int b1)
 }
 
 // ------------------------------------------------------------------ b1 error sums
-// tap_sums[oc][tap] += sum of e3[n,y,x,oc] over the pixels for which the tap falls inside the image (the weight gradient
+// tap_sums[oc][tap] = sum of e3[n,y,x,oc] over the pixels for which the tap falls inside the image (the weight gradient
 // adds b1 times this to every input channel).  Only border rows and columns ever fall outside a tap, so with T the sum over
 // all pixels, R_i and C_j those over the i-th border row and the j-th border column, and P_ij those over their crossings,
 //   tap sum = T - sum of R_i - sum of C_j + sum of P_ij   over the border rows and columns the tap does not take.
 // Every term is a plain sum over a regular set of pixels.  A block covers a range of rows and a slab of channels; a lane
 // keeps 16 channels (one 128-bit load per pixel, several in flight) in packed 16-bit halves (codes offset by 128, so that
-// no carry crosses; one instruction per code).  All warps sum T, then each takes its share of the border sets; the block
-// forms its tap sums in shared memory and adds each with one 64-bit atomic.
-// Bound by the latency of a few dependent rounds of loads, so behind a single layer's GEMM the blocks run beside it
-// (`beside`): the GEMM starts them once its own wait for the kernels in front, e3's among them, is over, they take e3 from the
-// L2, and wait for the GEMM's end only before their atomics, whose cells it clears.  A launch of many layers behind other work
-// waits first.  Backward of the 512-channel 7 x 7 layer at batch 64 60.5 -> 56.5 us, the single 16-channel layer 38.7 -> 36.1.
-// With a border class and a 32-bit addition per byte the four
-// stages of ResNet-18 at batch 64 took 228 us (now 117 us, beside the backward chain), the 512-channel 7 x 7 layer alone
-// 11.1 us (8.8), the single 16-channel layer 5.3 us behind a memset (5.4 without one).
+// no carry crosses; one instruction per code).  All warps sum T, then share out the border sets.
+// A slab's rows are dealt to the kTapReplicas copies of its cells, and a copy's to the blocks of a cluster, whose sums meet in
+// distributed shared memory: a copy is stored, not added to, so nothing clears the cells and no order against the GEMM is needed.
+// Bound by the latency of a few dependent rounds of loads.  A single layer's sums therefore go in front of its GEMM, which is let
+// in at once and runs beside them (conv_wgrad_impl).  With atomics into cells that the GEMM cleared they came behind it and ended
+// 3 to 8 us after it: backward of the 512-channel 7 x 7 layer at batch 64 60.6 -> 59.0 us, bottleneck block of ResNet-50 at batch 32
+// 270 -> 264, and fewer SMs taken from the error chain of a step (ResNet-18 at batch 13 621 -> 608).
 struct PixelSum {
     uint32_t even[4], odd[4];
     int count;
@@ -128,112 +127,169 @@ __device__ __forceinline__ bool tap_takes(int y, int k, int stride, int pad, int
     return src >= 0 && src < extent_in;
 }
 
-// Block `local` of the item's tap blocks.  sets: [1 + border rows][1 + border columns][kClassSlab]; index 0 = all rows / columns.
-template <int kT>   // threads of the block
-__device__ __forceinline__ void finish_taps_block(const FinishItem &it, int local, int32_t *sets)
+// Border rows / columns of the item that a filter row / column does not take, as bits.
+struct TapMasks {
+    unsigned long long rows[16], cols[16];
+};
+__device__ __forceinline__ void tap_masks(const FinishItem &it, int nr, int nc, TapMasks &m)
 {
-    __shared__ unsigned long long rows_out[16], cols_out[16];  // per filter row / column: the border rows / columns it does not take
     const eoq_conv_desc_t &d = it.d;
     const BorderClasses &bc = it.bc;
-    const int bx = local % it.tap_grid_x, by = local / it.tap_grid_x;
-    const int ho = it.ho, wo = it.wo, c_out = d.c_out;
-    const int nr = border_count(ho, bc.nlo_h, bc.nhi_h, bc.nrc), nc = border_count(wo, bc.nlo_w, bc.nhi_w, bc.ncc);
-    const int nsets = (1 + nr) * (1 + nc);
-    for (int i = threadIdx.x; i < nsets * kClassSlab; i += kT) sets[i] = 0;
     if (threadIdx.x < d.kh) {
-        unsigned long long m = 0;
+        unsigned long long out = 0;
         for (int i = 0; i < nr; ++i)
-            if (!tap_takes(border_at(i, ho, bc.nlo_h, bc.nhi_h, bc.nrc), threadIdx.x, d.stride, d.pad, d.h)) m |= 1ull << i;
-        rows_out[threadIdx.x] = m;
+            if (!tap_takes(border_at(i, it.ho, bc.nlo_h, bc.nhi_h, bc.nrc), threadIdx.x, d.stride, d.pad, d.h)) out |= 1ull << i;
+        m.rows[threadIdx.x] = out;
     } else if (threadIdx.x >= 32 && threadIdx.x < 32 + d.kw) {
-        unsigned long long m = 0;
+        unsigned long long out = 0;
         for (int i = 0; i < nc; ++i)
-            if (!tap_takes(border_at(i, wo, bc.nlo_w, bc.nhi_w, bc.ncc), threadIdx.x - 32, d.stride, d.pad, d.w)) m |= 1ull << i;
-        cols_out[threadIdx.x - 32] = m;
-    }
-    __syncthreads();
-    const int slab_ch = min(kClassSlab, c_out - by * kClassSlab);  // channels of this slab (multiple of 16)
-    const int lanes_per_pix = slab_ch / 16, pix_per_step = 32 / lanes_per_pix;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane % lanes_per_pix, slot = lane / lanes_per_pix;
-    const int r_begin = bx * it.rows_per_block, r_end = min(d.n * ho, r_begin + it.rows_per_block);
-    const int8_t *base = it.e3 + by * kClassSlab + sub * 16;
-    const int4 zero = make_int4(0, 0, 0, 0);
-    if (slot < pix_per_step) {
-        PixelSum acc;
-        acc.clear();
-        {   // T
-            constexpr int kUnroll = 8;
-            const size_t p_end = (size_t)r_end * wo;
-            const int step = (kT / 32) * pix_per_step;
-            for (size_t p0 = (size_t)r_begin * wo + warp * pix_per_step; p0 < p_end; p0 += kUnroll * step) {   // the same in all lanes
-                int4 v[kUnroll];
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    const size_t p = p0 + slot + u * step;
-                    v[u] = p < p_end ? __ldcg(reinterpret_cast<const int4 *>(base + p * c_out)) : zero;
-                }
-                acc.add_group(v, sets + sub * 16, lanes_per_pix);
-            }
-            if (acc.count) acc.flush(sets + sub * 16, lanes_per_pix);
-        }
-        for (int set = 1 + warp; set < nsets; set += kT / 32) {
-            constexpr int kUnroll = 4;
-            const int i = set / (1 + nc), j = set - i * (1 + nc);
-            int32_t *dst = sets + set * kClassSlab + sub * 16;
-            // rows first + q * row_step of the block's range, columns x0 .. x0 + cols - 1
-            int first = r_begin, row_step = 1, x0 = 0, cols = wo;
-            if (i > 0) {
-                const int y = border_at(i - 1, ho, bc.nlo_h, bc.nhi_h, bc.nrc);
-                row_step = ho;
-                first = r_begin + (y - r_begin % ho + ho) % ho;
-            }
-            if (j > 0) {
-                x0 = border_at(j - 1, wo, bc.nlo_w, bc.nhi_w, bc.ncc);
-                cols = 1;
-            }
-            const int rows = first < r_end ? (r_end - first + row_step - 1) / row_step : 0;
-            const int pixels = rows * cols;
-            for (int q0 = 0; q0 < pixels; q0 += kUnroll * pix_per_step) {
-                int4 v[kUnroll];
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    const int q = q0 + slot + u * pix_per_step, rq = cols == 1 ? q : q / wo;
-                    const int r = first + rq * row_step, x = x0 + (q - rq * cols);
-                    v[u] = q < pixels ? __ldcg(reinterpret_cast<const int4 *>(base + ((size_t)r * wo + x) * c_out)) : zero;
-                }
-                acc.add_group(v, dst, lanes_per_pix);
-            }
-            if (acc.count) acc.flush(dst, lanes_per_pix);
-        }
-    }
-    __syncthreads();
-    ptx::grid_dep_wait();   // (the GEMM kernel clears the cells)
-    // the blocks spread their atomics over the kTapReplicas copies of a cell
-    long long *tap_sums = it.tap_sums + bx % kTapReplicas;
-    const int taps = d.kh * d.kw;
-    for (int i = threadIdx.x; i < taps * slab_ch; i += kT) {   // consecutive threads: neighbouring cells of [oc][tap]
-        const int c = i / taps, tap = i - c * taps, kh = tap / d.kw, kw = tap - kh * d.kw;
-        const unsigned long long rm = rows_out[kh], cm = cols_out[kw];
-        const int32_t *cell = sets + c;
-        auto over_columns = [&](const int32_t *row) {
-            int v = row[0];
-            for (unsigned long long m = cm; m; m &= m - 1) v -= row[__ffsll((long long)m) * kClassSlab];
-            return v;
-        };
-        int sum = over_columns(cell);
-        for (unsigned long long m = rm; m; m &= m - 1) sum -= over_columns(cell + __ffsll((long long)m) * (1 + nc) * kClassSlab);
-        if (sum)
-            atomicAdd(reinterpret_cast<unsigned long long *>(tap_sums + ((size_t)(by * kClassSlab + c) * taps + tap) * kTapReplicas),
-                      (unsigned long long)(long long)sum);
+            if (!tap_takes(border_at(i, it.wo, bc.nlo_w, bc.nhi_w, bc.ncc), threadIdx.x - 32, d.stride, d.pad, d.w)) out |= 1ull << i;
+        m.cols[threadIdx.x - 32] = out;
     }
 }
 
-__global__ void __launch_bounds__(kThreads) finish_taps_kernel(const __grid_constant__ FinishBatch b, int beside)
+// Rows [r_begin, r_end) of a slab into sets[1 + border rows][1 + border columns][kTapSlab]; index 0 = all rows / columns.
+template <int kT>   // threads of the block
+__device__ __forceinline__ void tap_sets(const FinishItem &it, int slab, int slab_ch, int r_begin, int r_end, int nr, int nc, int32_t *sets)
 {
-    if (!beside) ptx::grid_dep_wait();
-    extern __shared__ int32_t sets[];
+    const eoq_conv_desc_t &d = it.d;
+    const BorderClasses &bc = it.bc;
+    const int ho = it.ho, wo = it.wo, c_out = d.c_out, nsets = (1 + nr) * (1 + nc);
+    for (int i = threadIdx.x; i < nsets * kTapSlab; i += kT) sets[i] = 0;
+    __syncthreads();
+    const int lanes_per_pix = slab_ch / 16, pix_per_step = 32 / lanes_per_pix;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lane_ch = (lane % lanes_per_pix) * 16, slot = lane / lanes_per_pix;
+    const int8_t *base = it.e3 + slab * kTapSlab + lane_ch;
+    const int4 zero = make_int4(0, 0, 0, 0);
+    PixelSum acc;
+    acc.clear();
+    {   // T
+        constexpr int kUnroll = 8;
+        const size_t p_end = (size_t)r_end * wo;
+        const int step = (kT / 32) * pix_per_step;
+        for (size_t p0 = (size_t)r_begin * wo + warp * pix_per_step; p0 < p_end; p0 += kUnroll * step) {   // the same in all lanes
+            int4 v[kUnroll];
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const size_t p = p0 + slot + u * step;
+                v[u] = p < p_end ? __ldcg(reinterpret_cast<const int4 *>(base + p * c_out)) : zero;
+            }
+            acc.add_group(v, sets + lane_ch, lanes_per_pix);
+        }
+        if (acc.count) acc.flush(sets + lane_ch, lanes_per_pix);
+    }
+    // the border sets, each by as many warps as there are for one
+    const int share = max(1, (kT / 32) / max(1, nsets - 1));
+    for (int turn = warp; turn < (nsets - 1) * share; turn += kT / 32) {
+        constexpr int kUnroll = 4;
+        const int set = 1 + turn / share, part = turn % share;
+        const int i = set / (1 + nc), j = set - i * (1 + nc);
+        int32_t *dst = sets + set * kTapSlab + lane_ch;
+        // rows first + q * row_step of the range, columns x0 .. x0 + cols - 1
+        int first = r_begin, row_step = 1, x0 = 0, cols = wo;
+        if (i > 0) {
+            const int y = border_at(i - 1, ho, bc.nlo_h, bc.nhi_h, bc.nrc);
+            row_step = ho;
+            first = r_begin + (y - r_begin % ho + ho) % ho;
+        }
+        if (j > 0) {
+            x0 = border_at(j - 1, wo, bc.nlo_w, bc.nhi_w, bc.ncc);
+            cols = 1;
+        }
+        const int rows = first < r_end ? (r_end - first + row_step - 1) / row_step : 0;
+        const int pixels = rows * cols, step = share * pix_per_step;
+        for (int q0 = part * pix_per_step; q0 < pixels; q0 += kUnroll * step) {
+            int4 v[kUnroll];
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const int q = q0 + slot + u * step, rq = cols == 1 ? q : q / wo;
+                const int r = first + rq * row_step, x = x0 + (q - rq * cols);
+                v[u] = q < pixels ? __ldcg(reinterpret_cast<const int4 *>(base + ((size_t)r * wo + x) * c_out)) : zero;
+            }
+            acc.add_group(v, dst, lanes_per_pix);
+        }
+        if (acc.count) acc.flush(dst, lanes_per_pix);
+    }
+    __syncthreads();
+}
+
+// Copy `copy` (of `copies`) of the slab's tap sums, over range copy * cluster + rank of its rows, by the calling block and its
+// cluster.  sets, loc: shared memory of tap_set_bytes and kMaxTaps * kTapSlab words (loc only in a cluster).
+template <int kT>
+__device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab, int copy, int copies, int cluster, int rank, int32_t *sets, int32_t *loc)
+{
+    __shared__ TapMasks masks;
+    const eoq_conv_desc_t &d = it.d;
+    const BorderClasses &bc = it.bc;
+    const int nr = border_count(it.ho, bc.nlo_h, bc.nhi_h, bc.nrc), nc = border_count(it.wo, bc.nlo_w, bc.nhi_w, bc.ncc);
+    tap_masks(it, nr, nc, masks);   // (published by the barriers of tap_sets)
+    const int slab_ch = min(kTapSlab, d.c_out - slab * kTapSlab);  // channels of this slab (16 or 32)
+    const int taps = d.kh * d.kw, items = taps * slab_ch;
+    const int rows = d.n * it.ho, ranges = copies * cluster, rows_here = (rows + ranges - 1) / ranges;
+    const int begin = min((long long)rows, (long long)(copy * cluster + rank) * rows_here), end = min((long long)rows, (long long)begin + rows_here);
+    constexpr int kMost = (kMaxTaps * kTapSlab + kT - 1) / kT;   // items of a thread
+    long long total[kMost] = {};
+    const int chunk = max(1, (1 << 23) / it.wo);   // keeps the int32 sets exact
+    for (int at = 0; at < rows_here; at += chunk) {
+        const int r0 = min(end, begin + at), r1 = min(end, r0 + min(chunk, rows_here - at));
+        tap_sets<kT>(it, slab, slab_ch, r0, r1, nr, nc, sets);
+        auto tap_sum = [&](int i) {
+            const int c = i / taps, tap = i - c * taps, kh = tap / d.kw, kw = tap - kh * d.kw;
+            const unsigned long long rm = masks.rows[kh], cm = masks.cols[kw];
+            const int32_t *cell = sets + c;
+            auto over_columns = [&](const int32_t *row) {
+                int v = row[0];
+                for (unsigned long long m = cm; m; m &= m - 1) v -= row[__ffsll((long long)m) * kTapSlab];
+                return v;
+            };
+            int sum = over_columns(cell);
+            for (unsigned long long m = rm; m; m &= m - 1) sum -= over_columns(cell + __ffsll((long long)m) * (1 + nc) * kTapSlab);
+            return sum;
+        };
+        if (cluster > 1) {
+            for (int i = threadIdx.x; i < items; i += kT) loc[i] = tap_sum(i);
+            ptx::cluster_sync();
+#pragma unroll
+            for (int k = 0; k < kMost; ++k) {
+                const int i = (k * cluster + rank) * kT + (int)threadIdx.x;
+                if (i < items)
+                    for (int q = 0; q < cluster; ++q) total[k] += ptx::ld_cluster_32(ptx::cluster_addr(ptx::smem_u32(loc + i), q));
+            }
+            ptx::cluster_sync();   // the peers are through with this block's sums
+        } else {
+#pragma unroll
+            for (int k = 0; k < kMost; ++k) {
+                const int i = k * kT + (int)threadIdx.x;
+                if (i < items) total[k] += tap_sum(i);
+            }
+            __syncthreads();
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kMost; ++k) {
+        const int i = (k * cluster + rank) * kT + (int)threadIdx.x;   // neighbouring cells of [oc][tap]
+        if (i >= items) continue;
+        long long *cell = it.tap_sums + ((size_t)slab * kTapSlab * taps + i) * kTapReplicas;
+        cell[copy] = total[k];
+        if (copy == 0)
+            for (int r = copies; r < kTapReplicas; ++r) cell[r] = 0;
+    }
+}
+
+__host__ __device__ inline int tap_slabs(const FinishItem &it) { return (it.d.c_out + kTapSlab - 1) / kTapSlab; }
+
+// kLetIn: the launch behind this one is the layer's GEMM (see conv_wgrad_impl)
+template <bool kLetIn>
+// (at most 64 registers: a block and a CTA of the GEMM share an SM)
+__global__ void __launch_bounds__(kTapThreads, 2) finish_taps_kernel(const __grid_constant__ FinishBatch b)
+{
+    ptx::grid_dep_wait();
+    if (kLetIn) ptx::grid_dep_launch();
+    extern __shared__ __align__(16) int32_t dyn[];
     const int k = finish_item_of(b.tap_first, b.num, (int)blockIdx.x);
-    if (b.item[k].use_b1) finish_taps_block<kThreads>(b.item[k], (int)blockIdx.x - b.tap_first[k], sets);
+    const int local = (int)blockIdx.x - b.tap_first[k], per_slab = b.item[k].tap_copies * b.tap_cluster, part = local % per_slab;
+    finish_taps_slab<kTapThreads>(b.item[k], local / per_slab, part / b.tap_cluster, b.item[k].tap_copies, b.tap_cluster, part % b.tap_cluster,
+                                  dyn + kMaxTaps * kTapSlab, dyn);
 }
 
 // ------------------------------------------------------------------ exact sums and their maximum
@@ -424,7 +480,7 @@ __device__ __forceinline__ long long finish_b1_term_fresh(const FinishItem &it, 
     return (long long)b1 * (lo.x + lo.y + hi.x + hi.y);
 }
 
-__global__ void __launch_bounds__(kSmallThreads) finish_small_kernel(const __grid_constant__ FinishItem it, unsigned *status, int beside)
+__global__ void __launch_bounds__(kSmallThreads + 160) finish_small_kernel(const __grid_constant__ FinishItem it, unsigned *status, int beside)
 {
     extern __shared__ __align__(16) int32_t dyn[];   // the tap kernel's sets, then this CTA's sums, four to a quad
     __shared__ long long part[kSmallThreads][4];
@@ -433,13 +489,9 @@ __global__ void __launch_bounds__(kSmallThreads) finish_small_kernel(const __gri
     if (!beside) ptx::grid_dep_wait();
     const int rank = (int)blockIdx.x;
     if (it.use_b1) {
-        for (int i = rank; i < it.tap_blocks; i += kSmallCtas) {
-            finish_taps_block<kSmallThreads>(it, i, dyn);
-            __syncthreads();
-        }
+        const int slabs = tap_slabs(it), copies = slabs <= kSmallCtas / 4 ? 4 : (slabs <= kSmallCtas / 2 ? 2 : 1);
+        for (int i = rank; i < slabs * copies; i += kSmallCtas) finish_taps_slab<kSmallThreads>(it, i / copies, i % copies, copies, 1, 0, dyn, nullptr);
     }
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
     ptx::cluster_wait();
     if (it.use_b1) {
         __threadfence();
@@ -447,57 +499,57 @@ __global__ void __launch_bounds__(kSmallThreads) finish_small_kernel(const __gri
     }
     long long *sums = reinterpret_cast<long long *>(dyn);
     const int groups = it.groups, bw = kSmallThreads / groups, tx = threadIdx.x % bw, ty = threadIdx.x / bw;
-    const uint32_t quads = (uint32_t)(it.n / 4), mine = (quads + kSmallCtas - 1) / kSmallCtas;   // quads of a CTA
-    const uint32_t first = rank * mine, end = min(quads, first + mine);
-    const int b1 = it.use_b1 ? finish_b1(it) : 0;
+    const uint32_t quads = (uint32_t)(it.n / 4), mine = (quads + kSmallCtas - 1) / kSmallCtas;   // quads of a CTA: at most bw
+    const uint32_t first = rank * mine, end = min(quads, first + mine), q = first + tx;
+    const bool in = q < end;
+    // the b1 term of the thread's quad is at hand when the GEMM ends
+    const long long term = it.use_b1 && ty == 0 && in ? finish_b1_term_fresh(it, finish_b1(it), q) : 0;
+    __syncthreads();   // (the sums go where the tap sums' sets were)
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
     unsigned long long mx = 0;
-    for (uint32_t base = first; base < end; base += bw) {
-        const uint32_t q = base + tx;
-        const bool in = q < end;
-        long long v[4] = {0, 0, 0, 0};
-        if (in) {
-            const int4 *p = reinterpret_cast<const int4 *>(it.parts) + q;
-            int s = ty;
-            for (; s + 7 * groups < it.num_parts; s += 8 * groups) {
-                int4 a[8];
+    long long v[4] = {0, 0, 0, 0};
+    if (in) {
+        const int4 *p = reinterpret_cast<const int4 *>(it.parts) + q;
+        int s = ty;
+        for (; s + 7 * groups < it.num_parts; s += 8 * groups) {
+            int4 a[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) a[u] = __ldg(p + (size_t)(s + u * groups) * quads);
+            for (int u = 0; u < 8; ++u) a[u] = __ldg(p + (size_t)(s + u * groups) * quads);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    v[0] += a[u].x;
-                    v[1] += a[u].y;
-                    v[2] += a[u].z;
-                    v[3] += a[u].w;
-                }
-            }
-            for (; s < it.num_parts; s += groups) {
-                const int4 a = __ldg(p + (size_t)s * quads);
-                v[0] += a.x;
-                v[1] += a.y;
-                v[2] += a.z;
-                v[3] += a.w;
+            for (int u = 0; u < 8; ++u) {
+                v[0] += a[u].x;
+                v[1] += a[u].y;
+                v[2] += a[u].z;
+                v[3] += a[u].w;
             }
         }
-        if (groups > 1) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) part[threadIdx.x][c] = v[c];
-            __syncthreads();
-            if (ty == 0)
-                for (int u = 1; u < groups; ++u)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) v[c] += part[u * bw + tx][c];
-            __syncthreads();
+        for (; s < it.num_parts; s += groups) {
+            const int4 a = __ldg(p + (size_t)s * quads);
+            v[0] += a.x;
+            v[1] += a.y;
+            v[2] += a.z;
+            v[3] += a.w;
         }
-        if (ty == 0 && in) {
-            const long long t = it.use_b1 ? finish_b1_term_fresh(it, b1, q) : 0;
+    }
+    if (groups > 1) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                v[c] += t;
-                sums[4 * (size_t)(q - first) + c] = v[c];
-                if (it.copy_out) it.copy_out[4 * (size_t)q + c] = v[c];
-                const unsigned long long a = (unsigned long long)(v[c] < 0 ? -v[c] : v[c]);
-                mx = a > mx ? a : mx;
-            }
+        for (int c = 0; c < 4; ++c) part[threadIdx.x][c] = v[c];
+        __syncthreads();
+        if (ty == 0)
+            for (int u = 1; u < groups; ++u)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[c] += part[u * bw + tx][c];
+        __syncthreads();
+    }
+    if (ty == 0 && in) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            v[c] += term;
+            sums[4 * (size_t)(q - first) + c] = v[c];
+            if (it.copy_out) it.copy_out[4 * (size_t)q + c] = v[c];
+            const unsigned long long a = (unsigned long long)(v[c] < 0 ? -v[c] : v[c]);
+            mx = a > mx ? a : mx;
         }
     }
     mx = block_max_u64(mx);   // (its barriers also publish the sums to the block)
@@ -532,22 +584,26 @@ __global__ void __launch_bounds__(kSmallThreads) finish_small_kernel(const __gri
 
 }  // namespace
 
+// Copies of the item's tap sums, and blocks of a cluster for each: a block reads 16 KB of e3 or more (a fraction of a round of its
+// loads; the small ones of a batch of 1 leave SMs to the error chain), and up to 128 KB, two rounds, as long as a cluster can grow.
+static unsigned long long tap_bytes(const FinishItem &it) { return it.pixels * (it.d.c_out < kTapSlab ? it.d.c_out : kTapSlab); }
+static int tap_copies(const FinishItem &it)
+{
+    int copies = 1;
+    while (copies < kTapReplicas && tap_bytes(it) > (16ull << 10) * copies) copies *= 2;
+    return copies;
+}
+static int tap_cluster(const FinishItem &it)
+{
+    int cluster = 1;
+    while (cluster < kTapMostCluster && tap_bytes(it) > (128ull << 10) * kTapReplicas * cluster) cluster *= 2;
+    return cluster;
+}
+
 // The launch geometry of an item, from its sizes.
 static void plan_finish_item(FinishItem &it, int sm_count, bool alone)
 {
-    const int slabs = (it.d.c_out + kClassSlab - 1) / kClassSlab, rows = it.d.n * it.ho;
-    // Every block ends in one atomic per (channel, tap), so a block gets kTapBytes of e3 (the time of its reads then covers
-    // that of its atomics) as long as that leaves no more than one block per SM, and at least a row per warp.
-    const int slab_bytes_blocks = (int)(((long long)rows * it.wo * (it.d.c_out < kClassSlab ? it.d.c_out : kClassSlab) + kTapBytes - 1) / kTapBytes);
-    int blocks = (sm_count + slabs - 1) / slabs;
-    if (blocks > slab_bytes_blocks) blocks = slab_bytes_blocks;
-    int rpb = (rows + blocks - 1) / blocks;
-    if (rpb < kThreads / 32) rpb = kThreads / 32;
-    const int most = (1 << 23) / it.wo;           // keeps the int32 class sums exact
-    if (rpb > most) rpb = most < 1 ? 1 : most;
-    it.rows_per_block = rpb;
-    it.tap_grid_x = (rows + rpb - 1) / rpb;
-    it.tap_blocks = it.use_b1 ? it.tap_grid_x * slabs : 0;
+    it.tap_copies = tap_copies(it);
     it.groups = it.num_parts >= 64 ? 16 : (it.num_parts >= 32 ? 8 : (it.num_parts >= 8 ? 4 : 1));
     const size_t quads = (size_t)it.n / 4, bw = kThreads / it.groups;
     size_t fb = (quads + bw - 1) / bw;
@@ -560,13 +616,16 @@ static void plan_finish_item(FinishItem &it, int sm_count, bool alone)
 void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, const ReduceHook &hook)
 {
     b.num = num;
+    b.tap_cluster = 1;
+    for (int k = 0; k < num; ++k)
+        if (items[k].use_b1 && tap_cluster(items[k]) > b.tap_cluster) b.tap_cluster = tap_cluster(items[k]);
     b.tap_first[0] = b.fin_first[0] = b.sq_first[0] = 0;
     for (int k = 0; k < num; ++k) {
         FinishItem &it = b.item[k];
         it = items[k];
         it.keep_sums = hook.fn != nullptr;
         plan_finish_item(it, sm_count, num == 1);
-        b.tap_first[k + 1] = b.tap_first[k] + it.tap_blocks;
+        b.tap_first[k + 1] = b.tap_first[k] + (it.use_b1 ? tap_slabs(it) * it.tap_copies * b.tap_cluster : 0);
         b.fin_first[k + 1] = b.fin_first[k] + it.fin_blocks;
         b.sq_first[k + 1] = b.sq_first[k] + it.sq_blocks;
     }
@@ -575,7 +634,7 @@ void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count,
 // shared memory of an item's tap blocks: at least (1 + border rows)(1 + border columns) sets
 static size_t tap_set_bytes(const FinishItem &it)
 {
-    return it.use_b1 ? sizeof(int32_t) * kClassSlab * (1 + it.bc.nrc) * (1 + it.bc.ncc) : 0;
+    return it.use_b1 ? sizeof(int32_t) * kTapSlab * (1 + it.bc.nrc) * (1 + it.bc.ncc) : 0;
 }
 
 // slice groups of the small kernel: as many as leave its CTAs one pass over their quads
@@ -598,28 +657,30 @@ cudaError_t launch_finish_small(FinishItem it, unsigned *status, int sm_count, b
     it.keep_sums = 0;
     plan_finish_item(it, sm_count, true);
     it.groups = small_groups(it);
-    // one range of rows per CTA and slab of channels
-    const int rows = it.d.n * it.ho, rpb = (rows + kSmallCtas - 1) / kSmallCtas;
-    it.rows_per_block = rpb;
-    it.tap_grid_x = (rows + rpb - 1) / rpb;
-    it.tap_blocks = it.use_b1 ? it.tap_grid_x * ((it.d.c_out + kClassSlab - 1) / kClassSlab) : 0;
     const size_t sums = (it.n / 4 + kSmallCtas - 1) / kSmallCtas * 4 * sizeof(long long), sets = tap_set_bytes(it);
-    static std::atomic<unsigned long long> allowed;   // 16 KB of sums, or 130 sets (at most 64 border classes)
-    const cudaError_t e = allow_smem((const void *)finish_small_kernel, 72 * 1024, allowed);
-    if (e != cudaSuccess) return e;
-    return launch_chained_clusters(kSmallCtas, finish_small_kernel, kSmallCtas, kSmallThreads, sums > sets ? sums : sets, s, it, status, (int)beside);
+    return launch_chained_clusters(kSmallCtas, finish_small_kernel, kSmallCtas, kSmallThreads, sums > sets ? sums : sets, s, it, status,
+                                   (int)beside);   // (16 KB of sums, or 17 KB of sets)
 }
 
-cudaError_t launch_finish_taps(const FinishBatch &b, bool beside, cudaStream_t s)
+cudaError_t launch_finish_taps(const FinishBatch &b, bool let_in, cudaStream_t s)
 {
     size_t smem = 0;
     for (int k = 0; k < b.num; ++k) smem = tap_set_bytes(b.item[k]) > smem ? tap_set_bytes(b.item[k]) : smem;
-    if (smem > 48 * 1024) {   // at most 64 classes: 130 sets
-        const cudaError_t e = cudaFuncSetAttribute(finish_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
+    smem += sizeof(int32_t) * kMaxTaps * kTapSlab;   // (at most 64 border classes, 130 sets: 25 KB in all)
+    if (!let_in) return launch_chained_clusters(b.tap_cluster, finish_taps_kernel<false>, b.tap_first[b.num], kTapThreads, smem, s, b);
+    // An SM divides its memory between L1 and shared memory when it is idle: the GEMM's CTAs find room beside these blocks only if
+    // they leave it as much shared memory as there is.
+    static std::atomic<unsigned long long> divided;
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = device < 64 ? 1ull << device : 0ull;
+    if (!(divided.load(std::memory_order_relaxed) & bit)) {
+        e = cudaFuncSetAttribute(finish_taps_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
+        divided.fetch_or(bit, std::memory_order_relaxed);
     }
-    launch_chained(finish_taps_kernel, b.tap_first[b.num], kThreads, smem, s, b, (int)beside);
-    return cudaGetLastError();
+    return launch_chained_clusters(b.tap_cluster, finish_taps_kernel<true>, b.tap_first[b.num], kTapThreads, smem, s, b);
 }
 
 cudaError_t launch_finish_sums(const FinishBatch &b, unsigned *status, cudaStream_t s, const ReduceHook &hook)

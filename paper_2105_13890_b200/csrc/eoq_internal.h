@@ -274,9 +274,9 @@ struct WgradParams {
     int row_window_kw;   // 0, or the filter width when an M tile is one filter row of 8 x 16 bytes (7 real taps of 8)
     unsigned char tap_dh[kMaxTaps], tap_dw[kMaxTaps];
     int32_t *partials;   // [num_k_splits][c_out][taps][c_in] partial sums, a slice per split
-    int4 *zero;          // the cells of the kernels that follow (tap sums, maximum): cleared here, zero_n16 groups of 16 bytes
-    unsigned zero_n16;
-    int launch_early;    // the next kernel on the stream starts beside this one (see launch_finish_taps)
+    unsigned long long *zero;   // the cell of the maximum that the kernels behind reduce: cleared here
+    int launch_early;    // the next kernel on the stream starts beside this one (see launch_finish_small)
+    int wait_late;       // the launch in front is the layer's launch_finish_taps: this one runs beside it and waits for it at its end
     DeviceState *dev;
 };
 
@@ -306,9 +306,8 @@ struct WgradPatchPlan {
     int num_stages;
     int rows_total;      // taps * c_in
     int32_t *partials;   // [num_splits][c_out][taps][c_in]
-    int4 *zero;          // as in WgradParams
-    unsigned zero_n16;
-    int launch_early;
+    unsigned long long *zero;   // as in WgradParams
+    int launch_early, wait_late;
     DeviceState *dev;
 };
 constexpr int kWgradPatchThreads = 192;  // warp 0 loads, warp 1 MMA + TMEM, warps 2..5 epilogue
@@ -325,8 +324,7 @@ struct WgradRowsPlan {
     int rows_per_split, num_splits;
     int rows_total;      // kh * kw * c_in
     int32_t *partials;   // [num_splits][c_out][kh][kw][c_in]
-    int4 *zero;          // as in WgradParams
-    unsigned zero_n16;
+    unsigned long long *zero;   // as in WgradParams
     DeviceState *dev;
 };
 cudaError_t launch_wgrad_rows(const WgradRowsPlan &pl, const CUtensorMap &map_x, const CUtensorMap &map_e, cudaStream_t stream);
@@ -394,7 +392,7 @@ struct BorderClasses {
 };
 cudaError_t launch_b1_weight_table(const int8_t *w, int32_t *table, const eoq_conv_desc_t &d, const BorderClasses &bc,
                                    cudaStream_t s);
-constexpr int kTapReplicas = 4;  // copies of the b1 error sums of a weight gradient the blocks spread their atomics over
+constexpr int kTapReplicas = 4;  // copies of the b1 error sums of a weight gradient, each over a part of the rows
 constexpr int kMaxBorderClasses = 64;  // classes (rows x columns) the b1 kernels keep in shared memory
 
 // eoq_weight_prep: one launch derives the b1 tables (and the row-padded first-layer weights) of up to kPrepChunk layers
@@ -465,7 +463,7 @@ struct FinishItem {
     const int32_t *b1_dev;         // b1 in device memory, or null: b1_c
     int32_t b1_c;
     int use_b1;                    // 0: no b1 term (then the tap sums are neither formed nor read)
-    long long *tap_sums;           // [oc][tap][kTapReplicas copies]; cleared by the GEMM kernel
+    long long *tap_sums;           // [oc][tap][kTapReplicas copies]
     unsigned long long *max_cell;  // max |sum| of the layer (behind the tap sums); cleared by the GEMM kernel
     long long *acc;                // where the slices' sums [oc][tap][ic] go: 64-bit, or int32 when they provably fit
     const int32_t *parts;          // int32 split-K slices of the GEMM
@@ -478,21 +476,23 @@ struct FinishItem {
     BorderClasses bc;
     int ho, wo, num_parts;
     // filled by plan_finish
-    int rows_per_block, tap_grid_x, tap_blocks, groups, fin_blocks, sq_blocks;
+    int tap_copies, groups, fin_blocks, sq_blocks;
     int keep_sums;                 // reduce hook: the sums are completed by an all-reduce before their maximum is taken
 };
 struct FinishBatch {
     int num;
+    int tap_cluster;   // blocks of a cluster of the tap sums' launch
     int tap_first[kFinishChunk + 1], fin_first[kFinishChunk + 1], sq_first[kFinishChunk + 1];
     FinishItem item[kFinishChunk];
 };
 // Lays out the launches of up to kFinishChunk items; then, in this order on one stream, the b1 error sums (only where an item
 // has a b1 term: tap_first[num] > 0) and the sums with Q_g (two kernels, a third per item under a reduce hook).
-// beside: the launch in front on the stream is the item's GEMM, which lets its successor start once e3 is complete
-// (launch_early); the error sums are then formed beside it, and wait for its end only before they go into the cells.
+// let_in: the launch behind the error sums is the item's GEMM with wait_late, which runs beside them: they let it in once everything
+// in front of them is complete, and it waits for them at its end.
 void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, const ReduceHook &hook);
-cudaError_t launch_finish_taps(const FinishBatch &b, bool beside, cudaStream_t s);
-// ... or all of it in one launch, for one small item (no reduce hook)
+cudaError_t launch_finish_taps(const FinishBatch &b, bool let_in, cudaStream_t s);
+// ... or all of it in one launch, for one small item (no reduce hook).  beside: the launch in front on the stream is the item's GEMM,
+// which lets its successor start once e3 is complete (launch_early); the error sums are then formed beside it.
 bool finish_is_small(const FinishItem &it, const ReduceHook &hook);
 cudaError_t launch_finish_small(FinishItem it, unsigned *status, int sm_count, bool beside, cudaStream_t s);
 cudaError_t launch_finish_sums(const FinishBatch &b, unsigned *status, cudaStream_t s, const ReduceHook &hook);

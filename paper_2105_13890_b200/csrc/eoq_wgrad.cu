@@ -102,9 +102,11 @@ wgrad_kernel(const __grid_constant__ WgradParams p, const __grid_constant__ CUte
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    ptx::grid_dep_wait();   // everything up to here touched no global memory
+    // Everything up to here touched no global memory.  Behind the layer's tap sums the kernels that wrote the operands are complete
+    // already (they were when the tap sums let this launch in), and the tap sums write nothing that it reads.
+    if (!p.wait_late) ptx::grid_dep_wait();
     if (p.launch_early) ptx::grid_dep_launch();
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < p.zero_n16; i += gridDim.x * blockDim.x) p.zero[i] = make_int4(0, 0, 0, 0);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *p.zero = 0;
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, p.dev};
 
@@ -235,6 +237,7 @@ wgrad_kernel(const __grid_constant__ WgradParams p, const __grid_constant__ CUte
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, tmem_cols);
     }
+    if (p.wait_late) ptx::grid_dep_wait();   // (what comes behind this launch waits for it alone)
 }
 
 }  // namespace
@@ -252,7 +255,8 @@ cudaError_t launch_wgrad(const WgradParams &p, const CUtensorMap &map_x, const C
     const cudaError_t e = allow_smem((const void *)wgrad_kernel, 208 * 1024, allowed);
     if (e != cudaSuccess) return e;
     const int grid = p.num_m_groups * p.num_n_tiles * p.num_k_splits;
-    return launch_chained(wgrad_kernel, grid, kWgradThreads, wgrad_smem_bytes(p), stream, p, map_x, map_e);
+    const size_t need = wgrad_smem_bytes(p), least = p.wait_late ? 116 * 1024 : 0;   // (as launch_wgrad_patch)
+    return launch_chained(wgrad_kernel, grid, kWgradThreads, need > least ? need : least, stream, p, map_x, map_e);
 }
 
 }  // namespace eoq

@@ -87,9 +87,11 @@ wgrad_patch_kernel(const __grid_constant__ WgradPatchPlan pl, const __grid_const
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    ptx::grid_dep_wait();   // everything up to here touched no global memory
+    // Everything up to here touched no global memory.  Behind the layer's tap sums the kernels that wrote the operands are complete
+    // already (they were when the tap sums let this launch in), and the tap sums write nothing that it reads.
+    if (!pl.wait_late) ptx::grid_dep_wait();
     if (pl.launch_early) ptx::grid_dep_launch();
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < pl.zero_n16; i += gridDim.x * blockDim.x) pl.zero[i] = make_int4(0, 0, 0, 0);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *pl.zero = 0;
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, pl.dev};
 
@@ -200,6 +202,7 @@ wgrad_patch_kernel(const __grid_constant__ WgradPatchPlan pl, const __grid_const
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, tmem_cols);
     }
+    if (pl.wait_late) ptx::grid_dep_wait();   // (what comes behind this launch waits for it alone)
 }
 
 }  // namespace
@@ -215,8 +218,9 @@ cudaError_t launch_wgrad_patch(const WgradPatchPlan &pl, const CUtensorMap &map_
     static std::atomic<unsigned long long> allowed;
     const cudaError_t e = allow_smem((const void *)wgrad_patch_kernel, 208 * 1024, allowed);
     if (e != cudaSuccess) return e;
-    return launch_chained(wgrad_patch_kernel, pl.num_groups * pl.num_splits, kWgradPatchThreads, wgrad_patch_smem_bytes(pl), stream, pl, map_x,
-                                                                                                                 map_e);
+    // (beside the tap sums, CTAs of less than half an SM's shared memory would meet on the SMs that those leave empty)
+    const size_t need = wgrad_patch_smem_bytes(pl), least = pl.wait_late ? 116 * 1024 : 0;
+    return launch_chained(wgrad_patch_kernel, pl.num_groups * pl.num_splits, kWgradPatchThreads, need > least ? need : least, stream, pl, map_x, map_e);
 }
 
 }  // namespace eoq

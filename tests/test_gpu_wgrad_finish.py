@@ -153,3 +153,35 @@ def test_error_sums_beside_the_gemm(d):
         e3_o, p3, _ = oracle.sq_int(e0.astype(np.int64) * 128, -7)
         want, p, _ = oracle.sq_int(oracle.conv_wgrad_acc(d, e3_o, x0, -37), p3 - 7)
         assert np.array_equal(G.host(g), want) and pg.item() == p
+
+
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("case", [
+    (1, 5, 6, 16, 16, 3, 1, 1, 7),           # fewer rows than copies of the error sums
+    (3, 70, 45, 16, 48, 3, 2, 1, -3),        # a slab of 32 channels and one of 16
+    (5, 65, 64, 16, 32, 3, 1, 1, 9),         # clusters of two blocks
+    (9, 66, 64, 32, 80, 1, 1, 0, 11),        # of four
+    (33, 66, 65, 16, 32, 5, 1, 2, -128),     # of eight, four border rows and columns
+    (1, 3, 300, 16, 32, 7, 1, 3, 100),       # every row a class of its own
+], ids=lambda c: "n%d_%dx%d_%d_%d_k%ds%d" % c[:7])
+def test_error_sums_of_every_cluster_size(case, batched):
+    """The b1 term against the oracle where a layer's error sums are formed by one block, or by clusters of two to eight; a single
+    call (sums in front of the GEMM and beside it) and a finish of two layers, twice on one workspace whose contents are arbitrary."""
+    hd = G.handle()
+    d, e3, x0, b1, g_o, pg_o = make(case, 8960)
+    gd, ws = G.gdesc(d), G.workspace(G.gdesc(d), eoq.EOQ_PASS_WGRAD)
+    ws.fill_(0x5A)
+    e3_d, pe, x_d, b1_d = G.dev(e3), G.dev(np.array([-12], dtype=np.int32)), G.dev(x0), G.dev(np.array([b1], dtype=np.int32))
+    for _ in range(2):
+        g, pg = G.empty(g_o.shape, torch.int8), G.zeros(1, torch.int32)
+        if batched:
+            d2, e2, x2, c2, g2_o, pg2_o = make(LAYERS[1], 8961)
+            ws2, g2, pg2 = G.workspace(G.gdesc(d2), eoq.EOQ_PASS_WGRAD), G.empty(g2_o.shape, torch.int8), G.zeros(1, torch.int32)
+            e2_d = G.dev(e2)
+            parts = [eoq.eoq_conv_wgrad_gemm(hd, gd, e3_d, pe, x_d, ws), eoq.eoq_conv_wgrad_gemm(hd, G.gdesc(d2), e2_d, pe, G.dev(x2), ws2)]
+            eoq.eoq_wgrad_finish(hd, [gd, G.gdesc(d2)], [e3_d, e2_d], [pe, pe], [b1_d, G.dev(np.array([c2], dtype=np.int32))], [g, g2],
+                                 [pg, pg2], [ws, ws2], parts)
+            assert np.array_equal(G.host(g2), g2_o) and pg2.item() == pg2_o
+        else:
+            eoq.eoq_conv_wgrad_dev(hd, gd, e3_d, pe, x_d, b1_d, g, pg, ws)
+        assert G.status_clear() == 0 and np.array_equal(G.host(g), g_o) and pg.item() == pg_o
