@@ -67,7 +67,7 @@ struct AbsMax16 {
 };
 
 // Bound by HBM / L2 reads (1 B per weight).  The 21 M weights of ResNet-34: 13.4 us with a 32-bit maximum per code, 7.4 us
-// with packed 16-bit ones.
+// with packed 16-bit ones, 6.7 with both loads of a thread in flight.
 __global__ void __launch_bounds__(kThreads) update_absmax_kernel(const __grid_constant__ UpdateBatch b, DeviceState *dev)
 {
     ptx::grid_dep_wait_launch_small();
@@ -81,8 +81,15 @@ __global__ void __launch_bounds__(kThreads) update_absmax_kernel(const __grid_co
         const bool vec = (reinterpret_cast<uintptr_t>(T.g) & 15) == 0;
         AbsMax16 am;
         if (vec) {
-            for (size_t i = begin + (size_t)threadIdx.x * 16; i + 16 <= end; i += (size_t)kThreads * 16)
-                am.add(__ldg(reinterpret_cast<const int4 *>(T.g + i)));
+            constexpr int kLoads = kUpdElemsPerBlock / (kThreads * 16);   // all in flight together
+            int4 v[kLoads];
+#pragma unroll
+            for (int q = 0; q < kLoads; ++q) {
+                const size_t i = begin + ((size_t)q * kThreads + threadIdx.x) * 16;
+                v[q] = i + 16 <= end ? __ldg(reinterpret_cast<const int4 *>(T.g + i)) : make_int4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int q = 0; q < kLoads; ++q) am.add(v[q]);
         }
         mx = am.value();
         // remaining elements of this block's range
@@ -95,19 +102,21 @@ __global__ void __launch_bounds__(kThreads) update_absmax_kernel(const __grid_co
 
 // What the update of one tensor needs, the same for all its elements.
 struct UpdateRule {
-    int mul, sh, half_m1;  // u = sat(R(mul * g / 2^sh))
     int d;                 // exponent of u relative to the weight grid 2^-7: w - u * 2^d
+    float scale;           // u = sat(R(g * scale))
+    bool same, clips;      // u = g; some |g| reaches beyond 127
     unsigned long long key;
 };
 
-__device__ __forceinline__ UpdateRule update_rule(uint32_t M, int g_exp, int lr_mant, int lr_exp, int stochastic, unsigned long long seed,
+// `max_g`: the largest |g| of the tensor, M = lr_mant * max_g != 0
+__device__ __forceinline__ UpdateRule update_rule(uint32_t max_g, int g_exp, int lr_mant, int lr_exp, int stochastic, unsigned long long seed,
                                                   unsigned long long step, int tensor)
 {
     UpdateRule r;
-    const int t = round_log2_u32(M);
-    r.mul = t < 7 ? lr_mant << (7 - t) : lr_mant;
-    r.sh = t < 7 ? 0 : t - 7;
-    r.half_m1 = r.sh ? (1 << (r.sh - 1)) - 1 : 0;
+    const int t = round_log2_u32(max_g * (uint32_t)lr_mant);
+    r.scale = (float)lr_mant * __int_as_float((127 + 7 - t) << 23);   // exact, as every g * scale is
+    r.clips = (float)max_g * r.scale >= 127.5f;                       // (which ties to 128)
+    r.same = r.scale == 1.0f && !r.clips;
     r.d = (g_exp + lr_exp + t - 7) + 7;
     r.key = 0;
     if (stochastic) {
@@ -131,82 +140,161 @@ __device__ __forceinline__ UpdateMode update_mode(const UpdateRule &r, int stoch
     return r.d < -7 ? kKeep : kNearest;
 }
 
-// One code; z: the element's hash counter key + (index + 1) * golden (stochastic modes).  The result still needs the
-// upper clamp at 127 (the packing saturates there); the lower one at -127 is applied here.
-template <UpdateMode kMode>
-__device__ __forceinline__ int update_code(int w, int g, const UpdateRule &r, unsigned long long z)
+// How u comes from g: as it is (a learning rate that is a power of two, behind Q_g, whose largest code is 91 or more), by a rounded
+// product, or by one that the quantizer clips.
+enum UpdateCode { kSame, kScaled, kClipped };
+
+// What the loops keep in registers.
+struct UpdateLoop {
+    int s;                 // -d
+    uint32_t mask, one;    // 2^s - 1; 1, though the compiler does not know: a multiply-add adds it on the multiply-add pipe
+    float scale;           // -scale of the rule
+};
+__device__ __forceinline__ UpdateLoop update_loop(const UpdateRule &r)
 {
-    if (kMode == kKeep) return max(w, -127);
-    int u = r.mul * g;
-    if (r.sh) u = (u + r.half_m1 + ((u >> r.sh) & 1)) >> r.sh;
-    u = clampi(u, -127, 127);
-    int next;
-    if (kMode == kShiftUp) {
-        next = w - u * (1 << min(r.d, 9));  // any |u| * 2^9 saturates, as any larger power would
-    } else if (kMode == kNearest) {
-        const int s = -r.d, v = w * (1 << s) - u;
-        next = (v + ((1 << (s - 1)) - 1) + ((v >> s) & 1)) >> s;
-    } else if (kMode == kStochastic) {
-        // floor((w 2^s - u + rand) / 2^s) = w + floor((rand - u) / 2^s)
-        const int s = -r.d;
-        next = w + (((int)((uint32_t)mix64(z) & ((1u << s) - 1u)) - u) >> s);
-    } else {
-        const int s = -r.d;
-        next = w + (int)(((long long)(mix64(z) & ((1ull << s) - 1ull)) - u) >> s);
-    }
-    return max(next, -127);
+    UpdateLoop l;
+    l.s = -r.d;
+    l.mask = r.d < 0 && r.d >= -30 ? (1u << -r.d) - 1u : 0u;
+    asm volatile("mov.u32 %0, 1;" : "=r"(l.one));
+    l.scale = -r.scale;
+    return l;
 }
 
-template <UpdateMode kMode>
-__device__ __forceinline__ int4 update_16(const int4 &wv, const int4 &gv, const UpdateRule &r, size_t i)
+__device__ __forceinline__ uint32_t mad_lo(uint32_t a, uint32_t b, uint32_t c)
+{
+    uint32_t d;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
+// Low words of mix64 under a mask, the products on 32-bit halves.
+__device__ __forceinline__ uint32_t mix64_low(unsigned long long z, uint32_t mask)
+{
+    constexpr uint32_t kLo1 = 0x1CE4E5B9u, kHi1 = 0xBF58476Du, kLo2 = 0x133111EBu, kHi2 = 0x94D049BBu;
+    uint32_t lo = (uint32_t)z, hi = (uint32_t)(z >> 32);
+    uint32_t a = lo ^ __funnelshift_r(lo, hi, 30), b = hi ^ (hi >> 30);
+    unsigned long long p = (unsigned long long)a * kLo1;
+    lo = (uint32_t)p;
+    hi = mad_lo(b, kLo1, mad_lo(a, kHi1, (uint32_t)(p >> 32)));
+    a = lo ^ __funnelshift_r(lo, hi, 27);
+    b = hi ^ (hi >> 27);
+    p = (unsigned long long)a * kLo2;
+    lo = (uint32_t)p;
+    hi = mad_lo(b, kLo2, mad_lo(a, kHi2, (uint32_t)(p >> 32)));
+    return (lo ^ __funnelshift_r(lo, hi, 31)) & mask;
+}
+
+// byte k of `codes` (signed) times +-1, plus c: a byte dot product takes the code out of its word on the multiply-add pipe
+template <int k, bool kMinus>
+__device__ __forceinline__ int add_code(uint32_t codes, int c)
+{
+    int d;
+    asm("dp4a.s32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(codes), "r"((kMinus ? 0xffu : 1u) << (8 * k)), "r"(c));
+    return d;
+}
+
+constexpr uint32_t kUpdateMagic = 0x4B400000u;   // 1.5 * 2^23 as a float
+// c - u of the code in byte k of `g` (`biased`: the word with its sign bits flipped).  -u = R(g * -scale) by one multiply-add: the
+// byte above 2^23 is a float, 2^23 + 128 off it leaves g.
+template <UpdateCode kCode, int k>
+__device__ __forceinline__ int subtract_u(int c, uint32_t g, uint32_t biased, const UpdateLoop &l)
+{
+    if (kCode == kSame) return add_code<k, true>(g, c);
+    const float x = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7540 | k)) - 8388736.0f;
+    const int bits = (int)__float_as_uint(__fmaf_rn(x, l.scale, 12582912.0f));
+    if (kCode == kScaled) return c + bits - (int)kUpdateMagic;
+    return c + min(__viaddmax_s32(bits, -(int)kUpdateMagic, -127), 127);
+}
+
+// New code of byte k of w; z: the element's hash counter key + (index + 1) * golden (stochastic modes).  The result still needs the
+// upper clamp at 127 (the packing saturates there); the lower one at -127 is applied here.
+template <UpdateMode kMode, UpdateCode kCode, int k>
+__device__ __forceinline__ int update_code(uint32_t w, uint32_t g, uint32_t biased, const UpdateLoop &l, unsigned long long z)
+{
+    if (kMode == kKeep) return max(sbyte<k>(w), -127);
+    if (kMode == kShiftUp) {
+        return max(sbyte<k>(w) + subtract_u<kCode, k>(0, g, biased, l) * (1 << min(-l.s, 9)), -127);   // any |u| * 2^9 saturates, as any larger power would
+    } else if (kMode == kNearest) {
+        const int v = subtract_u<kCode, k>(sbyte<k>(w) * (1 << l.s), g, biased, l);
+        return max((v + ((1 << (l.s - 1)) - 1) + ((v >> l.s) & 1)) >> l.s, -127);
+    } else if (kMode == kStochastic) {
+        // floor((w 2^s - u + rand) / 2^s) = w + floor((rand - u) / 2^s)
+        return max(add_code<k, false>(w, subtract_u<kCode, k>((int)mix64_low(z, l.mask), g, biased, l) >> l.s), -127);
+    } else {
+        return max(sbyte<k>(w) + (int)(((long long)(mix64(z) & ((1ull << l.s) - 1ull)) + subtract_u<kCode, k>(0, g, biased, l)) >> l.s), -127);
+    }
+}
+
+template <UpdateMode kMode, UpdateCode kCode>
+__device__ __forceinline__ int4 update_16(const int4 &wv, const int4 &gv, const UpdateLoop &l, unsigned long long key, size_t i)
 {
     const uint32_t ww[4] = {(uint32_t)wv.x, (uint32_t)wv.y, (uint32_t)wv.z, (uint32_t)wv.w};
     const uint32_t gw[4] = {(uint32_t)gv.x, (uint32_t)gv.y, (uint32_t)gv.z, (uint32_t)gv.w};
     uint32_t o[4];
-    unsigned long long z = r.key + kGolden * ((unsigned long long)i + 1);
+    unsigned long long z = key + kGolden * ((unsigned long long)i + 1);
+    auto next = [&]() {   // z, and on to the next element's: z + golden as two multiply-adds
+        const unsigned long long now = z;
+        if (kMode == kStochastic) {
+            asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(z) : "r"(l.one), "r"((uint32_t)kGolden), "l"(now));
+            z = (unsigned long long)mad_lo(l.one, (uint32_t)(kGolden >> 32), (uint32_t)(z >> 32)) << 32 | (uint32_t)z;
+        } else {
+            z += kGolden;
+        }
+        return now;
+    };
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        int c[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k, z += kGolden)
-            c[k] = update_code<kMode>((int)(int8_t)(ww[q] >> (8 * k)), (int)(int8_t)(gw[q] >> (8 * k)), r, z);
-        o[q] = pack4_sat(c[0], c[1], c[2], c[3]);
+        const uint32_t b = gw[q] ^ 0x80808080u;
+        const int c0 = update_code<kMode, kCode, 0>(ww[q], gw[q], b, l, next());
+        const int c1 = update_code<kMode, kCode, 1>(ww[q], gw[q], b, l, next());
+        const int c2 = update_code<kMode, kCode, 2>(ww[q], gw[q], b, l, next());
+        const int c3 = update_code<kMode, kCode, 3>(ww[q], gw[q], b, l, next());
+        o[q] = pack4_sat(c0, c1, c2, c3);
     }
     return make_int4((int)o[0], (int)o[1], (int)o[2], (int)o[3]);
 }
 
 // elements [begin, end) of one tensor by the calling block
-template <UpdateMode kMode>
+template <UpdateMode kMode, UpdateCode kCode>
 __device__ __forceinline__ void update_range(const UpdateTensor &T, size_t begin, size_t end, const UpdateRule &r)
 {
+    const UpdateLoop l = update_loop(r);
     const bool vec = ((reinterpret_cast<uintptr_t>(T.g) | reinterpret_cast<uintptr_t>(T.w)) & 15) == 0;
     if (vec)
         for (size_t i = begin + (size_t)threadIdx.x * 16; i + 16 <= end; i += (size_t)blockDim.x * 16) {
             const int4 gv = kMode == kKeep ? make_int4(0, 0, 0, 0) : __ldg(reinterpret_cast<const int4 *>(T.g + i));
             const int4 wv = *reinterpret_cast<const int4 *>(T.w + i);
-            *reinterpret_cast<int4 *>(T.w + i) = update_16<kMode>(wv, gv, r, i);
+            *reinterpret_cast<int4 *>(T.w + i) = update_16<kMode, kCode>(wv, gv, l, r.key, i);
         }
     const size_t tail = vec ? begin + ((end - begin) / 16) * 16 : begin;
-    for (size_t j = tail + threadIdx.x; j < end; j += blockDim.x)
-        T.w[j] = (int8_t)min(update_code<kMode>(T.w[j], T.g[j], r, r.key + kGolden * ((unsigned long long)j + 1)), 127);
-}
-
-__device__ __forceinline__ void update_range(UpdateMode mode, const UpdateTensor &T, size_t begin, size_t end, const UpdateRule &r)
-{
-    switch (mode) {
-        case kShiftUp: update_range<kShiftUp>(T, begin, end, r); break;
-        case kNearest: update_range<kNearest>(T, begin, end, r); break;
-        case kKeep: update_range<kKeep>(T, begin, end, r); break;
-        case kStochastic: update_range<kStochastic>(T, begin, end, r); break;
-        default: update_range<kStochasticWide>(T, begin, end, r); break;
+    for (size_t j = tail + threadIdx.x; j < end; j += blockDim.x) {
+        const uint32_t g = (uint8_t)T.g[j];
+        T.w[j] = (int8_t)min(update_code<kMode, kCode, 0>((uint8_t)T.w[j], g, g ^ 0x80u, l, r.key + kGolden * ((unsigned long long)j + 1)), 127);
     }
 }
 
-// w <- Q_w(w - Q_u(lr * g)).  Bound by the integer pipe under stochastic rounding: 43 instructions a weight, most of them the 64-bit
-// hash's, 24 of which go to the pipe that takes one every two cycles and scheduler: 27.5 of the 37 us that the 21 M weights of
-// ResNet-34 take (the pipe is 79% busy while an SM has work).  Rounding to nearest takes 14 instructions and 15 us; its largest stall
-// is that of its loads.  Every rounding mode is a loop of its own on 32-bit values: one 64-bit sequence for all modes took 58 us.
-__global__ void __launch_bounds__(kThreads)
+// (only the stochastic loop, the one that arithmetic bounds, is worth a form without the clamps or the product)
+__device__ __forceinline__ void update_range(UpdateMode mode, const UpdateTensor &T, size_t begin, size_t end, const UpdateRule &r)
+{
+    switch (mode) {
+        case kShiftUp: update_range<kShiftUp, kClipped>(T, begin, end, r); break;
+        case kNearest: update_range<kNearest, kClipped>(T, begin, end, r); break;
+        case kKeep: update_range<kKeep, kSame>(T, begin, end, r); break;
+        case kStochastic:
+            if (r.same) update_range<kStochastic, kSame>(T, begin, end, r);
+            else if (!r.clips) update_range<kStochastic, kScaled>(T, begin, end, r);
+            else update_range<kStochastic, kClipped>(T, begin, end, r);
+            break;
+        default: update_range<kStochasticWide, kClipped>(T, begin, end, r); break;
+    }
+}
+
+// w <- Q_w(w - Q_u(lr * g)).  Bound by the integer pipe and by issue under stochastic rounding: 32 instructions a weight, of which the
+// 64-bit hash's shifts and exclusive-ors, 10, can go nowhere else (the pipe takes an instruction every two cycles and scheduler); codes
+// are taken out of their words, scaled and added on the multiply-add pipe.  The 21 M weights of ResNet-34: 37.3 us with 43
+// instructions, 24 of them on that pipe, 28.6 with 15 and six blocks to an SM (31.0 with four).  Rounding to nearest is bound by its
+// loads.  Every rounding mode is a loop of its own on 32-bit values.
+__global__ void __launch_bounds__(kThreads, 6)
 update_apply_kernel(const __grid_constant__ UpdateBatch b, int32_t lr_mant, int32_t lr_exp, int stochastic, unsigned long long seed,
                     unsigned long long step, unsigned long long *step_dev, DeviceState *dev)
 {
@@ -223,9 +311,8 @@ update_apply_kernel(const __grid_constant__ UpdateBatch b, int32_t lr_mant, int3
     __syncthreads();
     bool last = false;
     if (threadIdx.x == 0) last = last_reader(dev);
-    const uint32_t M = max_s * (uint32_t)lr_mant;  // max |lr_mant * g| < 2^15
-    if (M != 0) {
-        const UpdateRule r = update_rule(M, g_exp, lr_mant, lr_exp, stochastic, seed, step_s, b.tensor_base + k);
+    if (max_s != 0) {
+        const UpdateRule r = update_rule(max_s, g_exp, lr_mant, lr_exp, stochastic, seed, step_s, b.tensor_base + k);
         const size_t begin = (size_t)(blockIdx.x - b.first_block[k]) * kUpdElemsPerBlock;
         update_range(update_mode(r, stochastic), T, begin, min((size_t)T.n, begin + kUpdElemsPerBlock), r);
     } else if (threadIdx.x == 0 && (int)blockIdx.x == b.first_block[k]) {
@@ -284,9 +371,8 @@ update_small_kernel(const __grid_constant__ UpdateBatch b, int parts, int32_t lr
     }
     bool last = false;
     if (threadIdx.x == 0) last = last_reader(dev);
-    const uint32_t M = mx * (uint32_t)lr_mant;
-    if (M != 0) {
-        const UpdateRule r = update_rule(M, g_exp, lr_mant, lr_exp, stochastic, seed, step_s, b.tensor_base + k);
+    if (mx != 0) {
+        const UpdateRule r = update_rule(mx, g_exp, lr_mant, lr_exp, stochastic, seed, step_s, b.tensor_base + k);
         update_range(update_mode(r, stochastic), T, begin, end, r);
     } else if (threadIdx.x == 0 && part == 0) {
         atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);

@@ -55,6 +55,30 @@ def test_update_one_block_per_tensor(lr, stochastic):
             assert np.array_equal(G.host(w_d[i]).astype(np.int32), ws[i]), (k, i)
 
 
+@pytest.mark.parametrize("max_g", [1, 3, 45, 90, 91, 127, 128])
+@pytest.mark.parametrize("lr_mant", [1, 2, 3, 181, 255])
+def test_update_codes_of_every_form(lr_mant, max_g):
+    """The update's codes as they are, scaled, and clipped, by the largest gradient code and the learning rate (-128, which Q_g does not
+    form, among them); rounding shifts of 1 to 40 bits, a length that is no multiple of 16 and codes off the 16-byte grid."""
+    n = 66000 + 7
+    g = np.clip(synth.normal_codes(n, 1525, max_g, std_codes=40).astype(np.int32), -max_g, max_g - (max_g == 128)).astype(np.int8)
+    g[5], g[n - 1] = -max_g, max_g - (max_g == 128)
+    w = synth.int8_uniform(n, 1526, lr_mant)
+    t = int(oracle.sq_int(np.array([max_g * lr_mant], dtype=np.int64), 0)[1]) + 7   # R(log2 max)
+    lead = 3
+    for s in (0, 1, 2, 6, 9, 17, 29, 30, 31, 40, 41):
+        p = -s - (t - 7) - 7   # so that w - u 2^d has d = -s
+        for offset in (0, lead):
+            w_d, g_d = torch.zeros(n + 16, dtype=torch.int8, device="cuda:0"), torch.zeros(n + 16, dtype=torch.int8, device="cuda:0")
+            w_d[offset:offset + n], g_d[offset:offset + n] = G.dev(w), G.dev(g)
+            eoq.eoq_update(G.handle(), [w_d[offset:offset + n]], [g_d[offset:offset + n]], [G.dev(np.array([p], dtype=np.int32))], lr_mant, 0,
+                           eoq.EOQ_ROUND_STOCHASTIC, seed=12, step=4)
+            want, _, _ = oracle.update(w, g, p, lr_mant, 0, stochastic=True, seed=12, step=4, tensor_id=0)
+            assert G.status_clear() == 0
+            assert np.array_equal(G.host(w_d[offset:offset + n]).astype(np.int32), want), (s, offset)
+            assert not G.host(w_d[:offset]).any() and not G.host(w_d[offset + n:]).any()
+
+
 @pytest.mark.parametrize("n,c,hw,classes", [(1, 16, 1, 1), (8, 36, 4, 63), (9, 528, 9, 65), (3, 1536, 4, 130)])
 def test_float_head_remainders(n, c, hw, classes):
     """Folded and separate pooling (8 samples), channel counts beyond one 512-channel part, classes around a tile of 64."""
