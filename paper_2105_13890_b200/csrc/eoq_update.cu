@@ -17,9 +17,12 @@ constexpr int kUpdElemsPerBlock = 8192;  // elements one block covers
 // (36,864 codes: 11 us, a cluster of eight 6 us).
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallGroups = 4;          // 16-code groups per thread
+constexpr size_t kSmallElems = (size_t)kSmallThreads * kSmallGroups * 16;
 constexpr size_t kSmallPart = 8192;
 constexpr int kSmallMostParts = 8;
-constexpr size_t kSmallElems = (size_t)kSmallThreads * kSmallGroups * 16;
+// A block of a cluster has one group per thread at most.  At 64 registers two such blocks share an SM, so that the clusters of 37
+// tensors start together (blocks of 1024 threads: of 18; the 22 tensors of ResNet-20 8.9 us, with 512 threads 8.3 us).
+constexpr int kSmallPartThreads = (int)(kSmallElems / kSmallMostParts / 16);
 
 struct UpdateBatch {
     UpdateTensor t[kUpdChunk];
@@ -347,12 +350,12 @@ update_small_kernel(const __grid_constant__ UpdateBatch b, int parts, int32_t lr
     if (vec) {
 #pragma unroll
         for (int q = 0; q < kSmallGroups; ++q) {
-            const size_t i = begin + ((size_t)q * kSmallThreads + threadIdx.x) * 16;
+            const size_t i = begin + ((size_t)q * blockDim.x + threadIdx.x) * 16;
             if (i + 16 <= end) am.add(__ldg(reinterpret_cast<const int4 *>(T.g + i)));
         }
     }
     uint32_t mx = am.value();
-    for (size_t j = (vec ? begin + (end - begin) / 16 * 16 : begin) + threadIdx.x; j < end; j += kSmallThreads)
+    for (size_t j = (vec ? begin + (end - begin) / 16 * 16 : begin) + threadIdx.x; j < end; j += blockDim.x)
         mx = max(mx, (uint32_t)abs((int)T.g[j]));
     mx = block_max_u32(mx);
     if (parts > 1) {
@@ -477,6 +480,7 @@ cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32
     int parts = 1;
     for (int i = 0; i < num; ++i)
         if (stochastic && t[i].n > kSmallPart) parts = kSmallMostParts;   // (the hash is what takes the time)
+    const int threads = parts > 1 ? kSmallPartThreads : kSmallThreads;
     UpdateBatch b;
     if (!small)
         for (int base = 0; base < num; base += kUpdChunk) {
@@ -485,7 +489,7 @@ cudaError_t launch_update(const UpdateTensor *t, int num, int32_t lr_mant, int32
         }
     for (int base = 0; base < num; base += kUpdChunk) {
         const int blocks = fill_batch(b, t, num, base, first, last);
-        if (small) launch_chained_clusters(parts, update_small_kernel, b.num * parts, kSmallThreads, 0, s, b, parts, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
+        if (small) launch_chained_clusters(parts, update_small_kernel, b.num * parts, threads, 0, s, b, parts, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
         else launch_chained(update_apply_kernel, blocks, kThreads, 0, s, b, lr_mant, lr_exp, stochastic, seed, step, step_dev, dev);
     }
     return cudaGetLastError();
