@@ -25,10 +25,9 @@ inline int blocks_for(size_t items, int sm_count, int per_sm = 8)
 // pass = 0: max |S| into the handle's 64-bit cell; pass = 1: codes of SQ(S), their sum, exponent; cells back to zero.
 // kNext: the error head of the layer that consumes the joined error rides along (see NextHead): pass 0 also reduces
 // the maximum over the positions that layer's ReLU lets through, pass 1 also writes that layer's e3 and its two sums.
-// Bound by instruction issue and by the latency of its loads: a thread's next group travels while it works on one, operands whose
-// exponents lie at most 7 octaves apart (the usual case) are scaled, added and biased by one byte dot product per element and
-// rounded by one multiply-add, and a dropped operand is a factor of 0, not a case for 64 bits.  With the same in the Q_e passes
-// (sq_i32_kernel): ResNet-18 batch 64 1450 -> 1419 us, batch 1 456 -> 445, ResNet-20 batch 2 329 -> 313.
+// Bound by memory and by the latency of its loads: a thread's next group travels while it works on one, operands are scaled, added and
+// biased by one dot product per element whatever lies between their exponents (see join_mul) and rounded by one multiply-add.  Every
+// distance in 32 bits, in the Q_e passes (sq_i32_kernel) too: ResNet-18 step at batch 64 1338 -> 1240 us, at batch 13 604 -> 583.
 template <int kPass, bool kNext>
 __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, const int8_t *__restrict__ b, const int32_t *b_exp,
                             const uint8_t *__restrict__ mask_b, size_t n16, int8_t *out, int32_t *out_exp, long long *sum_out,
@@ -47,7 +46,6 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
         }
     }
     const JoinShift j = join_shift(__ldg(a_exp), __ldg(b_exp));
-    unsigned long long mx = 0, mxm = 0;
     long long sum = 0, s1 = 0, s2 = 0;
     int t = 7;
     NextHead nh = {};
@@ -80,13 +78,8 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
         }
     }
     const JoinMul jm = join_mul(j);
+    const JoinCode jc = join_code(jm, M, t);
     uint32_t mx32 = 0, mxm32 = 0;
-    // sums below 2^31 - 2^(t - 8): a right shift in few 32-bit operations (see sq_pack4_shr)
-    const int sh = t - 7;
-    const bool fast = !jm.wide && sh >= 1 && M < 0x7e000000ull;
-    const int32_t half_m1 = fast ? (1 << (sh - 1)) - 1 : 0, lo = fast ? -(127 << sh) : 0;
-    // near operands (sums below 2^15): the rounding is one multiply-add, as in prescale_apply_kernel
-    const float scale = __int_as_float((127 - (jm.near ? sh : 0)) << 23), rest = 12582912.0f - 12582912.0f * scale;
     struct Group {
         int4 a, b;
         uint32_t m, nm;
@@ -115,44 +108,22 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const uint32_t g = bw[q] & bits_to_bytes(cur.m >> (4 * q));
-            if (kPass == 1 && jm.near) {
-                uint32_t u[4];
-                int32_t v[4];
-                join_near(jm, aw[q], g, kHeadMagic, u);
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    v[k] = __viaddmax_s32((int32_t)__float_as_uint(__fmaf_rn(__uint_as_float(u[k]), scale, rest)), -(int32_t)kHeadMagic, -127);
-                cw[q] = pack4_sat(v[0], v[1], v[2], v[3]);
-            } else if (!jm.wide) {
-                int32_t s32[4];
-                join_narrow(jm, aw[q], g, s32);
-                if (kPass == 0) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const uint32_t v = (uint32_t)abs(s32[k]);
-                        mx32 = max(mx32, v);
-                        if (kNext && ((nm >> (4 * q + k)) & 1u)) mxm32 = max(mxm32, v);
-                    }
-                } else {
-                    cw[q] = fast ? sq_pack4_shr(s32, sh, half_m1, lo)
-                                 : pack4_sat(sq_code32(s32[0], t), sq_code32(s32[1], t), sq_code32(s32[2], t), sq_code32(s32[3], t));
-                }
-            } else {
-                const int av[4] = {sbyte<0>(aw[q]), sbyte<1>(aw[q]), sbyte<2>(aw[q]), sbyte<3>(aw[q])};
-                const int bv[4] = {sbyte<0>(g), sbyte<1>(g), sbyte<2>(g), sbyte<3>(g)};
-                int c[4];
+            uint32_t u[4];
+            if (kPass == 0) {
+                join_sums(jm.pair, aw[q], g, 0u, u);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const long long s = join_one(av[k], bv[k], j);
-                    if (kPass == 0) {
-                        const unsigned long long u = (unsigned long long)(s < 0 ? -s : s);
-                        mx = u > mx ? u : mx;
-                        if (kNext && ((nm >> (4 * q + k)) & 1u)) mxm = u > mxm ? u : mxm;
-                    } else {
-                        c[k] = sq_code64(s, t);
-                    }
+                    const uint32_t v = (uint32_t)abs((int32_t)u[k]);
+                    mx32 = max(mx32, v);
+                    if (kNext && ((nm >> (4 * q + k)) & 1u)) mxm32 = max(mxm32, v);
                 }
-                if (kPass == 1) cw[q] = pack4_sat(c[0], c[1], c[2], c[3]);
+            } else {
+                int32_t v[4];
+                join_sums(jc.pair, aw[q], g, kHeadMagic, u);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    v[k] = __viaddmax_s32((int32_t)__float_as_uint(__fmaf_rn(__uint_as_float(u[k]), jc.scale, jc.rest)), -(int32_t)kHeadMagic, -127);
+                cw[q] = pack4_sat(v[0], v[1], v[2], v[3]);
             }
         }
         if (kPass == 1) {
@@ -179,11 +150,12 @@ __global__ void join_kernel(const int8_t *__restrict__ a, const int32_t *a_exp, 
     }
     ptx::grid_dep_launch();
     if (kPass == 0) {
-        mx = block_max_u64(mx > mx32 ? mx : (unsigned long long)mx32);
-        if (kNext) mxm = block_max_u64(mxm > mxm32 ? mxm : (unsigned long long)mxm32);
+        mx32 = block_max_u32(mx32);
+        __syncthreads();
+        if (kNext) mxm32 = block_max_u32(mxm32);
         if (threadIdx.x == 0) {
-            if (mx) atomicMax(&dev->absmax_u64, mx);
-            if (kNext && mxm) atomicMax(&dev->absmax2_u64, mxm);
+            if (mx32) atomicMax(&dev->absmax_u64, join_magnitude(jm, mx32));
+            if (kNext && mxm32) atomicMax(&dev->absmax2_u64, join_magnitude(jm, mxm32));
         }
     } else {
         long long v[3] = {sum, s1, s2};

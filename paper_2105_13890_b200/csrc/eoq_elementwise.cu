@@ -519,13 +519,8 @@ __global__ void sq_i32_kernel(const void *__restrict__ src_any, const int32_t *s
     }
     long long sum = 0, s1 = 0, s2 = 0;
     const int sh = t - 7;
-    JoinShift js = {0, 0, 0};
     JoinMul jm = {};
-    unsigned long long jmx = 0, jmxm = 0;
-    if (kJoin) {
-        js = join_shift(p0, __ldg(join.b_exp));
-        jm = join_mul(js);
-    }
+    if (kJoin) jm = join_mul(join_shift(p0, __ldg(join.b_exp)));
     // the maximum bounds every element, so |a| + 2^(sh-1) cannot wrap as long as M + M / 2^7 < 2^31
     const bool fast = sh >= 1 && M < 0x7e000000u;
     const int32_t half_m1 = fast ? (1 << (sh - 1)) - 1 : 0, lo = fast ? -(127 << sh) : 0;
@@ -557,33 +552,15 @@ __global__ void sq_i32_kernel(const void *__restrict__ src_any, const int32_t *s
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const uint32_t g = bw[q] & bits_to_bytes(cur.gate >> (4 * q)), m = cur.nm >> (4 * q);
-                if (!jm.wide) {
-                    int32_t v[4];
-                    if (jm.near) {
-                        uint32_t u[4];
-                        join_near(jm, cw[q], g, 0u, u);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) v[k] = (int32_t)u[k];
-                    } else {
-                        join_narrow(jm, cw[q], g, v);
-                    }
-                    const uint32_t u0 = (uint32_t)abs(v[0]), u1 = (uint32_t)abs(v[1]), u2 = (uint32_t)abs(v[2]), u3 = (uint32_t)abs(v[3]);
-                    jm32 = max(max(jm32, u0), max(u1, max(u2, u3)));
-                    if (m & 1u) jmm32 = max(jmm32, u0);
-                    if (m & 2u) jmm32 = max(jmm32, u1);
-                    if (m & 4u) jmm32 = max(jmm32, u2);
-                    if (m & 8u) jmm32 = max(jmm32, u3);
-                } else {
-                    const int bv[4] = {sbyte<0>(g), sbyte<1>(g), sbyte<2>(g), sbyte<3>(g)};
-                    const int cv[4] = {sbyte<0>(cw[q]), sbyte<1>(cw[q]), sbyte<2>(cw[q]), sbyte<3>(cw[q])};
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const long long v = join_one(cv[k], bv[k], js);
-                        const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
-                        jmx = u > jmx ? u : jmx;
-                        if (m & (1u << k)) jmxm = u > jmxm ? u : jmxm;
-                    }
-                }
+                uint32_t u[4];
+                join_sums(jm.pair, cw[q], g, 0u, u);
+                const uint32_t u0 = (uint32_t)abs((int32_t)u[0]), u1 = (uint32_t)abs((int32_t)u[1]), u2 = (uint32_t)abs((int32_t)u[2]),
+                               u3 = (uint32_t)abs((int32_t)u[3]);
+                jm32 = max(max(jm32, u0), max(u1, max(u2, u3)));
+                if (m & 1u) jmm32 = max(jmm32, u0);
+                if (m & 2u) jmm32 = max(jmm32, u1);
+                if (m & 4u) jmm32 = max(jmm32, u2);
+                if (m & 8u) jmm32 = max(jmm32, u3);
             }
         }
         if (kNext) {
@@ -631,11 +608,12 @@ __global__ void sq_i32_kernel(const void *__restrict__ src_any, const int32_t *s
     }
     if (kJoin) {
         // the join's second pass (the next kernel on the stream) reads these cells and puts them back to zero
-        jmx = block_max_u64(jmx > jm32 ? jmx : (unsigned long long)jm32);
-        jmxm = block_max_u64(jmxm > jmm32 ? jmxm : (unsigned long long)jmm32);
+        jm32 = block_max_u32(jm32);
+        __syncthreads();
+        jmm32 = block_max_u32(jmm32);
         if (threadIdx.x == 0) {
-            if (jmx) atomicMax(&dev->absmax_u64, jmx);
-            if (jmxm) atomicMax(&dev->absmax2_u64, jmxm);
+            if (jm32) atomicMax(&dev->absmax_u64, join_magnitude(jm, jm32));
+            if (jmm32) atomicMax(&dev->absmax2_u64, join_magnitude(jm, jmm32));
         }
     }
     if (last) {

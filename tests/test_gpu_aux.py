@@ -1,5 +1,5 @@
 """The glue entry points (eoq_aux_*) one by one against the oracle, element by element: pooling over several window
-geometries and ragged image sizes, the error join over exponent gaps that exercise the narrow path, the 64-bit path
+geometries and ragged image sizes, the error join over exponent gaps on both sides of those where another form of the sums is taken
 and the dropping rule, the float head bit for bit, and the error it hands back."""
 import numpy as np
 import pytest
@@ -112,7 +112,7 @@ def test_avgpool_sum(n, hw, c):
 @pytest.mark.parametrize("pa,pb", [(-12, -12), (-11, -14), (-14, -11), (-10, -33), (-5, -40), (-40, -5), (-20, -51), (-52, -20)])
 @pytest.mark.parametrize("gated", [False, True])
 def test_join(pa, pb, gated):
-    """Equal exponents, small gaps (32-bit path), gaps above 23 octaves (64-bit path) and above 31 (the smaller
+    """Equal exponents, small gaps, gaps above 23 octaves and above 31 (the smaller
     operand is dropped), with and without the gate bits of operand b."""
     hd = G.handle()
     shape = (3, 9, 7, 48)                      # 9072 codes: whole 16-code groups, several blocks, a ragged tail
@@ -129,10 +129,33 @@ def test_join(pa, pb, gated):
     assert eoq.eoq_last_status(hd) == 0
 
 
+@pytest.mark.parametrize("gap", [0, 1, 7, 8, 9, 13, 14, 15, 16, 17, 22, 23, 24, 30, 31, 32, 40])
+@pytest.mark.parametrize("most", [0, 1, 2, 90, 91, 127, 128])
+def test_join_of_every_pair_of_codes(gap, most):
+    """All pairs of a code of at most `most` at the higher exponent and any code at the lower one, at the distances where the sums are
+    formed in another way; either operand may be the higher one.  (-128 is no code of Q_e, but the call takes it.)"""
+    hd = G.handle()
+    high, low = np.meshgrid(np.arange(-most, min(most, 127) + 1), np.arange(-128, 128), indexing="ij")
+    n = (high.size + 15) // 16 * 16
+    high, low = (np.resize(v.astype(np.int8).ravel(), n) for v in (high, low))
+    mask01 = synth.bits((n,), 8440 + gap, most, 0.5)
+    for a, pa, b, pb in ((high, -40 + gap, low, -40), (low, -40, high, -40 + gap)):
+        S, p = oracle.join(a, pa, b, pb, None)
+        codes, p_out, _ = oracle.sq_int(S, p)
+        want_e3, want_p3, want_s1, _, _ = oracle.err_prescale(codes.astype(np.int8), p_out, mask01, None, 97)
+        out, pout, ssum, e3, p3, s1 = G.zeros((n,), torch.int8), G.zeros(1, torch.int32), G.zeros(1, torch.int64), G.zeros((n,), torch.int8), G.zeros(1, torch.int32), G.zeros(1, torch.int64)
+        eoq.eoq_aux_join_head(hd, G.dev(a), i32(pa), G.dev(b), i32(pb), None, n, out, pout, ssum, G.dev(G.pack_mask(mask01)), None, i32(97),
+                              e3, p3, s1, None)
+        torch.cuda.synchronize()
+        eoq.eoq_last_status(hd)   # (all codes zero is flagged)
+        assert np.array_equal(G.host(out), codes) and pout.item() == p_out and ssum.item() == int(codes.astype(np.int64).sum())
+        assert np.array_equal(G.host(e3), want_e3) and p3.item() == want_p3 and s1.item() == want_s1
+
+
 @pytest.mark.parametrize("pa,pb", [(-12, -12), (-11, -14), (-10, -36), (-40, -5)])
 @pytest.mark.parametrize("gamma,with_x2", [(118, True), (128, False), (-77, True)])
 def test_join_with_the_consumer_error_head_fused(pa, pb, gamma, with_x2):
-    """eoq_aux_join_head against the oracle's join followed by its error head (both 32- and 64-bit paths of the join)."""
+    """eoq_aux_join_head against the oracle's join followed by its error head (near and far exponents)."""
     hd = G.handle()
     shape = (3, 9, 7, 48)
     a = synth.normal_codes(shape, 8450, 0)
@@ -253,8 +276,8 @@ def test_dgrad_head_refuses_the_compact_strided_1x1_case():
 @pytest.mark.parametrize("n,h,w,c_in,c_out,k,stride,pad", DGRADS)
 @pytest.mark.parametrize("pb,gated,with_head", [(-17, True, True), (-20, False, True), (-50, True, False), (-3, True, True)])
 def test_dgrad_join_and_head_in_one_call(n, h, w, c_in, c_out, k, stride, pad, pb, gated, with_head):
-    """eoq_conv_dgrad_join_head against the oracle's dgrad + Q_e, join + Q_e and error head (join exponents that take the
-    32-bit path, the 64-bit path and the dropping rule in both directions)."""
+    """eoq_conv_dgrad_join_head against the oracle's dgrad + Q_e, join + Q_e and error head (near and far
+    exponents of the join and the dropping rule in both directions)."""
     hd = G.handle()
     d = ConvDesc(n, h, w, c_in, c_out, k, k, stride, pad)
     gd = G.gdesc(d)
