@@ -141,15 +141,17 @@ class ChainedStep:
         ws = max(ws, n * self.c_last * 4)
         self.workspace = torch.empty(ws, dtype=torch.uint8, device=dev)
         dev_index = dev.index if dev.index is not None else 0
-        self.h_sides = [eoq.eoq_create(dev_index) for _ in range(side_streams + 1)]   # the last: finishing and updating stages
-        self.workspace_sides = [torch.empty(ws, dtype=torch.uint8, device=dev) for _ in range(side_streams)]
+        # weight gradients, projections (`branch`), and the last: finishing and updating stages
+        self.h_sides = [eoq.eoq_create(dev_index) for _ in range(side_streams + 2)]
+        self.workspace_sides = [torch.empty(ws, dtype=torch.uint8, device=dev) for _ in range(side_streams + 1)]
         # a third of the SMs for each of the weight-gradient GEMMs, so that the error chain finds free ones (ResNet-18 step at
         # batch 64: 1576 us with all SMs, 1502 with half, 1474 with a third, 1480 with a quarter; at batch 13: 769, 727, 717, 715)
         third = torch.cuda.get_device_properties(dev).multi_processor_count // 3
-        for hs in self.h_sides:
-            eoq.eoq_set_gemm_ctas(hs, third)
-        self.sides = [torch.cuda.Stream(device=dev) for _ in range(side_streams + 1)]
-        self.wgrad_sides = side_streams
+        self.wgrad_sides = self.branch = side_streams
+        for k, hs in enumerate(self.h_sides):
+            if k != self.branch:
+                eoq.eoq_set_gemm_ctas(hs, third)
+        self.sides = [torch.cuda.Stream(device=dev, priority=-1 if k == self.branch else 0) for k in range(side_streams + 2)]
         if finish_together:
             for u in self.units:
                 u.wgrad_ws = torch.empty(max(256, eoq.eoq_workspace_size(u.desc, eoq.EOQ_PASS_WGRAD)), dtype=torch.uint8, device=dev)
@@ -215,11 +217,25 @@ class ChainedStep:
         if self.pool:
             k, s, p = self.pool
             eoq.eoq_aux_maxpool_fwd(h, stem.x5, fl.n, fl.ho, fl.wo, fl.c_out, k, s, p, self.pooled, self.pool_arg)
+        # a projection runs beside the block's first unit, forward and backward: on a stream and a handle of its own
+        branch = self.sides[self.branch] if overlap else main
+        h_br, ws_br = (self.h_sides[self.branch], self.workspace_sides[self.branch]) if overlap else (h, ws)
+
+        work = self.sides[:self.branch] + self.sides[self.branch + 1:]   # (what runs on `branch` is met by each block)
+
+        def meet(stream, other) -> None:
+            if overlap:
+                stream.wait_stream(other)
+
         for blk in self.blocks:
             a, b, pr = blk.a, blk.b, blk.proj
+            if pr:
+                meet(branch, main)
             eoq.eoq_conv_fwd_dev(h, a.desc, a.x0, None, a.scal, a.w, a.prep, None, True, a.x5, None, a.mask)
             if pr:
-                eoq.eoq_conv_fwd_dev(h, pr.desc, pr.x0, None, pr.scal, pr.w, pr.prep, None, False, pr.x5, None, None)
+                with torch.cuda.stream(branch):
+                    eoq.eoq_conv_fwd_dev(h_br, pr.desc, pr.x0, None, pr.scal, pr.w, pr.prep, None, False, pr.x5, None, None)
+                meet(main, branch)
             eoq.eoq_conv_fwd_dev(h, b.desc, b.x0, None, b.scal, b.w, b.prep, blk.shortcut, True, b.x5, b.x2, b.mask)
         last = self.blocks[-1].b
         n = fl.n
@@ -242,11 +258,11 @@ class ChainedStep:
             else:
                 eoq.eoq_conv_wgrad_dev(hh, u.desc, u.e3, u.e3_exp, u.x0, b1_dev, u.g, u.g_exp, wsp)
 
-        def wgrad(u: UnitBuffers, b1_dev) -> None:
+        def wgrad(u: UnitBuffers, b1_dev, behind=main) -> None:
             if overlap:
                 k = side_no[0] % self.wgrad_sides
                 side_no[0] += 1
-                self.sides[k].wait_stream(main)
+                self.sides[k].wait_stream(behind)
                 with torch.cuda.stream(self.sides[k]):
                     wgrad_call(self.h_sides[k], u, b1_dev, self.workspace_sides[k])
             else:
@@ -277,7 +293,7 @@ class ChainedStep:
                     update(us, h, False)
                 return
             fin, h_fin = self.sides[-1], self.h_sides[-1]
-            for side in self.sides[:-1]:
+            for side in self.sides[:self.wgrad_sides]:
                 fin.wait_stream(side)
             with torch.cuda.stream(fin):
                 finish(us, h_fin)
@@ -300,15 +316,20 @@ class ChainedStep:
             if not head_done:
                 eoq.eoq_err_prescale_dev(h, e_out, e_exp, b.mask, b.x2, b.n_out, b.scal[1:2], b.e3, b.e3_exp, b.sum_e1, b.sum_e1x2)
             wgrad(b, b.scal[0:1])
+            if pr:
+                # the error entering the shortcut is e1 of unit B: e_out gated by unit B's ReLU mask
+                meet(branch, main)
+                with torch.cuda.stream(branch):
+                    eoq.eoq_err_prescale_dev(h_br, e_out, e_exp, b.mask, None, pr.n_out, self.c128, pr.e3, pr.e3_exp, pr.sum_e1, None)
             # error back through unit B; the error head of unit A rides on its Q_e
             eoq.eoq_conv_dgrad_head(h, b.desc, b.e3, b.e3_exp, b.w, b.e4, b.e4_exp, b.sum_e4, a.mask, None, a.scal[1:2], a.e3,
                                     a.e3_exp, a.sum_e1, None, ws)
             wgrad(a, a.scal[0:1])
             if pr:
-                # the error entering the shortcut is e1 of unit B: e_out gated by unit B's ReLU mask
-                eoq.eoq_err_prescale_dev(h, e_out, e_exp, b.mask, None, pr.n_out, self.c128, pr.e3, pr.e3_exp, pr.sum_e1, None)
-                wgrad(pr, a.scal[0:1])
-                eoq.eoq_conv_dgrad(h, pr.desc, pr.e3, pr.e3_exp, pr.w, pr.e4, pr.e4_exp, pr.sum_e4, None, ws)
+                wgrad(pr, a.scal[0:1], branch)
+                with torch.cuda.stream(branch):
+                    eoq.eoq_conv_dgrad(h_br, pr.desc, pr.e3, pr.e3_exp, pr.w, pr.e4, pr.e4_exp, pr.sum_e4, None, ws_br)
+                meet(main, branch)
                 j_b, j_b_exp, j_mask = pr.e4, pr.e4_exp, None
             else:
                 j_b, j_b_exp, j_mask = e_out, e_exp, b.mask
@@ -354,13 +375,13 @@ class ChainedStep:
             wgrad_call(h, stem, None, ws)
             finish([stem], h)
             if overlap:
-                for side in self.sides:
+                for side in work:
                     main.wait_stream(side)
             update(pending + [stem], h, True)
             return
         wgrad(stem, None)
         if overlap:
-            for side in self.sides:
+            for side in work:
                 main.wait_stream(side)
         scalar_update(h)
         eoq.eoq_update_dev(h, [u.w for u in self.units], [u.g for u in self.units], [u.g_exp for u in self.units],
