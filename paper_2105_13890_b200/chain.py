@@ -251,8 +251,10 @@ class ChainedStep:
 
         side_no = [0]
 
-        def wgrad_call(hh, u: UnitBuffers, b1_dev, wsp) -> None:
-            if self.finish_together:
+        def wgrad_call(hh, u: UnitBuffers, b1_dev, wsp, whole=False) -> None:
+            if whole:
+                eoq.eoq_conv_wgrad_dev(hh, u.desc, u.e3, u.e3_exp, u.x0, b1_dev, u.g, u.g_exp, u.wgrad_ws)
+            elif self.finish_together:
                 u.b1_dev = b1_dev
                 u.wgrad_parts = eoq.eoq_conv_wgrad_gemm(hh, u.desc, u.e3, u.e3_exp, u.x0, u.wgrad_ws)
             else:
@@ -264,7 +266,7 @@ class ChainedStep:
                 side_no[0] += 1
                 self.sides[k].wait_stream(behind)
                 with torch.cuda.stream(self.sides[k]):
-                    wgrad_call(self.h_sides[k], u, b1_dev, self.workspace_sides[k])
+                    wgrad_call(self.h_sides[k], u, b1_dev, self.workspace_sides[k], front_block)
             else:
                 wgrad_call(h, u, b1_dev, ws)
 
@@ -304,6 +306,9 @@ class ChainedStep:
         e_out, e_exp = self.e_head, self.e_head_exp
         head_done = False   # the error head of this block's last unit already ran inside the join of the block behind it
         pending = []        # units whose weight-gradient GEMM is issued and not yet finished
+        # the gradients of the front block end the step: they are finished one by one, their b1 sums beside their GEMMs, and what
+        # the blocks of its stage behind it left is finished beside the block
+        front_block, front = False, []
         stage = None
         for i in reversed(range(len(self.blocks))):
             blk = self.blocks[i]
@@ -312,7 +317,12 @@ class ChainedStep:
                 stage_done(pending, False)
                 pending = []
             stage = a.layer.name.split(".")[0]
-            pending += [b, a] + ([pr] if pr else [])
+            if i == 0 and overlap and self.finish_together:
+                front_block, front = True, [b, a] + ([pr] if pr else [])
+                if pending:
+                    stage_done(pending, True)
+            else:
+                pending += [b, a] + ([pr] if pr else [])
             if not head_done:
                 eoq.eoq_err_prescale_dev(h, e_out, e_exp, b.mask, b.x2, b.n_out, b.scal[1:2], b.e3, b.e3_exp, b.sum_e1, b.sum_e1x2)
             wgrad(b, b.scal[0:1])
@@ -346,7 +356,8 @@ class ChainedStep:
                                              blk.e_in_exp, blk.sum_join, workspace=ws)
                 head_done = False
             e_out, e_exp = blk.e_in, blk.e_in_exp
-        stage_done(pending, True)
+        if not front_block:
+            stage_done(pending, True)
         if self.pool:
             k, s, p = self.pool
             # pool backward and the first layer's error head in one pair of kernels; the error between them (51 MB at
@@ -367,7 +378,8 @@ class ChainedStep:
         if self.finish_together:
             # the first layer's weight gradient ends the chain; the scalars are updated beside it, behind the last reader of b1
             if overlap:
-                self.sides[-1].wait_stream(main)
+                for side in [main] + self.sides[:self.wgrad_sides]:
+                    self.sides[-1].wait_stream(side)
                 with torch.cuda.stream(self.sides[-1]):
                     scalar_update(self.h_sides[-1])
             else:
@@ -377,7 +389,7 @@ class ChainedStep:
             if overlap:
                 for side in work:
                     main.wait_stream(side)
-            update(pending + [stem], h, True)
+            update(pending + front + [stem], h, True)
             return
         wgrad(stem, None)
         if overlap:
