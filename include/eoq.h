@@ -502,8 +502,8 @@ EOQ_API int eoq_probe_mma_i8(eoq_handle_t handle, int n_cols, int iters, int lau
  * reports; the format is not an interface).  buf receives at most buf_bytes bytes, NUL-terminated. */
 EOQ_API int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *desc, int pass, char *buf, size_t buf_bytes);
 
-/* Self-test of the bounded device waits: the next eoq_err_prescale / eoq_err_prescale_dev call on this handle that
- * takes the one-kernel path waits at its grid-wide barrier for one block more than exists, with a limit of 2048
+/* Self-test of the bounded device waits: the next eoq_err_prescale / eoq_err_prescale_dev call on this handle
+ * waits, in the place of its work, for one arrival more than there are, with a limit of 2048
  * polls (about 0.2 ms).  The wait runs out, the kernel raises EOQ_DEV_TIMEOUT, writes no output and returns;
  * eoq_last_status then reports the bit and puts the handle's reduction cells back to zero.  Nothing faults or
  * hangs; one call only, then the handle behaves normally again. */

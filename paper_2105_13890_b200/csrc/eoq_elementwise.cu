@@ -674,63 +674,74 @@ __global__ void sq_sums_scatter_kernel(const uint16_t *__restrict__ src, const i
 
 // ------------------------------------------------------------------ head of the error chain
 
-// Pass 1: max |e1| and the sums behind g_b2 and g_gamma, with e1 = e0 * [x4 > 0].
-__global__ void prescale_reduce_kernel(const int8_t *__restrict__ e0, const uint8_t *__restrict__ mask,
-                                       const int16_t *__restrict__ x2, size_t n16, DeviceState *dev)
-{
-    uint32_t mx4 = 0;  // four running byte maxima of |e1|
-    long long s1 = 0, s2 = 0;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    // four independent 16-element groups per iteration keep enough loads in flight to cover DRAM latency
-    for (size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n16; i0 += 4 * stride) {
-        int4 ev[4];
-        uint32_t mv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t i = i0 + u * stride;
-            const bool in = i < n16;
-            ev[u] = in ? __ldg(reinterpret_cast<const int4 *>(e0) + i) : make_int4(0, 0, 0, 0);
-            mv[u] = (in && mask) ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(mask) + i) : 0xffffu;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint32_t w[4] = {(uint32_t)ev[u].x, (uint32_t)ev[u].y, (uint32_t)ev[u].z, (uint32_t)ev[u].w};
-            int a1 = 0;
-            uint32_t e1w[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                e1w[q] = w[q] & bits_to_bytes(mv[u] >> (4 * q));  // e1 = e0 * [x4 > 0], four codes per word
-                mx4 = __vmaxu4(mx4, __vabsss4(e1w[q]));
-                a1 = __dp4a((int)e1w[q], 0x01010101, a1);
-            }
-            s1 += a1;
-            if (x2) {
-                const size_t i = i0 + u * stride;
-                if (i < n16) {
-                    const int4 lo = __ldg(reinterpret_cast<const int4 *>(x2) + 2 * i);
-                    const int4 hi = __ldg(reinterpret_cast<const int4 *>(x2) + 2 * i + 1);
-                    const int16_t *pl = reinterpret_cast<const int16_t *>(&lo), *ph = reinterpret_cast<const int16_t *>(&hi);
-                    const int8_t *eb = reinterpret_cast<const int8_t *>(e1w);
-                    int a2 = 0;  // |e1 * x2| < 2^22, 16 terms
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) a2 += (int)eb[k] * pl[k] + (int)eb[8 + k] * ph[k];
-                    s2 += a2;
-                }
-            }
-        }
+// Two chained passes over e0 and the mask, the second out of the L2.  Bound by launch latency up to a million codes, then by the
+// latency of the loads: a thread's next group travels while it works on one.  One cooperative kernel that kept e1 in registers read
+// everything once, but cannot be chained to its predecessor: 0.26, 1.6, 6.4 and 12.8 M codes with x2 took it 8.1, 8.2, 9.6 and 13.4
+// us in a row of calls, the two 4.1, 4.8, 7.7 and 11.2 (backward of 512 channels 7 x 7 at batch 64 58.6 -> 52.2 us).
+
+// largest |code| of a byte word, running (a code of -128 counts as 127)
+struct HeadMax {
+    uint32_t mx = 0, mn = 0;   // packed 16-bit halves
+    __device__ __forceinline__ void add(uint32_t w)
+    {
+        uint32_t even, odd;   // sign-extended by one permute per two codes
+        asm("prmt.b32 %0, %1, %1, 0xA280;" : "=r"(even) : "r"(w));
+        asm("prmt.b32 %0, %1, %1, 0xB391;" : "=r"(odd) : "r"(w));
+        mx = __vimax3_s16x2(mx, even, odd);
+        mn = __vimin3_s16x2(mn, even, odd);
     }
-    uint32_t mx = max(max(mx4 & 0xffu, (mx4 >> 8) & 0xffu), max((mx4 >> 16) & 0xffu, mx4 >> 24));
-    mx = (uint32_t)block_max_u64(mx);
-    s1 = block_sum_i64(s1);
-    s2 = block_sum_i64(s2);
+    __device__ __forceinline__ uint32_t value() const
+    {
+        const int hi = max((int)(int16_t)mx, (int)mx >> 16), lo = min((int)(int16_t)mn, (int)mn >> 16);
+        return (uint32_t)min(max(hi, -lo), 127);
+    }
+};
+
+// Pass 1: max |e1| and the sums behind g_b2 and g_gamma, with e1 = e0 * [x4 > 0].
+__global__ void __launch_bounds__(kThreads)
+prescale_reduce_kernel(const int8_t *__restrict__ e0, const uint8_t *__restrict__ mask, const int16_t *__restrict__ x2, size_t n16,
+                       DeviceState *dev)
+{
+    ptx::grid_dep_wait_launch_small();
+    HeadMax most;
+    long long v[2] = {0, 0};
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    struct Group {
+        int4 e;
+        uint32_t m;
+    } cur = {};
+    auto load = [&](size_t i) {
+        if (x2) ptx::prefetch_l1(x2 + i * 16);
+        return Group{__ldg(reinterpret_cast<const int4 *>(e0) + i), mask ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(mask) + i) : 0xffffu};
+    };
+    if (i < n16) cur = load(i);
+    for (; i < n16; i += stride) {
+        Group ahead = {};
+        if (i + stride < n16) ahead = load(i + stride);
+        const uint32_t w[4] = {(uint32_t)cur.e.x, (uint32_t)cur.e.y, (uint32_t)cur.e.z, (uint32_t)cur.e.w};
+        uint32_t e1[4];
+        int a1 = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            e1[q] = w[q] & bits_to_bytes(cur.m >> (4 * q));
+            most.add(e1[q]);
+            a1 = __dp4a((int)e1[q], 0x01010101, a1);
+        }
+        v[0] += a1;
+        if (x2) v[1] += dot16_s8_s16(e1, reinterpret_cast<const int4 *>(x2) + 2 * i);
+        cur = ahead;
+    }
+    ptx::grid_dep_launch();
+    const uint32_t mx = block_max_u32(most.value());
+    block_sums_i64(v);
     if (threadIdx.x == 0) {
         if (mx) atomicMax(&dev->absmax_u32, mx);
-        if (s1) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)s1);
-        if (s2) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum1), (unsigned long long)s2);
+        if (v[0]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)v[0]);
+        if (v[1]) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum1), (unsigned long long)v[1]);
     }
 }
 
-// Pass 2: e3 = Q_e(gamma * e1) under the reduced maximum.
 // gamma of a launch: the host value, or the code read from device memory (clamped to 16 bits, EOQ_DEV_RANGE raised)
 __device__ __forceinline__ int32_t load_gamma(int32_t gamma_c, const int32_t *gamma_dev, DeviceState *dev)
 {
@@ -743,183 +754,83 @@ __device__ __forceinline__ int32_t load_gamma(int32_t gamma_c, const int32_t *ga
     return g;
 }
 
-__global__ void prescale_apply_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp,
-                                      const uint8_t *__restrict__ mask, size_t n16, int32_t gamma_c,
-                                      const int32_t *gamma_dev, int8_t *e3, int32_t *e3_exp, long long *sum_e1,
-                                      long long *sum_e1x2, DeviceState *dev)
+// Pass 2: e3 = Q_e(gamma * e1) under the reduced maximum.
+__global__ void __launch_bounds__(kThreads)
+prescale_apply_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, const uint8_t *__restrict__ mask, size_t n16, int32_t gamma_c,
+                      const int32_t *gamma_dev, int8_t *e3, int32_t *e3_exp, long long *sum_e1, long long *sum_e1x2, DeviceState *dev)
 {
+    ptx::grid_dep_wait_launch_small();
+    __shared__ uint32_t max_s;   // (the protocol of sq_i32_kernel)
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    struct Group {
+        int4 e;
+        uint32_t m;
+    } cur = {};
+    auto load = [&](size_t i) {
+        return Group{__ldg(reinterpret_cast<const int4 *>(e0) + i), mask ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(mask) + i) : 0xffffu};
+    };
+    if (i < n16) cur = load(i);
+    if (threadIdx.x == 0) max_s = *reinterpret_cast<volatile unsigned *>(&dev->absmax_u32);
     gamma_c = load_gamma(gamma_c, gamma_dev, dev);
-    const uint32_t M = dev->absmax_u32 * (uint32_t)abs(gamma_c);  // max |gamma * e1| < 2^7 * 2^15
+    __syncthreads();
+    const uint32_t M = max_s * (uint32_t)abs(gamma_c);  // max |gamma * e1| < 2^7 * 2^15
     const int t = M ? round_log2_u32(M) : 7;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const int p_in = *e0_exp - 7;
-        *e3_exp = M ? p_in + t - 7 : p_in;
-        if (!M) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-        if (sum_e1) *sum_e1 = dev->sum0;
-        if (sum_e1x2) *sum_e1x2 = dev->sum1;
+    bool last = false;
+    if (threadIdx.x == 0) {
+        if (blockIdx.x == 0) {
+            const int p_in = *e0_exp - 7;
+            *e3_exp = M ? p_in + t - 7 : p_in;
+            if (!M) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
+            if (sum_e1) *sum_e1 = *reinterpret_cast<volatile long long *>(&dev->sum0);
+            if (sum_e1x2) *sum_e1x2 = *reinterpret_cast<volatile long long *>(&dev->sum1);
+            __threadfence();   // read before the block counts as a reader
+        }
+        last = last_reader(dev);
     }
-    // R(v * 2^(7-t)) for v = gamma * e1 (|v| < 2^22) on the floating-point pipe: kMagic + v read as a float is
+    // R(v * 2^(7-t)) for v = gamma * e1 (|v| < 2^22) on the floating-point pipe: kHeadMagic + v read as a float is
     // 1.5 * 2^23 + v exactly; one fused multiply-add forms 1.5 * 2^23 + v * 2^(7-t) (the products are exact, the sum
     // is rounded once, to nearest even at unit spacing), so the low bits of the result are the rounded quotient.
     // For t < 7 the scaling is a left shift and nothing is rounded; either way |result| < 2^22 keeps the binade.
-    constexpr uint32_t kMagic = 0x4B400000u;  // 1.5 * 2^23
-    const float scale = __int_as_float((127 + 7 - t) << 23);  // 2^(7-t), t in [0, 22]
-    const float rest = 12582912.0f - 12582912.0f * scale;  // exact: a multiple of a power of two below 2^31
-    const uint32_t g = (uint32_t)gamma_c;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n16; i0 += 4 * stride) {
-        int4 ev[4];
-        uint32_t mv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t i = i0 + u * stride;
-            const bool in = i < n16;
-            ev[u] = in ? __ldg(reinterpret_cast<const int4 *>(e0) + i) : make_int4(0, 0, 0, 0);
-            mv[u] = (in && mask) ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(mask) + i) : 0xffffu;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t i = i0 + u * stride;
-            if (i >= n16) continue;
-            const uint32_t w[4] = {(uint32_t)ev[u].x, (uint32_t)ev[u].y, (uint32_t)ev[u].z, (uint32_t)ev[u].w};
-            int c[16];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t e1w = w[q] & bits_to_bytes(mv[u] >> (4 * q));  // e1 = e0 * [x4 > 0], four codes
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int32_t e1 = (int32_t)(int8_t)(e1w >> (8 * k));
-                    const uint32_t biased = g * (uint32_t)e1 + kMagic;
-                    const uint32_t r = __float_as_uint(__fmaf_rn(__uint_as_float(biased), scale, rest));
-                    c[4 * q + k] = clampi((int32_t)(r - kMagic), -127, 127);
-                }
-            }
-            reinterpret_cast<int4 *>(e3)[i] =
-                make_int4((int)pack4(c[0], c[1], c[2], c[3]), (int)pack4(c[4], c[5], c[6], c[7]),
-                          (int)pack4(c[8], c[9], c[10], c[11]), (int)pack4(c[12], c[13], c[14], c[15]));
-        }
-    }
-    if (last_block_done(dev)) {
-        dev->absmax_u32 = 0;
-        dev->sum0 = 0;
-        dev->sum1 = 0;
-    }
-}
-
-// Both passes of the error head in one kernel, for tensors small enough that every thread keeps its share of e1
-// (up to kFusedGroups groups of 16 codes) in registers between the passes: e0 and the mask are read once and no
-// second launch is needed.  Between the passes all blocks meet at a grid-wide barrier (a counter in the handle's
-// device state), so the kernel is launched cooperatively: the launch guarantees that all its blocks are resident
-// together.  The wait is bounded like every wait of the library; on timeout the kernel flags it and writes nothing.
-constexpr int kFusedGroups = 6;
-__global__ void __launch_bounds__(kThreads)
-prescale_fused_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, const uint8_t *__restrict__ mask,
-                      const int16_t *__restrict__ x2, size_t n16, int32_t gamma_c, const int32_t *gamma_dev, int8_t *e3,
-                      int32_t *e3_exp, long long *sum_e1, long long *sum_e1x2, DeviceState *dev, unsigned expected_blocks,
-                      uint32_t spin_limit)
-{
-    if (gridDim.x <= kPartSms) ptx::grid_dep_launch();   // (its successor may come up beside it)
-    __shared__ unsigned go_s;
-    __shared__ uint32_t max_s;
-    __shared__ long long total_s[2];
-    gamma_c = load_gamma(gamma_c, gamma_dev, dev);
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t e1w[kFusedGroups][4];
-    uint32_t mx4 = 0;
-    long long s1 = 0, s2 = 0;
-    {
-        int4 ev[kFusedGroups];
-        uint32_t mv[kFusedGroups];
-#pragma unroll
-        for (int u = 0; u < kFusedGroups; ++u) {
-            const size_t i = i0 + u * stride;
-            const bool in = i < n16;
-            ev[u] = in ? __ldg(reinterpret_cast<const int4 *>(e0) + i) : make_int4(0, 0, 0, 0);
-            mv[u] = (in && mask) ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(mask) + i) : 0xffffu;
-        }
-#pragma unroll
-        for (int u = 0; u < kFusedGroups; ++u) {
-            const uint32_t w[4] = {(uint32_t)ev[u].x, (uint32_t)ev[u].y, (uint32_t)ev[u].z, (uint32_t)ev[u].w};
-            int a1 = 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                e1w[u][q] = w[q] & bits_to_bytes(mv[u] >> (4 * q));  // e1 = e0 * [x4 > 0], four codes per word
-                mx4 = __vmaxu4(mx4, __vabsss4(e1w[u][q]));
-                a1 = __dp4a((int)e1w[u][q], 0x01010101, a1);
-            }
-            s1 += a1;
-            const size_t i = i0 + u * stride;
-            if (x2 && i < n16) s2 += dot16_s8_s16(e1w[u], reinterpret_cast<const int4 *>(x2) + 2 * i);
-        }
-    }
-    uint32_t mx = max(max(mx4 & 0xffu, (mx4 >> 8) & 0xffu), max((mx4 >> 16) & 0xffu, mx4 >> 24));
-    mx = block_max_u32(mx);
-    long long sums[2] = {s1, s2};
-    block_sums_i64(sums);
-    s1 = sums[0];
-    s2 = sums[1];
-    if (threadIdx.x == 0) {
-        if (mx) atomicMax(&dev->absmax_u32, mx);
-        if (s1) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum0), (unsigned long long)s1);
-        if (s2) atomicAdd(reinterpret_cast<unsigned long long *>(&dev->sum1), (unsigned long long)s2);
-        // grid-wide barrier: every block's contribution is in the cells once all have arrived
-        __threadfence();
-        atomicAdd(&dev->arrivals, 1u);
-        unsigned ok = 0;
-        // (expected_blocks is the grid size; a larger value, which only the library's self-test passes, makes this
-        // wait run out)
-        for (uint32_t it = 0; it < spin_limit; ++it) {
-            if (*reinterpret_cast<volatile unsigned *>(&dev->arrivals) >= expected_blocks) { ok = 1; break; }
-            __nanosleep(100);
-        }
-        if (!ok) atomicOr(&dev->status, EOQ_DEV_TIMEOUT);
-        __threadfence();
-        go_s = ok;
-        max_s = *reinterpret_cast<volatile unsigned *>(&dev->absmax_u32);
-        total_s[0] = *reinterpret_cast<volatile long long *>(&dev->sum0);
-        total_s[1] = *reinterpret_cast<volatile long long *>(&dev->sum1);
-    }
-    __syncthreads();
-    if (!go_s) return;
-    bool last = false;
-    if (threadIdx.x == 0) last = last_reader(dev);   // the last block to have read the cells clears them at its end
-    const uint32_t M = max_s * (uint32_t)abs(gamma_c);
-    const int t = M ? round_log2_u32(M) : 7;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const int p_in = *e0_exp - 7;
-        *e3_exp = M ? p_in + t - 7 : p_in;
-        if (!M) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
-        if (sum_e1) *sum_e1 = total_s[0];
-        if (sum_e1x2) *sum_e1x2 = total_s[1];
-    }
-    // same rounding as prescale_apply_kernel: R(gamma * e1 * 2^(7-t)) with one FMA
     NextHead nh;
     nh.g = (uint32_t)gamma_c;
-    nh.scale = __int_as_float((127 + 7 - t) << 23);
-    nh.rest = 12582912.0f - 12582912.0f * nh.scale;
-#pragma unroll
-    for (int u = 0; u < kFusedGroups; ++u) {
-        const size_t i = i0 + u * stride;
-        if (i >= n16) continue;
+    nh.scale = __int_as_float((127 + 7 - t) << 23);   // 2^(7-t), t in [0, 22]
+    nh.rest = 12582912.0f - 12582912.0f * nh.scale;   // exact: a multiple of a power of two below 2^31
+    for (; i < n16; i += stride) {
+        Group ahead = {};
+        if (i + stride < n16) ahead = load(i + stride);
+        const uint32_t w[4] = {(uint32_t)cur.e.x, (uint32_t)cur.e.y, (uint32_t)cur.e.z, (uint32_t)cur.e.w};
         uint32_t c3[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) c3[q] = next_head_codes(nh, e1w[u][q]);
+        for (int q = 0; q < 4; ++q) c3[q] = next_head_codes(nh, w[q] & bits_to_bytes(cur.m >> (4 * q)));
         reinterpret_cast<int4 *>(e3)[i] = make_int4((int)c3[0], (int)c3[1], (int)c3[2], (int)c3[3]);
+        cur = ahead;
     }
+    ptx::grid_dep_launch();
     if (last) {
         dev->absmax_u32 = 0;
         dev->sum0 = 0;
         dev->sum1 = 0;
-        dev->arrivals = 0;
     }
 }
 
-// The same in one cluster of up to kHeadCluster blocks, for tensors of that many blocks' shares: the maxima and sums meet in
-// distributed shared memory instead of the handle's cells and a counter, and the launch can be chained to its predecessor, which a
-// cooperative one cannot.  Bound by latency: ResNet-18 step at batch 1 445 -> 437 us, backward of the 48 -> 80 channel strided layer
-// called by itself 45 -> 40.
-constexpr int kHeadCluster = 8;
+// Self-test of the library's bounded waits (eoq_debug_force_wait_timeout): waits for `expected` arrivals of which it makes one, gives up
+// after `spin_limit` polls, flags it and returns; it takes the place of the call's passes, so nothing is written.
+__global__ void wait_self_test_kernel(DeviceState *dev, unsigned expected, uint32_t spin_limit)
+{
+    atomicAdd(&dev->arrivals, 1u);
+    for (uint32_t it = 0; it < spin_limit; ++it) {
+        if (*reinterpret_cast<volatile unsigned *>(&dev->arrivals) >= expected) return;
+        __nanosleep(100);
+    }
+    atomicOr(&dev->status, EOQ_DEV_TIMEOUT);
+}
+
+// The same in one cluster of up to kHeadCluster blocks, for tensors of that many blocks' shares: every thread keeps its share of e1 (up to
+// kHeadGroups groups of 16 codes) in registers between the passes, the maxima and sums meet in distributed shared memory, and one launch
+// does it.  Bound by latency: 4.6 us for 65,536 codes with x2, as long as the two passes take; at 196,608 codes, six groups a thread,
+// 6.3 us and they 4.6.  (It is one launch less where calls are issued one by one.)
+constexpr int kHeadCluster = 8, kHeadGroups = 2;
 __global__ void __launch_bounds__(kThreads)
 prescale_cluster_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, const uint8_t *__restrict__ mask,
                         const int16_t *__restrict__ x2, size_t n16, int32_t gamma_c, const int32_t *gamma_dev, int8_t *e3,
@@ -932,21 +843,21 @@ prescale_cluster_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, co
     gamma_c = load_gamma(gamma_c, gamma_dev, dev);
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t e1w[kFusedGroups][4];
+    uint32_t e1w[kHeadGroups][4];
     uint32_t mx4 = 0;
     long long s1 = 0, s2 = 0;
     {
-        int4 ev[kFusedGroups];
-        uint32_t mv[kFusedGroups];
+        int4 ev[kHeadGroups];
+        uint32_t mv[kHeadGroups];
 #pragma unroll
-        for (int u = 0; u < kFusedGroups; ++u) {
+        for (int u = 0; u < kHeadGroups; ++u) {
             const size_t i = i0 + u * stride;
             const bool in = i < n16;
             ev[u] = in ? __ldg(reinterpret_cast<const int4 *>(e0) + i) : make_int4(0, 0, 0, 0);
             mv[u] = (in && mask) ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(mask) + i) : 0xffffu;
         }
 #pragma unroll
-        for (int u = 0; u < kFusedGroups; ++u) {
+        for (int u = 0; u < kHeadGroups; ++u) {
             const uint32_t w[4] = {(uint32_t)ev[u].x, (uint32_t)ev[u].y, (uint32_t)ev[u].z, (uint32_t)ev[u].w};
             int a1 = 0;
 #pragma unroll
@@ -997,7 +908,7 @@ prescale_cluster_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, co
     nh.scale = __int_as_float((127 + 7 - t) << 23);
     nh.rest = 12582912.0f - 12582912.0f * nh.scale;
 #pragma unroll
-    for (int u = 0; u < kFusedGroups; ++u) {
+    for (int u = 0; u < kHeadGroups; ++u) {
         const size_t i = i0 + u * stride;
         if (i >= n16) continue;
         uint32_t c3[4];
@@ -1287,8 +1198,13 @@ cudaError_t launch_err_prescale(const int8_t *e0, const int32_t *e0_exp, const u
 {
     const size_t n16 = n_el / 16;
     *kernels = 2;
-    const size_t share = (size_t)kThreads * kFusedGroups;
-    if (!hook.fn && !force_timeout && n16 > 0 && n16 <= kHeadCluster * share) {
+    const size_t share = (size_t)kThreads * kHeadGroups;
+    if (force_timeout) {
+        *kernels = 1;
+        wait_self_test_kernel<<<1, 1, 0, s>>>(dev, 2u, 2048u);
+        return cudaGetLastError();
+    }
+    if (!hook.fn && n16 > 0 && n16 <= kHeadCluster * share) {
         // few blocks: one cluster (twice the blocks that its registers need, up to its size: the loads of a block are in turn)
         int blocks = 1;
         while (blocks < kHeadCluster && (size_t)blocks * kThreads * 2 < n16) blocks *= 2;
@@ -1296,43 +1212,11 @@ cudaError_t launch_err_prescale(const int8_t *e0, const int32_t *e0_exp, const u
         return launch_chained_clusters(blocks, prescale_cluster_kernel, blocks, kThreads, 0, s, e0, e0_exp, mask, x2, n16, gamma_c, gamma_dev, e3,
                                        e3_exp, sum_e1, sum_e1x2, dev);
     }
-    // one cooperative kernel when every thread can hold its share of the tensor between the two passes
-    static int blocks_per_sm = -1;
-    static bool coop = false;
-    if (blocks_per_sm < 0) {
-        int dev_id = 0, can = 0, bps = 0;
-        if (cudaGetDevice(&dev_id) == cudaSuccess &&
-            cudaDeviceGetAttribute(&can, cudaDevAttrCooperativeLaunch, dev_id) == cudaSuccess && can &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, prescale_fused_kernel, kThreads, 0) == cudaSuccess && bps > 0) {
-            coop = true;
-            blocks_per_sm = bps > 4 ? 4 : bps;  // leaves room on every SM for kernels of other streams
-        } else {
-            blocks_per_sm = 0;
-        }
-    }
-    const size_t max_blocks = (size_t)blocks_per_sm * sm_count;
-    const size_t need_blocks = (n16 + (size_t)kThreads * kFusedGroups - 1) / ((size_t)kThreads * kFusedGroups);
-    if (coop && !hook.fn && n16 > 0 && need_blocks <= max_blocks) {
-        // self-test of the bounded wait: one arrival more than there are blocks and a short limit
-        unsigned expected = (unsigned)need_blocks + (force_timeout ? 1u : 0u);
-        uint32_t spin_limit = force_timeout ? 2048u : kSpinLimit;
-        void *args[] = {(void *)&e0, (void *)&e0_exp, (void *)&mask, (void *)&x2, (void *)&n16, (void *)&gamma_c,
-                        (void *)&gamma_dev, (void *)&e3, (void *)&e3_exp, (void *)&sum_e1, (void *)&sum_e1x2, (void *)&dev,
-                        (void *)&expected, (void *)&spin_limit};
-        // (not a chained launch: together with the cooperative attribute that takes about 2 us more than it saves)
-        const cudaError_t e = cudaLaunchCooperativeKernel((const void *)prescale_fused_kernel, dim3((unsigned)need_blocks),
-                                                          dim3(kThreads), args, 0, s);
-        if (e != cudaErrorCooperativeLaunchTooLarge) {
-            *kernels = 1;
-            return e;
-        }
-        (void)cudaGetLastError();  // fewer SMs at hand than at start-up (e.g. a partitioned device): two kernels instead
-    }
-    prescale_reduce_kernel<<<grid_for(n16, sm_count), kThreads, 0, s>>>(e0, mask, x2, n16, dev);
+    const int grid = grid_for(n16, sm_count, 5);
+    launch_chained(prescale_reduce_kernel, grid, kThreads, 0, s, e0, mask, x2, n16, dev);
     hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
     hook(&dev->sum0, 2, EOQ_REDUCE_I64, EOQ_REDUCE_SUM, s);  // sum0 and sum1 are adjacent
-    prescale_apply_kernel<<<grid_for(n16, sm_count), kThreads, 0, s>>>(e0, e0_exp, mask, n16, gamma_c, gamma_dev, e3,
-                                                                       e3_exp, sum_e1, sum_e1x2, dev);
+    launch_chained(prescale_apply_kernel, grid, kThreads, 0, s, e0, e0_exp, mask, n16, gamma_c, gamma_dev, e3, e3_exp, sum_e1, sum_e1x2, dev);
     return cudaGetLastError();
 }
 

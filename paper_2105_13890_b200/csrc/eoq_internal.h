@@ -71,7 +71,7 @@ struct DeviceState {
     unsigned long long absmax2_u64;  // second maximum of a call that also serves its consumer's error head (masked |.|)
     unsigned tensor_absmax[256];  // per-tensor maxima of the multi-tensor update (zero between calls)
     unsigned ticket;       // blocks of the kernel that consumes the cells last count themselves here (see last_block_done)
-    unsigned arrivals;     // grid-wide barrier of the one-kernel error head (cooperative launch)
+    unsigned arrivals;     // what the self-test of the bounded waits waits for
     unsigned long long probe_cycles;  // eoq_probe_mma_i8: longest issue loop of the last launch, in SM clock cycles
 };
 // Invariant: absmax_u32, absmax_u64, absmax2_u64, sum0, sum1, ticket and arrivals are zero whenever no call is in flight on the handle.

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("groups", [1, 511, 512, 513, 2047, 2049, 4097, 12287, 12288, 12289])
 @pytest.mark.parametrize("gamma,with_x2", [(118, True), (128, False), (-700, True), (0, False)])
 def test_error_head_sizes(groups, gamma, with_x2):
-    """Groups of 16 codes: clusters of 1, 2, 4 and 8 blocks with up to six groups a thread, then the cooperative kernel."""
+    """Groups of 16 codes: clusters of 1, 2, 4 and 8 blocks with up to two groups a thread, then two kernels."""
     n = 16 * groups
     e0 = synth.normal_codes(n, 2900, groups, std_codes=30)
     mask = (synth.int8_uniform(n, 2901, groups) > -20).astype(np.uint8)
@@ -29,6 +29,27 @@ def test_error_head_sizes(groups, gamma, with_x2):
         assert s1.item() == int(e1.sum()) and (x2 is None or s2.item() == int((e1 * x2).sum()))
         want, pw, _ = oracle.sq_int(e1 * gamma, -12 - 7)
         assert np.array_equal(G.host(e3), want) and p.item() == pw
+
+
+@pytest.mark.parametrize("groups", [4096, 189440, 189441, 3 * 189440 - 7])
+@pytest.mark.parametrize("masked", [False, True])
+def test_error_head_of_several_groups_to_a_thread(groups, masked):
+    """The largest cluster, and two kernels whose threads take one to three groups (five blocks of 256 threads to an SM), a maximum that
+    only the last group holds among them."""
+    n = 16 * groups
+    e0 = synth.normal_codes(n, 2910, groups, std_codes=9).clip(-60, 60).astype(np.int8)
+    e0[n - 1] = -127
+    mask = synth.bits(n, 2911, groups, 0.5) if masked else None
+    if masked:
+        mask[n - 1] = 1
+    x2 = synth.int8_uniform(n, 2912, groups).astype(np.int16) * 250
+    e1 = e0.astype(np.int64) * (1 if mask is None else mask)
+    e3, p, s1, s2 = G.empty((n,), torch.int8), G.zeros(1, torch.int32), G.zeros(1, torch.int64), G.zeros(1, torch.int64)
+    eoq.eoq_err_prescale(G.handle(), G.dev(e0), torch.tensor([-12], dtype=torch.int32, device="cuda:0"), G.dev(G.pack_mask(mask)) if masked else None,
+                         G.dev(x2), n, 118, e3, p, s1, s2)
+    want, pw, _ = oracle.sq_int(e1 * 118, -12 - 7)
+    assert G.status_clear() == 0 and np.array_equal(G.host(e3), want) and p.item() == pw
+    assert s1.item() == int(e1.sum()) and s2.item() == int((e1 * x2).sum())
 
 
 GEOMETRIES = [
