@@ -291,7 +291,18 @@ void plan_igemm(IgemmParams &p, int src_channels, int ntaps, int sm_count)
     // An MMA costs at least ~57 cycles whatever its width and reaches the tensor peak only from 128 columns
     // up, so tiles stay 128 wide even when that leaves some SMs without one; 256 when there are tiles to spare.
     int tn = p.N < 256 ? p.N : 256;
-    if (tn == 256 && (long long)p.num_m_tiles * ((p.N + 255) / 256) < 2LL * sm_count) tn = 128;
+    const bool spare = (long long)p.num_m_tiles * ((p.N + 255) / 256) >= 2LL * sm_count;
+    if (tn == 256 && !spare) tn = 128;
+    if (p.N > 128 && !p.b_mn) {
+        // Forward: cuts of equal width (28 x 28 at batch 64, 1024 -> 304 channels: two of 160 instead of 256 and 48, 28.3 -> 25.9 us).  Up to
+        // 512 terms the epilogue bounds the layer, and its time goes by the columns of the busiest CTA: narrow tiles then where that has
+        // at least four wide ones and they leave it fewer columns (64 -> 512 channels with shortcut 54.3 -> 45.0 us, 512 -> 512 59.6 -> 53.7; without shortcut 1024 -> 256
+        // at 14 x 14, batch 512: 35.6 us wide, 36.6 narrow).
+        auto cut = [&](int most) { const int parts = (p.N + most - 1) / most; return ((p.N + parts - 1) / parts + 15) / 16 * 16; };
+        auto columns = [&](int cols) { return ((long long)p.num_m_tiles * ((p.N + cols - 1) / cols) + sm_count - 1) / sm_count * cols; };
+        tn = tn < 256 && p.N < 256 ? tn : cut(tn);
+        if (p.N >= 256 && spare && ntaps * src_channels <= 512 && columns(tn) >= 4 * tn && columns(cut(128)) < columns(tn)) tn = cut(128);
+    }
     set_columns(p, tn, 1);
     p.a_rows = kTileM;   // a problem of fewer pixels loads no more of them (TMA time goes by rows; the rest of the tile is never stored)
     while (p.a_rows > 16 && p.M <= p.a_rows / 2) p.a_rows /= 2;

@@ -46,6 +46,31 @@ def test_few_tiles(d, relu):
     assert np.array_equal(G.host(e4), want) and e4_exp.item() == p and total.item() == int(want.astype(np.int64).sum())
 
 
+WIDE = [
+    oracle.ConvDesc(150, 14, 14, 64, 512, 1, 1, 1, 0),    # narrow tiles for their even shares
+    oracle.ConvDesc(100, 14, 14, 64, 528, 1, 1, 1, 0),    # five of 112, the last one of 80
+    oracle.ConvDesc(100, 14, 14, 576, 304, 1, 1, 1, 0),   # two of 160, the last one of 144
+    oracle.ConvDesc(20, 14, 14, 64, 304, 1, 1, 1, 0),     # few tiles: three of 112, the last one of 80
+    oracle.ConvDesc(31, 27, 27, 48, 272, 3, 3, 2, 1),     # three of 96, strided, 16-byte chunks
+]
+
+
+@pytest.mark.parametrize("d", WIDE, ids=lambda d: "n%d_%dx%d_%d_%d_k%ds%d" % (d.n, d.h, d.w, d.c_in, d.c_out, d.kh, d.stride))
+@pytest.mark.parametrize("gamma", [118, 128])
+def test_forward_column_cuts(d, gamma):
+    """More than 128 output channels: equal cuts, and tiles that reach past the last channel."""
+    x0, w = synth.int8_uniform((d.n, d.h, d.w, d.c_in), 2705, d.c_in), synth.normal_codes((d.c_out, d.kh, d.kw, d.c_in), 2706, d.c_out, std_codes=6)
+    out = (d.n, d.ho, d.wo, d.c_out)
+    shortcut = synth.int8_uniform(out, 2707, d.h) if gamma != 128 else None
+    gd = G.gdesc(d)
+    ref = oracle.layer_forward(d, x0, -2, w, gamma, 3, shortcut, True)
+    x5, x2, mask = G.zeros(out, torch.int8), G.zeros(out, torch.int16) if gamma != 128 else None, G.zeros((ref["x5"].size + 7) // 8, torch.uint8)
+    eoq.eoq_conv_fwd(G.handle(), gd, G.dev(x0), None, -2, G.dev(w), gamma, 3, None if shortcut is None else G.dev(shortcut), True, x5, x2, mask, None,
+                     G.workspace(gd, eoq.EOQ_PASS_FWD))
+    assert G.status_clear() == 0 and np.array_equal(G.host(x5), ref["x5"]) and np.array_equal(G.unpack_mask(mask, out), ref["mask"])
+    assert x2 is None or np.array_equal(G.host(x2).astype(np.int32), ref["x2"])
+
+
 @pytest.mark.parametrize("b2", [0, 3, -5, 16384, -16384, 16385, -32768, 32767])
 @pytest.mark.parametrize("relu", [True, False])
 def test_unit_gamma_without_shortcut(relu, b2):
