@@ -48,3 +48,21 @@ def test_strided_classes(d, cap):
         assert np.array_equal(G.host(e4), want) and e4_exp.item() == p and total.item() == int(want.astype(np.int64).sum())
         assert dump is None or np.array_equal(G.host(dump), acc)
     eoq.eoq_destroy(h)
+
+
+@pytest.mark.parametrize("d", [
+    oracle.ConvDesc(3, 7, 9, 16, 16, 1, 1, 2, 0),       # one group of channels
+    oracle.ConvDesc(5, 40, 41, 48, 32, 1, 1, 3, 0),     # three, a stride of three
+    oracle.ConvDesc(97, 28, 28, 112, 64, 1, 1, 2, 0),   # two rounds and a bit of items to a thread
+    oracle.ConvDesc(1, 1, 260, 80, 16, 1, 1, 7, 0),     # one row
+], ids=lambda d: "n%d_%dx%d_%d_%d_s%d" % (d.n, d.h, d.w, d.c_in, d.c_out, d.stride))
+def test_scattered_codes(d):
+    """Strided 1x1 filters: codes on the grid, zeros elsewhere, for groups, widths, heights and strides that are no powers of two."""
+    gd = G.gdesc(d)
+    e3, w = synth.normal_codes((d.n, d.ho, d.wo, d.c_out), 2740, d.h, std_codes=24), synth.normal_codes((d.c_out, 1, 1, d.c_in), 2741, d.w, std_codes=6)
+    want, p, _ = oracle.sq_int(oracle.conv_dgrad_acc(d, e3, w), -9 - 7)
+    e4, e4_exp, total = torch.full(want.shape, 77, dtype=torch.int8, device="cuda:0"), G.zeros(1, torch.int32), G.empty(1, torch.int64)
+    eoq.eoq_conv_dgrad(G.handle(), gd, G.dev(e3), torch.tensor([-9], dtype=torch.int32, device="cuda:0"), G.dev(w), e4, e4_exp, total, None,
+                       G.workspace(gd, eoq.EOQ_PASS_DGRAD))
+    assert G.status_clear() == 0 and np.array_equal(G.host(e4), want) and e4_exp.item() == p
+    assert total.item() == int(want.astype(np.int64).sum())
