@@ -231,34 +231,39 @@ maxpool_bwd_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, const uin
 // The same for the pool of the ImageNet networks: window 3, stride 2, padding 1.  Position 2q of an axis lies in window q
 // alone (as its row 1), position 2q + 1 in windows q (row 2) and q + 1 (row 0), so a thread owns the 2 x 2 positions of
 // quad (qy, qx) for 16 channels and loads the four windows (qy, qx) .. (qy + 1, qx + 1) once for all nine pairs of
-// position and window.  Codes are kept with an offset of 128 per window in unsigned 16-bit halves, so that they add
-// without carries; a half joined with the upper half of 1.5 * 2^23 is that number plus the (offset) sum as a float, and
-// one fused multiply-add takes the offset out, scales and rounds it to nearest even (see rne7_magic).
-// Bound by instruction issue: about 8 instructions per code in pass 0, 14 in pass 1.  At batch 64, 51 M codes: pass 0
-// 78 us, pass 1 90 us with a gather per position and 32-bit sums; now 39 and 49 us (both beside weight-gradient work).
-struct PoolQuad {
-    uint32_t even[4][4], odd[4][4];   // [position][word]: offset sums of channels 0, 2 / 1, 3 of the word's four
-};
-// offset of a position's halves: 128 per window pair, in both halves
-__device__ __forceinline__ constexpr uint32_t quad_offset(int pos) { return 0x00800080u * (pos == 0 ? 1u : (pos == 3 ? 4u : 2u)); }
+// position and window.  A sum is one byte dot product of a channel's four error codes with zeros and ones, and these come out of an
+// eight-byte table by one permute for all four windows: its selector is four digits, one per window, that say which of the
+// quad's positions the window elected (0: (1,1), 1: (1,0), 3: (0,1), 4: (0,0); every other digit finds a zero).
+// Bound by instruction issue, of the integer pipe above all.  With a compare and two additions per pair, position and code, in
+// 16-bit halves, 51 M codes took 30.8 us in pass 0 and 41.6 in pass 1, now 25.5 and 32.0.
 
-// adds one window to one position; kFirst: it is the position's first
-template <bool kFirst>
-__device__ __forceinline__ void quad_add(uint32_t (&even)[4], uint32_t (&odd)[4], const uint32_t (&e)[4], const uint32_t (&a)[4], uint32_t idx)
+// The positions of the quad are numbered 2 * row + column, the windows likewise.
+__device__ __forceinline__ uint32_t table_bytes(uint32_t lo, uint32_t hi, uint32_t digits)
 {
-    const uint32_t me = idx * 0x01010101u;
+    uint32_t r;   // (a digit of 8 or more repeats the sign of a byte: zero, as all of them are 0 or 1)
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(lo), "r"(hi), "r"(digits));
+    return r;
+}
+
+// Sums of the four positions for the four channels of a word, each plus `bias`: e, a = the word of every window (positions 0 to 8).
+__device__ __forceinline__ void quad_sums(const uint32_t (&e)[4], const uint32_t (&a)[4], uint32_t bias, uint32_t (&s)[4][4])
+{
+    // Digits.  8 - a, 6 - a, 2 - a and -a modulo 16 are 0 where a window elects position 3; the same differences give the others their
+    // digits.  Window 1 also shows 4 and 1 for positions that are not the quad's: it is left out where it has no part.
+    const uint32_t v0 = (0x18181818u - a[0]) & 0x0f0f0f0fu, v1 = (0x16161616u - a[1]) & 0x0f0f0f0fu, v2 = (0x12121212u - a[2]) & 0x0f0f0f0fu,
+                   v3 = (0x10101010u - a[3]) & 0x0f0f0f0fu;
+    const uint32_t lo = v1 * 16u + v0, hi = v3 * 16u + v2;
+    // the codes of a channel side by side
+    const uint32_t t0 = __byte_perm(e[0], e[1], 0x5140), t1 = __byte_perm(e[0], e[1], 0x7362), t2 = __byte_perm(e[2], e[3], 0x5140),
+                   t3 = __byte_perm(e[2], e[3], 0x7362);
+    const uint32_t codes[4] = {__byte_perm(t0, t2, 0x5410), __byte_perm(t0, t2, 0x7632), __byte_perm(t1, t3, 0x5410), __byte_perm(t1, t3, 0x7632)};
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const uint32_t x = a[q] ^ me;
-        const uint32_t other = prmt<0xba98>(((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x, 0u);  // 0xff in the bytes another position won
-        const uint32_t v = (e[q] & ~other) ^ 0x80808080u;
-        if (kFirst) {
-            even[q] = v & 0x00ff00ffu;
-            odd[q] = prmt<0x4341>(v, 0u);
-        } else {
-            even[q] += v & 0x00ff00ffu;
-            odd[q] += prmt<0x4341>(v, 0u);
-        }
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t digits = __byte_perm(lo, hi, (uint32_t)((4 + k) << 4 | k)), but1 = codes[k] & 0xffff00ffu;
+        s[0][k] = (uint32_t)__dp4a((int)but1, (int)table_bytes(0u, 0x00000001u, digits), (int)bias);
+        s[1][k] = (uint32_t)__dp4a((int)codes[k], (int)table_bytes(0x01000000u, 0u, digits), (int)bias);
+        s[2][k] = (uint32_t)__dp4a((int)but1, (int)table_bytes(0x00000100u, 0u, digits), (int)bias);
+        s[3][k] = (uint32_t)__dp4a((int)codes[k], (int)table_bytes(0x00000001u, 0u, digits), (int)bias);
     }
 }
 
@@ -288,7 +293,6 @@ maxpool_bwd_quad_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, cons
     const uint32_t quad = (live ? i : 0u) / (uint32_t)groups, row = quad / (uint32_t)wo;
     const int g = (int)((live ? i : 0u) - quad * (uint32_t)groups), qx = (int)(quad - row * (uint32_t)wo);
     const int b = (int)(row / (uint32_t)ho), qy = (int)(row - (uint32_t)b * (uint32_t)ho);
-    PoolQuad s;
     uint32_t mbits[4];
     bool in[4];
     const bool dn = qy + 1 < ho, rt = qx + 1 < wo;
@@ -298,51 +302,65 @@ maxpool_bwd_quad_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, cons
     in[3] = in[1] && in[2];
     const uint32_t pix = ((uint32_t)b * h + 2 * qy) * w + 2 * qx;   // 16-channel items stay below 2^31 (checked by the caller)
     const uint32_t at[4] = {pix * groups + g, (pix + 1) * groups + g, (pix + w) * groups + g, (pix + w + 1) * groups + g};
+    uint32_t ew[4][4], aw[4][4];   // [window][word]
     {
         const size_t o = ((size_t)row * wo + qx) * c + g * 16;
-        uint32_t e0[4], a0[4], e1[4], a1[4], e2[4], a2[4], e4[4], a4[4];
-        quad_load(e, arg, o, live, e0, a0);
-        quad_load(e, arg, o + c, live && rt, e1, a1);
-        quad_load(e, arg, o + (size_t)wo * c, live && dn, e2, a2);
-        quad_load(e, arg, o + (size_t)(wo + 1) * c, live && rt && dn, e4, a4);
+        quad_load(e, arg, o, live, ew[0], aw[0]);
+        quad_load(e, arg, o + c, live && rt, ew[1], aw[1]);
+        quad_load(e, arg, o + (size_t)wo * c, live && dn, ew[2], aw[2]);
+        quad_load(e, arg, o + (size_t)(wo + 1) * c, live && rt && dn, ew[3], aw[3]);
 #pragma unroll
         for (int p = 0; p < 4; ++p)
             mbits[p] = (kNext && in[p]) ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(next_mask) + at[p]) : 0u;
-        quad_add<true>(s.even[0], s.odd[0], e0, a0, 4);
-        quad_add<true>(s.even[1], s.odd[1], e0, a0, 5);
-        quad_add<false>(s.even[1], s.odd[1], e1, a1, 3);
-        quad_add<true>(s.even[2], s.odd[2], e0, a0, 7);
-        quad_add<false>(s.even[2], s.odd[2], e2, a2, 1);
-        quad_add<true>(s.even[3], s.odd[3], e0, a0, 8);
-        quad_add<false>(s.even[3], s.odd[3], e1, a1, 6);
-        quad_add<false>(s.even[3], s.odd[3], e2, a2, 2);
-        quad_add<false>(s.even[3], s.odd[3], e4, a4, 0);
+        // a byte beyond 8 elects nothing (the forward pass writes none)
+        uint32_t any = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) any |= aw[u][q] | (aw[u][q] + 0x07070707u);
+        if (any & 0xf0f0f0f0u) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t beyond = prmt<0xba98>(((aw[u][q] & 0x7f7f7f7fu) + 0x77777777u) | aw[u][q], 0u);
+                    ew[u][q] &= ~beyond;
+                    aw[u][q] &= ~beyond;
+                }
+        }
     }
+    auto word_sums = [&](int q, uint32_t bias, uint32_t (&s)[4][4]) {
+        const uint32_t e4[4] = {ew[0][q], ew[1][q], ew[2][q], ew[3][q]}, a4[4] = {aw[0][q], aw[1][q], aw[2][q], aw[3][q]};
+        quad_sums(e4, a4, bias, s);
+    };
     if (kPass == 0) {
-        uint32_t mx = 0, mx_masked = 0;
+        // sums plus 1024 (|sum| <= 4 * 128), two to a word
+        constexpr uint32_t kOff = 0x04000400u;
+        uint32_t hi = kOff, lo = kOff, him = kOff, lom = kOff;
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            if (!in[p]) continue;
-            const uint32_t off = quad_offset(p);
-            uint32_t hi = off, lo = off, him = off, lom = off;
+        for (int q = 0; q < 4; ++q) {
+            uint32_t s[4][4];
+            word_sums(q, 1024u, s);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                hi = __vimax3_u16x2(hi, s.even[p][q], s.odd[p][q]);
-                lo = __vimin3_u16x2(lo, s.even[p][q], s.odd[p][q]);
+            for (int p = 0; p < 4; ++p) {
+                const uint32_t s01 = s[p][1] * 65536u + s[p][0], s23 = s[p][3] * 65536u + s[p][2];
+                if (in[p]) {
+                    hi = __vimax3_u16x2(hi, s01, s23);
+                    lo = __vimin3_u16x2(lo, s01, s23);
+                }
                 if (kNext) {
                     const uint32_t sg = nibble_signs(mbits[p], q);
-                    const uint32_t me = prmt<0xaa88>(sg, 0u), mo = prmt<0xbb99>(sg, 0u);   // 0xffff in the halves the ReLU lets through
-                    const uint32_t ev = (s.even[p][q] & me) | (off & ~me), ov = (s.odd[p][q] & mo) | (off & ~mo);
-                    him = __vimax3_u16x2(him, ev, ov);
-                    lom = __vimin3_u16x2(lom, ev, ov);
+                    const uint32_t m01 = prmt<0x9988>(sg, 0u), m23 = prmt<0xbbaa>(sg, 0u);   // 0xffff in the halves the ReLU lets through
+                    const uint32_t e01 = (s01 & m01) | (kOff & ~m01), e23 = (s23 & m23) | (kOff & ~m23);
+                    him = __vimax3_u16x2(him, e01, e23);
+                    lom = __vimin3_u16x2(lom, e01, e23);
                 }
             }
-            const int o1 = (int)(off & 0xffffu);
-            mx = max(mx, (uint32_t)max(max((int)(hi & 0xffffu), (int)(hi >> 16)) - o1, o1 - min((int)(lo & 0xffffu), (int)(lo >> 16))));
-            if (kNext)
-                mx_masked = max(mx_masked,
-                                (uint32_t)max(max((int)(him & 0xffffu), (int)(him >> 16)) - o1, o1 - min((int)(lom & 0xffffu), (int)(lom >> 16))));
         }
+        auto most = [&](uint32_t h, uint32_t l) {
+            return (uint32_t)max(max((int)(h & 0xffffu), (int)(h >> 16)) - 1024, 1024 - min((int)(l & 0xffffu), (int)(l >> 16)));
+        };
+        uint32_t mx = most(hi, lo), mx_masked = kNext ? most(him, lom) : 0u;
         // both maxima are below 2^10: one reduction for the pair would need them ordered apart, so two
         __shared__ uint32_t red[2];
         if (threadIdx.x < 2) red[threadIdx.x] = 0;
@@ -379,39 +397,34 @@ maxpool_bwd_quad_kernel(const int8_t *__restrict__ e, const int32_t *e_exp, cons
             if (!M) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
             if (kNext) next_head_exponent(nh, p0, e3_exp, dev);
         }
-        constexpr int kLo = (int)kHeadMagic - 127, kHi = (int)kHeadMagic + 127;
         const float scale = __int_as_float((127 + 7 - t) << 23);   // 2^(7 - t), t in [0, 9]
-        const uint32_t head_add = kHeadMagic - nh.g * kHeadMagic;
+        const float rest = 12582912.0f - 12582912.0f * scale;      // exact; the sums arrive plus 1.5 * 2^23 (see next_head_codes)
         int s1 = 0;
+        uint32_t cw[4][4], hw[4][4];   // [position][word]
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const float rest = 12582912.0f - (12582912.0f + (float)(quad_offset(p) & 0xffffu)) * scale;  // exact
-            uint32_t cw[4], hw[4];
+        for (int q = 0; q < 4; ++q) {
+            uint32_t s[4][4];
+            word_sums(q, kHeadMagic, s);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t half[4] = {prmt<0x7610>(s.even[p][q], kHeadMagic), prmt<0x7610>(s.odd[p][q], kHeadMagic),
-                                          prmt<0x7632>(s.even[p][q], kHeadMagic), prmt<0x7632>(s.odd[p][q], kHeadMagic)};
-                int r[4], r3[4];
+            for (int p = 0; p < 4; ++p) {
+                int r[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    r[k] = clampi((int)__float_as_uint(__fmaf_rn(__uint_as_float(half[k]), scale, rest)), kLo, kHi);
-                    if (kNext) {
-                        const uint32_t biased = nh.g * (uint32_t)r[k] + head_add;   // gamma * code + 1.5 * 2^23
-                        r3[k] = __viaddmax_s32((int)__float_as_uint(__fmaf_rn(__uint_as_float(biased), nh.scale, nh.rest)), -(int)kHeadMagic, -127);
-                    }
-                }
-                cw[q] = prmt<0x5410>(prmt<0x0040>((uint32_t)r[0], (uint32_t)r[1]), prmt<0x0040>((uint32_t)r[2], (uint32_t)r[3]));
+                for (int k = 0; k < 4; ++k)
+                    r[k] = __viaddmax_s32((int)__float_as_uint(__fmaf_rn(__uint_as_float(s[p][k]), scale, rest)), -(int)kHeadMagic, -127);
+                cw[p][q] = pack4_sat(r[0], r[1], r[2], r[3]);
                 if (kNext) {
-                    const uint32_t m = prmt<0xba98>(nibble_signs(mbits[p], q), 0u);
-                    s1 = __dp4a((int)(cw[q] & m), 0x01010101, s1);
-                    hw[q] = pack4_sat(r3[0], r3[1], r3[2], r3[3]) & m;   // the code of zero is zero
+                    const uint32_t e1 = cw[p][q] & prmt<0xba98>(nibble_signs(mbits[p], q), 0u);
+                    s1 = __dp4a((int)e1, 0x01010101, s1);
+                    hw[p][q] = next_head_codes(nh, e1);
                 }
-            }
-            if (in[p]) {
-                if (e_in) reinterpret_cast<uint4 *>(e_in)[at[p]] = make_uint4(cw[0], cw[1], cw[2], cw[3]);
-                if (kNext) reinterpret_cast<uint4 *>(e3)[at[p]] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
             }
         }
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            if (in[p]) {
+                if (e_in) reinterpret_cast<uint4 *>(e_in)[at[p]] = make_uint4(cw[p][0], cw[p][1], cw[p][2], cw[p][3]);
+                if (kNext) reinterpret_cast<uint4 *>(e3)[at[p]] = make_uint4(hw[p][0], hw[p][1], hw[p][2], hw[p][3]);
+            }
         if (kNext && sum_e1) {
             s1 = __reduce_add_sync(0xffffffffu, s1);
             if ((threadIdx.x & 31) == 0 && s1) atomicAdd(&sum_s, s1);

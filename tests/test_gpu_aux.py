@@ -85,6 +85,35 @@ def test_maxpool_backward_with_the_error_head_fused(n, h, w, c, k, s, p, gamma):
         assert np.array_equal(G.host(e3), want_e3) and p3.item() == want_p3 and s1.item() == want_s1
 
 
+@pytest.mark.parametrize("h,w", [(1, 1), (2, 5), (13, 8), (40, 41)])
+@pytest.mark.parametrize("most", [8, 15, 255])
+def test_maxpool_backward_of_any_recorded_position(h, w, most):
+    """Window 3, stride 2, padding 1: every recorded position in every window, those outside the image (which no forward pass records)
+    and bytes beyond 8 (which elect nothing) among them, and the largest sums, against a plain gather."""
+    n, c, (ho, wo) = 2, 48, ((h - 1) // 2 + 1, (w - 1) // 2 + 1)
+    r = synth.rng(8180 + h, most)
+    e = np.where(r.random((n, ho, wo, c)) < 0.2, 127, r.integers(-127, 128, (n, ho, wo, c))).astype(np.int8)
+    arg = np.where(r.random((n, ho, wo, c)) < 0.5, r.integers(0, 9, (n, ho, wo, c)), r.integers(0, most + 1, (n, ho, wo, c))).astype(np.uint8)
+    S = np.zeros((n, h + 2, w + 2, c), dtype=np.int64)
+    for oy in range(ho):
+        for ox in range(wo):
+            for a in range(9):
+                y, x = 2 * oy + a // 3, 2 * ox + a % 3   # (one row and column of padding in front)
+                if y < h + 2 and x < w + 2:
+                    S[:, y, x] += np.where(arg[:, oy, ox] == a, e[:, oy, ox], 0)
+    S = np.ascontiguousarray(S[:, 1:1 + h, 1:1 + w])
+    e0, p0, _ = oracle.sq_int(S, -12)
+    mask01 = synth.bits((n, h, w, c), 8181, most, 0.5)
+    want_e3, want_p3, want_s1, _, _ = oracle.err_prescale(e0.astype(np.int8), p0, mask01, None, 97)
+    hd = G.handle()
+    ein, pin, e3, p3, s1 = G.empty(S.shape, torch.int8), G.zeros(1, torch.int32), G.empty(S.shape, torch.int8), G.zeros(1, torch.int32), G.zeros(1, torch.int64)
+    eoq.eoq_aux_maxpool_bwd_head(hd, G.dev(e), i32(-12), G.dev(arg), n, h, w, c, 3, 2, 1, ein, pin, G.dev(G.pack_mask(mask01)), i32(97), e3, p3, s1)
+    torch.cuda.synchronize()
+    eoq.eoq_last_status(hd)   # (nothing elected is flagged)
+    assert np.array_equal(G.host(ein), e0) and pin.item() == p0
+    assert np.array_equal(G.host(e3), want_e3) and p3.item() == want_p3 and s1.item() == want_s1
+
+
 def test_maxpool_backward_of_a_zero_error_keeps_the_exponent():
     hd = G.handle()
     n, h, w, c = 1, 6, 6, 16
