@@ -38,80 +38,53 @@ __device__ __forceinline__ bool finish_narrow(const FinishItem &it, int b1)
 // all pixels, R_i and C_j those over the i-th border row and the j-th border column, and P_ij those over their crossings,
 //   tap sum = T - sum of R_i - sum of C_j + sum of P_ij   over the border rows and columns the tap does not take.
 // Every term is a plain sum over a regular set of pixels.  A block covers a range of rows and a slab of channels; a lane
-// keeps 16 channels (one 128-bit load per pixel, several in flight) in packed 16-bit halves (codes offset by 128, so that
-// no carry crosses; one instruction per code).  All warps sum T, then share out the border sets.
+// keeps the sums of 16 channels (one 128-bit load per pixel, several in flight).  All warps sum T, then share out the border sets.
 // A slab's rows are dealt to the kTapReplicas copies of its cells, and a copy's to the blocks of a cluster, whose sums meet in
 // distributed shared memory: a copy is stored, not added to, so nothing clears the cells and no order against the GEMM is needed.
 // Bound by the latency of a few dependent rounds of loads.  A single layer's sums therefore go in front of its GEMM, which is let
 // in at once and runs beside them (conv_wgrad_impl).  With atomics into cells that the GEMM cleared they came behind it and ended
 // 3 to 8 us after it: backward of the 512-channel 7 x 7 layer at batch 64 60.6 -> 59.0 us, bottleneck block of ResNet-50 at batch 32
-// 270 -> 264, and fewer SMs taken from the error chain of a step (ResNet-18 at batch 13 621 -> 608).
+// 270 -> 264, and fewer SMs taken from the error chain of a step (ResNet-18 at batch 13 621 -> 608).  Sums of four pixels by dot products
+// and no divisions in front of the first load: the kernel 7.5 -> 5.5 us for the 48 -> 80 channel strided layer, whose backward went 26.5
+// -> 24.7.
 struct PixelSum {
-    uint32_t even[4], odd[4];
-    int count;
-    __device__ __forceinline__ void clear()
+    int v[16] = {};
+    // adds four pixels: the codes of a channel side by side, then one byte dot product
+    __device__ __forceinline__ void add4(const int4 &p0, const int4 &p1, const int4 &p2, const int4 &p3)
     {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) even[q] = odd[q] = 0;
-        count = 0;
-    }
-    __device__ __forceinline__ void add(const int4 &v)
-    {
-        const uint32_t w[4] = {(uint32_t)v.x, (uint32_t)v.y, (uint32_t)v.z, (uint32_t)v.w};
+        const uint32_t w0[4] = {(uint32_t)p0.x, (uint32_t)p0.y, (uint32_t)p0.z, (uint32_t)p0.w}, w1[4] = {(uint32_t)p1.x, (uint32_t)p1.y, (uint32_t)p1.z, (uint32_t)p1.w};
+        const uint32_t w2[4] = {(uint32_t)p2.x, (uint32_t)p2.y, (uint32_t)p2.z, (uint32_t)p2.w}, w3[4] = {(uint32_t)p3.x, (uint32_t)p3.y, (uint32_t)p3.z, (uint32_t)p3.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const uint32_t u = w[q] ^ 0x80808080u;
-            even[q] += u & 0x00ff00ffu;
-            odd[q] += __byte_perm(u, 0u, 0x4341);
+            const uint32_t t0 = __byte_perm(w0[q], w1[q], 0x5140), t1 = __byte_perm(w0[q], w1[q], 0x7362), t2 = __byte_perm(w2[q], w3[q], 0x5140),
+                           t3 = __byte_perm(w2[q], w3[q], 0x7362);
+            v[4 * q] = __dp4a((int)__byte_perm(t0, t2, 0x5410), 0x01010101, v[4 * q]);
+            v[4 * q + 1] = __dp4a((int)__byte_perm(t0, t2, 0x7632), 0x01010101, v[4 * q + 1]);
+            v[4 * q + 2] = __dp4a((int)__byte_perm(t1, t3, 0x5410), 0x01010101, v[4 * q + 2]);
+            v[4 * q + 3] = __dp4a((int)__byte_perm(t1, t3, 0x7632), 0x01010101, v[4 * q + 3]);
         }
     }
-    // Adds the warp's sums to the cells of a set: `dst` is the lane's first channel, `lanes` the lanes of a pixel.  Lanes
-    // that hold the same channels would queue at the cells (32 of them for 16 channels), so where `lanes` is a power of two
-    // they first halve their channels among each other, pairwise, and every channel is added once per warp.
+    // Adds the warp's sums to the cells of a set: `dst` is the lane's first channel, `lanes` (1 or 2) the lanes of a pixel.  Lanes
+    // that hold the same channels would queue at the cells (32 of them for 16 channels), so they first halve their channels among
+    // each other, pairwise, and every channel is added once per warp.
     __device__ __forceinline__ void flush(int32_t *dst, int lanes)
     {
-        int v[16];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            v[4 * q] = (int)(even[q] & 0xffffu) - 128 * count;
-            v[4 * q + 1] = (int)(odd[q] & 0xffffu) - 128 * count;
-            v[4 * q + 2] = (int)(even[q] >> 16) - 128 * count;
-            v[4 * q + 3] = (int)(odd[q] >> 16) - 128 * count;
-        }
-        clear();
         const int lane = threadIdx.x & 31;
-        if (lanes & (lanes - 1)) {
+        int off = 0;
 #pragma unroll
-            for (int c = 0; c < 16; ++c) atomicAdd(dst + c, v[c]);
-            return;
-        }
-        int have = 16, off = 0;
+        for (int m = 16, half = 8; half >= 1; m >>= 1, half >>= 1) {
+            const bool up = (lane & m) != 0;
 #pragma unroll
-        for (int m = 16, half = 8; half >= 1; m >>= 1, half >>= 1)
-            if (m >= lanes) {
-                const bool up = (lane & m) != 0;
-#pragma unroll
-                for (int c = 0; c < half; ++c) {
-                    const int keep = up ? v[c + half] : v[c], send = up ? v[c] : v[c + half];
-                    v[c] = keep + __shfl_xor_sync(0xffffffffu, send, m);
-                }
-                off += up ? half : 0;
-                have = half;
+            for (int c = 0; c < half; ++c) {
+                const int keep = up ? v[c + half] : v[c], send = up ? v[c] : v[c + half];
+                v[c] = keep + __shfl_xor_sync(0xffffffffu, send, m);
             }
+            off += up ? half : 0;
+        }
         if (lanes == 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-        if (lanes > 1 || !(lane & 1))
+        if (lanes > 1 || !(lane & 1)) atomicAdd(dst + off, v[0]);
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < have) atomicAdd(dst + off + c, v[c]);
-    }
-    // adds kUnroll pixels (a zero one adds the offset alone); all lanes of the warp call it together
-    template <int kUnroll>
-    __device__ __forceinline__ void add_group(const int4 (&v)[kUnroll], int32_t *dst, int lanes)
-    {
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) add(v[u]);
-        count += kUnroll;
-        if (count > 256 - kUnroll) flush(dst, lanes);   // 255 * 257 is the most a half holds
+        for (int c = 0; c < 16; ++c) v[c] = 0;
     }
 };
 
@@ -157,12 +130,11 @@ __device__ __forceinline__ void tap_sets(const FinishItem &it, int slab, int sla
     const int ho = it.ho, wo = it.wo, c_out = d.c_out, nsets = (1 + nr) * (1 + nc);
     for (int i = threadIdx.x; i < nsets * kTapSlab; i += kT) sets[i] = 0;
     __syncthreads();
-    const int lanes_per_pix = slab_ch / 16, pix_per_step = 32 / lanes_per_pix;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lane_ch = (lane % lanes_per_pix) * 16, slot = lane / lanes_per_pix;
+    const int two = slab_ch >> 5, lanes_per_pix = 1 + two, pix_per_step = 32 >> two;   // (a slab has 16 or 32 channels)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lane_ch = (lane & two) * 16, slot = lane >> two;
     const int8_t *base = it.e3 + slab * kTapSlab + lane_ch;
     const int4 zero = make_int4(0, 0, 0, 0);
     PixelSum acc;
-    acc.clear();
     {   // T
         constexpr int kUnroll = 8;
         const size_t p_end = (size_t)r_end * wo;
@@ -174,41 +146,46 @@ __device__ __forceinline__ void tap_sets(const FinishItem &it, int slab, int sla
                 const size_t p = p0 + slot + u * step;
                 v[u] = p < p_end ? __ldcg(reinterpret_cast<const int4 *>(base + p * c_out)) : zero;
             }
-            acc.add_group(v, sets + lane_ch, lanes_per_pix);
+            acc.add4(v[0], v[1], v[2], v[3]);
+            acc.add4(v[4], v[5], v[6], v[7]);
         }
-        if (acc.count) acc.flush(sets + lane_ch, lanes_per_pix);
+        acc.flush(sets + lane_ch, lanes_per_pix);
     }
-    // the border sets, each by as many warps as there are for one
-    const int share = max(1, (kT / 32) / max(1, nsets - 1));
-    for (int turn = warp; turn < (nsets - 1) * share; turn += kT / 32) {
-        constexpr int kUnroll = 4;
-        const int set = 1 + turn / share, part = turn % share;
-        const int i = set / (1 + nc), j = set - i * (1 + nc);
-        int32_t *dst = sets + set * kTapSlab + lane_ch;
-        // rows first + q * row_step of the range, columns x0 .. x0 + cols - 1
-        int first = r_begin, row_step = 1, x0 = 0, cols = wo;
-        if (i > 0) {
-            const int y = border_at(i - 1, ho, bc.nlo_h, bc.nhi_h, bc.nrc);
-            row_step = ho;
-            first = r_begin + (y - r_begin % ho + ho) % ho;
-        }
-        if (j > 0) {
-            x0 = border_at(j - 1, wo, bc.nlo_w, bc.nhi_w, bc.ncc);
-            cols = 1;
-        }
-        const int rows = first < r_end ? (r_end - first + row_step - 1) / row_step : 0;
-        const int pixels = rows * cols, step = share * pix_per_step;
-        for (int q0 = part * pix_per_step; q0 < pixels; q0 += kUnroll * step) {
-            int4 v[kUnroll];
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                const int q = q0 + slot + u * step, rq = cols == 1 ? q : q / wo;
-                const int r = first + rq * row_step, x = x0 + (q - rq * cols);
-                v[u] = q < pixels ? __ldcg(reinterpret_cast<const int4 *>(base + ((size_t)r * wo + x) * c_out)) : zero;
+    if (nsets > 1) {
+        // the border sets, each by as many warps as there are for one
+        const int share = max(1, (kT / 32) / (nsets - 1)), r_at = r_begin % ho;
+        const float per_row = 1.0f / (float)wo;
+        for (int turn = warp; turn < (nsets - 1) * share; turn += kT / 32) {
+            constexpr int kUnroll = 4;
+            const int set = 1 + turn / share, part = turn % share;
+            const int i = set / (1 + nc), j = set - i * (1 + nc);
+            int32_t *dst = sets + set * kTapSlab + lane_ch;
+            // rows first + q * row_step of the range, columns x0 .. x0 + cols - 1
+            int first = r_begin, row_step = 1, x0 = 0, cols = wo;
+            if (i > 0) {
+                const int y = border_at(i - 1, ho, bc.nlo_h, bc.nhi_h, bc.nrc);
+                row_step = ho;
+                first = r_begin + y - r_at + (y < r_at ? ho : 0);
             }
-            acc.add_group(v, dst, lanes_per_pix);
+            if (j > 0) {
+                x0 = border_at(j - 1, wo, bc.nlo_w, bc.nhi_w, bc.ncc);
+                cols = 1;
+            }
+            const int rows = first < r_end ? (r_end - first + row_step - 1) / row_step : 0;
+            const int pixels = rows * cols, step = share * pix_per_step;
+            for (int q0 = part * pix_per_step; q0 < pixels; q0 += kUnroll * step) {
+                int4 v[kUnroll];
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) {
+                    // (q / wo: below 2^20 the product is off by less than the half that is added)
+                    const int q = q0 + slot + u * step, rq = cols == 1 ? q : (pixels < (1 << 20) ? (int)(((float)q + 0.5f) * per_row) : q / wo);
+                    const int r = first + rq * row_step, x = x0 + (q - rq * cols);
+                    v[u] = q < pixels ? __ldcg(reinterpret_cast<const int4 *>(base + ((size_t)r * wo + x) * c_out)) : zero;
+                }
+                acc.add4(v[0], v[1], v[2], v[3]);
+            }
+            acc.flush(dst, lanes_per_pix);
         }
-        if (acc.count) acc.flush(dst, lanes_per_pix);
     }
     __syncthreads();
 }
@@ -225,16 +202,17 @@ __device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab,
     tap_masks(it, nr, nc, masks);   // (published by the barriers of tap_sets)
     const int slab_ch = min(kTapSlab, d.c_out - slab * kTapSlab);  // channels of this slab (16 or 32)
     const int taps = d.kh * d.kw, items = taps * slab_ch;
-    const int rows = d.n * it.ho, ranges = copies * cluster, rows_here = (rows + ranges - 1) / ranges;
+    const int rows = d.n * it.ho, ranges = copies * cluster, rows_here = (rows + ranges - 1) >> (31 - __clz(ranges));   // (powers of two)
     const int begin = min((long long)rows, (long long)(copy * cluster + rank) * rows_here), end = min((long long)rows, (long long)begin + rows_here);
     constexpr int kMost = (kMaxTaps * kTapSlab + kT - 1) / kT;   // items of a thread
     long long total[kMost] = {};
-    const int chunk = max(1, (1 << 23) / it.wo);   // keeps the int32 sets exact
+    const int chunk = (long long)rows_here * it.wo <= (1 << 23) ? max(1, rows_here) : max(1, (1 << 23) / it.wo);   // keeps the int32 sets exact
+    const int ch_shift = 31 - __clz(slab_ch), per_kw = 65536 / d.kw + 1;   // tap / kw = tap * per_kw >> 16 for the few taps there are
     for (int at = 0; at < rows_here; at += chunk) {
         const int r0 = min(end, begin + at), r1 = min(end, r0 + min(chunk, rows_here - at));
         tap_sets<kT>(it, slab, slab_ch, r0, r1, nr, nc, sets);
         auto tap_sum = [&](int i) {
-            const int c = i / taps, tap = i - c * taps, kh = tap / d.kw, kw = tap - kh * d.kw;
+            const int tap = i >> ch_shift, c = i & (slab_ch - 1), kh = tap * per_kw >> 16, kw = tap - kh * d.kw;
             const unsigned long long rm = masks.rows[kh], cm = masks.cols[kw];
             const int32_t *cell = sets + c;
             auto over_columns = [&](const int32_t *row) {
@@ -267,9 +245,10 @@ __device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab,
     }
 #pragma unroll
     for (int k = 0; k < kMost; ++k) {
-        const int i = (k * cluster + rank) * kT + (int)threadIdx.x;   // neighbouring cells of [oc][tap]
+        const int i = (k * cluster + rank) * kT + (int)threadIdx.x;   // [tap][channel], stored at [oc][tap]
         if (i >= items) continue;
-        long long *cell = it.tap_sums + ((size_t)slab * kTapSlab * taps + i) * kTapReplicas;
+        const int tap = i >> ch_shift, c = i & (slab_ch - 1);
+        long long *cell = it.tap_sums + ((size_t)(slab * kTapSlab + c) * taps + tap) * kTapReplicas;
         cell[copy] = total[k];
         if (copy == 0)
             for (int r = copies; r < kTapReplicas; ++r) cell[r] = 0;
@@ -287,9 +266,10 @@ __global__ void __launch_bounds__(kTapThreads, 2) finish_taps_kernel(const __gri
     if (kLetIn) ptx::grid_dep_launch();
     extern __shared__ __align__(16) int32_t dyn[];
     const int k = finish_item_of(b.tap_first, b.num, (int)blockIdx.x);
-    const int local = (int)blockIdx.x - b.tap_first[k], per_slab = b.item[k].tap_copies * b.tap_cluster, part = local % per_slab;
-    finish_taps_slab<kTapThreads>(b.item[k], local / per_slab, part / b.tap_cluster, b.item[k].tap_copies, b.tap_cluster, part % b.tap_cluster,
-                                  dyn + kMaxTaps * kTapSlab, dyn);
+    // (copies and clusters come in powers of two)
+    const int local = (int)blockIdx.x - b.tap_first[k], copies = b.item[k].tap_copies, cluster_log = 31 - __clz(b.tap_cluster);
+    const int copy = (local >> cluster_log) & (copies - 1), slab = local >> (cluster_log + 31 - __clz(copies));
+    finish_taps_slab<kTapThreads>(b.item[k], slab, copy, copies, b.tap_cluster, local & (b.tap_cluster - 1), dyn + kMaxTaps * kTapSlab, dyn);
 }
 
 // ------------------------------------------------------------------ exact sums and their maximum
