@@ -1014,11 +1014,11 @@ __global__ void b1_weight_table_kernel(const int8_t *__restrict__ w, int32_t *ta
 
 // What eoq_weight_prep derives from the weights of several layers in one launch: the b1 table of every layer
 // (as b1_weight_table_kernel builds it) and, for a first layer on the filter-row path, the weights re-packed as
-// [oc][kh][8][c_in] with zero taps.  One block per (layer, output channel), bound by latency: all chunks of a channel are
-// loaded at once and added to their tap's cell, while the taps that each border class takes are worked out.
+// [oc][kh][8][c_in] with zero taps.  One block per (layer, output channel), bound by latency: the taps that each
+// border class takes are worked out while the kernel in front runs, all chunks of a channel are loaded at once and added to their tap's
+// cell (a single 16-channel layer's calls 35.0 -> 34.0 us with the former in front of the wait).
 __global__ void weight_prep_kernel(const __grid_constant__ PrepBatch b)
 {
-    ptx::grid_dep_wait_launch_small();
     __shared__ int32_t tap_sum[kMaxTaps];
     int k = 0;
     for (int hi = b.num - 1; k < hi;) {
@@ -1032,6 +1032,19 @@ __global__ void weight_prep_kernel(const __grid_constant__ PrepBatch b)
     const int oc = blockIdx.x - b.first_block[k];
     const int taps = d.kh * d.kw, width = d.c_in == 8 ? 8 : 16, per_tap = d.c_in / width, chunks = taps * per_tap;
     const int8_t *w = it.w + (size_t)oc * taps * d.c_in;
+    // what the launch's parameters give, while the kernels in front still run
+    for (int t = threadIdx.x; t < taps; t += blockDim.x) tap_sum[t] = 0;
+    const int classes = bc.nrc * bc.ncc;   // at most kMaxBorderClasses, fewer than threads
+    unsigned long long takes = 0;          // the taps of this thread's class that fall inside the image
+    if ((int)threadIdx.x < classes) {
+        const int rc = threadIdx.x / bc.ncc, cc = threadIdx.x - rc * bc.ncc;
+        unsigned long long row = 0;
+        for (int kw = 0; kw < d.kw; ++kw)
+            if (tap_valid(cc, kw, it.wo, d.w, bc.nlo_w, bc.nhi_w, bc.ncc, d.stride, d.pad)) row |= 1ull << kw;
+        for (int kh = 0; kh < d.kh; ++kh)
+            if (tap_valid(rc, kh, it.ho, d.h, bc.nlo_h, bc.nhi_h, bc.nrc, d.stride, d.pad)) takes |= row << (kh * d.kw);
+    }
+    ptx::grid_dep_wait_launch_small();
     auto load = [&](int i) {
         if (width == 16) return __ldg(reinterpret_cast<const int4 *>(w) + i);
         const int2 v = __ldg(reinterpret_cast<const int2 *>(w) + i);   // the 8-channel first layer: one 8-byte pixel per tap
@@ -1044,16 +1057,15 @@ __global__ void weight_prep_kernel(const __grid_constant__ PrepBatch b)
         const int i = threadIdx.x + u * blockDim.x;
         if (i < chunks) v[u] = load(i);
     }
-    for (int t = threadIdx.x; t < taps; t += blockDim.x) tap_sum[t] = 0;
-    const int classes = bc.nrc * bc.ncc;   // at most kMaxBorderClasses, fewer than threads
-    unsigned long long takes = 0;          // the taps of this thread's class that fall inside the image
-    if ((int)threadIdx.x < classes) {
-        const int rc = threadIdx.x / bc.ncc, cc = threadIdx.x - rc * bc.ncc;
-        unsigned long long row = 0;
-        for (int kw = 0; kw < d.kw; ++kw)
-            if (tap_valid(cc, kw, it.wo, d.w, bc.nlo_w, bc.nhi_w, bc.ncc, d.stride, d.pad)) row |= 1ull << kw;
-        for (int kh = 0; kh < d.kh; ++kh)
-            if (tap_valid(rc, kh, it.ho, d.h, bc.nlo_h, bc.nhi_h, bc.nrc, d.stride, d.pad)) takes |= row << (kh * d.kw);
+    if (it.w_rows) {
+        // this output channel's filter rows, each widened to 8 taps (c_in is 16 or 8: 4 or 2 words per tap)
+        const int words = d.c_in / 4;
+        const int32_t *src = reinterpret_cast<const int32_t *>(it.w) + (size_t)oc * taps * words;
+        int32_t *dst = reinterpret_cast<int32_t *>(it.w_rows) + (size_t)oc * d.kh * 8 * words;
+        for (int i = threadIdx.x; i < d.kh * 8 * words; i += blockDim.x) {
+            const int r = i / (8 * words), t = (i / words) % 8, wd = i % words;
+            dst[i] = t < d.kw ? __ldg(src + (r * d.kw + t) * words + wd) : 0;
+        }
     }
     __syncthreads();
     auto add = [&](int i, const int4 &q) {
@@ -1076,16 +1088,6 @@ __global__ void weight_prep_kernel(const __grid_constant__ PrepBatch b)
         int32_t sum = 0;
         for (unsigned long long m = takes; m; m &= m - 1) sum += tap_sum[__ffsll((long long)m) - 1];
         it.table[(size_t)threadIdx.x * d.c_out + oc] = sum;
-    }
-    if (it.w_rows) {
-        // this output channel's filter rows, each widened to 8 taps (c_in is 16 or 8: 4 or 2 words per tap)
-        const int words = d.c_in / 4;
-        const int32_t *src = reinterpret_cast<const int32_t *>(it.w) + (size_t)oc * taps * words;
-        int32_t *dst = reinterpret_cast<int32_t *>(it.w_rows) + (size_t)oc * d.kh * 8 * words;
-        for (int i = threadIdx.x; i < d.kh * 8 * words; i += blockDim.x) {
-            const int r = i / (8 * words), t = (i / words) % 8, wd = i % words;
-            dst[i] = t < d.kw ? __ldg(src + (r * d.kw + t) * words + wd) : 0;
-        }
     }
 }
 
