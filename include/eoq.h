@@ -437,7 +437,7 @@ EOQ_API int eoq_last_status(eoq_handle_t handle, void *stream, unsigned *bits);
 #define EOQ_PROF_IGEMM_FWD 0     /* the forward implicit-GEMM kernel, one launch per group */
 #define EOQ_PROF_IGEMM_DGRAD 1   /* the dgrad implicit-GEMM kernel, one launch per group */
 #define EOQ_PROF_WGRAD 2         /* the weight-gradient GEMM kernel */
-#define EOQ_PROF_ERR_HEAD 3      /* eoq_err_prescale (one kernel; two for tensors beyond the one-kernel capacity) */
+#define EOQ_PROF_ERR_HEAD 3      /* eoq_err_prescale (one kernel for small tensors, else two) */
 #define EOQ_PROF_DGRAD_AUX 4     /* Q_e phase 2 */
 #define EOQ_PROF_WGRAD_AUX 5     /* slice sum + b1 term + Q_g behind the weight-gradient GEMM */
 #define EOQ_PROF_FWD_AUX 6       /* b1 weight table, weight row padding (eoq_weight_prep, or per call without it) */

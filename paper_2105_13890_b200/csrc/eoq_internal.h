@@ -127,7 +127,7 @@ struct Handle {
     bool profiling;
     ReduceHook hook;              // all-reduce between the phases of every batch-wide reduction (data-parallel replicas)
     bool gemm_only;               // timing aid: dgrad and wgrad calls launch their GEMM kernel only (eoq_profile_gemm_only)
-    bool force_timeout;           // self-test: the next error-head call makes its grid-wide wait run out
+    bool force_timeout;           // self-test: the next error-head call is a bounded wait that runs out
     int num_records;
     ProfRecord *records;          // kMaxProfRecords entries, allocated on first eoq_profile_start
     int gemm_ctas;                // most CTAs a GEMM call of this handle may use (eoq_set_gemm_ctas; default: one per SM)

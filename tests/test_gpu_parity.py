@@ -554,7 +554,7 @@ def test_wgrad_two_kernel_finish_path():
 # ------------------------------------------------------------------ a bounded wait that runs out
 
 def test_wait_that_runs_out_reports_timeout_and_leaves_the_handle_usable():
-    """The grid-wide wait of the one-kernel error head is made to run out (it waits for one block more than
+    """A bounded wait in the place of an error head is made to run out (it waits for one arrival more than
     exists, with a short limit).  Nothing traps or hangs: the kernel returns, EOQ_DEV_TIMEOUT is reported, no output
     is written, the reduction cells are clean again, and the next call on the handle is bit-exact."""
     n_el = 1 << 16
