@@ -21,7 +21,7 @@
  *     library never allocates or frees tensor memory.  Tensor pointers must be
  *     16-byte aligned.  Scratch memory is the caller's `workspace` (device, 256-byte
  *     aligned, at least eoq_workspace_size() bytes; contents are undefined on
- *     entry and on return).  The handle owns only some kilobytes of device
+ *     entry and on return).  The handle owns some 64 KB of device
  *     state (status word, small reduction cells, the shifts of SQ's tiles).
  *     A handle serves one call at a time: calls that may overlap on the
  *     device (different streams) need a handle and a workspace each.
