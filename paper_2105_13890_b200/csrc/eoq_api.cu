@@ -1309,6 +1309,87 @@ struct JoinCall {
     const NextHeadArgs *next;
 };
 
+// A strided 1x1 filter without padding reaches only the pixels on the stride grid: its one GEMM leaves compact sums
+// [n][hq][wq][c_in] and Q_e scatters them into the full tensor (zeros elsewhere), so nothing is cleared.
+static bool compact_sums(const eoq_conv_desc_t &d)
+{
+    return d.kh == 1 && d.kw == 1 && d.pad == 0 && d.stride > 1 && (size_t)d.n * d.h * d.w * (d.c_in / 16) <= 0xffffffffull;
+}
+
+// First tap of each class of a launch, in error pixels (what the im2col loads start from).
+struct ClassCorners {
+    int dh[kMaxClasses], dw[kMaxClasses];
+};
+
+// The residue classes (y mod stride, x mod stride) of the input pixels that some tap reaches: within a class the taps kh with
+// (y + pad - kh) divisible by the stride form a unit-stride correlation over e3.  They write disjoint pixels, so up to kMaxClasses of
+// them share a launch, each with its share of the CTAs.  launch(classes, corners) is called for every launch, its GEMMs planned.
+template <typename Launch>
+static int each_class_launch(const eoq_conv_desc_t &d, bool compact, int sm_count, int ctas, Launch launch)
+{
+    IgemmClasses cl;
+    ClassCorners at;
+    cl.num = 0;
+    auto flush = [&]() -> int {
+        if (cl.num == 0) return EOQ_OK;
+        plan_classes(cl, ctas);
+        const int st = launch(cl, at);
+        cl.num = 0;
+        return st;
+    };
+    for (int py = 0; py < d.stride && py < d.h; ++py)
+        for (int px = 0; px < d.stride && px < d.w; ++px) {
+            int dh[16], dw[16], kh_of[16], kw_of[16], nh = 0, nw = 0, min_h = 0, min_w = 0;
+            for (int kh = 0; kh < d.kh; ++kh)
+                if ((py + d.pad - kh) % d.stride == 0) {
+                    // floor division is exact here; negative quotients are rows above the image
+                    dh[nh] = (py + d.pad - kh) / d.stride;
+                    kh_of[nh] = kh;
+                    if (dh[nh] < min_h) min_h = dh[nh];
+                    ++nh;
+                }
+            for (int kw = 0; kw < d.kw; ++kw)
+                if ((px + d.pad - kw) % d.stride == 0) {
+                    dw[nw] = (px + d.pad - kw) / d.stride;
+                    kw_of[nw] = kw;
+                    if (dw[nw] < min_w) min_w = dw[nw];
+                    ++nw;
+                }
+            if (nh == 0 || nw == 0) continue;  // no tap reaches this class: its sums stay zero
+            int st = EOQ_OK;
+            if (cl.num == kMaxClasses && (st = flush()) != EOQ_OK) return st;
+            at.dh[cl.num] = min_h;
+            at.dw[cl.num] = min_w;
+            IgemmParams &p = cl.p[cl.num++];
+            memset(&p, 0, sizeof(p));
+            p.hq = (d.h - py + d.stride - 1) / d.stride;
+            p.wq = (d.w - px + d.stride - 1) / d.stride;
+            p.M = d.n * p.hq * p.wq;
+            p.N = d.c_in;
+            p.b_mn = 1;   // (the weights stay where they are, as for the patch kernel)
+            plan_igemm(p, d.c_out, nh * nw, sm_count);
+            p.src_stride = 1;
+            p.src_stride_w = 1;
+            p.base_h = min_h;
+            p.base_w = min_w;
+            for (int a = 0; a < nh; ++a)
+                for (int b = 0; b < nw; ++b) {
+                    const int t = a * nw + b;
+                    if (dh[a] - min_h > 255 || dw[b] - min_w > 255) return EOQ_ERR_UNSUPPORTED;
+                    p.tap_dh[t] = (unsigned char)(dh[a] - min_h);
+                    p.tap_dw[t] = (unsigned char)(dw[b] - min_w);
+                    p.tap_b[t] = (unsigned char)(kh_of[a] * d.kw + kw_of[b]);
+                }
+            p.out_h = compact ? p.hq : d.h;
+            p.out_w = compact ? p.wq : d.w;
+            p.out_step = compact ? 1 : d.stride;
+            p.out_off_h = py;
+            p.out_off_w = px;
+            p.epilogue = kEpiDgrad;
+        }
+    return flush();
+}
+
 // `next`: the error head of the layer that consumes e4, fused into Q_e (null for the plain call); `jc`: see JoinCall
 static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, const int8_t *e3, const int32_t *e3_exp,
                            const int8_t *w, int8_t *e4, int32_t *e4_exp, int64_t *sum_e4, int32_t *acc_dump,
@@ -1383,8 +1464,6 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     long long *const zero_sums[4] = {reinterpret_cast<long long *>(sum_e4), jc ? jc->sum_out : nullptr, any_next ? any_next->sum_e1 : nullptr,
                                      any_next ? any_next->sum_e1x2 : nullptr};
 
-    // One GEMM per residue class (y mod stride, x mod stride) of the input pixels: within a class the taps
-    // kh with (y + pad - kh) divisible by the stride form a unit-stride correlation over e3.
     if (d.stride == 1 && d.kh == d.kw && d.kh - 1 - d.pad >= 0) {
         // stride 1: one correlation of e3 with the flipped filter, padding k - 1 - pad
         IgemmParams p;
@@ -1435,98 +1514,36 @@ static int conv_dgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
         for (int kw = 0; kw < d.kw; ++kw) hit_w |= (r + d.pad - kw) % d.stride == 0;
         any_empty |= (r < d.h && !hit_h) || (r < d.w && !hit_w);
     }
-    // A strided 1x1 filter without padding reaches only the pixels on the stride grid: its one GEMM leaves compact
-    // sums [n][hq][wq][c_in] and Q_e scatters them into the full tensor (zeros elsewhere), so nothing is cleared.
-    const bool compact = d.kh == 1 && d.kw == 1 && d.pad == 0 && d.stride > 1 && !acc_dump &&
-                         (size_t)d.n * d.h * d.w * (d.c_in / 16) <= 0xffffffffull;
+    const bool compact = !acc_dump && compact_sums(d);
     if (any_empty && !compact) {
         e = acc_dump ? cudaMemsetAsync(acc_dump, 0, g.in_elems * sizeof(int32_t), s)
                      : cudaMemsetAsync(sums16, 0, g.in_elems * sizeof(uint16_t), s);
         if (e != cudaSuccess) return record(h, e);
     }
-    // The classes write disjoint pixels: up to kMaxClasses of them share a launch, each with its share of the CTAs.
-    IgemmClasses cl;
-    cl.num = 0;
-    int dw_of[kMaxClasses], dh_of[kMaxClasses];
-    auto launch_classes = [&]() -> int {
-        if (cl.num == 0) return EOQ_OK;
-        plan_classes(cl, h->gemm_ctas);
+    int classes = 0;
+    st = each_class_launch(d, compact, h->sm_count, h->gemm_ctas, [&](IgemmClasses &cl, const ClassCorners &at) -> int {
         for (int k = 0; k < cl.num; ++k) {
-            const IgemmParams &p = cl.p[k];
-            if (!make_im2col_map(&cl.map_a[k], e3, d.n, g.ho, g.wo, d.c_out, dw_of[k], dh_of[k], p.wq, p.hq, 1, p.kc, p.a_rows) ||
-                !make_weight_map(&cl.map_b[k], w, d.c_out, g.taps, d.c_in, p.b_row, p.kc))
-                return EOQ_ERR_UNSUPPORTED;
-        }
-        count_launches(h, 1);
-        ProfScope prof(h, EOQ_PROF_IGEMM_DGRAD, s);
-        e = cl.num == 1 ? launch_igemm(cl.p[0], cl.map_a[0], cl.map_b[0], cl.first[1], s) : launch_igemm_classes(cl, s);
-        cl.num = 0;
-        if (e != cudaSuccess) {
-            launch_reset_cells(h->dev, s);  // GEMMs already queued have touched the maximum cell
-            return record(h, e);
-        }
-        return EOQ_OK;
-    };
-    int class_no = 0;
-    for (int py = 0; py < d.stride && py < d.h; ++py)
-        for (int px = 0; px < d.stride && px < d.w; ++px) {
-            int dh[16], dw[16], kh_of[16], kw_of[16], nh = 0, nw = 0, min_h = 0, min_w = 0;
-            for (int kh = 0; kh < d.kh; ++kh)
-                if ((py + d.pad - kh) % d.stride == 0) {
-                    // floor division is exact here; negative quotients are rows above the image
-                    dh[nh] = (py + d.pad - kh) / d.stride;
-                    kh_of[nh] = kh;
-                    if (dh[nh] < min_h) min_h = dh[nh];
-                    ++nh;
-                }
-            for (int kw = 0; kw < d.kw; ++kw)
-                if ((px + d.pad - kw) % d.stride == 0) {
-                    dw[nw] = (px + d.pad - kw) / d.stride;
-                    kw_of[nw] = kw;
-                    if (dw[nw] < min_w) min_w = dw[nw];
-                    ++nw;
-                }
-            const int hq = (d.h - py + d.stride - 1) / d.stride, wq = (d.w - px + d.stride - 1) / d.stride;
-            if (nh == 0 || nw == 0) continue;  // no tap reaches this class: its sums stay zero
-            if (cl.num == kMaxClasses && (st = launch_classes()) != EOQ_OK) return st;
-            dh_of[cl.num] = min_h;
-            dw_of[cl.num] = min_w;
-            IgemmParams &p = cl.p[cl.num++];
-            memset(&p, 0, sizeof(p));
-            ++class_no;
-            p.M = d.n * hq * wq;
-            p.N = d.c_in;
-            p.hq = hq;
-            p.wq = wq;
-            p.b_mn = 1;   // (the weights stay where they are, as for the patch kernel)
-            plan_igemm(p, d.c_out, nh * nw, h->sm_count);
-            p.src_stride = 1;
-            p.src_stride_w = 1;
-            p.base_h = min_h;
-            p.base_w = min_w;
-            for (int a = 0; a < nh; ++a)
-                for (int b = 0; b < nw; ++b) {
-                    const int t = a * nw + b;
-                    if (dh[a] - min_h > 255 || dw[b] - min_w > 255) return EOQ_ERR_UNSUPPORTED;
-                    p.tap_dh[t] = (unsigned char)(dh[a] - min_h);
-                    p.tap_dw[t] = (unsigned char)(dw[b] - min_w);
-                    p.tap_b[t] = (unsigned char)(kh_of[a] * d.kw + kw_of[b]);
-                }
-            p.out_h = compact ? hq : d.h;
-            p.out_w = compact ? wq : d.w;
-            p.out_step = compact ? 1 : d.stride;
-            p.out_off_h = py;
-            p.out_off_w = px;
-            p.epilogue = kEpiDgrad;
+            IgemmParams &p = cl.p[k];
             memcpy(p.zero_sums, zero_sums, sizeof(zero_sums));
             p.acc_out = acc_dump;
             p.sums16 = sums16;
             p.dev = h->dev;
             p.next_mask = next ? next->mask : nullptr;
+            if (!make_im2col_map(&cl.map_a[k], e3, d.n, g.ho, g.wo, d.c_out, at.dw[k], at.dh[k], p.wq, p.hq, 1, p.kc, p.a_rows) ||
+                !make_weight_map(&cl.map_b[k], w, d.c_out, g.taps, d.c_in, p.b_row, p.kc))
+                return EOQ_ERR_UNSUPPORTED;
         }
-    if ((st = launch_classes()) != EOQ_OK) return st;
+        classes += cl.num;
+        count_launches(h, 1);
+        ProfScope prof(h, EOQ_PROF_IGEMM_DGRAD, s);
+        const cudaError_t err = cl.num == 1 ? launch_igemm(cl.p[0], cl.map_a[0], cl.map_b[0], cl.first[1], s) : launch_igemm_classes(cl, s);
+        if (err == cudaSuccess) return EOQ_OK;
+        launch_reset_cells(h->dev, s);  // GEMMs already queued have touched the maximum cell
+        return record(h, err);
+    });
+    if (st != EOQ_OK) return st;
     if (h->gemm_only) return EOQ_OK;
-    if (class_no == 0)   // no tap reaches any pixel: no GEMM ran
+    if (classes == 0)   // no tap reaches any pixel: no GEMM ran
         for (long long *z : zero_sums)
             if (z && (e = cudaMemsetAsync(z, 0, sizeof(*z), s)) != cudaSuccess) return record(h, e);
     // Q_e over the whole tensor: the maximum is complete only now
@@ -1902,13 +1919,34 @@ extern "C" int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *des
                      igemm_patch_lean(p, pl) ? " registers=72" : "");
             return EOQ_OK;
         }
-        const int hq = (d.h + d.stride - 1) / d.stride, wq = (d.w + d.stride - 1) / d.stride;
-        p.M = d.n * hq * wq;
-        p.N = d.c_in;
-        plan_igemm(p, d.c_out, ((d.kh + d.stride - 1) / d.stride) * ((d.kw + d.stride - 1) / d.stride), h->sm_count);
-        if (d.stride == 1) plan_few_tiles(p, h->gemm_ctas);
-        snprintf(buf, buf_bytes, "kernel=igemm classes=%d tile_n=%d m_tiles=%d n_tiles=%d kc=%d split=%d", d.stride * d.stride, p.tile_n,
-                 p.num_m_tiles, p.num_n_tiles, p.kc, p.split);
+        // as the call without a dump of the sums: a number per class, the classes of a launch apart by commas, launches by slashes
+        struct List {
+            char text[256];
+            size_t used;
+            void add(const char *separator, int v)
+            {
+                const int n = snprintf(text + used, sizeof(text) - used, "%s%d", separator, v);
+                if (n > 0) used = used + n < sizeof(text) ? used + n : sizeof(text) - 1;
+            }
+        } tile_n = {}, m_tiles = {}, n_tiles = {}, ctas = {}, split = {};
+        int classes = 0, launches = 0, kc = 0;
+        st = each_class_launch(d, compact_sums(d), h->sm_count, h->gemm_ctas, [&](const IgemmClasses &cl, const ClassCorners &) -> int {
+            const char *const next_launch = launches++ ? "/" : "";
+            for (int k = 0; k < cl.num; ++k) {
+                const char *const separator = k ? "," : next_launch;
+                tile_n.add(separator, cl.p[k].tile_n);
+                m_tiles.add(separator, cl.p[k].num_m_tiles);
+                n_tiles.add(separator, cl.p[k].num_n_tiles);
+                ctas.add(separator, cl.first[k + 1] - cl.first[k]);
+                kc = cl.p[k].kc;
+            }
+            split.add(next_launch, cl.p[0].split);
+            classes += cl.num;
+            return EOQ_OK;
+        });
+        if (st != EOQ_OK) return st;
+        snprintf(buf, buf_bytes, "kernel=igemm classes=%d tile_n=%s m_tiles=%s n_tiles=%s kc=%d split=%s launches=%d ctas=%s", classes, tile_n.text,
+                 m_tiles.text, n_tiles.text, kc, split.text, launches, ctas.text);
         return EOQ_OK;
     }
     if (pass == EOQ_PASS_WGRAD) {

@@ -412,8 +412,8 @@ def eoq_update_part(handle, first: int, last: bool, w: Sequence, g: Sequence, g_
 
 
 def eoq_describe_plan(handle, desc, pass_: int) -> str:
-    buf = C.create_string_buffer(256)
-    _check(lib().eoq_describe_plan(handle, C.byref(desc), int(pass_), buf, 256), "eoq_describe_plan")
+    buf = C.create_string_buffer(1024)
+    _check(lib().eoq_describe_plan(handle, C.byref(desc), int(pass_), buf, 1024), "eoq_describe_plan")
     return buf.value.decode()
 
 

@@ -66,3 +66,40 @@ def test_scattered_codes(d):
                        G.workspace(gd, eoq.EOQ_PASS_DGRAD))
     assert G.status_clear() == 0 and np.array_equal(G.host(e4), want) and e4_exp.item() == p
     assert total.item() == int(want.astype(np.int64).sum())
+
+
+@pytest.mark.parametrize("cap", [0, 7])
+@pytest.mark.parametrize("d", GEOMETRIES, ids=lambda d: "n%d_%dx%d_%d_%d_k%ds%d" % (d.n, d.h, d.w, d.c_in, d.c_out, d.kh, d.stride))
+def test_the_report_names_what_is_launched(d, cap):
+    """Classes that a tap reaches, with their tiles and their shares of the CTAs, and the launches of the call."""
+    gd, h = G.gdesc(d), eoq.eoq_create(0)
+    if cap:
+        eoq.eoq_set_gemm_ctas(h, cap)
+    plan = dict(f.split("=") for f in eoq.eoq_describe_plan(h, gd, eoq.EOQ_PASS_DGRAD).split())
+
+    def pixels(extent, k, r):
+        return len(range(r, extent, d.stride)) if any((r + d.pad - q) % d.stride == 0 for q in range(k)) else 0
+
+    rows = [d.n * pixels(d.h, d.kh, py) * pixels(d.w, d.kw, px) for py in range(d.stride) for px in range(d.stride)]
+    live = [m for m in rows if m]
+    if plan["kernel"] == "igemm":
+        launches = -(-len(live) // 4)
+        numbers = {f: [[int(v) for v in part.split(",")] for part in plan[f].split("/")] for f in ("tile_n", "m_tiles", "n_tiles", "ctas", "split")}
+        assert int(plan["classes"]) == len(live) and int(plan["launches"]) == launches
+        assert sum(numbers["m_tiles"], []) == [-(-m // 128) for m in live]
+        assert all(n == -(-d.c_in // t) for n, t in zip(sum(numbers["n_tiles"], []), sum(numbers["tile_n"], [])))
+        for tiles_m, tiles_n, ctas, (split,) in zip(numbers["m_tiles"], numbers["n_tiles"], numbers["ctas"], numbers["split"]):
+            assert sum(ctas) <= max(cap or torch.cuda.get_device_properties(0).multi_processor_count, len(ctas))
+            assert all(c % split == 0 and c <= m * n * split for c, m, n in zip(ctas, tiles_m, tiles_n))
+            assert split == 1 or ctas == [m * n * split for m, n in zip(tiles_m, tiles_n)]   # (a cluster has one tile)
+        if (d.n, d.c_out, d.stride, cap) == (1, 512, 2, 0):
+            assert numbers["split"][0][0] > 1
+    else:
+        launches = 1
+    e4, e4_exp = G.empty((d.n, d.h, d.w, d.c_in), torch.int8), G.zeros(1, torch.int32)
+    before = eoq.eoq_launch_count(h)
+    eoq.eoq_conv_dgrad(h, gd, G.zeros((d.n, d.ho, d.wo, d.c_out), torch.int8), G.zeros(1, torch.int32), G.zeros((d.c_out, d.kh, d.kw, d.c_in), torch.int8),
+                       e4, e4_exp, None, None, G.workspace(gd, eoq.EOQ_PASS_DGRAD))
+    assert eoq.eoq_launch_count(h) - before == launches + 1   # Q_e behind them
+    eoq.eoq_last_status(h)   # (an error that is all zero is flagged)
+    eoq.eoq_destroy(h)
