@@ -424,22 +424,28 @@ void plan_classes(IgemmClasses &cl, int ctas)
         cost[k] = 2 * cl.p[k].ntaps + 1;
         work += (long long)tiles[k] * cost[k];
     }
-    // (a time of all tiles on a single CTA each is always enough: the search ends)
-    for (long long time = work / ctas;; ++time) {
+    // The least time from work / ctas on in which the classes get by with `ctas` CTAs, or with one each: by bisection, as they need fewer
+    // the longer it is, and one each once it covers all tiles of every class.  (Counted up one by one, 12,544 tiles a class under a cap of three
+    // CTAs took 20,908 steps.)
+    auto divide = [&](long long time) -> bool {
         int used = 0;
-        bool fits = true;
         cl.first[0] = 0;
         for (int k = 0; k < cl.num; ++k) {
             const long long per_cta = cl.p[0].split > 1 ? 1 : time / cost[k];   // (a cluster has one tile)
-            if (per_cta < 1) {
-                fits = false;
-                break;
-            }
+            if (per_cta < 1) return false;
             used += (int)((tiles[k] + per_cta - 1) / per_cta);
             cl.first[k + 1] = used * cl.p[0].split;
         }
-        if (fits && (used <= ctas || used <= cl.num)) break;
+        return used <= ctas || used <= cl.num;
+    };
+    long long low = work / ctas, high = low;   // `high` is enough, times below `low` are not
+    for (int k = 0; k < cl.num; ++k) high = std::max(high, (long long)tiles[k] * cost[k]);
+    while (low < high) {
+        const long long mid = (low + high) / 2;
+        if (divide(mid)) high = mid;
+        else low = mid + 1;
     }
+    divide(high);
     for (int k = 0; k < cl.num; ++k) plan_epilogue(cl.p[k], (cl.first[k + 1] - cl.first[k]) / cl.p[0].split);
 }
 

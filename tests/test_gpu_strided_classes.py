@@ -1,5 +1,7 @@
 """Error back-propagation by the im2col kernel: the residue classes of a strided layer share launches of up to four GEMMs, and the
 weights are read where they are whatever the number of channels."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -102,4 +104,32 @@ def test_the_report_names_what_is_launched(d, cap):
                        e4, e4_exp, None, None, G.workspace(gd, eoq.EOQ_PASS_DGRAD))
     assert eoq.eoq_launch_count(h) - before == launches + 1   # Q_e behind them
     eoq.eoq_last_status(h)   # (an error that is all zero is flagged)
+    eoq.eoq_destroy(h)
+
+
+@pytest.mark.parametrize("cap", [1, 3, 5, 7, 148])
+@pytest.mark.parametrize("d", [
+    oracle.ConvDesc(512, 112, 112, 16, 16, 3, 3, 2, 1),   # 12,544 tiles a class
+    oracle.ConvDesc(300, 61, 53, 96, 48, 3, 3, 2, 1),     # classes of other sizes
+    oracle.ConvDesc(64, 64, 64, 32, 64, 2, 2, 2, 0),      # four classes of one tap
+], ids=lambda d: "n%d_%dx%d_%d_%d_k%ds%d" % (d.n, d.h, d.w, d.c_in, d.c_out, d.kh, d.stride))
+def test_shares_of_the_classes(d, cap):
+    """The division of the CTAs is that of the least time that suffices, counted up one by one; a plan of many tiles under a small cap
+    is quick on the host all the same (12,544 tiles a class under three CTAs, counted up: 0.36 ms)."""
+    gd, h = G.gdesc(d), eoq.eoq_create(0)
+    eoq.eoq_set_gemm_ctas(h, cap)
+    quickest = 1.0
+    for _ in range(20):
+        t = time.perf_counter()
+        text = eoq.eoq_describe_plan(h, gd, eoq.EOQ_PASS_DGRAD)
+        quickest = min(quickest, time.perf_counter() - t)
+    plan = dict(f.split("=") for f in text.split())
+    taps = [sum((r + d.pad - k) % d.stride == 0 for k in range(d.kh)) for r in range(d.stride)]
+    cost = [2 * a * b + 1 for a in taps for b in taps]
+    tiles = [int(m) * int(n) for m, n in zip(plan["m_tiles"].split(","), plan["n_tiles"].split(","))]
+    at = sum(c * t for c, t in zip(cost, tiles)) // cap
+    while at < max(cost) or not (sum(-(-t // (at // c)) for c, t in zip(cost, tiles)) <= max(cap, len(tiles))):
+        at += 1
+    assert [int(c) for c in plan["ctas"].split(",")] == [-(-t // (at // c)) for c, t in zip(cost, tiles)]
+    assert quickest < 1.5e-4
     eoq.eoq_destroy(h)
