@@ -2129,7 +2129,7 @@ extern "C" int eoq_quantize_image(eoq_handle_t handle, const float *src, int n, 
     if ((c_dst % 16 && c_dst != 8) || c_dst > 64 || !aligned16(src) || !aligned16(dst)) return EOQ_ERR_ALIGNMENT;
     count_launches(h, 2);
     ProfScope prof(h, EOQ_PROF_INPUT_Q, reinterpret_cast<cudaStream_t>(stream));
-    return record(h, launch_quantize_image(src, n, hh, ww, c_src, c_dst, wmargin, dst, dst_exp, h->tile_shift, h->dev, h->sm_count,
+    return record(h, launch_quantize_image(src, n, hh, ww, c_src, c_dst, wmargin, dst, dst_exp, h->dev,
                                            reinterpret_cast<cudaStream_t>(stream), h->hook));
 }
 

@@ -58,27 +58,86 @@ __device__ __forceinline__ void quantize_store4(void *dst, size_t i, const Pow2S
     else reinterpret_cast<uint32_t *>(dst)[i] = pack4_sat(a, b, c, d);
 }
 
-// kMode 0: Q -> int16, 1: CQ -> int8.  Bound by memory: 4 B in, 1 or 2 B out.  A block takes one tile of kQuantTile float4, eight
-// independent, coalesced loads per thread.
-constexpr int kQuantLoads = 8, kQuantTile = kThreads * kQuantLoads;
-template <int kMode>
-__global__ void __launch_bounds__(kThreads)
-quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp)
+__device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ uint32_t abs_bits(const float4 &v)
 {
-    ptx::grid_dep_wait_launch_small();
-    const size_t n4 = n / 4, base = (size_t)blockIdx.x * kQuantTile + threadIdx.x;
-    float4 v[kQuantLoads];
+    return max(max(abs_bits(v.x), abs_bits(v.y)), max(abs_bits(v.z), abs_bits(v.w)));
+}
+
+// A block takes one tile of kQuantTile float4, eight independent, coalesced loads per thread.
+constexpr int kQuantLoads = 8, kQuantTile = kThreads * kQuantLoads;
+__device__ __forceinline__ void load_tile(const float *__restrict__ src, size_t n4, size_t tile, float4 (&v)[kQuantLoads])
+{
 #pragma unroll
     for (int u = 0; u < kQuantLoads; ++u) {
-        const size_t i = base + (size_t)u * kThreads;
-        if (i < n4) v[u] = __ldg(reinterpret_cast<const float4 *>(src) + i);
+        const size_t i = tile * kQuantTile + (size_t)u * kThreads + threadIdx.x;
+        v[u] = i < n4 ? __ldg(reinterpret_cast<const float4 *>(src) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    constexpr int up = 7;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && dst_exp) *dst_exp = -up;
+}
+
+// ------------------------------------------------------------------ SQ of a tensor beyond one cluster, and of images
+// Two passes: the maximum, then the codes, the second read out of the L2.  Whole tiles of loads are in flight in both, and the second
+// pass's blocks read theirs while the first pass ends.  Floats from memory, what a row of calls on other tensors takes each: 1 M 4.8 us, 4 M
+// 7.2, 12.8 M 17.1 (of one tensor again and again 4.0, 5.7 and 11.0).  A pass for the maximum with one load of a thread in flight: 5.6, 9.3 and
+// 20.8.  Codes formed in the first pass under a guess, and again where the guess was wrong: 5.0, 8.8 and 15.9 where it never is, 6.2, 10.9
+// and 18.8 under one element beyond all others; 64 images 224 x 224 18.5 and 25.9, so 19.9 whatever they hold.
+
+// First pass: the largest |x|.  Bound by memory (4 B in).
+__global__ void __launch_bounds__(kThreads) absmax_f32_kernel(const float *__restrict__ src, size_t n, DeviceState *dev)
+{
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    float4 v[kQuantLoads];
+    load_tile(src, n / 4, blockIdx.x, v);
+    uint32_t mx = 0;
+    if (blockIdx.x == 0 && threadIdx.x < (n & 3)) mx = abs_bits(src[n / 4 * 4 + threadIdx.x]);
+#pragma unroll
+    for (int u = 0; u < kQuantLoads; ++u) mx = max(mx, abs_bits(v[u]));
+    mx = block_max_u32(mx);
+    if (threadIdx.x == 0) {
+        if (mx) atomicMax(&dev->absmax_u32, mx);
+        if (mx >= 0x7f800000u) atomicOr(&dev->status, EOQ_DEV_NONFINITE);
+    }
+}
+
+// What a block of SQ's second pass does with the maximum once its operands are on their way: the shift, and the exponent (one block).
+// All threads; `tid` in the block.  True in one thread of the grid, which clears the cell when its block is done.
+__device__ __forceinline__ bool sq_shift(int tid, int32_t *dst_exp, DeviceState *dev, int *up)
+{
+    __shared__ uint32_t max_s;
+    if (tid == 0) max_s = *reinterpret_cast<volatile uint32_t *>(&dev->absmax_u32);
+    __syncthreads();
+    *up = sq_up(max_s);
+    if (tid != 0) return false;
+    if (blockIdx.x == 0) {
+        *dst_exp = -*up;
+        if (max_s == 0) atomicOr(&dev->status, EOQ_DEV_SQ_ZERO);
+    }
+    return last_reader(dev);
+}
+
+// kMode 0: Q -> int16, 1: CQ -> int8, 2: SQ -> int8 under the reduced maximum (tiles backwards: the first pass read the last ones last).
+// Bound by memory: 4 B in (SQ: from L2 where it holds the tensor), 1 or 2 B out.
+// early (SQ): the first pass is the launch in front and lets this one in once the source is complete, so its tiles are read ahead of
+// the wait.
+template <int kMode>
+__global__ void __launch_bounds__(kThreads)
+quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev, int early)
+{
+    const size_t n4 = n / 4, tile = kMode == 2 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    if (!early) ptx::grid_dep_wait();
+    float4 v[kQuantLoads];
+    load_tile(src, n4, tile, v);
+    if (early) ptx::grid_dep_wait();
+    if (gridDim.x <= kPartSms) ptx::grid_dep_launch();
+    int up = 7;
+    bool last = false;
+    if (kMode == 2) last = sq_shift(threadIdx.x, dst_exp, dev, &up);
+    else if (blockIdx.x == 0 && threadIdx.x == 0 && dst_exp) *dst_exp = -up;
     const Pow2Scale sc = pow2_scale(up);
 #pragma unroll
     for (int u = 0; u < kQuantLoads; ++u) {
-        const size_t i = base + (size_t)u * kThreads;
+        const size_t i = tile * kQuantTile + (size_t)u * kThreads + threadIdx.x;
         if (i < n4) quantize_store4<kMode>(dst, i, sc, v[u]);
     }
     if (blockIdx.x == 0 && threadIdx.x < (n & 3)) {
@@ -87,15 +146,15 @@ quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t 
         if (kMode == 0) reinterpret_cast<int16_t *>(dst)[i] = (int16_t)c;
         else reinterpret_cast<int8_t *>(dst)[i] = (int8_t)c;
     }
+    if (last) dev->absmax_u32 = 0;
 }
 
-// ------------------------------------------------------------------ SQ of a tensor beyond one cluster
-// The codes of SQ depend on the tensor's maximum through R(log2 max) alone, and a tile of a few thousand elements mostly has the
-// tensor's R(log2 max) already.  So the first pass reads the tensor once, codes every tile under the larger of its own maximum
-// and what other blocks have reduced by then, and leaves the shift it used; the second pass, under the whole maximum, codes again
-// the tiles whose shift was another one, and returns where there are none.  Bound by memory.  12.8 M normal floats from memory: 13.1
-// us for a maximum's pass and 8.2 for the codes before; now 12.3 + 3.7, of which the second returns at once, and 12.6 + 6.4 where every
-// tile was wrong (one element beyond all others).  4 M floats: 6.3 + 3.9 before, 6.2 + 3.1 now, 6.0 + 6.0 at worst.
+// ------------------------------------------------------------------ SQ of a tensor beyond the L2 cache
+// A second read comes from memory there.  The codes depend on the tensor's maximum through R(log2 max) alone, and a tile of a few
+// thousand elements often has the tensor's R(log2 max) already.  So the first pass codes every tile under the larger of its own maximum
+// and what other blocks have reduced by then, and leaves the shift it used; the second pass, under the whole maximum, codes again the
+// tiles whose shift was another one, and returns where there are none.  Bound by memory.  28 M normal floats, from memory: 27.8 us, 38.6 under
+// one element beyond all others, 37.9 in either case when read twice; 24 M 25 to 34, and 32 when read twice.
 
 // shift of a tile: what its codes were formed under, or one of
 constexpr int kTileAny = 0x7fff;     // all of it is zero: codes 0 under any shift
@@ -135,7 +194,7 @@ struct TileGuess {
 };
 
 // Second pass: calls again(tile, scale) in all threads of a block for those of its tiles that need it; tiles are dealt out from the
-// tensor's end, which the first pass read last.  `owner`: the thread that writes the exponent.
+// tensor's end, which the first pass read last.  Thread 0 of block 0 writes the exponent.
 template <typename Again>
 __device__ __forceinline__ void recode_tiles(const int16_t *tile_shift, int tiles, int tid, int32_t *dst_exp, DeviceState *dev, Again again)
 {
@@ -164,15 +223,7 @@ __device__ __forceinline__ void recode_tiles(const int16_t *tile_shift, int tile
     if (last) dev->absmax_u32 = 0;
 }
 
-// Part `p` of the tensor is kQuantTile float4; a tile is `reps` of them.
-__device__ __forceinline__ void load_part(const float *src, size_t n4, size_t p, float4 (&v)[kQuantLoads])
-{
-#pragma unroll
-    for (int u = 0; u < kQuantLoads; ++u) {
-        const size_t i = p * kQuantTile + (size_t)u * kThreads + threadIdx.x;
-        v[u] = i < n4 ? __ldg(reinterpret_cast<const float4 *>(src) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-}
+// Part `p` of the tensor is a tile of load_tile; a tile here is `reps` of them.
 __device__ __forceinline__ void store_part(int8_t *dst, size_t n4, size_t p, const Pow2Scale &sc, const float4 (&v)[kQuantLoads])
 {
 #pragma unroll
@@ -181,7 +232,6 @@ __device__ __forceinline__ void store_part(int8_t *dst, size_t n4, size_t p, con
         if (i < n4) quantize_store4<2>(dst, i, sc, v[u]);
     }
 }
-__device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
 
 __global__ void __launch_bounds__(kThreads)
 quantize_sq_kernel(const float *__restrict__ src, size_t n, int8_t *dst, int16_t *tile_shift, int reps, DeviceState *dev)
@@ -192,13 +242,13 @@ quantize_sq_kernel(const float *__restrict__ src, size_t n, int8_t *dst, int16_t
     for (int r = 0; r < reps; ++r) {
         const size_t p = (size_t)blockIdx.x * reps + r;
         float4 v[kQuantLoads];
-        load_part(src, n4, p, v);
+        load_tile(src, n4, p, v);
         uint32_t mx = 0;
         // (the up to three elements behind the last float4 are coded by the second pass)
         if (blockIdx.x == 0 && r == 0 && threadIdx.x < (n & 3)) mx = abs_bits(src[n4 * 4 + threadIdx.x]);
 #pragma unroll
         for (int u = 0; u < kQuantLoads; ++u)
-            mx = max(max(mx, max(abs_bits(v[u].x), abs_bits(v[u].y))), max(abs_bits(v[u].z), abs_bits(v[u].w)));
+            mx = max(mx, abs_bits(v[u]));
         store_part(dst, n4, p, pow2_scale(guess.part(mx, threadIdx.x, dev)), v);
     }
     guess.publish(threadIdx.x, tile_shift + blockIdx.x, dev);
@@ -217,7 +267,7 @@ quantize_sq_again_kernel(const float *__restrict__ src, size_t n, int8_t *dst, i
     recode_tiles(tile_shift, tiles, threadIdx.x, dst_exp, dev, [&](int tile, const Pow2Scale &sc) {
         for (int r = 0; r < reps; ++r) {
             float4 v[kQuantLoads];
-            load_part(src, n4, (size_t)tile * reps + r, v);
+            load_tile(src, n4, (size_t)tile * reps + r, v);
             store_part(dst, n4, (size_t)tile * reps + r, sc, v);
         }
     });
@@ -271,16 +321,14 @@ quantize_sq_small_kernel(const float *__restrict__ src, size_t n, int8_t *dst, i
     cluster.sync();  // no block leaves while another may still read its maximum
 }
 
-// SQ of an fp32 image: c_src channels in, c_dst (zero-padded) channels out, rows widened by `wmargin` zero pixels at both ends.  A
-// thread writes kG = 16 or 8 channels of a pixel.  The same two passes: a part is kImageRows * blockDim.y rows, a tile `reps` of them.
-// Bound by memory (12 B in, 8 or 16 B out per RGB pixel).  A block is tx pixels x ty rows and a thread takes its pixel in
-// kImageRows rows, all loads issued before the maximum is needed, no divisions.  64 images 224 x 224: 10.7 us for the maximum and 13.4
-// for the codes before; now 16.0 + 2.8, and 16.0 + 13.6 where every tile was wrong.
+// SQ of an fp32 image under the reduced maximum: c_src channels in, c_dst (zero-padded) channels out, rows widened by `wmargin` zero
+// pixels at both ends.  A thread writes kG = 16 or 8 channels of a pixel.  Bound by memory (12 B in, 8 or 16 B out per RGB pixel).  A block is
+// tx pixels x ty rows and a thread takes its pixel in kImageRows rows, all loads issued before the maximum is needed, no divisions.
 constexpr int kImageRows = 4;
 struct ImageShape {
     int rows, w, c_src, c_dst, wmargin;
 };
-// 16 or 8 codes of an output pixel from the values of its channels (`more`: those beyond the first four, read again)
+// 16 or 8 codes of an output pixel from the values of its channels (`more`: those beyond the first four, read here)
 template <int kG>
 __device__ __forceinline__ void image_store(int8_t *dst, size_t o, const Pow2Scale &sc, const float (&v)[4], const float *more, int nch)
 {
@@ -295,116 +343,81 @@ __device__ __forceinline__ void image_store(int8_t *dst, size_t o, const Pow2Sca
         reinterpret_cast<uint2 *>(dst)[o] = make_uint2(pack4_sat(c[0], c[1], c[2], c[3]), pack4_sat(c[4], c[5], c[6], c[7]));
 }
 
-// One part (`first_row`: the thread's first): scale_of(maximum of the thread's channels) gives the scale, once per round of a row
-// (one unless a row is wider than the block).
-template <int kG, typename ScaleOf>
-__device__ __forceinline__ void image_part(const float *__restrict__ src, const ImageShape &s, int first_row, int8_t *dst, ScaleOf scale_of)
-{
-    const int groups = s.c_dst / kG, items = (s.w + 2 * s.wmargin) * groups;
-    for (int x0 = 0; x0 < items; x0 += blockDim.x) {
-        const int it = x0 + threadIdx.x;
-        const int xp = groups == 1 ? it : it / groups, g = groups == 1 ? 0 : it - xp * groups, xm = xp - s.wmargin;
-        const int nch = min(kG, s.c_src - g * kG);       // real channels of this group (none or fewer beyond c_src)
-        const bool in = it < items && xm >= 0 && xm < s.w;
-        float v[kImageRows][4];
-        uint32_t mx = 0;
-#pragma unroll
-        for (int u = 0; u < kImageRows; ++u) {
-            const int row = first_row + u * blockDim.y;
-            const float *p = src + ((size_t)row * s.w + xm) * s.c_src + g * kG;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) v[u][k] = (in && row < s.rows && k < nch) ? __ldg(p + k) : 0.0f;
-            if (in && row < s.rows)
-                for (int k = 4; k < nch; ++k) mx = max(mx, abs_bits(__ldg(p + k)));
-        }
-#pragma unroll
-        for (int u = 0; u < kImageRows; ++u)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) mx = max(mx, abs_bits(v[u][k]));
-        const Pow2Scale sc = scale_of(mx);
-#pragma unroll
-        for (int u = 0; u < kImageRows; ++u) {
-            const int row = first_row + u * blockDim.y;
-            if (it >= items || row >= s.rows) continue;
-            image_store<kG>(dst, (size_t)row * items + it, sc, v[u], in && nch > 4 ? src + ((size_t)row * s.w + xm) * s.c_src + g * kG : nullptr, nch);
-        }
-    }
-}
-
-// First pass over images of up to four channels in one group, no row wider than the block: a part is then a run of at most
-// 4 * kThreads pixels, which the block reads as float4 and hands out through shared memory (a pixel's channels read one by one, 64
-// images 224 x 224: 19.7 us, 16.0 so).
-template <int kG>
-__device__ __forceinline__ void image_part_staged(const float *__restrict__ src, const ImageShape &s, int part, int tid, TileGuess &guess, int8_t *dst,
-                                                  DeviceState *dev)
-{
-    __shared__ __align__(16) float stage[4 * kImageRows * kThreads];
-    const int part_rows = kImageRows * blockDim.y, row0 = part * part_rows, rows = min(part_rows, s.rows - row0);
-    const int count = rows > 0 ? rows * s.w * s.c_src : 0;
-    const float *p = src + (size_t)row0 * s.w * s.c_src;   // (16-byte aligned: part_rows is a multiple of 4)
-    float4 v[kImageRows];
-    uint32_t mx = 0;
-#pragma unroll
-    for (int u = 0; u < kImageRows; ++u) {
-        const int i = u * kThreads + tid;
-        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (4 * i + 3 < count) v[u] = __ldg(reinterpret_cast<const float4 *>(p) + i);
-        else if (4 * i < count) {
-            v[u].x = __ldg(p + 4 * i);
-            if (4 * i + 1 < count) v[u].y = __ldg(p + 4 * i + 1);
-            if (4 * i + 2 < count) v[u].z = __ldg(p + 4 * i + 2);
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < kImageRows; ++u) {
-        mx = max(max(mx, max(abs_bits(v[u].x), abs_bits(v[u].y))), max(abs_bits(v[u].z), abs_bits(v[u].w)));
-        reinterpret_cast<float4 *>(stage)[u * kThreads + tid] = v[u];
-    }
-    const Pow2Scale sc = pow2_scale(guess.part(mx, tid, dev));   // (its barrier also publishes the stage)
-    const int w_mem = s.w + 2 * s.wmargin, xm = (int)threadIdx.x - s.wmargin;
-    const bool in = xm >= 0 && xm < s.w;
-#pragma unroll
-    for (int u = 0; u < kImageRows; ++u) {
-        const int r = threadIdx.y + u * blockDim.y;
-        if ((int)threadIdx.x >= w_mem || r >= rows) continue;
-        const float *q = stage + (r * s.w + xm) * s.c_src;
-        float f[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) f[k] = in && k < s.c_src ? q[k] : 0.0f;
-        image_store<kG>(dst, (size_t)(row0 + r) * w_mem + threadIdx.x, sc, f, nullptr, 0);
-    }
-}
-
+// kStaged: images of up to four channels in one group, no row wider than the block: a block's rows are then a run of at most 4 * kThreads
+// pixels, read as float4 and handed out through shared memory.
 template <int kG, bool kStaged>
 __global__ void __launch_bounds__(kThreads)
-quantize_image_kernel(const float *__restrict__ src, ImageShape s, int8_t *dst, int16_t *tile_shift, int reps, DeviceState *dev)
+quantize_image_kernel(const float *__restrict__ src, ImageShape s, int8_t *dst, int32_t *dst_exp, DeviceState *dev, int early)
 {
-    ptx::grid_dep_wait_launch_small();
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    TileGuess guess;
-    for (int r = 0; r < reps; ++r) {
-        const int part = (int)blockIdx.x * reps + r;
-        if (kStaged) {
-            if (r > 0) __syncthreads();   // (the stage is read)
-            image_part_staged<kG>(src, s, part, tid, guess, dst, dev);
-        } else {
-            image_part<kG>(src, s, part * kImageRows * (int)blockDim.y + threadIdx.y, dst, [&](uint32_t mx) { return pow2_scale(guess.part(mx, tid, dev)); });
+    if (!early) ptx::grid_dep_wait();   // (see quantize_f32_kernel)
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x, block = (int)(gridDim.x - 1 - blockIdx.x);
+    const int row0 = block * kImageRows * (int)blockDim.y, w_mem = s.w + 2 * s.wmargin;
+    int up = 7;
+    bool last = false;
+    if (kStaged) {
+        __shared__ __align__(16) float stage[4 * kImageRows * kThreads];
+        const int rows = min(kImageRows * (int)blockDim.y, s.rows - row0), count = rows * s.w * s.c_src;
+        const float *p = src + (size_t)row0 * s.w * s.c_src;   // (16-byte aligned: row0 is a multiple of 4)
+        float4 v[kImageRows];
+#pragma unroll
+        for (int u = 0; u < kImageRows; ++u) {
+            const int i = u * kThreads + tid;
+            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (4 * i + 3 < count) v[u] = __ldg(reinterpret_cast<const float4 *>(p) + i);
+            else if (4 * i < count) {
+                v[u].x = __ldg(p + 4 * i);
+                if (4 * i + 1 < count) v[u].y = __ldg(p + 4 * i + 1);
+                if (4 * i + 2 < count) v[u].z = __ldg(p + 4 * i + 2);
+            }
+        }
+        if (early) ptx::grid_dep_wait();
+        if (gridDim.x <= kPartSms) ptx::grid_dep_launch();
+#pragma unroll
+        for (int u = 0; u < kImageRows; ++u) reinterpret_cast<float4 *>(stage)[u * kThreads + tid] = v[u];
+        last = sq_shift(tid, dst_exp, dev, &up);   // (its barrier also publishes the stage)
+        const Pow2Scale sc = pow2_scale(up);
+        const int xm = (int)threadIdx.x - s.wmargin;
+        const bool in = xm >= 0 && xm < s.w;
+#pragma unroll
+        for (int u = 0; u < kImageRows; ++u) {
+            const int r = threadIdx.y + u * blockDim.y;
+            if ((int)threadIdx.x >= w_mem || r >= rows) continue;
+            const float *q = stage + (r * s.w + xm) * s.c_src;
+            float f[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) f[k] = in && k < s.c_src ? q[k] : 0.0f;
+            image_store<kG>(dst, (size_t)(row0 + r) * w_mem + threadIdx.x, sc, f, nullptr, 0);
+        }
+    } else {
+        const int groups = s.c_dst / kG, items = w_mem * groups;
+        for (int x0 = 0; x0 < items; x0 += blockDim.x) {   // one round unless a row is wider than the block
+            const int it = x0 + threadIdx.x;
+            const int xp = groups == 1 ? it : it / groups, g = groups == 1 ? 0 : it - xp * groups, xm = xp - s.wmargin;
+            const int nch = min(kG, s.c_src - g * kG);       // real channels of this group (none or fewer beyond c_src)
+            const bool in = it < items && xm >= 0 && xm < s.w;
+            float v[kImageRows][4];                          // the first four channels; more are read when they are coded
+#pragma unroll
+            for (int u = 0; u < kImageRows; ++u) {
+                const int row = row0 + threadIdx.y + u * blockDim.y;
+                const float *p = src + ((size_t)row * s.w + xm) * s.c_src + g * kG;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[u][k] = (in && row < s.rows && k < nch) ? __ldg(p + k) : 0.0f;
+            }
+            if (x0 == 0) {
+                if (early) ptx::grid_dep_wait();
+                if (gridDim.x <= kPartSms) ptx::grid_dep_launch();
+                last = sq_shift(tid, dst_exp, dev, &up);
+            }
+            const Pow2Scale sc = pow2_scale(up);
+#pragma unroll
+            for (int u = 0; u < kImageRows; ++u) {
+                const int row = row0 + threadIdx.y + u * blockDim.y;
+                if (it >= items || row >= s.rows) continue;
+                image_store<kG>(dst, (size_t)row * items + it, sc, v[u], in && nch > 4 ? src + ((size_t)row * s.w + xm) * s.c_src + g * kG : nullptr, nch);
+            }
         }
     }
-    guess.publish(tid, tile_shift + blockIdx.x, dev);
-}
-
-template <int kG>
-__global__ void __launch_bounds__(kThreads, kAgainPerSm)
-quantize_image_again_kernel(const float *__restrict__ src, ImageShape s, int8_t *dst, int32_t *dst_exp, const int16_t *tile_shift, int tiles,
-                            int reps, DeviceState *dev)
-{
-    ptx::grid_dep_wait_launch_small();
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x, part_rows = kImageRows * blockDim.y;
-    recode_tiles(tile_shift, tiles, tid, dst_exp, dev, [&](int tile, const Pow2Scale &sc) {
-        for (int r = 0; r < reps; ++r)
-            image_part<kG>(src, s, (tile * reps + r) * part_rows + threadIdx.y, dst, [&](uint32_t) { return sc; });
-    });
+    if (last) dev->absmax_u32 = 0;
 }
 
 // w[oc][kh][kw][c] -> wp[oc][kh][8][c] with zeros in the unused taps; c = 16 (Pixel = int4) or 8 (int2)
@@ -1104,7 +1117,12 @@ cudaError_t launch_reset_cells(DeviceState *dev, cudaStream_t s)
 
 bool quantize_is_small(int mode, size_t n, const ReduceHook &hook) { return mode == 2 && !hook.fn && n <= kSmallElems * kSmallCluster; }
 
-// Tiles of the two-pass SQ: `reps` parts each, more than one only where the handle has no cell for every part; the second pass's
+// Largest tensor whose codes wait for the maximum: what the L2 (126 MB) holds of it is read from there, see quantize_sq_kernel.
+constexpr size_t kSqResident = 24u << 20;
+
+static unsigned quantize_tiles(size_t n) { return n / 4 > kQuantTile ? (unsigned)((n / 4 + kQuantTile - 1) / kQuantTile) : 1u; }
+
+// Tiles of the SQ that guesses: `reps` parts each, more than one only where the handle has no cell for every part; the second pass's
 // blocks look after at most kThreads tiles each.
 struct TileSplit {
     int reps, tiles, again_blocks;
@@ -1117,6 +1135,13 @@ static TileSplit split_tiles(size_t parts, int sm_count)
     const int least = (t.tiles + kThreads - 1) / kThreads, most = kAgainPerSm * sm_count;
     t.again_blocks = t.tiles < most ? t.tiles : (least > most ? least : most);
     return t;
+}
+
+// The largest |x| into the cell (and its exchange: float bit patterns of |x| order like integers).
+static void launch_sq_maximum(const float *src, size_t n, DeviceState *dev, cudaStream_t s, const ReduceHook &hook)
+{
+    launch_chained(absmax_f32_kernel, quantize_tiles(n), kThreads, 0, s, src, n, dev);
+    hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
 }
 
 cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst, int32_t *dst_exp, int16_t *tile_shift, DeviceState *dev,
@@ -1136,36 +1161,36 @@ cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst,
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, quantize_sq_small_kernel, src, n, static_cast<int8_t *>(dst), dst_exp, dev);
     }
-    const size_t parts = (n / 4 + kQuantTile - 1) / kQuantTile > 0 ? (n / 4 + kQuantTile - 1) / kQuantTile : 1;
-    if (mode == 0) launch_chained(quantize_f32_kernel<0>, (unsigned)parts, kThreads, 0, s, src, n, dst, dst_exp);
-    else if (mode == 1) launch_chained(quantize_f32_kernel<1>, (unsigned)parts, kThreads, 0, s, src, n, dst, dst_exp);
-    else {
-        const TileSplit t = split_tiles(parts, sm_count);
+    const unsigned tiles = quantize_tiles(n);
+    if (mode == 2 && n > kSqResident) {
+        const TileSplit t = split_tiles(tiles, sm_count);
         launch_chained(quantize_sq_kernel, t.tiles, kThreads, 0, s, src, n, static_cast<int8_t *>(dst), tile_shift, t.reps, dev);
-        hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);  // float bit patterns of |x| order like integers
+        hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
         launch_chained(quantize_sq_again_kernel, t.again_blocks, kThreads, 0, s, src, n, static_cast<int8_t *>(dst), dst_exp,
                        (const int16_t *)tile_shift, t.tiles, t.reps, dev);
+        return cudaGetLastError();
     }
+    if (mode == 2) launch_sq_maximum(src, n, dev, s, hook);
+    const int early = mode == 2 && !hook.fn;
+    const auto kernel = mode == 0 ? quantize_f32_kernel<0> : (mode == 1 ? quantize_f32_kernel<1> : quantize_f32_kernel<2>);
+    launch_chained(kernel, tiles, kThreads, 0, s, src, n, dst, dst_exp, dev, early);
     return cudaGetLastError();
 }
 
 cudaError_t launch_quantize_image(const float *src, int n, int h, int w, int c_src, int c_dst, int wmargin, int8_t *dst, int32_t *dst_exp,
-                                  int16_t *tile_shift, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook)
+                                  DeviceState *dev, cudaStream_t s, const ReduceHook &hook)
 {
+    launch_sq_maximum(src, (size_t)n * h * w * c_src, dev, s, hook);
     const int g = c_dst % 16 == 0 ? 16 : 8, items = (w + 2 * wmargin) * (c_dst / g);
     const ImageShape shape{n * h, w, c_src, c_dst, wmargin};
     int tx = 32;
     while (tx < items && tx < kThreads) tx *= 2;
     const dim3 block(tx, kThreads / tx);
-    const int part_rows = kImageRows * (int)block.y;
-    const TileSplit t = split_tiles((size_t)(shape.rows + part_rows - 1) / part_rows, sm_count);
+    const int block_rows = kImageRows * (int)block.y;
     const bool staged = c_src <= 4 && c_dst == g && items <= kThreads;
-    const auto first = staged ? (g == 16 ? quantize_image_kernel<16, true> : quantize_image_kernel<8, true>)
-                              : (g == 16 ? quantize_image_kernel<16, false> : quantize_image_kernel<8, false>);
-    launch_chained(first, t.tiles, block, 0, s, src, shape, dst, tile_shift, t.reps, dev);
-    hook(&dev->absmax_u32, 1, EOQ_REDUCE_I32, EOQ_REDUCE_MAX, s);
-    launch_chained(g == 16 ? quantize_image_again_kernel<16> : quantize_image_again_kernel<8>, t.again_blocks, block, 0, s, src, shape, dst,
-                   dst_exp, (const int16_t *)tile_shift, t.tiles, t.reps, dev);
+    const auto kernel = staged ? (g == 16 ? quantize_image_kernel<16, true> : quantize_image_kernel<8, true>)
+                               : (g == 16 ? quantize_image_kernel<16, false> : quantize_image_kernel<8, false>);
+    launch_chained(kernel, (unsigned)((shape.rows + block_rows - 1) / block_rows), block, 0, s, src, shape, dst, dst_exp, dev, (int)!hook.fn);
     return cudaGetLastError();
 }
 

@@ -345,7 +345,7 @@ cudaError_t launch_probe_mma_i8(int n_cols, int iters, int grid, DeviceState *de
 // ---------------------------------------------------------------------------------------------
 cudaError_t launch_reset_cells(DeviceState *dev, cudaStream_t s);
 cudaError_t launch_quantize_image(const float *src, int n, int h, int w, int c_src, int c_dst, int wmargin, int8_t *dst, int32_t *dst_exp,
-                                  int16_t *tile_shift, DeviceState *dev, int sm_count, cudaStream_t s, const ReduceHook &hook);
+                                  DeviceState *dev, cudaStream_t s, const ReduceHook &hook);
 // w[oc][kh][kw][16] -> wp[oc][kh][8][16], zero in the taps kw..7 (weights of the filter-row path)
 cudaError_t launch_weight_pad_rows(const int8_t *w, int8_t *wp, int c_out, int kh, int kw, int c_in, cudaStream_t s);
 bool quantize_is_small(int mode, size_t n, const ReduceHook &hook);  // one launch instead of two

@@ -445,6 +445,87 @@ def test_quantize_float_of_more_parts_than_cells():
     assert bool((out.view(times, run) == torch.from_numpy(codes).cuda()).all())
 
 
+@pytest.mark.parametrize("kind", ["even", "rising", "one tile", "zero tiles", "nan"])
+@pytest.mark.parametrize("n", [24 << 20, (24 << 20) + 1, 26000003])
+def test_quantize_float_on_both_sides_of_the_cache(n, kind):
+    """The largest tensor that is read twice, and those whose tiles are coded before the maximum is known."""
+    x = synth.normal_f32(n, 3043, 0)
+    part = np.arange(n) // 8192
+    if kind == "rising":
+        x *= np.exp2(part % 97 - 40).astype(np.float32)
+    elif kind == "one tile":
+        x[n - 1] = 3000.0
+    elif kind == "zero tiles":
+        x[(part % 3) != 1] = -0.0
+    elif kind == "nan":
+        x[n // 2] = np.nan
+    h, out, ex = G.handle(), G.empty((n,), torch.int8), G.zeros(1, torch.int32)
+    eoq.eoq_quantize(h, eoq.EOQ_SQ, G.dev(x), True, None, n, out, ex)
+    assert G.status_clear() == (eoq.EOQ_DEV_NONFINITE if kind == "nan" else 0)
+    if kind == "nan":   # flagged; the codes are those at an exponent of -7
+        c, p = np.clip(np.rint(np.nan_to_num(x) * np.float32(128)), -127, 127).astype(np.int8), -7
+    else:
+        c, p, _ = oracle.quantize_f32(oracle.MODE_SQ, x)
+    assert ex.item() == p and np.array_equal(G.host(out), c)
+
+
+@pytest.mark.parametrize("image", [False, True])
+def test_quantize_float_reads_what_the_stream_wrote_last(image):
+    """The second pass reads the source ahead of the first one's end; a source rewritten between calls is the new one all the same."""
+    shape = (40, 96, 100, 3) if image else (5000003,)
+    n, h = int(np.prod(shape)), eoq.eoq_create(0)
+    xs = [torch.from_numpy(synth.normal_f32(shape, 3044, k)).cuda() * 2.0 ** k for k in range(3)]
+    want = [oracle.quantize_f32(oracle.MODE_SQ, x.cpu().numpy().reshape(-1))[:2] for x in xs]
+    src, got = torch.empty_like(xs[0]), []
+    for k in range(30):
+        out, ex = G.empty(shape[:3] + (8,) if image else shape, torch.int8), G.zeros(1, torch.int32)
+        src.copy_(xs[k % 3])
+        if image:
+            eoq.eoq_quantize_image(h, src, *shape, 8, 0, out, ex)
+        else:
+            eoq.eoq_quantize(h, eoq.EOQ_SQ, src, True, None, n, out, ex)
+        got.append((out, ex))
+    torch.cuda.synchronize()
+    for k, (out, ex) in enumerate(got):
+        codes = G.host(out[..., :3] if image else out)
+        assert ex.item() == want[k % 3][1] and np.array_equal(codes.reshape(-1), want[k % 3][0]), k
+    eoq.eoq_destroy(h)
+
+
+@pytest.mark.parametrize("shape", [(1 << 20,), (1 << 22,), (64, 224, 224, 3), (128, 32, 32, 3)])
+def test_quantize_float_takes_no_longer_for_an_outlier(shape):
+    """A maximum that only one element has costs nothing: codes of a tensor that is read twice are formed once.  (Formed once under a
+    guess and once more, 4 M floats took 34% longer, 64 images 224 x 224 took 50%.)"""
+    n, h = int(np.prod(shape)), eoq.eoq_create(0)
+    x = torch.from_numpy(synth.normal_f32(shape, 3045, 0)).cuda().clamp_(-4.0, 4.0)
+    y = x.clone()
+    y.view(-1)[n // 3] = 300.0
+    out, ex, graphs = G.empty(shape[:3] + (8,) if len(shape) == 4 else shape, torch.int8), G.zeros(1, torch.int32), []
+    for src in (x, y):
+        def call():
+            if len(shape) == 4:
+                eoq.eoq_quantize_image(h, src, *shape, 8, 0, out, ex)
+            else:
+                eoq.eoq_quantize(h, eoq.EOQ_SQ, src, True, None, n, out, ex)
+        call()
+        torch.cuda.synchronize()
+        graphs.append(torch.cuda.CUDAGraph())
+        with torch.cuda.graph(graphs[-1]):
+            for _ in range(20):
+                call()
+    best = [1e9, 1e9]
+    for _ in range(10):
+        for k, g in enumerate(graphs):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            g.replay()
+            b.record()
+            torch.cuda.synchronize()
+            best[k] = min(best[k], a.elapsed_time(b))
+    assert best[1] < 1.06 * best[0], best
+    eoq.eoq_destroy(h)
+
+
 @pytest.mark.parametrize("n", [262144, 6000001, 64 * 56 * 56 * 64 + 1])
 def test_quantize_float_runs_beside_a_long_kernel(n):
     """SQ needs no SM for itself alone: it ends while a kernel of another stream still occupies one (a convolution capped to one CTA,
