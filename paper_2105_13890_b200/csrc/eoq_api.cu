@@ -1646,12 +1646,12 @@ static FinishItem finish_item(const eoq_conv_desc_t &d, const Geometry &g, const
     return it;
 }
 
-// The b1 error sums of the batch (let_in: see launch_finish_taps).
-static int finish_taps(Handle *h, const FinishBatch &b, bool let_in, cudaStream_t s)
+// The b1 error sums of the batch.
+static int finish_taps(Handle *h, const FinishBatch &b, TapsOrder order, cudaStream_t s)
 {
     ProfScope prof(h, EOQ_PROF_WGRAD_TAPS, s);
     count_launches(h, 1);
-    return record(h, launch_finish_taps(b, let_in, s));
+    return record(h, launch_finish_taps(b, order, s));
 }
 
 // Sums and Q_g of the batch, whose GEMMs and b1 error sums are in front on the stream.
@@ -1685,42 +1685,47 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
     const bool use_b1 = b1_dev != nullptr || b1_c != 0;
     if (use_b1 && bc.nrc * bc.ncc > kMaxBorderClasses) return EOQ_ERR_UNSUPPORTED;
     const WgradSpace w = wgrad_space(d, g, workspace);
-    // A layer's b1 error sums go in front of its GEMM, which they let in and which runs beside them; a small layer is finished by one
-    // launch behind it, which forms them too and runs beside it up to there.
+    // The b1 error sums run beside the GEMM (whose kernel leaves sums as [oc][tap][ic], the layout of g), launched behind it or in front;
+    // then come the sums of its slices with Q_g.  A small layer is finished by one launch, which forms the b1 sums beside the GEMM too.
     FinishItem item = finish_item(d, g, w, e3, e3_exp, b1_c, b1_dev, gq, g_exp, 0);
     item.copy_out = reinterpret_cast<long long *>(acc_dump);
     FinishBatch batch;
     bool small = false, taps_first = false;
-    auto begin = [&](int num_parts, bool beside) -> int {   // beside: the GEMM's kernel can run beside its neighbours
+    // Fills in what the GEMM's plan says of its neighbours.  Its kernel clears the maximum's cell, and the tap sums' where they may be added up.
+    auto begin = [&](int num_parts, auto &plan, bool beside) -> int {   // beside: the kernel can run beside them
         if (num_parts_out) *num_parts_out = num_parts;
-        if (gemm_only) return EOQ_OK;
-        item.num_parts = num_parts;
-        small = !h->profiling && finish_is_small(item, h->hook);   // (a profile brackets the b1 sums as a kind of their own)
-        if (small) return EOQ_OK;
-        plan_finish(batch, &item, 1, h->sm_count, h->hook);
-        if (!use_b1) return EOQ_OK;
-        taps_first = beside;
-        return finish_taps(h, batch, beside, s);
+        bool add = num_parts_out != nullptr;
+        if (!gemm_only) {
+            item.num_parts = num_parts;
+            small = !h->profiling && finish_is_small(item, h->hook);   // (a profile brackets the b1 sums as a kind of their own)
+            if (!small) plan_finish(batch, &item, 1, h->sm_count, h->gemm_ctas >= h->sm_count, h->hook);
+            add = !small && use_b1 && batch.item[0].tap_add;
+            taps_first = beside && use_b1 && !small && finish_taps_first(batch.item[0]);
+        }
+        plan.zero = add ? reinterpret_cast<int4 *>(w.tap_sums) : reinterpret_cast<int4 *>(w.max_cell);
+        plan.zero_n16 = (unsigned)(reinterpret_cast<int4 *>(w.max_cell) + 1 - plan.zero);
+        return taps_first ? finish_taps(h, batch, kTapsFirst, s) : EOQ_OK;
     };
-    // behind the GEMM (whose kernel leaves sums as [oc][tap][ic], the layout of g)
-    auto finish = [&](cudaError_t e) -> int {
+    auto finish = [&](cudaError_t e, bool beside) -> int {
         if (e != cudaSuccess || gemm_only) return record(h, e);
-        if (!small) return finish_sums(h, batch, s);
-        count_launches(h, 1);
-        return record(h, launch_finish_small(item, &h->dev->status, h->sm_count, use_b1, s));
+        if (small) {
+            count_launches(h, 1);
+            return record(h, launch_finish_small(item, &h->dev->status, h->sm_count, beside && use_b1, s));
+        }
+        if (use_b1 && !taps_first && (st = finish_taps(h, batch, beside ? kTapsBeside : kTapsBehind, s)) != EOQ_OK) return st;
+        return finish_sums(h, batch, s);
     };
 
     WgradPatchPlan wp;
     if (plan_wgrad_patch(wp, d, g.ho, g.wo, h->gemm_ctas < kWgradTargetCtas ? h->gemm_ctas : kWgradTargetCtas)) {
         wp.partials = w.parts;
-        wp.zero = w.max_cell;
         wp.dev = h->dev;
         CUtensorMap map_x, map_e;
         if (!make_patch_map(&map_x, x, d.n, d.h, d.w, d.c_in, wp.kc, wp.pw, wp.r_rows + d.kh - 1) ||
             !make_patch_map(&map_e, e3, d.n, g.ho, g.wo, d.c_out, wp.tile_n, wp.pw, wp.r_rows))
             return EOQ_ERR_UNSUPPORTED;
-        if ((st = begin(wp.num_splits, true)) != EOQ_OK) return st;
-        wp.launch_early = small && use_b1;
+        if ((st = begin(wp.num_splits, wp, true)) != EOQ_OK) return st;
+        wp.launch_early = use_b1 && !gemm_only && !taps_first;
         wp.wait_late = taps_first;
         count_launches(h, 1);
         cudaError_t e;
@@ -1728,34 +1733,32 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
             ProfScope prof(h, EOQ_PROF_WGRAD, s);
             e = launch_wgrad_patch(wp, map_x, map_e, s);
         }
-        return finish(e);
+        return finish(e, true);
     }
 
     const int w_mem = d.w + 2 * d.x_wmargin;
     WgradRowsPlan rp;
     if (plan_wgrad_rows(rp, d, g, h->gemm_ctas)) {
         rp.partials = w.parts;
-        rp.zero = w.max_cell;
         rp.dev = h->dev;
         CUtensorMap map_x, map_e;
         if (!make_matrix_map(&map_e, e3, (size_t)d.n * g.ho * g.wo, d.c_out, rp.nc, g.wo) ||
             !make_row_window_map(&map_x, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, g.wo, g.ho, d.stride, d.pad, g.wo))
             return EOQ_ERR_UNSUPPORTED;
-        if ((st = begin(rp.num_splits, false)) != EOQ_OK) return st;
+        if ((st = begin(rp.num_splits, rp, false)) != EOQ_OK) return st;
         count_launches(h, 1);
         cudaError_t e;
         {
             ProfScope prof(h, EOQ_PROF_WGRAD, s);
             e = launch_wgrad_rows(rp, map_x, map_e, s);
         }
-        return finish(e);
+        return finish(e, false);
     }
 
     WgradParams p;
     if (!plan_wgrad(p, d, g, h->gemm_ctas)) return EOQ_ERR_UNSUPPORTED;
     const bool row_window = p.row_window_kw != 0;
     p.partials = w.parts;
-    p.zero = w.max_cell;
     p.dev = h->dev;
 
     cudaError_t e;
@@ -1766,15 +1769,15 @@ static int conv_wgrad_impl(eoq_handle_t handle, const eoq_conv_desc_t *desc, con
                    : !make_im2col_map(&map_x, x, d.n, d.h, w_mem, d.c_in, d.x_wmargin - d.pad, -d.pad, g.wo, g.ho, d.stride,
                                       p.kc, p.pixels_per_stage))
         return EOQ_ERR_UNSUPPORTED;
-    if ((st = begin(p.num_k_splits, true)) != EOQ_OK) return st;
-    p.launch_early = small && use_b1;
+    if ((st = begin(p.num_k_splits, p, true)) != EOQ_OK) return st;
+    p.launch_early = use_b1 && !gemm_only && !taps_first;
     p.wait_late = taps_first;
     count_launches(h, 1);
     {
         ProfScope prof(h, EOQ_PROF_WGRAD, s);
         e = launch_wgrad(p, map_x, map_e, s);
     }
-    return finish(e);
+    return finish(e, true);
 }
 
 extern "C" int eoq_conv_wgrad(eoq_handle_t handle, const eoq_conv_desc_t *desc, const int8_t *e3,
@@ -1828,6 +1831,7 @@ extern "C" int eoq_wgrad_finish(eoq_handle_t handle, int num, const eoq_conv_des
             check_desc(&d, &g);
             items[k] = finish_item(d, g, wgrad_space(d, g, workspace[base + k]), e3[base + k], e3_exp[base + k], 0, b1_c[base + k],
                                    gq[base + k], g_exp[base + k], num_parts[base + k]);
+            items[k].tap_clear = 1;
         }
         if (count == 1 && !h->profiling && finish_is_small(items[0], h->hook)) {
             count_launches(h, 1);
@@ -1836,8 +1840,8 @@ extern "C" int eoq_wgrad_finish(eoq_handle_t handle, int num, const eoq_conv_des
             continue;
         }
         FinishBatch b;
-        plan_finish(b, items, count, h->sm_count, h->hook);
-        int st = b.tap_first[count] > 0 ? finish_taps(h, b, false, s) : EOQ_OK;
+        plan_finish(b, items, count, h->sm_count, h->gemm_ctas >= h->sm_count, h->hook);
+        int st = b.tap_first[count] > 0 ? finish_taps(h, b, kTapsBehind, s) : EOQ_OK;
         if (st == EOQ_OK) st = finish_sums(h, b, s);
         if (st != EOQ_OK) return st;
     }

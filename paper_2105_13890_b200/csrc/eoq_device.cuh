@@ -364,12 +364,6 @@ __device__ __forceinline__ void st_cluster_32(uint32_t addr, uint32_t v)
 {
     asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-__device__ __forceinline__ int32_t ld_cluster_32(uint32_t addr)
-{
-    int32_t v;
-    asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
 __device__ __forceinline__ int4 ld_shared_128(uint32_t addr)
 {
     int4 v;

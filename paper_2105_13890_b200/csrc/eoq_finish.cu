@@ -1,7 +1,7 @@
 // What follows the weight-gradient GEMM (arXiv 2105.13890, Sec. 3.2.1: g_w = Q_g(e3 * x1) with x1 = x0 + Q_b(b1)), for one
 // layer or for many layers in the same three launches: the b1 error sums (one pass over e3), the exact sums (split-K slices
 // plus the b1 term) reduced to their maximum, and Q_g.  Blocks find their layer by their index.
-// The maximum's cell is cleared by the GEMM kernel.
+// The maximum's cell is cleared by the GEMM kernel, as are the b1 error sums' cells where these are added up (FinishItem::tap_add).
 #include "eoq_device.cuh"
 #include "eoq_internal.h"
 
@@ -12,7 +12,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kTapSlab = 32;      // channels one block of the error sums covers: a 32-byte sector of a pixel
 constexpr int kTapThreads = 512;
-constexpr int kTapMostCluster = 8;
 
 __device__ __forceinline__ int finish_item_of(const int *first, int num, int block)
 {
@@ -39,14 +38,17 @@ __device__ __forceinline__ bool finish_narrow(const FinishItem &it, int b1)
 //   tap sum = T - sum of R_i - sum of C_j + sum of P_ij   over the border rows and columns the tap does not take.
 // Every term is a plain sum over a regular set of pixels.  A block covers a range of rows and a slab of channels; a lane
 // keeps the sums of 16 channels (one 128-bit load per pixel, several in flight).  All warps sum T, then share out the border sets.
-// A slab's rows are dealt to the kTapReplicas copies of its cells, and a copy's to the blocks of a cluster, whose sums meet in
-// distributed shared memory: a copy is stored, not added to, so nothing clears the cells and no order against the GEMM is needed.
-// Bound by the latency of a few dependent rounds of loads.  A single layer's sums therefore go in front of its GEMM, which is let
-// in at once and runs beside them (conv_wgrad_impl).  With atomics into cells that the GEMM cleared they came behind it and ended
-// 3 to 8 us after it: backward of the 512-channel 7 x 7 layer at batch 64 60.6 -> 59.0 us, bottleneck block of ResNet-50 at batch 32
-// 270 -> 264, and fewer SMs taken from the error chain of a step (ResNet-18 at batch 13 621 -> 608).  Sums of four pixels by dot products
-// and no divisions in front of the first load: the kernel 7.5 -> 5.5 us for the 48 -> 80 channel strided layer, whose backward went 26.5
-// -> 24.7.
+// A slab's rows are dealt to its blocks.  Up to kTapReplicas blocks store a copy of the cells each; more of them add to the copies, which
+// the GEMM has cleared.
+// Bound by the latency of a few dependent rounds of loads.  A single layer's sums run beside its GEMM, which lets them in once it has seen
+// e3 complete; they wait for its end before they add, or before they end.  Up to kTapsFirstBytes of errors they go in front and let the GEMM
+// in, which waits for them at its end: they would be the last to end behind it (48 -> 80 channels, stride 2, 37 x 29 at batch 5: 12.4 us for the
+// weight gradient, 11.6 so; 64 channels 56 x 56 at batch 4, 0.8 M errors, 15.6 beside, 17.2 in front).  Whichever comes second finds
+// room because the first asks its SMs for all the shared memory there is: an SM divides its memory between L1 and shared memory when it is
+// idle.  All sums in front of the GEMM, in clusters of up to eight blocks that stored what they had summed through distributed shared
+// memory, left few slabs too few blocks, and the GEMM waited for many: 16 -> 32 channels 56 x 56 at batch 512 68.3 us for the weight gradient, 58.2 so, 64 -> 64 99 and 82, 16 -> 240 by 1 x 1, 64 x 64 at batch 40,
+// 35.5 and 28.3; 64 -> 128 channels 56 x 56, stride 2, batch 64 19.9 and 19.5, 1024 -> 256 by 1 x 1, 14 x 14, batch 32 14.8 and 14.0.  Sums of
+// four pixels by dot products and no divisions in front of the first load: the kernel 7.5 -> 5.5 us for the 48 -> 80 channel strided layer.
 struct PixelSum {
     int v[16] = {};
     // adds four pixels: the codes of a channel side by side, then one byte dot product
@@ -190,10 +192,10 @@ __device__ __forceinline__ void tap_sets(const FinishItem &it, int slab, int sla
     __syncthreads();
 }
 
-// Copy `copy` (of `copies`) of the slab's tap sums, over range copy * cluster + rank of its rows, by the calling block and its
-// cluster.  sets, loc: shared memory of tap_set_bytes and kMaxTaps * kTapSlab words (loc only in a cluster).
-template <int kT>
-__device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab, int copy, int copies, int cluster, int rank, int32_t *sets, int32_t *loc)
+// Range `range` (of `ranges`) of a slab's rows into its tap sums, by the calling block.  sets: shared memory of tap_set_bytes.
+// kBeside: the layer's GEMM is the launch in front and may still run.
+template <int kT, bool kBeside>
+__device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab, int range, int ranges, int32_t *sets)
 {
     __shared__ TapMasks masks;
     const eoq_conv_desc_t &d = it.d;
@@ -202,8 +204,8 @@ __device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab,
     tap_masks(it, nr, nc, masks);   // (published by the barriers of tap_sets)
     const int slab_ch = min(kTapSlab, d.c_out - slab * kTapSlab);  // channels of this slab (16 or 32)
     const int taps = d.kh * d.kw, items = taps * slab_ch;
-    const int rows = d.n * it.ho, ranges = copies * cluster, rows_here = (rows + ranges - 1) >> (31 - __clz(ranges));   // (powers of two)
-    const int begin = min((long long)rows, (long long)(copy * cluster + rank) * rows_here), end = min((long long)rows, (long long)begin + rows_here);
+    const int rows = d.n * it.ho, rows_here = (int)(((long long)rows + ranges - 1) / ranges);
+    const int begin = (int)min((long long)rows, (long long)range * rows_here), end = (int)min((long long)rows, (long long)begin + rows_here);
     constexpr int kMost = (kMaxTaps * kTapSlab + kT - 1) / kT;   // items of a thread
     long long total[kMost] = {};
     const int chunk = (long long)rows_here * it.wo <= (1 << 23) ? max(1, rows_here) : max(1, (1 << 23) / it.wo);   // keeps the int32 sets exact
@@ -211,7 +213,10 @@ __device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab,
     for (int at = 0; at < rows_here; at += chunk) {
         const int r0 = min(end, begin + at), r1 = min(end, r0 + min(chunk, rows_here - at));
         tap_sets<kT>(it, slab, slab_ch, r0, r1, nr, nc, sets);
-        auto tap_sum = [&](int i) {
+#pragma unroll
+        for (int k = 0; k < kMost; ++k) {
+            const int i = k * kT + (int)threadIdx.x;   // [tap][channel]
+            if (i >= items) continue;
             const int tap = i >> ch_shift, c = i & (slab_ch - 1), kh = tap * per_kw >> 16, kw = tap - kh * d.kw;
             const unsigned long long rm = masks.rows[kh], cm = masks.cols[kw];
             const int32_t *cell = sets + c;
@@ -222,54 +227,40 @@ __device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab,
             };
             int sum = over_columns(cell);
             for (unsigned long long m = rm; m; m &= m - 1) sum -= over_columns(cell + __ffsll((long long)m) * (1 + nc) * kTapSlab);
-            return sum;
-        };
-        if (cluster > 1) {
-            for (int i = threadIdx.x; i < items; i += kT) loc[i] = tap_sum(i);
-            ptx::cluster_sync();
-#pragma unroll
-            for (int k = 0; k < kMost; ++k) {
-                const int i = (k * cluster + rank) * kT + (int)threadIdx.x;
-                if (i < items)
-                    for (int q = 0; q < cluster; ++q) total[k] += ptx::ld_cluster_32(ptx::cluster_addr(ptx::smem_u32(loc + i), q));
-            }
-            ptx::cluster_sync();   // the peers are through with this block's sums
-        } else {
-#pragma unroll
-            for (int k = 0; k < kMost; ++k) {
-                const int i = k * kT + (int)threadIdx.x;
-                if (i < items) total[k] += tap_sum(i);
-            }
-            __syncthreads();
+            total[k] += sum;
         }
+        __syncthreads();
     }
+    if (kBeside && it.tap_add) ptx::grid_dep_wait();   // (the GEMM has cleared the cells)
 #pragma unroll
     for (int k = 0; k < kMost; ++k) {
-        const int i = (k * cluster + rank) * kT + (int)threadIdx.x;   // [tap][channel], stored at [oc][tap]
+        const int i = k * kT + (int)threadIdx.x;   // stored at [oc][tap]
         if (i >= items) continue;
         const int tap = i >> ch_shift, c = i & (slab_ch - 1);
         long long *cell = it.tap_sums + ((size_t)(slab * kTapSlab + c) * taps + tap) * kTapReplicas;
-        cell[copy] = total[k];
-        if (copy == 0)
-            for (int r = copies; r < kTapReplicas; ++r) cell[r] = 0;
+        if (it.tap_add) {
+            if (total[k]) atomicAdd(reinterpret_cast<unsigned long long *>(cell + range % kTapReplicas), (unsigned long long)total[k]);
+            continue;
+        }
+        cell[range] = total[k];
+        if (range == 0)
+            for (int r = ranges; r < kTapReplicas; ++r) cell[r] = 0;
     }
 }
 
 __host__ __device__ inline int tap_slabs(const FinishItem &it) { return (it.d.c_out + kTapSlab - 1) / kTapSlab; }
 
-// kLetIn: the launch behind this one is the layer's GEMM (see conv_wgrad_impl)
-template <bool kLetIn>
+template <TapsOrder kOrder>
 // (at most 64 registers: a block and a CTA of the GEMM share an SM)
 __global__ void __launch_bounds__(kTapThreads, 2) finish_taps_kernel(const __grid_constant__ FinishBatch b)
 {
-    ptx::grid_dep_wait();
-    if (kLetIn) ptx::grid_dep_launch();
-    extern __shared__ __align__(16) int32_t dyn[];
+    if (kOrder != kTapsBeside) ptx::grid_dep_wait();
+    if (kOrder == kTapsFirst) ptx::grid_dep_launch();
+    extern __shared__ __align__(16) int32_t sets[];
     const int k = finish_item_of(b.tap_first, b.num, (int)blockIdx.x);
-    // (copies and clusters come in powers of two)
-    const int local = (int)blockIdx.x - b.tap_first[k], copies = b.item[k].tap_copies, cluster_log = 31 - __clz(b.tap_cluster);
-    const int copy = (local >> cluster_log) & (copies - 1), slab = local >> (cluster_log + 31 - __clz(copies));
-    finish_taps_slab<kTapThreads>(b.item[k], slab, copy, copies, b.tap_cluster, local & (b.tap_cluster - 1), dyn + kMaxTaps * kTapSlab, dyn);
+    const int local = (int)blockIdx.x - b.tap_first[k], ranges = b.item[k].tap_ranges, slab = local / ranges;
+    finish_taps_slab<kTapThreads, kOrder == kTapsBeside>(b.item[k], slab, local - slab * ranges, ranges, sets);
+    if (kOrder == kTapsBeside) ptx::grid_dep_wait();   // (what comes behind this launch waits for it alone)
 }
 
 // ------------------------------------------------------------------ exact sums and their maximum
@@ -412,6 +403,11 @@ __global__ void __launch_bounds__(kThreads) finish_code_kernel(const __grid_cons
         *it.g_exp = M ? p_in + t - 7 : p_in;
         if (!M) atomicOr(status, EOQ_DEV_SQ_ZERO);
     }
+    if (it.tap_clear)
+        for (uint32_t i = (uint32_t)bx * kThreads + threadIdx.x; i < (uint32_t)(it.d.c_out * it.d.kh * it.d.kw); i += (uint32_t)it.sq_blocks * kThreads) {
+            longlong2 *cell = reinterpret_cast<longlong2 *>(it.tap_sums) + (size_t)i * (kTapReplicas / 2);
+            cell[0] = cell[1] = make_longlong2(0, 0);
+        }
     // sums below 2^31 - 2^(t - 8): a right shift in four 32-bit operations (see sq_code32_shr)
     const bool fast = t >= 8 && M < 0x7e000000ull;
     const int sh = t - 7, half_m1 = fast ? (1 << (sh - 1)) - 1 : 0;
@@ -470,7 +466,7 @@ __global__ void __launch_bounds__(kSmallThreads + 160) finish_small_kernel(const
     const int rank = (int)blockIdx.x;
     if (it.use_b1) {
         const int slabs = tap_slabs(it), copies = slabs <= kSmallCtas / 4 ? 4 : (slabs <= kSmallCtas / 2 ? 2 : 1);
-        for (int i = rank; i < slabs * copies; i += kSmallCtas) finish_taps_slab<kSmallThreads>(it, i / copies, i % copies, copies, 1, 0, dyn, nullptr);
+        for (int i = rank; i < slabs * copies; i += kSmallCtas) finish_taps_slab<kSmallThreads, false>(it, i / copies, i % copies, copies, dyn);
     }
     ptx::cluster_wait();
     if (it.use_b1) {
@@ -564,26 +560,23 @@ __global__ void __launch_bounds__(kSmallThreads + 160) finish_small_kernel(const
 
 }  // namespace
 
-// Copies of the item's tap sums, and blocks of a cluster for each: a block reads 16 KB of e3 or more (a fraction of a round of its
-// loads; the small ones of a batch of 1 leave SMs to the error chain), and up to 128 KB, two rounds, as long as a cluster can grow.
-static unsigned long long tap_bytes(const FinishItem &it) { return it.pixels * (it.d.c_out < kTapSlab ? it.d.c_out : kTapSlab); }
-static int tap_copies(const FinishItem &it)
+// Ranges of rows of a slab's tap sums, a block each.  A block reads at least 16 KB of e3 (a fraction of a round of its loads; the small
+// ones of a batch of 1 leave SMs to the error chain) and beyond kTapReplicas blocks 128 KB, two rounds: fewer of them leave the chain beside them
+// more of the device (ResNet-20 step at batch 128 with 32 KB 532 us, with 128 KB 516).  A layer that has the device to itself (`alone`) is split
+// down to 32 KB, into a block for every SM in all (512 -> 2048 channels by 1 x 1, 7 x 7, batch 32, 256 blocks: 19.2 us for the weight gradient, 128: 16.7).
+static int split_taps(const FinishItem &it, int sm_count, bool alone)
 {
-    int copies = 1;
-    while (copies < kTapReplicas && tap_bytes(it) > (16ull << 10) * copies) copies *= 2;
-    return copies;
-}
-static int tap_cluster(const FinishItem &it)
-{
-    int cluster = 1;
-    while (cluster < kTapMostCluster && tap_bytes(it) > (128ull << 10) * kTapReplicas * cluster) cluster *= 2;
-    return cluster;
+    const unsigned long long bytes = it.pixels * (it.d.c_out < kTapSlab ? it.d.c_out : kTapSlab), share = (alone ? 32ull : 128ull) << 10;
+    const int most = !alone ? 32 : (sm_count / tap_slabs(it) > 0 ? sm_count / tap_slabs(it) : 1);
+    int ranges = 1;
+    while (ranges < kTapReplicas && 2 * ranges <= most && bytes > (16ull << 10) * ranges) ranges *= 2;
+    const unsigned long long want = (bytes + share - 1) / share;
+    return want <= (unsigned long long)ranges ? ranges : (want < (unsigned long long)most ? (int)want : (most > ranges ? most : ranges));
 }
 
 // The launch geometry of an item, from its sizes.
 static void plan_finish_item(FinishItem &it, int sm_count, bool alone)
 {
-    it.tap_copies = tap_copies(it);
     it.groups = it.num_parts >= 64 ? 16 : (it.num_parts >= 32 ? 8 : (it.num_parts >= 8 ? 4 : 1));
     const size_t quads = (size_t)it.n / 4, bw = kThreads / it.groups;
     size_t fb = (quads + bw - 1) / bw;
@@ -593,19 +586,19 @@ static void plan_finish_item(FinishItem &it, int sm_count, bool alone)
     it.sq_blocks = (int)(qb < 1 ? 1 : (qb > cap ? cap : qb));
 }
 
-void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, const ReduceHook &hook)
+void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, bool whole_device, const ReduceHook &hook)
 {
     b.num = num;
-    b.tap_cluster = 1;
-    for (int k = 0; k < num; ++k)
-        if (items[k].use_b1 && tap_cluster(items[k]) > b.tap_cluster) b.tap_cluster = tap_cluster(items[k]);
     b.tap_first[0] = b.fin_first[0] = b.sq_first[0] = 0;
     for (int k = 0; k < num; ++k) {
         FinishItem &it = b.item[k];
         it = items[k];
         it.keep_sums = hook.fn != nullptr;
+        it.tap_ranges = split_taps(it, sm_count, num == 1 && whole_device);
+        it.tap_add = it.tap_ranges > kTapReplicas;
+        it.tap_clear = it.tap_clear && it.use_b1 && (split_taps(it, sm_count, true) > kTapReplicas || split_taps(it, sm_count, false) > kTapReplicas);
         plan_finish_item(it, sm_count, num == 1);
-        b.tap_first[k + 1] = b.tap_first[k] + (it.use_b1 ? tap_slabs(it) * it.tap_copies * b.tap_cluster : 0);
+        b.tap_first[k + 1] = b.tap_first[k] + (it.use_b1 ? tap_slabs(it) * it.tap_ranges : 0);
         b.fin_first[k + 1] = b.fin_first[k] + it.fin_blocks;
         b.sq_first[k + 1] = b.sq_first[k] + it.sq_blocks;
     }
@@ -634,7 +627,7 @@ bool finish_is_small(const FinishItem &it, const ReduceHook &hook)
 
 cudaError_t launch_finish_small(FinishItem it, unsigned *status, int sm_count, bool beside, cudaStream_t s)
 {
-    it.keep_sums = 0;
+    it.keep_sums = it.tap_add = 0;
     plan_finish_item(it, sm_count, true);
     it.groups = small_groups(it);
     const size_t sums = (it.n / 4 + kSmallCtas - 1) / kSmallCtas * 4 * sizeof(long long), sets = tap_set_bytes(it);
@@ -642,25 +635,24 @@ cudaError_t launch_finish_small(FinishItem it, unsigned *status, int sm_count, b
                                    (int)beside);   // (16 KB of sums, or 17 KB of sets)
 }
 
-cudaError_t launch_finish_taps(const FinishBatch &b, bool let_in, cudaStream_t s)
+bool finish_taps_first(const FinishItem &it)
 {
-    size_t smem = 0;
+    constexpr size_t kTapsFirstBytes = 256 * 1024;
+    return !it.tap_add && it.pixels * it.d.c_out <= kTapsFirstBytes;
+}
+
+cudaError_t launch_finish_taps(const FinishBatch &b, TapsOrder order, cudaStream_t s)
+{
+    size_t smem = 0;   // at most 64 border classes, 130 sets: 17 KB
     for (int k = 0; k < b.num; ++k) smem = tap_set_bytes(b.item[k]) > smem ? tap_set_bytes(b.item[k]) : smem;
-    smem += sizeof(int32_t) * kMaxTaps * kTapSlab;   // (at most 64 border classes, 130 sets: 25 KB in all)
-    if (!let_in) return launch_chained_clusters(b.tap_cluster, finish_taps_kernel<false>, b.tap_first[b.num], kTapThreads, smem, s, b);
-    // An SM divides its memory between L1 and shared memory when it is idle: the GEMM's CTAs find room beside these blocks only if
-    // they leave it as much shared memory as there is.
-    static std::atomic<unsigned long long> divided;
-    int device = 0;
-    cudaError_t e = cudaGetDevice(&device);
-    if (e != cudaSuccess) return e;
-    const unsigned long long bit = device < 64 ? 1ull << device : 0ull;
-    if (!(divided.load(std::memory_order_relaxed) & bit)) {
-        e = cudaFuncSetAttribute(finish_taps_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (order == kTapsFirst) {
+        static std::atomic<unsigned long long> allowed;
+        const cudaError_t e = allow_smem((const void *)finish_taps_kernel<kTapsFirst>, 48 * 1024, allowed, true);
         if (e != cudaSuccess) return e;
-        divided.fetch_or(bit, std::memory_order_relaxed);
     }
-    return launch_chained_clusters(b.tap_cluster, finish_taps_kernel<true>, b.tap_first[b.num], kTapThreads, smem, s, b);
+    const auto kernel = order == kTapsFirst ? finish_taps_kernel<kTapsFirst> : (order == kTapsBeside ? finish_taps_kernel<kTapsBeside> : finish_taps_kernel<kTapsBehind>);
+    launch_chained(kernel, b.tap_first[b.num], kTapThreads, smem, s, b);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_finish_sums(const FinishBatch &b, unsigned *status, cudaStream_t s, const ReduceHook &hook)

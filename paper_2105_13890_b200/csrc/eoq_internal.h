@@ -21,14 +21,16 @@ constexpr uint32_t kSpinLimit = 1u << 22;  // polls before a wait gives up (norm
 
 // Lets a kernel have `bytes` of dynamic shared memory; asked once per kernel and device (`done`: a bit per device), since the
 // runtime call costs as much host time as a quarter of a launch.
-inline cudaError_t allow_smem(const void *kernel, int bytes, std::atomic<unsigned long long> &done)
+// leave_room: its SMs also get all the shared memory there is, so that blocks of a later launch find some beside it.
+inline cudaError_t allow_smem(const void *kernel, int bytes, std::atomic<unsigned long long> &done, bool leave_room = false)
 {
     int device = 0;
     const cudaError_t got = cudaGetDevice(&device);
     if (got != cudaSuccess) return got;
     const unsigned long long bit = device < 64 ? 1ull << device : 0ull;
     if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && leave_room) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
     return e;
 }
@@ -274,8 +276,9 @@ struct WgradParams {
     int row_window_kw;   // 0, or the filter width when an M tile is one filter row of 8 x 16 bytes (7 real taps of 8)
     unsigned char tap_dh[kMaxTaps], tap_dw[kMaxTaps];
     int32_t *partials;   // [num_k_splits][c_out][taps][c_in] partial sums, a slice per split
-    unsigned long long *zero;   // the cell of the maximum that the kernels behind reduce: cleared here
-    int launch_early;    // the next kernel on the stream starts beside this one (see launch_finish_small)
+    int4 *zero;          // cells that the kernels behind reduce into: cleared here, zero_n16 groups of 16 bytes
+    unsigned zero_n16;
+    int launch_early;    // the next kernel on the stream starts beside this one (see launch_finish_taps, launch_finish_small)
     int wait_late;       // the launch in front is the layer's launch_finish_taps: this one runs beside it and waits for it at its end
     DeviceState *dev;
 };
@@ -306,7 +309,8 @@ struct WgradPatchPlan {
     int num_stages;
     int rows_total;      // taps * c_in
     int32_t *partials;   // [num_splits][c_out][taps][c_in]
-    unsigned long long *zero;   // as in WgradParams
+    int4 *zero;          // as in WgradParams
+    unsigned zero_n16;
     int launch_early, wait_late;
     DeviceState *dev;
 };
@@ -324,7 +328,8 @@ struct WgradRowsPlan {
     int rows_per_split, num_splits;
     int rows_total;      // kh * kw * c_in
     int32_t *partials;   // [num_splits][c_out][kh][kw][c_in]
-    unsigned long long *zero;   // as in WgradParams
+    int4 *zero;          // as in WgradParams
+    unsigned zero_n16;
     DeviceState *dev;
 };
 cudaError_t launch_wgrad_rows(const WgradRowsPlan &pl, const CUtensorMap &map_x, const CUtensorMap &map_e, cudaStream_t stream);
@@ -392,7 +397,7 @@ struct BorderClasses {
 };
 cudaError_t launch_b1_weight_table(const int8_t *w, int32_t *table, const eoq_conv_desc_t &d, const BorderClasses &bc,
                                    cudaStream_t s);
-constexpr int kTapReplicas = 4;  // copies of the b1 error sums of a weight gradient, each over a part of the rows
+constexpr int kTapReplicas = 4;  // copies of the b1 error sums of a weight gradient, each over its part of the rows
 constexpr int kMaxBorderClasses = 64;  // classes (rows x columns) the b1 kernels keep in shared memory
 
 // eoq_weight_prep: one launch derives the b1 tables (and the row-padded first-layer weights) of up to kPrepChunk layers
@@ -476,21 +481,26 @@ struct FinishItem {
     BorderClasses bc;
     int ho, wo, num_parts;
     // filled by plan_finish
-    int tap_copies, groups, fin_blocks, sq_blocks;
+    int tap_ranges, groups, fin_blocks, sq_blocks;
+    int tap_add;                   // the tap sums are added to cells that the GEMM has cleared (else stored)
+    int tap_clear;                 // the codes' kernel clears them again: the slices can be finished once more, under any plan (set by the caller where
+                                   // the GEMM was another call)
     int keep_sums;                 // reduce hook: the sums are completed by an all-reduce before their maximum is taken
 };
 struct FinishBatch {
     int num;
-    int tap_cluster;   // blocks of a cluster of the tap sums' launch
     int tap_first[kFinishChunk + 1], fin_first[kFinishChunk + 1], sq_first[kFinishChunk + 1];
     FinishItem item[kFinishChunk];
 };
 // Lays out the launches of up to kFinishChunk items; then, in this order on one stream, the b1 error sums (only where an item
 // has a b1 term: tap_first[num] > 0) and the sums with Q_g (two kernels, a third per item under a reduce hook).
-// let_in: the launch behind the error sums is the item's GEMM with wait_late, which runs beside them: they let it in once everything
-// in front of them is complete, and it waits for them at its end.
-void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, const ReduceHook &hook);
-cudaError_t launch_finish_taps(const FinishBatch &b, bool let_in, cudaStream_t s);
+// whole_device: the GEMMs of the handle may use all SMs, so nothing of another stream is expected beside a single item's error sums.
+// Where the b1 error sums stand: first: the launch behind them is the item's GEMM with wait_late, which they let in; beside: the launch in
+// front of them is the item's GEMM with launch_early; behind: neither, they wait for what is in front.
+enum TapsOrder { kTapsFirst, kTapsBeside, kTapsBehind };
+bool finish_taps_first(const FinishItem &it);
+void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count, bool whole_device, const ReduceHook &hook);
+cudaError_t launch_finish_taps(const FinishBatch &b, TapsOrder order, cudaStream_t s);
 // ... or all of it in one launch, for one small item (no reduce hook).  beside: the launch in front on the stream is the item's GEMM,
 // which lets its successor start once e3 is complete (launch_early); the error sums are then formed beside it.
 bool finish_is_small(const FinishItem &it, const ReduceHook &hook);

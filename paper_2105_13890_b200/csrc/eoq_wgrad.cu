@@ -106,7 +106,7 @@ wgrad_kernel(const __grid_constant__ WgradParams p, const __grid_constant__ CUte
     // already (they were when the tap sums let this launch in), and the tap sums write nothing that it reads.
     if (!p.wait_late) ptx::grid_dep_wait();
     if (p.launch_early) ptx::grid_dep_launch();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *p.zero = 0;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < p.zero_n16; i += gridDim.x * blockDim.x) p.zero[i] = make_int4(0, 0, 0, 0);
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, p.dev};
 
@@ -252,7 +252,7 @@ size_t wgrad_smem_bytes(const WgradParams &p)
 cudaError_t launch_wgrad(const WgradParams &p, const CUtensorMap &map_x, const CUtensorMap &map_e, cudaStream_t stream)
 {
     static std::atomic<unsigned long long> allowed;
-    const cudaError_t e = allow_smem((const void *)wgrad_kernel, 208 * 1024, allowed);
+    const cudaError_t e = allow_smem((const void *)wgrad_kernel, 208 * 1024, allowed, true);
     if (e != cudaSuccess) return e;
     const int grid = p.num_m_groups * p.num_n_tiles * p.num_k_splits;
     const size_t need = wgrad_smem_bytes(p), least = p.wait_late ? 116 * 1024 : 0;   // (as launch_wgrad_patch)

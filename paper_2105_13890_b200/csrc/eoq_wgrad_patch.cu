@@ -91,7 +91,7 @@ wgrad_patch_kernel(const __grid_constant__ WgradPatchPlan pl, const __grid_const
     // already (they were when the tap sums let this launch in), and the tap sums write nothing that it reads.
     if (!pl.wait_late) ptx::grid_dep_wait();
     if (pl.launch_early) ptx::grid_dep_launch();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *pl.zero = 0;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < pl.zero_n16; i += gridDim.x * blockDim.x) pl.zero[i] = make_int4(0, 0, 0, 0);
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, pl.dev};
 
@@ -216,9 +216,9 @@ cudaError_t launch_wgrad_patch(const WgradPatchPlan &pl, const CUtensorMap &map_
                                cudaStream_t stream)
 {
     static std::atomic<unsigned long long> allowed;
-    const cudaError_t e = allow_smem((const void *)wgrad_patch_kernel, 208 * 1024, allowed);
+    const cudaError_t e = allow_smem((const void *)wgrad_patch_kernel, 208 * 1024, allowed, true);
     if (e != cudaSuccess) return e;
-    // (beside the tap sums, CTAs of less than half an SM's shared memory would meet on the SMs that those leave empty)
+    // (behind the tap sums, CTAs of less than half an SM's shared memory would meet on the SMs that those leave empty)
     const size_t need = wgrad_patch_smem_bytes(pl), least = pl.wait_late ? 116 * 1024 : 0;
     return launch_chained(wgrad_patch_kernel, pl.num_groups * pl.num_splits, kWgradPatchThreads, need > least ? need : least, stream, pl, map_x, map_e);
 }

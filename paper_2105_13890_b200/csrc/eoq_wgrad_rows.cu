@@ -90,7 +90,7 @@ wgrad_rows_kernel(const __grid_constant__ WgradRowsPlan pl, const __grid_constan
     __syncthreads();
     ptx::tc_fence_after();
     ptx::grid_dep_wait();   // everything up to here touched no global memory
-    if (blockIdx.x == 0 && threadIdx.x == 0) *pl.zero = 0;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < pl.zero_n16; i += gridDim.x * blockDim.x) pl.zero[i] = make_int4(0, 0, 0, 0);
     const uint32_t tmem_base = tmem_base_s;
     const RoleCtx ctx{&abort_s, pl.dev};
 
