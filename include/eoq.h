@@ -503,10 +503,11 @@ EOQ_API int eoq_probe_mma_i8(eoq_handle_t handle, int n_cols, int iters, int lau
 EOQ_API int eoq_describe_plan(eoq_handle_t handle, const eoq_conv_desc_t *desc, int pass, char *buf, size_t buf_bytes);
 
 /* Self-test of the bounded device waits: the next eoq_err_prescale / eoq_err_prescale_dev call on this handle
- * waits, in the place of its work, for one arrival more than there are, with a limit of 2048
- * polls (about 0.2 ms).  The wait runs out, the kernel raises EOQ_DEV_TIMEOUT, writes no output and returns;
- * eoq_last_status then reports the bit and puts the handle's reduction cells back to zero.  Nothing faults or
- * hangs; one call only, then the handle behaves normally again. */
+ * runs, in the place of its work, the waits of the GEMM kernels on a barrier that gets one arrival too few, one of them
+ * with a limit of 256 polls.  It runs out and raises EOQ_DEV_TIMEOUT, the other leaves by the abort flag; the kernel leaves
+ * the handle's reduction cells as one that gave up may leave them, writes no output and returns.  eoq_last_status then
+ * reports the bit and puts the cells back to zero; call it before the next use of the handle, which then behaves
+ * normally again.  Nothing faults or hangs. */
 EOQ_API int eoq_debug_force_wait_timeout(eoq_handle_t handle);
 
 /* The last cudaError_t a call on this handle recorded (0 if none); handle = NULL: the last one of

@@ -7,6 +7,7 @@
 
 #include "eoq_cells.cuh"
 #include "eoq_device.cuh"
+#include "eoq_epilogue.cuh"
 #include "eoq_internal.h"
 #include "eoq_next_head.cuh"
 
@@ -858,16 +859,34 @@ prescale_apply_kernel(const int8_t *__restrict__ e0, const int32_t *e0_exp, cons
     }
 }
 
-// Self-test of the library's bounded waits (eoq_debug_force_wait_timeout): waits for `expected` arrivals of which it makes one, gives up
-// after `spin_limit` polls, flags it and returns; it takes the place of the call's passes, so nothing is written.
-__global__ void wait_self_test_kernel(DeviceState *dev, unsigned expected, uint32_t spin_limit)
+// Self-test of the bounded waits (eoq_debug_force_wait_timeout), in the place of the call's passes: an mbarrier of two arrivals gets one.
+// Warp 0 waits as the GEMM kernels' MMA issuer does, runs into `limit`, raises the abort flag and flags the handle; warp 1 waits as their
+// loaders and epilogues do, sixteen times as long, and leaves by the abort flag.  Behind them the reduction cells are what a kernel that gave
+// up may leave behind.  Writes nothing else.
+__global__ void __launch_bounds__(64) wait_self_test_kernel(DeviceState *dev, uint32_t limit)
 {
-    atomicAdd(&dev->arrivals, 1u);
-    for (uint32_t it = 0; it < spin_limit; ++it) {
-        if (*reinterpret_cast<volatile unsigned *>(&dev->arrivals) >= expected) return;
-        __nanosleep(100);
+    __shared__ __align__(8) uint64_t bar_s;
+    __shared__ volatile uint32_t abort_s;
+    const uint32_t bar = ptx::smem_u32(&bar_s);
+    if (threadIdx.x == 0) {
+        abort_s = 0;
+        ptx::mbar_init(bar, 2);
+        ptx::fence_barrier_init();
     }
-    atomicOr(&dev->status, EOQ_DEV_TIMEOUT);
+    __syncthreads();
+    const RoleCtx ctx{&abort_s, dev};
+    bool met;
+    if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) ptx::mbar_arrive(bar);
+        met = __all_sync(0xffffffffu, wait_bar(bar, 0, ctx, limit));
+    } else {
+        met = __all_sync(0xffffffffu, wait_bar<64>(bar, 0, ctx, 16 * limit));
+    }
+    if (__syncthreads_or(met) || threadIdx.x != 0) return;
+    dev->absmax_u32 = 0x7f000000u;
+    dev->absmax_u64 = dev->absmax2_u64 = 1ull << 40;
+    dev->sum0 = dev->sum1 = -1;
+    dev->ticket = 1;
 }
 
 // The same in one cluster of up to kHeadCluster blocks, for tensors of that many blocks' shares: every thread keeps its share of e1 (up to
@@ -1263,7 +1282,7 @@ cudaError_t launch_err_prescale(const int8_t *e0, const int32_t *e0_exp, const u
     const size_t share = (size_t)kThreads * kHeadGroups;
     if (force_timeout) {
         *kernels = 1;
-        wait_self_test_kernel<<<1, 1, 0, s>>>(dev, 2u, 2048u);
+        wait_self_test_kernel<<<1, 64, 0, s>>>(dev, 256u);
         return cudaGetLastError();
     }
     if (!hook.fn && n16 > 0 && n16 <= kHeadCluster * share) {

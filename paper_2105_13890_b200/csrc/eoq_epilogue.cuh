@@ -1,4 +1,4 @@
-// Pieces shared by the two implicit-GEMM kernels: bounded barrier waits and the register epilogues of the
+// Pieces shared by the GEMM kernels: bounded barrier waits, and the register epilogues of the
 // forward chain and of error back-propagation (arXiv 2105.13890, Sec. 3.2.1).
 #pragma once
 #include "eoq_device.cuh"
@@ -14,10 +14,11 @@ struct RoleCtx {
 // Bounded wait on an mbarrier phase.  Every polling warp takes issue slots from the warp that feeds the tensor
 // core (one thread, whose scalar work between two MMAs is on the critical path), so waiters that can afford a
 // few dozen nanoseconds of extra latency (loaders, epilogue) back off between polls; the MMA issuer does not.
+// Only the self-test of the waits gives another `limit`.
 template <int kBackoffNs = 0>
-__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const RoleCtx &c)
+__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const RoleCtx &c, uint32_t limit = kSpinLimit)
 {
-    for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    for (uint32_t i = 0; i < limit; ++i) {
         if (ptx::mbar_try_wait(bar, parity)) return true;
         if (*c.abort_flag) return false;
         if (kBackoffNs > 0) __nanosleep(kBackoffNs);

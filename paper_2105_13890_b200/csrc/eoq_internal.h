@@ -73,10 +73,9 @@ struct DeviceState {
     unsigned long long absmax2_u64;  // second maximum of a call that also serves its consumer's error head (masked |.|)
     unsigned tensor_absmax[256];  // per-tensor maxima of the multi-tensor update (zero between calls)
     unsigned ticket;       // blocks of the kernel that consumes the cells last count themselves here (see last_block_done)
-    unsigned arrivals;     // what the self-test of the bounded waits waits for
     unsigned long long probe_cycles;  // eoq_probe_mma_i8: longest issue loop of the last launch, in SM clock cycles
 };
-// Invariant: absmax_u32, absmax_u64, absmax2_u64, sum0, sum1, ticket and arrivals are zero whenever no call is in flight on the handle.
+// Invariant: absmax_u32, absmax_u64, absmax2_u64, sum0, sum1 and ticket are zero whenever no call is in flight on the handle.
 // The kernel that reads a call's reductions last puts the cells it used back to zero (its last block does), so
 // no call starts with a memset.  A kernel that gave up on a wait (EOQ_DEV_TIMEOUT) may leave them dirty:
 // eoq_last_status clears them again when it reports that bit.
@@ -129,7 +128,7 @@ struct Handle {
     bool profiling;
     ReduceHook hook;              // all-reduce between the phases of every batch-wide reduction (data-parallel replicas)
     bool gemm_only;               // timing aid: dgrad and wgrad calls launch their GEMM kernel only (eoq_profile_gemm_only)
-    bool force_timeout;           // self-test: the next error-head call is a bounded wait that runs out
+    bool force_timeout;           // self-test: the next error-head call is a pair of bounded waits that run out
     int num_records;
     ProfRecord *records;          // kMaxProfRecords entries, allocated on first eoq_profile_start
     int gemm_ctas;                // most CTAs a GEMM call of this handle may use (eoq_set_gemm_ctas; default: one per SM)

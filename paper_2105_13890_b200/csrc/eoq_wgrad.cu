@@ -10,6 +10,7 @@
 // stages rotate over the three producers and a stage's loads go out by the lanes of one.  With a thread each for a third of every
 // stage's loads the 64 -> 128 channel 3x3/2 layer at batch 64 took 23.0 us (now 11.0), 512 -> 256 1x1 28 x 28 at batch 32 17.4 (9.6).
 #include "eoq_device.cuh"
+#include "eoq_epilogue.cuh"
 #include "eoq_internal.h"
 
 namespace eoq {
@@ -18,22 +19,6 @@ namespace {
 
 constexpr int kMaxStages = 8;
 constexpr int kProducers = 3;
-
-struct RoleCtx {
-    volatile uint32_t *abort_flag;
-    DeviceState *dev;
-};
-
-__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const RoleCtx &c)
-{
-    for (uint32_t i = 0; i < kSpinLimit; ++i) {
-        if (ptx::mbar_try_wait(bar, parity)) return true;
-        if (*c.abort_flag) return false;
-    }
-    *c.abort_flag = 1u;
-    atomicOr(&c.dev->status, EOQ_DEV_TIMEOUT);
-    return false;
-}
 
 // Descriptor of an MN-major operand made of sub-tiles [pixels][row_bytes], `sub_bytes` apart along M/N.
 // Swizzled rows: atoms along M/N are `sub_bytes` apart (leading offset), 8-pixel groups 8*row_bytes apart

@@ -418,7 +418,7 @@ def eoq_describe_plan(handle, desc, pass_: int) -> str:
 
 
 def eoq_debug_force_wait_timeout(handle) -> None:
-    """Makes the next error-head call on this handle a bounded wait that runs out."""
+    """Makes the next error-head call on this handle a bounded wait that runs out; eoq_last_status then clears the handle."""
     _check(lib().eoq_debug_force_wait_timeout(handle), "eoq_debug_force_wait_timeout")
 
 
