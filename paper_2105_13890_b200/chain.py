@@ -143,7 +143,10 @@ class ChainedStep:
         dev_index = dev.index if dev.index is not None else 0
         # weight gradients, projections (`branch`), and the last: finishing and updating stages
         self.h_sides = [eoq.eoq_create(dev_index) for _ in range(side_streams + 2)]
-        self.workspace_sides = [torch.empty(ws, dtype=torch.uint8, device=dev) for _ in range(side_streams + 1)]
+        self.workspace_sides = [torch.empty(ws, dtype=torch.uint8, device=dev) for _ in range(side_streams)]
+        # (`branch` back-propagates the errors of projections and nothing else)
+        self.workspace_sides.append(torch.empty(max([256] + [eoq.eoq_workspace_size(blk.proj.desc, eoq.EOQ_PASS_DGRAD)
+                                                             for blk in self.blocks if blk.proj]), dtype=torch.uint8, device=dev))
         # a third of the SMs for each of the weight-gradient GEMMs, so that the error chain finds free ones (ResNet-18 step at
         # batch 64: 1576 us with all SMs, 1502 with half, 1474 with a third, 1480 with a quarter; at batch 13: 769, 727, 717, 715)
         third = torch.cuda.get_device_properties(dev).multi_processor_count // 3
