@@ -263,6 +263,12 @@ __global__ void __launch_bounds__(kTapThreads, 2) finish_taps_kernel(const __gri
     if (kOrder == kTapsBeside) ptx::grid_dep_wait();   // (what comes behind this launch waits for it alone)
 }
 
+__device__ __forceinline__ void clear_tap_cell(const FinishItem &it, uint32_t i)
+{
+    longlong2 *cell = reinterpret_cast<longlong2 *>(it.tap_sums) + (size_t)i * (kTapReplicas / 2);
+    cell[0] = cell[1] = make_longlong2(0, 0);
+}
+
 // ------------------------------------------------------------------ exact sums and their maximum
 // A thread owns four neighbouring weights (c_in is a multiple of 4: they share their (oc, tap)); a block is (256 / groups) such
 // quads x `groups` slice groups that meet in shared memory.  The sums are written once, as int32 where they provably fit.
@@ -404,10 +410,8 @@ __global__ void __launch_bounds__(kThreads) finish_code_kernel(const __grid_cons
         if (!M) atomicOr(status, EOQ_DEV_SQ_ZERO);
     }
     if (it.tap_clear)
-        for (uint32_t i = (uint32_t)bx * kThreads + threadIdx.x; i < (uint32_t)(it.d.c_out * it.d.kh * it.d.kw); i += (uint32_t)it.sq_blocks * kThreads) {
-            longlong2 *cell = reinterpret_cast<longlong2 *>(it.tap_sums) + (size_t)i * (kTapReplicas / 2);
-            cell[0] = cell[1] = make_longlong2(0, 0);
-        }
+        for (uint32_t i = (uint32_t)bx * kThreads + threadIdx.x; i < (uint32_t)(it.d.c_out * it.d.kh * it.d.kw); i += (uint32_t)it.sq_blocks * kThreads)
+            clear_tap_cell(it, i);
     // sums below 2^31 - 2^(t - 8): a right shift in four 32-bit operations (see sq_code32_shr)
     const bool fast = t >= 8 && M < 0x7e000000ull;
     const int sh = t - 7, half_m1 = fast ? (1 << (sh - 1)) - 1 : 0;
@@ -536,6 +540,9 @@ __global__ void __launch_bounds__(kSmallThreads + 160) finish_small_kernel(const
         ptx::st_cluster_128(ptx::cluster_addr(ptx::smem_u32(&max_s[rank][0]), threadIdx.x), (uint32_t)m, (uint32_t)(m >> 32), 0u, 0u);
     }
     ptx::cluster_sync();
+    if (it.use_b1 && it.tap_clear)   // (every CTA has read the cells)
+        for (uint32_t i = rank * kSmallThreads + threadIdx.x; i < (uint32_t)(it.d.c_out * it.d.kh * it.d.kw); i += kSmallCtas * kSmallThreads)
+            clear_tap_cell(it, i);
     unsigned long long M = 0;
 #pragma unroll
     for (int r = 0; r < kSmallCtas; ++r) M = max_s[r][0] > M ? max_s[r][0] : M;

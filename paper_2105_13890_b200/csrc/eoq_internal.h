@@ -482,7 +482,7 @@ struct FinishItem {
     // filled by plan_finish
     int tap_ranges, groups, fin_blocks, sq_blocks;
     int tap_add;                   // the tap sums are added to cells that the GEMM has cleared (else stored)
-    int tap_clear;                 // the codes' kernel clears them again: the slices can be finished once more, under any plan (set by the caller where
+    int tap_clear;                 // the last kernel clears them again: the slices can be finished once more, under any plan (set by the caller where
                                    // the GEMM was another call)
     int keep_sums;                 // reduce hook: the sums are completed by an all-reduce before their maximum is taken
 };

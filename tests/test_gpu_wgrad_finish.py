@@ -216,6 +216,30 @@ def test_slices_finished_more_than_once(case):
     eoq.eoq_destroy(capped)
 
 
+@pytest.mark.parametrize("case", [(12, 32, 32, 16, 16, 3, 1, 1, -2), (7, 31, 33, 16, 32, 3, 1, 1, 5)], ids=["16", "32"])
+def test_small_slices_finished_again_under_another_plan(case):
+    """A small layer is finished by one launch that stores its error sums; a profile has them added up by a kernel of their own."""
+    d, e3, x0, b1, g_o, pg_o = make(case, 8980)
+    gd, h, capped = G.gdesc(d), eoq.eoq_create(0), eoq.eoq_create(0)
+    eoq.eoq_set_gemm_ctas(capped, 40)   # (few slices: a small layer)
+    ws = G.workspace(gd, eoq.EOQ_PASS_WGRAD)
+    ws.fill_(0x5A)
+    e3_d, pe, b1_d = G.dev(e3), G.dev(np.array([-12], dtype=np.int32)), G.dev(np.array([b1], dtype=np.int32))
+    parts = eoq.eoq_conv_wgrad_gemm(capped, gd, e3_d, pe, G.dev(x0), ws)
+    for profiled in (False, True, False, True):
+        g, pg = G.empty(g_o.shape, torch.int8), G.zeros(1, torch.int32)
+        if profiled:
+            eoq.eoq_profile_start(h)
+        before = eoq.eoq_launch_count(h)
+        eoq.eoq_wgrad_finish(h, [gd], [e3_d], [pe], [b1_d], [g], [pg], [ws], [parts])
+        assert eoq.eoq_launch_count(h) - before == (3 if profiled else 1)
+        if profiled:
+            eoq.eoq_profile_stop(h)
+        assert eoq.eoq_last_status(h) == 0 and np.array_equal(G.host(g), g_o) and pg.item() == pg_o
+    eoq.eoq_destroy(h)
+    eoq.eoq_destroy(capped)
+
+
 @pytest.mark.parametrize("n,extent,c_in,c_out", [(512, 56, 64, 64), (512, 56, 16, 32), (256, 112, 32, 32)])
 def test_error_sums_of_few_channels_hide_beside_the_gemm(n, extent, c_in, c_out):
     """A bias in front of the convolution costs a large weight gradient the adding up of its error sums and little more: they are read beside
