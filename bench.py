@@ -412,7 +412,8 @@ def run_gpu(args):
                        "update": "stochastic rounding (extension)" if args.stochastic else "round to nearest even (Sec. 3.2.2)",
                        "parallelism": f"replicas x{world}",
                        "launch": "eager, one stream" if args.eager else
-                                 "CUDA graph replay, weight-gradient GEMMs on two side streams, stages finished and updated on a third" if chained
+                                 "CUDA graph replay, weight-gradient GEMMs on two side streams, projections on a third, "
+                                 "stages finished and updated on a fourth" if chained
                                  else "CUDA graph replay, wgrad chains on two side streams"},
             "clocks": clocks,
             "e2e": {"value": tops_e2e, "unit": "TOPS", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,

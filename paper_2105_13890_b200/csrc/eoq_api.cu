@@ -294,10 +294,10 @@ void plan_igemm(IgemmParams &p, int src_channels, int ntaps, int sm_count)
     const bool spare = (long long)p.num_m_tiles * ((p.N + 255) / 256) >= 2LL * sm_count;
     if (tn == 256 && !spare) tn = 128;
     if (p.N > 128 && !p.b_mn) {
-        // Forward: cuts of equal width (28 x 28 at batch 64, 1024 -> 304 channels: two of 160 instead of 256 and 48, 28.3 -> 25.9 us).  Up to
-        // 512 terms the epilogue bounds the layer, and its time goes by the columns of the busiest CTA: narrow tiles then where that has
-        // at least four wide ones and they leave it fewer columns (64 -> 512 channels with shortcut 54.3 -> 45.0 us, 512 -> 512 59.6 -> 53.7; without shortcut 1024 -> 256
-        // at 14 x 14, batch 512: 35.6 us wide, 36.6 narrow).
+        // Forward: cuts of equal width (28 x 28 at batch 64, 1024 -> 304 channels: two of 160 instead of 256 and 48, 28.3 -> 25.9 us).
+        // Up to 512 terms the epilogue bounds the layer, and its time goes by the columns of the busiest CTA: narrow tiles then where
+        // that has at least four wide ones and they leave it fewer columns (64 -> 512 channels with shortcut 54.3 -> 45.0 us,
+        // 512 -> 512 59.6 -> 53.7; without shortcut 1024 -> 256 at 14 x 14, batch 512: 35.6 us wide, 36.6 narrow).
         auto cut = [&](int most) { const int parts = (p.N + most - 1) / most; return ((p.N + parts - 1) / parts + 15) / 16 * 16; };
         auto columns = [&](int cols) { return ((long long)p.num_m_tiles * ((p.N + cols - 1) / cols) + sm_count - 1) / sm_count * cols; };
         tn = tn < 256 && p.N < 256 ? tn : cut(tn);
@@ -859,7 +859,7 @@ extern "C" int eoq_create(eoq_handle_t *handle, int device)
     h->hook = ReduceHook{nullptr, nullptr};
     h->num_records = 0;
     h->records = nullptr;
-    // two attributes: cudaGetDeviceProperties took 2.5 of the call's 3.1 ms, and a training step creates four handles
+    // two attributes: cudaGetDeviceProperties took 2.5 of the call's 3.1 ms, and a training step creates five handles
     int major = 0;
     cudaError_t e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
@@ -1055,8 +1055,9 @@ extern "C" int eoq_workspace_size(const eoq_conv_desc_t *desc, int pass, size_t 
             *bytes = round256((size_t)bc.nrc * bc.ncc * desc->c_out * sizeof(int32_t)) +
                      (use_row_window(*desc, g.wo) ? round256((size_t)desc->c_out * desc->kh * 8 * desc->c_in) : 0);
             return EOQ_OK;
-        // a copy of the weights (no kernel makes one any more) + sums.  The room is that of int32 sums; as 16-bit words they fill half of it.  The size is part of
-        // the interface: callers keep buffers of it, and the allocation-free entry point accepts geometries by it.
+        // Sums behind room for a copy of the weights.  The 16-bit words of the sums fill half of theirs, and no kernel makes the copy
+        // any more.  The size is part of the interface all the same: callers keep buffers of it, and the allocation-free entry point
+        // accepts and refuses geometries by it.
         case EOQ_PASS_DGRAD:
             *bytes = round256(g.w_elems) + round256(g.in_elems * sizeof(int32_t));
             return EOQ_OK;

@@ -1286,9 +1286,9 @@ cudaError_t launch_err_prescale(const int8_t *e0, const int32_t *e0_exp, const u
         return cudaGetLastError();
     }
     if (!hook.fn && n16 > 0 && n16 <= kHeadCluster * share) {
-        // few blocks: one cluster (twice the blocks that its registers need, up to its size: the loads of a block are in turn)
+        // one cluster, of the fewest blocks that hold the tensor
         int blocks = 1;
-        while (blocks < kHeadCluster && (size_t)blocks * kThreads * 2 < n16) blocks *= 2;
+        while ((size_t)blocks * share < n16) blocks *= 2;
         *kernels = 1;
         return launch_chained_clusters(blocks, prescale_cluster_kernel, blocks, kThreads, 0, s, e0, e0_exp, mask, x2, n16, gamma_c, gamma_dev, e3,
                                        e3_exp, sum_e1, sum_e1x2, dev);

@@ -46,16 +46,19 @@ __device__ __forceinline__ bool finish_narrow(const FinishItem &it, int b1)
 // weight gradient, 11.6 so; 64 channels 56 x 56 at batch 4, 0.8 M errors, 15.6 beside, 17.2 in front).  Whichever comes second finds
 // room because the first asks its SMs for all the shared memory there is: an SM divides its memory between L1 and shared memory when it is
 // idle.  All sums in front of the GEMM, in clusters of up to eight blocks that stored what they had summed through distributed shared
-// memory, left few slabs too few blocks, and the GEMM waited for many: 16 -> 32 channels 56 x 56 at batch 512 68.3 us for the weight gradient, 58.2 so, 64 -> 64 99 and 82, 16 -> 240 by 1 x 1, 64 x 64 at batch 40,
-// 35.5 and 28.3; 64 -> 128 channels 56 x 56, stride 2, batch 64 19.9 and 19.5, 1024 -> 256 by 1 x 1, 14 x 14, batch 32 14.8 and 14.0.  Sums of
-// four pixels by dot products and no divisions in front of the first load: the kernel 7.5 -> 5.5 us for the 48 -> 80 channel strided layer.
+// memory, left few slabs too few blocks, and the GEMM waited for many: 16 -> 32 channels 56 x 56 at batch 512 68.3 us for the weight
+// gradient, 58.2 so, 64 -> 64 99 and 82, 16 -> 240 by 1 x 1, 64 x 64 at batch 40, 35.5 and 28.3; 64 -> 128 channels 56 x 56, stride 2, batch 64
+// 19.9 and 19.5, 1024 -> 256 by 1 x 1, 14 x 14, batch 32 14.8 and 14.0.  Sums of four pixels by dot products and no divisions in front of the
+// first load: the kernel 7.5 -> 5.5 us for the 48 -> 80 channel strided layer.
 struct PixelSum {
     int v[16] = {};
     // adds four pixels: the codes of a channel side by side, then one byte dot product
     __device__ __forceinline__ void add4(const int4 &p0, const int4 &p1, const int4 &p2, const int4 &p3)
     {
-        const uint32_t w0[4] = {(uint32_t)p0.x, (uint32_t)p0.y, (uint32_t)p0.z, (uint32_t)p0.w}, w1[4] = {(uint32_t)p1.x, (uint32_t)p1.y, (uint32_t)p1.z, (uint32_t)p1.w};
-        const uint32_t w2[4] = {(uint32_t)p2.x, (uint32_t)p2.y, (uint32_t)p2.z, (uint32_t)p2.w}, w3[4] = {(uint32_t)p3.x, (uint32_t)p3.y, (uint32_t)p3.z, (uint32_t)p3.w};
+        const uint32_t w0[4] = {(uint32_t)p0.x, (uint32_t)p0.y, (uint32_t)p0.z, (uint32_t)p0.w};
+        const uint32_t w1[4] = {(uint32_t)p1.x, (uint32_t)p1.y, (uint32_t)p1.z, (uint32_t)p1.w};
+        const uint32_t w2[4] = {(uint32_t)p2.x, (uint32_t)p2.y, (uint32_t)p2.z, (uint32_t)p2.w};
+        const uint32_t w3[4] = {(uint32_t)p3.x, (uint32_t)p3.y, (uint32_t)p3.z, (uint32_t)p3.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const uint32_t t0 = __byte_perm(w0[q], w1[q], 0x5140), t1 = __byte_perm(w0[q], w1[q], 0x7362), t2 = __byte_perm(w2[q], w3[q], 0x5140),
@@ -450,7 +453,10 @@ __global__ void __launch_bounds__(kThreads) finish_code_kernel(const __grid_cons
 // four rounds of loads (34,560 weights of a 48 -> 80 layer in 17 passes took 39 us where the three launches take 14).  The 16-channel
 // layer at batch 8 called by itself 42.2 -> 39.3 us with it and the error head in a cluster, the backward of the 16-channel layer
 // 32 x 32 at batch 2 29.7 -> 24.8, of a 256 -> 64 1 x 1 layer 28.2 -> 23.5.
-constexpr int kSmallCtas = 8, kSmallThreads = 512;
+// The block shares an SM with a CTA of the GEMM, beside which it comes up: launch bounds of more threads than it has keep it at 80 registers,
+// so that 24,576 of an SM's are left, a quarter of them in each of its four parts (the GEMMs take 13,824 or 16,384); without them it took 103
+// and left 12,288.  The single 16-channel layer takes the same time with either (33.4 and 33.3 us), as its GEMM leaves some SMs alone.
+constexpr int kSmallCtas = 8, kSmallThreads = 512, kSmallBounds = kSmallThreads + 160;
 constexpr size_t kSmallErrorBytes = 256 * 1024;
 
 __device__ __forceinline__ long long finish_b1_term_fresh(const FinishItem &it, int b1, uint32_t q)   // (cells written in this launch)
@@ -460,7 +466,7 @@ __device__ __forceinline__ long long finish_b1_term_fresh(const FinishItem &it, 
     return (long long)b1 * (lo.x + lo.y + hi.x + hi.y);
 }
 
-__global__ void __launch_bounds__(kSmallThreads + 160) finish_small_kernel(const __grid_constant__ FinishItem it, unsigned *status, int beside)
+__global__ void __launch_bounds__(kSmallBounds) finish_small_kernel(const __grid_constant__ FinishItem it, unsigned *status, int beside)
 {
     extern __shared__ __align__(16) int32_t dyn[];   // the tap kernel's sets, then this CTA's sums, four to a quad
     __shared__ long long part[kSmallThreads][4];
@@ -657,7 +663,9 @@ cudaError_t launch_finish_taps(const FinishBatch &b, TapsOrder order, cudaStream
         const cudaError_t e = allow_smem((const void *)finish_taps_kernel<kTapsFirst>, 48 * 1024, allowed, true);
         if (e != cudaSuccess) return e;
     }
-    const auto kernel = order == kTapsFirst ? finish_taps_kernel<kTapsFirst> : (order == kTapsBeside ? finish_taps_kernel<kTapsBeside> : finish_taps_kernel<kTapsBehind>);
+    const auto kernel = order == kTapsFirst    ? finish_taps_kernel<kTapsFirst>
+                        : order == kTapsBeside ? finish_taps_kernel<kTapsBeside>
+                                               : finish_taps_kernel<kTapsBehind>;
     launch_chained(kernel, b.tap_first[b.num], kTapThreads, smem, s, b);
     return cudaGetLastError();
 }

@@ -276,7 +276,9 @@ __device__ __forceinline__ void update_range(const UpdateTensor &T, size_t begin
     }
 }
 
-// (only the stochastic loop, the one that arithmetic bounds, is worth a form without the clamps or the product)
+// (Only the stochastic loop, the one that arithmetic bounds, is worth a form without the clamps or the product: the whole call for the
+// 21 M weights of ResNet-34 takes 32.9 us with u = g, 35.5 with a product and 37.3 with the clamps too, 42.5 before there were forms.  To
+// nearest all take the form with the clamps: 18.8 to 25.6 us, by the shift, 21.2 to 30.4 before.)
 __device__ __forceinline__ void update_range(UpdateMode mode, const UpdateTensor &T, size_t begin, size_t end, const UpdateRule &r)
 {
     switch (mode) {
