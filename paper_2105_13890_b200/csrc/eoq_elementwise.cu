@@ -117,25 +117,12 @@ __device__ __forceinline__ bool sq_shift(int tid, int32_t *dst_exp, DeviceState 
     return last_reader(dev);
 }
 
-// kMode 0: Q -> int16, 1: CQ -> int8, 2: SQ -> int8 under the reduced maximum (tiles backwards: the first pass read the last ones last).
-// Bound by memory: 4 B in (SQ: from L2 where it holds the tensor), 1 or 2 B out.
-// early (SQ): the first pass is the launch in front and lets this one in once the source is complete, so its tiles are read ahead of
-// the wait.
+// Codes of a tile whose values are at hand, kMode 0: Q -> int16, 1: CQ -> int8, 2: SQ -> int8; block 0 also those of the up to three
+// elements behind the last float4.
 template <int kMode>
-__global__ void __launch_bounds__(kThreads)
-quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp, DeviceState *dev, int early)
+__device__ __forceinline__ void store_tile(void *dst, const float *src, size_t n, size_t tile, const Pow2Scale &sc, const float4 (&v)[kQuantLoads])
 {
-    const size_t n4 = n / 4, tile = kMode == 2 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
-    if (!early) ptx::grid_dep_wait();
-    float4 v[kQuantLoads];
-    load_tile(src, n4, tile, v);
-    if (early) ptx::grid_dep_wait();
-    if (gridDim.x <= kPartSms) ptx::grid_dep_launch();
-    int up = 7;
-    bool last = false;
-    if (kMode == 2) last = sq_shift(threadIdx.x, dst_exp, dev, &up);
-    else if (blockIdx.x == 0 && threadIdx.x == 0 && dst_exp) *dst_exp = -up;
-    const Pow2Scale sc = pow2_scale(up);
+    const size_t n4 = n / 4;
 #pragma unroll
     for (int u = 0; u < kQuantLoads; ++u) {
         const size_t i = tile * kQuantTile + (size_t)u * kThreads + threadIdx.x;
@@ -147,6 +134,35 @@ quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t 
         if (kMode == 0) reinterpret_cast<int16_t *>(dst)[i] = (int16_t)c;
         else reinterpret_cast<int8_t *>(dst)[i] = (int8_t)c;
     }
+}
+
+// Q and CQ.  Bound by memory: 4 B in, 1 or 2 B out; up to some 2 M floats by the rate of launches, which goes by a kernel's parameters
+// too: 3.0 us a call in a row of calls, 3.4 with the two more that SQ's second pass takes.
+template <int kMode>
+__global__ void __launch_bounds__(kThreads) quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp)
+{
+    ptx::grid_dep_wait_launch_small();
+    float4 v[kQuantLoads];
+    load_tile(src, n / 4, blockIdx.x, v);
+    constexpr int up = 7;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && dst_exp) *dst_exp = -up;
+    store_tile<kMode>(dst, src, n, blockIdx.x, pow2_scale(up), v);
+}
+
+// SQ under the reduced maximum (tiles backwards: the first pass read the last ones last).  Bound by memory: 4 B in, from L2 where it holds
+// the tensor, 1 B out.
+// early: the first pass is the launch in front and lets this one in once the source is complete, so its tiles are read ahead of the wait.
+__global__ void __launch_bounds__(kThreads)
+quantize_sq_second_kernel(const float *__restrict__ src, size_t n, int8_t *dst, int32_t *dst_exp, DeviceState *dev, int early)
+{
+    const size_t tile = gridDim.x - 1 - blockIdx.x;
+    if (!early) ptx::grid_dep_wait_launch_small();
+    float4 v[kQuantLoads];
+    load_tile(src, n / 4, tile, v);
+    if (early) ptx::grid_dep_wait_launch_small();
+    int up;
+    const bool last = sq_shift(threadIdx.x, dst_exp, dev, &up);
+    store_tile<2>(dst, src, n, tile, pow2_scale(up), v);
     if (last) dev->absmax_u32 = 0;
 }
 
@@ -248,8 +264,7 @@ quantize_sq_kernel(const float *__restrict__ src, size_t n, int8_t *dst, int16_t
         // (the up to three elements behind the last float4 are coded by the second pass)
         if (blockIdx.x == 0 && r == 0 && threadIdx.x < (n & 3)) mx = abs_bits(src[n4 * 4 + threadIdx.x]);
 #pragma unroll
-        for (int u = 0; u < kQuantLoads; ++u)
-            mx = max(mx, abs_bits(v[u]));
+        for (int u = 0; u < kQuantLoads; ++u) mx = max(mx, abs_bits(v[u]));
         store_part(dst, n4, p, pow2_scale(guess.part(mx, threadIdx.x, dev)), v);
     }
     guess.publish(threadIdx.x, tile_shift + blockIdx.x, dev);
@@ -350,7 +365,7 @@ template <int kG, bool kStaged>
 __global__ void __launch_bounds__(kThreads)
 quantize_image_kernel(const float *__restrict__ src, ImageShape s, int8_t *dst, int32_t *dst_exp, DeviceState *dev, int early)
 {
-    if (!early) ptx::grid_dep_wait();   // (see quantize_f32_kernel)
+    if (!early) ptx::grid_dep_wait_launch_small();   // (see quantize_sq_second_kernel)
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, block = (int)(gridDim.x - 1 - blockIdx.x);
     const int row0 = block * kImageRows * (int)blockDim.y, w_mem = s.w + 2 * s.wmargin;
     int up = 7;
@@ -371,8 +386,7 @@ quantize_image_kernel(const float *__restrict__ src, ImageShape s, int8_t *dst, 
                 if (4 * i + 2 < count) v[u].z = __ldg(p + 4 * i + 2);
             }
         }
-        if (early) ptx::grid_dep_wait();
-        if (gridDim.x <= kPartSms) ptx::grid_dep_launch();
+        if (early) ptx::grid_dep_wait_launch_small();
 #pragma unroll
         for (int u = 0; u < kImageRows; ++u) reinterpret_cast<float4 *>(stage)[u * kThreads + tid] = v[u];
         last = sq_shift(tid, dst_exp, dev, &up);   // (its barrier also publishes the stage)
@@ -405,8 +419,7 @@ quantize_image_kernel(const float *__restrict__ src, ImageShape s, int8_t *dst, 
                 for (int k = 0; k < 4; ++k) v[u][k] = (in && row < s.rows && k < nch) ? __ldg(p + k) : 0.0f;
             }
             if (x0 == 0) {
-                if (early) ptx::grid_dep_wait();
-                if (gridDim.x <= kPartSms) ptx::grid_dep_launch();
+                if (early) ptx::grid_dep_wait_launch_small();
                 last = sq_shift(tid, dst_exp, dev, &up);
             }
             const Pow2Scale sc = pow2_scale(up);
@@ -1189,10 +1202,14 @@ cudaError_t launch_quantize_f32(int mode, const float *src, size_t n, void *dst,
                        (const int16_t *)tile_shift, t.tiles, t.reps, dev);
         return cudaGetLastError();
     }
-    if (mode == 2) launch_sq_maximum(src, n, dev, s, hook);
-    const int early = mode == 2 && !hook.fn;
-    const auto kernel = mode == 0 ? quantize_f32_kernel<0> : (mode == 1 ? quantize_f32_kernel<1> : quantize_f32_kernel<2>);
-    launch_chained(kernel, tiles, kThreads, 0, s, src, n, dst, dst_exp, dev, early);
+    if (mode == 2) {
+        launch_sq_maximum(src, n, dev, s, hook);
+        launch_chained(quantize_sq_second_kernel, tiles, kThreads, 0, s, src, n, static_cast<int8_t *>(dst), dst_exp, dev, (int)!hook.fn);
+    } else if (mode == 0) {
+        launch_chained(quantize_f32_kernel<0>, tiles, kThreads, 0, s, src, n, dst, dst_exp);
+    } else {
+        launch_chained(quantize_f32_kernel<1>, tiles, kThreads, 0, s, src, n, dst, dst_exp);
+    }
     return cudaGetLastError();
 }
 
