@@ -60,9 +60,9 @@ __device__ __forceinline__ void quantize_store4(void *dst, size_t i, const Pow2S
 }
 
 __device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
-__device__ __forceinline__ uint32_t abs_bits(const float4 &v)
+__device__ __forceinline__ uint32_t max_abs(uint32_t mx, const float4 &v)
 {
-    return max(max(abs_bits(v.x), abs_bits(v.y)), max(abs_bits(v.z), abs_bits(v.w)));
+    return max(max(mx, max(abs_bits(v.x), abs_bits(v.y))), max(abs_bits(v.z), abs_bits(v.w)));
 }
 
 // A block takes one tile of kQuantTile float4, eight independent, coalesced loads per thread.
@@ -79,9 +79,9 @@ __device__ __forceinline__ void load_tile(const float *__restrict__ src, size_t 
 // ------------------------------------------------------------------ SQ of a tensor beyond one cluster, and of images
 // Two passes: the maximum, then the codes, the second read out of the L2.  Whole tiles of loads are in flight in both, and the second
 // pass's blocks read theirs while the first pass ends.  Floats from memory, what a row of calls on other tensors takes each: 1 M 4.8 us, 4 M
-// 7.2, 12.8 M 17.1 (of one tensor again and again 4.0, 5.7 and 11.0).  A pass for the maximum with one load of a thread in flight: 5.6, 9.3 and
-// 20.8.  Codes formed in the first pass under a guess, and again where the guess was wrong: 5.0, 8.8 and 15.9 where it never is, 6.2, 10.9
-// and 18.8 under one element beyond all others; 64 images 224 x 224 18.5 and 25.9, so 19.9 whatever they hold.
+// 7.2, 8 M 12.6 (of one tensor again and again 4.0, 5.7 and 8.3).  A pass for the maximum with one load of a thread in flight: 5.6, 9.3 and
+// 16.0.  Codes formed in the first pass under a guess, and again where the guess was wrong: 5.0, 8.8 and 13.3 where it never is, 6.2, 10.9
+// and 15.3 under one element beyond all others; 64 images 224 x 224 18.5 and 25.9, so 19.9 whatever they hold.
 
 // First pass: the largest |x|.  Bound by memory (4 B in).
 __global__ void __launch_bounds__(kThreads) absmax_f32_kernel(const float *__restrict__ src, size_t n, DeviceState *dev)
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kThreads) absmax_f32_kernel(const float *__res
     uint32_t mx = 0;
     if (blockIdx.x == 0 && threadIdx.x < (n & 3)) mx = abs_bits(src[n / 4 * 4 + threadIdx.x]);
 #pragma unroll
-    for (int u = 0; u < kQuantLoads; ++u) mx = max(mx, abs_bits(v[u]));
+    for (int u = 0; u < kQuantLoads; ++u) mx = max_abs(mx, v[u]);
     mx = block_max_u32(mx);
     if (threadIdx.x == 0) {
         if (mx) atomicMax(&dev->absmax_u32, mx);
@@ -136,8 +136,8 @@ __device__ __forceinline__ void store_tile(void *dst, const float *src, size_t n
     }
 }
 
-// Q and CQ.  Bound by memory: 4 B in, 1 or 2 B out; up to some 2 M floats by the rate of launches, which goes by a kernel's parameters
-// too: 3.0 us a call in a row of calls, 3.4 with the two more that SQ's second pass takes.
+// Q and CQ.  Bound by memory: 4 B in, 1 or 2 B out; up to some 2 M floats by the rate of launches: 3.0 us a call in a row of calls, 3.4 as
+// instances of SQ's second pass, with its two more parameters and a wait that goes by one of them.
 template <int kMode>
 __global__ void __launch_bounds__(kThreads) quantize_f32_kernel(const float *__restrict__ src, size_t n, void *dst, int32_t *dst_exp)
 {
@@ -166,12 +166,11 @@ quantize_sq_second_kernel(const float *__restrict__ src, size_t n, int8_t *dst, 
     if (last) dev->absmax_u32 = 0;
 }
 
-// ------------------------------------------------------------------ SQ of a tensor beyond the L2 cache
-// A second read comes from memory there.  The codes depend on the tensor's maximum through R(log2 max) alone, and a tile of a few
-// thousand elements often has the tensor's R(log2 max) already.  So the first pass codes every tile under the larger of its own maximum
-// and what other blocks have reduced by then, and leaves the shift it used; the second pass, under the whole maximum, codes again the
-// tiles whose shift was another one, and returns where there are none.  Bound by memory.  28 M normal floats, from memory: 27.8 us, 38.6 under
-// one element beyond all others, 37.9 in either case when read twice; 24 M 25 to 34, and 32 when read twice.
+// ------------------------------------------------------------------ SQ of a tensor much of which a second read takes from memory
+// The codes depend on the tensor's maximum through R(log2 max) alone, and a tile of a few thousand elements often has the tensor's
+// R(log2 max) already.  So the first pass codes every tile under the larger of its own maximum and what other blocks have reduced by
+// then, and leaves the shift it used; the second pass, under the whole maximum, codes again the tiles whose shift was another one, and
+// returns where there are none.  Bound by memory; times at kSqResident.
 
 // shift of a tile: what its codes were formed under, or one of
 constexpr int kTileAny = 0x7fff;     // all of it is zero: codes 0 under any shift
@@ -264,7 +263,7 @@ quantize_sq_kernel(const float *__restrict__ src, size_t n, int8_t *dst, int16_t
         // (the up to three elements behind the last float4 are coded by the second pass)
         if (blockIdx.x == 0 && r == 0 && threadIdx.x < (n & 3)) mx = abs_bits(src[n4 * 4 + threadIdx.x]);
 #pragma unroll
-        for (int u = 0; u < kQuantLoads; ++u) mx = max(mx, abs_bits(v[u]));
+        for (int u = 0; u < kQuantLoads; ++u) mx = max_abs(mx, v[u]);
         store_part(dst, n4, p, pow2_scale(guess.part(mx, threadIdx.x, dev)), v);
     }
     guess.publish(threadIdx.x, tile_shift + blockIdx.x, dev);
@@ -1149,8 +1148,12 @@ cudaError_t launch_reset_cells(DeviceState *dev, cudaStream_t s)
 
 bool quantize_is_small(int mode, size_t n, const ReduceHook &hook) { return mode == 2 && !hook.fn && n <= kSmallElems * kSmallCluster; }
 
-// Largest tensor whose codes wait for the maximum: what the L2 (126 MB) holds of it is read from there, see quantize_sq_kernel.
-constexpr size_t kSqResident = 24u << 20;
+// Largest tensor whose codes wait for the maximum (see quantize_sq_kernel).  Normal numbers / one element beyond all others / tiles of
+// unequal size, us, tensors from memory: 8 M floats 13.3 / 15.3 / 15.1 under the guess, 12.6 read twice; 10.5 M 15.3 / 16.8 / 17.1 and 15.3, the
+// line; 12.8 M 17.4 / 18.6 / 18.4 and 17.4 (in a row of calls on three tensors 16.4 or 17.7 from process to process, and 17.5); 21 M 23.0 /
+// 27.5 / 26.7 and 27.9; 34 M 39.1 / 36.7 / 37.3 and 44.0.  The worst of them is no slower than a maximum's pass with one load of a thread in
+// flight was (17.7, 21.3, 32.4, 50.4); below the line it is (4 M: 12.0 and 10.2).
+constexpr size_t kSqResident = 10u << 20;
 
 static unsigned quantize_tiles(size_t n) { return n / 4 > kQuantTile ? (unsigned)((n / 4 + kQuantTile - 1) / kQuantTile) : 1u; }
 

@@ -446,9 +446,9 @@ def test_quantize_float_of_more_parts_than_cells():
 
 
 @pytest.mark.parametrize("kind", ["even", "rising", "one tile", "zero tiles", "nan"])
-@pytest.mark.parametrize("n", [24 << 20, (24 << 20) + 1, 26000003])
+@pytest.mark.parametrize("n", [10 << 20, (10 << 20) + 1, 12000002, 24 << 20, (24 << 20) + 1, 26000003])
 def test_quantize_float_on_both_sides_of_the_cache(n, kind):
-    """The largest tensor that is read twice, and those whose tiles are coded before the maximum is known."""
+    """Tensors that are read twice, and those whose tiles are coded before the maximum is known (beyond 10 M floats)."""
     x = synth.normal_f32(n, 3043, 0)
     part = np.arange(n) // 8192
     if kind == "rising":

@@ -199,8 +199,8 @@ def test_bench_launcher_starts_the_ranks_itself():
 
 
 def test_small_quantizers_have_no_parameters_of_the_scale_quantizer():
-    """Calls in a row on a small tensor go by the rate of launches, and that by a kernel's parameters: Q and CQ need no maximum and carry
-    none of its parameters (3.4 us a call with two more, 3.0 without)."""
+    """Q and CQ need no maximum and carry none of SQ's parameters: calls in a row on a small tensor go by the rate of launches (3.4 us a
+    call as instances of SQ's second pass, 3.0 by themselves)."""
     from paper_2105_13890_b200 import build
 
     with open(os.path.join(build.CSRC, "eoq_elementwise.cu")) as f:
