@@ -195,10 +195,10 @@ __device__ __forceinline__ void tap_sets(const FinishItem &it, int slab, int sla
     __syncthreads();
 }
 
-// Range `range` (of `ranges`) of a slab's rows into its tap sums, by the calling block.  sets: shared memory of tap_set_bytes.
-// kBeside: the layer's GEMM is the launch in front and may still run.
-template <int kT, bool kBeside>
-__device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab, int range, int ranges, int32_t *sets)
+// Range `range` (of `ranges`, each of rows_here rows) of a slab's rows into its tap sums, by the calling block.  sets: shared memory of
+// tap_set_bytes.  kMayAdd: false where no item adds (tap_add); kBeside: the layer's GEMM is the launch in front and may still run.
+template <int kT, bool kMayAdd, bool kBeside>
+__device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab, int range, int ranges, int rows_here, int32_t *sets)
 {
     __shared__ TapMasks masks;
     const eoq_conv_desc_t &d = it.d;
@@ -207,19 +207,16 @@ __device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab,
     tap_masks(it, nr, nc, masks);   // (published by the barriers of tap_sets)
     const int slab_ch = min(kTapSlab, d.c_out - slab * kTapSlab);  // channels of this slab (16 or 32)
     const int taps = d.kh * d.kw, items = taps * slab_ch;
-    const int rows = d.n * it.ho, rows_here = (int)(((long long)rows + ranges - 1) / ranges);
-    const int begin = (int)min((long long)rows, (long long)range * rows_here), end = (int)min((long long)rows, (long long)begin + rows_here);
-    constexpr int kMost = (kMaxTaps * kTapSlab + kT - 1) / kT;   // items of a thread
-    long long total[kMost] = {};
+    const int rows = d.n * it.ho;   // (sums below: ranges * rows_here is less than rows + ranges)
+    const int begin = (int)min((uint32_t)rows, (uint32_t)range * rows_here), end = (int)min((uint32_t)rows, (uint32_t)begin + rows_here);
     const int chunk = (long long)rows_here * it.wo <= (1 << 23) ? max(1, rows_here) : max(1, (1 << 23) / it.wo);   // keeps the int32 sets exact
     const int ch_shift = 31 - __clz(slab_ch), per_kw = 65536 / d.kw + 1;   // tap / kw = tap * per_kw >> 16 for the few taps there are
+    const bool add = kMayAdd && it.tap_add;
     for (int at = 0; at < rows_here; at += chunk) {
         const int r0 = min(end, begin + at), r1 = min(end, r0 + min(chunk, rows_here - at));
         tap_sets<kT>(it, slab, slab_ch, r0, r1, nr, nc, sets);
-#pragma unroll
-        for (int k = 0; k < kMost; ++k) {
-            const int i = k * kT + (int)threadIdx.x;   // [tap][channel]
-            if (i >= items) continue;
+        if (kBeside && add) ptx::grid_dep_wait();   // (the GEMM has cleared the cells)
+        for (int i = threadIdx.x; i < items; i += kT) {   // [tap][channel], stored at [oc][tap]
             const int tap = i >> ch_shift, c = i & (slab_ch - 1), kh = tap * per_kw >> 16, kw = tap - kh * d.kw;
             const unsigned long long rm = masks.rows[kh], cm = masks.cols[kw];
             const int32_t *cell = sets + c;
@@ -230,24 +227,16 @@ __device__ __forceinline__ void finish_taps_slab(const FinishItem &it, int slab,
             };
             int sum = over_columns(cell);
             for (unsigned long long m = rm; m; m &= m - 1) sum -= over_columns(cell + __ffsll((long long)m) * (1 + nc) * kTapSlab);
-            total[k] += sum;
+            long long *copies = it.tap_sums + ((size_t)(slab * kTapSlab + c) * taps + tap) * kTapReplicas;
+            if (add) {
+                if (sum) atomicAdd(reinterpret_cast<unsigned long long *>(copies + range % kTapReplicas), (unsigned long long)(long long)sum);
+                continue;
+            }
+            copies[range] = at == 0 ? sum : copies[range] + sum;   // (its own copy)
+            if (range == 0 && at == 0)
+                for (int r = ranges; r < kTapReplicas; ++r) copies[r] = 0;
         }
         __syncthreads();
-    }
-    if (kBeside && it.tap_add) ptx::grid_dep_wait();   // (the GEMM has cleared the cells)
-#pragma unroll
-    for (int k = 0; k < kMost; ++k) {
-        const int i = k * kT + (int)threadIdx.x;   // stored at [oc][tap]
-        if (i >= items) continue;
-        const int tap = i >> ch_shift, c = i & (slab_ch - 1);
-        long long *cell = it.tap_sums + ((size_t)(slab * kTapSlab + c) * taps + tap) * kTapReplicas;
-        if (it.tap_add) {
-            if (total[k]) atomicAdd(reinterpret_cast<unsigned long long *>(cell + range % kTapReplicas), (unsigned long long)total[k]);
-            continue;
-        }
-        cell[range] = total[k];
-        if (range == 0)
-            for (int r = ranges; r < kTapReplicas; ++r) cell[r] = 0;
     }
 }
 
@@ -262,7 +251,8 @@ __global__ void __launch_bounds__(kTapThreads, 2) finish_taps_kernel(const __gri
     extern __shared__ __align__(16) int32_t sets[];
     const int k = finish_item_of(b.tap_first, b.num, (int)blockIdx.x);
     const int local = (int)blockIdx.x - b.tap_first[k], ranges = b.item[k].tap_ranges, slab = local / ranges;
-    finish_taps_slab<kTapThreads, kOrder == kTapsBeside>(b.item[k], slab, local - slab * ranges, ranges, sets);
+    finish_taps_slab<kTapThreads, kOrder != kTapsFirst, kOrder == kTapsBeside>(b.item[k], slab, local - slab * ranges, ranges, b.item[k].tap_rows,
+                                                                             sets);
     if (kOrder == kTapsBeside) ptx::grid_dep_wait();   // (what comes behind this launch waits for it alone)
 }
 
@@ -475,8 +465,10 @@ __global__ void __launch_bounds__(kSmallBounds) finish_small_kernel(const __grid
     if (!beside) ptx::grid_dep_wait();
     const int rank = (int)blockIdx.x;
     if (it.use_b1) {
-        const int slabs = tap_slabs(it), copies = slabs <= kSmallCtas / 4 ? 4 : (slabs <= kSmallCtas / 2 ? 2 : 1);
-        for (int i = rank; i < slabs * copies; i += kSmallCtas) finish_taps_slab<kSmallThreads, false>(it, i / copies, i % copies, copies, dyn);
+        const int slabs = tap_slabs(it), copies_log = slabs <= kSmallCtas / 4 ? 2 : (slabs <= kSmallCtas / 2 ? 1 : 0), copies = 1 << copies_log;
+        const int rows_here = (it.d.n * it.ho + copies - 1) >> copies_log;
+        for (int i = rank; i < slabs * copies; i += kSmallCtas)
+            finish_taps_slab<kSmallThreads, false, false>(it, i >> copies_log, i & (copies - 1), copies, rows_here, dyn);
     }
     ptx::cluster_wait();
     if (it.use_b1) {
@@ -608,6 +600,7 @@ void plan_finish(FinishBatch &b, const FinishItem *items, int num, int sm_count,
         it = items[k];
         it.keep_sums = hook.fn != nullptr;
         it.tap_ranges = split_taps(it, sm_count, num == 1 && whole_device);
+        it.tap_rows = (it.d.n * it.ho - 1) / it.tap_ranges + 1;
         it.tap_add = it.tap_ranges > kTapReplicas;
         it.tap_clear = it.tap_clear && it.use_b1 && (split_taps(it, sm_count, true) > kTapReplicas || split_taps(it, sm_count, false) > kTapReplicas);
         plan_finish_item(it, sm_count, num == 1);

@@ -480,7 +480,7 @@ struct FinishItem {
     BorderClasses bc;
     int ho, wo, num_parts;
     // filled by plan_finish
-    int tap_ranges, groups, fin_blocks, sq_blocks;
+    int tap_ranges, tap_rows, groups, fin_blocks, sq_blocks;   // (tap_rows: of a range; divided here, not in front of the first load)
     int tap_add;                   // the tap sums are added to cells that the GEMM has cleared (else stored)
     int tap_clear;                 // the last kernel clears them again: the slices can be finished once more, under any plan (set by the caller where
                                    // the GEMM was another call)
