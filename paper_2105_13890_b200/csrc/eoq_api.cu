@@ -424,9 +424,9 @@ void plan_classes(IgemmClasses &cl, int ctas)
         cost[k] = 2 * cl.p[k].ntaps + 1;
         work += (long long)tiles[k] * cost[k];
     }
-    // The least time from work / ctas on in which the classes get by with `ctas` CTAs, or with one each: by bisection, as they need fewer
-    // the longer it is, and one each once it covers all tiles of every class.  (Counted up one by one, 12,544 tiles a class under a cap of three
-    // CTAs took 20,908 steps.)
+    // The least time from work / ctas on in which the classes get by with `ctas` CTAs, or with one each: they need fewer the longer it is,
+    // and one each once it covers all tiles of every class.  It is mostly near: steps that double, then bisection.  (Counted up one by one,
+    // 12,544 tiles a class under a cap of three CTAs took 20,908 steps.)
     auto divide = [&](long long time) -> bool {
         int used = 0;
         cl.first[0] = 0;
@@ -438,8 +438,12 @@ void plan_classes(IgemmClasses &cl, int ctas)
         }
         return used <= ctas || used <= cl.num;
     };
-    long long low = work / ctas, high = low;   // `high` is enough, times below `low` are not
-    for (int k = 0; k < cl.num; ++k) high = std::max(high, (long long)tiles[k] * cost[k]);
+    long long low = work / ctas, high = low, most = low;   // `most` is enough, times below `low` are not
+    for (int k = 0; k < cl.num; ++k) most = std::max(most, (long long)tiles[k] * cost[k]);
+    for (long long step = 1; high < most && !divide(high); step *= 2) {
+        low = high + 1;
+        high = std::min(most, high + step);
+    }
     while (low < high) {
         const long long mid = (low + high) / 2;
         if (divide(mid)) high = mid;
